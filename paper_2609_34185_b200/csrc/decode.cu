@@ -44,7 +44,8 @@ namespace {
 constexpr uint32_t kChains = EP_CHAINS;
 constexpr int kWarps = EP_WARPS;                             // warps per CTA (one CTA per SM)
 constexpr int kThreads = kWarps * 32;
-constexpr uint32_t kTilesPerRound = kWarps * kChains;        // 48 tiles per CTA at a time
+constexpr uint32_t kTilesPerRound = kWarps * kChains;        // tiles per CTA at a time, at most (see split_rounds)
+constexpr uint32_t kMinWarps = 8;                            // threads that copy the tables, however few tiles a CTA has
 static_assert(kTilesPerRound == ep::kDecodeTilesPerCta, "tile-size suggestions assume this many tiles per CTA");
 constexpr uint32_t kLutEntries = 2048;                       // 2^11 slots per table
 constexpr uint32_t kLutStride = kLutEntries * 4;             // bytes per table in shared memory
@@ -109,8 +110,8 @@ struct JobParams {
     uint32_t V, n_tiles, b;       // n_tiles: tiles of the whole tensor
     uint32_t tile0, tile_cnt;     // the tiles this launch decodes: [tile0, tile0 + tile_cnt)
     int32_t zlo;                  // even, <= -2
-    uint32_t rounds;              // ceil(tile_cnt / 48): in one round the warps of a CTA take 48 consecutive tiles
-    uint32_t round_cost;          // work of one round in groups of 32 vectors (ceil(V / 32))
+    uint32_t rounds;              // ceil(tile_cnt / tiles per round): in one round the warps of a CTA take consecutive tiles
+    uint32_t round_cost;          // work of one round in groups of 32 vectors (ceil(V / 32)), or 1 (see split_rounds)
     uint32_t cost_begin;          // sum of rounds * round_cost over the jobs before this one
     uint32_t row_bytes;           // output bytes per row
     uint32_t row_rcp;             // ceil(2^32 / row_bytes)
@@ -123,6 +124,7 @@ struct JobParams {
 struct BatchParams {
     JobParams job[EP_MAX_BATCH];
     uint32_t cost_per_cta;        // ceil(sum of rounds * round_cost over all jobs / CTAs of the launch)
+    uint32_t tiles_per_round;     // tiles a CTA works on at a time: one per warp and chain, at most kTilesPerRound
     int32_t n_jobs;
 };
 
@@ -250,7 +252,7 @@ __device__ __forceinline__ void build_one_table(const JobParams &J, uint32_t t, 
 }
 
 __device__ __forceinline__ void build_tables_smem(const JobParams &J, uint32_t lut_addr, uint32_t warp, uint32_t lane) {
-    for (uint32_t t = 1 + warp; t < EP_NUM_TABLES; t += kWarps) {
+    for (uint32_t t = 1 + warp; t < EP_NUM_TABLES; t += blockDim.x >> 5) {
         const uint32_t base = lut_addr + (t - 1) * kLutStride;
         build_one_table(J, t, lane, [base](uint32_t slot, uint32_t e) { sts32(base + 4u * slot, e); });
     }
@@ -260,9 +262,10 @@ __device__ __forceinline__ void build_tables_smem(const JobParams &J, uint32_t l
 // copy is only started here; whoever reads the tables first waits for it (cp.async.wait_group, then a CTA barrier).
 __device__ __forceinline__ void copy_tables_smem(const uint32_t *image, uint32_t lut_addr, bool two_level) {
     const uint64_t src = reinterpret_cast<uint64_t>(image);
-    for (uint32_t o = 16u * threadIdx.x; o < kLutBytes; o += 16u * kThreads) cp_async16(lut_addr + o, src + o, 16);
+    const uint32_t step = 16u * blockDim.x;
+    for (uint32_t o = 16u * threadIdx.x; o < kLutBytes; o += step) cp_async16(lut_addr + o, src + o, 16);
     if (kTwoLevelInLoop && two_level)        // the hot part of the second level follows the image
-        for (uint32_t o = 16u * threadIdx.x; o < kHotBytes; o += 16u * kThreads)
+        for (uint32_t o = 16u * threadIdx.x; o < kHotBytes; o += step)
             cp_async16(lut_addr + kHotBase + o, src + kLutBytes + o, 16);
     cp_async_commit();
 }
@@ -1054,21 +1057,22 @@ __device__ __forceinline__ void decode_tile_plain(const JobParams &J, uint32_t t
 // `tables_pending`: the job's lookup tables are still being written (by this CTA's own stores or copies): the
 // tiles' records and first payload chunks are requested first, the CTA barrier comes after.
 template <int DT, int B>
-__device__ __forceinline__ void decode_tiles_fast(const JobParams &J, uint32_t first, uint32_t lut_addr, CosetFreq cf,
-                                                  uint32_t ring, uint32_t ctx, uint32_t lane, bool tables_pending) {
+__device__ __forceinline__ void decode_tiles_fast(const JobParams &J, uint32_t first, uint32_t tiles_per_round, uint32_t lut_addr,
+                                                  CosetFreq cf, uint32_t ring, uint32_t ctx, uint32_t lane, bool tables_pending) {
     constexpr uint32_t BB = Out<DT>::kBlockBytes;
     const uint32_t lt = (1u << lane) - 1u, lane16 = 16u * lane;
     uint32_t x[kChains], a[kChains], bal[kChains], doff[kChains], off[kChains], end[kChains], lead[kChains];
     bool valid[kChains];
 #pragma unroll
     for (uint32_t c = 0; c < kChains; ++c) {
-        valid[c] = first + c < J.tile_cnt;
+        // (a warp without a tile in this round - the job's last round, or a CTA with more warps than tiles - has no block)
+        valid[c] = first + c < J.tile_cnt && kChains * (threadIdx.x >> 5) + c < tiles_per_round;
         const uint32_t tile = J.tile0 + min(first + c, J.tile_cnt - 1u);
         const uint32_t rg = ring + c * kRingStride, cctx = ctx + kCtxChain + c * kCtxChainStride;
         const TileSetup T = tile_setup(J, tile, valid[c], lane);
         for (uint32_t k = 0; k < kRingSlots; ++k) ring_issue(rg, T.a0, T.room, k, lane);
         // the record of the tile this chain takes in the CTA's next round (132 bytes: two lines), into L2
-        if (lane < 2u && tile + kTilesPerRound < J.n_tiles) prefetch_l2(J.tile_index + size_t(tile + kTilesPerRound) * 33u + 32u * lane);
+        if (lane < 2u && tile + tiles_per_round < J.n_tiles) prefetch_l2(J.tile_index + size_t(tile + tiles_per_round) * 33u + 32u * lane);
         if (lane == 0) {                 // the next request is chunk 3, into slot 0
             prefetch_l2(J.scales + min(T.v0 / J.per_row, J.row_max));      // the first row scale the loop will ask for
             sts64(cctx + kCcSrc, T.a0 + kRingBytes);
@@ -1163,13 +1167,13 @@ __global__ void __launch_bounds__(kThreads, 1) ep_decode_smem_kernel(const __gri
         }
         __syncwarp();
         for (uint32_t r = r0; r < r1; ++r) {
-            const uint32_t base = r * kTilesPerRound + kChains * warp;
+            const uint32_t base = r * P.tiles_per_round + kChains * warp;
             if constexpr (DT != EP_FIELDS_I32) {
                 if (fast) {
                     if (kTwoLevelInLoop && J.b == 12u) {
-                        if constexpr (kTwoLevelInLoop) decode_tiles_fast<DT, 12>(J, base, lut_addr, cf, ring, ctx, lane, tables_pending);
+                        if constexpr (kTwoLevelInLoop) decode_tiles_fast<DT, 12>(J, base, P.tiles_per_round, lut_addr, cf, ring, ctx, lane, tables_pending);
                     } else {
-                        decode_tiles_fast<DT, 11>(J, base, lut_addr, cf, ring, ctx, lane, tables_pending);
+                        decode_tiles_fast<DT, 11>(J, base, P.tiles_per_round, lut_addr, cf, ring, ctx, lane, tables_pending);
                     }
                     tables_pending = false;
                     continue;
@@ -1181,7 +1185,7 @@ __global__ void __launch_bounds__(kThreads, 1) ep_decode_smem_kernel(const __gri
                 tables_pending = false;
             }
             for (uint32_t c = 0; c < kChains; ++c)
-                if (base + c < J.tile_cnt) decode_tile_plain<DT>(J, J.tile0 + base + c, lut_addr, cf, ring, lane);
+                if (base + c < J.tile_cnt && kChains * warp + c < P.tiles_per_round) decode_tile_plain<DT>(J, J.tile0 + base + c, lut_addr, cf, ring, lane);
         }
     }
 }
@@ -1778,6 +1782,42 @@ void fill_table_params(JobParams &J, const ep_info &I) {
     }
 }
 
+// How the tiles of a launch are spread over its CTAs (persistent, one per SM): sets tiles_per_round, every job's rounds and
+// costs and cost_per_cta; returns the grid size, 0 if the counts do not fit 32 bits.
+// A round is one tile per warp, and its warps share an SM's issue slots: 32 of them take 1.05 us for a group of 32 blocks
+// each, 8 take 0.7.  So the fewest rounds per CTA that 32 tiles at a time allow are kept, and then a round gets no more
+// tiles than it takes to spread them over all SMs in that many rounds: a 4096 x 4096 tensor of 1152 tiles runs as 144
+// CTAs of eight warps, not as 36 of 32.  With one round per CTA every CTA simply takes one; with more, the
+// cost-weighted list of all rounds is split evenly.
+uint32_t split_rounds(BatchParams &P, uint32_t sms) {
+    auto rounds_at = [&](uint32_t tpr) {
+        uint64_t n = 0;
+        for (int i = 0; i < P.n_jobs; ++i) n += (uint64_t(P.job[i].tile_cnt) + tpr - 1u) / tpr;
+        return n;
+    };
+    const uint64_t most = (rounds_at(kTilesPerRound) + sms - 1u) / sms * sms;
+    uint32_t lo = 1, hi = kTilesPerRound;                      // smallest tiles_per_round with at most `most` rounds
+    while (lo < hi) {
+        const uint32_t mid = (lo + hi) / 2u;
+        if (rounds_at(mid) <= most) hi = mid; else lo = mid + 1u;
+    }
+    P.tiles_per_round = lo;
+    const uint64_t rounds_total = rounds_at(lo);
+    uint64_t cost = 0;
+    for (int i = 0; i < P.n_jobs; ++i) {
+        JobParams &J = P.job[i];
+        J.rounds = (J.tile_cnt + lo - 1u) / lo;
+        J.round_cost = rounds_total <= sms ? 1u : (J.V + 31u) / 32u;
+        J.cost_begin = uint32_t(cost);
+        cost += uint64_t(J.rounds) * J.round_cost;
+    }
+    const uint32_t grid = uint32_t(rounds_total < sms ? rounds_total : sms);
+    // (a tensor has under 2^27 blocks, so sixteen of them cost under 2^26 groups: 32-bit arithmetic in the kernel)
+    if (cost + grid >= (1ull << 31)) return 0;
+    P.cost_per_cta = uint32_t((cost + grid - 1u) / grid);
+    return grid;
+}
+
 template <int DT>
 cudaError_t launch_smem(const BatchParams &P, uint32_t grid, cudaStream_t st) {
     static bool configured[64] = {};   // the attribute is per device
@@ -1789,7 +1829,8 @@ cudaError_t launch_smem(const BatchParams &P, uint32_t grid, cudaStream_t st) {
         if (e != cudaSuccess) return e;
         if (dev >= 0 && dev < 64) configured[dev] = true;
     }
-    ep_decode_smem_kernel<DT><<<grid, kThreads, kSmemBytes, st>>>(P);
+    const uint32_t warps = (P.tiles_per_round + kChains - 1u) / kChains;
+    ep_decode_smem_kernel<DT><<<grid, 32u * (warps < kMinWarps ? kMinWarps : warps), kSmemBytes, st>>>(P);
     return cudaGetLastError();
 }
 
@@ -2039,9 +2080,6 @@ extern "C" int ep_decode_batch(const ep_decode_job *jobs_in, int32_t n_in, void 
     GBatchParams B12;               // two-level tables that have to be built into scratch first
     std::memset(&B12, 0, sizeof(B12));
     int n_build12 = 0;
-    // persistent CTAs, one per SM (fewer if the launch has fewer rounds than SMs); the kernel splits the
-    // cost-weighted list of all rounds evenly over them
-    uint64_t rounds_total = 0, cost = 0;
     for (int i = 0; i < n_jobs; ++i) {
         const ep_decode_job &jb = *fast[i];
         const ep_info &I = *jb.info;
@@ -2080,20 +2118,13 @@ extern "C" int ep_decode_batch(const ep_decode_job *jobs_in, int32_t n_in, void 
         J.row_bytes = J.per_row * block_bytes;
         J.row_rcp = uint32_t(0xFFFFFFFFu / J.row_bytes + 1u);
         J.row_max = I.R - 1u;
-        J.rounds = (my_tiles + kTilesPerRound - 1u) / kTilesPerRound;
-        J.round_cost = (I.V + 31u) / 32u;
-        J.cost_begin = uint32_t(cost);
-        cost += uint64_t(J.rounds) * J.round_cost;
-        rounds_total += J.rounds;
     }
+    const uint32_t next = split_rounds(P, uint32_t(sms));      // grid size
+    if (next == 0) return EP_ERR_UNSUPPORTED;
     if (n_build12) {
         B12.n_jobs = n_build12;
         if (launch_build12(B12, n_build12, st) != cudaSuccess) return EP_ERR_CUDA;
     }
-    const uint32_t next = uint32_t(rounds_total < uint64_t(sms) ? rounds_total : uint64_t(sms));   // grid size
-    // a tensor has under 2^27 blocks, so sixteen of them cost under 2^26 groups: 32-bit arithmetic in the kernel
-    if (cost + next >= (1ull << 31)) return EP_ERR_UNSUPPORTED;
-    P.cost_per_cta = uint32_t((cost + next - 1u) / next);
     cudaError_t e;
     switch (dt) {
     case EP_BF16: e = launch_smem<EP_BF16>(P, next, st); break;
