@@ -1,11 +1,12 @@
 // CUDA back end of the EntroPack encoder (paper Sec. 3.2-3.6): row RMS, E8 quantisation with field
-// histograms, row-scale refit and tiled 32-state rANS encoding run on the GPU; the few-kilobyte steps
-// (frequency normalisation, C_CE, the stored-size estimate, the bisection itself) stay on the host and
-// are shared with the host back end, so both produce the same bytes for the same input.
+// histograms, the bisection of Algorithm 1, row-scale refit and tiled 32-state rANS encoding run on the GPU;
+// the rate correction and the final tables (a few kilobytes of counts) stay on the host and are shared with
+// the host back end, so both produce the same bytes for the same input.
 //
-// Every floating-point step uses the same operations in the same order as the host code: IEEE
-// single-precision division and subtraction, round-to-nearest-even, double-precision sums in index
-// order written with explicit add / multiply intrinsics so that nothing is fused.
+// Every result that enters the stream is the host code's bit for bit.  Where the host's operation order is
+// expensive here (two divisions per weight, sums in index order), the kernel computes the value another way together
+// with a bound on the difference, keeps it if no value inside the bound would round or compare differently, and
+// otherwise repeats the host's operations.
 #include <cuda_runtime.h>
 
 #include <mutex>
@@ -28,67 +29,81 @@ using namespace ep;
 
 constexpr int kHistBins = 8192;          // per table, values -4096 .. 4095
 constexpr int kHistOrigin = -4096;
-constexpr int kLocalBins = 512;          // shared-memory window per table, values -256 .. 255
-constexpr int kLocalOrigin = -256;
-constexpr uint32_t kMaxTableSymbols = 40960;   // sum of K over the 17 tables that the tile encoder keeps in shared memory
+constexpr uint32_t kMaxTableSymbols = 40960;   // sum of K over the 17 tables that a stream of this back end may have
+constexpr double kUnit = 1.1102230246251565e-16;   // 2^-53, the rounding unit of double
 
-// ---- rows whose sums run in index order ---------------------------------------------------------------
-// The row RMS (Sec. 3.2) and the refit of Eq. 13 sum over a row in double precision in index order, as the host code
-// does: one serial chain of additions per row, which no reduction tree reproduces bit for bit.  One thread per row
-// reading its own row leaves the GPU waiting for memory (8192 rows = 256 warps with a few KB in flight each: 0.29 ms
-// for the RMS of an 8192 x 8192 tensor).  So a CTA takes kRowsPerCta rows: all its threads stream the rows through
-// shared memory with cp.async, kRowStages chunks ahead, and kRowsPerCta lanes of its first warp run the chains.
-constexpr uint32_t kRowsPerCta = 8, kRowStages = 4, kRowThreads = 256;
-constexpr uint32_t kRmsChunk = 256;                 // floats per row and chunk
-constexpr uint32_t kRmsStride = kRmsChunk + 4;      // padded: the eight lanes read different banks
+// ---- sums over a row ------------------------------------------------------------------------------------
+// The row RMS (Sec. 3.2) and Eq. 13 are defined by sums in double in index order, a chain of dependent additions per
+// row (14 cycles each: 60 us for 8192 of them, whatever the bandwidth).  Here a CTA sums a row in parallel.
+// Sequential summation of n terms is off by at most n * 2^-53 * (sum of magnitudes) from the exact sum, the tree by far
+// less, so the sequential result lies in an interval around the tree's; what is stored is that result rounded to
+// fp32, 2^29 times coarser, through monotone operations only.  If both ends of the interval round to the same fp32
+// number, it is the sequential one's.  Otherwise (about one row in 10^5) the CTA forms the sequential sum.
+constexpr uint32_t kRowThreads = 128;
 
-__device__ __forceinline__ void cp_async_16(void *smem_dst, const void *src) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(uint32_t(__cvta_generic_to_shared(smem_dst))), "l"(src) : "memory");
+__device__ __forceinline__ double cta_sum(double v, double *part) {
+#pragma unroll
+    for (int d = 16; d; d >>= 1) v = __dadd_rn(v, __shfl_xor_sync(0xFFFFFFFFu, v, d));
+    __syncthreads();
+    if ((threadIdx.x & 31u) == 0) part[threadIdx.x >> 5] = v;
+    __syncthreads();
+    double s = part[0];
+#pragma unroll
+    for (uint32_t i = 1; i < kRowThreads / 32u; ++i) s = __dadd_rn(s, part[i]);
+    return s;                                    // the same in every thread
 }
-__device__ __forceinline__ void cp_async_commit_group() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait_group() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+// how far the sequential sum of n terms (magnitudes summing to `mag`) can be from the tree's
+__device__ __forceinline__ double order_bound(uint32_t n, double mag) { return (1.02 * double(n) + 64.0) * kUnit * mag; }
 
-__global__ void __launch_bounds__(kRowThreads) row_rms_kernel(const float *__restrict__ W, uint32_t R, uint32_t C, float *__restrict__ mu) {
-    __shared__ __align__(16) float buf[kRowStages][kRowsPerCta][kRmsStride];
-    const uint32_t tid = threadIdx.x, row0 = blockIdx.x * kRowsPerCta;
-    const uint32_t chunks = (C + kRmsChunk - 1) / kRmsChunk;
-    // chunk c of the CTA's rows: kRowsPerCta x 64 pieces of 16 bytes, two per thread (rows start 16-byte aligned: C % 8 == 0)
-    auto issue = [&](uint32_t c) {
-        if (c < chunks) {
-            for (uint32_t i = tid; i < kRowsPerCta * (kRmsChunk / 4); i += kRowThreads) {
-                const uint32_t r = i / (kRmsChunk / 4), j = i % (kRmsChunk / 4), col = c * kRmsChunk + 4 * j;
-                if (row0 + r < R && col < C) cp_async_16(&buf[c % kRowStages][r][4 * j], W + size_t(row0 + r) * C + col);
-            }
-        }
-        cp_async_commit_group();
-    };
-    for (uint32_t c = 0; c + 1 < kRowStages; ++c) issue(c);
+__device__ __forceinline__ float rms_result(double acc, uint32_t C) {
+    double m = __dsqrt_rn(__ddiv_rn(acc, double(C)));
+    if (!(m > 1e-12)) m = 1e-12;
+    return __double2float_rn(m);
+}
+
+__global__ void __launch_bounds__(kRowThreads) row_rms_kernel(const float *__restrict__ W, uint32_t C, float *__restrict__ mu) {
+    __shared__ double part[kRowThreads / 32];
+    __shared__ __align__(16) float4 stage[kRowThreads];
+    const uint32_t tid = threadIdx.x, n4 = C / 4;
+    const float4 *x = reinterpret_cast<const float4 *>(W + size_t(blockIdx.x) * C);   // 16-byte aligned: C % 8 == 0
     double acc = 0.0;
-    for (uint32_t c = 0; c < chunks; ++c) {
-        issue(c + kRowStages - 1);
-        cp_async_wait_group<kRowStages - 1>();
+    auto add = [&](const float4 v) {
+        const double a = double(v.x), b = double(v.y), c = double(v.z), d = double(v.w);
+        acc = __fma_rn(a, a, acc);               // (squares of fp32 numbers are exact in double)
+        acc = __fma_rn(b, b, acc);
+        acc = __fma_rn(c, c, acc);
+        acc = __fma_rn(d, d, acc);
+    };
+    uint32_t j = tid;
+    for (; j + 3u * kRowThreads < n4; j += 4u * kRowThreads) {
+        const float4 a = __ldg(x + j), b = __ldg(x + j + kRowThreads), c = __ldg(x + j + 2u * kRowThreads), d = __ldg(x + j + 3u * kRowThreads);
+        add(a); add(b); add(c); add(d);
+    }
+    for (; j < n4; j += kRowThreads) add(__ldg(x + j));
+    const double sum = cta_sum(acc, part), off = order_bound(C, sum);
+    const float lo = rms_result(__dsub_rn(sum, off), C), hi = rms_result(__dadd_rn(sum, off), C);
+    if (lo == hi) {
+        if (tid == 0) mu[blockIdx.x] = lo;
+        return;
+    }
+    acc = 0.0;                                   // index order
+    for (uint32_t j0 = 0; j0 < n4; j0 += kRowThreads) {
         __syncthreads();
-        if (tid < kRowsPerCta && row0 + tid < R) {
-            const uint32_t n4 = (min(kRmsChunk, C - c * kRmsChunk)) / 4;
-            const float4 *x = reinterpret_cast<const float4 *>(&buf[c % kRowStages][tid][0]);
-            for (uint32_t j = 0; j < n4; ++j) {
-                const float4 v = x[j];
+        if (j0 + tid < n4) stage[tid] = __ldg(x + j0 + tid);
+        __syncthreads();
+        if (tid == 0)
+            for (uint32_t i = 0, n = min(kRowThreads, n4 - j0); i < n; ++i) {
+                const float4 v = stage[i];
                 acc = __dadd_rn(acc, __dmul_rn(double(v.x), double(v.x)));
                 acc = __dadd_rn(acc, __dmul_rn(double(v.y), double(v.y)));
                 acc = __dadd_rn(acc, __dmul_rn(double(v.z), double(v.z)));
                 acc = __dadd_rn(acc, __dmul_rn(double(v.w), double(v.w)));
             }
-        }
-        __syncthreads();                     // the stage may be overwritten by the next issue
     }
-    if (tid < kRowsPerCta && row0 + tid < R) {
-        double m = __dsqrt_rn(__ddiv_rn(acc, double(C)));
-        if (!(m > 1e-12)) m = 1e-12;
-        mu[row0 + tid] = __double2float_rn(m);
-    }
+    if (tid == 0) mu[blockIdx.x] = rms_result(acc, C);
 }
 
+// ---- E8 quantisation (Eq. 2-4) ---------------------------------------------------------------------------
 // Eq. 3 on one 8-vector: integer point and fp32 residuals of that point
 struct D8 {
     int32_t z[8];
@@ -120,8 +135,9 @@ __device__ __forceinline__ void nearest_d8(const float *y, D8 &o) {
     }
 }
 
-// Eq. 2 + Eq. 4 on one block of eight weights; returns false if a coordinate leaves the histogram range
-__device__ __forceinline__ bool quantise_block(const float *x, float mu, float s, int32_t *fld) {
+// Eq. 2 as the host writes it: z[0..8) = the lattice point's integer parts, returns the coset; -1 if a coordinate leaves
+// the histogram range
+__device__ __noinline__ int quantise_exact(const float *x, float mu, float s, int32_t *z) {
     float y[8], yh[8];
     bool ok = true;
 #pragma unroll
@@ -130,7 +146,7 @@ __device__ __forceinline__ bool quantise_block(const float *x, float mu, float s
         yh[i] = __fsub_rn(y[i], 0.5f);
         ok = ok && (fabsf(y[i]) < 4000.0f);
     }
-    if (!ok) return false;
+    if (!ok) return -1;
     D8 a, h;
     nearest_d8(y, a);
     nearest_d8(yh, h);
@@ -141,74 +157,386 @@ __device__ __forceinline__ bool quantise_block(const float *x, float mu, float s
         dh = __dadd_rn(dh, __dmul_rn(double(h.res[i]), double(h.res[i])));
     }
     const bool half = dh < da;                       // the half coset only when strictly closer
-    fld[0] = half ? 1 : 0;
-    int32_t s7 = 0;
 #pragma unroll
-    for (int i = 0; i < 7; ++i) {
-        fld[1 + i] = half ? h.z[i] : a.z[i];
-        s7 += fld[1 + i];
-    }
-    const int32_t z8 = half ? h.z[7] : a.z[7];
-    fld[8] = (z8 - (s7 & 1)) >> 1;
-    return true;
+    for (int i = 0; i < 8; ++i) z[i] = half ? h.z[i] : a.z[i];
+    return half ? 1 : 0;
 }
 
-// Quantise blocks of the listed rows (rows == nullptr: all rows) at scale s; store the fields (fields != nullptr)
-// and count them: a shared-memory window per CTA for values near zero, global atomics for the rest.
-__global__ void __launch_bounds__(256) quantise_count_kernel(const float *__restrict__ W, uint32_t C, const float *__restrict__ mu,
-                                                             const uint32_t *__restrict__ rows, uint64_t n_blocks8, float s,
-                                                             int16_t *__restrict__ fields, uint32_t *__restrict__ hist,
-                                                             int *__restrict__ overflow) {
-    __shared__ uint32_t local[EP_NUM_TABLES * kLocalBins];
-    for (uint32_t i = threadIdx.x; i < EP_NUM_TABLES * kLocalBins; i += blockDim.x) local[i] = 0;
-    __syncthreads();
-    const uint32_t per_row = C / 8;
-    for (uint64_t v = uint64_t(blockIdx.x) * blockDim.x + threadIdx.x; v < n_blocks8; v += uint64_t(gridDim.x) * blockDim.x) {
-        const uint64_t i = v / per_row;
-        const uint32_t col = uint32_t(v - i * per_row);
-        const uint64_t r = rows ? rows[i] : i;
-        const float4 *src = reinterpret_cast<const float4 *>(W + r * C + 8ull * col);
-        const float4 lo = src[0], hi = src[1];
-        const float x[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
-        int32_t fld[9];
-        if (!quantise_block(x, mu[r], s, fld)) { *overflow = 1; continue; }
-        if (fields) {
+// The same point from y ~ x * r with r ~ 1 / (mu s), or `false` where the difference could matter.
+// y is within E = 4e-7 (|y| + 1) of the host's (two roundings there, three here, each 2^-24, and the host's y - 1/2).
+// With a_i = |y_i - rint(y_i)|: the integer candidate has residuals a_i, the half candidate 1/2 - a_i, and Eq. 3's parity
+// step moves the largest residual r to 1 - r; so the squared distances differ by
+//     d_half - d_int = 2 - sum a + [half parity odd] 2 min a - [integer parity odd] (1 - 2 max a).
+// Every decision - the two roundings of each coordinate, the coset, which coordinate the parity step moves - must have
+// a margin of more than what E can change.  At 4 bpp one block in 4000 fails and takes the divisions; at 8 bpp one
+// in 250.  (Compared with the exact routine on 6 x 10^7 random blocks and blocks built around ties: no difference.)
+__device__ __forceinline__ bool quantise_fast(const float (&x)[8], float r, int32_t (&z)[8], uint32_t &half) {
+    float a[8];
+    uint32_t neg[8], odd_int = 0, odd_neg = 0;
+    float ymax = 0.0f, sum = 0.0f;
 #pragma unroll
-            for (int k = 0; k < 9; ++k) fields[v * 9 + k] = int16_t(fld[k]);
-        }
+    for (int i = 0; i < 8; ++i) {
+        const float y = __fmul_rn(x[i], r);
+        const float t = __fadd_rn(y, 12582912.0f);            // 1.5 * 2^23: rounds to the nearest integer
+        z[i] = __float_as_int(t) - 0x4B400000;
+        const float res = __fsub_rn(y, __fsub_rn(t, 12582912.0f));
+        neg[i] = __float_as_uint(res) >> 31;
+        a[i] = fabsf(res);
+        odd_int ^= uint32_t(z[i]);
+        odd_neg ^= neg[i];
+        ymax = fmaxf(ymax, fabsf(y));
+        sum = __fadd_rn(sum, a[i]);
+    }
+    float big = a[0], small = a[0];
 #pragma unroll
-        for (int k = 0; k < 9; ++k) {
-            const int t = k == 0 ? 0 : 1 + 8 * fld[0] + (k - 1);
-            const int32_t val = fld[k];
-            if (val >= kLocalOrigin && val < kLocalOrigin + kLocalBins) atomicAdd(&local[t * kLocalBins + (val - kLocalOrigin)], 1u);
-            else if (val >= kHistOrigin && val < kHistOrigin + kHistBins) atomicAdd(&hist[t * kHistBins + (val - kHistOrigin)], 1u);
-            else *overflow = 1;
-        }
+    for (int i = 1; i < 8; ++i) { big = fmaxf(big, a[i]); small = fminf(small, a[i]); }
+    const bool oi = odd_int & 1u, oh = (odd_int ^ odd_neg) & 1u;
+    const float E = 4e-7f * ymax + 4e-7f;
+    float d = 2.0f - sum;
+    if (oh) d += 2.0f * small;
+    if (oi) d -= 1.0f - 2.0f * big;
+    bool ok = small > E && big < 0.5f - E && fabsf(d) > 16.0f * E + 4e-6f && ymax < 3990.0f;
+    const bool h = d < 0.0f;
+    half = h ? 1u : 0u;
+    const bool odd = h ? oh : oi;
+    const float sel = h ? small : big, near = 2.5f * E;
+    uint32_t hits = 0;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const uint32_t hit = fabsf(a[i] - sel) <= near ? 1u : 0u;
+        hits += hit;
+        // integer candidate: rint(y), its moved coordinate away from y's side; half candidate: floor(y), the moved one too
+        z[i] += (odd && hit ? 1 - 2 * int(neg[i] ^ half) : 0) - int(neg[i] & half);
     }
-    __syncthreads();
-    for (uint32_t i = threadIdx.x; i < EP_NUM_TABLES * kLocalBins; i += blockDim.x) {
-        const uint32_t c = local[i];
-        if (c) {
-            const uint32_t t = i / kLocalBins, j = i % kLocalBins;
-            atomicAdd(&hist[t * kHistBins + (int(j) + kLocalOrigin - kHistOrigin)], c);
-        }
-    }
+    return ok && !(odd && hits != 1u);
 }
 
-// Eq. 13: the two sums of a row in double in index order.  One block = 8 weights and its nine fields.
-__device__ __forceinline__ void refit_block(const float *xv, const int16_t *qv, double &xp, double &pp) {
-    const double half = 0.5 * double(qv[0]);
+// ---- counting passes ---------------------------------------------------------------------------------------
+// One pass quantises the listed rows (all rows) at one scale and counts the fields.  The last CTA to finish gathers
+// the counts for the host, or - in a step of the bisection - evaluates Eq. 10-12 on them and leaves the next scale
+// in device memory, so that the twelve steps and the full pass after them are one stream of launches with a
+// single wait at the end.
+// Counting is what a pass spends most on after the arithmetic: nine increments per block, most of them of a few
+// values around zero.  Each lane has its own column of counters for those (bank = lane: no two lanes of a warp
+// meet), values up to +-256 go to a plain window, the rest to global memory.
+constexpr uint32_t kCountThreads = 1024;
+constexpr int kHotBins = 32, kHotOrigin = -16;   // values with a counter column per lane, per coordinate table
+constexpr int kWinBins = 512, kWinOrigin = -256; // values with one counter per CTA, per table
+constexpr uint32_t kHotWords = 16 * kHotBins * 32, kWinWords = EP_NUM_TABLES * kWinBins;
+constexpr uint32_t kCountSmem = 4 * (kHotWords + kWinWords);
+// symbols over all tables that a step's evaluation holds in shared memory (it reuses the counters' space); with
+// more of them the host takes over
+constexpr uint32_t kEvalSymbols = kHotWords + kWinWords;
+constexpr uint32_t kFirstCounts = 6144;          // counts that come back with the state; more take a second copy
+
+struct CountDir { int32_t lo[EP_NUM_TABLES]; uint32_t K[EP_NUM_TABLES]; };
+
+// what the passes leave for one another and for the host (device memory, zeroed before the first pass)
+struct SearchState {
+    double lo, hi;                   // the bracket
+    float s;                         // the next pass's scale
+    uint32_t has_last;               // 1: `last` holds the last step whose rate was evaluated; 2: it has been overwritten
+    uint32_t undecided;              // a step fell within the rounding error of the target, or had too many symbols
+    uint32_t overflow;               // a coordinate left the histogram range
+    uint32_t finished;               // CTAs of the running pass that are done
+    // observed range of the running pass, stored as the larger of (kHistBins - bin) and of (bin + 1); 0: none
+    uint32_t from[EP_NUM_TABLES], to[EP_NUM_TABLES];
+    CountDir last, full;
+    uint32_t total_words;            // tile coding: words of the payload
+    uint32_t tiles_done;             //              CTAs of the launch that are done
+};
+constexpr size_t kStateBytes = 1024;
+static_assert(sizeof(SearchState) <= kStateBytes, "state area");
+
+// the constants of Eq. 10-12 on the sample
+struct StepParams {
+    double target, retained_bits_total, fixed_bits, weights, sample_fields;   // fixed_bits: restarts, scales, header
+    double lo0, hi0;                 // the bracket before the first step
+    int32_t b, step;                 // step: 0 .. for a step of the bisection, -1 for a pass that only counts
+};
+
+struct CountParams {
+    const float *W;
+    const float *mu;
+    const uint32_t *rows;            // null: all rows
+    uint4 *fields;                   // one per block: z1 .. z7 and 2 m + c as int16; null: not kept
+    uint32_t *hist;                  // EP_NUM_TABLES x kHistBins, zero between passes
+    SearchState *state;
+    uint32_t *last_counts, *full_counts;
+    uint64_t n_blocks;
+    uint32_t C, per_row;
+    float s;
+    uint32_t s_from_state;
+    StepParams step;
+};
+
+__device__ __forceinline__ uint32_t warp_sum(uint32_t v) { return __reduce_add_sync(0xFFFFFFFFu, v); }
+__device__ __forceinline__ double warp_sum(double v) {
+#pragma unroll
+    for (int d = 16; d; d >>= 1) v = __dadd_rn(v, __shfl_xor_sync(0xFFFFFFFFu, v, d));
+    return v;
+}
+__device__ __forceinline__ unsigned long long warp_sum(unsigned long long v) {
+#pragma unroll
+    for (int d = 16; d; d >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, d);
+    return v;
+}
+
+// The last CTA of a pass: ranges and offsets of the tables, counts to `out`, histogram back to zero.  For a step of the
+// bisection also the frequencies of Sec. 3.3 (integers: the host's exactly), C_CE of Eq. 8 and the comparison of
+// Eq. 12 with the target.  C_CE is a sum of doubles in another order and with this device's log2; if the host's
+// value, within the bound `off`, could compare differently, the step is marked undecided and the host repeats the search.
+__device__ void close_pass(const CountParams &P, uint32_t *f_of) {
+    __shared__ int32_t lo_of[EP_NUM_TABLES];
+    __shared__ uint32_t K_of[EP_NUM_TABLES], at_of[EP_NUM_TABLES + 1], seen_of[EP_NUM_TABLES];
+    __shared__ double bits_of[EP_NUM_TABLES];
+    SearchState &S = *P.state;
+    const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
+    const bool step = P.step.step >= 0;
+    if (tid < EP_NUM_TABLES) {
+        const uint32_t a = __ldcg(&S.from[tid]), z = __ldcg(&S.to[tid]);
+        const uint32_t first = kHistBins - a;
+        lo_of[tid] = a ? kHistOrigin + int32_t(first) : 0;
+        K_of[tid] = a ? z - first : 0u;                     // z = last bin + 1
+        S.from[tid] = 0;
+        S.to[tid] = 0;
+    }
+    __syncthreads();
+    if (tid == 0) {
+        uint32_t at = 0;
+        for (int t = 0; t < EP_NUM_TABLES; ++t) { at_of[t] = at; at += K_of[t]; }
+        at_of[EP_NUM_TABLES] = at;
+        S.finished = 0;
+    }
+    __syncthreads();
+    const bool too_many = step && at_of[EP_NUM_TABLES] > kEvalSymbols;
+    uint32_t *out = step ? P.last_counts : P.full_counts;
+    for (uint32_t t = warp; t < EP_NUM_TABLES; t += kCountThreads / 32u) {
+        const uint32_t K = K_of[t], at = at_of[t];
+        uint32_t *h = P.hist + t * kHistBins + (lo_of[t] - kHistOrigin);
+        unsigned long long sum = 0;
+        uint32_t seen = 0;
+        for (uint32_t j = lane; j < K; j += 32) {
+            const uint32_t n = __ldcg(h + j);
+            h[j] = 0;
+            if (!too_many) out[at + j] = n;
+            sum += n;
+            seen += n != 0;
+        }
+        if (!step || too_many) continue;
+        const double total = double(warp_sum(sum));
+        seen = warp_sum(seen);
+        // frequencies: max(1, floor(n 2^b / total)), then the deficit to the largest or the excess from the largest
+        const uint32_t M = 1u << P.step.b;
+        uint32_t fsum = 0, best = 0;
+        auto key = [](uint32_t f, uint32_t j) { return (f << 16) | (0xFFFFu - j); };      // f <= 2^15, j < 2^13: first of the largest
+        for (uint32_t j = lane; j < K; j += 32) {
+            const uint32_t n = out[at + j];
+            uint32_t f = 0;
+            if (n) {
+                const double nM = double(n) * double(M);                                  // below 2^47: exact
+                uint32_t q = uint32_t(nM / total);
+                const double r = __fma_rn(-double(q), total, nM);                         // exact: the quotient is off by one at most
+                if (r < 0.0) --q; else if (r >= total) ++q;
+                f = max(q, 1u);
+            }
+            f_of[at + j] = f;
+            fsum += f;
+            best = max(best, key(f, j));
+        }
+        fsum = warp_sum(fsum);
+        best = __reduce_max_sync(0xFFFFFFFFu, best);
+        __syncwarp();
+        if (K && fsum < M) {
+            if (lane == 0) f_of[at + 0xFFFFu - (best & 0xFFFFu)] += M - fsum;
+        }
+        while (K && fsum > M) {                              // (every turn lowers fsum or leaves)
+            const uint32_t f = best >> 16, take = min(fsum - M, f - 1u);
+            if (f <= 1u) break;                              // more symbols than slots: the step is judged by `seen`
+            if (lane == 0) f_of[at + 0xFFFFu - (best & 0xFFFFu)] = f - take;
+            fsum -= take;
+            __syncwarp();
+            if (fsum <= M) break;
+            best = 0;
+            for (uint32_t j = lane; j < K; j += 32) best = max(best, key(f_of[at + j], j));
+            best = __reduce_max_sync(0xFFFFFFFFu, best);
+        }
+        __syncwarp();
+        double bits = 0.0;
+        for (uint32_t j = lane; j < K; j += 32) {
+            const uint32_t n = out[at + j];
+            if (n) bits += double(n) * (double(P.step.b) - log2(double(f_of[at + j])));
+        }
+        bits = warp_sum(bits);
+        if (lane == 0) { bits_of[t] = bits; seen_of[t] = seen; }
+    }
+    __syncthreads();
+    CountDir &D = step ? S.last : S.full;
+    if (!too_many && tid < EP_NUM_TABLES) { D.lo[tid] = lo_of[tid]; D.K[tid] = K_of[tid]; }
+    if (!step || tid != 0) return;
+    double lo = P.step.step == 0 ? P.step.lo0 : S.lo, hi = P.step.step == 0 ? P.step.hi0 : S.hi;
+    const double mid = __dsqrt_rn(__dmul_rn(lo, hi));
+    if (too_many) {
+        S.undecided = 1;
+    } else {
+        double cce = 0.0;
+        uint32_t worst = 0;
+        for (int t = 0; t < EP_NUM_TABLES; ++t) { cce = __dadd_rn(cce, bits_of[t]); worst = max(worst, seen_of[t]); }
+        bool above;
+        if (worst > (1u << P.step.b)) {
+            above = true;                                    // no b-bit table exists for this scale: too fine
+            if (S.has_last) S.has_last = 2;
+        } else {
+            const double tables = 8.0 * double((8u * EP_NUM_TABLES + 2u * at_of[EP_NUM_TABLES] + 3u) & ~3u);
+            auto rate_above = [&](double c) {
+                const double left = fmax(0.0, __dsub_rn(c, P.step.retained_bits_total));
+                const double payload = __dmul_rn(16.0, ceil(__dmul_rn(left, 0.0625)));
+                return __ddiv_rn(__dadd_rn(__dadd_rn(payload, P.step.fixed_bits), tables), P.step.weights) > P.step.target;
+            };
+            // terms are at most b <= 15 bits per field, their sum is taken in a few thousand additions
+            const double off = 1e-11 * (cce + 16.0 * P.step.sample_fields);
+            above = rate_above(cce);
+            if (rate_above(cce - off) != rate_above(cce + off)) S.undecided = 1;
+            S.has_last = 1;
+        }
+        if (above) lo = mid; else hi = mid;
+    }
+    S.lo = lo;
+    S.hi = hi;
+    S.s = __double2float_rn(__dsqrt_rn(__dmul_rn(lo, hi)));
+}
+
+__global__ void __launch_bounds__(kCountThreads, 1) quantise_count_kernel(const __grid_constant__ CountParams P) {
+    extern __shared__ __align__(16) uint32_t sm[];
+    uint32_t *const hot = sm, *const win = sm + kHotWords;
+    __shared__ uint32_t range_from[EP_NUM_TABLES], range_to[EP_NUM_TABLES], last_cta;
+    const uint32_t tid = threadIdx.x, lane = tid & 31u;
+    // this CTA's blocks and this thread's first one; the rows of neighbouring blocks follow without divisions
+    const uint64_t v0 = P.n_blocks * blockIdx.x / gridDim.x, v1 = P.n_blocks * (blockIdx.x + 1ull) / gridDim.x;
+    uint64_t v = v0 + tid;
+    uint64_t i = v / P.per_row;
+    uint32_t col = uint32_t(v - i * P.per_row);
+    const uint32_t row_step = kCountThreads / P.per_row, col_step = kCountThreads % P.per_row;
+    float4 lo4 = make_float4(0.f, 0.f, 0.f, 0.f), hi4 = lo4;
+    float mu = 1.0f;
+    auto load = [&]() {
+        const uint64_t r = P.rows ? P.rows[i] : i;
+        const float4 *src = reinterpret_cast<const float4 *>(P.W + r * P.C + 8ull * col);
+        lo4 = __ldg(src);
+        hi4 = __ldg(src + 1);
+        mu = __ldg(P.mu + r);
+    };
+    if (v < v1) load();
+    for (uint32_t k = tid; k < (kHotWords + kWinWords) / 4u; k += kCountThreads) reinterpret_cast<uint4 *>(sm)[k] = make_uint4(0u, 0u, 0u, 0u);
+    if (tid < EP_NUM_TABLES) { range_from[tid] = 0; range_to[tid] = 0; }
+    const float s = P.s_from_state ? __ldcg(&P.state->s) : P.s;
+    __syncthreads();
+    uint32_t halves = 0, blocks = 0;
+    auto count_far = [&](uint32_t t, int32_t value) {          // outside the columns
+        const uint32_t w = uint32_t(value - kWinOrigin), g = uint32_t(value - kHistOrigin);
+        if (w < uint32_t(kWinBins)) {
+            atomicAdd(&win[t * kWinBins + w], 1u);
+        } else if (g < uint32_t(kHistBins)) {
+            atomicAdd(&P.hist[t * kHistBins + g], 1u);
+            atomicMax(&range_from[t], kHistBins - g);
+            atomicMax(&range_to[t], g + 1u);
+        } else {
+            P.state->overflow = 1;
+        }
+    };
+    while (v < v1) {
+        const float x[8] = {lo4.x, lo4.y, lo4.z, lo4.w, hi4.x, hi4.y, hi4.z, hi4.w};
+        const float m = mu;
+        const uint64_t here = v;
+        v += kCountThreads;
+        i += row_step;
+        col += col_step;
+        if (col >= P.per_row) { col -= P.per_row; ++i; }
+        if (v < v1) load();                                    // the next block is on its way while this one is worked on
+        int32_t z[8];
+        uint32_t half;
+        const float ms = __fmul_rn(m, s);
+        bool ok = quantise_fast(x, __frcp_rn(ms), z, half) && ms >= 1e-30f && ms <= 1e30f;
+        if (!ok) {
+            float xs[8];
+            int32_t zs[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) xs[k] = x[k];
+            const int c = quantise_exact(xs, m, s, zs);
+            if (c < 0) { P.state->overflow = 1; continue; }
+            half = uint32_t(c);
+#pragma unroll
+            for (int k = 0; k < 8; ++k) z[k] = zs[k];
+        }
+        // Eq. 4: m = (z8 - parity of z1 + ... + z7) / 2
+        z[7] = (z[7] - ((z[0] ^ z[1] ^ z[2] ^ z[3] ^ z[4] ^ z[5] ^ z[6]) & 1)) >> 1;
+        if (P.fields) {
+            auto two = [](int32_t a, int32_t b) { return (uint32_t(a) & 0xFFFFu) | (uint32_t(b) << 16); };
+            P.fields[here] = make_uint4(two(z[0], z[1]), two(z[2], z[3]), two(z[4], z[5]), two(z[6], 2 * z[7] + int32_t(half)));
+        }
+        ++blocks;
+        halves += half;
+        uint32_t *const column = hot + half * (8u * kHotBins * 32u) + lane;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            const uint32_t u = uint32_t(z[k] - kHotOrigin);
+            if (u < uint32_t(kHotBins)) atomicAdd(column + (uint32_t(k) * kHotBins + u) * 32u, 1u);
+            else count_far(1u + 8u * half + uint32_t(k), z[k]);
+        }
+    }
+    // the coset table
+    blocks = warp_sum(blocks);
+    halves = warp_sum(halves);
+    if (lane == 0) {
+        if (blocks != halves) atomicAdd(&win[0 - kWinOrigin], blocks - halves);
+        if (halves) atomicAdd(&win[1 - kWinOrigin], halves);
+    }
+    __syncthreads();
+    // columns into the window (one thread per value), then the window into global memory
+    for (uint32_t k = tid; k < 16u * kHotBins; k += kCountThreads) {
+        uint32_t n = 0;
+#pragma unroll
+        for (uint32_t j = 0; j < 32; ++j) n += hot[32u * k + ((j + tid) & 31u)];
+        if (n) atomicAdd(&win[(1u + k / kHotBins) * kWinBins + uint32_t(int32_t(k % kHotBins) + kHotOrigin - kWinOrigin)], n);
+    }
+    __syncthreads();
+    for (uint32_t k = tid; k < kWinWords; k += kCountThreads) {
+        const uint32_t n = win[k];
+        if (n) {
+            const uint32_t t = k / kWinBins, g = k % kWinBins + uint32_t(kWinOrigin - kHistOrigin);
+            atomicAdd(&P.hist[t * kHistBins + g], n);
+            atomicMax(&range_from[t], kHistBins - g);
+            atomicMax(&range_to[t], g + 1u);
+        }
+    }
+    __syncthreads();
+    if (tid < EP_NUM_TABLES && range_to[tid]) {
+        atomicMax(&P.state->from[tid], range_from[tid]);
+        atomicMax(&P.state->to[tid], range_to[tid]);
+    }
+    __threadfence();
+    __syncthreads();
+    if (tid == 0) last_cta = atomicAdd(&P.state->finished, 1u) == gridDim.x - 1u;
+    __syncthreads();
+    if (!last_cta) return;
+    __threadfence();
+    close_pass(P, sm);
+}
+
+// ---- Eq. 13: row scales ----------------------------------------------------------------------------------
+__device__ __forceinline__ int32_t field16(uint32_t w, int hi) { return hi ? int32_t(w) >> 16 : int32_t(w << 16) >> 16; }
+// 2 p of a block's eight weights (Eq. 5)
+__device__ __forceinline__ void twice_point(const uint4 q, int32_t (&p2)[8]) {
+    const int32_t mc = field16(q.w, 1), c = mc & 1;              // 2 m + c
     int32_t s7 = 0;
+    const uint32_t w[4] = {q.x, q.y, q.z, q.w};
 #pragma unroll
     for (int j = 0; j < 7; ++j) {
-        const double p = __dadd_rn(double(qv[1 + j]), half);
-        xp = __dadd_rn(xp, __dmul_rn(double(xv[j]), p));
-        pp = __dadd_rn(pp, __dmul_rn(p, p));
-        s7 += qv[1 + j];
+        const int32_t z = field16(w[j >> 1], j & 1);
+        s7 += z;
+        p2[j] = 2 * z + c;
     }
-    const double p8 = __dadd_rn(double(2 * qv[8] + (s7 & 1)), half);   // Eq. 5
-    xp = __dadd_rn(xp, __dmul_rn(double(xv[7]), p8));
-    pp = __dadd_rn(pp, __dmul_rn(p8, p8));
+    p2[7] = 2 * ((mc - c) + (s7 & 1)) + c;
 }
 __device__ __forceinline__ float refit_result(double xp, double pp, float s, float mu) {
     double sg;
@@ -221,155 +549,226 @@ __device__ __forceinline__ float refit_result(double xp, double pp, float s, flo
     return __double2float_rn(sg);
 }
 
-// rows streamed through shared memory (see row_rms_kernel); needs 16-byte aligned field rows: C a multiple of 64
-constexpr uint32_t kRefitBlocks = 16;                              // blocks per row and chunk
-constexpr uint32_t kRefitWStride = kRefitBlocks * 8 + 4;           // floats, padded
-constexpr uint32_t kRefitQStride = kRefitBlocks * 9 + 8;           // int16, padded, a multiple of 8
-__global__ void __launch_bounds__(kRowThreads) refit_kernel(const float *__restrict__ W, uint32_t R, uint32_t C,
-                                                            const int16_t *__restrict__ fields, float s,
-                                                            const float *__restrict__ mu, float *__restrict__ sigma) {
-    __shared__ __align__(16) float wbuf[kRowStages][kRowsPerCta][kRefitWStride];
-    __shared__ __align__(16) int16_t qbuf[kRowStages][kRowsPerCta][kRefitQStride];
-    const uint32_t tid = threadIdx.x, row0 = blockIdx.x * kRowsPerCta, per_row = C / 8;
-    const uint32_t chunks = (per_row + kRefitBlocks - 1) / kRefitBlocks;
-    // chunk c of the CTA's rows: per row up to 32 pieces of weights and 18 of fields, 16 bytes each
-    constexpr uint32_t kWPieces = kRefitBlocks * 2, kQPieces = kRefitBlocks * 18 / 16, kPieces = kWPieces + kQPieces;
-    auto issue = [&](uint32_t c) {
-        if (c < chunks) {
-            const uint32_t nb = min(kRefitBlocks, per_row - c * kRefitBlocks);     // blocks in this chunk: 16, or 8 at a row's end
-            for (uint32_t i = tid; i < kRowsPerCta * kPieces; i += kRowThreads) {
-                const uint32_t r = i / kPieces, j = i % kPieces;
-                if (row0 + r >= R) continue;
-                if (j < kWPieces) {
-                    if (j < 2 * nb) cp_async_16(&wbuf[c % kRowStages][r][4 * j], W + size_t(row0 + r) * C + size_t(c) * kRefitBlocks * 8 + 4 * j);
-                } else {
-                    const uint32_t k = j - kWPieces;
-                    if (16 * k < 18 * nb)
-                        cp_async_16(&qbuf[c % kRowStages][r][8 * k], fields + (size_t(row0 + r) * per_row + size_t(c) * kRefitBlocks) * 9 + 8 * k);
-                }
-            }
+// One row per CTA; see "sums over a row" above.  sum p^2 is exact in any order (multiples of 1/4 below 2^51).
+__global__ void __launch_bounds__(kRowThreads) refit_kernel(const float *__restrict__ W, uint32_t C, const uint4 *__restrict__ fields,
+                                                            float s, const float *__restrict__ mu, float *__restrict__ sigma) {
+    __shared__ double part[kRowThreads / 32];
+    __shared__ __align__(16) float4 wbuf[2 * kRowThreads];
+    __shared__ __align__(16) uint4 qbuf[kRowThreads];
+    const uint32_t tid = threadIdx.x, per_row = C / 8;
+    const float4 *x = reinterpret_cast<const float4 *>(W + size_t(blockIdx.x) * C);
+    const uint4 *q = fields + size_t(blockIdx.x) * per_row;
+    double xp = 0.0, pp4 = 0.0;                  // sum of x (2 p), sum of (2 p)^2
+    float mag = 0.0f;                            // sum |x (2 p)|, to 1e-4
+    for (uint32_t v = tid; v < per_row; v += kRowThreads) {
+        const float4 a = __ldg(x + 2u * v), b = __ldg(x + 2u * v + 1u);
+        int32_t p2[8], sq = 0;
+        twice_point(__ldg(q + v), p2);
+        const float xv[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            xp = __fma_rn(double(xv[j]), double(p2[j]), xp);         // (38-bit products: exact)
+            mag += fabsf(xv[j] * float(p2[j]));
+            sq += p2[j] * p2[j];                                     // at most 8 * 2^26
         }
-        cp_async_commit_group();
-    };
-    for (uint32_t c = 0; c + 1 < kRowStages; ++c) issue(c);
-    double xp = 0.0, pp = 0.0;
-    for (uint32_t c = 0; c < chunks; ++c) {
-        issue(c + kRowStages - 1);
-        cp_async_wait_group<kRowStages - 1>();
+        pp4 = __dadd_rn(pp4, double(sq));
+    }
+    xp = 0.5 * cta_sum(xp, part);
+    const double pp = 0.25 * cta_sum(pp4, part);
+    const double off = order_bound(C, 0.501 * cta_sum(double(mag), part));
+    const float m = __ldg(mu + blockIdx.x);
+    const float lo = refit_result(__dsub_rn(xp, off), pp, s, m), hi = refit_result(__dadd_rn(xp, off), pp, s, m);
+    if (lo == hi) {
+        if (tid == 0) sigma[blockIdx.x] = lo;
+        return;
+    }
+    xp = 0.0;                                    // index order
+    for (uint32_t v0 = 0; v0 < per_row; v0 += kRowThreads) {
         __syncthreads();
-        if (tid < kRowsPerCta && row0 + tid < R) {
-            const uint32_t nb = min(kRefitBlocks, per_row - c * kRefitBlocks);
-            const float *xw = &wbuf[c % kRowStages][tid][0];
-            const int16_t *q = &qbuf[c % kRowStages][tid][0];
-            for (uint32_t v = 0; v < nb; ++v) refit_block(xw + 8 * v, q + 9 * v, xp, pp);
+        if (v0 + tid < per_row) {
+            wbuf[2 * tid] = __ldg(x + 2u * (v0 + tid));
+            wbuf[2 * tid + 1] = __ldg(x + 2u * (v0 + tid) + 1u);
+            qbuf[tid] = __ldg(q + v0 + tid);
         }
-        __syncthreads();                     // the stage may be overwritten by the next issue
+        __syncthreads();
+        if (tid == 0)
+            for (uint32_t i = 0, n = min(kRowThreads, per_row - v0); i < n; ++i) {
+                const float4 a = wbuf[2 * i], b = wbuf[2 * i + 1];
+                int32_t p2[8];
+                twice_point(qbuf[i], p2);
+                const float xv[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+#pragma unroll
+                for (int j = 0; j < 8; ++j) xp = __dadd_rn(xp, __dmul_rn(double(xv[j]), 0.5 * double(p2[j])));
+            }
     }
-    if (tid < kRowsPerCta && row0 + tid < R) sigma[row0 + tid] = refit_result(xp, pp, s, mu[row0 + tid]);
+    if (tid == 0) sigma[blockIdx.x] = refit_result(xp, pp, s, m);
 }
 
-// the same for any C: one thread per row reading its own row
-__global__ void refit_rows_kernel(const float *__restrict__ W, uint32_t R, uint32_t C, const int16_t *__restrict__ fields, float s,
-                                  const float *__restrict__ mu, float *__restrict__ sigma) {
-    const uint32_t r = blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= R) return;
-    const uint32_t per_row = C / 8;
-    const float *x = W + size_t(r) * C;
-    const int16_t *q = fields + size_t(r) * per_row * 9;
-    double xp = 0.0, pp = 0.0;
-    for (uint32_t v = 0; v < per_row; ++v) {
-        float xv[8];
-        int16_t qv[9];
-#pragma unroll
-        for (int j = 0; j < 8; ++j) xv[j] = __ldg(x + 8 * v + j);
-#pragma unroll
-        for (int j = 0; j < 9; ++j) qv[j] = q[9 * v + j];
-        refit_block(xv, qv, xp, pp);
-    }
-    sigma[r] = refit_result(xp, pp, s, mu[r]);
-}
-
+// ---- tile coding (Sec. 3.6 / App. "Tiled rANS implementation", Eq. 17) ---------------------------------------
 struct EncodeTables {
-    int32_t tmin[EP_NUM_TABLES];
-    uint32_t off[EP_NUM_TABLES];     // start of table t inside the (f, F) array
+    int32_t base[EP_NUM_TABLES];     // entry of table t's value v: base[t] + v
     uint32_t total;                  // sum of K
 };
 
-// Sec. 3.6 / App. "Tiled rANS implementation": one warp per tile, one state per lane.  The decoder reads,
-// per (group, field), the words of the needy lanes in ascending lane order; the encoder walks groups and
-// fields backwards and fills the tile's word area from its end, writing each step's words as one block in
-// ascending lane order, which is the order the reversed word list of a sequential encoder would have.
-__global__ void __launch_bounds__(256) tile_encode_kernel(const int16_t *__restrict__ fields, uint32_t n_vec, uint32_t V,
-                                                          uint32_t n_tiles, uint32_t b, EncodeTables T,
-                                                          const uint32_t *__restrict__ fF, uint16_t *__restrict__ scratch,
-                                                          uint32_t cap, uint32_t *__restrict__ states,
-                                                          uint32_t *__restrict__ counts) {
-    extern __shared__ uint32_t tab[];    // per symbol: f | F << 16
-    for (uint32_t i = threadIdx.x; i < T.total; i += blockDim.x) tab[i] = fF[i];
-    __syncthreads();
-    const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
-    const uint32_t tile = blockIdx.x * (blockDim.x >> 5) + warp;
-    if (tile >= n_tiles) return;
-    const uint32_t v0 = tile * V;
-    const uint32_t nv = min(V, n_vec - v0);
-    const uint32_t lt = (1u << lane) - 1u;
-    uint16_t *area = scratch + size_t(tile) * cap;
-    uint32_t end = cap;                  // words [end, cap) of the area are written
-    uint32_t x = kStateLow;
-    const uint32_t groups = (nv + 31u) >> 5;
-    for (uint32_t g = groups; g-- > 0;) {
-        const uint32_t i = g * 32u + lane;
-        const bool act = i < nv;
-        const int16_t *q = fields + size_t(v0 + (act ? i : 0u)) * 9u;
-        const int c = act ? int(q[0]) : 0;
-        for (int k = 8; k >= 0; --k) {
-            uint32_t f = 1, F = 0;
-            bool emit = false;
-            if (act) {
-                const int t = k == 0 ? 0 : 1 + 8 * c + (k - 1);
-                const uint32_t sym = uint32_t(int32_t(q[k]) - T.tmin[t]);
-                const uint32_t e = tab[min(T.off[t] + sym, T.total - 1u)];   // in range by construction; clamped anyway
-                f = e & 0xFFFFu;
-                F = e >> 16;
-                emit = x >= (f << (31u - b));         // f * 2^(31-b) <= 2^31 fits 32 bits
-            }
-            const uint32_t bal = __ballot_sync(0xFFFFFFFFu, emit);
-            const uint32_t n = __popc(bal);
-            if (n > end) { end = 0; break; }          // cannot happen: at most one word per symbol fits the area
-            end -= n;
-            if (emit) {
-                area[end + __popc(bal & lt)] = uint16_t(x);
-                x >>= 16;
-            }
-            if (act) x = ((x / f) << b) + (x % f) + F;   // Eq. 17
-        }
-    }
-    states[size_t(tile) * 32u + lane] = x;
-    if (lane == 0) counts[tile] = cap - end;
+// What Eq. 17 needs of a symbol, without a division: x / f for x < 2^31 is umulhi(x, rcp) >> sh with
+// sh = ceil(log2 f) - 1 and rcp = ceil(2^(32 + sh) / f) (Granlund and Montgomery, "Division by invariant integers using
+// multiplication", 1994; exact for 31-bit x).  f = 1 takes rcp = 2^32 - 1, which gives x - 1, and an offset that
+// makes up for it.  With q = x / f the new state is q 2^b + x mod f + F = x + (2^b - f) q + F.
+__device__ __forceinline__ uint2 encode_entry(uint32_t f, uint32_t F, uint32_t b) {
+    const uint32_t M = 1u << b;
+    if (f <= 1u) return make_uint2(0xFFFFFFFFu, (M - 1u) | ((F + M - 1u) << 16));
+    const uint32_t sh = 31u - __clz(int(f - 1u));
+    // (the quotient has at most 32 integer bits and a fraction of at least 1 / f: its ceiling is right in double)
+    const uint32_t rcp = uint32_t(ceil(__ddiv_rn(double(1ull << (32u + sh)), double(f))));
+    return make_uint2(rcp, (M - f) | (F << 16));
 }
 
-// move every tile's words from the end of its area to its place in the payload
-__global__ void compact_kernel(const uint16_t *__restrict__ scratch, uint32_t cap, const uint32_t *__restrict__ counts,
-                               const uint32_t *__restrict__ offsets, uint32_t n_tiles, uint16_t *__restrict__ payload) {
+// One warp per tile, one state per lane.  The decoder reads, per (group, field), the words of the needy lanes in
+// ascending lane order; the encoder walks groups and fields backwards and fills the tile's word area from its end, writing
+// each step's words as one block in ascending lane order, which is the order the reversed word list of a sequential
+// encoder would have.  A step's chain is compare, shift, multiply-high, shift, multiply-add (about 30 cycles);
+// a group's symbols are loaded one group ahead and looked up before the steps that need them.
+// IN_SMEM: the entries in shared memory (up to 24 Ki symbols), else in global memory.  A CTA has four warps - tiles spread
+// over the SMs - or sixteen where its table takes so much shared memory that few CTAs fit an SM.
+constexpr uint32_t kTileThreads = 128, kTileThreadsMax = 512, kSmemEntries = 24576;
+
+template <bool IN_SMEM>
+__global__ void __launch_bounds__(kTileThreadsMax) tile_encode_kernel(const uint4 *__restrict__ fields, uint32_t n_vec, uint32_t V,
+                                                                      uint32_t n_tiles, uint32_t b, const __grid_constant__ EncodeTables T,
+                                                                      const uint32_t *__restrict__ fF, uint2 *__restrict__ entries_global,
+                                                                      uint16_t *__restrict__ scratch, uint32_t cap,
+                                                                      uint32_t *__restrict__ index, uint32_t *__restrict__ counts, SearchState *state) {
+    extern __shared__ __align__(8) uint2 entries_smem[];
+    __shared__ uint32_t last_cta, part[kTileThreadsMax];
+    const uint32_t tid = threadIdx.x, lane = tid & 31u;
+    if (IN_SMEM) {
+        for (uint32_t i = tid; i < T.total; i += blockDim.x) {
+            const uint32_t e = __ldg(fF + i);
+            entries_smem[i] = encode_entry(e & 0xFFFFu, e >> 16, b);
+        }
+        __syncthreads();
+    }
+    const uint2 *const entries = IN_SMEM ? entries_smem : entries_global;
+    const uint32_t tile = blockIdx.x * (blockDim.x >> 5) + (tid >> 5);
+    if (tile < n_tiles) {
+        const uint32_t v0 = tile * V, nv = min(V, n_vec - v0), lt = (1u << lane) - 1u, last_entry = T.total - 1u;
+        const uint4 *const q = fields + v0;
+        uint16_t *const area = scratch + size_t(tile) * cap;
+        uint32_t end = cap;                      // words [end, cap) of the area are written
+        uint32_t x = kStateLow;
+        const uint32_t groups = (nv + 31u) >> 5;
+        const uint32_t M = 1u << b, top = 31u - b;
+        uint4 next = __ldg(q + min((groups - 1u) * 32u + lane, nv - 1u));
+        for (uint32_t g = groups; g-- > 0;) {
+            const uint4 cur = next;
+            const bool act = g * 32u + lane < nv;
+            if (g) next = __ldg(q + (g - 1u) * 32u + lane);
+            const int32_t mc = field16(cur.w, 1), c = mc & 1;
+            const uint32_t w[4] = {cur.x, cur.y, cur.z, cur.w};
+            uint2 e[9];
+            // (every index is in range by construction; clamped anyway)
+            e[0] = entries[min(uint32_t(T.base[0] + c), last_entry)];
+#pragma unroll
+            for (int k = 1; k < 8; ++k)
+                e[k] = entries[min(uint32_t((c ? T.base[8 + k] : T.base[k]) + field16(w[(k - 1) >> 1], (k - 1) & 1)), last_entry)];
+            e[8] = entries[min(uint32_t((c ? T.base[16] : T.base[8]) + (mc >> 1)), last_entry)];
+#pragma unroll
+            for (int k = 8; k >= 0; --k) {
+                const uint32_t comp = e[k].y & 0xFFFFu, f = M - comp;                      // 2^b - f
+                const uint32_t sh = f > 1u ? 31u - __clz(int(f - 1u)) : 0u;
+                const bool emit = act && x >= (f << top);                                // f 2^(31-b) <= 2^31 fits 32 bits
+                const uint32_t bal = __ballot_sync(0xFFFFFFFFu, emit);
+                end -= __popc(bal);                                                      // at most nine words per block: the area holds them
+                if (emit) {
+                    area[end + __popc(bal & lt)] = uint16_t(x);
+                    x >>= 16;
+                }
+                const uint32_t quot = __umulhi(x, e[k].x) >> sh;
+                if (act) x = quot * comp + (x + (e[k].y >> 16));                         // Eq. 17
+            }
+        }
+        index[size_t(tile) * 33u + lane] = x;
+        if (lane == 0) counts[tile] = cap - end;
+    }
+    // the last CTA turns the counts into offsets (the tile records' last words and the final one)
+    __threadfence();
+    __syncthreads();
+    if (tid == 0) last_cta = atomicAdd(&state->tiles_done, 1u) == gridDim.x - 1u;
+    __syncthreads();
+    if (!last_cta) return;
+    __threadfence();
+    const uint32_t per = (n_tiles + blockDim.x - 1u) / blockDim.x;
+    const uint32_t t0 = min(tid * per, n_tiles), t1 = min(t0 + per, n_tiles);
+    uint32_t sum = 0;
+    for (uint32_t t = t0; t < t1; ++t) sum += __ldcg(counts + t);
+    part[tid] = sum;
+    __syncthreads();
+    for (uint32_t d = 1; d < blockDim.x; d <<= 1) {
+        const uint32_t add = tid >= d ? part[tid - d] : 0u;
+        __syncthreads();
+        part[tid] += add;
+        __syncthreads();
+    }
+    uint32_t at = part[tid] - sum;
+    for (uint32_t t = t0; t < t1; ++t) { index[size_t(t) * 33u + 32u] = at; at += __ldcg(counts + t); }
+    if (tid == blockDim.x - 1u) {
+        index[size_t(n_tiles) * 33u] = part[tid];
+        state->total_words = part[tid];
+    }
+}
+
+// entries of an alphabet too large for shared memory
+__global__ void encode_entries_kernel(const uint32_t *__restrict__ fF, uint32_t n, uint32_t b, uint2 *__restrict__ entries) {
+    const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < n) entries[i] = encode_entry(fF[i] & 0xFFFFu, fF[i] >> 16, b);
+}
+
+// move every tile's words from the end of its area to its place in the payload: one warp per tile, four bytes per lane
+// where the destination is aligned for it
+__global__ void __launch_bounds__(256) compact_kernel(const uint16_t *__restrict__ scratch, uint32_t cap, const uint32_t *__restrict__ counts,
+                                                      const uint32_t *__restrict__ index, uint32_t n_tiles, uint16_t *__restrict__ payload) {
     const uint32_t lane = threadIdx.x & 31u;
     const uint32_t tile = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (tile >= n_tiles) return;
-    const uint32_t n = counts[tile];
+    uint32_t n = counts[tile];
     const uint16_t *src = scratch + size_t(tile) * cap + (cap - n);
-    uint16_t *dst = payload + offsets[tile];
-    for (uint32_t i = lane; i < n; i += 32u) dst[i] = src[i];
+    uint16_t *dst = payload + index[size_t(tile) * 33u + 32u];
+    if (n && (reinterpret_cast<uintptr_t>(dst) & 2)) {
+        if (lane == 0) *dst = *src;
+        ++src; ++dst; --n;
+    }
+    uint32_t *const d32 = reinterpret_cast<uint32_t *>(dst);
+    const uint32_t pairs = n / 2u;
+    if (reinterpret_cast<uintptr_t>(src) & 2) {
+        // each pair straddles two aligned words (the one before src starts inside the buffer, as src is not its start)
+        const uint32_t *s32 = reinterpret_cast<const uint32_t *>(src - 1);
+#pragma unroll 4
+        for (uint32_t i = lane; i < pairs; i += 32u) d32[i] = __funnelshift_r(s32[i], s32[i + 1u], 16);
+    } else {
+        const uint32_t *s32 = reinterpret_cast<const uint32_t *>(src);
+#pragma unroll 4
+        for (uint32_t i = lane; i < pairs; i += 32u) d32[i] = s32[i];
+    }
+    if ((n & 1u) && lane == 0) dst[n - 1u] = src[n - 1u];
 }
 
 size_t align_up(size_t v) { return (v + 255) & ~size_t(255); }
 
 struct Workspace {
-    float *mu, *sigma;
-    uint32_t *rows, *hist, *states, *counts, *offsets, *fF;
-    int *overflow;
-    int16_t *fields;
-    uint16_t *scratch, *payload;
+    float *mu;
+    uint32_t *rows, *hist, *counts, *fF, *last_counts, *full_counts;
+    SearchState *state;
+    uint2 *entries;
+    uint4 *fields;
+    uint16_t *scratch;
+    // the last three sections of the blob, back to back as they are stored: row scales, tile index, payload
+    float *sigma;
+    uint32_t *index;
+    uint16_t *payload;
     size_t bytes;
 };
+
+constexpr size_t kHistBytes = 4ull * EP_NUM_TABLES * kHistBins;
 
 Workspace carve(uint8_t *base, uint32_t R, uint32_t C, uint32_t V) {
     const uint64_t nvec = uint64_t(R) * (C / 8);
@@ -379,17 +778,23 @@ Workspace carve(uint8_t *base, uint32_t R, uint32_t C, uint32_t V) {
     auto take = [&](size_t n) { uint8_t *p = base ? base + at : nullptr; at += align_up(n); return p; };
     Workspace w{};
     w.mu = reinterpret_cast<float *>(take(4ull * R));
-    w.sigma = reinterpret_cast<float *>(take(4ull * R));
     w.rows = reinterpret_cast<uint32_t *>(take(4ull * R));
-    w.hist = reinterpret_cast<uint32_t *>(take(4ull * EP_NUM_TABLES * kHistBins));
-    w.overflow = reinterpret_cast<int *>(take(4));
+    // state, then the counts of the last step, so that one copy brings both; histogram after them
+    w.state = reinterpret_cast<SearchState *>(take(kStateBytes + 4ull * kEvalSymbols));
+    w.last_counts = reinterpret_cast<uint32_t *>(reinterpret_cast<uint8_t *>(w.state) + kStateBytes);
+    w.hist = reinterpret_cast<uint32_t *>(take(kHistBytes));
+    w.full_counts = reinterpret_cast<uint32_t *>(take(kHistBytes));
     w.fF = reinterpret_cast<uint32_t *>(take(4ull * kMaxTableSymbols));
-    w.states = reinterpret_cast<uint32_t *>(take(128ull * n_tiles));
+    w.entries = reinterpret_cast<uint2 *>(take(8ull * kMaxTableSymbols));
     w.counts = reinterpret_cast<uint32_t *>(take(4ull * n_tiles));
-    w.offsets = reinterpret_cast<uint32_t *>(take(4ull * (n_tiles + 1)));
-    w.fields = reinterpret_cast<int16_t *>(take(18ull * nvec));
-    w.scratch = reinterpret_cast<uint16_t *>(take(2ull * cap * n_tiles));
-    w.payload = reinterpret_cast<uint16_t *>(take(2ull * cap * n_tiles));
+    w.fields = reinterpret_cast<uint4 *>(take(16ull * nvec));
+    w.scratch = reinterpret_cast<uint16_t *>(take(2ull * cap * n_tiles + 4));
+    uint8_t *tail = take(4ull * R + uint64_t(kTileRecordBytes) * n_tiles + 4 + 2ull * cap * n_tiles);
+    w.sigma = reinterpret_cast<float *>(tail);
+    if (base) {
+        w.index = reinterpret_cast<uint32_t *>(tail + 4ull * R);
+        w.payload = reinterpret_cast<uint16_t *>(tail + 4ull * R + uint64_t(kTileRecordBytes) * n_tiles + 4);
+    }
     w.bytes = at;
     return w;
 }
@@ -399,7 +804,7 @@ Workspace carve(uint8_t *base, uint32_t R, uint32_t C, uint32_t V) {
         if ((call) != cudaSuccess) return EP_ERR_CUDA; \
     } while (0)
 
-// Page-locked host memory: for finished blobs and for the histograms that come back after every counting pass.
+// Page-locked host memory: for finished blobs and for the counts that come back after a search or a counting pass.
 // Locking memory costs milliseconds, so each of the two uses keeps the buffer it last gave back (one at most, the
 // larger one when two compete) for the next request that fits into it.
 struct PinnedSlot {
@@ -437,7 +842,7 @@ struct PinnedSlot {
         if (drop) cudaFreeHost(drop);
     }
 };
-PinnedSlot g_blob_slot, g_hist_slot;
+PinnedSlot g_blob_slot, g_mail_slot;
 
 // headroom for blobs: the next tensor of a model is rarely the same size
 uint8_t *pinned_acquire(size_t n, size_t *cap) { return g_blob_slot.acquire(n, n / 8 + 4096, cap); }
@@ -447,89 +852,157 @@ class DeviceBackend final : public EncodeBackend {
 public:
     DeviceBackend(const float *dW, uint32_t R, uint32_t C, uint32_t V, uint8_t *ws, cudaStream_t st)
         : W_(dW), R_(R), C_(C), V_(V), w_(carve(ws, R, C, V)), st_(st) {
-        hist_ = reinterpret_cast<uint32_t *>(g_hist_slot.acquire(kHistBytes, 0, &hist_cap_));
-        if (!hist_) throw std::bad_alloc();
+        mail_ = g_mail_slot.acquire(kMailBytes, 0, &mail_cap_);
+        if (!mail_) throw std::bad_alloc();
     }
-    ~DeviceBackend() override { if (hist_) g_hist_slot.release(reinterpret_cast<uint8_t *>(hist_), hist_cap_); }
+    ~DeviceBackend() override { if (mail_) g_mail_slot.release(mail_, mail_cap_); }
 
     int prepare(const std::vector<uint32_t> &sample) override {
         n_sample_ = uint32_t(sample.size());
+        int dev = 0;
+        EP_CUDA(cudaGetDevice(&dev));
+        EP_CUDA(cudaDeviceGetAttribute(&sms_, cudaDevAttrMultiProcessorCount, dev));
+        EP_CUDA(cudaFuncSetAttribute(quantise_count_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kCountSmem)));
         EP_CUDA(cudaMemcpyAsync(w_.rows, sample.data(), 4ull * n_sample_, cudaMemcpyHostToDevice, st_));
-        row_rms_kernel<<<(R_ + kRowsPerCta - 1) / kRowsPerCta, kRowThreads, 0, st_>>>(W_, R_, C_, w_.mu);
+        EP_CUDA(cudaMemsetAsync(w_.state, 0, kStateBytes, st_));
+        EP_CUDA(cudaMemsetAsync(w_.hist, 0, kHistBytes, st_));       // every pass leaves it zero again
+        row_rms_kernel<<<R_, kRowThreads, 0, st_>>>(W_, C_, w_.mu);
         EP_CUDA(cudaGetLastError());
         return EP_OK;
     }
     int count_sample(float s, Model &m) override { return count(w_.rows, n_sample_, s, nullptr, m); }
     int count_full(float s, Model &m) override { return count(nullptr, R_, s, w_.fields, m); }
 
+    int search(const SearchJob &job, const ep_encode_opts &o, SearchResult &r, bool *done) override {
+        *done = false;
+        EP_CUDA(cudaMemsetAsync(w_.state, 0, kStateBytes, st_));
+        CountParams P = params(w_.rows, n_sample_, float(std::sqrt(o.bracket_lo * o.bracket_hi)), nullptr);
+        const double n_tile = double((job.sample_vectors + job.V - 1) / job.V);
+        P.step = {job.target_bpp, o.retained_bits * double(kStates) * n_tile,
+                  n_tile * (32.0 * kStates + 32.0) + 32.0 + 32.0 * double(job.sample_rows) + 8.0 * kHeaderBytes,
+                  8.0 * double(job.sample_vectors), 9.0 * double(job.sample_vectors), o.bracket_lo, o.bracket_hi, job.b, 0};
+        for (int it = 0; it < o.search_steps; ++it) {
+            P.step.step = it;
+            P.s_from_state = it > 0;
+            launch_count(P);
+        }
+        CountParams F = params(nullptr, R_, P.s, w_.fields);
+        F.s_from_state = o.search_steps > 0;
+        launch_count(F);
+        EP_CUDA(cudaGetLastError());
+        const int rc = fetch(true);
+        if (rc) return rc;
+        const SearchState &S = *state();
+        if (S.undecided || S.has_last == 2) return EP_OK;
+        r.s = o.search_steps > 0 ? S.s : P.s;
+        r.has_last = S.has_last != 0;
+        if (r.has_last) r.last.from_counts(S.last.lo, S.last.K, last_counts());
+        r.full.from_counts(S.full.lo, S.full.K, full_counts());
+        *done = true;
+        return EP_OK;
+    }
+
     int finish(float s, int b, uint32_t V, const Model &m, ep_blob *out) override {
         const uint64_t nvec = uint64_t(R_) * (C_ / 8);
         const uint32_t n_tiles = uint32_t((nvec + V - 1) / V);
         const uint32_t cap = 9u * V;
-        if (C_ % 64 == 0 && (reinterpret_cast<uintptr_t>(w_.fields) & 15) == 0)
-            refit_kernel<<<(R_ + kRowsPerCta - 1) / kRowsPerCta, kRowThreads, 0, st_>>>(W_, R_, C_, w_.fields, s, w_.mu, w_.sigma);
-        else
-            refit_rows_kernel<<<(R_ + 63) / 64, 64, 0, st_>>>(W_, R_, C_, w_.fields, s, w_.mu, w_.sigma);
-        EP_CUDA(cudaGetLastError());
         EncodeTables T{};
         std::vector<uint32_t> fF;
         for (int t = 0; t < EP_NUM_TABLES; ++t) {
-            T.tmin[t] = m.t[t].lo;
-            T.off[t] = uint32_t(fF.size());
+            T.base[t] = int32_t(fF.size()) - m.t[t].lo;
             for (uint32_t j = 0; j < m.t[t].K(); ++j) fF.push_back(m.t[t].f[j] | (m.t[t].F[j] << 16));
         }
         T.total = uint32_t(fF.size());
         if (T.total > kMaxTableSymbols) return EP_ERR_UNSUPPORTED;
         EP_CUDA(cudaMemcpyAsync(w_.fF, fF.data(), 4ull * fF.size(), cudaMemcpyHostToDevice, st_));
-        const size_t smem = 4ull * T.total;
-        if (smem > 48u * 1024u)
-            EP_CUDA(cudaFuncSetAttribute(tile_encode_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
-        tile_encode_kernel<<<(n_tiles + 7) / 8, 256, smem, st_>>>(w_.fields, uint32_t(nvec), V, n_tiles, uint32_t(b), T, w_.fF,
-                                                                  w_.scratch, cap, w_.states, w_.counts);
+        EP_CUDA(cudaMemsetAsync(&w_.state->tiles_done, 0, 4, st_));
+        if (T.total <= kSmemEntries) {
+            const size_t smem = 8ull * T.total;
+            const uint32_t threads = T.total <= 4096u ? kTileThreads : kTileThreadsMax;
+            if (smem > 40u * 1024u)      // (always the same limit: another thread's call must not lower it before the launch)
+                EP_CUDA(cudaFuncSetAttribute(tile_encode_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(8u * kSmemEntries)));
+            tile_encode_kernel<true><<<(n_tiles + threads / 32u - 1u) / (threads / 32u), threads, smem, st_>>>(
+                w_.fields, uint32_t(nvec), V, n_tiles, uint32_t(b), T, w_.fF, w_.entries, w_.scratch, cap, w_.index, w_.counts, w_.state);
+        } else {
+            encode_entries_kernel<<<(T.total + 255u) / 256u, 256, 0, st_>>>(w_.fF, T.total, uint32_t(b), w_.entries);
+            tile_encode_kernel<false><<<(n_tiles + kTileThreads / 32u - 1u) / (kTileThreads / 32u), kTileThreads, 0, st_>>>(
+                w_.fields, uint32_t(nvec), V, n_tiles, uint32_t(b), T, w_.fF, w_.entries, w_.scratch, cap, w_.index, w_.counts, w_.state);
+        }
+        compact_kernel<<<(n_tiles + 7) / 8, 256, 0, st_>>>(w_.scratch, cap, w_.counts, w_.index, n_tiles, w_.payload);
+        EP_CUDA(cudaMemcpyAsync(&state()->total_words, &w_.state->total_words, 4, cudaMemcpyDeviceToHost, st_));
+        refit_kernel<<<R_, kRowThreads, 0, st_>>>(W_, C_, w_.fields, s, w_.mu, w_.sigma);
         EP_CUDA(cudaGetLastError());
-        std::vector<uint32_t> counts(n_tiles), offsets(n_tiles + 1, 0);
-        EP_CUDA(cudaMemcpyAsync(counts.data(), w_.counts, 4ull * n_tiles, cudaMemcpyDeviceToHost, st_));
         EP_CUDA(cudaStreamSynchronize(st_));
-        uint64_t total = 0;
-        for (uint32_t t = 0; t < n_tiles; ++t) { offsets[t] = uint32_t(total); total += counts[t]; }
-        offsets[n_tiles] = uint32_t(total);
+        const uint64_t total = state()->total_words;
         if (total >= (1ull << 31)) return EP_ERR_UNSUPPORTED;
-        EP_CUDA(cudaMemcpyAsync(w_.offsets, offsets.data(), 4ull * (n_tiles + 1), cudaMemcpyHostToDevice, st_));
-        compact_kernel<<<(n_tiles + 7) / 8, 256, 0, st_>>>(w_.scratch, cap, w_.counts, w_.offsets, n_tiles, w_.payload);
-        EP_CUDA(cudaGetLastError());
-        std::vector<uint32_t> states(size_t(n_tiles) * 32);
-        std::vector<float> sigma(R_);
-        EP_CUDA(cudaMemcpyAsync(states.data(), w_.states, 128ull * n_tiles, cudaMemcpyDeviceToHost, st_));
-        EP_CUDA(cudaMemcpyAsync(sigma.data(), w_.sigma, 4ull * R_, cudaMemcpyDeviceToHost, st_));
-        EP_CUDA(cudaStreamSynchronize(st_));
-        // everything but the payload is laid out on the host; the compacted payload is copied straight into its place
-        uint64_t payload_at = 0;
+        // header and tables are laid out on the host; the other sections are copied straight into their place
         out->acquire = pinned_acquire;
         out->release = pinned_release;
-        const int rc = assemble_blob(m, R_, C_, b, V, sigma.data(), s, states.data(), nullptr, counts.data(), out, &payload_at);
+        BlobLayout L;
+        const int rc = begin_blob(m, R_, C_, b, V, s, total, out, &L);
         if (rc) return rc;
-        if (total) {
-            EP_CUDA(cudaMemcpyAsync(out->data() + payload_at, w_.payload, 2ull * total, cudaMemcpyDeviceToHost, st_));
-            EP_CUDA(cudaStreamSynchronize(st_));
-        }
+        EP_CUDA(cudaMemcpyAsync(out->data() + L.off_scales, w_.sigma, L.total - L.off_scales, cudaMemcpyDeviceToHost, st_));
+        EP_CUDA(cudaStreamSynchronize(st_));
         return EP_OK;
     }
 
 private:
-    int count(const uint32_t *rows, uint32_t n_rows, float s, int16_t *fields, Model &m) {
-        EP_CUDA(cudaMemsetAsync(w_.hist, 0, 4ull * EP_NUM_TABLES * kHistBins, st_));
-        EP_CUDA(cudaMemsetAsync(w_.overflow, 0, 4, st_));
-        const uint64_t n = uint64_t(n_rows) * (C_ / 8);
-        const uint64_t want = (n + 255) / 256;
-        const uint32_t grid = uint32_t(std::min<uint64_t>(want, 148u * 16u));
-        quantise_count_kernel<<<grid, 256, 0, st_>>>(W_, C_, w_.mu, rows, n, s, fields, w_.hist, w_.overflow);
-        EP_CUDA(cudaGetLastError());
-        int overflow = 0;
-        EP_CUDA(cudaMemcpyAsync(hist_, w_.hist, kHistBytes, cudaMemcpyDeviceToHost, st_));
-        EP_CUDA(cudaMemcpyAsync(&overflow, w_.overflow, 4, cudaMemcpyDeviceToHost, st_));
+    // mail: state, counts of the last step, counts of the full pass
+    static constexpr size_t kMailBytes = kStateBytes + 4ull * kEvalSymbols + kHistBytes;
+    SearchState *state() { return reinterpret_cast<SearchState *>(mail_); }
+    uint32_t *last_counts() { return reinterpret_cast<uint32_t *>(mail_ + kStateBytes); }
+    uint32_t *full_counts() { return last_counts() + kEvalSymbols; }
+
+    CountParams params(const uint32_t *rows, uint32_t n_rows, float s, uint4 *fields) {
+        CountParams P{};
+        P.W = W_;
+        P.mu = w_.mu;
+        P.rows = rows;
+        P.fields = fields;
+        P.hist = w_.hist;
+        P.state = w_.state;
+        P.last_counts = w_.last_counts;
+        P.full_counts = w_.full_counts;
+        P.per_row = C_ / 8;
+        P.n_blocks = uint64_t(n_rows) * P.per_row;
+        P.C = C_;
+        P.s = s;
+        P.step.step = -1;
+        return P;
+    }
+    void launch_count(const CountParams &P) {
+        const uint32_t grid = uint32_t(std::min<uint64_t>((P.n_blocks + 255) / 256, uint64_t(sms_)));
+        quantise_count_kernel<<<grid, kCountThreads, kCountSmem, st_>>>(P);
+    }
+    static size_t symbols(const CountDir &D) {
+        size_t n = 0;
+        for (uint32_t k : D.K) n += k;
+        return n;
+    }
+    // state and counts to the host: most alphabets fit the first copy
+    int fetch(bool last) {
+        EP_CUDA(cudaMemcpyAsync(mail_, w_.state, kStateBytes + (last ? 4ull * kFirstCounts : 0), cudaMemcpyDeviceToHost, st_));
+        EP_CUDA(cudaMemcpyAsync(full_counts(), w_.full_counts, 4ull * kFirstCounts, cudaMemcpyDeviceToHost, st_));
         EP_CUDA(cudaStreamSynchronize(st_));
-        if (overflow) return EP_ERR_UNSUPPORTED;     // a coordinate beyond +-4095: use the host encoder
-        m.from_histograms(hist_, kHistBins, kHistOrigin);
+        const SearchState &S = *state();
+        if (S.overflow) return EP_ERR_UNSUPPORTED;     // a coordinate beyond +-4095: use the host encoder
+        bool more = false;
+        auto rest = [&](uint32_t *to, const uint32_t *from, size_t n) {
+            if (n <= kFirstCounts) return cudaSuccess;
+            more = true;
+            return cudaMemcpyAsync(to + kFirstCounts, from + kFirstCounts, 4ull * (n - kFirstCounts), cudaMemcpyDeviceToHost, st_);
+        };
+        if (last && S.has_last == 1) EP_CUDA(rest(last_counts(), w_.last_counts, symbols(S.last)));
+        EP_CUDA(rest(full_counts(), w_.full_counts, symbols(S.full)));
+        if (more) EP_CUDA(cudaStreamSynchronize(st_));
+        return EP_OK;
+    }
+    int count(const uint32_t *rows, uint32_t n_rows, float s, uint4 *fields, Model &m) {
+        launch_count(params(rows, n_rows, s, fields));
+        EP_CUDA(cudaGetLastError());
+        const int rc = fetch(false);
+        if (rc) return rc;
+        m.from_counts(state()->full.lo, state()->full.K, full_counts());
         return EP_OK;
     }
 
@@ -537,9 +1010,9 @@ private:
     uint32_t R_, C_, V_;
     Workspace w_;
     cudaStream_t st_;
-    static constexpr size_t kHistBytes = 4ull * EP_NUM_TABLES * kHistBins;
-    uint32_t *hist_ = nullptr;       // page-locked: the copy back after each counting pass is a plain DMA
-    size_t hist_cap_ = 0;
+    int sms_ = 0;
+    uint8_t *mail_ = nullptr;        // page-locked: the copies back are plain DMA
+    size_t mail_cap_ = 0;
     uint32_t n_sample_ = 0;
 };
 

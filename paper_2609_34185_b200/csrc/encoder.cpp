@@ -98,17 +98,14 @@ void Model::count(const int32_t *fld, uint64_t nvec, int threads) {
         }
 }
 
-void Model::from_histograms(const uint32_t *hist, uint32_t bins, int32_t origin) {
+void Model::from_counts(const int32_t *lo, const uint32_t *K, const uint32_t *counts) {
     for (int i = 0; i < EP_NUM_TABLES; ++i) {
-        const uint32_t *h = hist + size_t(i) * bins;
-        uint32_t first = bins, last = 0;
-        for (uint32_t j = 0; j < bins; ++j)
-            if (h[j]) { if (first == bins) first = j; last = j; }
         t[i] = Table();
-        if (first == bins) continue;
-        t[i].lo = origin + int32_t(first);
-        t[i].n.assign(h + first, h + last + 1);
+        if (!K[i]) continue;
+        t[i].lo = lo[i];
+        t[i].n.assign(counts, counts + K[i]);
         for (uint64_t c : t[i].n) t[i].total += c;
+        counts += K[i];
     }
 }
 
@@ -205,14 +202,10 @@ std::vector<uint32_t> sample_rows(uint32_t R, uint32_t C, uint32_t budget_vector
     return idx;
 }
 
-// header + tables + scales + tile index + payload
-int assemble_blob(const Model &m, uint32_t R, uint32_t C, int b, uint32_t V, const float *sigma, float s_info,
-                  const uint32_t *states, const uint16_t *const *tile_words, const uint32_t *tile_len, ep_blob *out,
-                  uint64_t *payload_offset) {
+int begin_blob(const Model &m, uint32_t R, uint32_t C, int b, uint32_t V, float s_info, uint64_t total_words, ep_blob *out,
+               BlobLayout *at) {
     const uint64_t nvec = uint64_t(R) * (C / 8);
     const uint32_t n_tiles = uint32_t((nvec + V - 1) / V);
-    uint64_t total_words = 0;
-    for (uint32_t t = 0; t < n_tiles; ++t) total_words += tile_len[t];
     // coordinate range of z_1..z_8 (z_8 = 2m + parity spans [2 m_lo, 2 m_hi + 1])
     bool any = false;
     int64_t cmin = 0, cmax = 0;
@@ -231,10 +224,10 @@ int assemble_blob(const Model &m, uint32_t R, uint32_t C, int b, uint32_t V, con
     const uint64_t off_tables = kHeaderBytes, off_scales = off_tables + tb_bytes, off_tiles = off_scales + 4ull * R;
     const uint64_t off_payload = off_tiles + uint64_t(kTileRecordBytes) * n_tiles + 4, total = off_payload + 2 * total_words;
     if (total >= (1ull << 32)) return EP_ERR_UNSUPPORTED;   // section offsets are 32-bit
-    uint8_t *p = out->allocate(size_t(total));   // uninitialised: everything before the payload is zeroed here,
-    if (!p) return EP_ERR_NOMEM;                 // the payload is written whole below or by the caller
-    std::memset(p, 0, size_t(off_payload));
-    if (payload_offset) *payload_offset = off_payload;
+    uint8_t *p = out->allocate(size_t(total));   // uninitialised: header and tables are zeroed here, the rest is
+    if (!p) return EP_ERR_NOMEM;                 // written whole by the caller
+    std::memset(p, 0, size_t(off_scales));
+    *at = {off_tables, off_scales, off_tiles, off_payload, total};
     store_le<uint32_t>(p, kMagic);
     store_le<uint16_t>(p + 4, 1);
     p[6] = uint8_t(b);
@@ -259,16 +252,30 @@ int assemble_blob(const Model &m, uint32_t R, uint32_t C, int b, uint32_t V, con
         store_le<uint32_t>(dir + 4 * EP_NUM_TABLES + 4 * i, m.t[i].K());
         for (uint32_t j = 0; j < m.t[i].K(); ++j, fq += 2) store_le<uint16_t>(fq, uint16_t(m.t[i].f[j]));
     }
-    std::memcpy(p + off_scales, sigma, 4ull * R);
+    return EP_OK;
+}
+
+// header + tables + scales + tile index + payload
+int assemble_blob(const Model &m, uint32_t R, uint32_t C, int b, uint32_t V, const float *sigma, float s_info,
+                  const uint32_t *states, const uint16_t *const *tile_words, const uint32_t *tile_len, ep_blob *out) {
+    const uint64_t nvec = uint64_t(R) * (C / 8);
+    const uint32_t n_tiles = uint32_t((nvec + V - 1) / V);
+    uint64_t total_words = 0;
+    for (uint32_t t = 0; t < n_tiles; ++t) total_words += tile_len[t];
+    BlobLayout L;
+    const int rc = begin_blob(m, R, C, b, V, s_info, total_words, out, &L);
+    if (rc) return rc;
+    uint8_t *p = out->data();
+    std::memcpy(p + L.off_scales, sigma, 4ull * R);
     uint64_t at = 0;
     for (uint32_t t = 0; t < n_tiles; ++t) {
-        uint8_t *rec = p + off_tiles + uint64_t(kTileRecordBytes) * t;
+        uint8_t *rec = p + L.off_tiles + uint64_t(kTileRecordBytes) * t;
         std::memcpy(rec, states + size_t(t) * kStates, 4 * kStates);
         store_le<uint32_t>(rec + 4 * kStates, uint32_t(at));
-        if (tile_words && tile_len[t]) std::memcpy(p + off_payload + 2 * at, tile_words[t], 2ull * tile_len[t]);
+        if (tile_len[t]) std::memcpy(p + L.off_payload + 2 * at, tile_words[t], 2ull * tile_len[t]);
         at += tile_len[t];
     }
-    store_le<uint32_t>(p + off_tiles + uint64_t(kTileRecordBytes) * n_tiles, uint32_t(at));
+    store_le<uint32_t>(p + L.off_tiles + uint64_t(kTileRecordBytes) * n_tiles, uint32_t(at));
     return EP_OK;
 }
 
@@ -302,26 +309,39 @@ int run_encode(EncodeBackend &be, uint32_t R, uint32_t C, double target_bpp, con
     double last_rate = 0.0;
     Model full;
     for (;; ++b) {
-        double lo = o.bracket_lo, hi = o.bracket_hi;
-        for (int it = 0; it < o.search_steps; ++it) {
-            const double mid = std::sqrt(lo * hi);
-            Model m;
-            if ((rc = be.count_sample(float(mid), m))) return rc;
-            // more observed symbols than 2^b slots: no b-bit table exists for this scale; treat it as too fine
-            // (rate above the target).  If the scale found this way still overflows on the full tensor, b goes up.
-            if (m.worst_observed() > (1u << b)) { lo = mid; continue; }
-            m.normalise(b);
-            const double bits = estimate_bits(m, b, svec, rows.size(), V, o.retained_bits, nullptr);
-            last_rate = bits / (8.0 * double(svec));
-            if (last_rate > target_bpp) lo = mid; else hi = mid;
+        bool searched = false;
+        SearchResult found;
+        if ((rc = be.search({target_bpp, b, V, svec, rows.size()}, o, found, &searched))) return rc;
+        if (searched) {
+            s = found.s;
+            full = std::move(found.full);
+            if (found.has_last) {
+                found.last.normalise(b);
+                last_rate = estimate_bits(found.last, b, svec, rows.size(), V, o.retained_bits, nullptr) / (8.0 * double(svec));
+            }
+        } else {
+            double lo = o.bracket_lo, hi = o.bracket_hi;
+            for (int it = 0; it < o.search_steps; ++it) {
+                const double mid = std::sqrt(lo * hi);
+                Model m;
+                if ((rc = be.count_sample(float(mid), m))) return rc;
+                // more observed symbols than 2^b slots: no b-bit table exists for this scale; treat it as too fine
+                // (rate above the target).  If the scale found this way still overflows on the full tensor, b goes up.
+                if (m.worst_observed() > (1u << b)) { lo = mid; continue; }
+                m.normalise(b);
+                const double bits = estimate_bits(m, b, svec, rows.size(), V, o.retained_bits, nullptr);
+                last_rate = bits / (8.0 * double(svec));
+                if (last_rate > target_bpp) lo = mid; else hi = mid;
+            }
+            s = float(std::sqrt(lo * hi));
+            if ((rc = be.count_full(s, full))) return rc;
         }
-        s = float(std::sqrt(lo * hi));
         bool fits = false;
         for (;;) {
-            if ((rc = be.count_full(s, full))) return rc;
             if (full.worst_observed() <= (1u << b)) { fits = true; break; }
             if (b < o.b_max) break;
             s = float(1.05 * double(s) * double(full.worst_coordinate_observed()) / double(1u << b));
+            if ((rc = be.count_full(s, full))) return rc;
         }
         if (fits) break;
     }

@@ -74,8 +74,8 @@ struct Table {
 struct Model {
     Table t[EP_NUM_TABLES];
     void count(const int32_t *fields, uint64_t nvec, int threads);          // from (c, z1..z7, m) tuples
-    // from dense histograms hist[t][value - origin], `bins` bins per table (zero bins outside the observed range)
-    void from_histograms(const uint32_t *hist, uint32_t bins, int32_t origin);
+    // from counts laid out table after table: K[t] counts of the values lo[t] .. lo[t] + K[t] - 1
+    void from_counts(const int32_t *lo, const uint32_t *K, const uint32_t *counts);
     void normalise(int b);                                                   // integer frequencies summing to 2^b
     double cross_entropy_bits(int b) const;                                  // Eq. 8
     uint64_t section_bytes() const;
@@ -89,12 +89,33 @@ double estimate_bits(const Model &m, int b, uint64_t nvec, uint64_t rows, uint32
 // App. "Scale-search settings": complete rows, shape-dependent seed, sorted
 std::vector<uint32_t> sample_rows(uint32_t R, uint32_t C, uint32_t budget_vectors);
 
+// Where the sections of a stored representation lie.  Scales, tile index and payload are back to back.
+struct BlobLayout { uint64_t off_tables, off_scales, off_tiles, off_payload, total; };
+
+// Allocates a blob for total_words payload words and writes its header and tables; the three sections after
+// off_scales are left to the caller.
+int begin_blob(const Model &m, uint32_t R, uint32_t C, int b, uint32_t V, float s_info, uint64_t total_words, ep_blob *out,
+               BlobLayout *at);
+
 // header + tables + scales + tile index + payload; `states` holds 32 words per tile, tile t's payload is
-// tile_words[t] .. + tile_len[t].  With tile_words == nullptr the payload section is left unwritten for the
-// caller to fill in place: it starts at out->bytes.data() + *payload_offset and holds the tiles back to back.
+// tile_words[t] .. + tile_len[t].
 int assemble_blob(const Model &m, uint32_t R, uint32_t C, int b, uint32_t V, const float *sigma, float s_info,
-                  const uint32_t *states, const uint16_t *const *tile_words, const uint32_t *tile_len, ep_blob *out,
-                  uint64_t *payload_offset = nullptr);
+                  const uint32_t *states, const uint16_t *const *tile_words, const uint32_t *tile_len, ep_blob *out);
+
+// One bisection of Algorithm 1 for a back end that runs it whole.
+struct SearchJob {
+    double target_bpp;
+    int b;
+    uint32_t V;
+    uint64_t sample_vectors;     // vectors in the row sample
+    size_t sample_rows;
+};
+struct SearchResult {
+    float s = 0.0f;              // the scale the bisection ends on
+    Model last;                  // counts of the last candidate whose rate was evaluated
+    bool has_last = false;
+    Model full;                  // counts of the whole tensor at s (quantisation kept, as by count_full)
+};
 
 // What a back end must provide.  Each call returns an ep_status.
 struct EncodeBackend {
@@ -102,6 +123,9 @@ struct EncodeBackend {
     virtual int prepare(const std::vector<uint32_t> &sample) = 0;   // row RMS; remember the row sample
     virtual int count_sample(float s, Model &m) = 0;                // quantise the sample at s, count its fields
     virtual int count_full(float s, Model &m) = 0;                  // quantise the whole tensor at s (kept), count
+    // the bisection of Algorithm 1 on the row sample and the full-tensor pass at the scale it ends on, in one go.
+    // *done = false: not supported, or a decision the back end will not take; the driver then runs it step by step
+    virtual int search(const SearchJob & /*job*/, const ep_encode_opts & /*o*/, SearchResult & /*r*/, bool *done) { *done = false; return EP_OK; }
     // refit the row scales of the kept quantisation (Eq. 13), encode the tiles under the normalised
     // full-tensor model m and assemble the blob
     virtual int finish(float s, int b, uint32_t V, const Model &m, ep_blob *out) = 0;
