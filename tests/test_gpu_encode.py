@@ -86,3 +86,38 @@ def test_device_encoder_blobs_keep_their_bytes_while_buffers_are_reused():
         assert np.array_equal(b.data, ref_b)
         del b
         gc.collect()
+
+
+def _wide_alphabet(magnitude):
+    # a few outliers of up to `magnitude` row sigmas in every coordinate position stretch the tables
+    W = synth.gaussian_rows(256, 2048, 5)
+    rng = np.random.default_rng(5)
+    sig = W.std(1)
+    for i in range(400):
+        r = rng.integers(256)
+        W[r, rng.integers(2048)] = magnitude * sig[r] * (1 if i % 2 else -1) * rng.uniform(0.8, 1.0)
+    return W
+
+
+def _grid(R, C):
+    # weights on a coarse grid, half the rows all zero: quantiser inputs on ties, where only the exact path decides
+    W = np.round(synth.gaussian_rows(R, C, 6) * 64).astype(np.float32) / 64
+    W[::2] = 0.0
+    return W
+
+
+@pytest.mark.parametrize("W,bpp,kw", [
+    (_wide_alphabet(20.0), 6.0, {}),          # 7 k symbols: counts that take a second copy, wide code tables
+    (_wide_alphabet(20.0), 8.0, {}),          # 20 k symbols
+    (_wide_alphabet(40.0), 8.0, {}),          # over 25 k: a step the device hands to the host, tables in global memory
+    (_grid(64, 1024), 3.0, {}),
+    (_grid(5, 8), 2.0, {}),
+    (synth.laplace_rows(1, 40960, 7), 4.0, dict(tile_vectors=33)),       # one long row, ragged tiles
+    (synth.gaussian_rows(3000, 8, 8), 4.0, dict(polish_steps=0)),        # one block per row
+    (synth.gaussian_rows(300, 1032, 9), 5.0, dict(search_steps=0)),
+    (synth.gaussian_rows(300, 1032, 9), 5.0, dict(b_start=9, b_max=13, sample_vectors=500)),
+])
+def test_device_encoder_bytes_at_the_edges_of_its_paths(W, bpp, kw):
+    host = ep.encode(W, bpp, **kw)
+    dev = ep.encode_device(torch.from_numpy(np.ascontiguousarray(W, np.float32)).cuda(), bpp, **kw)
+    assert np.array_equal(dev.data, host.data) and dev.report == host.report
