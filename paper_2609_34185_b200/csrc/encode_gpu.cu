@@ -30,6 +30,7 @@ using namespace ep;
 constexpr int kHistBins = 8192;          // per table, values -4096 .. 4095
 constexpr int kHistOrigin = -4096;
 constexpr uint32_t kMaxTableSymbols = 40960;   // sum of K over the 17 tables that a stream of this back end may have
+constexpr uint32_t kMaxEntries = 2 * kMaxTableSymbols + 2;     // the tile coder's entries (see EncodeTables)
 constexpr double kUnit = 1.1102230246251565e-16;   // 2^-53, the rounding unit of double
 
 // ---- sums over a row ------------------------------------------------------------------------------------
@@ -162,112 +163,166 @@ __device__ __noinline__ int quantise_exact(const float *x, float mu, float s, in
     return half ? 1 : 0;
 }
 
-// The same point from y ~ x * r with r ~ 1 / (mu s), or `false` where the difference could matter.
-// y is within E = 4e-7 (|y| + 1) of the host's (two roundings there, three here, each 2^-24, and the host's y - 1/2).
+// two fp32 numbers per instruction
+__device__ __forceinline__ float2 add2(float2 a, float2 b) {
+    float2 r;
+    asm("{\n\t.reg .b64 x, y;\n\tmov.b64 x, {%2, %3};\n\tmov.b64 y, {%4, %5};\n\tadd.rn.f32x2 x, x, y;\n\tmov.b64 {%0, %1}, x;\n\t}"
+        : "=f"(r.x), "=f"(r.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return r;
+}
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) {
+    float2 r;
+    asm("{\n\t.reg .b64 x, y;\n\tmov.b64 x, {%2, %3};\n\tmov.b64 y, {%4, %5};\n\tmul.rn.f32x2 x, x, y;\n\tmov.b64 {%0, %1}, x;\n\t}"
+        : "=f"(r.x), "=f"(r.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return r;
+}
+// a - b, exactly fp32's: b's sign flips without rounding
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) {
+    float2 r;
+    asm("{\n\t.reg .b64 x, y;\n\tmov.b64 x, {%2, %3};\n\tmov.b64 y, {%4, %5};\n\tsub.rn.f32x2 x, x, y;\n\tmov.b64 {%0, %1}, x;\n\t}"
+        : "=f"(r.x), "=f"(r.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return r;
+}
+__device__ __forceinline__ float rcp_approx(float v) {
+    float r;
+    asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(v));            // within 2^-23
+    return r;
+}
+// The same point from y ~ x * r with r ~ 1 / (mu s), or `false` where the difference could matter.  z comes back as the
+// bits of 1.5 * 2^23 + z.
+// y is within E = 5e-7 (|y| + 1) of the host's (two roundings of 2^-24 there; a product, a reciprocal within 2^-23
+// and a product here; and y - 1/2 on either side).
 // With a_i = |y_i - rint(y_i)|: the integer candidate has residuals a_i, the half candidate 1/2 - a_i, and Eq. 3's parity
 // step moves the largest residual r to 1 - r; so the squared distances differ by
 //     d_half - d_int = 2 - sum a + [half parity odd] 2 min a - [integer parity odd] (1 - 2 max a).
 // Every decision - the two roundings of each coordinate, the coset, which coordinate the parity step moves - must have
-// a margin of more than what E can change.  At 4 bpp one block in 4000 fails and takes the divisions; at 8 bpp one
-// in 250.  (Compared with the exact routine on 6 x 10^7 random blocks and blocks built around ties: no difference.)
-__device__ __forceinline__ bool quantise_fast(const float (&x)[8], float r, int32_t (&z)[8], uint32_t &half) {
-    float a[8];
-    uint32_t neg[8], odd_int = 0, odd_neg = 0;
-    float ymax = 0.0f, sum = 0.0f;
+// a margin of more than what E can change.  At 4 bpp one block in 3000 fails and takes the divisions; at 8 bpp one
+// in 200.  (Compared with the exact routine on 6 x 10^7 random blocks and blocks built around ties: no difference.)
+// About 17 instructions per coordinate, most on the multiply-add pipe, two coordinates at a time where possible.
+__device__ __forceinline__ bool quantise_fast(const float (&x)[8], float r, uint32_t (&z)[8], uint32_t &half) {
+    const float2 magic = make_float2(12582912.0f, 12582912.0f), rr = make_float2(r, r);   // 1.5 * 2^23: rounds to the nearest integer
+    float2 y[4];
+    uint32_t parity = 0, signs = 0;
+    float ymax = 0.0f, big = 0.0f, small = 1.0f, sum = 0.0f;
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        const float y = __fmul_rn(x[i], r);
-        const float t = __fadd_rn(y, 12582912.0f);            // 1.5 * 2^23: rounds to the nearest integer
-        z[i] = __float_as_int(t) - 0x4B400000;
-        const float res = __fsub_rn(y, __fsub_rn(t, 12582912.0f));
-        neg[i] = __float_as_uint(res) >> 31;
-        a[i] = fabsf(res);
-        odd_int ^= uint32_t(z[i]);
-        odd_neg ^= neg[i];
-        ymax = fmaxf(ymax, fabsf(y));
-        sum = __fadd_rn(sum, a[i]);
+    for (int i = 0; i < 4; ++i) {
+        y[i] = mul2(make_float2(x[2 * i], x[2 * i + 1]), rr);
+        const float2 t = add2(y[i], magic), res = sub2(y[i], sub2(t, magic));
+        parity ^= __float_as_uint(t.x) ^ __float_as_uint(t.y);
+        signs ^= __float_as_uint(res.x) ^ __float_as_uint(res.y);
+        ymax = fmaxf(fmaxf(ymax, fabsf(y[i].x)), fabsf(y[i].y));
+        big = fmaxf(fmaxf(big, fabsf(res.x)), fabsf(res.y));
+        small = fminf(fminf(small, fabsf(res.x)), fabsf(res.y));
+        sum += fabsf(res.x) + fabsf(res.y);
     }
-    float big = a[0], small = a[0];
-#pragma unroll
-    for (int i = 1; i < 8; ++i) { big = fmaxf(big, a[i]); small = fminf(small, a[i]); }
-    const bool oi = odd_int & 1u, oh = (odd_int ^ odd_neg) & 1u;
-    const float E = 4e-7f * ymax + 4e-7f;
+    const bool odd_int = parity & 1u, odd_half = (parity ^ (signs >> 31)) & 1u;
+    const float E = 5e-7f * ymax + 5e-7f;
     float d = 2.0f - sum;
-    if (oh) d += 2.0f * small;
-    if (oi) d -= 1.0f - 2.0f * big;
-    bool ok = small > E && big < 0.5f - E && fabsf(d) > 16.0f * E + 4e-6f && ymax < 3990.0f;
-    const bool h = d < 0.0f;
+    if (odd_half) d += 2.0f * small;
+    if (odd_int) d -= 1.0f - 2.0f * big;
+    const bool h = d < 0.0f, odd = h ? odd_half : odd_int;
     half = h ? 1u : 0u;
-    const bool odd = h ? oh : oi;
-    const float sel = h ? small : big, near = 2.5f * E;
-    uint32_t hits = 0;
+    const bool ok = small > E && big < 0.5f - E && fabsf(d) > 16.0f * E + 4e-6f && ymax < 3990.0f;
+    // the chosen candidate: y or y - 1/2 rounded, its largest residual moved away from y if the coordinate sum is odd
+    const float shift = h ? -0.5f : 0.0f;
+    const float most = odd ? (h ? 0.5f - small : big) - 2.5f * E : 2.0f;
+    float hits = 0.0f;
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        const uint32_t hit = fabsf(a[i] - sel) <= near ? 1u : 0u;
-        hits += hit;
-        // integer candidate: rint(y), its moved coordinate away from y's side; half candidate: floor(y), the moved one too
-        z[i] += (odd && hit ? 1 - 2 * int(neg[i] ^ half) : 0) - int(neg[i] & half);
+    for (int i = 0; i < 4; ++i) {
+        const float2 v = add2(y[i], make_float2(shift, shift));
+        float2 t = add2(v, magic);
+        const float2 res = sub2(v, sub2(t, magic));
+        if (fabsf(res.x) >= most) { hits += 1.0f; t.x += __uint_as_float((__float_as_uint(res.x) & 0x80000000u) | 0x3F800000u); }
+        if (fabsf(res.y) >= most) { hits += 1.0f; t.y += __uint_as_float((__float_as_uint(res.y) & 0x80000000u) | 0x3F800000u); }
+        z[2 * i] = __float_as_uint(t.x);
+        z[2 * i + 1] = __float_as_uint(t.y);
     }
-    return ok && !(odd && hits != 1u);
+    return ok && !(odd && hits != 1.0f);
 }
 
 // ---- counting passes ---------------------------------------------------------------------------------------
-// One pass quantises the listed rows (all rows) at one scale and counts the fields.  The last CTA to finish gathers
-// the counts for the host, or - in a step of the bisection - evaluates Eq. 10-12 on them and leaves the next scale
-// in device memory, so that the twelve steps and the full pass after them are one stream of launches with a
-// single wait at the end.
-// Counting is what a pass spends most on after the arithmetic: nine increments per block, most of them of a few
-// values around zero.  Each lane has its own column of counters for those (bank = lane: no two lanes of a warp
-// meet), values up to +-256 go to a plain window, the rest to global memory.
+// A pass quantises the listed rows (all rows) at a scale and counts the fields.  The whole search of Algorithm 1 and
+// the rate correction after it are one stream of launches with one wait at the end: the last CTA of a pass evaluates
+// Eq. 10-12 on the counts and leaves the next scale in device memory.
+//
+// A step of the bisection costs about 14 us whatever the sample (launch, clearing and flushing counters, the evaluation's
+// chain of dependent reads), and counting the sample only 4 us more.  So one launch takes three steps: seven scales
+// at once, the bracket's middle and the middles of the brackets that its two, then four, outcomes lead to, each counted
+// and evaluated by CTAs of its own; the last one to finish walks the tree.  (The first launches take one and two steps:
+// the outer candidates of a wide bracket are so fine - s = 0.003 - that all they count goes to global memory, 120 us.)
+//
+// Counting: nine increments per block, most of them of a few values around zero.  Each lane has its own column of
+// counters for those (bank = lane: no two lanes of a warp meet), values up to +-256 go to a plain window, the rest to
+// global memory.
 constexpr uint32_t kCountThreads = 1024;
 constexpr int kHotBins = 32, kHotOrigin = -16;   // values with a counter column per lane, per coordinate table
+constexpr uint32_t kHotStride = (kHotBins + 1) * 32;   // words per table: one more row takes what lies outside
 constexpr int kWinBins = 512, kWinOrigin = -256; // values with one counter per CTA, per table
-constexpr uint32_t kHotWords = 16 * kHotBins * 32, kWinWords = EP_NUM_TABLES * kWinBins;
+constexpr uint32_t kHotWords = 16 * kHotStride, kWinWords = EP_NUM_TABLES * kWinBins;
 constexpr uint32_t kCountSmem = 4 * (kHotWords + kWinWords);
-// symbols over all tables that a step's evaluation holds in shared memory (it reuses the counters' space); with
-// more of them the host takes over
-constexpr uint32_t kEvalSymbols = kHotWords + kWinWords;
+// symbols over all tables that an evaluation holds in shared memory (it reuses the counters' space); with more of
+// them the host takes over
+constexpr uint32_t kEvalSymbols = 24576;
+static_assert(kEvalSymbols <= kHotWords + kWinWords, "evaluation space");
 constexpr uint32_t kFirstCounts = 6144;          // counts that come back with the state; more take a second copy
+constexpr uint32_t kLevels = 3, kCandidates = (1u << kLevels) - 1u;
 
 struct CountDir { int32_t lo[EP_NUM_TABLES]; uint32_t K[EP_NUM_TABLES]; };
 
-// what the passes leave for one another and for the host (device memory, zeroed before the first pass)
+// one scale of a pass (device memory)
+struct Candidate {
+    CountDir dir;
+    // observed range, stored as the larger of (kHistBins - bin) and of (bin + 1); 0: none
+    uint32_t from[EP_NUM_TABLES], to[EP_NUM_TABLES];
+    uint32_t finished;               // its CTAs that are done
+    uint32_t overflow;               // a coordinate left the histogram range
+    uint32_t verdict;                // kValid ...
+};
+// a b-bit table exists; the rate lies above the target; too close to say
+constexpr uint32_t kValid = 1, kAbove = 2, kUndecided = 4, kOverflow = 8;
+// what the passes leave for one another and for the host (device memory, zeroed before a search)
 struct SearchState {
     double lo, hi;                   // the bracket
+    double last_log_s, last_rate;    // rate correction: the last point
     float s;                         // the next pass's scale
-    uint32_t has_last;               // 1: `last` holds the last step whose rate was evaluated; 2: it has been overwritten
-    uint32_t undecided;              // a step fell within the rounding error of the target, or had too many symbols
+    float s_counted;                 // the scale of the full counts
+    uint32_t has_last;               // `last` holds the counts of the last step whose rate was evaluated
+    uint32_t undecided;              // a decision within the rounding error, or too many symbols: the host repeats the search
     uint32_t overflow;               // a coordinate left the histogram range
-    uint32_t finished;               // CTAs of the running pass that are done
-    // observed range of the running pass, stored as the larger of (kHistBins - bin) and of (bin + 1); 0: none
-    uint32_t from[EP_NUM_TABLES], to[EP_NUM_TABLES];
+    uint32_t closed;                 // candidates of the running pass that are evaluated
+    uint32_t stop;                   // the full passes are over
+    uint32_t polished;               // ... because the rate correction ended (0: the tensor overflows the tables, the host decides)
     CountDir last, full;
     uint32_t total_words;            // tile coding: words of the payload
     uint32_t tiles_done;             //              CTAs of the launch that are done
+    Candidate cand[kCandidates];
 };
-constexpr size_t kStateBytes = 1024;
+constexpr size_t kStateBytes = 6144;
 static_assert(sizeof(SearchState) <= kStateBytes, "state area");
 
-// the constants of Eq. 10-12 on the sample
-struct StepParams {
-    double target, retained_bits_total, fixed_bits, weights, sample_fields;   // fixed_bits: restarts, scales, header
-    double lo0, hi0;                 // the bracket before the first step
-    int32_t b, step;                 // step: 0 .. for a step of the bisection, -1 for a pass that only counts
+// the constants of Eq. 10-12
+struct RateParams {
+    double target, retained_bits_total, fixed_bits, weights, fields;   // fixed_bits: restarts, scales, header
+    int32_t b;
 };
+enum PassMode { kPassCount, kPassSearch, kPassPolish };   // counts only; steps of the bisection; a pass of the rate correction
 
 struct CountParams {
     const float *W;
     const float *mu;
     const uint32_t *rows;            // null: all rows
     uint4 *fields;                   // one per block: z1 .. z7 and 2 m + c as int16; null: not kept
-    uint32_t *hist;                  // EP_NUM_TABLES x kHistBins, zero between passes
+    uint32_t *hist;                  // per candidate EP_NUM_TABLES x kHistBins, zero between passes
     SearchState *state;
+    uint32_t *cand_counts;           // per candidate kEvalSymbols
     uint32_t *last_counts, *full_counts;
-    uint64_t n_blocks;
-    uint32_t C, per_row;
-    float s;
-    uint32_t s_from_state;
-    StepParams step;
+    uint32_t n_blocks, C, per_row;
+    uint32_t mode, levels, ctas;     // ctas: per candidate
+    uint32_t first;                  // first pass of the search: the bracket is {lo0, hi0}; of the rate correction: step 0
+    float s;                         // mode kPassCount
+    RateParams rate;
+    double lo0, hi0;                 // the search bracket
+    int32_t step, last_step;         // rate correction: passes done so far, and allowed
 };
 
 __device__ __forceinline__ uint32_t warp_sum(uint32_t v) { return __reduce_add_sync(0xFFFFFFFFu, v); }
@@ -282,56 +337,88 @@ __device__ __forceinline__ unsigned long long warp_sum(unsigned long long v) {
     return v;
 }
 
-// The last CTA of a pass: ranges and offsets of the tables, counts to `out`, histogram back to zero.  For a step of the
-// bisection also the frequencies of Sec. 3.3 (integers: the host's exactly), C_CE of Eq. 8 and the comparison of
-// Eq. 12 with the target.  C_CE is a sum of doubles in another order and with this device's log2; if the host's
-// value, within the bound `off`, could compare differently, the step is marked undecided and the host repeats the search.
-__device__ void close_pass(const CountParams &P, uint32_t *f_of) {
+// bracket of candidate k: the tree's nodes in heap order, the left child of a node being the outcome "rate above target"
+__device__ __forceinline__ void bracket_of(uint32_t k, double &lo, double &hi) {
+    const uint32_t n = k + 1u;
+    for (int bit = 30 - __clz(int(n)); bit >= 0; --bit) {
+        const double mid = __dsqrt_rn(__dmul_rn(lo, hi));
+        if ((n >> bit) & 1u) hi = mid; else lo = mid;
+    }
+}
+
+// Eq. 10-11 for a given C_CE, as the host computes it (everything but the first difference is exact)
+__device__ __forceinline__ double bits_at(const RateParams &P, double tables, double cce) {
+    const double left = fmax(0.0, __dsub_rn(cce, P.retained_bits_total));
+    return __dadd_rn(__dadd_rn(__dmul_rn(16.0, ceil(__dmul_rn(left, 0.0625))), P.fixed_bits), tables);
+}
+
+struct Evaluation { double cce, tables; uint32_t worst; bool too_many; };
+
+// All threads of a candidate's last CTA: ranges and offsets of its tables, counts to `out`, histogram back to zero; unless
+// only counts are wanted, the frequencies of Sec. 3.3 (integers: the host's exactly), C_CE of Eq. 8 and the largest alphabet.
+__device__ __forceinline__ Evaluation gather_counts(const CountParams &P, uint32_t k, uint32_t *out, uint32_t *f_of) {
     __shared__ int32_t lo_of[EP_NUM_TABLES];
     __shared__ uint32_t K_of[EP_NUM_TABLES], at_of[EP_NUM_TABLES + 1], seen_of[EP_NUM_TABLES];
     __shared__ double bits_of[EP_NUM_TABLES];
-    SearchState &S = *P.state;
+    Candidate &S = P.state->cand[k];
     const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
-    const bool step = P.step.step >= 0;
-    if (tid < EP_NUM_TABLES) {
-        const uint32_t a = __ldcg(&S.from[tid]), z = __ldcg(&S.to[tid]);
-        const uint32_t first = kHistBins - a;
-        lo_of[tid] = a ? kHistOrigin + int32_t(first) : 0;
-        K_of[tid] = a ? z - first : 0u;                     // z = last bin + 1
-        S.from[tid] = 0;
-        S.to[tid] = 0;
+    if (warp == 0) {
+        uint32_t K = 0;
+        int32_t lo = 0;
+        if (lane < EP_NUM_TABLES) {
+            const uint32_t a = __ldcg(&S.from[lane]), z = __ldcg(&S.to[lane]);
+            const uint32_t first = kHistBins - a;
+            lo = a ? kHistOrigin + int32_t(first) : 0;
+            K = a ? z - first : 0u;                         // z = last bin + 1
+            S.from[lane] = 0;
+            S.to[lane] = 0;
+            S.dir.lo[lane] = lo;
+            S.dir.K[lane] = K;
+        }
+        uint32_t incl = K;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const uint32_t n = __shfl_up_sync(0xFFFFFFFFu, incl, d);
+            if (lane >= uint32_t(d)) incl += n;
+        }
+        if (lane < EP_NUM_TABLES) { lo_of[lane] = lo; K_of[lane] = K; at_of[lane + 1] = incl; }
+        if (lane == 0) { at_of[0] = 0; S.finished = 0; }
     }
     __syncthreads();
-    if (tid == 0) {
-        uint32_t at = 0;
-        for (int t = 0; t < EP_NUM_TABLES; ++t) { at_of[t] = at; at += K_of[t]; }
-        at_of[EP_NUM_TABLES] = at;
-        S.finished = 0;
-    }
-    __syncthreads();
-    const bool too_many = step && at_of[EP_NUM_TABLES] > kEvalSymbols;
-    uint32_t *out = step ? P.last_counts : P.full_counts;
+    const bool evaluate = P.mode != kPassCount;
+    Evaluation E;
+    E.too_many = at_of[EP_NUM_TABLES] > kEvalSymbols;       // (only full_counts has room for more)
+    E.tables = 8.0 * double((8u * EP_NUM_TABLES + 2u * at_of[EP_NUM_TABLES] + 3u) & ~3u);
+    const bool keep = !E.too_many || P.mode != kPassSearch;
     for (uint32_t t = warp; t < EP_NUM_TABLES; t += kCountThreads / 32u) {
         const uint32_t K = K_of[t], at = at_of[t];
-        uint32_t *h = P.hist + t * kHistBins + (lo_of[t] - kHistOrigin);
+        uint32_t *h = P.hist + (k * EP_NUM_TABLES + t) * kHistBins + (lo_of[t] - kHistOrigin);
         unsigned long long sum = 0;
         uint32_t seen = 0;
-        for (uint32_t j = lane; j < K; j += 32) {
-            const uint32_t n = __ldcg(h + j);
-            h[j] = 0;
-            if (!too_many) out[at + j] = n;
-            sum += n;
-            seen += n != 0;
+        for (uint32_t j0 = lane; j0 < K; j0 += 8u * 32u) {     // eight loads under way at a time
+            uint32_t n[8];
+#pragma unroll
+            for (uint32_t u = 0; u < 8; ++u) n[u] = j0 + 32u * u < K ? __ldcg(h + j0 + 32u * u) : 0u;
+#pragma unroll
+            for (uint32_t u = 0; u < 8; ++u) {
+                const uint32_t j = j0 + 32u * u;
+                if (j >= K) break;
+                h[j] = 0;
+                if (keep) out[at + j] = n[u];
+                if (!E.too_many) f_of[at + j] = n[u];
+                sum += n[u];
+                seen += n[u] != 0;
+            }
         }
-        if (!step || too_many) continue;
+        if (!evaluate || E.too_many) continue;
         const double total = double(warp_sum(sum));
         seen = warp_sum(seen);
         // frequencies: max(1, floor(n 2^b / total)), then the deficit to the largest or the excess from the largest
-        const uint32_t M = 1u << P.step.b;
+        const uint32_t M = 1u << P.rate.b;
         uint32_t fsum = 0, best = 0;
         auto key = [](uint32_t f, uint32_t j) { return (f << 16) | (0xFFFFu - j); };      // f <= 2^15, j < 2^13: first of the largest
         for (uint32_t j = lane; j < K; j += 32) {
-            const uint32_t n = out[at + j];
+            const uint32_t n = f_of[at + j];
             uint32_t f = 0;
             if (n) {
                 const double nM = double(n) * double(M);                                  // below 2^47: exact
@@ -352,7 +439,7 @@ __device__ void close_pass(const CountParams &P, uint32_t *f_of) {
         }
         while (K && fsum > M) {                              // (every turn lowers fsum or leaves)
             const uint32_t f = best >> 16, take = min(fsum - M, f - 1u);
-            if (f <= 1u) break;                              // more symbols than slots: the step is judged by `seen`
+            if (f <= 1u) break;                              // more symbols than slots: judged by `worst`
             if (lane == 0) f_of[at + 0xFFFFu - (best & 0xFFFFu)] = f - take;
             fsum -= take;
             __syncwarp();
@@ -363,125 +450,220 @@ __device__ void close_pass(const CountParams &P, uint32_t *f_of) {
         }
         __syncwarp();
         double bits = 0.0;
+#pragma unroll 4
         for (uint32_t j = lane; j < K; j += 32) {
-            const uint32_t n = out[at + j];
-            if (n) bits += double(n) * (double(P.step.b) - log2(double(f_of[at + j])));
+            const uint32_t f = f_of[at + j];
+            if (f) bits += double(out[at + j]) * (double(P.rate.b) - log2(double(f)));
         }
         bits = warp_sum(bits);
         if (lane == 0) { bits_of[t] = bits; seen_of[t] = seen; }
     }
     __syncthreads();
-    CountDir &D = step ? S.last : S.full;
-    if (!too_many && tid < EP_NUM_TABLES) { D.lo[tid] = lo_of[tid]; D.K[tid] = K_of[tid]; }
-    if (!step || tid != 0) return;
-    double lo = P.step.step == 0 ? P.step.lo0 : S.lo, hi = P.step.step == 0 ? P.step.hi0 : S.hi;
-    const double mid = __dsqrt_rn(__dmul_rn(lo, hi));
-    if (too_many) {
-        S.undecided = 1;
-    } else {
-        double cce = 0.0;
-        uint32_t worst = 0;
-        for (int t = 0; t < EP_NUM_TABLES; ++t) { cce = __dadd_rn(cce, bits_of[t]); worst = max(worst, seen_of[t]); }
-        bool above;
-        if (worst > (1u << P.step.b)) {
-            above = true;                                    // no b-bit table exists for this scale: too fine
-            if (S.has_last) S.has_last = 2;
-        } else {
-            const double tables = 8.0 * double((8u * EP_NUM_TABLES + 2u * at_of[EP_NUM_TABLES] + 3u) & ~3u);
-            auto rate_above = [&](double c) {
-                const double left = fmax(0.0, __dsub_rn(c, P.step.retained_bits_total));
-                const double payload = __dmul_rn(16.0, ceil(__dmul_rn(left, 0.0625)));
-                return __ddiv_rn(__dadd_rn(__dadd_rn(payload, P.step.fixed_bits), tables), P.step.weights) > P.step.target;
-            };
-            // terms are at most b <= 15 bits per field, their sum is taken in a few thousand additions
-            const double off = 1e-11 * (cce + 16.0 * P.step.sample_fields);
-            above = rate_above(cce);
-            if (rate_above(cce - off) != rate_above(cce + off)) S.undecided = 1;
-            S.has_last = 1;
-        }
-        if (above) lo = mid; else hi = mid;
+    E.cce = 0.0;
+    E.worst = 0;
+    if (evaluate && !E.too_many && warp == 0) {
+        E.cce = warp_sum(lane < EP_NUM_TABLES ? bits_of[lane] : 0.0);
+        E.worst = __reduce_max_sync(0xFFFFFFFFu, lane < EP_NUM_TABLES ? seen_of[lane] : 0u);
     }
-    S.lo = lo;
-    S.hi = hi;
-    S.s = __double2float_rn(__dsqrt_rn(__dmul_rn(lo, hi)));
+    return E;                                                // (cce and worst in warp 0)
+}
+// C_CE above is a sum in another order, with this device's log2 (within one unit in the last place; terms of at most 15 bits
+// per field, a few thousand additions).  How far the host's can be:
+__device__ __forceinline__ double cce_bound(const RateParams &P, double cce) { return 1e-11 * (cce + 16.0 * P.fields); }
+
+// thread 0 after a candidate of the search is gathered: is its rate above the target?
+__device__ void judge_candidate(const CountParams &P, uint32_t k, const Evaluation &E) {
+    uint32_t v = 0;
+    if (E.too_many) {
+        v = kUndecided;
+    } else if (E.worst > (1u << P.rate.b)) {
+        v = kAbove;                                              // no b-bit table exists for this scale: too fine
+    } else {
+        const double off = cce_bound(P.rate, E.cce);
+        auto above = [&](double cce) { return __ddiv_rn(bits_at(P.rate, E.tables, cce), P.rate.weights) > P.rate.target; };
+        v = kValid | (above(E.cce) ? kAbove : 0u) | (above(E.cce - off) != above(E.cce + off) ? kUndecided : 0u);
+    }
+    P.state->cand[k].verdict = v;
+}
+
+// all threads of the pass's last CTA: the steps' outcomes in order
+__device__ void walk_tree(const CountParams &P) {
+    __shared__ int32_t chosen;
+    SearchState &S = *P.state;
+    if (threadIdx.x == 0) {
+        double lo = P.first ? P.lo0 : S.lo, hi = P.first ? P.hi0 : S.hi;
+        int32_t last = -1;
+        uint32_t k = 0, verdict[kCandidates];
+#pragma unroll
+        for (uint32_t i = 0; i < kCandidates; ++i) verdict[i] = __ldcg(&S.cand[i].verdict) | (__ldcg(&S.cand[i].overflow) ? kOverflow : 0u);
+#pragma unroll
+        for (uint32_t i = 0; i < kCandidates; ++i) S.cand[i].overflow = 0;
+        for (uint32_t l = 0; l < P.levels; ++l) {
+            uint32_t v = verdict[0];
+#pragma unroll
+            for (uint32_t i = 1; i < kCandidates; ++i) if (i == k) v = verdict[i];
+            if (v & kOverflow) S.overflow = 1;
+            if (v & kUndecided) S.undecided = 1;
+            if (v & kValid) last = int32_t(k);
+            const double mid = __dsqrt_rn(__dmul_rn(lo, hi));
+            if (v & kAbove) { lo = mid; k = 2u * k + 1u; } else { hi = mid; k = 2u * k + 2u; }
+        }
+        S.lo = lo;
+        S.hi = hi;
+        S.s = __double2float_rn(__dsqrt_rn(__dmul_rn(lo, hi)));
+        S.closed = 0;
+        if (last >= 0) S.has_last = 1;
+        chosen = last;
+    }
+    __syncthreads();
+    if (chosen < 0) return;
+    // the host reports the rate of the last evaluated step: its counts
+    const Candidate &c = S.cand[chosen];
+    uint32_t n = 0;
+    for (int t = 0; t < EP_NUM_TABLES; ++t) n += __ldcg(&c.dir.K[t]);
+    for (uint32_t i = threadIdx.x; i < n; i += kCountThreads) P.last_counts[i] = __ldcg(P.cand_counts + size_t(chosen) * kEvalSymbols + i);
+    if (threadIdx.x < EP_NUM_TABLES) {
+        S.last.lo[threadIdx.x] = __ldcg(&c.dir.lo[threadIdx.x]);
+        S.last.K[threadIdx.x] = __ldcg(&c.dir.K[threadIdx.x]);
+    }
+}
+
+// thread 0 after a full pass: the rate correction's next scale, or its end (run_encode has the same steps)
+__device__ void polish(const CountParams &P, float s, const Evaluation &E) {
+    SearchState &S = *P.state;
+    S.s_counted = s;
+    if (E.too_many) { S.undecided = 1; S.stop = 1; return; }
+    if (E.worst > (1u << P.rate.b)) {                            // before the first move: the host raises b or s
+        if (P.step > 0) S.undecided = 1;
+        S.stop = 1;
+        return;
+    }
+    S.polished = 1;
+    if (P.step >= P.last_step) { S.stop = 1; return; }
+    const double off = cce_bound(P.rate, E.cce), bits = bits_at(P.rate, E.tables, E.cce);
+    // the payload estimate is rounded up to words: if it is the same at both ends of the interval it is the host's exactly
+    if (bits_at(P.rate, E.tables, E.cce - off) != bits_at(P.rate, E.tables, E.cce + off)) { S.undecided = 1; S.stop = 1; return; }
+    const double est = __ddiv_rn(bits, P.rate.weights);
+    if (fabs(__dsub_rn(est, P.rate.target)) <= __dmul_rn(0.002, P.rate.target)) { S.stop = 1; return; }
+    const double log_s = log2(double(s));
+    double per_doubling = 1.0;
+    if (P.step > 0 && log_s != S.last_log_s) {
+        per_doubling = -__ddiv_rn(__dsub_rn(est, S.last_rate), __dsub_rn(log_s, S.last_log_s));
+        if (!(per_doubling >= 0.5)) per_doubling = 0.5;
+        if (per_doubling > 4.0) per_doubling = 4.0;
+    }
+    S.last_log_s = log_s;
+    S.last_rate = est;
+    // log2 and exp2 may differ from the host's in the last place (of numbers up to ten, divided by a slope of at least 1/2, and
+    // by a move of at least 2^-20 in the secant): far less than 1e-8
+    const double moved = exp2(__dadd_rn(log_s, __ddiv_rn(__dsub_rn(est, P.rate.target), per_doubling)));
+    auto next = [&](double m) {
+        if (!(m >= P.lo0)) m = P.lo0;
+        if (m > P.hi0) m = P.hi0;
+        return __double2float_rn(m);
+    };
+    const float to = next(moved);
+    if (next(moved * (1.0 - 1e-10)) != to || next(moved * (1.0 + 1e-10)) != to) { S.undecided = 1; S.stop = 1; return; }
+    if (to == s) { S.stop = 1; return; }
+    S.s = to;
 }
 
 __global__ void __launch_bounds__(kCountThreads, 1) quantise_count_kernel(const __grid_constant__ CountParams P) {
     extern __shared__ __align__(16) uint32_t sm[];
     uint32_t *const hot = sm, *const win = sm + kHotWords;
     __shared__ uint32_t range_from[EP_NUM_TABLES], range_to[EP_NUM_TABLES], last_cta;
+    __shared__ float s_shared;
     const uint32_t tid = threadIdx.x, lane = tid & 31u;
-    // this CTA's blocks and this thread's first one; the rows of neighbouring blocks follow without divisions
-    const uint64_t v0 = P.n_blocks * blockIdx.x / gridDim.x, v1 = P.n_blocks * (blockIdx.x + 1ull) / gridDim.x;
-    uint64_t v = v0 + tid;
-    uint64_t i = v / P.per_row;
-    uint32_t col = uint32_t(v - i * P.per_row);
+    const uint32_t k = blockIdx.x / P.ctas, part = blockIdx.x - k * P.ctas;      // candidate, and this CTA's share of the blocks
+    Candidate &S = P.state->cand[k];
+    if (P.mode == kPassPolish && __ldcg(&P.state->stop)) return;                 // (the same for all CTAs: set by an earlier launch)
+    const uint32_t v0 = uint32_t(uint64_t(P.n_blocks) * part / P.ctas), v1 = uint32_t(uint64_t(P.n_blocks) * (part + 1u) / P.ctas);
+    uint32_t v = v0 + tid;                                                       // (n_blocks < 2^31: see the launcher)
+    uint32_t i = v / P.per_row, col = v - i * P.per_row;                         // rows of later blocks follow without divisions
     const uint32_t row_step = kCountThreads / P.per_row, col_step = kCountThreads % P.per_row;
     float4 lo4 = make_float4(0.f, 0.f, 0.f, 0.f), hi4 = lo4;
     float mu = 1.0f;
     auto load = [&]() {
-        const uint64_t r = P.rows ? P.rows[i] : i;
-        const float4 *src = reinterpret_cast<const float4 *>(P.W + r * P.C + 8ull * col);
+        const uint32_t r = P.rows ? __ldg(P.rows + i) : i;
+        const float4 *src = reinterpret_cast<const float4 *>(P.W + size_t(r) * P.C) + 2u * col;
         lo4 = __ldg(src);
         hi4 = __ldg(src + 1);
         mu = __ldg(P.mu + r);
     };
     if (v < v1) load();
-    for (uint32_t k = tid; k < (kHotWords + kWinWords) / 4u; k += kCountThreads) reinterpret_cast<uint4 *>(sm)[k] = make_uint4(0u, 0u, 0u, 0u);
+    for (uint32_t j = tid; j < (kHotWords + kWinWords) / 4u; j += kCountThreads) reinterpret_cast<uint4 *>(sm)[j] = make_uint4(0u, 0u, 0u, 0u);
     if (tid < EP_NUM_TABLES) { range_from[tid] = 0; range_to[tid] = 0; }
-    const float s = P.s_from_state ? __ldcg(&P.state->s) : P.s;
+    if (tid == 0) {
+        if (P.mode == kPassSearch) {
+            double lo = P.first ? P.lo0 : __ldcg(&P.state->lo), hi = P.first ? P.hi0 : __ldcg(&P.state->hi);
+            bracket_of(k, lo, hi);
+            s_shared = __double2float_rn(__dsqrt_rn(__dmul_rn(lo, hi)));
+        } else {
+            s_shared = P.mode == kPassPolish ? __ldcg(&P.state->s) : P.s;
+        }
+    }
     __syncthreads();
+    const float s = s_shared;
     uint32_t halves = 0, blocks = 0;
     auto count_far = [&](uint32_t t, int32_t value) {          // outside the columns
         const uint32_t w = uint32_t(value - kWinOrigin), g = uint32_t(value - kHistOrigin);
         if (w < uint32_t(kWinBins)) {
             atomicAdd(&win[t * kWinBins + w], 1u);
         } else if (g < uint32_t(kHistBins)) {
-            atomicAdd(&P.hist[t * kHistBins + g], 1u);
+            atomicAdd(P.hist + (k * EP_NUM_TABLES + t) * kHistBins + g, 1u);
             atomicMax(&range_from[t], kHistBins - g);
             atomicMax(&range_to[t], g + 1u);
         } else {
-            P.state->overflow = 1;
+            S.overflow = 1;
         }
     };
     while (v < v1) {
         const float x[8] = {lo4.x, lo4.y, lo4.z, lo4.w, hi4.x, hi4.y, hi4.z, hi4.w};
         const float m = mu;
-        const uint64_t here = v;
+        const uint32_t here = v;
         v += kCountThreads;
         i += row_step;
         col += col_step;
         if (col >= P.per_row) { col -= P.per_row; ++i; }
         if (v < v1) load();                                    // the next block is on its way while this one is worked on
-        int32_t z[8];
-        uint32_t half;
+        uint32_t z[8], half;                                   // coordinates as bits of 1.5 * 2^23 + z
         const float ms = __fmul_rn(m, s);
-        bool ok = quantise_fast(x, __frcp_rn(ms), z, half) && ms >= 1e-30f && ms <= 1e30f;
+        const bool ok = quantise_fast(x, rcp_approx(ms), z, half) && ms >= 1e-30f && ms <= 1e30f;
         if (!ok) {
             float xs[8];
             int32_t zs[8];
 #pragma unroll
-            for (int k = 0; k < 8; ++k) xs[k] = x[k];
+            for (int j = 0; j < 8; ++j) xs[j] = x[j];
             const int c = quantise_exact(xs, m, s, zs);
-            if (c < 0) { P.state->overflow = 1; continue; }
+            if (c < 0) { S.overflow = 1; continue; }
             half = uint32_t(c);
 #pragma unroll
-            for (int k = 0; k < 8; ++k) z[k] = zs[k];
+            for (int j = 0; j < 8; ++j) z[j] = 0x4B400000u + uint32_t(zs[j]);
         }
-        // Eq. 4: m = (z8 - parity of z1 + ... + z7) / 2
-        z[7] = (z[7] - ((z[0] ^ z[1] ^ z[2] ^ z[3] ^ z[4] ^ z[5] ^ z[6]) & 1)) >> 1;
-        if (P.fields) {
-            auto two = [](int32_t a, int32_t b) { return (uint32_t(a) & 0xFFFFu) | (uint32_t(b) << 16); };
-            P.fields[here] = make_uint4(two(z[0], z[1]), two(z[2], z[3]), two(z[4], z[5]), two(z[6], 2 * z[7] + int32_t(half)));
+        // Eq. 4: m = (z8 - parity of z1 + ... + z7) / 2; `mc` = 2 m + c
+        const uint32_t odd = (z[0] ^ z[1] ^ z[2] ^ z[3] ^ z[4] ^ z[5] ^ z[6]) & 1u;
+        const int32_t m2 = int32_t(z[7] - odd - 0x4B400000u);
+        z[7] = 0x4B400000u + uint32_t(m2 >> 1);
+        if (P.fields) {                                        // (0x4B400000 has no bits below 2^22: the low halves are the values')
+            P.fields[here] = make_uint4(__byte_perm(z[0], z[1], 0x5410), __byte_perm(z[2], z[3], 0x5410), __byte_perm(z[4], z[5], 0x5410),
+                                        __byte_perm(z[6], uint32_t(m2) + half, 0x5410));
         }
         ++blocks;
         halves += half;
-        uint32_t *const column = hot + half * (8u * kHotBins * 32u) + lane;
+        uint32_t *const column = hot + (half ? 8u * kHotStride : 0u) + lane;
+        uint32_t far = 0;
 #pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            const uint32_t u = uint32_t(z[k] - kHotOrigin);
-            if (u < uint32_t(kHotBins)) atomicAdd(column + (uint32_t(k) * kHotBins + u) * 32u, 1u);
-            else count_far(1u + 8u * half + uint32_t(k), z[k]);
+        for (int j = 0; j < 8; ++j) {
+            const uint32_t u = min(z[j] - (0x4B400000u + uint32_t(kHotOrigin)), uint32_t(kHotBins));
+            far |= u;
+            atomicAdd(column + uint32_t(j) * kHotStride + u * 32u, 1u);
+        }
+        if (far & uint32_t(kHotBins)) {
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                const int32_t value = int32_t(z[j] - 0x4B400000u);
+                if (uint32_t(value - kHotOrigin) >= uint32_t(kHotBins)) count_far(1u + 8u * half + uint32_t(j), value);
+            }
         }
     }
     // the coset table
@@ -492,35 +674,56 @@ __global__ void __launch_bounds__(kCountThreads, 1) quantise_count_kernel(const 
         if (halves) atomicAdd(&win[1 - kWinOrigin], halves);
     }
     __syncthreads();
-    // columns into the window (one thread per value), then the window into global memory
-    for (uint32_t k = tid; k < 16u * kHotBins; k += kCountThreads) {
+    // columns into the window (two threads per value), then the window into global memory
+    {
+        const uint32_t bin = tid >> 1, t = bin / kHotBins, u = bin % kHotBins;
+        static_assert(16u * kHotBins * 2u == kCountThreads, "two threads per value");
         uint32_t n = 0;
 #pragma unroll
-        for (uint32_t j = 0; j < 32; ++j) n += hot[32u * k + ((j + tid) & 31u)];
-        if (n) atomicAdd(&win[(1u + k / kHotBins) * kWinBins + uint32_t(int32_t(k % kHotBins) + kHotOrigin - kWinOrigin)], n);
+        for (uint32_t j = 0; j < 16; ++j) n += hot[t * kHotStride + u * 32u + ((j + (tid >> 1)) & 15u) + 16u * (tid & 1u)];
+        if (n) atomicAdd(&win[(1u + t) * kWinBins + uint32_t(int32_t(u) + kHotOrigin - kWinOrigin)], n);
     }
     __syncthreads();
-    for (uint32_t k = tid; k < kWinWords; k += kCountThreads) {
-        const uint32_t n = win[k];
+    for (uint32_t j = tid; j < kWinWords; j += kCountThreads) {
+        const uint32_t n = win[j];
         if (n) {
-            const uint32_t t = k / kWinBins, g = k % kWinBins + uint32_t(kWinOrigin - kHistOrigin);
-            atomicAdd(&P.hist[t * kHistBins + g], n);
+            const uint32_t t = j / kWinBins, g = j % kWinBins + uint32_t(kWinOrigin - kHistOrigin);
+            atomicAdd(P.hist + (k * EP_NUM_TABLES + t) * kHistBins + g, n);
             atomicMax(&range_from[t], kHistBins - g);
             atomicMax(&range_to[t], g + 1u);
         }
     }
     __syncthreads();
     if (tid < EP_NUM_TABLES && range_to[tid]) {
-        atomicMax(&P.state->from[tid], range_from[tid]);
-        atomicMax(&P.state->to[tid], range_to[tid]);
+        atomicMax(&S.from[tid], range_from[tid]);
+        atomicMax(&S.to[tid], range_to[tid]);
     }
     __threadfence();
     __syncthreads();
-    if (tid == 0) last_cta = atomicAdd(&P.state->finished, 1u) == gridDim.x - 1u;
+    if (tid == 0) last_cta = atomicAdd(&S.finished, 1u) == P.ctas - 1u;
     __syncthreads();
     if (!last_cta) return;
     __threadfence();
-    close_pass(P, sm);
+    const Evaluation E = gather_counts(P, k, P.mode == kPassSearch ? P.cand_counts + size_t(k) * kEvalSymbols : P.full_counts, sm);
+    if (P.mode == kPassSearch) {
+        if (tid == 0) judge_candidate(P, k, E);
+        __threadfence();
+        __syncthreads();
+        if (tid == 0) last_cta = atomicAdd(&P.state->closed, 1u) == (1u << P.levels) - 2u;
+        __syncthreads();
+        if (!last_cta) return;
+        __threadfence();
+        walk_tree(P);
+        return;
+    }
+    if (tid < EP_NUM_TABLES) {
+        P.state->full.lo[tid] = S.dir.lo[tid];
+        P.state->full.K[tid] = S.dir.K[tid];
+    }
+    if (tid == 0) {
+        if (__ldcg(&S.overflow)) P.state->overflow = 1;
+        if (P.mode == kPassPolish) polish(P, s, E);
+    }
 }
 
 // ---- Eq. 13: row scales ----------------------------------------------------------------------------------
@@ -605,86 +808,83 @@ __global__ void __launch_bounds__(kRowThreads) refit_kernel(const float *__restr
 }
 
 // ---- tile coding (Sec. 3.6 / App. "Tiled rANS implementation", Eq. 17) ---------------------------------------
+// Symbols' entries by (coset, field, value): the two cosets' tables of a field have the same range here (the wider of
+// both ends), so that the second coset's entries follow at one distance.
 struct EncodeTables {
-    int32_t base[EP_NUM_TABLES];     // entry of table t's value v: base[t] + v
-    uint32_t total;                  // sum of K
+    uint32_t base[9];                // byte offset of value 0's entry of field k (0: the coset) under coset 0, modulo 2^32
+    uint32_t coset;                  // bytes from coset 0's entries to coset 1's
+    uint32_t total;                  // entries
 };
 
 // What Eq. 17 needs of a symbol, without a division: x / f for x < 2^31 is umulhi(x, rcp) >> sh with
 // sh = ceil(log2 f) - 1 and rcp = ceil(2^(32 + sh) / f) (Granlund and Montgomery, "Division by invariant integers using
 // multiplication", 1994; exact for 31-bit x).  f = 1 takes rcp = 2^32 - 1, which gives x - 1, and an offset that
 // makes up for it.  With q = x / f the new state is q 2^b + x mod f + F = x + (2^b - f) q + F.
-__device__ __forceinline__ uint2 encode_entry(uint32_t f, uint32_t F, uint32_t b) {
-    const uint32_t M = 1u << b;
-    if (f <= 1u) return make_uint2(0xFFFFFFFFu, (M - 1u) | ((F + M - 1u) << 16));
+// {rcp, first state that gives off a word: f 2^(31-b), 2^b - f, sh | offset << 16}
+__device__ __forceinline__ uint4 encode_entry(uint32_t fF, uint32_t b) {
+    const uint32_t M = 1u << b, f = max(fF & 0xFFFFu, 1u), F = fF >> 16;
+    if (f == 1u) return make_uint4(0xFFFFFFFFu, 1u << (31u - b), M - 1u, (F + M - 1u) << 16);
     const uint32_t sh = 31u - __clz(int(f - 1u));
     // (the quotient has at most 32 integer bits and a fraction of at least 1 / f: its ceiling is right in double)
     const uint32_t rcp = uint32_t(ceil(__ddiv_rn(double(1ull << (32u + sh)), double(f))));
-    return make_uint2(rcp, (M - f) | (F << 16));
+    return make_uint4(rcp, f << (31u - b), M - f, sh | (F << 16));
 }
 
 // One warp per tile, one state per lane.  The decoder reads, per (group, field), the words of the needy lanes in
 // ascending lane order; the encoder walks groups and fields backwards and fills the tile's word area from its end, writing
 // each step's words as one block in ascending lane order, which is the order the reversed word list of a sequential
 // encoder would have.  A step's chain is compare, shift, multiply-high, shift, multiply-add (about 30 cycles);
-// a group's symbols are loaded one group ahead and looked up before the steps that need them.
-// IN_SMEM: the entries in shared memory (up to 24 Ki symbols), else in global memory.  A CTA has four warps - tiles spread
-// over the SMs - or sixteen where its table takes so much shared memory that few CTAs fit an SM.
-constexpr uint32_t kTileThreads = 128, kTileThreadsMax = 512, kSmemEntries = 24576;
+// a group's fields are loaded one group ahead and its symbols looked up before the steps that need them.
+// IN_SMEM: the symbols' entries in shared memory (up to 12 Ki symbols), else in global memory.  A CTA has four warps -
+// tiles spread over the SMs - or sixteen where its table takes so much shared memory that few CTAs fit an SM.
+constexpr uint32_t kTileThreads = 128, kTileThreadsMax = 512, kSmemEntries = 12288;
 
 template <bool IN_SMEM>
 __global__ void __launch_bounds__(kTileThreadsMax) tile_encode_kernel(const uint4 *__restrict__ fields, uint32_t n_vec, uint32_t V,
                                                                       uint32_t n_tiles, uint32_t b, const __grid_constant__ EncodeTables T,
-                                                                      const uint32_t *__restrict__ fF, uint2 *__restrict__ entries_global,
+                                                                      const uint32_t *__restrict__ fF, const uint4 *__restrict__ entries_global,
                                                                       uint16_t *__restrict__ scratch, uint32_t cap,
                                                                       uint32_t *__restrict__ index, uint32_t *__restrict__ counts, SearchState *state) {
-    extern __shared__ __align__(8) uint2 entries_smem[];
+    extern __shared__ __align__(16) uint4 entries_smem[];
     __shared__ uint32_t last_cta, part[kTileThreadsMax];
     const uint32_t tid = threadIdx.x, lane = tid & 31u;
     if (IN_SMEM) {
-        for (uint32_t i = tid; i < T.total; i += blockDim.x) {
-            const uint32_t e = __ldg(fF + i);
-            entries_smem[i] = encode_entry(e & 0xFFFFu, e >> 16, b);
-        }
+        for (uint32_t i = tid; i < T.total; i += blockDim.x) entries_smem[i] = encode_entry(__ldg(fF + i), b);
         __syncthreads();
     }
-    const uint2 *const entries = IN_SMEM ? entries_smem : entries_global;
+    const uint8_t *const entries = reinterpret_cast<const uint8_t *>(IN_SMEM ? entries_smem : entries_global);
     const uint32_t tile = blockIdx.x * (blockDim.x >> 5) + (tid >> 5);
     if (tile < n_tiles) {
-        const uint32_t v0 = tile * V, nv = min(V, n_vec - v0), lt = (1u << lane) - 1u, last_entry = T.total - 1u;
+        const uint32_t v0 = tile * V, nv = min(V, n_vec - v0), lt = (1u << lane) - 1u;
         const uint4 *const q = fields + v0;
         uint16_t *const area = scratch + size_t(tile) * cap;
         uint32_t end = cap;                      // words [end, cap) of the area are written
         uint32_t x = kStateLow;
         const uint32_t groups = (nv + 31u) >> 5;
-        const uint32_t M = 1u << b, top = 31u - b;
         uint4 next = __ldg(q + min((groups - 1u) * 32u + lane, nv - 1u));
         for (uint32_t g = groups; g-- > 0;) {
             const uint4 cur = next;
-            const bool act = g * 32u + lane < nv;
             if (g) next = __ldg(q + (g - 1u) * 32u + lane);
-            const int32_t mc = field16(cur.w, 1), c = mc & 1;
-            const uint32_t w[4] = {cur.x, cur.y, cur.z, cur.w};
-            uint2 e[9];
-            // (every index is in range by construction; clamped anyway)
-            e[0] = entries[min(uint32_t(T.base[0] + c), last_entry)];
+            const int32_t mc = field16(cur.w, 1);
+            const uint32_t w[4] = {cur.x, cur.y, cur.z, cur.w}, coset = (mc & 1) ? T.coset : 0u;
+            uint4 e[9];                          // (every offset is in range: these are the fields the tables were counted from)
+            e[0] = *reinterpret_cast<const uint4 *>(entries + (T.base[0] + 16u * uint32_t(mc & 1)));
 #pragma unroll
             for (int k = 1; k < 8; ++k)
-                e[k] = entries[min(uint32_t((c ? T.base[8 + k] : T.base[k]) + field16(w[(k - 1) >> 1], (k - 1) & 1)), last_entry)];
-            e[8] = entries[min(uint32_t((c ? T.base[16] : T.base[8]) + (mc >> 1)), last_entry)];
+                e[k] = *reinterpret_cast<const uint4 *>(entries + (T.base[k] + coset + 16u * uint32_t(field16(w[(k - 1) >> 1], (k - 1) & 1))));
+            e[8] = *reinterpret_cast<const uint4 *>(entries + (T.base[8] + coset + 16u * uint32_t(mc >> 1)));
+            if (g * 32u + lane >= nv) {          // no block (the tile's last group): the state stays, no word
+#pragma unroll
+                for (int k = 0; k < 9; ++k) e[k] = make_uint4(0u, 0xFFFFFFFFu, 0u, 0u);
+            }
 #pragma unroll
             for (int k = 8; k >= 0; --k) {
-                const uint32_t comp = e[k].y & 0xFFFFu, f = M - comp;                      // 2^b - f
-                const uint32_t sh = f > 1u ? 31u - __clz(int(f - 1u)) : 0u;
-                const bool emit = act && x >= (f << top);                                // f 2^(31-b) <= 2^31 fits 32 bits
-                const uint32_t bal = __ballot_sync(0xFFFFFFFFu, emit);
-                end -= __popc(bal);                                                      // at most nine words per block: the area holds them
-                if (emit) {
-                    area[end + __popc(bal & lt)] = uint16_t(x);
-                    x >>= 16;
-                }
-                const uint32_t quot = __umulhi(x, e[k].x) >> sh;
-                if (act) x = quot * comp + (x + (e[k].y >> 16));                         // Eq. 17
+                const bool emit = x >= e[k].y;
+                const uint32_t bal = __ballot_sync(0xFFFFFFFFu, emit), word = x;
+                if (emit) x >>= 16;
+                x = __funnelshift_r(__umulhi(x, e[k].x), 0u, e[k].w) * e[k].z + (x + (e[k].w >> 16));   // Eq. 17 (the shift takes sh)
+                end -= __popc(bal);              // at most nine words per block: the area holds them
+                if (emit) area[end + __popc(bal & lt)] = uint16_t(word);
             }
         }
         index[size_t(tile) * 33u + lane] = x;
@@ -718,23 +918,23 @@ __global__ void __launch_bounds__(kTileThreadsMax) tile_encode_kernel(const uint
 }
 
 // entries of an alphabet too large for shared memory
-__global__ void encode_entries_kernel(const uint32_t *__restrict__ fF, uint32_t n, uint32_t b, uint2 *__restrict__ entries) {
+__global__ void encode_entries_kernel(const uint32_t *__restrict__ fF, uint32_t n, uint32_t b, uint4 *__restrict__ entries) {
     const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) entries[i] = encode_entry(fF[i] & 0xFFFFu, fF[i] >> 16, b);
+    if (i < n) entries[i] = encode_entry(fF[i], b);
 }
 
-// move every tile's words from the end of its area to its place in the payload: one warp per tile, four bytes per lane
-// where the destination is aligned for it
-__global__ void __launch_bounds__(256) compact_kernel(const uint16_t *__restrict__ scratch, uint32_t cap, const uint32_t *__restrict__ counts,
-                                                      const uint32_t *__restrict__ index, uint32_t n_tiles, uint16_t *__restrict__ payload) {
-    const uint32_t lane = threadIdx.x & 31u;
-    const uint32_t tile = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (tile >= n_tiles) return;
+// Move every tile's words from the end of its area to its place in the payload: one CTA per tile (with a warp per tile the
+// copy of 20 MB took 34 us, all of it waiting for loads), four bytes per lane, the destination aligned.
+constexpr uint32_t kCompactThreads = 128;
+__global__ void __launch_bounds__(kCompactThreads) compact_kernel(const uint16_t *__restrict__ scratch, uint32_t cap,
+                                                                  const uint32_t *__restrict__ counts, const uint32_t *__restrict__ index,
+                                                                  uint16_t *__restrict__ payload) {
+    const uint32_t tid = threadIdx.x, tile = blockIdx.x;
     uint32_t n = counts[tile];
     const uint16_t *src = scratch + size_t(tile) * cap + (cap - n);
     uint16_t *dst = payload + index[size_t(tile) * 33u + 32u];
     if (n && (reinterpret_cast<uintptr_t>(dst) & 2)) {
-        if (lane == 0) *dst = *src;
+        if (tid == 0) *dst = *src;
         ++src; ++dst; --n;
     }
     uint32_t *const d32 = reinterpret_cast<uint32_t *>(dst);
@@ -743,22 +943,22 @@ __global__ void __launch_bounds__(256) compact_kernel(const uint16_t *__restrict
         // each pair straddles two aligned words (the one before src starts inside the buffer, as src is not its start)
         const uint32_t *s32 = reinterpret_cast<const uint32_t *>(src - 1);
 #pragma unroll 4
-        for (uint32_t i = lane; i < pairs; i += 32u) d32[i] = __funnelshift_r(s32[i], s32[i + 1u], 16);
+        for (uint32_t i = tid; i < pairs; i += kCompactThreads) d32[i] = __funnelshift_r(s32[i], s32[i + 1u], 16);
     } else {
         const uint32_t *s32 = reinterpret_cast<const uint32_t *>(src);
 #pragma unroll 4
-        for (uint32_t i = lane; i < pairs; i += 32u) d32[i] = s32[i];
+        for (uint32_t i = tid; i < pairs; i += kCompactThreads) d32[i] = s32[i];
     }
-    if ((n & 1u) && lane == 0) dst[n - 1u] = src[n - 1u];
+    if ((n & 1u) && tid == 0) dst[n - 1u] = src[n - 1u];
 }
 
 size_t align_up(size_t v) { return (v + 255) & ~size_t(255); }
 
 struct Workspace {
     float *mu;
-    uint32_t *rows, *hist, *counts, *fF, *last_counts, *full_counts;
+    uint32_t *rows, *hist, *counts, *fF, *cand_counts, *last_counts, *full_counts;
     SearchState *state;
-    uint2 *entries;
+    uint4 *entries;
     uint4 *fields;
     uint16_t *scratch;
     // the last three sections of the blob, back to back as they are stored: row scales, tile index, payload
@@ -779,13 +979,14 @@ Workspace carve(uint8_t *base, uint32_t R, uint32_t C, uint32_t V) {
     Workspace w{};
     w.mu = reinterpret_cast<float *>(take(4ull * R));
     w.rows = reinterpret_cast<uint32_t *>(take(4ull * R));
-    // state, then the counts of the last step, so that one copy brings both; histogram after them
+    // state, then the counts of the last step, so that one copy brings both
     w.state = reinterpret_cast<SearchState *>(take(kStateBytes + 4ull * kEvalSymbols));
     w.last_counts = reinterpret_cast<uint32_t *>(reinterpret_cast<uint8_t *>(w.state) + kStateBytes);
-    w.hist = reinterpret_cast<uint32_t *>(take(kHistBytes));
+    w.hist = reinterpret_cast<uint32_t *>(take(kCandidates * kHistBytes));
+    w.cand_counts = reinterpret_cast<uint32_t *>(take(4ull * kCandidates * kEvalSymbols));
     w.full_counts = reinterpret_cast<uint32_t *>(take(kHistBytes));
-    w.fF = reinterpret_cast<uint32_t *>(take(4ull * kMaxTableSymbols));
-    w.entries = reinterpret_cast<uint2 *>(take(8ull * kMaxTableSymbols));
+    w.fF = reinterpret_cast<uint32_t *>(take(4ull * kMaxEntries));
+    w.entries = reinterpret_cast<uint4 *>(take(16ull * kMaxEntries));
     w.counts = reinterpret_cast<uint32_t *>(take(4ull * n_tiles));
     w.fields = reinterpret_cast<uint4 *>(take(16ull * nvec));
     w.scratch = reinterpret_cast<uint16_t *>(take(2ull * cap * n_tiles + 4));
@@ -865,7 +1066,7 @@ public:
         EP_CUDA(cudaFuncSetAttribute(quantise_count_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kCountSmem)));
         EP_CUDA(cudaMemcpyAsync(w_.rows, sample.data(), 4ull * n_sample_, cudaMemcpyHostToDevice, st_));
         EP_CUDA(cudaMemsetAsync(w_.state, 0, kStateBytes, st_));
-        EP_CUDA(cudaMemsetAsync(w_.hist, 0, kHistBytes, st_));       // every pass leaves it zero again
+        EP_CUDA(cudaMemsetAsync(w_.hist, 0, kCandidates * kHistBytes, st_));       // every pass leaves it zero again
         row_rms_kernel<<<R_, kRowThreads, 0, st_>>>(W_, C_, w_.mu);
         EP_CUDA(cudaGetLastError());
         return EP_OK;
@@ -876,25 +1077,37 @@ public:
     int search(const SearchJob &job, const ep_encode_opts &o, SearchResult &r, bool *done) override {
         *done = false;
         EP_CUDA(cudaMemsetAsync(w_.state, 0, kStateBytes, st_));
-        CountParams P = params(w_.rows, n_sample_, float(std::sqrt(o.bracket_lo * o.bracket_hi)), nullptr);
-        const double n_tile = double((job.sample_vectors + job.V - 1) / job.V);
-        P.step = {job.target_bpp, o.retained_bits * double(kStates) * n_tile,
-                  n_tile * (32.0 * kStates + 32.0) + 32.0 + 32.0 * double(job.sample_rows) + 8.0 * kHeaderBytes,
-                  8.0 * double(job.sample_vectors), 9.0 * double(job.sample_vectors), o.bracket_lo, o.bracket_hi, job.b, 0};
-        for (int it = 0; it < o.search_steps; ++it) {
-            P.step.step = it;
-            P.s_from_state = it > 0;
+        CountParams P = params(w_.rows, n_sample_, 0.0f, nullptr);
+        P.mode = kPassSearch;
+        P.rate = rate_params(job.target_bpp, o.retained_bits, job.sample_vectors, job.sample_rows, job.V, job.b);
+        P.lo0 = o.bracket_lo;
+        P.hi0 = o.bracket_hi;
+        const float s0 = float(std::sqrt(o.bracket_lo * o.bracket_hi));
+        if (o.search_steps == 0) EP_CUDA(cudaMemcpyAsync(&w_.state->s, &s0, 4, cudaMemcpyHostToDevice, st_));
+        P.first = 1;
+        for (int left = o.search_steps, pass = 0; left > 0; ++pass) {
+            P.levels = uint32_t(std::min<int>(left, std::min<int>(pass + 1, kLevels)));
             launch_count(P);
+            left -= int(P.levels);
+            P.first = 0;
         }
-        CountParams F = params(nullptr, R_, P.s, w_.fields);
-        F.s_from_state = o.search_steps > 0;
-        launch_count(F);
+        CountParams F = params(nullptr, R_, 0.0f, w_.fields);
+        F.mode = kPassPolish;
+        F.rate = rate_params(job.target_bpp, o.polish_retained_bits, F.n_blocks, R_, job.V, job.b);
+        F.lo0 = o.bracket_lo;
+        F.hi0 = o.bracket_hi;
+        F.last_step = o.polish_steps;
+        for (F.step = 0; F.step <= o.polish_steps; ++F.step) launch_count(F);
         EP_CUDA(cudaGetLastError());
         const int rc = fetch(true);
         if (rc) return rc;
         const SearchState &S = *state();
-        if (S.undecided || S.has_last == 2) return EP_OK;
-        r.s = o.search_steps > 0 ? S.s : P.s;
+        if (S.undecided) {
+            EP_CUDA(cudaMemsetAsync(w_.state, 0, kStateBytes, st_));
+            return EP_OK;
+        }
+        r.s = S.s_counted;
+        r.polished = S.polished != 0;
         r.has_last = S.has_last != 0;
         if (r.has_last) r.last.from_counts(S.last.lo, S.last.K, last_counts());
         r.full.from_counts(S.full.lo, S.full.K, full_counts());
@@ -902,25 +1115,51 @@ public:
         return EP_OK;
     }
 
-    int finish(float s, int b, uint32_t V, const Model &m, ep_blob *out) override {
+    int begin_finish(float s, int b, uint32_t V, const Model &m) override {
         const uint64_t nvec = uint64_t(R_) * (C_ / 8);
         const uint32_t n_tiles = uint32_t((nvec + V - 1) / V);
         const uint32_t cap = 9u * V;
-        EncodeTables T{};
-        std::vector<uint32_t> fF;
-        for (int t = 0; t < EP_NUM_TABLES; ++t) {
-            T.base[t] = int32_t(fF.size()) - m.t[t].lo;
-            for (uint32_t j = 0; j < m.t[t].K(); ++j) fF.push_back(m.t[t].f[j] | (m.t[t].F[j] << 16));
+        uint64_t symbols = 0;
+        for (int t = 0; t < EP_NUM_TABLES; ++t) symbols += m.t[t].K();
+        if (symbols > kMaxTableSymbols) return EP_ERR_UNSUPPORTED;
+        // per field the range of both cosets' tables
+        int32_t lo[9], hi[9];
+        uint32_t first[9], size = 0;
+        for (int k = 0; k < 9; ++k) {
+            lo[k] = hi[k] = 0;                   // (k = 0: the coset itself, 0 or 1)
+            bool any = false;
+            for (int c = 0; c < 2 && k > 0; ++c) {
+                const Table &tb = m.t[table_id(c, k)];
+                if (!tb.K()) continue;
+                lo[k] = any ? std::min(lo[k], tb.lo) : tb.lo;
+                hi[k] = any ? std::max(hi[k], tb.lo + int32_t(tb.K())) : tb.lo + int32_t(tb.K());
+                any = true;
+            }
+            if (k == 0) continue;
+            first[k] = size;
+            size += uint32_t(hi[k] - lo[k]);
         }
-        T.total = uint32_t(fF.size());
-        if (T.total > kMaxTableSymbols) return EP_ERR_UNSUPPORTED;
+        EncodeTables T{};
+        T.coset = 16u * size;
+        T.total = 2u * size + 2u;
+        std::vector<uint32_t> fF(T.total, 0);
+        for (int k = 1; k < 9; ++k) {
+            T.base[k] = 16u * (first[k] - uint32_t(lo[k]));
+            for (int c = 0; c < 2; ++c) {
+                const Table &tb = m.t[table_id(c, k)];
+                uint32_t *to = fF.data() + uint32_t(c) * size + first[k] + uint32_t(tb.lo - lo[k]);
+                for (uint32_t j = 0; j < tb.K(); ++j) to[j] = tb.f[j] | (tb.F[j] << 16);
+            }
+        }
+        T.base[0] = 32u * size;                  // the coset's two entries last
+        for (uint32_t j = 0; j < m.t[0].K(); ++j) fF[2u * size + uint32_t(m.t[0].lo) + j] = m.t[0].f[j] | (m.t[0].F[j] << 16);
         EP_CUDA(cudaMemcpyAsync(w_.fF, fF.data(), 4ull * fF.size(), cudaMemcpyHostToDevice, st_));
         EP_CUDA(cudaMemsetAsync(&w_.state->tiles_done, 0, 4, st_));
         if (T.total <= kSmemEntries) {
-            const size_t smem = 8ull * T.total;
-            const uint32_t threads = T.total <= 4096u ? kTileThreads : kTileThreadsMax;
+            const size_t smem = 16ull * T.total;
+            const uint32_t threads = T.total <= 2048u ? kTileThreads : kTileThreadsMax;
             if (smem > 40u * 1024u)      // (always the same limit: another thread's call must not lower it before the launch)
-                EP_CUDA(cudaFuncSetAttribute(tile_encode_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(8u * kSmemEntries)));
+                EP_CUDA(cudaFuncSetAttribute(tile_encode_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(16u * kSmemEntries)));
             tile_encode_kernel<true><<<(n_tiles + threads / 32u - 1u) / (threads / 32u), threads, smem, st_>>>(
                 w_.fields, uint32_t(nvec), V, n_tiles, uint32_t(b), T, w_.fF, w_.entries, w_.scratch, cap, w_.index, w_.counts, w_.state);
         } else {
@@ -928,10 +1167,13 @@ public:
             tile_encode_kernel<false><<<(n_tiles + kTileThreads / 32u - 1u) / (kTileThreads / 32u), kTileThreads, 0, st_>>>(
                 w_.fields, uint32_t(nvec), V, n_tiles, uint32_t(b), T, w_.fF, w_.entries, w_.scratch, cap, w_.index, w_.counts, w_.state);
         }
-        compact_kernel<<<(n_tiles + 7) / 8, 256, 0, st_>>>(w_.scratch, cap, w_.counts, w_.index, n_tiles, w_.payload);
+        compact_kernel<<<n_tiles, kCompactThreads, 0, st_>>>(w_.scratch, cap, w_.counts, w_.index, w_.payload);
         EP_CUDA(cudaMemcpyAsync(&state()->total_words, &w_.state->total_words, 4, cudaMemcpyDeviceToHost, st_));
         refit_kernel<<<R_, kRowThreads, 0, st_>>>(W_, C_, w_.fields, s, w_.mu, w_.sigma);
         EP_CUDA(cudaGetLastError());
+        return EP_OK;
+    }
+    int end_finish(float s, int b, uint32_t V, const Model &m, ep_blob *out) override {
         EP_CUDA(cudaStreamSynchronize(st_));
         const uint64_t total = state()->total_words;
         if (total >= (1ull << 31)) return EP_ERR_UNSUPPORTED;
@@ -963,16 +1205,25 @@ private:
         P.state = w_.state;
         P.last_counts = w_.last_counts;
         P.full_counts = w_.full_counts;
+        P.cand_counts = w_.cand_counts;
         P.per_row = C_ / 8;
-        P.n_blocks = uint64_t(n_rows) * P.per_row;
+        P.n_blocks = n_rows * P.per_row;
         P.C = C_;
+        P.mode = kPassCount;
+        P.levels = 1;
         P.s = s;
-        P.step.step = -1;
         return P;
     }
-    void launch_count(const CountParams &P) {
-        const uint32_t grid = uint32_t(std::min<uint64_t>((P.n_blocks + 255) / 256, uint64_t(sms_)));
-        quantise_count_kernel<<<grid, kCountThreads, kCountSmem, st_>>>(P);
+    static RateParams rate_params(double target, double retained, uint64_t n, uint64_t rows, uint32_t V, int b) {
+        const double tiles = double((n + V - 1) / V);
+        return {target, retained * double(kStates) * tiles, tiles * (32.0 * kStates + 32.0) + 32.0 + 32.0 * double(rows) + 8.0 * kHeaderBytes,
+                8.0 * double(n), 9.0 * double(n), b};
+    }
+    // one CTA per SM over all candidates of the pass, each with at least a few hundred blocks
+    void launch_count(CountParams P) {
+        const uint32_t cands = (1u << P.levels) - 1u;
+        P.ctas = std::max(1u, std::min((P.n_blocks + 255u) / 256u, uint32_t(sms_) / cands));
+        quantise_count_kernel<<<cands * P.ctas, kCountThreads, kCountSmem, st_>>>(P);
     }
     static size_t symbols(const CountDir &D) {
         size_t n = 0;
@@ -985,14 +1236,15 @@ private:
         EP_CUDA(cudaMemcpyAsync(full_counts(), w_.full_counts, 4ull * kFirstCounts, cudaMemcpyDeviceToHost, st_));
         EP_CUDA(cudaStreamSynchronize(st_));
         const SearchState &S = *state();
-        if (S.overflow) return EP_ERR_UNSUPPORTED;     // a coordinate beyond +-4095: use the host encoder
+        // (after a step it could not decide a search may have gone where the host's does not)
+        if (S.overflow && !(last && S.undecided)) return EP_ERR_UNSUPPORTED;     // a coordinate beyond +-4095: use the host encoder
         bool more = false;
         auto rest = [&](uint32_t *to, const uint32_t *from, size_t n) {
             if (n <= kFirstCounts) return cudaSuccess;
             more = true;
             return cudaMemcpyAsync(to + kFirstCounts, from + kFirstCounts, 4ull * (n - kFirstCounts), cudaMemcpyDeviceToHost, st_);
         };
-        if (last && S.has_last == 1) EP_CUDA(rest(last_counts(), w_.last_counts, symbols(S.last)));
+        if (last && S.has_last) EP_CUDA(rest(last_counts(), w_.last_counts, symbols(S.last)));
         EP_CUDA(rest(full_counts(), w_.full_counts, symbols(S.full)));
         if (more) EP_CUDA(cudaStreamSynchronize(st_));
         return EP_OK;
@@ -1038,7 +1290,7 @@ extern "C" int ep_encode_device(const float *d_W, uint32_t R, uint32_t C, double
     if (bad) return bad;
     if ((reinterpret_cast<uintptr_t>(d_W) & 15) || (reinterpret_cast<uintptr_t>(d_workspace) & 255)) return EP_ERR_BAD_ARG;
     const uint32_t V = tile_vectors_of(o, target_bpp);
-    if (uint64_t(V) * 9u >= (1ull << 31)) return EP_ERR_UNSUPPORTED;
+    if (uint64_t(V) * 9u >= (1ull << 31) || uint64_t(R) * (C / 8) >= (1ull << 31)) return EP_ERR_UNSUPPORTED;
     if (workspace_bytes < carve(nullptr, R, C, V).bytes) return EP_ERR_SCRATCH;
     try {
         DeviceBackend be(d_W, R, C, V, static_cast<uint8_t *>(d_workspace), static_cast<cudaStream_t>(stream));

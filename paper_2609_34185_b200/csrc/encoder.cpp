@@ -307,7 +307,9 @@ int run_encode(EncodeBackend &be, uint32_t R, uint32_t C, double target_bpp, con
     if (rc) return rc;
     float s = 0.0f;
     double last_rate = 0.0;
-    Model full;
+    Model full, last_step;       // last_step: counts of the last candidate a back end evaluated in a search of its own,
+    int last_b = 0;              // and its precision (0: last_rate stands)
+    bool polished = false;
     for (;; ++b) {
         bool searched = false;
         SearchResult found;
@@ -315,9 +317,10 @@ int run_encode(EncodeBackend &be, uint32_t R, uint32_t C, double target_bpp, con
         if (searched) {
             s = found.s;
             full = std::move(found.full);
+            polished = found.polished;
             if (found.has_last) {
-                found.last.normalise(b);
-                last_rate = estimate_bits(found.last, b, svec, rows.size(), V, o.retained_bits, nullptr) / (8.0 * double(svec));
+                last_step = std::move(found.last);
+                last_b = b;
             }
         } else {
             double lo = o.bracket_lo, hi = o.bracket_hi;
@@ -331,6 +334,7 @@ int run_encode(EncodeBackend &be, uint32_t R, uint32_t C, double target_bpp, con
                 m.normalise(b);
                 const double bits = estimate_bits(m, b, svec, rows.size(), V, o.retained_bits, nullptr);
                 last_rate = bits / (8.0 * double(svec));
+                last_b = 0;
                 if (last_rate > target_bpp) lo = mid; else hi = mid;
             }
             s = float(std::sqrt(lo * hi));
@@ -339,6 +343,7 @@ int run_encode(EncodeBackend &be, uint32_t R, uint32_t C, double target_bpp, con
         bool fits = false;
         for (;;) {
             if (full.worst_observed() <= (1u << b)) { fits = true; break; }
+            polished = false;
             if (b < o.b_max) break;
             s = float(1.05 * double(s) * double(full.worst_coordinate_observed()) / double(1u << b));
             if ((rc = be.count_full(s, full))) return rc;
@@ -349,7 +354,7 @@ int run_encode(EncodeBackend &be, uint32_t R, uint32_t C, double target_bpp, con
     // law (Eq. 9), then by the measured slope.  The sampled tables miss rare symbols of the full tensor, which
     // costs rate on heavy tails.
     struct { double log_s, rate; bool valid; } last{0.0, 0.0, false};
-    for (int step = 0; step < o.polish_steps; ++step) {
+    for (int step = 0; step < o.polish_steps && !polished; ++step) {
         Model m = full;
         m.normalise(b);
         const double est = estimate_bits(m, b, nvec, R, V, o.polish_retained_bits, nullptr) / (double(R) * double(C));
@@ -378,15 +383,22 @@ int run_encode(EncodeBackend &be, uint32_t R, uint32_t C, double target_bpp, con
     }
     if (o.rdo_candidates > 1 && (rc = be.refine(s, b, V, o, full))) return rc;
     full.normalise(b);
+    if ((rc = be.begin_finish(s, b, V, full))) return rc;
+    // the report's figures, while the back end may be at work
+    const double cce = full.cross_entropy_bits(b);
+    if (last_b) {
+        last_step.normalise(last_b);
+        last_rate = estimate_bits(last_step, last_b, svec, rows.size(), V, o.retained_bits, nullptr) / (8.0 * double(svec));
+    }
     ep_blob *blob = new ep_blob();
-    rc = be.finish(s, b, V, full, blob);
+    rc = be.end_finish(s, b, V, full, blob);
     if (rc) { delete blob; return rc; }
     blob->report.s = double(s);
     blob->report.b = b;
     blob->report.bytes = blob->size();
     blob->report.stored_bpp = 8.0 * double(blob->size()) / (double(R) * double(C));
     blob->report.est_bpp_sample = last_rate;
-    blob->report.cce_bits = full.cross_entropy_bits(b);
+    blob->report.cce_bits = cce;
     blob->report.sample_rows = uint32_t(rows.size());
     *out = blob;
     return EP_OK;
@@ -578,7 +590,8 @@ public:
         m.count(fields_.data(), uint64_t(R_) * (C_ / 8), threads_);
         return EP_OK;
     }
-    int finish(float s, int b, uint32_t V, const Model &m, ep_blob *out) override {
+    int begin_finish(float, int, uint32_t, const Model &) override { return EP_OK; }
+    int end_finish(float s, int b, uint32_t V, const Model &m, ep_blob *out) override {
         std::vector<float> sigma(R_);
         if (refined_sigma_.empty()) refit(W_, R_, C_, fields_.data(), s, mu_.data(), sigma.data(), threads_);
         else sigma = refined_sigma_;

@@ -111,7 +111,8 @@ struct SearchJob {
     size_t sample_rows;
 };
 struct SearchResult {
-    float s = 0.0f;              // the scale the bisection ends on
+    float s = 0.0f;              // the scale the bisection, or the rate correction after it, ends on
+    bool polished = false;       // the rate correction is done as well
     Model last;                  // counts of the last candidate whose rate was evaluated
     bool has_last = false;
     Model full;                  // counts of the whole tensor at s (quantisation kept, as by count_full)
@@ -123,12 +124,14 @@ struct EncodeBackend {
     virtual int prepare(const std::vector<uint32_t> &sample) = 0;   // row RMS; remember the row sample
     virtual int count_sample(float s, Model &m) = 0;                // quantise the sample at s, count its fields
     virtual int count_full(float s, Model &m) = 0;                  // quantise the whole tensor at s (kept), count
-    // the bisection of Algorithm 1 on the row sample and the full-tensor pass at the scale it ends on, in one go.
+    // the bisection of Algorithm 1 on the row sample, the full-tensor pass at the scale it ends on and, if that fits the
+    // tables, the rate correction, in one go.
     // *done = false: not supported, or a decision the back end will not take; the driver then runs it step by step
     virtual int search(const SearchJob & /*job*/, const ep_encode_opts & /*o*/, SearchResult & /*r*/, bool *done) { *done = false; return EP_OK; }
-    // refit the row scales of the kept quantisation (Eq. 13), encode the tiles under the normalised
-    // full-tensor model m and assemble the blob
-    virtual int finish(float s, int b, uint32_t V, const Model &m, ep_blob *out) = 0;
+    // refit the row scales of the kept quantisation (Eq. 13), encode the tiles under the normalised full-tensor model m
+    // and assemble the blob; the driver has work of its own between the two calls
+    virtual int begin_finish(float s, int b, uint32_t V, const Model &m) = 0;
+    virtual int end_finish(float s, int b, uint32_t V, const Model &m, ep_blob *out) = 0;
     // per-row rate-distortion refinement of the kept quantisation (Sec. 3.5, Alg. 2); on success `m` holds the
     // counts of the refined fields and finish() uses the refined row scales.  Optional.
     virtual int refine(float /*s*/, int /*b*/, uint32_t /*V*/, const ep_encode_opts & /*o*/, Model & /*m*/) { return EP_ERR_UNSUPPORTED; }
