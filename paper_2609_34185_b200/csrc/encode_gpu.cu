@@ -319,6 +319,7 @@ struct CountParams {
     uint32_t n_blocks, C, per_row;
     uint32_t mode, levels, ctas;     // ctas: per candidate
     uint32_t first;                  // first pass of the search: the bracket is {lo0, hi0}; of the rate correction: step 0
+    uint32_t last_pass;              // last pass of the search
     float s;                         // mode kPassCount
     RateParams rate;
     double lo0, hi0;                 // the search bracket
@@ -471,19 +472,19 @@ __device__ __forceinline__ Evaluation gather_counts(const CountParams &P, uint32
 // per field, a few thousand additions).  How far the host's can be:
 __device__ __forceinline__ double cce_bound(const RateParams &P, double cce) { return 1e-11 * (cce + 16.0 * P.fields); }
 
-// thread 0 after a candidate of the search is gathered: is its rate above the target?
-__device__ void judge_candidate(const CountParams &P, uint32_t k, const Evaluation &E) {
-    uint32_t v = 0;
-    if (E.too_many) {
-        v = kUndecided;
-    } else if (E.worst > (1u << P.rate.b)) {
-        v = kAbove;                                              // no b-bit table exists for this scale: too fine
-    } else {
-        const double off = cce_bound(P.rate, E.cce);
-        auto above = [&](double cce) { return __ddiv_rn(bits_at(P.rate, E.tables, cce), P.rate.weights) > P.rate.target; };
-        v = kValid | (above(E.cce) ? kAbove : 0u) | (above(E.cce - off) != above(E.cce + off) ? kUndecided : 0u);
-    }
+// warp 0 after a candidate of the search is gathered: is its rate above the target?
+__device__ __forceinline__ void judge_candidate(const CountParams &P, uint32_t k, const Evaluation &E) {
+    // lane 1 at the estimate, lanes 0 and 2 at the ends of its interval
+    const uint32_t lane = threadIdx.x & 31u;
+    const double cce = E.cce + (double(lane) - 1.0) * cce_bound(P.rate, E.cce);
+    const bool above = __ddiv_rn(bits_at(P.rate, E.tables, cce), P.rate.weights) > P.rate.target;
+    const uint32_t b = __ballot_sync(0xFFFFFFFFu, above) & 7u;
+    if (lane != 0) return;
+    uint32_t v = kValid | ((b & 2u) ? kAbove : 0u) | ((b == 0u || b == 7u) ? 0u : kUndecided);
+    if (E.worst > (1u << P.rate.b)) v = kAbove;                  // no b-bit table exists for this scale: too fine
+    if (E.too_many) v = kUndecided;
     P.state->cand[k].verdict = v;
+    __threadfence();
 }
 
 // all threads of the pass's last CTA: the steps' outcomes in order
@@ -513,7 +514,8 @@ __device__ void walk_tree(const CountParams &P) {
         S.s = __double2float_rn(__dsqrt_rn(__dmul_rn(lo, hi)));
         S.closed = 0;
         if (last >= 0) S.has_last = 1;
-        chosen = last;
+        else if (P.last_pass && S.has_last) S.undecided = 1;     // (its counts are gone)
+        chosen = P.last_pass ? last : -1;
     }
     __syncthreads();
     if (chosen < 0) return;
@@ -576,7 +578,8 @@ __global__ void __launch_bounds__(kCountThreads, 1) quantise_count_kernel(const 
     const uint32_t tid = threadIdx.x, lane = tid & 31u;
     const uint32_t k = blockIdx.x / P.ctas, part = blockIdx.x - k * P.ctas;      // candidate, and this CTA's share of the blocks
     Candidate &S = P.state->cand[k];
-    if (P.mode == kPassPolish && __ldcg(&P.state->stop)) return;                 // (the same for all CTAs: set by an earlier launch)
+    // Launched before the previous pass has ended (see launch_count): only W, mu and rows, which are older than that, are
+    // read before the wait, and only then may the next launch come up.
     const uint32_t v0 = uint32_t(uint64_t(P.n_blocks) * part / P.ctas), v1 = uint32_t(uint64_t(P.n_blocks) * (part + 1u) / P.ctas);
     uint32_t v = v0 + tid;                                                       // (n_blocks < 2^31: see the launcher)
     uint32_t i = v / P.per_row, col = v - i * P.per_row;                         // rows of later blocks follow without divisions
@@ -593,6 +596,9 @@ __global__ void __launch_bounds__(kCountThreads, 1) quantise_count_kernel(const 
     if (v < v1) load();
     for (uint32_t j = tid; j < (kHotWords + kWinWords) / 4u; j += kCountThreads) reinterpret_cast<uint4 *>(sm)[j] = make_uint4(0u, 0u, 0u, 0u);
     if (tid < EP_NUM_TABLES) { range_from[tid] = 0; range_to[tid] = 0; }
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (P.mode == kPassPolish && __ldcg(&P.state->stop)) return;                 // (the same for all CTAs: set by an earlier launch)
     if (tid == 0) {
         if (P.mode == kPassSearch) {
             double lo = P.first ? P.lo0 : __ldcg(&P.state->lo), hi = P.first ? P.hi0 : __ldcg(&P.state->hi);
@@ -706,9 +712,7 @@ __global__ void __launch_bounds__(kCountThreads, 1) quantise_count_kernel(const 
     __threadfence();
     const Evaluation E = gather_counts(P, k, P.mode == kPassSearch ? P.cand_counts + size_t(k) * kEvalSymbols : P.full_counts, sm);
     if (P.mode == kPassSearch) {
-        if (tid == 0) judge_candidate(P, k, E);
-        __threadfence();
-        __syncthreads();
+        if (tid < 32u) judge_candidate(P, k, E);
         if (tid == 0) last_cta = atomicAdd(&P.state->closed, 1u) == (1u << P.levels) - 2u;
         __syncthreads();
         if (!last_cta) return;
@@ -852,7 +856,7 @@ __global__ void __launch_bounds__(kTileThreadsMax) tile_encode_kernel(const uint
         for (uint32_t i = tid; i < T.total; i += blockDim.x) entries_smem[i] = encode_entry(__ldg(fF + i), b);
         __syncthreads();
     }
-    const uint8_t *const entries = reinterpret_cast<const uint8_t *>(IN_SMEM ? entries_smem : entries_global);
+    const uint32_t entries = IN_SMEM ? uint32_t(__cvta_generic_to_shared(entries_smem)) : 0u;
     const uint32_t tile = blockIdx.x * (blockDim.x >> 5) + (tid >> 5);
     if (tile < n_tiles) {
         const uint32_t v0 = tile * V, nv = min(V, n_vec - v0), lt = (1u << lane) - 1u;
@@ -862,30 +866,44 @@ __global__ void __launch_bounds__(kTileThreadsMax) tile_encode_kernel(const uint
         uint32_t x = kStateLow;
         const uint32_t groups = (nv + 31u) >> 5;
         uint4 next = __ldg(q + min((groups - 1u) * 32u + lane, nv - 1u));
+        // one group; `all` = every lane has a block (a lane without one keeps its state and gives off no word)
+        auto code = [&](const uint4 cur, const bool all, const bool act) {
+            const int32_t mc = field16(cur.w, 1);
+            const uint32_t w[4] = {cur.x, cur.y, cur.z, cur.w}, coset = (mc & 1) ? entries + T.coset : entries;
+            uint4 e[9];                          // (every offset is in range: these are the fields the tables were counted from)
+            auto entry = [&](uint32_t at) {
+                uint4 v;
+                if (IN_SMEM) asm("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(at));
+                else v = __ldg(reinterpret_cast<const uint4 *>(reinterpret_cast<const uint8_t *>(entries_global) + at));
+                return v;
+            };
+            e[0] = entry(T.base[0] + entries + 16u * uint32_t(mc & 1));
+#pragma unroll
+            for (int k = 1; k < 8; ++k) e[k] = entry(16u * uint32_t(field16(w[(k - 1) >> 1], (k - 1) & 1)) + (coset + T.base[k]));
+            e[8] = entry(16u * uint32_t(mc >> 1) + (coset + T.base[8]));
+            uint32_t given = 0, held = 0;        // the last step's ballot and states: its words are stored one step later,
+#pragma unroll                                   // off the chain of states
+            for (int k = 8; k >= -1; --k) {
+                const uint32_t bal_before = given, word = held;
+                if (k >= 0) {
+                    const bool emit = x >= e[k].y && (all || act);
+                    given = __ballot_sync(0xFFFFFFFFu, emit);
+                    held = x;
+                    if (emit) x >>= 16;
+                    const uint32_t nx = __funnelshift_r(__umulhi(x, e[k].x), 0u, e[k].w) * e[k].z + (x + (e[k].w >> 16));   // Eq. 17 (the shift takes sh)
+                    x = all || act ? nx : x;
+                }
+                if (k < 8) {
+                    end -= __popc(bal_before);   // at most nine words per block: the area holds them
+                    if ((bal_before >> lane) & 1u) area[end + __popc(bal_before & lt)] = uint16_t(word);
+                }
+            }
+        };
         for (uint32_t g = groups; g-- > 0;) {
             const uint4 cur = next;
             if (g) next = __ldg(q + (g - 1u) * 32u + lane);
-            const int32_t mc = field16(cur.w, 1);
-            const uint32_t w[4] = {cur.x, cur.y, cur.z, cur.w}, coset = (mc & 1) ? T.coset : 0u;
-            uint4 e[9];                          // (every offset is in range: these are the fields the tables were counted from)
-            e[0] = *reinterpret_cast<const uint4 *>(entries + (T.base[0] + 16u * uint32_t(mc & 1)));
-#pragma unroll
-            for (int k = 1; k < 8; ++k)
-                e[k] = *reinterpret_cast<const uint4 *>(entries + (T.base[k] + coset + 16u * uint32_t(field16(w[(k - 1) >> 1], (k - 1) & 1))));
-            e[8] = *reinterpret_cast<const uint4 *>(entries + (T.base[8] + coset + 16u * uint32_t(mc >> 1)));
-            if (g * 32u + lane >= nv) {          // no block (the tile's last group): the state stays, no word
-#pragma unroll
-                for (int k = 0; k < 9; ++k) e[k] = make_uint4(0u, 0xFFFFFFFFu, 0u, 0u);
-            }
-#pragma unroll
-            for (int k = 8; k >= 0; --k) {
-                const bool emit = x >= e[k].y;
-                const uint32_t bal = __ballot_sync(0xFFFFFFFFu, emit), word = x;
-                if (emit) x >>= 16;
-                x = __funnelshift_r(__umulhi(x, e[k].x), 0u, e[k].w) * e[k].z + (x + (e[k].w >> 16));   // Eq. 17 (the shift takes sh)
-                end -= __popc(bal);              // at most nine words per block: the area holds them
-                if (emit) area[end + __popc(bal & lt)] = uint16_t(word);
-            }
+            if (g * 32u + 32u <= nv) code(cur, true, true);
+            else code(cur, false, g * 32u + lane < nv);
         }
         index[size_t(tile) * 33u + lane] = x;
         if (lane == 0) counts[tile] = cap - end;
@@ -1087,7 +1105,8 @@ public:
         P.first = 1;
         for (int left = o.search_steps, pass = 0; left > 0; ++pass) {
             P.levels = uint32_t(std::min<int>(left, std::min<int>(pass + 1, kLevels)));
-            launch_count(P);
+            P.last_pass = left == int(P.levels);
+            EP_CUDA(launch_count(P, pass > 0));
             left -= int(P.levels);
             P.first = 0;
         }
@@ -1097,8 +1116,7 @@ public:
         F.lo0 = o.bracket_lo;
         F.hi0 = o.bracket_hi;
         F.last_step = o.polish_steps;
-        for (F.step = 0; F.step <= o.polish_steps; ++F.step) launch_count(F);
-        EP_CUDA(cudaGetLastError());
+        for (F.step = 0; F.step <= o.polish_steps; ++F.step) EP_CUDA(launch_count(F, F.step > 0 || o.search_steps > 0));
         const int rc = fetch(true);
         if (rc) return rc;
         const SearchState &S = *state();
@@ -1220,10 +1238,22 @@ private:
                 8.0 * double(n), 9.0 * double(n), b};
     }
     // one CTA per SM over all candidates of the pass, each with at least a few hundred blocks
-    void launch_count(CountParams P) {
+    cudaError_t launch_count(CountParams P, bool follows) {
         const uint32_t cands = (1u << P.levels) - 1u;
         P.ctas = std::max(1u, std::min((P.n_blocks + 255u) / 256u, uint32_t(sms_) / cands));
-        quantise_count_kernel<<<cands * P.ctas, kCountThreads, kCountSmem, st_>>>(P);
+        // A pass's last CTA works on alone for 8 us; with programmatic launch the next pass's CTAs come up meanwhile, load
+        // their first blocks and clear their counters.  Not the first pass: it reads what the kernel before it writes.
+        cudaLaunchAttribute attr{};
+        attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr.val.programmaticStreamSerializationAllowed = 1;
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3(cands * P.ctas);
+        cfg.blockDim = dim3(kCountThreads);
+        cfg.dynamicSmemBytes = kCountSmem;
+        cfg.stream = st_;
+        cfg.attrs = &attr;
+        cfg.numAttrs = follows ? 1u : 0u;
+        return cudaLaunchKernelEx(&cfg, quantise_count_kernel, P);
     }
     static size_t symbols(const CountDir &D) {
         size_t n = 0;
@@ -1250,8 +1280,7 @@ private:
         return EP_OK;
     }
     int count(const uint32_t *rows, uint32_t n_rows, float s, uint4 *fields, Model &m) {
-        launch_count(params(rows, n_rows, s, fields));
-        EP_CUDA(cudaGetLastError());
+        EP_CUDA(launch_count(params(rows, n_rows, s, fields), false));
         const int rc = fetch(false);
         if (rc) return rc;
         m.from_counts(state()->full.lo, state()->full.K, full_counts());
