@@ -834,6 +834,11 @@ __device__ __forceinline__ uint4 encode_entry(uint32_t fF, uint32_t b) {
     return make_uint4(rcp, f << (31u - b), M - f, sh | (F << 16));
 }
 
+__global__ void encode_entries_kernel(const uint32_t *__restrict__ fF, uint32_t n, uint32_t b, uint4 *__restrict__ entries) {
+    const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < n) entries[i] = encode_entry(fF[i], b);
+}
+
 // One warp per tile, one state per lane.  The decoder reads, per (group, field), the words of the needy lanes in
 // ascending lane order; the encoder walks groups and fields backwards and fills the tile's word area from its end, writing
 // each step's words as one block in ascending lane order, which is the order the reversed word list of a sequential
@@ -843,17 +848,45 @@ __device__ __forceinline__ uint4 encode_entry(uint32_t fF, uint32_t b) {
 // tiles spread over the SMs - or sixteen where its table takes so much shared memory that few CTAs fit an SM.
 constexpr uint32_t kTileThreads = 128, kTileThreadsMax = 512, kSmemEntries = 12288;
 
+// A group's nine steps.  A step's words are stored during the next one: ballot, population counts and address (some 60 cycles)
+// stay off the chain of states, and the store is predicated, not a branch.  P / Q: this and the previous step's
+// predicate, B / C their ballots, H / I their states before the shift.
+#define EP_CODE_LOAD(LD, J, A) LD " {a" J ", b" J ", c" J ", d" J "}, [" A "];\n\t"
+#define EP_CODE_STORE(Q, C, I)                                                                        \
+    "popc.b32 n, " C ";\n\t"  "and.b32 t, " C ", %3;\n\t"  "popc.b32 t, t;\n\t"  "sub.u32 %1, %1, n;\n\t" \
+    "add.u32 t, t, %1;\n\t"  "mad.wide.u32 ad, t, 2, %2;\n\t"  "@" Q " st.global.u16 [ad], " I ";\n\t"
+#define EP_CODE_STEP(J, P, B, H, STORE)                                                               \
+    "setp.ge.and.u32 " P ", %0, b" J ", act;\n\t"  "vote.sync.ballot.b32 " B ", " P ", 0xffffffff;\n\t"      \
+    "cvt.u16.u32 " H ", %0;\n\t"  "@" P " shr.u32 %0, %0, 16;\n\t"  "mul.hi.u32 q, %0, a" J ";\n\t" STORE  \
+    "shr.u32 o, d" J ", 16;\n\t"  "add.u32 o, o, %0;\n\t"  "shf.r.wrap.b32 q, q, 0, d" J ";\n\t"           \
+    "@act mad.lo.u32 %0, q, c" J ", o;\n\t"
+#define EP_CODE_REGS(J) ".reg .b32 a" J ", b" J ", c" J ", d" J ";\n\t"
+#define EP_CODE_GROUP(LD, RT, A8, A7, A6, A5, A4, A3, A2, A1, A0)                                      \
+    asm volatile("{\n\t.reg .pred act, pa, pb;\n\t.reg .b32 n, t, q, o, ba, bb;\n\t.reg .b16 ha, hb;\n\t.reg .b64 ad;\n\t"     \
+        EP_CODE_REGS("8") EP_CODE_REGS("7") EP_CODE_REGS("6") EP_CODE_REGS("5") EP_CODE_REGS("4") EP_CODE_REGS("3") EP_CODE_REGS("2")   \
+        EP_CODE_REGS("1") EP_CODE_REGS("0") "setp.ne.u32 act, %4, 0;\n\t"                                                        \
+        EP_CODE_LOAD(LD, "8", "%5") EP_CODE_LOAD(LD, "7", "%6") EP_CODE_LOAD(LD, "6", "%7") EP_CODE_LOAD(LD, "5", "%8")               \
+        EP_CODE_LOAD(LD, "4", "%9") EP_CODE_LOAD(LD, "3", "%10") EP_CODE_LOAD(LD, "2", "%11") EP_CODE_LOAD(LD, "1", "%12")           \
+        EP_CODE_LOAD(LD, "0", "%13")                                                                                                \
+        EP_CODE_STEP("8", "pa", "ba", "ha", "")                                                                                      \
+        EP_CODE_STEP("7", "pb", "bb", "hb", EP_CODE_STORE("pa", "ba", "ha")) EP_CODE_STEP("6", "pa", "ba", "ha", EP_CODE_STORE("pb", "bb", "hb")) \
+        EP_CODE_STEP("5", "pb", "bb", "hb", EP_CODE_STORE("pa", "ba", "ha")) EP_CODE_STEP("4", "pa", "ba", "ha", EP_CODE_STORE("pb", "bb", "hb")) \
+        EP_CODE_STEP("3", "pb", "bb", "hb", EP_CODE_STORE("pa", "ba", "ha")) EP_CODE_STEP("2", "pa", "ba", "ha", EP_CODE_STORE("pb", "bb", "hb")) \
+        EP_CODE_STEP("1", "pb", "bb", "hb", EP_CODE_STORE("pa", "ba", "ha")) EP_CODE_STEP("0", "pa", "ba", "ha", EP_CODE_STORE("pb", "bb", "hb")) \
+        EP_CODE_STORE("pa", "ba", "ha") "}"                                                                                          \
+        : "+r"(x), "+r"(end) : "l"(area), "r"(lt), "r"(act), RT(A8), RT(A7), RT(A6), RT(A5), RT(A4), RT(A3), RT(A2), RT(A1), RT(A0) : "memory")
+
 template <bool IN_SMEM>
 __global__ void __launch_bounds__(kTileThreadsMax) tile_encode_kernel(const uint4 *__restrict__ fields, uint32_t n_vec, uint32_t V,
-                                                                      uint32_t n_tiles, uint32_t b, const __grid_constant__ EncodeTables T,
-                                                                      const uint32_t *__restrict__ fF, const uint4 *__restrict__ entries_global,
+                                                                      uint32_t n_tiles, const __grid_constant__ EncodeTables T,
+                                                                      const uint4 *__restrict__ entries_global,
                                                                       uint16_t *__restrict__ scratch, uint32_t cap,
                                                                       uint32_t *__restrict__ index, uint32_t *__restrict__ counts, SearchState *state) {
     extern __shared__ __align__(16) uint4 entries_smem[];
     __shared__ uint32_t last_cta, part[kTileThreadsMax];
     const uint32_t tid = threadIdx.x, lane = tid & 31u;
     if (IN_SMEM) {
-        for (uint32_t i = tid; i < T.total; i += blockDim.x) entries_smem[i] = encode_entry(__ldg(fF + i), b);
+        for (uint32_t i = tid; i < T.total; i += blockDim.x) entries_smem[i] = __ldg(entries_global + i);
         __syncthreads();
     }
     const uint32_t entries = IN_SMEM ? uint32_t(__cvta_generic_to_shared(entries_smem)) : 0u;
@@ -866,44 +899,24 @@ __global__ void __launch_bounds__(kTileThreadsMax) tile_encode_kernel(const uint
         uint32_t x = kStateLow;
         const uint32_t groups = (nv + 31u) >> 5;
         uint4 next = __ldg(q + min((groups - 1u) * 32u + lane, nv - 1u));
-        // one group; `all` = every lane has a block (a lane without one keeps its state and gives off no word)
-        auto code = [&](const uint4 cur, const bool all, const bool act) {
-            const int32_t mc = field16(cur.w, 1);
-            const uint32_t w[4] = {cur.x, cur.y, cur.z, cur.w}, coset = (mc & 1) ? entries + T.coset : entries;
-            uint4 e[9];                          // (every offset is in range: these are the fields the tables were counted from)
-            auto entry = [&](uint32_t at) {
-                uint4 v;
-                if (IN_SMEM) asm("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(at));
-                else v = __ldg(reinterpret_cast<const uint4 *>(reinterpret_cast<const uint8_t *>(entries_global) + at));
-                return v;
-            };
-            e[0] = entry(T.base[0] + entries + 16u * uint32_t(mc & 1));
-#pragma unroll
-            for (int k = 1; k < 8; ++k) e[k] = entry(16u * uint32_t(field16(w[(k - 1) >> 1], (k - 1) & 1)) + (coset + T.base[k]));
-            e[8] = entry(16u * uint32_t(mc >> 1) + (coset + T.base[8]));
-            uint32_t given = 0, held = 0;        // the last step's ballot and states: its words are stored one step later,
-#pragma unroll                                   // off the chain of states
-            for (int k = 8; k >= -1; --k) {
-                const uint32_t bal_before = given, word = held;
-                if (k >= 0) {
-                    const bool emit = x >= e[k].y && (all || act);
-                    given = __ballot_sync(0xFFFFFFFFu, emit);
-                    held = x;
-                    if (emit) x >>= 16;
-                    const uint32_t nx = __funnelshift_r(__umulhi(x, e[k].x), 0u, e[k].w) * e[k].z + (x + (e[k].w >> 16));   // Eq. 17 (the shift takes sh)
-                    x = all || act ? nx : x;
-                }
-                if (k < 8) {
-                    end -= __popc(bal_before);   // at most nine words per block: the area holds them
-                    if ((bal_before >> lane) & 1u) area[end + __popc(bal_before & lt)] = uint16_t(word);
-                }
-            }
-        };
         for (uint32_t g = groups; g-- > 0;) {
             const uint4 cur = next;
             if (g) next = __ldg(q + (g - 1u) * 32u + lane);
-            if (g * 32u + 32u <= nv) code(cur, true, true);
-            else code(cur, false, g * 32u + lane < nv);
+            const int32_t mc = field16(cur.w, 1);
+            const uint32_t w[4] = {cur.x, cur.y, cur.z, cur.w}, coset = (mc & 1) ? entries + T.coset : entries;
+            uint32_t at[9];                      // (every offset is in range: these are the fields the tables were counted from)
+            at[0] = T.base[0] + entries + 16u * uint32_t(mc & 1);
+#pragma unroll
+            for (int k = 1; k < 8; ++k) at[k] = 16u * uint32_t(field16(w[(k - 1) >> 1], (k - 1) & 1)) + (coset + T.base[k]);
+            at[8] = 16u * uint32_t(mc >> 1) + (coset + T.base[8]);
+            const uint32_t act = g * 32u + lane < nv ? 1u : 0u;      // a lane without a block keeps its state and gives off no word
+            if (IN_SMEM) {
+                EP_CODE_GROUP("ld.shared.v4.u32", "r", at[8], at[7], at[6], at[5], at[4], at[3], at[2], at[1], at[0]);
+            } else {
+                const uint64_t e0 = reinterpret_cast<uint64_t>(entries_global);
+                EP_CODE_GROUP("ld.global.nc.v4.u32", "l", e0 + at[8], e0 + at[7], e0 + at[6], e0 + at[5], e0 + at[4], e0 + at[3], e0 + at[2],
+                              e0 + at[1], e0 + at[0]);
+            }
         }
         index[size_t(tile) * 33u + lane] = x;
         if (lane == 0) counts[tile] = cap - end;
@@ -933,12 +946,6 @@ __global__ void __launch_bounds__(kTileThreadsMax) tile_encode_kernel(const uint
         index[size_t(n_tiles) * 33u] = part[tid];
         state->total_words = part[tid];
     }
-}
-
-// entries of an alphabet too large for shared memory
-__global__ void encode_entries_kernel(const uint32_t *__restrict__ fF, uint32_t n, uint32_t b, uint4 *__restrict__ entries) {
-    const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) entries[i] = encode_entry(fF[i], b);
 }
 
 // Move every tile's words from the end of its area to its place in the payload: one CTA per tile (with a warp per tile the
@@ -1173,17 +1180,17 @@ public:
         for (uint32_t j = 0; j < m.t[0].K(); ++j) fF[2u * size + uint32_t(m.t[0].lo) + j] = m.t[0].f[j] | (m.t[0].F[j] << 16);
         EP_CUDA(cudaMemcpyAsync(w_.fF, fF.data(), 4ull * fF.size(), cudaMemcpyHostToDevice, st_));
         EP_CUDA(cudaMemsetAsync(&w_.state->tiles_done, 0, 4, st_));
+        encode_entries_kernel<<<(T.total + 127u) / 128u, 128, 0, st_>>>(w_.fF, T.total, uint32_t(b), w_.entries);
         if (T.total <= kSmemEntries) {
             const size_t smem = 16ull * T.total;
             const uint32_t threads = T.total <= 2048u ? kTileThreads : kTileThreadsMax;
             if (smem > 40u * 1024u)      // (always the same limit: another thread's call must not lower it before the launch)
                 EP_CUDA(cudaFuncSetAttribute(tile_encode_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(16u * kSmemEntries)));
             tile_encode_kernel<true><<<(n_tiles + threads / 32u - 1u) / (threads / 32u), threads, smem, st_>>>(
-                w_.fields, uint32_t(nvec), V, n_tiles, uint32_t(b), T, w_.fF, w_.entries, w_.scratch, cap, w_.index, w_.counts, w_.state);
+                w_.fields, uint32_t(nvec), V, n_tiles, T, w_.entries, w_.scratch, cap, w_.index, w_.counts, w_.state);
         } else {
-            encode_entries_kernel<<<(T.total + 255u) / 256u, 256, 0, st_>>>(w_.fF, T.total, uint32_t(b), w_.entries);
             tile_encode_kernel<false><<<(n_tiles + kTileThreads / 32u - 1u) / (kTileThreads / 32u), kTileThreads, 0, st_>>>(
-                w_.fields, uint32_t(nvec), V, n_tiles, uint32_t(b), T, w_.fF, w_.entries, w_.scratch, cap, w_.index, w_.counts, w_.state);
+                w_.fields, uint32_t(nvec), V, n_tiles, T, w_.entries, w_.scratch, cap, w_.index, w_.counts, w_.state);
         }
         compact_kernel<<<n_tiles, kCompactThreads, 0, st_>>>(w_.scratch, cap, w_.counts, w_.index, w_.payload);
         EP_CUDA(cudaMemcpyAsync(&state()->total_words, &w_.state->total_words, 4, cudaMemcpyDeviceToHost, st_));
