@@ -843,7 +843,7 @@ __global__ void encode_entries_kernel(const uint32_t *__restrict__ fF, uint32_t 
 // ascending lane order; the encoder walks groups and fields backwards and fills the tile's word area from its end, writing
 // each step's words as one block in ascending lane order, which is the order the reversed word list of a sequential
 // encoder would have.  A step's chain is compare, shift, multiply-high, shift, multiply-add (about 30 cycles);
-// a group's fields are loaded one group ahead and its symbols looked up before the steps that need them.
+// a group's fields are loaded four groups ahead and its symbols looked up before the steps that need them.
 // IN_SMEM: the symbols' entries in shared memory (up to 12 Ki symbols), else in global memory.  A CTA has four warps -
 // tiles spread over the SMs - or sixteen where its table takes so much shared memory that few CTAs fit an SM.
 constexpr uint32_t kTileThreads = 128, kTileThreadsMax = 512, kSmemEntries = 12288;
@@ -852,14 +852,14 @@ constexpr uint32_t kTileThreads = 128, kTileThreadsMax = 512, kSmemEntries = 122
 // stay off the chain of states, and the store is predicated, not a branch.  P / Q: this and the previous step's
 // predicate, B / C their ballots, H / I their states before the shift.
 #define EP_CODE_LOAD(LD, J, A) LD " {a" J ", b" J ", c" J ", d" J "}, [" A "];\n\t"
+#define EP_CODE_COUNT(C) "popc.b32 n, " C ";\n\t"  "and.b32 t, " C ", %3;\n\t"  "popc.b32 t, t;\n\t"
 #define EP_CODE_STORE(Q, C, I)                                                                        \
-    "popc.b32 n, " C ";\n\t"  "and.b32 t, " C ", %3;\n\t"  "popc.b32 t, t;\n\t"  "sub.u32 %1, %1, n;\n\t" \
-    "add.u32 t, t, %1;\n\t"  "mad.wide.u32 ad, t, 2, %2;\n\t"  "@" Q " st.global.u16 [ad], " I ";\n\t"
-#define EP_CODE_STEP(J, P, B, H, STORE)                                                               \
-    "setp.ge.and.u32 " P ", %0, b" J ", act;\n\t"  "vote.sync.ballot.b32 " B ", " P ", 0xffffffff;\n\t"      \
-    "cvt.u16.u32 " H ", %0;\n\t"  "@" P " shr.u32 %0, %0, 16;\n\t"  "mul.hi.u32 q, %0, a" J ";\n\t" STORE  \
-    "shr.u32 o, d" J ", 16;\n\t"  "add.u32 o, o, %0;\n\t"  "shf.r.wrap.b32 q, q, 0, d" J ";\n\t"           \
-    "@act mad.lo.u32 %0, q, c" J ", o;\n\t"
+    "sub.u32 %1, %1, n;\n\t"  "add.u32 t, t, %1;\n\t"  "mad.wide.u32 ad, t, 2, %2;\n\t"  "@" Q " st.global.u16 [ad], " I ";\n\t"
+#define EP_CODE_STEP(J, P, B, H, COUNT, STORE)                                                        \
+    COUNT "setp.ge.and.u32 " P ", %0, b" J ", act;\n\t"  "cvt.u16.u32 " H ", %0;\n\t"                        \
+    "@" P " shr.u32 %0, %0, 16;\n\t"  "mul.hi.u32 q, %0, a" J ";\n\t"                                         \
+    "vote.sync.ballot.b32 " B ", " P ", 0xffffffff;\n\t"  "shr.u32 o, d" J ", 16;\n\t"  "add.u32 o, o, %0;\n\t" \
+    "shf.r.wrap.b32 q, q, 0, d" J ";\n\t"  "@act mad.lo.u32 %0, q, c" J ", o;\n\t" STORE
 #define EP_CODE_REGS(J) ".reg .b32 a" J ", b" J ", c" J ", d" J ";\n\t"
 #define EP_CODE_GROUP(LD, RT, A8, A7, A6, A5, A4, A3, A2, A1, A0)                                      \
     asm volatile("{\n\t.reg .pred act, pa, pb;\n\t.reg .b32 n, t, q, o, ba, bb;\n\t.reg .b16 ha, hb;\n\t.reg .b64 ad;\n\t"     \
@@ -868,12 +868,12 @@ constexpr uint32_t kTileThreads = 128, kTileThreadsMax = 512, kSmemEntries = 122
         EP_CODE_LOAD(LD, "8", "%5") EP_CODE_LOAD(LD, "7", "%6") EP_CODE_LOAD(LD, "6", "%7") EP_CODE_LOAD(LD, "5", "%8")               \
         EP_CODE_LOAD(LD, "4", "%9") EP_CODE_LOAD(LD, "3", "%10") EP_CODE_LOAD(LD, "2", "%11") EP_CODE_LOAD(LD, "1", "%12")           \
         EP_CODE_LOAD(LD, "0", "%13")                                                                                                \
-        EP_CODE_STEP("8", "pa", "ba", "ha", "")                                                                                      \
-        EP_CODE_STEP("7", "pb", "bb", "hb", EP_CODE_STORE("pa", "ba", "ha")) EP_CODE_STEP("6", "pa", "ba", "ha", EP_CODE_STORE("pb", "bb", "hb")) \
-        EP_CODE_STEP("5", "pb", "bb", "hb", EP_CODE_STORE("pa", "ba", "ha")) EP_CODE_STEP("4", "pa", "ba", "ha", EP_CODE_STORE("pb", "bb", "hb")) \
-        EP_CODE_STEP("3", "pb", "bb", "hb", EP_CODE_STORE("pa", "ba", "ha")) EP_CODE_STEP("2", "pa", "ba", "ha", EP_CODE_STORE("pb", "bb", "hb")) \
-        EP_CODE_STEP("1", "pb", "bb", "hb", EP_CODE_STORE("pa", "ba", "ha")) EP_CODE_STEP("0", "pa", "ba", "ha", EP_CODE_STORE("pb", "bb", "hb")) \
-        EP_CODE_STORE("pa", "ba", "ha") "}"                                                                                          \
+        EP_CODE_STEP("8", "pa", "ba", "ha", "", "")                                                                                      \
+        EP_CODE_STEP("7", "pb", "bb", "hb", EP_CODE_COUNT("ba"), EP_CODE_STORE("pa", "ba", "ha")) EP_CODE_STEP("6", "pa", "ba", "ha", EP_CODE_COUNT("bb"), EP_CODE_STORE("pb", "bb", "hb")) \
+        EP_CODE_STEP("5", "pb", "bb", "hb", EP_CODE_COUNT("ba"), EP_CODE_STORE("pa", "ba", "ha")) EP_CODE_STEP("4", "pa", "ba", "ha", EP_CODE_COUNT("bb"), EP_CODE_STORE("pb", "bb", "hb")) \
+        EP_CODE_STEP("3", "pb", "bb", "hb", EP_CODE_COUNT("ba"), EP_CODE_STORE("pa", "ba", "ha")) EP_CODE_STEP("2", "pa", "ba", "ha", EP_CODE_COUNT("bb"), EP_CODE_STORE("pb", "bb", "hb")) \
+        EP_CODE_STEP("1", "pb", "bb", "hb", EP_CODE_COUNT("ba"), EP_CODE_STORE("pa", "ba", "ha")) EP_CODE_STEP("0", "pa", "ba", "ha", EP_CODE_COUNT("bb"), EP_CODE_STORE("pb", "bb", "hb")) \
+        EP_CODE_COUNT("ba") EP_CODE_STORE("pa", "ba", "ha") "}"                                                                                          \
         : "+r"(x), "+r"(end) : "l"(area), "r"(lt), "r"(act), RT(A8), RT(A7), RT(A6), RT(A5), RT(A4), RT(A3), RT(A2), RT(A1), RT(A0) : "memory")
 
 template <bool IN_SMEM>
@@ -898,10 +898,17 @@ __global__ void __launch_bounds__(kTileThreadsMax) tile_encode_kernel(const uint
         uint32_t end = cap;                      // words [end, cap) of the area are written
         uint32_t x = kStateLow;
         const uint32_t groups = (nv + 31u) >> 5;
-        uint4 next = __ldg(q + min((groups - 1u) * 32u + lane, nv - 1u));
+        // fields of the next groups: a group takes 0.4 us, a load from DRAM over 1 us
+        constexpr uint32_t kAhead = 4;
+        uint4 next[kAhead];
+#pragma unroll
+        for (uint32_t i = 0; i < kAhead; ++i)
+            next[i] = groups > i ? __ldg(q + min((groups - 1u - i) * 32u + lane, nv - 1u)) : make_uint4(0u, 0u, 0u, 0u);
         for (uint32_t g = groups; g-- > 0;) {
-            const uint4 cur = next;
-            if (g) next = __ldg(q + (g - 1u) * 32u + lane);
+            const uint4 cur = next[0];
+#pragma unroll
+            for (uint32_t i = 0; i + 1u < kAhead; ++i) next[i] = next[i + 1u];
+            if (g >= kAhead) next[kAhead - 1u] = __ldg(q + (g - kAhead) * 32u + lane);
             const int32_t mc = field16(cur.w, 1);
             const uint32_t w[4] = {cur.x, cur.y, cur.z, cur.w}, coset = (mc & 1) ? entries + T.coset : entries;
             uint32_t at[9];                      // (every offset is in range: these are the fields the tables were counted from)
