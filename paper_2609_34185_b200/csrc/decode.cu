@@ -45,6 +45,14 @@ constexpr uint32_t kChains = EP_CHAINS;
 constexpr int kWarps = EP_WARPS;                             // warps per CTA (one CTA per SM)
 constexpr int kThreads = kWarps * 32;
 constexpr uint32_t kTilesPerRound = kWarps * kChains;        // tiles per CTA at a time, at most (see split_rounds)
+#ifndef EP_FEW_TILES
+#define EP_FEW_TILES 12
+#endif
+#ifndef EP_GUESS_BITS
+#define EP_GUESS_BITS 4.5
+#endif
+constexpr uint32_t kFewTiles = EP_FEW_TILES;                 // most tiles per CTA for decode_tile_few
+constexpr double kGuessBits = EP_GUESS_BITS;                 // most payload bits per symbol for its guessing loop
 constexpr uint32_t kMinWarps = 8;                            // threads that copy the tables, however few tiles a CTA has
 static_assert(kTilesPerRound == ep::kDecodeTilesPerCta, "tile-size suggestions assume this many tiles per CTA");
 constexpr uint32_t kLutEntries = 2048;                       // 2^11 slots per table
@@ -58,8 +66,8 @@ constexpr uint32_t kRingBytes = kRingSlots * kChunk;         // 1536
 constexpr uint32_t kRingMirror = 512;                        // >= 7 words * 32 lanes * 2 bytes + one lane span (62)
 constexpr uint32_t kRingStride = kRingBytes + kRingMirror;   // 2048 per chain
 constexpr uint32_t kCtxBytes = 32 + 32 * kChains;            // per warp: what the rare paths of the hot loop need
-constexpr uint32_t kRingBase = kLutBytes;
-constexpr uint32_t kCtxBase = kRingBase + kWarps * kChains * kRingStride;
+constexpr uint32_t kCtxBase = kLutBytes;
+constexpr uint32_t kRingBase = kCtxBase + kWarps * kCtxBytes;
 // 2^12-slot streams: per table, the entries of the kHotSpan coordinate values around zero are kept in shared memory
 // (the rest is read from global memory); this fills what the tables, rings and context blocks of the 32-warp build
 // leave of the 227 KB
@@ -67,10 +75,11 @@ constexpr uint32_t kHotSpan = 528;                           // coordinate codes
 constexpr uint32_t kHotBytes = 16 * kHotSpan * 4;            // 33792
 constexpr uint32_t kColdCodes = 4096;                        // codes per table in the complete entry array (global memory)
 constexpr uint32_t kColdBytes = 16 * kColdCodes * 4;         // 262144
-constexpr uint32_t kHotBase = kCtxBase + kWarps * kCtxBytes;
+constexpr uint32_t kHotBase = kRingBase + kWarps * kChains * kRingStride;
 constexpr bool kTwoLevelInLoop = EP_CHAINS == 1 && kHotBase + kHotBytes <= 232448;
 constexpr uint32_t kSmemBytes = kHotBase + (kTwoLevelInLoop ? kHotBytes : 0);   // 232448 in the default build
 static_assert(kSmemBytes <= 232448, "more shared memory than an sm_100 CTA can have");
+constexpr uint32_t kStageBytes = kSmemBytes - kRingBase;     // with few tiles per CTA: room for their whole payloads (see decode_tile_few)
 constexpr uint32_t kCodeMask = 0x001FF800u;                  // 10-bit code field
 constexpr uint32_t kExp4096 = 0x45800000u;                   // fp32 bit pattern of 4096.0
 constexpr uint32_t kOwnSlots = 16;                           // table build: slots of a symbol that its own lane writes
@@ -116,6 +125,7 @@ struct JobParams {
     uint32_t row_bytes;           // output bytes per row
     uint32_t row_rcp;             // ceil(2^32 / row_bytes)
     uint32_t row_max;             // index of the last row
+    uint32_t guess;               // decode_tile_few: the loop that guesses (see EP_BODY11_GUESS)
     int16_t tmin[EP_NUM_TABLES];
     uint16_t tK[EP_NUM_TABLES];
     uint16_t foff[EP_NUM_TABLES]; // start of table t's frequencies, in u16 units
@@ -146,6 +156,14 @@ __device__ __forceinline__ void cp_async16(uint32_t dst, uint64_t src, uint32_t 
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
+// Programmatic launch: a kernel of this file may come up while the kernel before it in the stream still runs, and lets the
+// next one come up likewise.  Nothing is read or written before this wait, which ends when everything earlier in the stream
+// has, so the order of effects is the stream's; what overlaps is the launch itself (see launch_next).
+__device__ __forceinline__ void wait_for_stream() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
 
 __device__ __forceinline__ void prefetch_l2(const void *p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 
@@ -850,6 +868,79 @@ __device__ __forceinline__ void decode_tile_plain(const JobParams &J, uint32_t t
         EP_STEP12_ALL("e7", "49152", NA, NB, "12672", "98304") EP_ALL(EP_PAR3, "par", "e6", "e7") EP_ALL(EP_XA12, "e7") \
         EP_STEP12_ALL("e8", "57344", NB, BL, "14784", "114688") EP_ALL(EP_PARX12) EP_ALL(EP_X8_12) EP_PAIR_ALL EP_ALL(CVT, "3")
 
+// ---- the same group with a shorter chain, for few tiles per SM (2^11-slot streams) ---------------------------------
+// With a couple of warps per scheduler the time of a group is the latency of its nine steps, and in EP_BODY11 a step is one
+// chain: slot address and lookup (41 cycles), new state (8), ballot (18), rank (20), word (29), back into the state (4).
+// EP_BODY11_SHORT: the next slot is taken from the word itself, not from the state that the word goes into (va = the word
+// where one was taken, else the state: their low eleven bits are the same).  1138 -> 1066 cycles per group.
+#define EP_T_RENORM(BIN, BOUT)                                                                                        \
+        "setp.lt.and.u32 pA, %0, 32768, actA;\n\t" "vote.sync.ballot.b32 " BOUT ", pA, 0xffffffff;\n\t"               \
+        "mov.b32 va, %0;\n\t" "lop3.b32 tA, " EP_LT ", " BOUT ", " BIN ", 0xCA;\n\t" "popc.b32 tA, tA;\n\t"           \
+        "mad.lo.u32 %1, tA, 2, %1;\n\t" "@pA ld.shared.u16 va, [%1];\n\t" "@pA mad.lo.u32 %0, %0, 65536, va;\n\t"
+#define EP_T_STEP(E, OFF, BIN, BOUT)                                                                                  \
+        "and.b32 uA, va, 0x7FF;\n\t" "mad.lo.u32 uA, uA, 4, tabA;\n\t" "ld.shared.u32 " E "A, [uA+" OFF "];\n\t"      \
+        "shr.u32 qA, %0, 11;\n\t" "shr.u32 fA, " E "A, 21;\n\t" "and.b32 biA, " E "A, 0x7FF;\n\t"                     \
+        "@actA mad.lo.u32 %0, fA, qA, biA;\n\t" EP_T_RENORM(BIN, BOUT)
+#define EP_T_COSET                                                                                                    \
+        EP_ALL(EP_C1) EP_ALL(EP_C2) EP_ALL(EP_C3) EP_ALL(EP_C4) EP_ALL(EP_C5) EP_ALL(EP_C6) EP_ALL(EP_C7) EP_ALL(EP_C8)
+#define EP_BODY11_SHORT(CVT)                                                                                          \
+        EP_T_COSET EP_T_RENORM("%2", "naA")                                                                           \
+        EP_T_STEP("e1", "0", "naA", "nbA")     EP_ALL(EP_XA, "e1")                                                    \
+        EP_T_STEP("e2", "8192", "nbA", "naA")  EP_ALL(EP_XB, "e2") EP_PAIR_ALL EP_ALL(CVT, "0")                       \
+        EP_T_STEP("e3", "16384", "naA", "nbA") EP_ALL(EP_PAR3, "e1", "e2", "e3") EP_ALL(EP_XA, "e3")                  \
+        EP_T_STEP("e4", "24576", "nbA", "naA") EP_ALL(EP_XB, "e4") EP_PAIR_ALL EP_ALL(CVT, "1")                       \
+        EP_T_STEP("e5", "32768", "naA", "nbA") EP_ALL(EP_PAR3, "par", "e4", "e5") EP_ALL(EP_XA, "e5")                 \
+        EP_T_STEP("e6", "40960", "nbA", "naA") EP_ALL(EP_XB, "e6") EP_PAIR_ALL EP_ALL(CVT, "2")                       \
+        EP_T_STEP("e7", "49152", "naA", "nbA") EP_ALL(EP_PAR3, "par", "e6", "e7") EP_ALL(EP_XA, "e7")                 \
+        EP_T_STEP("e8", "57344", "nbA", "%2") EP_ALL(EP_PARX) EP_ALL(EP_X8) EP_PAIR_ALL EP_ALL(CVT, "3")
+
+// EP_BODY11_GUESS: a lane that takes a word in step k hardly ever takes another in step k + 1 (its state is then at least
+// 2^20 and usually above 2^26, and a step shortens a state by eleven bits at most), and no other lane needs a word to go on.
+// So the ballot of step k + 1 is taken of the lanes that did not take a word in step k, whose lookup has not waited for
+// step k's words.  The lanes that did follow with a lookup of their own and are back for the lookup of step k + 2.  If one
+// of them falls below 2^15 all the same (`lm`, the smallest such state), the ballots were wrong, and the group is decoded
+// again from its saved start by EP_BODY11_SHORT: no result depends on the guess.  Two steps take 160 cycles this way.
+// The order below follows the times at which operands arrive (a warp issues in order): rank of the words, the late lanes'
+// end of the previous step (TAIL, predicate NP from two steps ago), lookup, word, work for the output (FILL), the late
+// lanes' lookup, new state and ballot.
+// PB / PPB: ballots of the previous step and the one before; PP: the lanes that took a word; NB / NP: this step's.
+#define EP_G_TAIL(E, P)                                                                                               \
+        "shr.u32 f2, ea, 21;\n\t" "and.b32 b2, ea, 0x7FF;\n\t" "@" P " mad.lo.u32 %0, f2, q2, b2;\n\t"
+#define EP_G_TAIL_REST(E, P) "@" P " min.u32 lm, lm, %0;\n\t" "@" P " mov.b32 " E "A, ea;\n\t"
+#define EP_G_RANK(PB, PPB) "lop3.b32 tA, " EP_LT ", " PB ", " PPB ", 0xCA;\n\t" "popc.b32 tA, tA;\n\t"
+#define EP_G_STEP(E, OFF, PB, PPB, PP, NB, NP, TAIL, TAILREST, FILL)                                                  \
+        EP_G_RANK(PB, PPB) TAIL                                                                                       \
+        "and.b32 uA, %0, 0x7FF;\n\t" "mad.lo.u32 uA, uA, 4, tabA;\n\t" "ld.shared.u32 " E "A, [uA+" OFF "];\n\t"      \
+        "mad.lo.u32 %1, tA, 2, %1;\n\t" "@" PP " ld.shared.u16 wA, [%1];\n\t"                                         \
+        "shr.u32 qA, %0, 11;\n\t" "not.pred pn, " PP ";\n\t" "and.pred pn, pn, actA;\n\t" TAILREST FILL               \
+        "and.b32 va, wA, 0x7FF;\n\t" "mad.lo.u32 va, va, 4, tabA;\n\t" "@" PP " ld.shared.u32 ea, [va+" OFF "];\n\t"  \
+        "shr.u32 fA, " E "A, 21;\n\t" "and.b32 biA, " E "A, 0x7FF;\n\t" "@pn mad.lo.u32 %0, fA, qA, biA;\n\t"         \
+        "setp.lt.and.u32 " NP ", %0, 32768, pn;\n\t" "vote.sync.ballot.b32 " NB ", " NP ", 0xffffffff;\n\t"           \
+        "@" PP " mad.lo.u32 %0, %0, 65536, wA;\n\t" "shr.u32 q2, %0, 11;\n\t"
+#define EP_BODY11_GUESS(CVT)                                                                                          \
+        "mov.b32 lm, 0xffffffff;\n\t" "mov.b32 sx, %0;\n\t" "mov.b32 sa, %1;\n\t" "mov.b32 sb, %2;\n\t"               \
+        EP_T_COSET                                                                                                    \
+        "setp.lt.and.u32 pA, %0, 32768, actA;\n\t" "vote.sync.ballot.b32 naA, pA, 0xffffffff;\n\t"                    \
+        EP_G_STEP("e1", "0", "naA", "%2", "pA", "nbA", "ps", "", "", "")                                              \
+        EP_G_STEP("e2", "8192", "nbA", "naA", "ps", "%2", "pA", EP_G_TAIL("e1", "pA"), EP_G_TAIL_REST("e1", "pA"),    \
+                  EP_ALL(EP_XA, "e1"))                                                                                \
+        EP_G_STEP("e3", "16384", "%2", "nbA", "pA", "naA", "ps", EP_G_TAIL("e2", "ps"), EP_G_TAIL_REST("e2", "ps"),   \
+                  EP_ALL(EP_XB, "e2") EP_PAIR_ALL EP_ALL(CVT, "0"))                                                   \
+        EP_G_STEP("e4", "24576", "naA", "%2", "ps", "nbA", "pA", EP_G_TAIL("e3", "pA"), EP_G_TAIL_REST("e3", "pA"),   \
+                  EP_ALL(EP_PAR3, "e1", "e2", "e3") EP_ALL(EP_XA, "e3"))                                              \
+        EP_G_STEP("e5", "32768", "nbA", "naA", "pA", "%2", "ps", EP_G_TAIL("e4", "ps"), EP_G_TAIL_REST("e4", "ps"),   \
+                  EP_ALL(EP_XB, "e4") EP_PAIR_ALL EP_ALL(CVT, "1"))                                                   \
+        EP_G_STEP("e6", "40960", "%2", "nbA", "ps", "naA", "pA", EP_G_TAIL("e5", "pA"), EP_G_TAIL_REST("e5", "pA"),   \
+                  EP_ALL(EP_PAR3, "par", "e4", "e5") EP_ALL(EP_XA, "e5"))                                             \
+        EP_G_STEP("e7", "49152", "naA", "%2", "pA", "nbA", "ps", EP_G_TAIL("e6", "ps"), EP_G_TAIL_REST("e6", "ps"),   \
+                  EP_ALL(EP_XB, "e6") EP_PAIR_ALL EP_ALL(CVT, "2"))                                                   \
+        EP_G_STEP("e8", "57344", "nbA", "naA", "ps", "%2", "pA", EP_G_TAIL("e7", "pA"), EP_G_TAIL_REST("e7", "pA"),   \
+                  EP_ALL(EP_PAR3, "par", "e6", "e7") EP_ALL(EP_XA, "e7"))                                             \
+        EP_G_RANK("%2", "nbA") EP_G_TAIL("e8", "ps")                                                                  \
+        "mad.lo.u32 %1, tA, 2, %1;\n\t" "@pA ld.shared.u16 wA, [%1];\n\t" EP_G_TAIL_REST("e8", "ps")                  \
+        EP_ALL(EP_PARX) EP_ALL(EP_X8) EP_PAIR_ALL EP_ALL(CVT, "3")                                                    \
+        "@pA mad.lo.u32 %0, %0, 65536, wA;\n\t"
+
 // per output type: CVT(S, j, lo, hi) turns weights 2j, 2j+1 into their stored form, STORE(S) writes the block
 #define EP_CVT_BF16(S, X, AW, BAL, DOFF, CB, J) "cvt.rn.bf16x2.f32 o" J S ", wh" S ", wl" S ";\n\t"
 #define EP_CVT_FP16(S, X, AW, BAL, DOFF, CB, J) "cvt.rn.satfinite.f16x2.f32 o" J S ", wh" S ", wl" S ";\n\t"
@@ -1049,6 +1140,81 @@ __device__ __forceinline__ void decode_tile_plain(const JobParams &J, uint32_t t
           "r"(cf.f1), "r"(lane16), "l"(l2base), "r"(hs2), "n"(kHotBase)                                             \
         : "memory")
 
+// ---- the loop for few tiles per SM: one tile per warp, its whole payload in shared memory ---------------------------
+// Nothing else covers a warp's stalls here, so the rare work is kept short as well: no ring to refill, and the tile's row
+// scales are in shared memory too (a load from global memory at a row's start: 700 cycles every C / 256 groups).
+// GUESS: EP_GUESS_CHECK with EP_BODY11_GUESS - a group whose guess failed is decoded again and stored over -, else empty.
+#define EP_GUESS_CHECK(CVT, STORE, GROUP_BYTES)                                                                       \
+        "setp.lt.u32 pr, lm, 32768;\n\t"                                                                              \
+        "vote.sync.any.pred pr, pr, 0xffffffff;\n\t"                                                                  \
+        "@!pr bra.uni EP_RARE;\n\t"                                                                                   \
+        "mov.b32 %0, sx;\n\t" "mov.b32 %1, sa;\n\t" "mov.b32 %2, sb;\n\t" "sub.u32 %3, %3, " #GROUP_BYTES ";\n\t"     \
+        EP_BODY11_SHORT(CVT)                                                                                          \
+        EP_ALL(EP_ADDR) EP_ALL(STORE) EP_ALL(EP_ADVANCE, #GROUP_BYTES)
+#define EP_GUESS_NONE(CVT, STORE, GROUP_BYTES)
+#define EP_FEW_LOOP_ASM(BODY, GUESS, CVT, STORE, GROUP_BYTES)                                                         \
+    asm volatile(                                                                                                     \
+        "{\n\t"                                                                                                       \
+        EP_ALL(EP_REGS)                                                                                               \
+        ".reg .pred pq, pv, pr, ps, pn;\n\t"                                                                          \
+        ".reg .b32 r0, r1, r3, c0r, c1r, f0c, lm, sx, sa, sb, ea, va, f2, b2, q2, rp, rowb, endo;\n\t"     \
+        ".reg .b64 ra, rb;\n\t"                                                                                       \
+        ".reg .f32 k0f, k1f;\n\t"                                                                                     \
+        "mov.b64 {k0f, k1f}, " EP_KK ";\n\t"                                                                          \
+        "mov.b32 c0r, 0x45800000;\n\t"                                                                                \
+        "mov.b32 c1r, 0x45800400;\n\t"                                                                                \
+        "max.u32 f0c, " EP_F0 ", 1;\n\t"                                                                              \
+        "mov.b32 wA, 0;\n\t" "mov.b32 ea, 0x200000;\n\t" "mov.b32 q2, 0;\n\t" "mov.b32 lm, 0xffffffff;\n\t"           \
+        "mov.b32 rp, %12;\n\t" "mov.b32 limA, %13;\n\t" "mov.b32 wthrA, %14;\n\t"                                     \
+        "ld.shared.b32 sgA, [rp];\n\t" "mov.b32 r3, sgA;\n\t" "mov.b64 ssA, {r3, r3};\n\t"                            \
+        "ld.shared.u32 rowb, [" EP_CTX "+8];\n\t"                                                                     \
+        "ld.shared.u32 endo, [" EP_CTX "+56];\n\t"        /* offset after the tile's last block */                    \
+        "setp.lt.u32 actA, %3, endo;\n\t" "@!actA mov.u32 limA, 0xffffffff;\n\t"                                      \
+        "vote.sync.any.pred pr, actA, 0xffffffff;\n\t"                                                                \
+        "@!pr bra.uni EP_DONE;\n\t"                                                                                   \
+        "EP_LOOP:\n\t"                                                                                                \
+        BODY(CVT)                                                                                                     \
+        EP_ALL(EP_ADDR) EP_ALL(STORE) EP_ALL(EP_ADVANCE, #GROUP_BYTES)                                                \
+        EP_CALM_ALL                                                                                                   \
+        "setp.ge.and.u32 pq, lm, 32768, pq;\n\t"                                                                      \
+        "vote.sync.all.pred pq, pq, 0xffffffff;\n\t"                                                                  \
+        "@pq bra.uni EP_LOOP;\n\t"                                                                                    \
+        GUESS(CVT, STORE, GROUP_BYTES)                                                                                \
+        "EP_RARE:\n\t"                                                                                                \
+        /* lanes that reached their lim: into the next row (rows hold 32 blocks or more), or past the tile's last block */ \
+        "setp.ge.u32 pv, %3, limA;\n\t"                                                                               \
+        "vote.sync.any.pred pr, pv, 0xffffffff;\n\t"                                                                  \
+        "@!pr bra.uni EP_ROWS_END;\n\t"                                                                               \
+        "setp.lt.u32 actA, %3, endo;\n\t"                                                                             \
+        "@pv add.u32 rp, rp, 4;\n\t" "ld.shared.b32 sgA, [rp];\n\t" "@pv add.u32 limA, limA, rowb;\n\t"               \
+        "min.u32 limA, limA, endo;\n\t" "@!actA mov.u32 limA, 0xffffffff;\n\t"                                        \
+        "mov.b32 r3, sgA;\n\t" "mov.b64 ssA, {r3, r3};\n\t"                                                           \
+        "vote.sync.any.pred pr, actA, 0xffffffff;\n\t"                                                                \
+        "@!pr bra.uni EP_DONE;\n\t"                                                                                   \
+        "EP_ROWS_END:\n\t"                                                                                            \
+        /* the cursor reached the part that was still on its way at the start; a second time: past the payload, which only \
+           a damaged stream does - back to the front, and the position is spoilt so that the tile fails its check */   \
+        "setp.ge.u32 pr, %1, wthrA;\n\t"                                                                              \
+        "vote.sync.any.pred pr, pr, 0xffffffff;\n\t"                                                                  \
+        "@!pr bra.uni EP_LOOP;\n\t"                                                                                   \
+        "cp.async.wait_group 0;\n\t"                                                                                  \
+        "bar.warp.sync 0xffffffff;\n\t"                                                                               \
+        "ld.shared.v2.u32 {r0, r1}, [" EP_CTX "+48];\n\t"  /* ring base, position 0 */                                \
+        "ld.shared.u32 r3, [" EP_CTX "+44];\n\t"           /* the limit */                                            \
+        "setp.lt.u32 pq, wthrA, r3;\n\t"                                                                              \
+        "mov.b32 wthrA, r3;\n\t"                                                                                      \
+        "@pq bra.uni EP_LOOP;\n\t"                                                                                    \
+        "mov.b32 %1, r0;\n\t"                                                                                         \
+        "add.u32 r1, r1, 0x100000;\n\t"                                                                               \
+        "st.shared.u32 [" EP_CTX "+52], r1;\n\t"                                                                      \
+        "bra.uni EP_LOOP;\n\t"                                                                                        \
+        "EP_DONE:\n\t"                                                                                                \
+        "}"                                                                                                           \
+        : "+&r"(x), "+&r"(a), "+&r"(bal), "+&r"(doff)                                                                 \
+        : "r"(lt), "r"(lut_addr), "r"(lut_addr + kCosetStride), "r"(ctx), "l"(kk), "l"(out_base), "r"(cf.f0), "r"(cf.f1), \
+          "r"(rp), "r"(lim), "r"(wthr)                                                                                \
+        : "memory")
+
 // kChains tiles of a tensor whose rows hold at least 32 blocks and whose tables have 2^B slots (B = 11: one-level
 // tables; B = 12: two levels, see EP_M1); chain c takes tile
 // `first + c`.  A chain whose slot lies past the job's last tile gets that last tile's record, only so that its
@@ -1124,20 +1290,96 @@ __device__ __forceinline__ void decode_tiles_fast(const JobParams &J, uint32_t f
     __syncwarp();                 // the context block is rewritten by the next tiles
 }
 
+// One tile of a CTA that has few of them (2^11-slot streams, rows of 32 blocks or more): its payload is brought into shared
+// memory whole - the stages of a round's tiles share the space of the 32 rings and of the hot window - and decoded by the
+// loop that is short in latency, not in instructions.  A tile too long for its stage takes the ordinary loop, its ring at
+// the start of the stage.
+template <int DT>
+__device__ __forceinline__ void decode_tile_few(const JobParams &J, uint32_t first, uint32_t tiles_per_round, uint32_t lut_addr,
+                                                CosetFreq cf, uint32_t ctx, uint32_t lane, bool tables_pending) {
+    constexpr uint32_t BB = Out<DT>::kBlockBytes, kHead = 1024, kTail = 1024;
+    const uint32_t warp = threadIdx.x >> 5, space = kStageBytes / tiles_per_round & ~127u;
+    const bool valid = first < J.tile_cnt && warp < tiles_per_round;
+    const uint32_t scales = lut_addr + kRingBase + min(warp, tiles_per_round - 1u) * space;   // row scales, then the payload
+    const uint32_t tile = J.tile0 + min(first, J.tile_cnt - 1u);
+    const TileSetup T = tile_setup(J, tile, valid, lane);
+    const uint32_t row0 = T.v0 / J.per_row, rows = valid ? (T.v0 + T.nv - 1u) / J.per_row - row0 + 1u : 0u;
+    const uint32_t scale_bytes = (4u * rows + 4u + 127u) & ~127u, stage = scales + scale_bytes, room = space - scale_bytes;
+    const uint32_t bytes = valid ? T.lead + 2u * (min(T.end, J.total_words) - min(T.off, T.end)) : 0u;
+    if (valid && (scale_bytes >= space || bytes + kTail > room)) {            // (the same for all lanes)
+        decode_tiles_fast<DT, 11>(J, first, tiles_per_round, lut_addr, cf, scales, ctx, lane, tables_pending);
+        return;
+    }
+    // the scales and the first kilobyte, then the rest, as two groups of copies
+    for (uint32_t i = lane; i < rows; i += 32u)
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(scales + 4u * i), "l"(J.scales + row0 + i) : "memory");
+    for (uint32_t o = 16u * lane; o < min(bytes, kHead); o += 512u)
+        cp_async16(stage + o, T.a0 + (o < T.room ? o : 0u), o < T.room ? min(16u, T.room - o) : 0u);
+    cp_async_commit();
+    for (uint32_t o = kHead + 16u * lane; o < bytes; o += 512u)
+        cp_async16(stage + o, T.a0 + (o < T.room ? o : 0u), o < T.room ? min(16u, T.room - o) : 0u);
+    cp_async_commit();
+    uint32_t x = T.x, a = stage + T.lead, bal = 0, doff = (T.v0 + lane) * BB;
+    const uint32_t endo = (T.v0 + T.nv) * BB;
+    const uint32_t row = min(T.v0 + lane, T.v0 + T.nv - 1u) / J.per_row;
+    const uint32_t rp = scales + 4u * (row - row0), lim = min((row + 1u) * J.row_bytes, endo);
+    // a group reads at most 510 bytes from the cursor on; a valid tile's cursor never passes its last word
+    const uint32_t limit = stage + room - 512u, wthr = bytes > kHead ? stage + kHead - 512u : limit;
+    if (valid && lane == 0) {
+        sts32(ctx + kCtxChain + kCcDst, limit);
+        sts32(ctx + kCtxChain + kCcRing, stage);
+        sts32(ctx + kCtxChain + kCcWbase, stage);
+        sts32(ctx + kCtxChain + kCcEndo, endo);
+    }
+    cp_async_wait<1>();           // the table image, if any, and the first kilobyte
+    __syncwarp();
+    if (tables_pending) __syncthreads();
+    if (!valid) return;
+    const uint32_t k0 = __float_as_uint(float(4096 - J.zlo)), lt = (1u << lane) - 1u;
+    const uint64_t kk = pack64(k0, k0), out_base = reinterpret_cast<uint64_t>(J.out);
+    if (J.guess) {
+        if constexpr (DT == EP_BF16) EP_FEW_LOOP_ASM(EP_BODY11_GUESS, EP_GUESS_CHECK, EP_CVT_BF16, EP_ST_16, 512);
+        else if constexpr (DT == EP_FP16) EP_FEW_LOOP_ASM(EP_BODY11_GUESS, EP_GUESS_CHECK, EP_CVT_FP16, EP_ST_16, 512);
+        else if constexpr (DT == EP_FP8_E4M3) EP_FEW_LOOP_ASM(EP_BODY11_GUESS, EP_GUESS_CHECK, EP_CVT_E4M3, EP_ST_F8, 256);
+        else if constexpr (DT == EP_FP8_E5M2) EP_FEW_LOOP_ASM(EP_BODY11_GUESS, EP_GUESS_CHECK, EP_CVT_E5M2, EP_ST_F8, 256);
+        else if constexpr (DT == EP_FP32) EP_FEW_LOOP_ASM(EP_BODY11_GUESS, EP_GUESS_CHECK, EP_CVT_FP32, EP_ST_FP32, 1024);
+        else if constexpr (DT == EP_UINT8) EP_FEW_LOOP_ASM(EP_BODY11_GUESS, EP_GUESS_CHECK, EP_CVT_I8, EP_ST_UINT8, 256);
+        else EP_FEW_LOOP_ASM(EP_BODY11_GUESS, EP_GUESS_CHECK, EP_CVT_I8, EP_ST_INT8, 256);
+    } else {
+        if constexpr (DT == EP_BF16) EP_FEW_LOOP_ASM(EP_BODY11_SHORT, EP_GUESS_NONE, EP_CVT_BF16, EP_ST_16, 512);
+        else if constexpr (DT == EP_FP16) EP_FEW_LOOP_ASM(EP_BODY11_SHORT, EP_GUESS_NONE, EP_CVT_FP16, EP_ST_16, 512);
+        else if constexpr (DT == EP_FP8_E4M3) EP_FEW_LOOP_ASM(EP_BODY11_SHORT, EP_GUESS_NONE, EP_CVT_E4M3, EP_ST_F8, 256);
+        else if constexpr (DT == EP_FP8_E5M2) EP_FEW_LOOP_ASM(EP_BODY11_SHORT, EP_GUESS_NONE, EP_CVT_E5M2, EP_ST_F8, 256);
+        else if constexpr (DT == EP_FP32) EP_FEW_LOOP_ASM(EP_BODY11_SHORT, EP_GUESS_NONE, EP_CVT_FP32, EP_ST_FP32, 1024);
+        else if constexpr (DT == EP_UINT8) EP_FEW_LOOP_ASM(EP_BODY11_SHORT, EP_GUESS_NONE, EP_CVT_I8, EP_ST_UINT8, 256);
+        else EP_FEW_LOOP_ASM(EP_BODY11_SHORT, EP_GUESS_NONE, EP_CVT_I8, EP_ST_INT8, 256);
+    }
+    cp_async_wait<0>();           // nothing may still be landing in the stage when the next tile starts
+    __syncwarp();
+    const uint32_t cur = __shfl_sync(0xFFFFFFFFu, a, 0) + 2u * __popc(bal) - lds32(ctx + kCtxChain + kCcWbase);
+    const bool bad = (x != ep::kStateLow) || (T.off + ((cur - T.lead) >> 1) != T.end);
+    if (__any_sync(0xFFFFFFFFu, bad) && lane == 0) atomicOr(&g_ep_status, 1u);
+    __syncwarp();
+}
+
 // One persistent CTA per SM.  The rounds of all jobs of the launch form one list (job after job); CTA k takes the
 // rounds whose cumulative cost at their start lies in [k, k + 1) * ceil(total / gridDim.x) - a contiguous stretch,
 // usually inside one job - and sets the lookup tables up again when the stretch crosses into the next job.  Everything
 // that steers this (loop bounds, job changes) depends on blockIdx and kernel parameters only, so the compiler
 // sees warp-uniform control flow and puts no divergence guards around the warp votes of the hot loop; in the last
 // round of a job a chain past the job's last tile goes through the same code with no block to decode.
-template <int DT>
-__global__ void __launch_bounds__(kThreads, 1) ep_decode_smem_kernel(const __grid_constant__ BatchParams P) {
+// FEW: launches of few tiles per CTA (see decode_tile_few); a kernel of its own because it may use 168 registers where 32 warps
+// leave 64.
+template <int DT, bool FEW>
+__global__ void __launch_bounds__(FEW ? 32 * (kFewTiles > kMinWarps ? kFewTiles : kMinWarps) : kThreads, 1)
+ep_decode_smem_kernel(const __grid_constant__ BatchParams P) {
     extern __shared__ __align__(16) uint8_t smem[];
     const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
     const uint32_t lut_addr = uint32_t(__cvta_generic_to_shared(smem));
     const uint32_t ring = lut_addr + kRingBase + warp * (kChains * kRingStride);
     const uint32_t ctx = lut_addr + kCtxBase + warp * kCtxBytes;
     bool tables_in_use = false;
+    wait_for_stream();
     for (int j = 0; j < P.n_jobs; ++j) {
         const JobParams &J = P.job[j];
         // rounds r of this job with cost_begin + r * round_cost in [lo, hi), this CTA's share of the total cost
@@ -1172,6 +1414,8 @@ __global__ void __launch_bounds__(kThreads, 1) ep_decode_smem_kernel(const __gri
                 if (fast) {
                     if (kTwoLevelInLoop && J.b == 12u) {
                         if constexpr (kTwoLevelInLoop) decode_tiles_fast<DT, 12>(J, base, P.tiles_per_round, lut_addr, cf, ring, ctx, lane, tables_pending);
+                    } else if constexpr (FEW) {
+                        decode_tile_few<DT>(J, base, P.tiles_per_round, lut_addr, cf, ctx, lane, tables_pending);
                     } else {
                         decode_tiles_fast<DT, 11>(J, base, P.tiles_per_round, lut_addr, cf, ring, ctx, lane, tables_pending);
                     }
@@ -1782,6 +2026,23 @@ void fill_table_params(JobParams &J, const ep_info &I) {
     }
 }
 
+// A launch that may overlap the end of the kernel before it (see wait_for_stream, which `kernel` begins with): the next
+// decode is then resident when its turn comes instead of being launched then.
+template <class... A>
+cudaError_t launch_next(void (*kernel)(A...), uint32_t grid, uint32_t threads, uint32_t smem, cudaStream_t st, const A &...args) {
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
 // How the tiles of a launch are spread over its CTAs (persistent, one per SM): sets tiles_per_round, every job's rounds and
 // costs and cost_per_cta; returns the grid size, 0 if the counts do not fit 32 bits.
 // A round is one tile per warp, and its warps share an SM's issue slots: 32 of them take 1.05 us for a group of 32 blocks
@@ -1818,20 +2079,23 @@ uint32_t split_rounds(BatchParams &P, uint32_t sms) {
     return grid;
 }
 
-template <int DT>
-cudaError_t launch_smem(const BatchParams &P, uint32_t grid, cudaStream_t st) {
+template <int DT, bool FEW>
+cudaError_t launch_smem_as(const BatchParams &P, uint32_t grid, uint32_t warps, cudaStream_t st) {
     static bool configured[64] = {};   // the attribute is per device
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= 64 || !configured[dev]) {
-        e = cudaFuncSetAttribute(ep_decode_smem_kernel<DT>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kSmemBytes));
+        e = cudaFuncSetAttribute(ep_decode_smem_kernel<DT, FEW>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kSmemBytes));
         if (e != cudaSuccess) return e;
         if (dev >= 0 && dev < 64) configured[dev] = true;
     }
+    return launch_next(ep_decode_smem_kernel<DT, FEW>, grid, 32u * (warps < kMinWarps ? kMinWarps : warps), kSmemBytes, st, P);
+}
+template <int DT>
+cudaError_t launch_smem(const BatchParams &P, uint32_t grid, cudaStream_t st) {
     const uint32_t warps = (P.tiles_per_round + kChains - 1u) / kChains;
-    ep_decode_smem_kernel<DT><<<grid, 32u * (warps < kMinWarps ? kMinWarps : warps), kSmemBytes, st>>>(P);
-    return cudaGetLastError();
+    return kChains == 1 && warps <= kFewTiles ? launch_smem_as<DT, true>(P, grid, warps, st) : launch_smem_as<DT, false>(P, grid, warps, st);
 }
 
 size_t large_table_bytes(const ep_info &I) { return size_t(EP_NUM_TABLES) * (size_t(1) << I.b) * 4u; }
@@ -2118,6 +2382,7 @@ extern "C" int ep_decode_batch(const ep_decode_job *jobs_in, int32_t n_in, void 
         J.row_bytes = J.per_row * block_bytes;
         J.row_rcp = uint32_t(0xFFFFFFFFu / J.row_bytes + 1u);
         J.row_max = I.R - 1u;
+        J.guess = double(I.total_words) * 16.0 <= kGuessBits * 9.0 * double(J.n_vec);
     }
     const uint32_t next = split_rounds(P, uint32_t(sms));      // grid size
     if (next == 0) return EP_ERR_UNSUPPORTED;
