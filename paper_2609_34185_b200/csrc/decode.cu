@@ -876,15 +876,16 @@ __device__ __forceinline__ void decode_tile_plain(const JobParams &J, uint32_t t
 #define EP_T_RENORM(BIN, BOUT)                                                                                        \
         "setp.lt.and.u32 pA, %0, 32768, actA;\n\t" "vote.sync.ballot.b32 " BOUT ", pA, 0xffffffff;\n\t"               \
         "mov.b32 va, %0;\n\t" "lop3.b32 tA, " EP_LT ", " BOUT ", " BIN ", 0xCA;\n\t" "popc.b32 tA, tA;\n\t"           \
-        "mad.lo.u32 %1, tA, 2, %1;\n\t" "@pA ld.shared.u16 va, [%1];\n\t" "@pA mad.lo.u32 %0, %0, 65536, va;\n\t"
+        "mad.lo.u32 %1, tA, 2, %1;\n\t" "@pA ld.shared.u16 va, [%1];\n\t"
+#define EP_T_TAKE "@pA mad.lo.u32 %0, %0, 65536, va;\n\t"
 #define EP_T_STEP(E, OFF, BIN, BOUT)                                                                                  \
         "and.b32 uA, va, 0x7FF;\n\t" "mad.lo.u32 uA, uA, 4, tabA;\n\t" "ld.shared.u32 " E "A, [uA+" OFF "];\n\t"      \
         "shr.u32 qA, %0, 11;\n\t" "shr.u32 fA, " E "A, 21;\n\t" "and.b32 biA, " E "A, 0x7FF;\n\t"                     \
-        "@actA mad.lo.u32 %0, fA, qA, biA;\n\t" EP_T_RENORM(BIN, BOUT)
+        "@actA mad.lo.u32 %0, fA, qA, biA;\n\t" EP_T_RENORM(BIN, BOUT) EP_T_TAKE
 #define EP_T_COSET                                                                                                    \
         EP_ALL(EP_C1) EP_ALL(EP_C2) EP_ALL(EP_C3) EP_ALL(EP_C4) EP_ALL(EP_C5) EP_ALL(EP_C6) EP_ALL(EP_C7) EP_ALL(EP_C8)
 #define EP_BODY11_SHORT(CVT)                                                                                          \
-        EP_T_COSET EP_T_RENORM("%2", "naA")                                                                           \
+        EP_T_COSET EP_T_RENORM("%2", "naA") EP_T_TAKE                                                                 \
         EP_T_STEP("e1", "0", "naA", "nbA")     EP_ALL(EP_XA, "e1")                                                    \
         EP_T_STEP("e2", "8192", "nbA", "naA")  EP_ALL(EP_XB, "e2") EP_PAIR_ALL EP_ALL(CVT, "0")                       \
         EP_T_STEP("e3", "16384", "naA", "nbA") EP_ALL(EP_PAR3, "e1", "e2", "e3") EP_ALL(EP_XA, "e3")                  \
@@ -892,7 +893,11 @@ __device__ __forceinline__ void decode_tile_plain(const JobParams &J, uint32_t t
         EP_T_STEP("e5", "32768", "naA", "nbA") EP_ALL(EP_PAR3, "par", "e4", "e5") EP_ALL(EP_XA, "e5")                 \
         EP_T_STEP("e6", "40960", "nbA", "naA") EP_ALL(EP_XB, "e6") EP_PAIR_ALL EP_ALL(CVT, "2")                       \
         EP_T_STEP("e7", "49152", "naA", "nbA") EP_ALL(EP_PAR3, "par", "e6", "e7") EP_ALL(EP_XA, "e7")                 \
-        EP_T_STEP("e8", "57344", "nbA", "%2") EP_ALL(EP_PARX) EP_ALL(EP_X8) EP_PAIR_ALL EP_ALL(CVT, "3")
+        "and.b32 uA, va, 0x7FF;\n\t" "mad.lo.u32 uA, uA, 4, tabA;\n\t" "ld.shared.u32 e8A, [uA+57344];\n\t"           \
+        "shr.u32 qA, %0, 11;\n\t" "shr.u32 fA, e8A, 21;\n\t" "and.b32 biA, e8A, 0x7FF;\n\t"                           \
+        "@actA mad.lo.u32 %0, fA, qA, biA;\n\t" EP_T_RENORM("nbA", "%2")                                              \
+        EP_ALL(EP_PARX) EP_ALL(EP_X8) EP_PAIR_ALL EP_ALL(CVT, "3")
+#define EP_SHORT_FIN EP_T_TAKE      /* the last words go into the states after the loop's test: its vote fills the wait */
 
 // EP_BODY11_GUESS: a lane that takes a word in step k hardly ever takes another in step k + 1 (its state is then at least
 // 2^20 and usually above 2^26, and a step shortens a state by eleven bits at most), and no other lane needs a word to go on.
@@ -938,8 +943,8 @@ __device__ __forceinline__ void decode_tile_plain(const JobParams &J, uint32_t t
                   EP_ALL(EP_PAR3, "par", "e6", "e7") EP_ALL(EP_XA, "e7"))                                             \
         EP_G_RANK("%2", "nbA") EP_G_TAIL("e8", "ps")                                                                  \
         "mad.lo.u32 %1, tA, 2, %1;\n\t" "@pA ld.shared.u16 wA, [%1];\n\t" EP_G_TAIL_REST("e8", "ps")                  \
-        EP_ALL(EP_PARX) EP_ALL(EP_X8) EP_PAIR_ALL EP_ALL(CVT, "3")                                                    \
-        "@pA mad.lo.u32 %0, %0, 65536, wA;\n\t"
+        EP_ALL(EP_PARX) EP_ALL(EP_X8) EP_PAIR_ALL EP_ALL(CVT, "3")
+#define EP_GUESS_FIN "@pA mad.lo.u32 %0, %0, 65536, wA;\n\t"
 
 // per output type: CVT(S, j, lo, hi) turns weights 2j, 2j+1 into their stored form, STORE(S) writes the block
 #define EP_CVT_BF16(S, X, AW, BAL, DOFF, CB, J) "cvt.rn.bf16x2.f32 o" J S ", wh" S ", wl" S ";\n\t"
@@ -1149,15 +1154,15 @@ __device__ __forceinline__ void decode_tile_plain(const JobParams &J, uint32_t t
         "vote.sync.any.pred pr, pr, 0xffffffff;\n\t"                                                                  \
         "@!pr bra.uni EP_RARE;\n\t"                                                                                   \
         "mov.b32 %0, sx;\n\t" "mov.b32 %1, sa;\n\t" "mov.b32 %2, sb;\n\t" "sub.u32 %3, %3, " #GROUP_BYTES ";\n\t"     \
-        EP_BODY11_SHORT(CVT)                                                                                          \
+        EP_BODY11_SHORT(CVT) EP_SHORT_FIN                                                                             \
         EP_ALL(EP_ADDR) EP_ALL(STORE) EP_ALL(EP_ADVANCE, #GROUP_BYTES)
 #define EP_GUESS_NONE(CVT, STORE, GROUP_BYTES)
-#define EP_FEW_LOOP_ASM(BODY, GUESS, CVT, STORE, GROUP_BYTES)                                                         \
+#define EP_FEW_LOOP_ASM(BODY, FIN, GUESS, CVT, STORE, GROUP_BYTES)                                                    \
     asm volatile(                                                                                                     \
         "{\n\t"                                                                                                       \
         EP_ALL(EP_REGS)                                                                                               \
         ".reg .pred pq, pv, pr, ps, pn;\n\t"                                                                          \
-        ".reg .b32 r0, r1, r3, c0r, c1r, f0c, lm, sx, sa, sb, ea, va, f2, b2, q2, rp, rowb, endo;\n\t"     \
+        ".reg .b32 r0, r1, r2, r3, r4, r5, r6, r7, r10, r11, r12, c0r, c1r, f0c, lm, sx, sa, sb, ea, va, f2, b2, q2, rp, rowb, endo;\n\t"     \
         ".reg .b64 ra, rb;\n\t"                                                                                       \
         ".reg .f32 k0f, k1f;\n\t"                                                                                     \
         "mov.b64 {k0f, k1f}, " EP_KK ";\n\t"                                                                          \
@@ -1178,6 +1183,7 @@ __device__ __forceinline__ void decode_tile_plain(const JobParams &J, uint32_t t
         EP_CALM_ALL                                                                                                   \
         "setp.ge.and.u32 pq, lm, 32768, pq;\n\t"                                                                      \
         "vote.sync.all.pred pq, pq, 0xffffffff;\n\t"                                                                  \
+        FIN                                                                                                           \
         "@pq bra.uni EP_LOOP;\n\t"                                                                                    \
         GUESS(CVT, STORE, GROUP_BYTES)                                                                                \
         "EP_RARE:\n\t"                                                                                                \
@@ -1192,21 +1198,37 @@ __device__ __forceinline__ void decode_tile_plain(const JobParams &J, uint32_t t
         "vote.sync.any.pred pr, actA, 0xffffffff;\n\t"                                                                \
         "@!pr bra.uni EP_DONE;\n\t"                                                                                   \
         "EP_ROWS_END:\n\t"                                                                                            \
-        /* the cursor reached the part that was still on its way at the start; a second time: past the payload, which only \
-           a damaged stream does - back to the front, and the position is spoilt so that the tile fails its check */   \
         "setp.ge.u32 pr, %1, wthrA;\n\t"                                                                              \
         "vote.sync.any.pred pr, pr, 0xffffffff;\n\t"                                                                  \
         "@!pr bra.uni EP_LOOP;\n\t"                                                                                   \
+        /* the cursor reached what was still on its way when the loop began */                                        \
         "cp.async.wait_group 0;\n\t"                                                                                  \
         "bar.warp.sync 0xffffffff;\n\t"                                                                               \
-        "ld.shared.v2.u32 {r0, r1}, [" EP_CTX "+48];\n\t"  /* ring base, position 0 */                                \
-        "ld.shared.u32 r3, [" EP_CTX "+44];\n\t"           /* the limit */                                            \
-        "setp.lt.u32 pq, wthrA, r3;\n\t"                                                                              \
-        "mov.b32 wthrA, r3;\n\t"                                                                                      \
+        "ld.shared.v4.u32 {r11, r12, r1, r2}, [" EP_CTX "+32];\n\t"   /* source of the window, bytes from there, limit */ \
+        "ld.shared.v2.u32 {r10, r5}, [" EP_CTX "+48];\n\t"            /* window, address of position 0 */             \
+        "setp.lt.u32 pq, wthrA, r2;\n\t"                                                                              \
+        "mov.b32 wthrA, r2;\n\t"                                                                                      \
         "@pq bra.uni EP_LOOP;\n\t"                                                                                    \
-        "mov.b32 %1, r0;\n\t"                                                                                         \
-        "add.u32 r1, r1, 0x100000;\n\t"                                                                               \
-        "st.shared.u32 [" EP_CTX "+52], r1;\n\t"                                                                      \
+        /* or the window's end: the window moves on to the cursor (lane 0's address is the lowest), and all of it is copied */ \
+        "shfl.sync.idx.b32 r3, %1, 0, 31, 0xffffffff;\n\t"                                                            \
+        "sub.u32 r3, r3, r10;\n\t" "and.b32 r3, r3, 0xfffffff0;\n\t"                                                  \
+        "sub.u32 %1, %1, r3;\n\t" "sub.u32 r5, r5, r3;\n\t" "sub.s32 r1, r1, r3;\n\t"                                 \
+        "add.cc.u32 r11, r11, r3;\n\t" "addc.u32 r12, r12, 0;\n\t" "mov.b64 ra, {r11, r12};\n\t"                      \
+        "bar.warp.sync 0xffffffff;\n\t"                                                                               \
+        "st.shared.v2.u32 [" EP_CTX "+32], {r11, r12};\n\t" "st.shared.u32 [" EP_CTX "+40], r1;\n\t"                  \
+        "st.shared.u32 [" EP_CTX "+52], r5;\n\t"                                                                      \
+        "mov.b32 r0, " EP_LT ";\n\t" "popc.b32 r0, r0;\n\t" "shl.b32 r0, r0, 4;\n\t"      /* 16 * lane */             \
+        "sub.u32 r4, r2, r10;\n\t" "add.u32 r4, r4, 512;\n\t"                             /* the window's size */     \
+        "EP_FILL:\n\t"                                                                                                \
+        "sub.s32 r6, r1, r0;\n\t" "min.s32 r6, r6, 16;\n\t" "setp.gt.s32 pv, r6, 0;\n\t"                              \
+        "setp.lt.and.u32 pv, r0, r4, pv;\n\t"                                                                         \
+        "mad.wide.u32 rb, r0, 1, ra;\n\t" "add.u32 r7, r10, r0;\n\t"                                                  \
+        "@pv cp.async.cg.shared.global [r7], [rb], 16, r6;\n\t"                                                       \
+        "add.u32 r0, r0, 512;\n\t"                                                                                    \
+        "vote.sync.any.pred pv, pv, 0xffffffff;\n\t"                                                                  \
+        "@pv bra.uni EP_FILL;\n\t"                                                                                    \
+        "cp.async.wait_all;\n\t"                                                                                      \
+        "bar.warp.sync 0xffffffff;\n\t"                                                                               \
         "bra.uni EP_LOOP;\n\t"                                                                                        \
         "EP_DONE:\n\t"                                                                                                \
         "}"                                                                                                           \
@@ -1290,74 +1312,72 @@ __device__ __forceinline__ void decode_tiles_fast(const JobParams &J, uint32_t f
     __syncwarp();                 // the context block is rewritten by the next tiles
 }
 
-// One tile of a CTA that has few of them (2^11-slot streams, rows of 32 blocks or more): its payload is brought into shared
-// memory whole - the stages of a round's tiles share the space of the 32 rings and of the hot window - and decoded by the
-// loop that is short in latency, not in instructions.  A tile too long for its stage takes the ordinary loop, its ring at
-// the start of the stage.
+// One tile of a CTA that has few of them (2^11-slot streams, rows of 32 blocks or more), decoded by the loop that is short in
+// latency, not in instructions.  The tiles of a round share the space of the 32 rings and of the hot window: 8 KB for each
+// of twelve, which holds a tile's row scales and, usually, all of its payload.  (As in decode_tiles_fast every branch
+// depends on parameters or is a bra.uni on a vote: a guard around each vote would cost 25 cycles.)
 template <int DT>
 __device__ __forceinline__ void decode_tile_few(const JobParams &J, uint32_t first, uint32_t tiles_per_round, uint32_t lut_addr,
                                                 CosetFreq cf, uint32_t ctx, uint32_t lane, bool tables_pending) {
-    constexpr uint32_t BB = Out<DT>::kBlockBytes, kHead = 1024, kTail = 1024;
+    constexpr uint32_t BB = Out<DT>::kBlockBytes, kHead = 1024;
     const uint32_t warp = threadIdx.x >> 5, space = kStageBytes / tiles_per_round & ~127u;
     const bool valid = first < J.tile_cnt && warp < tiles_per_round;
-    const uint32_t scales = lut_addr + kRingBase + min(warp, tiles_per_round - 1u) * space;   // row scales, then the payload
+    const uint32_t scales = lut_addr + kRingBase + min(warp, tiles_per_round - 1u) * space;   // row scales, then the window
     const uint32_t tile = J.tile0 + min(first, J.tile_cnt - 1u);
     const TileSetup T = tile_setup(J, tile, valid, lane);
     const uint32_t row0 = T.v0 / J.per_row, rows = valid ? (T.v0 + T.nv - 1u) / J.per_row - row0 + 1u : 0u;
-    const uint32_t scale_bytes = (4u * rows + 4u + 127u) & ~127u, stage = scales + scale_bytes, room = space - scale_bytes;
-    const uint32_t bytes = valid ? T.lead + 2u * (min(T.end, J.total_words) - min(T.off, T.end)) : 0u;
-    if (valid && (scale_bytes >= space || bytes + kTail > room)) {            // (the same for all lanes)
-        decode_tiles_fast<DT, 11>(J, first, tiles_per_round, lut_addr, cf, scales, ctx, lane, tables_pending);
-        return;
-    }
+    const uint32_t scale_bytes = (4u * ((J.V + J.per_row - 1u) / J.per_row + 2u) + 127u) & ~127u;    // (checked by the launcher)
+    const uint32_t window = scales + scale_bytes, size = space - scale_bytes;
+    const uint32_t bytes = valid ? min(T.lead + 2u * (min(T.end, J.total_words) - min(T.off, T.end)), size) : 0u;
     // the scales and the first kilobyte, then the rest, as two groups of copies
     for (uint32_t i = lane; i < rows; i += 32u)
         asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(scales + 4u * i), "l"(J.scales + row0 + i) : "memory");
     for (uint32_t o = 16u * lane; o < min(bytes, kHead); o += 512u)
-        cp_async16(stage + o, T.a0 + (o < T.room ? o : 0u), o < T.room ? min(16u, T.room - o) : 0u);
+        cp_async16(window + o, T.a0 + (o < T.room ? o : 0u), o < T.room ? min(16u, T.room - o) : 0u);
     cp_async_commit();
     for (uint32_t o = kHead + 16u * lane; o < bytes; o += 512u)
-        cp_async16(stage + o, T.a0 + (o < T.room ? o : 0u), o < T.room ? min(16u, T.room - o) : 0u);
+        cp_async16(window + o, T.a0 + (o < T.room ? o : 0u), o < T.room ? min(16u, T.room - o) : 0u);
     cp_async_commit();
-    uint32_t x = T.x, a = stage + T.lead, bal = 0, doff = (T.v0 + lane) * BB;
+    uint32_t x = T.x, a = window + T.lead, bal = 0, doff = (T.v0 + lane) * BB;
     const uint32_t endo = (T.v0 + T.nv) * BB;
-    const uint32_t row = min(T.v0 + lane, T.v0 + T.nv - 1u) / J.per_row;
+    const uint32_t row = min(T.v0 + lane, T.v0 + max(T.nv, 1u) - 1u) / J.per_row;
     const uint32_t rp = scales + 4u * (row - row0), lim = min((row + 1u) * J.row_bytes, endo);
-    // a group reads at most 510 bytes from the cursor on; a valid tile's cursor never passes its last word
-    const uint32_t limit = stage + room - 512u, wthr = bytes > kHead ? stage + kHead - 512u : limit;
-    if (valid && lane == 0) {
+    // a group reads at most 510 bytes from the cursor on
+    const uint32_t limit = window + size - 512u, wthr = bytes > kHead ? window + kHead - 512u : limit;
+    if (lane == 0 && warp < tiles_per_round) {
+        sts64(ctx + kCtxChain + kCcSrc, T.a0);
+        sts32(ctx + kCtxChain + kCcRem, T.room);
         sts32(ctx + kCtxChain + kCcDst, limit);
-        sts32(ctx + kCtxChain + kCcRing, stage);
-        sts32(ctx + kCtxChain + kCcWbase, stage);
-        sts32(ctx + kCtxChain + kCcEndo, endo);
+        sts32(ctx + kCtxChain + kCcRing, window);
+        sts32(ctx + kCtxChain + kCcWbase, window);
     }
+    if (lane == 0) sts32(ctx + kCtxChain + kCcEndo, endo);
     cp_async_wait<1>();           // the table image, if any, and the first kilobyte
     __syncwarp();
     if (tables_pending) __syncthreads();
-    if (!valid) return;
     const uint32_t k0 = __float_as_uint(float(4096 - J.zlo)), lt = (1u << lane) - 1u;
     const uint64_t kk = pack64(k0, k0), out_base = reinterpret_cast<uint64_t>(J.out);
     if (J.guess) {
-        if constexpr (DT == EP_BF16) EP_FEW_LOOP_ASM(EP_BODY11_GUESS, EP_GUESS_CHECK, EP_CVT_BF16, EP_ST_16, 512);
-        else if constexpr (DT == EP_FP16) EP_FEW_LOOP_ASM(EP_BODY11_GUESS, EP_GUESS_CHECK, EP_CVT_FP16, EP_ST_16, 512);
-        else if constexpr (DT == EP_FP8_E4M3) EP_FEW_LOOP_ASM(EP_BODY11_GUESS, EP_GUESS_CHECK, EP_CVT_E4M3, EP_ST_F8, 256);
-        else if constexpr (DT == EP_FP8_E5M2) EP_FEW_LOOP_ASM(EP_BODY11_GUESS, EP_GUESS_CHECK, EP_CVT_E5M2, EP_ST_F8, 256);
-        else if constexpr (DT == EP_FP32) EP_FEW_LOOP_ASM(EP_BODY11_GUESS, EP_GUESS_CHECK, EP_CVT_FP32, EP_ST_FP32, 1024);
-        else if constexpr (DT == EP_UINT8) EP_FEW_LOOP_ASM(EP_BODY11_GUESS, EP_GUESS_CHECK, EP_CVT_I8, EP_ST_UINT8, 256);
-        else EP_FEW_LOOP_ASM(EP_BODY11_GUESS, EP_GUESS_CHECK, EP_CVT_I8, EP_ST_INT8, 256);
+        if constexpr (DT == EP_BF16) EP_FEW_LOOP_ASM(EP_BODY11_GUESS, EP_GUESS_FIN, EP_GUESS_CHECK, EP_CVT_BF16, EP_ST_16, 512);
+        else if constexpr (DT == EP_FP16) EP_FEW_LOOP_ASM(EP_BODY11_GUESS, EP_GUESS_FIN, EP_GUESS_CHECK, EP_CVT_FP16, EP_ST_16, 512);
+        else if constexpr (DT == EP_FP8_E4M3) EP_FEW_LOOP_ASM(EP_BODY11_GUESS, EP_GUESS_FIN, EP_GUESS_CHECK, EP_CVT_E4M3, EP_ST_F8, 256);
+        else if constexpr (DT == EP_FP8_E5M2) EP_FEW_LOOP_ASM(EP_BODY11_GUESS, EP_GUESS_FIN, EP_GUESS_CHECK, EP_CVT_E5M2, EP_ST_F8, 256);
+        else if constexpr (DT == EP_FP32) EP_FEW_LOOP_ASM(EP_BODY11_GUESS, EP_GUESS_FIN, EP_GUESS_CHECK, EP_CVT_FP32, EP_ST_FP32, 1024);
+        else if constexpr (DT == EP_UINT8) EP_FEW_LOOP_ASM(EP_BODY11_GUESS, EP_GUESS_FIN, EP_GUESS_CHECK, EP_CVT_I8, EP_ST_UINT8, 256);
+        else EP_FEW_LOOP_ASM(EP_BODY11_GUESS, EP_GUESS_FIN, EP_GUESS_CHECK, EP_CVT_I8, EP_ST_INT8, 256);
     } else {
-        if constexpr (DT == EP_BF16) EP_FEW_LOOP_ASM(EP_BODY11_SHORT, EP_GUESS_NONE, EP_CVT_BF16, EP_ST_16, 512);
-        else if constexpr (DT == EP_FP16) EP_FEW_LOOP_ASM(EP_BODY11_SHORT, EP_GUESS_NONE, EP_CVT_FP16, EP_ST_16, 512);
-        else if constexpr (DT == EP_FP8_E4M3) EP_FEW_LOOP_ASM(EP_BODY11_SHORT, EP_GUESS_NONE, EP_CVT_E4M3, EP_ST_F8, 256);
-        else if constexpr (DT == EP_FP8_E5M2) EP_FEW_LOOP_ASM(EP_BODY11_SHORT, EP_GUESS_NONE, EP_CVT_E5M2, EP_ST_F8, 256);
-        else if constexpr (DT == EP_FP32) EP_FEW_LOOP_ASM(EP_BODY11_SHORT, EP_GUESS_NONE, EP_CVT_FP32, EP_ST_FP32, 1024);
-        else if constexpr (DT == EP_UINT8) EP_FEW_LOOP_ASM(EP_BODY11_SHORT, EP_GUESS_NONE, EP_CVT_I8, EP_ST_UINT8, 256);
-        else EP_FEW_LOOP_ASM(EP_BODY11_SHORT, EP_GUESS_NONE, EP_CVT_I8, EP_ST_INT8, 256);
+        if constexpr (DT == EP_BF16) EP_FEW_LOOP_ASM(EP_BODY11_SHORT, EP_SHORT_FIN, EP_GUESS_NONE, EP_CVT_BF16, EP_ST_16, 512);
+        else if constexpr (DT == EP_FP16) EP_FEW_LOOP_ASM(EP_BODY11_SHORT, EP_SHORT_FIN, EP_GUESS_NONE, EP_CVT_FP16, EP_ST_16, 512);
+        else if constexpr (DT == EP_FP8_E4M3) EP_FEW_LOOP_ASM(EP_BODY11_SHORT, EP_SHORT_FIN, EP_GUESS_NONE, EP_CVT_E4M3, EP_ST_F8, 256);
+        else if constexpr (DT == EP_FP8_E5M2) EP_FEW_LOOP_ASM(EP_BODY11_SHORT, EP_SHORT_FIN, EP_GUESS_NONE, EP_CVT_E5M2, EP_ST_F8, 256);
+        else if constexpr (DT == EP_FP32) EP_FEW_LOOP_ASM(EP_BODY11_SHORT, EP_SHORT_FIN, EP_GUESS_NONE, EP_CVT_FP32, EP_ST_FP32, 1024);
+        else if constexpr (DT == EP_UINT8) EP_FEW_LOOP_ASM(EP_BODY11_SHORT, EP_SHORT_FIN, EP_GUESS_NONE, EP_CVT_I8, EP_ST_UINT8, 256);
+        else EP_FEW_LOOP_ASM(EP_BODY11_SHORT, EP_SHORT_FIN, EP_GUESS_NONE, EP_CVT_I8, EP_ST_INT8, 256);
     }
     cp_async_wait<0>();           // nothing may still be landing in the stage when the next tile starts
     __syncwarp();
     const uint32_t cur = __shfl_sync(0xFFFFFFFFu, a, 0) + 2u * __popc(bal) - lds32(ctx + kCtxChain + kCcWbase);
-    const bool bad = (x != ep::kStateLow) || (T.off + ((cur - T.lead) >> 1) != T.end);
+    const bool bad = valid && ((x != ep::kStateLow) || (T.off + ((cur - T.lead) >> 1) != T.end));
     if (__any_sync(0xFFFFFFFFu, bad) && lane == 0) atomicOr(&g_ep_status, 1u);
     __syncwarp();
 }
@@ -2095,7 +2115,10 @@ cudaError_t launch_smem_as(const BatchParams &P, uint32_t grid, uint32_t warps, 
 template <int DT>
 cudaError_t launch_smem(const BatchParams &P, uint32_t grid, cudaStream_t st) {
     const uint32_t warps = (P.tiles_per_round + kChains - 1u) / kChains;
-    return kChains == 1 && warps <= kFewTiles ? launch_smem_as<DT, true>(P, grid, warps, st) : launch_smem_as<DT, false>(P, grid, warps, st);
+    bool few = kChains == 1 && warps <= kFewTiles;
+    for (int i = 0; i < P.n_jobs && few; ++i)        // room for a tile's row scales and a window of 4 KB
+        few = 4u * (uint64_t(P.job[i].V) / P.job[i].per_row + 3u) + 128u + 4096u <= kStageBytes / warps;
+    return few ? launch_smem_as<DT, true>(P, grid, warps, st) : launch_smem_as<DT, false>(P, grid, warps, st);
 }
 
 size_t large_table_bytes(const ep_info &I) { return size_t(EP_NUM_TABLES) * (size_t(1) << I.b) * 4u; }
