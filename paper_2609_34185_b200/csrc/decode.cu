@@ -45,14 +45,9 @@ constexpr uint32_t kChains = EP_CHAINS;
 constexpr int kWarps = EP_WARPS;                             // warps per CTA (one CTA per SM)
 constexpr int kThreads = kWarps * 32;
 constexpr uint32_t kTilesPerRound = kWarps * kChains;        // tiles per CTA at a time, at most (see split_rounds)
-#ifndef EP_FEW_TILES
-#define EP_FEW_TILES 12
-#endif
-#ifndef EP_GUESS_BITS
-#define EP_GUESS_BITS 4.5
-#endif
-constexpr uint32_t kFewTiles = EP_FEW_TILES;                 // most tiles per CTA for decode_tile_few
-constexpr double kGuessBits = EP_GUESS_BITS;                 // most payload bits per symbol for its guessing loop
+// Most tiles per CTA for decode_tile_few: its 512 threads may use 128 registers.  1792-block tiles at 4 bpp to BF16, us, this
+// loop / the ordinary one: 4 tiles 37.1 / 40.0, 8: 38.7 / 41.3, 12: 41.8 / 43.8, 16: 45.4 / 46.6.
+constexpr uint32_t kFewTiles = 16;
 constexpr uint32_t kMinWarps = 8;                            // threads that copy the tables, however few tiles a CTA has
 static_assert(kTilesPerRound == ep::kDecodeTilesPerCta, "tile-size suggestions assume this many tiles per CTA");
 constexpr uint32_t kLutEntries = 2048;                       // 2^11 slots per table
@@ -125,6 +120,7 @@ struct JobParams {
     uint32_t row_bytes;           // output bytes per row
     uint32_t row_rcp;             // ceil(2^32 / row_bytes)
     uint32_t row_max;             // index of the last row
+    float payload_bits;           // mean payload bits per symbol
     uint32_t guess;               // decode_tile_few: the loop that guesses (see EP_BODY11_GUESS)
     int16_t tmin[EP_NUM_TABLES];
     uint16_t tK[EP_NUM_TABLES];
@@ -908,6 +904,10 @@ __device__ __forceinline__ void decode_tile_plain(const JobParams &J, uint32_t t
 // The order below follows the times at which operands arrive (a warp issues in order): rank of the words, the late lanes'
 // end of the previous step (TAIL, predicate NP from two steps ago), lookup, word, work for the output (FILL), the late
 // lanes' lookup, new state and ballot.
+// The assembler has an order of its own, 11 % slower (it takes the lookup of the late lanes and the work for the output
+// to where the ballot waits for them), but it moves nothing across a read of the clock: one after each ballot and one
+// after each word's load keep the order: 1070 -> 965 cycles per group.  (Their values have to be used: EP_G_KEEP, once
+// per tile.)
 // PB / PPB: ballots of the previous step and the one before; PP: the lanes that took a word; NB / NP: this step's.
 #define EP_G_TAIL(E, P)                                                                                               \
         "shr.u32 f2, ea, 21;\n\t" "and.b32 b2, ea, 0x7FF;\n\t" "@" P " mad.lo.u32 %0, f2, q2, b2;\n\t"
@@ -916,11 +916,12 @@ __device__ __forceinline__ void decode_tile_plain(const JobParams &J, uint32_t t
 #define EP_G_STEP(E, OFF, PB, PPB, PP, NB, NP, TAIL, TAILREST, FILL)                                                  \
         EP_G_RANK(PB, PPB) TAIL                                                                                       \
         "and.b32 uA, %0, 0x7FF;\n\t" "mad.lo.u32 uA, uA, 4, tabA;\n\t" "ld.shared.u32 " E "A, [uA+" OFF "];\n\t"      \
-        "mad.lo.u32 %1, tA, 2, %1;\n\t" "@" PP " ld.shared.u16 wA, [%1];\n\t"                                         \
+        "mad.lo.u32 %1, tA, 2, %1;\n\t" "@" PP " ld.shared.u16 wA, [%1];\n\t" "mov.u32 k" E ", %%clock;\n\t"          \
         "shr.u32 qA, %0, 11;\n\t" "not.pred pn, " PP ";\n\t" "and.pred pn, pn, actA;\n\t" TAILREST FILL               \
         "and.b32 va, wA, 0x7FF;\n\t" "mad.lo.u32 va, va, 4, tabA;\n\t" "@" PP " ld.shared.u32 ea, [va+" OFF "];\n\t"  \
         "shr.u32 fA, " E "A, 21;\n\t" "and.b32 biA, " E "A, 0x7FF;\n\t" "@pn mad.lo.u32 %0, fA, qA, biA;\n\t"         \
         "setp.lt.and.u32 " NP ", %0, 32768, pn;\n\t" "vote.sync.ballot.b32 " NB ", " NP ", 0xffffffff;\n\t"           \
+        "mov.u32 l" E ", %%clock;\n\t"                                                                                \
         "@" PP " mad.lo.u32 %0, %0, 65536, wA;\n\t" "shr.u32 q2, %0, 11;\n\t"
 #define EP_BODY11_GUESS(CVT)                                                                                          \
         "mov.b32 lm, 0xffffffff;\n\t" "mov.b32 sx, %0;\n\t" "mov.b32 sa, %1;\n\t" "mov.b32 sb, %2;\n\t"               \
@@ -944,6 +945,9 @@ __device__ __forceinline__ void decode_tile_plain(const JobParams &J, uint32_t t
         EP_G_RANK("%2", "nbA") EP_G_TAIL("e8", "ps")                                                                  \
         "mad.lo.u32 %1, tA, 2, %1;\n\t" "@pA ld.shared.u16 wA, [%1];\n\t" EP_G_TAIL_REST("e8", "ps")                  \
         EP_ALL(EP_PARX) EP_ALL(EP_X8) EP_PAIR_ALL EP_ALL(CVT, "3")
+#define EP_G_REGS ".reg .b32 ke1, ke2, ke3, ke4, ke5, ke6, ke7, ke8, le1, le2, le3, le4, le5, le6, le7, le8;\n\t"
+#define EP_G_KEEP2(A) "st.volatile.shared.u32 [" EP_CTX "+60], k" A ";\n\t" "st.volatile.shared.u32 [" EP_CTX "+60], l" A ";\n\t"
+#define EP_G_KEEP EP_G_KEEP2("e1") EP_G_KEEP2("e2") EP_G_KEEP2("e3") EP_G_KEEP2("e4") EP_G_KEEP2("e5") EP_G_KEEP2("e6") EP_G_KEEP2("e7") EP_G_KEEP2("e8")
 #define EP_GUESS_FIN "@pA mad.lo.u32 %0, %0, 65536, wA;\n\t"
 
 // per output type: CVT(S, j, lo, hi) turns weights 2j, 2j+1 into their stored form, STORE(S) writes the block
@@ -1157,10 +1161,10 @@ __device__ __forceinline__ void decode_tile_plain(const JobParams &J, uint32_t t
         EP_BODY11_SHORT(CVT) EP_SHORT_FIN                                                                             \
         EP_ALL(EP_ADDR) EP_ALL(STORE) EP_ALL(EP_ADVANCE, #GROUP_BYTES)
 #define EP_GUESS_NONE(CVT, STORE, GROUP_BYTES)
-#define EP_FEW_LOOP_ASM(BODY, FIN, GUESS, CVT, STORE, GROUP_BYTES)                                                    \
+#define EP_FEW_LOOP_ASM(BODY, FIN, GUESS, REGS, KEEP, CVT, STORE, GROUP_BYTES)                                        \
     asm volatile(                                                                                                     \
         "{\n\t"                                                                                                       \
-        EP_ALL(EP_REGS)                                                                                               \
+        EP_ALL(EP_REGS) REGS                                                                                          \
         ".reg .pred pq, pv, pr, ps, pn;\n\t"                                                                          \
         ".reg .b32 r0, r1, r2, r3, r4, r5, r6, r7, r10, r11, r12, c0r, c1r, f0c, lm, sx, sa, sb, ea, va, f2, b2, q2, rp, rowb, endo;\n\t"     \
         ".reg .b64 ra, rb;\n\t"                                                                                       \
@@ -1230,7 +1234,7 @@ __device__ __forceinline__ void decode_tile_plain(const JobParams &J, uint32_t t
         "cp.async.wait_all;\n\t"                                                                                      \
         "bar.warp.sync 0xffffffff;\n\t"                                                                               \
         "bra.uni EP_LOOP;\n\t"                                                                                        \
-        "EP_DONE:\n\t"                                                                                                \
+        "EP_DONE:\n\t" KEEP                                                                                           \
         "}"                                                                                                           \
         : "+&r"(x), "+&r"(a), "+&r"(bal), "+&r"(doff)                                                                 \
         : "r"(lt), "r"(lut_addr), "r"(lut_addr + kCosetStride), "r"(ctx), "l"(kk), "l"(out_base), "r"(cf.f0), "r"(cf.f1), \
@@ -1358,21 +1362,21 @@ __device__ __forceinline__ void decode_tile_few(const JobParams &J, uint32_t fir
     const uint32_t k0 = __float_as_uint(float(4096 - J.zlo)), lt = (1u << lane) - 1u;
     const uint64_t kk = pack64(k0, k0), out_base = reinterpret_cast<uint64_t>(J.out);
     if (J.guess) {
-        if constexpr (DT == EP_BF16) EP_FEW_LOOP_ASM(EP_BODY11_GUESS, EP_GUESS_FIN, EP_GUESS_CHECK, EP_CVT_BF16, EP_ST_16, 512);
-        else if constexpr (DT == EP_FP16) EP_FEW_LOOP_ASM(EP_BODY11_GUESS, EP_GUESS_FIN, EP_GUESS_CHECK, EP_CVT_FP16, EP_ST_16, 512);
-        else if constexpr (DT == EP_FP8_E4M3) EP_FEW_LOOP_ASM(EP_BODY11_GUESS, EP_GUESS_FIN, EP_GUESS_CHECK, EP_CVT_E4M3, EP_ST_F8, 256);
-        else if constexpr (DT == EP_FP8_E5M2) EP_FEW_LOOP_ASM(EP_BODY11_GUESS, EP_GUESS_FIN, EP_GUESS_CHECK, EP_CVT_E5M2, EP_ST_F8, 256);
-        else if constexpr (DT == EP_FP32) EP_FEW_LOOP_ASM(EP_BODY11_GUESS, EP_GUESS_FIN, EP_GUESS_CHECK, EP_CVT_FP32, EP_ST_FP32, 1024);
-        else if constexpr (DT == EP_UINT8) EP_FEW_LOOP_ASM(EP_BODY11_GUESS, EP_GUESS_FIN, EP_GUESS_CHECK, EP_CVT_I8, EP_ST_UINT8, 256);
-        else EP_FEW_LOOP_ASM(EP_BODY11_GUESS, EP_GUESS_FIN, EP_GUESS_CHECK, EP_CVT_I8, EP_ST_INT8, 256);
+        if constexpr (DT == EP_BF16) EP_FEW_LOOP_ASM(EP_BODY11_GUESS, EP_GUESS_FIN, EP_GUESS_CHECK, EP_G_REGS, EP_G_KEEP, EP_CVT_BF16, EP_ST_16, 512);
+        else if constexpr (DT == EP_FP16) EP_FEW_LOOP_ASM(EP_BODY11_GUESS, EP_GUESS_FIN, EP_GUESS_CHECK, EP_G_REGS, EP_G_KEEP, EP_CVT_FP16, EP_ST_16, 512);
+        else if constexpr (DT == EP_FP8_E4M3) EP_FEW_LOOP_ASM(EP_BODY11_GUESS, EP_GUESS_FIN, EP_GUESS_CHECK, EP_G_REGS, EP_G_KEEP, EP_CVT_E4M3, EP_ST_F8, 256);
+        else if constexpr (DT == EP_FP8_E5M2) EP_FEW_LOOP_ASM(EP_BODY11_GUESS, EP_GUESS_FIN, EP_GUESS_CHECK, EP_G_REGS, EP_G_KEEP, EP_CVT_E5M2, EP_ST_F8, 256);
+        else if constexpr (DT == EP_FP32) EP_FEW_LOOP_ASM(EP_BODY11_GUESS, EP_GUESS_FIN, EP_GUESS_CHECK, EP_G_REGS, EP_G_KEEP, EP_CVT_FP32, EP_ST_FP32, 1024);
+        else if constexpr (DT == EP_UINT8) EP_FEW_LOOP_ASM(EP_BODY11_GUESS, EP_GUESS_FIN, EP_GUESS_CHECK, EP_G_REGS, EP_G_KEEP, EP_CVT_I8, EP_ST_UINT8, 256);
+        else EP_FEW_LOOP_ASM(EP_BODY11_GUESS, EP_GUESS_FIN, EP_GUESS_CHECK, EP_G_REGS, EP_G_KEEP, EP_CVT_I8, EP_ST_INT8, 256);
     } else {
-        if constexpr (DT == EP_BF16) EP_FEW_LOOP_ASM(EP_BODY11_SHORT, EP_SHORT_FIN, EP_GUESS_NONE, EP_CVT_BF16, EP_ST_16, 512);
-        else if constexpr (DT == EP_FP16) EP_FEW_LOOP_ASM(EP_BODY11_SHORT, EP_SHORT_FIN, EP_GUESS_NONE, EP_CVT_FP16, EP_ST_16, 512);
-        else if constexpr (DT == EP_FP8_E4M3) EP_FEW_LOOP_ASM(EP_BODY11_SHORT, EP_SHORT_FIN, EP_GUESS_NONE, EP_CVT_E4M3, EP_ST_F8, 256);
-        else if constexpr (DT == EP_FP8_E5M2) EP_FEW_LOOP_ASM(EP_BODY11_SHORT, EP_SHORT_FIN, EP_GUESS_NONE, EP_CVT_E5M2, EP_ST_F8, 256);
-        else if constexpr (DT == EP_FP32) EP_FEW_LOOP_ASM(EP_BODY11_SHORT, EP_SHORT_FIN, EP_GUESS_NONE, EP_CVT_FP32, EP_ST_FP32, 1024);
-        else if constexpr (DT == EP_UINT8) EP_FEW_LOOP_ASM(EP_BODY11_SHORT, EP_SHORT_FIN, EP_GUESS_NONE, EP_CVT_I8, EP_ST_UINT8, 256);
-        else EP_FEW_LOOP_ASM(EP_BODY11_SHORT, EP_SHORT_FIN, EP_GUESS_NONE, EP_CVT_I8, EP_ST_INT8, 256);
+        if constexpr (DT == EP_BF16) EP_FEW_LOOP_ASM(EP_BODY11_SHORT, EP_SHORT_FIN, EP_GUESS_NONE, "", "", EP_CVT_BF16, EP_ST_16, 512);
+        else if constexpr (DT == EP_FP16) EP_FEW_LOOP_ASM(EP_BODY11_SHORT, EP_SHORT_FIN, EP_GUESS_NONE, "", "", EP_CVT_FP16, EP_ST_16, 512);
+        else if constexpr (DT == EP_FP8_E4M3) EP_FEW_LOOP_ASM(EP_BODY11_SHORT, EP_SHORT_FIN, EP_GUESS_NONE, "", "", EP_CVT_E4M3, EP_ST_F8, 256);
+        else if constexpr (DT == EP_FP8_E5M2) EP_FEW_LOOP_ASM(EP_BODY11_SHORT, EP_SHORT_FIN, EP_GUESS_NONE, "", "", EP_CVT_E5M2, EP_ST_F8, 256);
+        else if constexpr (DT == EP_FP32) EP_FEW_LOOP_ASM(EP_BODY11_SHORT, EP_SHORT_FIN, EP_GUESS_NONE, "", "", EP_CVT_FP32, EP_ST_FP32, 1024);
+        else if constexpr (DT == EP_UINT8) EP_FEW_LOOP_ASM(EP_BODY11_SHORT, EP_SHORT_FIN, EP_GUESS_NONE, "", "", EP_CVT_I8, EP_ST_UINT8, 256);
+        else EP_FEW_LOOP_ASM(EP_BODY11_SHORT, EP_SHORT_FIN, EP_GUESS_NONE, "", "", EP_CVT_I8, EP_ST_INT8, 256);
     }
     cp_async_wait<0>();           // nothing may still be landing in the stage when the next tile starts
     __syncwarp();
@@ -1388,7 +1392,7 @@ __device__ __forceinline__ void decode_tile_few(const JobParams &J, uint32_t fir
 // that steers this (loop bounds, job changes) depends on blockIdx and kernel parameters only, so the compiler
 // sees warp-uniform control flow and puts no divergence guards around the warp votes of the hot loop; in the last
 // round of a job a chain past the job's last tile goes through the same code with no block to decode.
-// FEW: launches of few tiles per CTA (see decode_tile_few); a kernel of its own because it may use 168 registers where 32 warps
+// FEW: launches of few tiles per CTA (see decode_tile_few); a kernel of its own because it may use 128 registers where 32 warps
 // leave 64.
 template <int DT, bool FEW>
 __global__ void __launch_bounds__(FEW ? 32 * (kFewTiles > kMinWarps ? kFewTiles : kMinWarps) : kThreads, 1)
@@ -2091,6 +2095,10 @@ uint32_t split_rounds(BatchParams &P, uint32_t sms) {
         J.round_cost = rounds_total <= sms ? 1u : (J.V + 31u) / 32u;
         J.cost_begin = uint32_t(cost);
         cost += uint64_t(J.rounds) * J.round_cost;
+        // The guess costs ten instructions per step and, at 4 bpp (3.5 bits per symbol), the repetition of one group in 70 (at
+        // 5 bpp one in 25, at 6 one in 6).  1792-block tiles, us, with / without: 2.5 bpp 4 tiles 32.7 / 36.8, 8: 37.0 / 38.4,
+        // 10: 43.1 / 41.1; 4 bpp 4 tiles 34.4 / 37.1, 8: 38.4 / 38.7; 4.5 bpp 4 tiles 34.9 / 37.1, 8: 39.7 / 38.7.
+        J.guess = (lo <= 4u && J.payload_bits <= 4.2f) || (lo <= 8u && J.payload_bits <= 3.6f);
     }
     const uint32_t grid = uint32_t(rounds_total < sms ? rounds_total : sms);
     // (a tensor has under 2^27 blocks, so sixteen of them cost under 2^26 groups: 32-bit arithmetic in the kernel)
@@ -2405,7 +2413,7 @@ extern "C" int ep_decode_batch(const ep_decode_job *jobs_in, int32_t n_in, void 
         J.row_bytes = J.per_row * block_bytes;
         J.row_rcp = uint32_t(0xFFFFFFFFu / J.row_bytes + 1u);
         J.row_max = I.R - 1u;
-        J.guess = double(I.total_words) * 16.0 <= kGuessBits * 9.0 * double(J.n_vec);
+        J.payload_bits = float(double(I.total_words) * 16.0 / (9.0 * double(J.n_vec)));
     }
     const uint32_t next = split_rounds(P, uint32_t(sms));      // grid size
     if (next == 0) return EP_ERR_UNSUPPORTED;
