@@ -452,66 +452,6 @@ __device__ __forceinline__ void decode_group_plain(uint32_t &x, uint32_t &wa, ui
     }
 }
 
-// ---- the same group with the hot loop's word addressing, for full groups of 2^11-slot streams -------------
-// Every lane keeps its own word address: the words taken in the previous step by this lane and the lanes above it
-// plus those taken in this step by the lanes below are one population count of a bit-select of the two ballots.
-// Used where the loop around the group is C++ (the kernel that feeds the tensor cores); BF16 block returned in `blk`.
-// renormalisation: lanes whose state fell below 2^15 take a word each, in lane order (the hot loop's seven instructions)
-__device__ __forceinline__ void lean_renorm(uint32_t &x, uint32_t &a, uint32_t &bal, uint32_t lt) {
-    asm volatile("{\n\t.reg .pred p;\n\t.reg .b32 now, t, w;\n\t"
-                 "setp.lt.u32 p, %0, 32768;\n\t"
-                 "vote.sync.ballot.b32 now, p, 0xffffffff;\n\t"
-                 "lop3.b32 t, %3, now, %2, 0xCA;\n\t"          // the lanes below: this step's ballot; this lane and above: the last one's
-                 "popc.b32 t, t;\n\t"
-                 "mad.lo.u32 %1, t, 2, %1;\n\t"
-                 "ld.shared.u16 w, [%1];\n\t"
-                 "@p mad.lo.u32 %0, %0, 65536, w;\n\t"
-                 "mov.b32 %2, now;\n\t}"
-                 : "+r"(x), "+r"(a), "+r"(bal) : "r"(lt) : "memory");
-}
-// one coordinate symbol (Eq. 18) from the table at shared-memory address `table`: returns the entry
-__device__ __forceinline__ uint32_t lean_step(uint32_t &x, uint32_t &a, uint32_t &bal, uint32_t table, uint32_t lt) {
-    uint32_t e;
-    asm volatile("{\n\t.reg .b32 q, u, f, bi;\n\t"
-                 "shr.u32 q, %0, 11;\n\t"
-                 "mad.lo.u32 u, q, 0xFFFFE000, %2;\n\t"        // slot address 4 (x & 2047) + table = 4 x - 8192 (x >> 11) + table
-                 "mad.lo.u32 u, %0, 4, u;\n\t"
-                 "ld.shared.u32 %1, [u];\n\t"
-                 "shr.u32 f, %1, 21;\n\t"
-                 "and.b32 bi, %1, 0x7FF;\n\t"
-                 "mad.lo.u32 %0, f, q, bi;\n\t}"
-                 : "+r"(x), "=r"(e) : "r"(table) : "memory");
-    lean_renorm(x, a, bal, lt);
-    return e;
-}
-__device__ __forceinline__ uint4 decode_group_lean_bf16(uint32_t &x, uint32_t &wa, uint32_t lut_addr, CosetFreq cf, uint32_t lt,
-                                                        uint32_t k0_bits, float sigma) {
-    uint32_t a = wa, bal = 0, e[9];
-    {   // the coset: slot below f0 -> 0, else 1
-        const uint32_t u = x & 2047u, q = x >> 11;
-        const bool c1 = u >= cf.f0;
-        x = (c1 ? cf.f1 : max(cf.f0, 1u)) * q + (c1 ? u - cf.f0 : u);
-        e[0] = c1 ? 1u : 0u;
-        lean_renorm(x, a, bal, lt);
-    }
-    const uint32_t tab = lut_addr + e[0] * kCosetStride;
-#pragma unroll
-    for (int k = 1; k <= 8; ++k) e[k] = lean_step(x, a, bal, tab + uint32_t(k - 1) * kLutStride, lt);
-    wa = __shfl_sync(0xFFFFFFFFu, a, 0) + 2u * __popc(bal);      // lane 0's address is the cursor before the last step
-    const uint32_t par = (e[1] ^ e[2] ^ e[3] ^ e[4] ^ e[5] ^ e[6] ^ e[7]) & 0x800u;
-    const uint32_t cc = kExp4096 | (e[0] << 10);
-    const uint64_t kk = pack64(k0_bits, k0_bits);
-    const uint64_t ss = pack64(__float_as_uint(sigma), __float_as_uint(sigma));
-    uint32_t xb[8];
-#pragma unroll
-    for (int k = 1; k <= 7; ++k) xb[k - 1] = (e[k] & kCodeMask) | cc;
-    xb[7] = (e[8] & kCodeMask) | par | cc;
-    float w[8];
-#pragma unroll
-    for (int i = 0; i < 8; i += 2) unpack64(mul2(sub2(pack64(xb[i], xb[i + 1]), kk), ss), w[i], w[i + 1]);
-    return make_uint4(pack_bf16(w[0], w[1]), pack_bf16(w[2], w[3]), pack_bf16(w[4], w[5]), pack_bf16(w[6], w[7]));
-}
-
 // ---- payload ring ------------------------------------------------------------------------------------
 // chunk c of a tile = global bytes [a0 + CHUNK c, a0 + CHUNK (c + 1)), a0 = tile's first word rounded down to
 // 16 bytes; it lives in ring slot c mod SLOTS, and a chunk in one of the slots that make up the ring's first 512
@@ -1465,24 +1405,26 @@ ep_decode_smem_kernel(const __grid_constant__ BatchParams P) {
 // straight into the shared-memory operand of a tcgen05 matrix instruction and never written to global memory.
 //
 // The stream must have one tile per row of W (V = C / 8) and C a multiple of 256.  The rows are spread evenly over
-// the SMs; a CTA takes its range 30 rows at a time, one row per warp: warps 0 .. 29 decode their rows group by group
-// (a group = 32 blocks = 256 columns), so after every group the CTA holds a 30 x 256 slab of W - the B operand
-// (N = 32 with two idle rows, K-major, 128-byte swizzle: a lane's 16-byte block is one piece of a swizzled row, so
-// the stores are conflict-free).  Warps 30 and 31 decode nothing.  One lane of warp 30 brings the matching 256
+// the SMs; a CTA takes its range in equal steps of at most 30 rows, one row per warp: warps 2 .. decode their rows group by
+// group (a group = 32 blocks = 256 columns), so after every group the CTA holds a 30 x 256 slab of W - the B operand
+// (N = 32 with unused rows zero, K-major, 128-byte swizzle: a lane's 16-byte block is one piece of a swizzled row, so
+// the stores are conflict-free).  Warps 0 and 1 decode nothing.  One lane of warp 0 brings the matching 256
 // columns of x in (A operand, M = 64 rows of which the first 16 or 32 are tokens; the others read whatever shared
 // memory follows and produce accumulator rows nobody stores) with four tensor copies (cp.async.bulk.tensor, the
-// copy engine swizzles).  One lane of warp 31 waits until x has landed and all rows of the slab are stored and
+// copy engine swizzles).  One lane of warp 1 waits until x has landed and all rows of the slab are stored and
 // issues the slab's sixteen K = 16 instructions.  (A decoding warp cannot do that on the side: whoever issues falls
 // behind by the time it takes, and with two slabs every warp is at most one group ahead of the slowest - measured
-// 138 us for the layer below; one warp for copies and instructions together 90 us, its single instruction stream
-// being the slowest in the CTA; two warps on two schedulers 84 us.)  The fp32 accumulator (64 lanes x 32 columns)
-// stays in tensor memory over the whole row and is read out once per step.
+// 138 us for the 10240 x 3840 layer; one warp for copies and instructions together 90 us, its single instruction stream
+// being the slowest in the CTA.)  The fp32 accumulator (64 lanes x 32 columns) stays in tensor memory over the whole row;
+// there are two, used in turn, and warps 0 and 1 - whose quarters of tensor memory hold the tokens - read one out while the
+// decoding warps are in the next step: nothing holds those up between steps.
+// 10240 x 3840, 16 tokens: steps of 30 + 30 + 10 rows, each ended by a CTA barrier around the read-out, the group in C++:
+// 74.3 us.
 //
-// Shared memory: the lookup tables (128 KB), 32 payload rings of 4 x 256 + 512 bytes (48 KB), then A (16 KB: two units
-// of x - a group's 256 columns of up to 16 tokens each, or half a group's of up to 32 -, refilled by the loading warp as
-// soon as the instructions that read a unit are done), B (two slabs of 16 KB: the warps decode the next group while the
-// tensor core reads the last one) and the mbarriers.  What bounds the token count: a group's columns of x must be in
-// flight while the group is decoded (about 1 us), every CTA re-reads x from L2, and 16 KB is the landing space left.
+// Shared memory: the lookup tables (128 KB), a payload ring of 4 x 256 + 512 bytes for each decoding warp, then A (units
+// of x, refilled by the loading warp as soon as the instructions that read them are done), B (two slabs: the warps decode
+// the next group while the tensor core reads the last one) and the mbarriers; see GemmShape.  What bounds the token count:
+// a group's columns of x must be in flight while the group is decoded (about 1 us), and every CTA re-reads x from L2.
 // Every wait on an mbarrier gives up after kSpinLimit polls, raises the abort word and lets the kernel run to its
 // end (wrong output, status flag set) instead of hanging.
 struct GemmParams {
@@ -1491,21 +1433,31 @@ struct GemmParams {
     float *y;                     // [T, R] fp32, row-major
     uint32_t T, Tpad;             // tokens; rows of x that are staged (16 or 32)
     uint32_t R, C;
-    uint32_t rows_per_cta;        // CTA k takes rows [k, k + 1) * rows_per_cta, 31 at a time
+    uint32_t rows_per_cta;        // CTA k takes rows [k, k + 1) * rows_per_cta,
+    uint32_t rows_per_step, steps;   // rows_per_step at a time
     uint32_t groups;              // C / 256
 };
 
 constexpr uint32_t kGemmChunk = 256, kGemmSlots = 4;     // payload ring of this kernel
 constexpr uint32_t kGemmRingStride = kGemmChunk * kGemmSlots + kRingMirror;   // 1536
-constexpr uint32_t kGemmA = kRingBase + 32u * kGemmRingStride;   // A operand: per stage four 64-column tiles of Tpad rows
-constexpr uint32_t kGemmB = kGemmA + 16384;              // B operand: two slabs of four 64-column tiles of 32 rows
-constexpr uint32_t kGemmBar = kGemmB + 32768;            // mbarriers, tensor-memory address, abort word, counter
-constexpr uint32_t kGemmSmem = kGemmBar + 256;
 constexpr uint32_t kSpinLimit = 1u << 18;             // attempts of about a microsecond each at most: a quarter of a second
-constexpr uint32_t kGemmRows = 30;                       // rows of W per step: warps 0 .. 29 decode one each, warp 30 brings x in, warp 31 issues the matrix instructions
-constexpr uint32_t kGemmIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((32u >> 3) << 17) | ((64u >> 4) << 24);   // f32 += bf16 x bf16, K-major both, N = 32, M = 64
-static_assert(kGemmA % 1024 == 0, "swizzled operand tiles start on 1024-byte boundaries");
-static_assert(kGemmSmem <= 232448, "more shared memory than an sm_100 CTA can have");
+// what depends on the number of tokens that are staged.  Up to 16: thirty rows of W per step, x in two units of a whole
+// group.  Up to 32 a group's columns of x fill 16 KB, and with no more than that a unit could be asked for only when the
+// instructions of the group before had read it (10240 x 3840, 32 tokens: 80.9 us): 24 rows per step make room for 32 KB,
+// four units of half a group each.
+template <uint32_t TPAD>
+struct GemmShape {
+    static constexpr uint32_t kRows = TPAD == 16 ? 30 : 24;              // most rows of W per step: one per decoding warp
+    static constexpr uint32_t kN = TPAD == 16 ? 32 : 24;                 // rows of the B operand
+    static constexpr uint32_t kUnits = TPAD == 16 ? 2 : 4;               // units of x, 8 KB each
+    static constexpr uint32_t kBTile = kN * 128, kSlab = 4 * kBTile;     // B: per slab four 64-column tiles of kN rows
+    static constexpr uint32_t kA = (kRingBase + kRows * kGemmRingStride + 1023u) & ~1023u;   // A operand (swizzled tiles start on 1024-byte boundaries)
+    static constexpr uint32_t kB = kA + kUnits * 8192;
+    static constexpr uint32_t kBar = kB + 2 * kSlab;                     // mbarriers, tensor-memory address, abort word
+    static constexpr uint32_t kSmem = kBar + 256;
+    static constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((kN >> 3) << 17) | ((64u >> 4) << 24);   // f32 += bf16 x bf16, K-major both, N = kN, M = 64
+    static_assert(kSmem <= 232448, "more shared memory than an sm_100 CTA can have");
+};
 
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
@@ -1553,6 +1505,28 @@ __device__ __forceinline__ void umma_commit(uint32_t bar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
 
+// one group of a row (EP_BODY11_SHORT, no store) with operands of its own: %0 .. %2 = x, a, bal, %3 .. %6 = the BF16 block
+#undef EP_LT
+#undef EP_LUT0
+#undef EP_LUT1
+#undef EP_KK
+#undef EP_F0
+#undef EP_F1
+#define EP_LT "%7"
+#define EP_LUT0 "%8"
+#define EP_LUT1 "%9"
+#define EP_KK "%10"
+#define EP_F0 "%11"
+#define EP_F1 "%12"
+#define EP_GEMM_GROUP_ASM                                                                                             \
+    asm volatile("{\n\t" EP_ALL(EP_REGS)                                                                              \
+                 ".reg .b32 c0r, c1r, f0c, va;\n\t" "mov.b32 c0r, 0x45800000;\n\t" "mov.b32 c1r, 0x45800400;\n\t"     \
+                 "max.u32 f0c, " EP_F0 ", 1;\n\t" "mov.b64 ssA, {%13, %13};\n\t" "setp.ne.u32 actA, %14, 0;\n\t"      \
+                 EP_BODY11_SHORT(EP_CVT_BF16) EP_SHORT_FIN                                                            \
+                 "mov.b32 %3, o0A;\n\t" "mov.b32 %4, o1A;\n\t" "mov.b32 %5, o2A;\n\t" "mov.b32 %6, o3A;\n\t}"         \
+                 : "+&r"(x), "+&r"(a), "+&r"(bal), "=&r"(blk.x), "=&r"(blk.y), "=&r"(blk.z), "=&r"(blk.w)             \
+                 : "r"(lt), "r"(lut_addr), "r"(lut_addr + kCosetStride), "l"(kk), "r"(cf.f0), "r"(cf.f1), "r"(sigma), "r"(act) : "memory")
+
 template <uint32_t TPAD>
 __global__ void __launch_bounds__(kThreads, 1) ep_decode_gemm_kernel(const __grid_constant__ GemmParams P,
                                                                      const __grid_constant__ CUtensorMap x_map) {
@@ -1560,35 +1534,35 @@ __global__ void __launch_bounds__(kThreads, 1) ep_decode_gemm_kernel(const __gri
     const JobParams &J = P.J;
     const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
     const uint32_t lut_addr = uint32_t(__cvta_generic_to_shared(smem));
-    const uint32_t ring = lut_addr + kRingBase + warp * kGemmRingStride;
-    const uint32_t a_base = lut_addr + kGemmA, b_base = lut_addr + kGemmB;
-    // A holds two units of x, a unit being half of what fits: four tiles of 64 columns x 16 rows (one group's columns), or
-    // two tiles x 32 rows (half a group's).  Per unit one mbarrier "landed" and one "read"; per slab of B one "rows stored"
-    // and one "read".
+    using G = GemmShape<TPAD>;
+    const uint32_t a_base = lut_addr + G::kA, b_base = lut_addr + G::kB;
+    // A holds two or four units of x: four tiles of 64 columns x 16 rows each (one group's columns), or two tiles x 32 rows
+    // (half a group's).  Per unit one mbarrier "landed" and one "read"; per slab of B one "rows stored" and one "read".
     constexpr uint32_t a_tile_bytes = TPAD * 128u, kUnitTiles = 8192u / a_tile_bytes, kUnitsPerGroup = 4u / kUnitTiles;
-    const uint32_t bar_a = lut_addr + kGemmBar, bar_afree = bar_a + 64u, bar_mma = bar_a + 128u, bar_b = bar_a + 144u,
+    const uint32_t bar_a = lut_addr + G::kBar, bar_afree = bar_a + 64u, bar_mma = bar_a + 128u, bar_b = bar_a + 144u,
                    slot = bar_a + 160u, abort_addr = bar_a + 164u;
     if (tid == 0) {
-        for (uint32_t i = 0; i < 2u; ++i) {
+        for (uint32_t i = 0; i < G::kUnits; ++i) {
             mbar_init(bar_a + 8u * i, 1u);       // the loading lane's arrival; completes when the unit's tiles have landed
             mbar_init(bar_afree + 8u * i, 1u);   // the commit after the matrix instructions that read the unit
         }
-        mbar_init(bar_mma, 1u);              // the commit after a group's matrix instructions
-        mbar_init(bar_mma + 8u, 1u);
-        mbar_init(bar_b, kGemmRows);         // every decoding warp, when its row of the slab is stored
-        mbar_init(bar_b + 8u, kGemmRows);
+        for (uint32_t i = 0; i < 2u; ++i) {
+            mbar_init(bar_mma + 8u * i, 1u);     // the commit after a group's matrix instructions
+            mbar_init(bar_b + 8u * i, P.rows_per_step);   // every decoding warp, when its row of the slab is stored
+        }
         sts32(abort_addr, (lut_addr & 1023u) ? 1u : 0u);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (warp == 0) {                         // 32 columns of tensor memory: the 64 x 32 fp32 accumulator
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(slot), "r"(32u) : "memory");
+    if (warp == 0) {                         // 64 columns of tensor memory: two 64 x 32 fp32 accumulators
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(slot), "r"(64u) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
-    if (warp >= kGemmRows) {                 // rows 30 and 31 of both slabs belong to no warp: zero (this warp's row, all its pieces)
-        for (uint32_t i = lane; i < 2u * 4u * 8u; i += 32u)
-            asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};" ::"r"(b_base + (i >> 5) * 16384u + ((i >> 3) & 3u) * 4096u + warp * 128u + (i & 7u) * 16u), "r"(0u) : "memory");
-        fence_async_smem();
+    // rows of the slabs that belong to no warp: zero
+    for (uint32_t i = tid; i < 2u * 4u * (G::kN - P.rows_per_step) * 8u; i += blockDim.x) {
+        const uint32_t piece = i & 7u, tile = (i >> 3) & 7u, row = P.rows_per_step + (i >> 6);
+        asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};" ::"r"(b_base + tile * G::kBTile + row * 128u + piece * 16u), "r"(0u) : "memory");
     }
+    wait_for_stream();
     copy_tables_smem(J.lut_image, lut_addr, false);
     const CosetFreq cf = load_coset(J);
     cp_async_wait<0>();
@@ -1598,35 +1572,54 @@ __global__ void __launch_bounds__(kThreads, 1) ep_decode_gemm_kernel(const __gri
     const uint32_t tmem = lds32(slot);
 
     const uint32_t row_begin = min(blockIdx.x * P.rows_per_cta, P.R), row_end = min(row_begin + P.rows_per_cta, P.R);
-    const uint32_t steps = (row_end - row_begin + kGemmRows - 1u) / kGemmRows;
-    const uint32_t q_total = steps * P.groups;               // groups this CTA hands to the tensor core
-    // usually the phase is long complete: one test by the whole warp; otherwise one lane polls and the warp follows
-    auto wait_warp = [&](uint32_t bar, uint32_t parity) {
-        if (mbar_test(bar, parity)) return;
-        if (lane == 0) mbar_wait(bar, parity, abort_addr);
+    // the accumulator of step s (tokens 16 quarter ..) to y: with M = 64, token 16 w + l is lane l < 16 of warp w's quarter;
+    // columns = rows of W
+    auto read_out = [&](uint32_t s, uint32_t quarter) {
+        tc_fence_after();
+        uint32_t v[32];
+        asm volatile("tcgen05.ld.sync.aligned.32x32b.x32.b32 "
+                     "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, %17, %18, %19, %20, %21, %22, "
+                     "%23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
+                     : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]), "=r"(v[8]),
+                       "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]), "=r"(v[16]),
+                       "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]), "=r"(v[24]),
+                       "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
+                     : "r"(tmem + ((quarter * 32u) << 16) + 32u * (s & 1u)));
+        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+        tc_fence_before();
+        const uint32_t t = quarter * 16u + lane, r0 = row_begin + s * P.rows_per_step;
+        if (lane < 16u && t < P.T && r0 < row_end) {
+            float *dst = P.y + size_t(t) * P.R + r0;
+            const uint32_t n = min(P.rows_per_step, row_end - r0);
+#pragma unroll
+            for (uint32_t i = 0; i < G::kRows; ++i)
+                if (i < n) dst[i] = __uint_as_float(v[i]);
+        }
         __syncwarp();
     };
     bool bad = false;
-    // the end of a step (accumulator read out, next rows may overwrite it) concerns the decoding warps and the issuing
-    // warp; the loading warp runs ahead of them across steps
-    auto step_sync = [&]() {
-        tc_fence_before();
-        asm volatile("bar.sync 1, %0;" ::"n"(kThreads - 32) : "memory");
-        tc_fence_after();
-    };
+    // unit j of x lies in buffer j mod 2^depth.  (Rows of one group have two half-group units per step: with four buffers the
+    // loading warp would be a step too far ahead of the read-out.)
+    const uint32_t depth = G::kUnits == 4u && P.groups > 1u ? 2u : 1u, units_mask = (1u << depth) - 1u;
 
-    if (warp == kGemmRows) {
-        // ---- the loading warp: one lane brings x into A, unit after unit, nothing else ----
+    if (warp == 0) {
+        // ---- the loading warp: one lane brings x into A, unit after unit; between two units the warp reads out accumulators ----
         // tile i of the CTA's sequence = columns [64 i, 64 i + 64) of x, counted over all groups (and again from column 0 for
         // every step); the copy engine lays it out and swizzles it; rows past the last token lie outside the tensor and
-        // arrive as zeros
-        if (lane == 0) {
-            const uint32_t tiles_per_step = 4u * P.groups;
-            for (uint32_t j = 0; j < kUnitsPerGroup * q_total; ++j) {
-                const uint32_t buf = j & 1u;
-                // (after a wait that ran out nothing is copied any more: re-arming a barrier whose phase never completed
-                // would overflow its transaction count)
-                if (j >= 2u && !mbar_wait(bar_afree + 8u * buf, ((j >> 1) - 1u) & 1u, abort_addr)) break;
+        // arrive as zeros.  A unit may overwrite the one before it in its buffer when that has been read; where that was a
+        // step's last, the step's accumulator is then complete, and it is read out before any unit is loaded that the next
+        // user of this accumulator waits for.
+        const uint32_t tiles_per_step = 4u * P.groups, units = kUnitsPerGroup * P.groups, total = units * P.steps;
+        for (uint32_t j = 0; j < total + units_mask + 1u; ++j) {
+            const uint32_t buf = j & units_mask;
+            uint32_t go = 1u;
+            // (after a wait that ran out nothing is copied any more: re-arming a barrier whose phase never completed
+            // would overflow its transaction count)
+            if (lane == 0 && j > units_mask) go = mbar_wait(bar_afree + 8u * buf, ((j >> depth) - 1u) & 1u, abort_addr);
+            go = __shfl_sync(0xFFFFFFFFu, go, 0);
+            if (!go) break;
+            if (j > units_mask && (j - units_mask) % units == 0u) read_out((j - units_mask) / units - 1u, 0u);
+            if (lane == 0 && j < total) {
                 asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar_a + 8u * buf), "r"(8192u) : "memory");
 #pragma unroll
                 for (uint32_t t = 0; t < kUnitTiles; ++t)
@@ -1635,115 +1628,104 @@ __global__ void __launch_bounds__(kThreads, 1) ep_decode_gemm_kernel(const __gri
                                    "r"(((j * kUnitTiles + t) % tiles_per_step) * 64u), "r"(0u), "r"(bar_a + 8u * buf)
                                  : "memory");
             }
-        }
-        __syncwarp();
-    } else if (warp == kGemmRows + 1u) {
-        // ---- the issuing warp: one lane waits for a group's rows and, unit by unit, for x, and issues the matrix instructions ----
-        for (uint32_t q = 0; q < q_total; ++q) {
-            const uint32_t g = q % P.groups;
-            if (lane == 0) {
-                bool ready = mbar_wait(bar_b + 8u * (q & 1u), (q >> 1) & 1u, abort_addr);
-                // descriptors differ in their address field only: low word + (bytes >> 4)
-                const uint64_t da = umma_desc(a_base), db = umma_desc(b_base + 16384u * (q & 1u));
-                const uint32_t da_hi = uint32_t(da >> 32), db_hi = uint32_t(db >> 32), da_lo = uint32_t(da), db_lo = uint32_t(db);
-#pragma unroll
-                for (uint32_t h = 0; h < kUnitsPerGroup; ++h) {
-                    const uint32_t j = kUnitsPerGroup * q + h, buf = j & 1u;
-                    ready = ready && mbar_wait(bar_a + 8u * buf, (j >> 1) & 1u, abort_addr);
-                    tc_fence_after();
-#pragma unroll
-                    for (uint32_t t = 0; t < kUnitTiles; ++t)
-#pragma unroll
-                        for (uint32_t k = 0; k < 4; ++k)             // 16 columns = 32 bytes further along the swizzled rows
-                            if (ready)                               // (operands that never arrived are not multiplied)
-                                umma_bf16(tmem, pack64(da_lo + ((buf * 8192u + t * a_tile_bytes + 32u * k) >> 4), da_hi),
-                                          pack64(db_lo + (((h * kUnitTiles + t) * 4096u + 32u * k) >> 4), db_hi), kGemmIdesc,
-                                          (g | h | t | k) ? 1u : 0u);
-                    umma_commit(bar_afree + 8u * buf);
-                }
-                umma_commit(bar_mma + 8u * (q & 1u));
-            }
             __syncwarp();
-            if (g + 1u == P.groups) step_sync();
         }
-    } else {
-        // ---- the decoding warps: one row of W each, group by group into the slabs of B ----
-        const uint32_t lt = (1u << lane) - 1u;
-        const uint32_t k0_bits = __float_as_uint(float(4096 - J.zlo));
-        // where this lane's block of a group goes in a slab: 64-column tile lane / 8, row = warp, piece lane % 8 of the row
-        const uint32_t b_dst = b_base + (lane >> 3) * 4096u + warp * 128u + (((lane & 7u) ^ (warp & 7u)) << 4);
+    } else if (warp == 1) {
+        // ---- the issuing warp: one lane waits for a group's rows and, unit by unit, for x, and issues the matrix instructions ----
         uint32_t q = 0;
-        for (uint32_t r0 = row_begin; r0 < row_end; r0 += kGemmRows) {
-            const bool active = r0 + warp < row_end;                    // the last rows of the CTA's range may be fewer than 31
-            const uint32_t tile = min(r0 + warp, P.R - 1u);             // = the row of W
-            const TileSetup Tl = tile_setup(J, tile, active, lane);
-            uint32_t x = Tl.x, pos = Tl.lead, threshold = kGemmChunk;
-            if (active) {
-                for (uint32_t c = 0; c < kGemmSlots; ++c) ring_issue<kGemmChunk, kGemmSlots>(ring, Tl.a0, Tl.room, c, lane);
-                cp_async_wait<1>();
+        for (uint32_t s = 0; s < P.steps; ++s) {
+            const uint32_t acc = tmem + 32u * (s & 1u);
+            for (uint32_t g = 0; g < P.groups; ++g, ++q) {
+                if (lane == 0) {
+                    bool ready = mbar_wait(bar_b + 8u * (q & 1u), (q >> 1) & 1u, abort_addr);
+                    fence_async_smem();      // the rows' stores, ordered before this by the mbarrier, are read through the async proxy
+                    // descriptors differ in their address field only: low word + (bytes >> 4)
+                    const uint64_t da = umma_desc(a_base), db = umma_desc(b_base + G::kSlab * (q & 1u));
+                    const uint32_t da_hi = uint32_t(da >> 32), db_hi = uint32_t(db >> 32), da_lo = uint32_t(da), db_lo = uint32_t(db);
+#pragma unroll
+                    for (uint32_t h = 0; h < kUnitsPerGroup; ++h) {
+                        const uint32_t j = kUnitsPerGroup * q + h, buf = j & units_mask;
+                        ready = ready && mbar_wait(bar_a + 8u * buf, (j >> depth) & 1u, abort_addr);
+                        tc_fence_after();
+#pragma unroll
+                        for (uint32_t t = 0; t < kUnitTiles; ++t)
+#pragma unroll
+                            for (uint32_t k = 0; k < 4; ++k)             // 16 columns = 32 bytes further along the swizzled rows
+                                if (ready)                               // (operands that never arrived are not multiplied)
+                                    umma_bf16(acc, pack64(da_lo + ((buf * 8192u + t * a_tile_bytes + 32u * k) >> 4), da_hi),
+                                              pack64(db_lo + (((h * kUnitTiles + t) * G::kBTile + 32u * k) >> 4), db_hi), G::kIdesc,
+                                              (g | h | t | k) ? 1u : 0u);
+                        umma_commit(bar_afree + 8u * buf);
+                    }
+                    umma_commit(bar_mma + 8u * (q & 1u));
+                }
                 __syncwarp();
             }
-            const float sigma = __ldg(J.scales + tile);
+            if (TPAD > 16u) {                // tokens 16 .. are in this warp's quarter
+                if (lane == 0) mbar_wait(bar_mma + 8u * ((q - 1u) & 1u), ((q - 1u) >> 1) & 1u, abort_addr);
+                __syncwarp();
+                read_out(s, 1u);
+            }
+        }
+    } else if (warp < 2u + P.rows_per_step) {
+        // ---- the decoding warps: one row of W each, group by group into the slabs of B ----
+        const uint32_t w = warp - 2u, lt = (1u << lane) - 1u, ring = lut_addr + kRingBase + w * kGemmRingStride;
+        const uint32_t k0 = __float_as_uint(float(4096 - J.zlo));
+        const uint64_t kk = pack64(k0, k0);
+        // where this lane's block of a group goes in a slab: 64-column tile lane / 8, row = w, piece lane % 8 of the row
+        const uint32_t b_dst = b_base + (lane >> 3) * G::kBTile + w * 128u + (((lane & 7u) ^ (w & 7u)) << 4);
+        uint32_t q = 0;
+        for (uint32_t s = 0; s < P.steps; ++s) {
+            const uint32_t r = row_begin + s * P.rows_per_step + w, act = r < row_end ? 1u : 0u;   // a CTA's last step may be short
+            const uint32_t tile = min(r, P.R - 1u);                     // = the row of W
+            const TileSetup Tl = tile_setup(J, tile, true, lane);
+            for (uint32_t c = 0; c < kGemmSlots; ++c) ring_issue<kGemmChunk, kGemmSlots>(ring, Tl.a0, Tl.room, c, lane);
+            const uint32_t sigma = __float_as_uint(__ldg(J.scales + tile));
             // the row this warp takes in the next step: its record is asked for now and, a few groups on, the start of
             // its payload is brought into L2, so that the next step does not begin with two reads from DRAM in a row
-            const bool has_next = r0 + kGemmRows + warp < row_end;
-            const uint32_t *rec_next = J.tile_index + size_t(min(tile + kGemmRows, P.R - 1u)) * 33u;
-            uint32_t off_next = 0;
-            if (has_next) off_next = __ldg(rec_next + 32);
+            const bool has_next = r + P.rows_per_step < row_end;
+            const uint32_t *rec_next = J.tile_index + size_t(min(r + P.rows_per_step, P.R - 1u)) * 33u;
+            const uint32_t off_next = __ldg(rec_next + 32);
             if (has_next && lane == 0) prefetch_l2(rec_next);
+            cp_async_wait<1>();
+            __syncwarp();
+            uint32_t x = Tl.x, bal = 0, a = ring + Tl.lead, wbase = ring, threshold = kGemmChunk, wthr = ring + kGemmChunk - 2u;
             for (uint32_t g = 0; g < P.groups; ++g, ++q) {
                 if (g == 2u && has_next) {
                     const uint64_t at = 2ull * min(off_next, J.total_words) + 128u * lane;      // 4 KB: the ring's first fill and more
                     if (at < 2ull * J.total_words) prefetch_l2(J.stream + J.off_payload + at);
                 }
-                uint4 blk = make_uint4(0u, 0u, 0u, 0u);
-                if (active) {
-                    if (pos >= threshold) ring_service<kGemmChunk, kGemmSlots>(ring, Tl.a0, Tl.room, pos, threshold, lane);
-                    const uint32_t wa0 = ring + pos % (kGemmChunk * kGemmSlots);
-                    uint32_t wa = wa0;
-                    blk = decode_group_lean_bf16(x, wa, lut_addr, cf, lt, k0_bits, sigma);
-                    pos += wa - wa0;
+                // is the slab free: is the tensor core done with the group that used it last, two groups ago?
+                const bool is_free = q < 2u || mbar_test(bar_mma + 8u * (q & 1u), ((q >> 1) - 1u) & 1u);
+                if (__any_sync(0xFFFFFFFFu, a >= wthr)) {               // the cursor left its chunk, or is about to
+                    const uint32_t pos = __shfl_sync(0xFFFFFFFFu, a, 0) + 2u * __popc(bal) - wbase;
+                    if (pos >= threshold) {
+                        ring_service<kGemmChunk, kGemmSlots>(ring, Tl.a0, Tl.room, pos, threshold, lane);
+                        if (pos + wbase - ring >= kGemmChunk * kGemmSlots) { a -= kGemmChunk * kGemmSlots; wbase -= kGemmChunk * kGemmSlots; }
+                        wthr = wbase + threshold - 2u;
+                    }
                 }
-                // the slab is free: the tensor core is done with the group that used it last, two groups ago
-                if (q >= 2u) wait_warp(bar_mma + 8u * (q & 1u), ((q >> 1) - 1u) & 1u);
-                asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(b_dst + 16384u * (q & 1u)), "r"(blk.x), "r"(blk.y), "r"(blk.z), "r"(blk.w) : "memory");
-                fence_async_smem();          // the stores above are read through the async proxy
+                uint4 blk;
+                EP_GEMM_GROUP_ASM;
+                if (!act) blk = make_uint4(0u, 0u, 0u, 0u);
+                if (!is_free) {
+                    if (lane == 0) mbar_wait(bar_mma + 8u * (q & 1u), ((q >> 1) - 1u) & 1u, abort_addr);
+                    __syncwarp();
+                }
+                asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(b_dst + G::kSlab * (q & 1u)), "r"(blk.x), "r"(blk.y), "r"(blk.z), "r"(blk.w) : "memory");
                 __syncwarp();
                 if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar_b + 8u * (q & 1u)) : "memory");
             }
-            // the accumulator of these rows: with M = 64, token 16 w + l is lane l < 16 of warp w's quarter; columns = rows of W
-            wait_warp(bar_mma + 8u * ((q - 1u) & 1u), ((q - 1u) >> 1) & 1u);
-            tc_fence_after();
-            if (warp < 2u) {
-                uint32_t v[32];
-                asm volatile("tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-                             "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, %17, %18, %19, %20, %21, %22, "
-                             "%23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-                             : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]), "=r"(v[8]),
-                               "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]), "=r"(v[16]),
-                               "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]), "=r"(v[24]),
-                               "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
-                             : "r"(tmem + ((warp * 32u) << 16)));
-                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-                const uint32_t t = warp * 16u + lane;
-                if (lane < 16u && t < P.T) {
-                    float *dst = P.y + size_t(t) * P.R + r0;
-                    const uint32_t n = min(kGemmRows, row_end - r0);
-#pragma unroll
-                    for (uint32_t i = 0; i < kGemmRows; ++i)
-                        if (i < n) dst[i] = __uint_as_float(v[i]);
-                }
-            }
             cp_async_wait<0>();              // nothing may still be landing in the ring when the next row starts
-            step_sync();                     // the accumulator has been read before the next rows overwrite it
-            bad |= active && ((x != ep::kStateLow) || (Tl.off + ((pos - Tl.lead) >> 1) != Tl.end));
+            const uint32_t pos = __shfl_sync(0xFFFFFFFFu, a, 0) + 2u * __popc(bal) - wbase;
+            bad |= act && ((x != ep::kStateLow) || (Tl.off + ((pos - Tl.lead) >> 1) != Tl.end));
         }
     }
     const bool aborted = lds32(abort_addr) != 0;
     if (__any_sync(0xFFFFFFFFu, bad) && lane == 0) atomicOr(&g_ep_status, 1u);
     if (aborted && tid == 0) atomicOr(&g_ep_status, 2u);
     __syncthreads();
-    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(32u) : "memory");
+    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(64u) : "memory");
 }
 
 // ======================================================================================================
@@ -2515,17 +2497,20 @@ extern "C" int ep_decode_gemm(const ep_info *info, const void *d_stream, const v
     P.Tpad = T <= 16 ? 16u : 32u;
     P.R = I.R;
     P.C = I.C;
-    // rows spread evenly over the SMs (a CTA takes its range 31 rows at a time; the last, shorter step runs with fewer
-    // warps and ends sooner than a full one)
+    // rows spread evenly over the SMs, and a CTA's rows over the fewest steps (thirty warps share an SM's issue slots: three
+    // steps of 24 rows take less time than 30 + 30 + 10)
     P.rows_per_cta = (I.R + uint32_t(sms) - 1u) / uint32_t(sms);
+    const uint32_t most = P.Tpad == 16u ? GemmShape<16>::kRows : GemmShape<32>::kRows;
+    P.steps = (P.rows_per_cta + most - 1u) / most;
+    P.rows_per_step = (P.rows_per_cta + P.steps - 1u) / P.steps;
     P.groups = I.C / 256u;
     if (I.n_tiles != I.R) return EP_ERR_BAD_ARG;
     static bool configured[64] = {};
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return EP_ERR_CUDA;
     if (dev < 0 || dev >= 64 || !configured[dev]) {
-        if (cudaFuncSetAttribute(ep_decode_gemm_kernel<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kGemmSmem)) != cudaSuccess ||
-            cudaFuncSetAttribute(ep_decode_gemm_kernel<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kGemmSmem)) != cudaSuccess)
+        if (cudaFuncSetAttribute(ep_decode_gemm_kernel<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(GemmShape<16>::kSmem)) != cudaSuccess ||
+            cudaFuncSetAttribute(ep_decode_gemm_kernel<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(GemmShape<32>::kSmem)) != cudaSuccess)
             return EP_ERR_CUDA;
         if (dev >= 0 && dev < 64) configured[dev] = true;
     }
@@ -2547,9 +2532,10 @@ extern "C" int ep_decode_gemm(const ep_info *info, const void *d_stream, const v
                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE,
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
         return EP_ERR_CUDA;
-    if (P.Tpad == 16u) ep_decode_gemm_kernel<16><<<grid, kThreads, kGemmSmem, st>>>(P, x_map);
-    else ep_decode_gemm_kernel<32><<<grid, kThreads, kGemmSmem, st>>>(P, x_map);
-    return cudaGetLastError() == cudaSuccess ? EP_OK : EP_ERR_CUDA;
+    const uint32_t threads = 32u * (2u + P.rows_per_step < kMinWarps ? kMinWarps : 2u + P.rows_per_step);
+    const cudaError_t e = P.Tpad == 16u ? launch_next(ep_decode_gemm_kernel<16>, grid, threads, GemmShape<16>::kSmem, st, P, x_map)
+                                        : launch_next(ep_decode_gemm_kernel<32>, grid, threads, GemmShape<32>::kSmem, st, P, x_map);
+    return e == cudaSuccess ? EP_OK : EP_ERR_CUDA;
 }
 
 extern "C" int ep_last_device_status(void *stream) {
