@@ -1407,7 +1407,7 @@ ep_decode_smem_kernel(const __grid_constant__ BatchParams P) {
 // The stream must have one tile per row of W (V = C / 8) and C a multiple of 256.  The rows are spread evenly over
 // the SMs; a CTA takes its range in equal steps of at most 30 rows, one row per warp: warps 2 .. decode their rows group by
 // group (a group = 32 blocks = 256 columns), so after every group the CTA holds a 30 x 256 slab of W - the B operand
-// (N = 32 with unused rows zero, K-major, 128-byte swizzle: a lane's 16-byte block is one piece of a swizzled row, so
+// (N = 32, K-major, 128-byte swizzle: a lane's 16-byte block is one piece of a swizzled row, so
 // the stores are conflict-free).  Warps 0 and 1 decode nothing.  One lane of warp 0 brings the matching 256
 // columns of x in (A operand, M = 64 rows of which the first 16 or 32 are tokens; the others read whatever shared
 // memory follows and produce accumulator rows nobody stores) with four tensor copies (cp.async.bulk.tensor, the
@@ -1505,34 +1505,111 @@ __device__ __forceinline__ void umma_commit(uint32_t bar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
 
-// one group of a row (EP_BODY11_SHORT, no store) with operands of its own: %0 .. %2 = x, a, bal, %3 .. %6 = the BF16 block
+// A row's groups (EP_BODY11_SHORT) with operands of its own: %0 .. %3 = x, a, bal and the group counter q, which goes on from
+// row to row.  In C++ around a group's asm this took 324 instructions per group, 80 of them guards around the votes and 40
+// for the ring; thirty warps are bound by just that number.
+// Per group: is the slab free, i.e. is the tensor core done with the group two before (tested ahead of the decode; a fresh
+// barrier passes for parity 1)?  Decode, wait if need be (kSpinLimit tries, or until the abort word is set), store the
+// block, arrive; then the ring (EP_SERVICE's steps for 4 chunks of 256 bytes; a group may leave two of them).
 #undef EP_LT
 #undef EP_LUT0
 #undef EP_LUT1
+#undef EP_CTX
 #undef EP_KK
 #undef EP_F0
 #undef EP_F1
-#define EP_LT "%7"
-#define EP_LUT0 "%8"
-#define EP_LUT1 "%9"
-#define EP_KK "%10"
-#define EP_F0 "%11"
-#define EP_F1 "%12"
-#define EP_GEMM_GROUP_ASM                                                                                             \
+#define EP_LT "%4"
+#define EP_LUT0 "%5"
+#define EP_LUT1 "%6"
+#define EP_CTX "%7"
+#define EP_KK "%8"
+#define EP_F0 "%9"
+#define EP_F1 "%10"
+#define EP_GEMM_ROW_ASM                                                                                               \
     asm volatile("{\n\t" EP_ALL(EP_REGS)                                                                              \
-                 ".reg .b32 c0r, c1r, f0c, va;\n\t" "mov.b32 c0r, 0x45800000;\n\t" "mov.b32 c1r, 0x45800400;\n\t"     \
-                 "max.u32 f0c, " EP_F0 ", 1;\n\t" "mov.b64 ssA, {%13, %13};\n\t" "setp.ne.u32 actA, %14, 0;\n\t"      \
-                 EP_BODY11_SHORT(EP_CVT_BF16) EP_SHORT_FIN                                                            \
-                 "mov.b32 %3, o0A;\n\t" "mov.b32 %4, o1A;\n\t" "mov.b32 %5, o2A;\n\t" "mov.b32 %6, o3A;\n\t}"         \
-                 : "+&r"(x), "+&r"(a), "+&r"(bal), "=&r"(blk.x), "=&r"(blk.y), "=&r"(blk.z), "=&r"(blk.w)             \
-                 : "r"(lt), "r"(lut_addr), "r"(lut_addr + kCosetStride), "l"(kk), "r"(cf.f0), "r"(cf.f1), "r"(sigma), "r"(act) : "memory")
+        ".reg .pred pq, pv, pr, pl;\n\t"                                                                              \
+        ".reg .b32 r0, r1, r2, r3, r4, r5, r6, r10, r11, r12, c0r, c1r, f0c, va, g, bar, par, odd, dst, tries;\n\t"   \
+        ".reg .b64 ra, rb, st;\n\t"                                                                                   \
+        "mov.b32 c0r, 0x45800000;\n\t" "mov.b32 c1r, 0x45800400;\n\t" "max.u32 f0c, " EP_F0 ", 1;\n\t"                \
+        "mov.b64 ssA, {%11, %11};\n\t" "setp.ne.u32 actA, %12, 0;\n\t" "mov.b32 g, %13;\n\t"                          \
+        "setp.eq.u32 pl, " EP_LT ", 0;\n\t"                  /* lane 0 */                                             \
+        "ld.shared.u32 r10, [" EP_CTX "+48];\n\t" "add.u32 wthrA, r10, 254;\n\t"                                      \
+        "EP_LOOP:\n\t"                                                                                                \
+        "and.b32 odd, %3, 1;\n\t" "mad.lo.u32 bar, odd, 8, %15;\n\t" "mad.lo.u32 dst, odd, %17, %14;\n\t"             \
+        "shr.u32 par, %3, 1;\n\t" "and.b32 par, par, 1;\n\t" "xor.b32 par, par, 1;\n\t"                               \
+        "mbarrier.test_wait.parity.shared::cta.b64 pv, [bar], par;\n\t"                                               \
+        EP_BODY11_SHORT(EP_CVT_BF16)                                                                                  \
+        "vote.sync.all.pred pv, pv, 0xffffffff;\n\t"                                                                  \
+        "@pv bra.uni EP_FREE;\n\t"                                                                                    \
+        "mov.b32 tries, %18;\n\t"                                                                                     \
+        "EP_WAIT:\n\t"                                                                                                \
+        "mbarrier.try_wait.parity.shared::cta.b64 pv, [bar], par, 1000;\n\t"                                          \
+        "vote.sync.any.pred pv, pv, 0xffffffff;\n\t"                                                                  \
+        "@pv bra.uni EP_FREE;\n\t"                                                                                    \
+        "ld.volatile.shared.u32 r0, [%16+100];\n\t" "setp.ne.u32 pv, r0, 0;\n\t"          /* the abort word */        \
+        "vote.sync.any.pred pv, pv, 0xffffffff;\n\t"                                                                  \
+        "@pv bra.uni EP_FREE;\n\t"                                                                                    \
+        "sub.u32 tries, tries, 1;\n\t" "setp.ne.u32 pv, tries, 0;\n\t"                                                \
+        "vote.sync.any.pred pv, pv, 0xffffffff;\n\t"                                                                  \
+        "@pv bra.uni EP_WAIT;\n\t"                                                                                    \
+        "mov.b32 r0, 1;\n\t" "st.volatile.shared.u32 [%16+100], r0;\n\t"                                              \
+        "EP_FREE:\n\t"                                                                                                \
+        "st.shared.v4.b32 [dst], {o0A, o1A, o2A, o3A};\n\t"                                                           \
+        "bar.warp.sync 0xffffffff;\n\t"                                                                               \
+        "mad.lo.u32 bar, odd, 8, %16;\n\t"                                                                            \
+        "@pl mbarrier.arrive.shared::cta.b64 st, [bar];\n\t"                                                          \
+        "add.u32 %3, %3, 1;\n\t" "sub.u32 g, g, 1;\n\t"                                                               \
+        "setp.lt.u32 pq, %1, wthrA;\n\t" "setp.ne.and.u32 pq, g, 0, pq;\n\t"                                          \
+        "vote.sync.all.pred pq, pq, 0xffffffff;\n\t"                                                                  \
+        EP_SHORT_FIN                                                                                                  \
+        "@pq bra.uni EP_LOOP;\n\t"                                                                                    \
+        "setp.eq.u32 pr, g, 0;\n\t"                                                                                   \
+        "vote.sync.any.pred pr, pr, 0xffffffff;\n\t"                                                                  \
+        "@pr bra.uni EP_DONE;\n\t"                                                                                    \
+        "EP_RING:\n\t"                                                                                                \
+        "shfl.sync.idx.b32 r6, %1, 0, 31, 0xffffffff;\n\t" "popc.b32 r0, %2;\n\t" "mad.lo.u32 r6, r0, 2, r6;\n\t"     \
+        "add.u32 r0, wthrA, 2;\n\t" "setp.lt.u32 pq, r6, r0;\n\t"                                                     \
+        "vote.sync.all.pred pq, pq, 0xffffffff;\n\t"                                                                  \
+        "@pq bra.uni EP_LOOP;\n\t"                           /* the cursor has not left its chunk */                  \
+        "ld.shared.v4.u32 {r11, r12, r1, r2}, [" EP_CTX "+32];\n\t"   /* source, bytes left, destination */           \
+        "mov.b64 ra, {r11, r12};\n\t"                                                                                 \
+        "popc.b32 r4, " EP_LT ";\n\t" "shl.b32 r4, r4, 4;\n\t"        /* 16 * lane */                                 \
+        "sub.s32 r3, r1, r4;\n\t" "min.s32 r3, r3, 16;\n\t"                                                           \
+        "setp.gt.s32 pv, r3, 0;\n\t" "setp.lt.and.u32 pv, r4, 256, pv;\n\t"                                           \
+        "mad.wide.u32 rb, r4, 1, ra;\n\t" "add.u32 r5, r2, r4;\n\t"                                                   \
+        "@pv cp.async.cg.shared.global [r5], [rb], 16, r3;\n\t"                                                       \
+        "sub.u32 r4, r2, r10;\n\t" "setp.lt.and.u32 pq, r4, 512, pv;\n\t"   /* slots 0 and 1 are written to the mirror as well */ \
+        "@pq cp.async.cg.shared.global [r5+1024], [rb], 16, r3;\n\t"                                                  \
+        "cp.async.commit_group;\n\t"                                                                                  \
+        "add.cc.u32 r11, r11, 256;\n\t" "addc.u32 r12, r12, 0;\n\t" "sub.s32 r1, r1, 256;\n\t"                        \
+        "add.u32 r2, r2, 256;\n\t" "setp.ge.u32 pv, r4, 768;\n\t" "selp.b32 r2, r10, r2, pv;\n\t"                     \
+        "bar.warp.sync 0xffffffff;\n\t"                                                                               \
+        "st.shared.v4.u32 [" EP_CTX "+32], {r11, r12, r1, r2};\n\t"                                                   \
+        "cp.async.wait_group 1;\n\t"                                                                                  \
+        "bar.warp.sync 0xffffffff;\n\t"                                                                               \
+        "add.u32 wthrA, wthrA, 256;\n\t" "sub.u32 r4, wthrA, r10;\n\t" "setp.lt.u32 pq, r4, 1278;\n\t"                \
+        "vote.sync.all.pred pq, pq, 0xffffffff;\n\t"                                                                  \
+        "@pq bra.uni EP_RING;\n\t"                                                                                    \
+        "sub.u32 wthrA, wthrA, 1024;\n\t" "sub.u32 %1, %1, 1024;\n\t"   /* past the fourth slot: everything back by the ring */ \
+        "ld.shared.u32 r5, [" EP_CTX "+52];\n\t" "sub.u32 r5, r5, 1024;\n\t"                                          \
+        "bar.warp.sync 0xffffffff;\n\t"                                                                               \
+        "st.shared.u32 [" EP_CTX "+52], r5;\n\t"                                                                      \
+        "bra.uni EP_RING;\n\t"                                                                                        \
+        "EP_DONE:\n\t"                                                                                                \
+        "}"                                                                                                           \
+        : "+&r"(x), "+&r"(a), "+&r"(bal), "+&r"(q)                                                                    \
+        : "r"(lt), "r"(lut_addr), "r"(lut_addr + kCosetStride), "r"(ctx), "l"(kk), "r"(cf.f0), "r"(cf.f1), "r"(sigma), "r"(act), \
+          "r"(P.groups), "r"(b_dst), "r"(bar_mma), "r"(bar_b), "n"(G::kSlab), "n"(kSpinLimit)                         \
+        : "memory")
 
 template <uint32_t TPAD>
 __global__ void __launch_bounds__(kThreads, 1) ep_decode_gemm_kernel(const __grid_constant__ GemmParams P,
                                                                      const __grid_constant__ CUtensorMap x_map) {
     extern __shared__ __align__(16) uint8_t smem[];      // (the operand tiles need 1024: checked at run time, see abort word)
     const JobParams &J = P.J;
-    const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
+    // (the warp's number by a shuffle: the compiler then knows that roles are warp-uniform and puts no guard around each vote
+    // of the decoding loop, which cost 500 of 1700 cycles per group)
+    const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = __shfl_sync(0xFFFFFFFFu, tid >> 5, 0);
     const uint32_t lut_addr = uint32_t(__cvta_generic_to_shared(smem));
     using G = GemmShape<TPAD>;
     const uint32_t a_base = lut_addr + G::kA, b_base = lut_addr + G::kB;
@@ -1540,7 +1617,7 @@ __global__ void __launch_bounds__(kThreads, 1) ep_decode_gemm_kernel(const __gri
     // (half a group's).  Per unit one mbarrier "landed" and one "read"; per slab of B one "rows stored" and one "read".
     constexpr uint32_t a_tile_bytes = TPAD * 128u, kUnitTiles = 8192u / a_tile_bytes, kUnitsPerGroup = 4u / kUnitTiles;
     const uint32_t bar_a = lut_addr + G::kBar, bar_afree = bar_a + 64u, bar_mma = bar_a + 128u, bar_b = bar_a + 144u,
-                   slot = bar_a + 160u, abort_addr = bar_a + 164u;
+                   slot = bar_a + 160u, abort_addr = bar_b + 100u;
     if (tid == 0) {
         for (uint32_t i = 0; i < G::kUnits; ++i) {
             mbar_init(bar_a + 8u * i, 1u);       // the loading lane's arrival; completes when the unit's tiles have landed
@@ -1557,11 +1634,8 @@ __global__ void __launch_bounds__(kThreads, 1) ep_decode_gemm_kernel(const __gri
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(slot), "r"(64u) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
-    // rows of the slabs that belong to no warp: zero
-    for (uint32_t i = tid; i < 2u * 4u * (G::kN - P.rows_per_step) * 8u; i += blockDim.x) {
-        const uint32_t piece = i & 7u, tile = (i >> 3) & 7u, row = P.rows_per_step + (i >> 6);
-        asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};" ::"r"(b_base + tile * G::kBTile + row * 128u + piece * 16u), "r"(0u) : "memory");
-    }
+    // (rows of the slabs that belong to no warp, or whose warp has no row in a CTA's last step, hold what they hold: they make
+    // columns of the accumulator that nobody stores)
     wait_for_stream();
     copy_tables_smem(J.lut_image, lut_addr, false);
     const CosetFreq cf = load_coset(J);
@@ -1669,7 +1743,7 @@ __global__ void __launch_bounds__(kThreads, 1) ep_decode_gemm_kernel(const __gri
         }
     } else if (warp < 2u + P.rows_per_step) {
         // ---- the decoding warps: one row of W each, group by group into the slabs of B ----
-        const uint32_t w = warp - 2u, lt = (1u << lane) - 1u, ring = lut_addr + kRingBase + w * kGemmRingStride;
+        const uint32_t w = warp - 2u, lt = (1u << lane) - 1u, ring = lut_addr + kRingBase + w * kGemmRingStride, ctx = lut_addr + kCtxBase + w * kCtxBytes;
         const uint32_t k0 = __float_as_uint(float(4096 - J.zlo));
         const uint64_t kk = pack64(k0, k0);
         // where this lane's block of a group goes in a slab: 64-column tile lane / 8, row = w, piece lane % 8 of the row
@@ -1681,44 +1755,32 @@ __global__ void __launch_bounds__(kThreads, 1) ep_decode_gemm_kernel(const __gri
             const TileSetup Tl = tile_setup(J, tile, true, lane);
             for (uint32_t c = 0; c < kGemmSlots; ++c) ring_issue<kGemmChunk, kGemmSlots>(ring, Tl.a0, Tl.room, c, lane);
             const uint32_t sigma = __float_as_uint(__ldg(J.scales + tile));
-            // the row this warp takes in the next step: its record is asked for now and, a few groups on, the start of
+            // the row this warp takes in the next step: its record is asked for now and, when that is here, the start of
             // its payload is brought into L2, so that the next step does not begin with two reads from DRAM in a row
             const bool has_next = r + P.rows_per_step < row_end;
             const uint32_t *rec_next = J.tile_index + size_t(min(r + P.rows_per_step, P.R - 1u)) * 33u;
             const uint32_t off_next = __ldg(rec_next + 32);
             if (has_next && lane == 0) prefetch_l2(rec_next);
+            if (lane == 0) {                 // the next request is chunk 4, into slot 0
+                sts64(ctx + kCtxChain + kCcSrc, Tl.a0 + kGemmChunk * kGemmSlots);
+                sts32(ctx + kCtxChain + kCcRem, Tl.room - kGemmChunk * kGemmSlots);
+                sts32(ctx + kCtxChain + kCcDst, ring);
+                sts32(ctx + kCtxChain + kCcRing, ring);
+                sts32(ctx + kCtxChain + kCcWbase, ring);
+            }
             cp_async_wait<1>();
             __syncwarp();
-            uint32_t x = Tl.x, bal = 0, a = ring + Tl.lead, wbase = ring, threshold = kGemmChunk, wthr = ring + kGemmChunk - 2u;
-            for (uint32_t g = 0; g < P.groups; ++g, ++q) {
-                if (g == 2u && has_next) {
-                    const uint64_t at = 2ull * min(off_next, J.total_words) + 128u * lane;      // 4 KB: the ring's first fill and more
-                    if (at < 2ull * J.total_words) prefetch_l2(J.stream + J.off_payload + at);
-                }
-                // is the slab free: is the tensor core done with the group that used it last, two groups ago?
-                const bool is_free = q < 2u || mbar_test(bar_mma + 8u * (q & 1u), ((q >> 1) - 1u) & 1u);
-                if (__any_sync(0xFFFFFFFFu, a >= wthr)) {               // the cursor left its chunk, or is about to
-                    const uint32_t pos = __shfl_sync(0xFFFFFFFFu, a, 0) + 2u * __popc(bal) - wbase;
-                    if (pos >= threshold) {
-                        ring_service<kGemmChunk, kGemmSlots>(ring, Tl.a0, Tl.room, pos, threshold, lane);
-                        if (pos + wbase - ring >= kGemmChunk * kGemmSlots) { a -= kGemmChunk * kGemmSlots; wbase -= kGemmChunk * kGemmSlots; }
-                        wthr = wbase + threshold - 2u;
-                    }
-                }
-                uint4 blk;
-                EP_GEMM_GROUP_ASM;
-                if (!act) blk = make_uint4(0u, 0u, 0u, 0u);
-                if (!is_free) {
-                    if (lane == 0) mbar_wait(bar_mma + 8u * (q & 1u), ((q >> 1) - 1u) & 1u, abort_addr);
-                    __syncwarp();
-                }
-                asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(b_dst + G::kSlab * (q & 1u)), "r"(blk.x), "r"(blk.y), "r"(blk.z), "r"(blk.w) : "memory");
-                __syncwarp();
-                if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar_b + 8u * (q & 1u)) : "memory");
+            if (has_next) {                  // 4 KB: the ring's first fill and more
+                const uint64_t at = 2ull * min(off_next, J.total_words) + 128u * lane;
+                if (at < 2ull * J.total_words) prefetch_l2(J.stream + J.off_payload + at);
             }
+            uint32_t x = Tl.x, bal = 0, a = ring + Tl.lead;
+            EP_GEMM_ROW_ASM;
             cp_async_wait<0>();              // nothing may still be landing in the ring when the next row starts
-            const uint32_t pos = __shfl_sync(0xFFFFFFFFu, a, 0) + 2u * __popc(bal) - wbase;
+            __syncwarp();
+            const uint32_t pos = __shfl_sync(0xFFFFFFFFu, a, 0) + 2u * __popc(bal) - lds32(ctx + kCtxChain + kCcWbase);
             bad |= act && ((x != ep::kStateLow) || (Tl.off + ((pos - Tl.lead) >> 1) != Tl.end));
+            __syncwarp();                    // the context block is rewritten for the next row
         }
     }
     const bool aborted = lds32(abort_addr) != 0;
