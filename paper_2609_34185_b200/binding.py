@@ -356,7 +356,10 @@ def upload(blob: Blob | np.ndarray, device="cuda", pinned=None, non_blocking=Fal
 
 def _stream_handle(stream) -> int:
     torch = _torch()
-    return (stream if stream is not None else torch.cuda.current_stream()).cuda_stream
+    if stream is not None:
+        return stream.cuda_stream
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)      # the same handle without building a Stream object (3 us)
+    return raw(torch.cuda.current_device()) if raw is not None else torch.cuda.current_stream().cuda_stream
 
 
 def decode(dblob: DeviceBlob, out_dtype: int = BF16, out=None, row_scales=None, stream=None):

@@ -220,8 +220,7 @@ __device__ __forceinline__ uint32_t cvt_s8(float v) {
 // a time: a warp scan gives each lane its symbol's first slot, every lane writes the first sixteen slots of
 // its own symbol, and the few symbols with more slots than that are then filled by the whole warp, one
 // after the other (that loop is serial: its length, not the number of stores, is what the build time
-// depends on).  `base` receives the 2048 entries: a shared-memory address here, see ep_prepare_tables_kernel
-// for the same routine writing a table image to global memory.
+// depends on).  `put` stores an entry.  (A prepared table image: ep_prepare_tables_kernel.)
 template <class Store>
 __device__ __forceinline__ void build_one_table(const JobParams &J, uint32_t t, uint32_t lane, Store put) {
     const uint32_t K = J.tK[t];
@@ -1835,12 +1834,33 @@ struct GBatchParams {
 constexpr int kGThreads = 256;
 constexpr int kGWarps = kGThreads / 32;
 
+// exclusive prefix sum over the 1024 threads of a CTA (one thread adding the 1024 parts up took 13 us of a table build)
+__device__ __forceinline__ uint32_t cta_exclusive_1024(uint32_t v, uint32_t *part) {
+    const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+    uint32_t incl = v;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const uint32_t n = __shfl_up_sync(0xFFFFFFFFu, incl, d);
+        if (lane >= uint32_t(d)) incl += n;
+    }
+    if (lane == 31) part[warp] = incl;
+    __syncthreads();
+    uint32_t w = part[lane];
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const uint32_t n = __shfl_up_sync(0xFFFFFFFFu, w, d);
+        if (lane >= uint32_t(d)) w += n;
+    }
+    const uint32_t before = __shfl_sync(0xFFFFFFFFu, w, int(warp) - 1 < 0 ? 0 : int(warp) - 1);
+    return (warp ? before : 0u) + incl - v;
+}
+
 // one CTA per (table, job): exclusive prefix sums of the frequencies in shared memory (as u16; the last
 // entry 2^b <= 32768 still fits), then every slot finds its symbol by binary search.  A table without symbols
 // (or whose frequencies fall short of 2^b in a damaged stream) gets index 0 with offset 0 in the slots nobody owns.
 __global__ void __launch_bounds__(1024) ep_build_tables_kernel(const __grid_constant__ GBatchParams P) {
     extern __shared__ __align__(16) uint8_t smem[];
-    __shared__ uint32_t part[1024];
+    __shared__ uint32_t part[32];
     const GJobParams &J = P.job[blockIdx.y];
     const uint32_t t = blockIdx.x, tid = threadIdx.x;
     const uint32_t K = J.tK[t];
@@ -1856,15 +1876,8 @@ __global__ void __launch_bounds__(1024) ep_build_tables_kernel(const __grid_cons
     const uint32_t j0 = min(tid * per, K), j1 = min(j0 + per, K);
     uint32_t sum = 0;
     for (uint32_t j = j0; j < j1; ++j) sum += fq[j];
-    part[tid] = sum;
-    __syncthreads();
-    if (tid == 0) {
-        uint32_t run = 0;
-        for (uint32_t i = 0; i < blockDim.x; ++i) { const uint32_t v = part[i]; part[i] = run; run += v; }
-        F[K] = uint16_t(min(run, M));                                // = 2^b for a valid stream
-    }
-    __syncthreads();
-    uint32_t run = part[tid];
+    uint32_t run = cta_exclusive_1024(sum, part);
+    if (tid == 1023u) F[K] = uint16_t(min(run + sum, M));            // = 2^b for a valid stream
     for (uint32_t j = j0; j < j1; ++j) { F[j] = uint16_t(min(run, M)); run += fq[j]; }
     __syncthreads();
     for (uint32_t u = tid; u < M; u += blockDim.x) {
@@ -1885,7 +1898,7 @@ __global__ void __launch_bounds__(1024) ep_build_tables_kernel(const __grid_cons
 // from producing states that take a word in every step).
 __global__ void __launch_bounds__(1024) ep_build_tables12_kernel(const __grid_constant__ GBatchParams P) {
     extern __shared__ __align__(16) uint8_t smem[];
-    __shared__ uint32_t part[1024];
+    __shared__ uint32_t part[32];
     const GJobParams &J = P.job[blockIdx.y];
     const uint32_t t = blockIdx.x + 1u, tid = threadIdx.x;
     const uint32_t K = J.tK[t];
@@ -1907,15 +1920,8 @@ __global__ void __launch_bounds__(1024) ep_build_tables12_kernel(const __grid_co
     const uint32_t j0 = min(tid * per, K), j1 = min(j0 + per, K);
     uint32_t sum = 0;
     for (uint32_t j = j0; j < j1; ++j) sum += fq[j];
-    part[tid] = sum;
-    __syncthreads();
-    if (tid == 0) {
-        uint32_t run = 0;
-        for (uint32_t i = 0; i < blockDim.x; ++i) { const uint32_t v = part[i]; part[i] = run; run += v; }
-        F[K] = uint16_t(min(run, M));
-    }
-    __syncthreads();
-    uint32_t run = part[tid];
+    uint32_t run = cta_exclusive_1024(sum, part);
+    if (tid == 1023u) F[K] = uint16_t(min(run + sum, M));
     for (uint32_t j = j0; j < j1; ++j) { F[j] = uint16_t(min(run, M)); run += fq[j]; }
     __syncthreads();
     for (uint32_t c = tid; c < kColdCodes; c += blockDim.x) {
@@ -2015,16 +2021,56 @@ __global__ void __launch_bounds__(kGThreads) ep_decode_glut_kernel(const __grid_
     }
 }
 
-// a prepared image of the sixteen shared-memory tables in global memory (ep_prepare_tables): warp w of the
-// job's CTA builds table w + 1 with the routine the decode kernel uses on shared memory
-__global__ void __launch_bounds__(512) ep_prepare_tables_kernel(const __grid_constant__ JobParams J, uint32_t *image) {
-    const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
-    const uint32_t t = 1u + warp;
-    if (t >= EP_NUM_TABLES) return;
-    uint32_t *dst = image + (t - 1u) * kLutEntries;
-    build_one_table(J, t, lane, [dst](uint32_t slot, uint32_t e) { dst[slot] = e; });
-    // b < 11: the slots above 2^b are never read, but the image is copied whole
-    for (uint32_t u = (1u << J.b) + lane; u < kLutEntries; u += 32) dst[u] = kEntryUnused;
+// A prepared image of the sixteen shared-memory tables in global memory (ep_prepare_tables): one CTA per table.  Prefix sums of
+// the frequencies, then every slot finds its symbol by binary search; the entries are build_one_table's.  (One CTA with
+// a warp per table, as in the decode kernel, took 8.4 us, most of it the serial loop over the symbols of many slots.)
+constexpr uint32_t kPrepThreads = 256, kPrepPer = kLutEntries / kPrepThreads;
+__global__ void __launch_bounds__(kPrepThreads) ep_prepare_tables_kernel(const __grid_constant__ JobParams J, uint32_t *image) {
+    __shared__ uint32_t first[kLutEntries + 1], part[kPrepThreads / 32];
+    const uint32_t tid = threadIdx.x, lane = tid & 31u, t = 1u + blockIdx.x, K = J.tK[t];      // K <= 2048 (see fits_smem_tables)
+    wait_for_stream();
+    const uint16_t *fq = reinterpret_cast<const uint16_t *>(J.stream + J.off_freq) + J.foff[t];
+    uint32_t f[kPrepPer], sum = 0;
+#pragma unroll
+    for (uint32_t i = 0; i < kPrepPer; ++i) {
+        const uint32_t j = tid * kPrepPer + i;
+        f[i] = j < K ? uint32_t(fq[j]) : 0u;
+        if (f[i] >= kLutEntries) atomicOr(&g_ep_status, 1u);
+        sum += f[i];
+    }
+    uint32_t incl = sum;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const uint32_t n = __shfl_up_sync(0xFFFFFFFFu, incl, d);
+        if (lane >= uint32_t(d)) incl += n;
+    }
+    if (lane == 31) part[tid >> 5] = incl;
+    __syncthreads();
+    uint32_t run = incl - sum;
+    for (uint32_t w = 0; w < tid >> 5; ++w) run += part[w];
+#pragma unroll
+    for (uint32_t i = 0; i < kPrepPer; ++i) {
+        if (tid * kPrepPer + i <= K) first[tid * kPrepPer + i] = run;
+        run += f[i];
+    }
+    if (tid == kPrepThreads - 1u && K == kLutEntries) first[K] = run;
+    __syncthreads();
+    const uint32_t total = first[K], slots = 1u << J.b;
+    const bool is_m = ((t - 1u) & 7u) == 7u;
+    for (uint32_t u = tid; u < kLutEntries; u += kPrepThreads) {
+        uint32_t e = kEntryUnused;                       // slots no symbol owns (a damaged stream) or that b < 11 does not have
+        if (u < min(total, slots)) {
+            uint32_t lo = 0, hi = K;                     // largest j with first[j] <= u
+            while (hi - lo > 1u) {
+                const uint32_t mid = (lo + hi) >> 1;
+                if (first[mid] <= u) lo = mid; else hi = mid;
+            }
+            const int32_t v = J.tmin[t] + int32_t(lo);
+            const uint32_t code = uint32_t((is_m ? 2 * v : v) - J.zlo);
+            e = (min(first[lo + 1u] - first[lo], kLutEntries - 1u) << 21) | ((code & 0x3FFu) << 11) | (u - first[lo]);
+        }
+        image[(t - 1u) * kLutEntries + u] = e;
+    }
 }
 
 // ---- host side -----------------------------------------------------------------------------------
@@ -2286,8 +2332,8 @@ extern "C" int ep_prepare_tables(const ep_info *info, const void *d_stream, void
         std::memset(&J, 0, sizeof(J));
         J.stream = static_cast<const uint8_t *>(d_stream);
         fill_table_params(J, I);
-        ep_prepare_tables_kernel<<<1, 512, 0, st>>>(J, static_cast<uint32_t *>(d_tables));
-        return cudaGetLastError() == cudaSuccess ? EP_OK : EP_ERR_CUDA;
+        return launch_next(ep_prepare_tables_kernel, EP_NUM_TABLES - 1, kPrepThreads, 0, st, J, static_cast<uint32_t *>(d_tables)) == cudaSuccess
+                   ? EP_OK : EP_ERR_CUDA;
     }
     GBatchParams P;
     std::memset(&P, 0, sizeof(P));
