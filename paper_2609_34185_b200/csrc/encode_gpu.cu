@@ -758,7 +758,8 @@ __device__ __forceinline__ float refit_result(double xp, double pp, float s, flo
 
 // One row per CTA; see "sums over a row" above.  sum p^2 is exact in any order (multiples of 1/4 below 2^51).
 __global__ void __launch_bounds__(kRowThreads) refit_kernel(const float *__restrict__ W, uint32_t C, const uint4 *__restrict__ fields,
-                                                            float s, const float *__restrict__ mu, float *__restrict__ sigma) {
+                                                            float s, const SearchState *__restrict__ state, const float *__restrict__ mu,
+                                                            float *__restrict__ sigma) {
     __shared__ double part[kRowThreads / 32];
     __shared__ __align__(16) float4 wbuf[2 * kRowThreads];
     __shared__ __align__(16) uint4 qbuf[kRowThreads];
@@ -783,6 +784,7 @@ __global__ void __launch_bounds__(kRowThreads) refit_kernel(const float *__restr
     xp = 0.5 * cta_sum(xp, part);
     const double pp = 0.25 * cta_sum(pp4, part);
     const double off = order_bound(C, 0.501 * cta_sum(double(mag), part));
+    if (state) s = state->s_counted;             // launched behind the search, before the host knows the scale
     const float m = __ldg(mu + blockIdx.x);
     const float lo = refit_result(__dsub_rn(xp, off), pp, s, m), hi = refit_result(__dadd_rn(xp, off), pp, s, m);
     if (lo == hi) {
@@ -1088,10 +1090,14 @@ public:
         mail_ = g_mail_slot.acquire(kMailBytes, 0, &mail_cap_);
         if (!mail_) throw std::bad_alloc();
     }
-    ~DeviceBackend() override { if (mail_) g_mail_slot.release(mail_, mail_cap_); }
+    ~DeviceBackend() override {
+        if (event_) cudaEventDestroy(event_);
+        if (mail_) g_mail_slot.release(mail_, mail_cap_);
+    }
 
     int prepare(const std::vector<uint32_t> &sample) override {
         n_sample_ = uint32_t(sample.size());
+        EP_CUDA(cudaEventCreateWithFlags(&event_, cudaEventDisableTiming));
         int dev = 0;
         EP_CUDA(cudaGetDevice(&dev));
         EP_CUDA(cudaDeviceGetAttribute(&sms_, cudaDevAttrMultiProcessorCount, dev));
@@ -1131,14 +1137,20 @@ public:
         F.hi0 = o.bracket_hi;
         F.last_step = o.polish_steps;
         for (F.step = 0; F.step <= o.polish_steps; ++F.step) EP_CUDA(launch_count(F, F.step > 0 || o.search_steps > 0));
-        const int rc = fetch(true);
+        // the row scales of the quantisation that is there now: while the host looks at the counts the GPU has nothing else to
+        // do (and if the host goes on to another scale, finish makes them again)
+        const int rc = fetch(true, [&] {
+            refit_kernel<<<R_, kRowThreads, 0, st_>>>(W_, C_, w_.fields, 0.0f, w_.state, w_.mu, w_.sigma);
+            return cudaGetLastError();
+        });
         if (rc) return rc;
         const SearchState &S = *state();
         if (S.undecided) {
             EP_CUDA(cudaMemsetAsync(w_.state, 0, kStateBytes, st_));
             return EP_OK;
         }
-        r.s = S.s_counted;
+        r.s = sigma_of_ = S.s_counted;
+        sigma_there_ = true;
         r.polished = S.polished != 0;
         r.has_last = S.has_last != 0;
         if (r.has_last) r.last.from_counts(S.last.lo, S.last.K, last_counts());
@@ -1201,23 +1213,34 @@ public:
         }
         compact_kernel<<<n_tiles, kCompactThreads, 0, st_>>>(w_.scratch, cap, w_.counts, w_.index, w_.payload);
         EP_CUDA(cudaMemcpyAsync(&state()->total_words, &w_.state->total_words, 4, cudaMemcpyDeviceToHost, st_));
-        refit_kernel<<<R_, kRowThreads, 0, st_>>>(W_, C_, w_.fields, s, w_.mu, w_.sigma);
+        if (!sigma_there_ || sigma_of_ != s) refit_kernel<<<R_, kRowThreads, 0, st_>>>(W_, C_, w_.fields, s, nullptr, w_.mu, w_.sigma);
         EP_CUDA(cudaGetLastError());
         return EP_OK;
     }
-    int end_finish(float s, int b, uint32_t V, const Model &m, ep_blob *out) override {
-        EP_CUDA(cudaStreamSynchronize(st_));
-        const uint64_t total = state()->total_words;
-        if (total >= (1ull << 31)) return EP_ERR_UNSUPPORTED;
-        // header and tables are laid out on the host; the other sections are copied straight into their place
+    int end_finish(float s, int b, uint32_t V, const Model &m, double cce, ep_blob *out) override {
+        const uint64_t nvec = uint64_t(R_) * (C_ / 8), n_tiles = (nvec + V - 1) / V;
+        // How many words the tiles have is known when the device is done; the copy is issued now, for a few more than the
+        // entropy says (coding loses about 1e-5 of it, and a tile's states keep some bits), never for more than the words' area
+        // holds.  Were they more even so, the blob is laid out again.
+        const uint64_t guess = uint64_t(cce / 16.0 * 1.001) + 8u * n_tiles + 256u;
+        uint64_t room = std::min(guess, std::min<uint64_t>(9ull * V * n_tiles, (1ull << 31) - 1u));
         out->acquire = pinned_acquire;
         out->release = pinned_release;
-        BlobLayout L;
-        const int rc = begin_blob(m, R_, C_, b, V, s, total, out, &L);
-        if (rc) return rc;
-        EP_CUDA(cudaMemcpyAsync(out->data() + L.off_scales, w_.sigma, L.total - L.off_scales, cudaMemcpyDeviceToHost, st_));
-        EP_CUDA(cudaStreamSynchronize(st_));
-        return EP_OK;
+        for (;;) {
+            // header and tables are laid out on the host; the other sections are copied straight into their place
+            BlobLayout L;
+            const int rc = begin_blob(m, R_, C_, b, V, s, room, out, &L);
+            if (rc) return rc;
+            EP_CUDA(cudaMemcpyAsync(out->data() + L.off_scales, w_.sigma, L.total - L.off_scales, cudaMemcpyDeviceToHost, st_));
+            EP_CUDA(cudaStreamSynchronize(st_));
+            const uint64_t total = state()->total_words;
+            if (total >= (1ull << 31)) return EP_ERR_UNSUPPORTED;
+            if (total <= room) {
+                end_blob(L, total, out);
+                return EP_OK;
+            }
+            room = total;
+        }
     }
 
 private:
@@ -1275,10 +1298,13 @@ private:
         return n;
     }
     // state and counts to the host: most alphabets fit the first copy
-    int fetch(bool last) {
+    template <class Meanwhile>
+    int fetch(bool last, Meanwhile launch) {
         EP_CUDA(cudaMemcpyAsync(mail_, w_.state, kStateBytes + (last ? 4ull * kFirstCounts : 0), cudaMemcpyDeviceToHost, st_));
         EP_CUDA(cudaMemcpyAsync(full_counts(), w_.full_counts, 4ull * kFirstCounts, cudaMemcpyDeviceToHost, st_));
-        EP_CUDA(cudaStreamSynchronize(st_));
+        EP_CUDA(cudaEventRecord(event_, st_));
+        EP_CUDA(launch());
+        EP_CUDA(cudaEventSynchronize(event_));
         const SearchState &S = *state();
         // (after a step it could not decide a search may have gone where the host's does not)
         if (S.overflow && !(last && S.undecided)) return EP_ERR_UNSUPPORTED;     // a coordinate beyond +-4095: use the host encoder
@@ -1295,7 +1321,8 @@ private:
     }
     int count(const uint32_t *rows, uint32_t n_rows, float s, uint4 *fields, Model &m) {
         EP_CUDA(launch_count(params(rows, n_rows, s, fields), false));
-        const int rc = fetch(false);
+        sigma_there_ = false;
+        const int rc = fetch(false, [] { return cudaSuccess; });
         if (rc) return rc;
         m.from_counts(state()->full.lo, state()->full.K, full_counts());
         return EP_OK;
@@ -1309,6 +1336,9 @@ private:
     uint8_t *mail_ = nullptr;        // page-locked: the copies back are plain DMA
     size_t mail_cap_ = 0;
     uint32_t n_sample_ = 0;
+    cudaEvent_t event_ = nullptr;
+    bool sigma_there_ = false;       // w_.sigma holds the row scales of the kept quantisation, which is at scale sigma_of_
+    float sigma_of_ = 0.0f;
 };
 
 uint32_t tile_vectors_of(const ep_encode_opts &o, double target_bpp) {

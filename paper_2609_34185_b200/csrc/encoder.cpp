@@ -255,6 +255,13 @@ int begin_blob(const Model &m, uint32_t R, uint32_t C, int b, uint32_t V, float 
     return EP_OK;
 }
 
+void end_blob(const BlobLayout &at, uint64_t total_words, ep_blob *out) {
+    const uint64_t total = at.off_payload + 2 * total_words;
+    store_le<uint64_t>(out->data() + 48, total);
+    store_le<uint32_t>(out->data() + 56, uint32_t(total_words));
+    out->shrink(size_t(total));
+}
+
 // header + tables + scales + tile index + payload
 int assemble_blob(const Model &m, uint32_t R, uint32_t C, int b, uint32_t V, const float *sigma, float s_info,
                   const uint32_t *states, const uint16_t *const *tile_words, const uint32_t *tile_len, ep_blob *out) {
@@ -391,7 +398,7 @@ int run_encode(EncodeBackend &be, uint32_t R, uint32_t C, double target_bpp, con
         last_rate = estimate_bits(last_step, last_b, svec, rows.size(), V, o.retained_bits, nullptr) / (8.0 * double(svec));
     }
     ep_blob *blob = new ep_blob();
-    rc = be.end_finish(s, b, V, full, blob);
+    rc = be.end_finish(s, b, V, full, cce, blob);
     if (rc) { delete blob; return rc; }
     blob->report.s = double(s);
     blob->report.b = b;
@@ -591,7 +598,7 @@ public:
         return EP_OK;
     }
     int begin_finish(float, int, uint32_t, const Model &) override { return EP_OK; }
-    int end_finish(float s, int b, uint32_t V, const Model &m, ep_blob *out) override {
+    int end_finish(float s, int b, uint32_t V, const Model &m, double, ep_blob *out) override {
         std::vector<float> sigma(R_);
         if (refined_sigma_.empty()) refit(W_, R_, C_, fields_.data(), s, mu_.data(), sigma.data(), threads_);
         else sigma = refined_sigma_;

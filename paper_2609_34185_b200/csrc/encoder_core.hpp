@@ -49,6 +49,8 @@ struct ep_blob {
         heap.resize(n);
         return heap.data();
     }
+    // the blob has only n of the bytes that were allocated
+    void shrink(size_t n) { if (ext) ext_size = n; else heap.resize(n); }
     const uint8_t *data() const { return ext ? ext : heap.data(); }
     uint8_t *data() { return ext ? ext : heap.data(); }
     size_t size() const { return ext ? ext_size : heap.size(); }
@@ -93,9 +95,10 @@ std::vector<uint32_t> sample_rows(uint32_t R, uint32_t C, uint32_t budget_vector
 struct BlobLayout { uint64_t off_tables, off_scales, off_tiles, off_payload, total; };
 
 // Allocates a blob for total_words payload words and writes its header and tables; the three sections after
-// off_scales are left to the caller.
+// off_scales are left to the caller.  If it turns out to have fewer words, end_blob corrects the size.
 int begin_blob(const Model &m, uint32_t R, uint32_t C, int b, uint32_t V, float s_info, uint64_t total_words, ep_blob *out,
                BlobLayout *at);
+void end_blob(const BlobLayout &at, uint64_t total_words, ep_blob *out);
 
 // header + tables + scales + tile index + payload; `states` holds 32 words per tile, tile t's payload is
 // tile_words[t] .. + tile_len[t].
@@ -131,7 +134,7 @@ struct EncodeBackend {
     // refit the row scales of the kept quantisation (Eq. 13), encode the tiles under the normalised full-tensor model m
     // and assemble the blob; the driver has work of its own between the two calls
     virtual int begin_finish(float s, int b, uint32_t V, const Model &m) = 0;
-    virtual int end_finish(float s, int b, uint32_t V, const Model &m, ep_blob *out) = 0;
+    virtual int end_finish(float s, int b, uint32_t V, const Model &m, double cce_bits, ep_blob *out) = 0;
     // per-row rate-distortion refinement of the kept quantisation (Sec. 3.5, Alg. 2); on success `m` holds the
     // counts of the refined fields and finish() uses the refined row scales.  Optional.
     virtual int refine(float /*s*/, int /*b*/, uint32_t /*V*/, const ep_encode_opts & /*o*/, Model & /*m*/) { return EP_ERR_UNSUPPORTED; }
