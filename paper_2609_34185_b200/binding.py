@@ -174,13 +174,19 @@ class Blob:
         return 8.0 * self.data.size / (self.info.R * self.info.C)
 
 
+# a memoryview of n bytes at an address (np.ctypeslib.as_array builds a ctypes type for every size: 15 us)
+_memory_view = C.pythonapi.PyMemoryView_FromMemory
+_memory_view.restype = C.py_object
+_memory_view.argtypes = [C.c_void_p, C.c_ssize_t, C.c_int]
+
+
 def _take(handle: C.c_void_p) -> Blob:
     L = load()
     n = L.ep_blob_bytes(handle)
     rep = EncodeReport()
     L.ep_blob_report(handle, C.byref(rep))
     # no copy: the array views the library's buffer, which is freed when the array (and every view of it) is gone
-    data = np.ctypeslib.as_array(C.cast(L.ep_blob_data(handle), C.POINTER(C.c_uint8)), shape=(n,))
+    data = np.frombuffer(_memory_view(L.ep_blob_data(handle), n, 0x200), np.uint8)      # (0x200: PyBUF_WRITE)
     weakref.finalize(data, L.ep_blob_free, handle)
     return Blob(data, rep.as_dict())
 

@@ -84,8 +84,7 @@ constexpr uint32_t kEntryUnused = 1u << 21;                  // f = 1: what a sl
 constexpr uint32_t kCtxScales = 0;         // u64 row scales
 constexpr uint32_t kCtxRowBytes = 8;       // u32 output bytes per row
 constexpr uint32_t kCtxRowMax = 12;        // u32 last row index
-constexpr uint32_t kCtxMul21 = 16;         // u32 2^21 and
-constexpr uint32_t kCtxMul11 = 20;         // u32 2^11: multipliers the hot loop must not see as constants (see EP_STEP)
+constexpr uint32_t kCtxTablesBar = 16;     // u64 warp 0's: the mbarrier of the table image's copy
 constexpr uint32_t kCtxRowRcp = 24;        // u32 ceil(2^32 / bytes per row)
 constexpr uint32_t kCtxChain = 32, kCtxChainStride = 32;
 constexpr uint32_t kCcSrc = 0;             // u64 global address of lane 0's 16 bytes of the next chunk to request
@@ -271,16 +270,47 @@ __device__ __forceinline__ void build_tables_smem(const JobParams &J, uint32_t l
     }
 }
 
-// the prepared image of the same sixteen tables: 128 KB copied by all threads of the CTA, 16 bytes each.  The
-// copy is only started here; whoever reads the tables first waits for it (cp.async.wait_group, then a CTA barrier).
-__device__ __forceinline__ void copy_tables_smem(const uint32_t *image, uint32_t lut_addr, bool two_level) {
-    const uint64_t src = reinterpret_cast<uint64_t>(image);
-    const uint32_t step = 16u * blockDim.x;
-    for (uint32_t o = 16u * threadIdx.x; o < kLutBytes; o += step) cp_async16(lut_addr + o, src + o, 16);
-    if (kTwoLevelInLoop && two_level)        // the hot part of the second level follows the image
-        for (uint32_t o = 16u * threadIdx.x; o < kHotBytes; o += step)
-            cp_async16(lut_addr + kHotBase + o, src + kLutBytes + o, 16);
-    cp_async_commit();
+// the prepared image of the same sixteen tables, 128 KB: one thread asks for it, the copy engine brings it in.  (256 threads
+// with 16 bytes per cp.async kept the load pipe busy for a microsecond, and the first tile's payload queued behind
+// it: 3.6 us from a launch's turn to its first group.)  Whoever reads the tables waits for the mbarrier first.
+__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
+}
+__device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+__device__ __forceinline__ void copy_tables_smem(const uint32_t *image, uint32_t lut_addr, uint32_t bar, bool two_level) {
+    constexpr uint32_t kPiece = 32768;
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(kLutBytes + (kTwoLevelInLoop && two_level ? kHotBytes : 0u)) : "memory");
+    auto piece = [&](uint32_t dst, uint32_t src, uint32_t bytes) {
+        asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                     ::"r"(dst), "l"(reinterpret_cast<uint64_t>(image) + src), "r"(bytes), "r"(bar) : "memory");
+    };
+    for (uint32_t o = 0; o < kLutBytes; o += kPiece) piece(lut_addr + o, o, kPiece);
+    if (kTwoLevelInLoop && two_level) piece(lut_addr + kHotBase, kLutBytes, kHotBytes);      // the hot part of the second level follows the image
+}
+
+// How the job's lookup tables come about, and the wait for them.  All branches are on votes or parameters (a guard around each
+// vote of the hot loop costs more than the wait).  A copy that does not end within the limit - there is no such case -
+// raises the integrity word; the tables then hold anything, which is safe (see build_one_table) but wrong.
+enum TablesPending : uint32_t { kTablesThere, kTablesBuilt, kTablesCopied };   // nothing to wait for; this CTA's stores; the copy
+struct TablesWait { uint32_t pending, bar, parity; };
+constexpr uint32_t kSpinLimit = 1u << 18;             // attempts of about a microsecond each at most: a quarter of a second
+__device__ __forceinline__ void wait_for_tables(const TablesWait &W) {
+    if (W.pending == kTablesBuilt) __syncthreads();
+    if (W.pending == kTablesCopied) {
+        uint32_t left;
+        asm volatile("{\n\t.reg .pred p;\n\tmov.b32 %0, %3;\n\t"
+                     "EP_TABLES_WAIT:\n\t"
+                     "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, 1000;\n\t"
+                     "vote.sync.all.pred p, p, 0xffffffff;\n\t"
+                     "@p bra.uni EP_TABLES_DONE;\n\t"
+                     "sub.u32 %0, %0, 1;\n\t"
+                     "setp.ne.u32 p, %0, 0;\n\t"
+                     "vote.sync.all.pred p, p, 0xffffffff;\n\t"
+                     "@p bra.uni EP_TABLES_WAIT;\n\t"
+                     "EP_TABLES_DONE:\n\t}"
+                     : "=&r"(left) : "r"(W.bar), "r"(W.parity), "n"(kSpinLimit) : "memory");
+        if (left == 0) atomicOr(&g_ep_status, 2u);
+    }
 }
 
 // frequencies of the two cosets as the decode uses them: u < f0 means coset 0.  A coset that never occurs
@@ -647,40 +677,12 @@ __device__ __forceinline__ void decode_tile_plain(const JobParams &J, uint32_t t
 #define EP_B_NB(S, BAL) "nb" S
 #define EP_B_BL(S, BAL) BAL
 // a coordinate field: table OFF / 8192 of the lane's coset (Eq. 18)
-#ifdef EP_STEP_WIDE
-// x * 2^21 as a 64-bit product gives x >> 11 in the high word and the slot in the top bits of the low word,
-// e * 2^11 gives f in the high word: both on the multiply-add pipe instead of shifts and masks on the ALU pipe
-// (the two multipliers come from memory so that the assembler does not turn the products back into shifts)
-#define EP_L1(S, X, AW, BAL, DOFF, CB, E, OFF, BIN, BOUT) "mul.wide.u32 xw" S ", " X ", m21;\n\t" "mov.b64 {u" S ", q" S "}, xw" S ";\n\t"
-#define EP_L2(S, X, AW, BAL, DOFF, CB, E, OFF, BIN, BOUT) "shr.u32 u" S ", u" S ", 19;\n\t" "add.u32 u" S ", u" S ", tab" S ";\n\t"
-#define EP_L3(S, X, AW, BAL, DOFF, CB, E, OFF, BIN, BOUT) "ld.shared.u32 " E S ", [u" S "+" OFF "];\n\t"
-#define EP_L4(S, X, AW, BAL, DOFF, CB, E, OFF, BIN, BOUT)
-#ifdef EP_STEP_WIDEQ
-#define EP_L5(S, X, AW, BAL, DOFF, CB, E, OFF, BIN, BOUT) "shr.u32 f" S ", " E S ", 21;\n\t"
-#else
-#define EP_L5(S, X, AW, BAL, DOFF, CB, E, OFF, BIN, BOUT) "mul.wide.u32 xw" S ", " E S ", m11;\n\t" "mov.b64 {bi" S ", f" S "}, xw" S ";\n\t"
-#endif
-#else
 // slot address 4 (x & 0x7FF) + tab as 4 x - 8192 (x >> 11) + tab: two multiply-adds instead of a mask and one (the
 // multiply-add pipe has room, the ALU pipe has not; measured + 0.3 % / + 0.8 % on the 8192^2 tensor / the layer)
-#ifndef EP_SLOT_MASK
 #define EP_L1(S, X, AW, BAL, DOFF, CB, E, OFF, BIN, BOUT) "shr.u32 q" S ", " X ", 11;\n\t" "mad.lo.u32 u" S ", q" S ", 0xFFFFE000, tab" S ";\n\t"
 #define EP_L2(S, X, AW, BAL, DOFF, CB, E, OFF, BIN, BOUT) "mad.lo.u32 u" S ", " X ", 4, u" S ";\n\t"
-#else
-#define EP_L1(S, X, AW, BAL, DOFF, CB, E, OFF, BIN, BOUT) "and.b32 u" S ", " X ", 0x7FF;\n\t"
-#define EP_L2(S, X, AW, BAL, DOFF, CB, E, OFF, BIN, BOUT) "mad.lo.u32 u" S ", u" S ", 4, tab" S ";\n\t"
-#endif
 #define EP_L3(S, X, AW, BAL, DOFF, CB, E, OFF, BIN, BOUT) "ld.shared.u32 " E S ", [u" S "+" OFF "];\n\t"
-#ifndef EP_SLOT_MASK
-#define EP_L4(S, X, AW, BAL, DOFF, CB, E, OFF, BIN, BOUT)
-#elif defined(EP_Q_MULHI)
-// x >> 11 as the high word of x * 2^21: on the multiply-add pipe, off the step's critical path
-#define EP_L4(S, X, AW, BAL, DOFF, CB, E, OFF, BIN, BOUT) "mul.hi.u32 q" S ", " X ", m21;\n\t"
-#else
-#define EP_L4(S, X, AW, BAL, DOFF, CB, E, OFF, BIN, BOUT) "shr.u32 q" S ", " X ", 11;\n\t"
-#endif
 #define EP_L5(S, X, AW, BAL, DOFF, CB, E, OFF, BIN, BOUT) "shr.u32 f" S ", " E S ", 21;\n\t"
-#endif
 #define EP_L6(S, X, AW, BAL, DOFF, CB, E, OFF, BIN, BOUT) "and.b32 bi" S ", " E S ", 0x7FF;\n\t"
 #define EP_L7(S, X, AW, BAL, DOFF, CB, E, OFF, BIN, BOUT) "@act" S " mad.lo.u32 " X ", f" S ", q" S ", bi" S ";\n\t"
 // renormalisation: lanes whose state fell below 2^15 take a word each, in lane order
@@ -698,7 +700,7 @@ __device__ __forceinline__ void decode_tile_plain(const JobParams &J, uint32_t t
     EP_ALL(EP_L14, E, OFF, BIN, BOUT)
 #define EP_STEP_ALL(E, OFF, BIN, BOUT)                                                               \
     EP_ALL(EP_L1, E, OFF, BIN, BOUT) EP_ALL(EP_L2, E, OFF, BIN, BOUT) EP_ALL(EP_L3, E, OFF, BIN, BOUT)   \
-    EP_ALL(EP_L4, E, OFF, BIN, BOUT) EP_ALL(EP_L5, E, OFF, BIN, BOUT) EP_ALL(EP_L6, E, OFF, BIN, BOUT)   \
+    EP_ALL(EP_L5, E, OFF, BIN, BOUT) EP_ALL(EP_L6, E, OFF, BIN, BOUT)   \
     EP_ALL(EP_L7, E, OFF, BIN, BOUT) EP_RENORM_ALL(E, OFF, BIN, BOUT)
 // the coset: slot below f0 -> coset 0 with frequency f0, else coset 1 with frequency f1 and offset f0
 #define EP_C1(S, X, AW, BAL, DOFF, CB) "and.b32 u" S ", " X ", 0x7FF;\n\t"
@@ -719,16 +721,6 @@ __device__ __forceinline__ void decode_tile_plain(const JobParams &J, uint32_t t
 #define EP_P2(S, X, AW, BAL, DOFF, CB) "sub.rn.f32x2 pr" S ", pr" S ", " EP_KK ";\n\t"
 #define EP_P3(S, X, AW, BAL, DOFF, CB) "mul.rn.f32x2 pr" S ", pr" S ", ss" S ";\n\t"
 #define EP_P4(S, X, AW, BAL, DOFF, CB) "mov.b64 {wl" S ", wh" S "}, pr" S ";\n\t"
-#ifdef EP_SCALAR_FP
-#undef EP_P1
-#undef EP_P2
-#undef EP_P3
-#undef EP_P4
-#define EP_P1(S, X, AW, BAL, DOFF, CB) "mov.b32 wl" S ", xa" S ";\n\t" "sub.rn.f32 wl" S ", wl" S ", k0f;\n\t"
-#define EP_P2(S, X, AW, BAL, DOFF, CB) "mov.b32 wh" S ", xb" S ";\n\t" "sub.rn.f32 wh" S ", wh" S ", k0f;\n\t"
-#define EP_P3(S, X, AW, BAL, DOFF, CB) "mul.rn.f32 wl" S ", wl" S ", sg" S ";\n\t"
-#define EP_P4(S, X, AW, BAL, DOFF, CB) "mul.rn.f32 wh" S ", wh" S ", sg" S ";\n\t"
-#endif
 #define EP_PAIR_ALL EP_ALL(EP_P1) EP_ALL(EP_P2) EP_ALL(EP_P3) EP_ALL(EP_P4)
 // parity of z1 + ... + z7 = xor of the codes' lowest bits (bit 11 of the entries; zlo is even): the lowest bit of z8
 #define EP_PAR3(S, X, AW, BAL, DOFF, CB, EA, EB, EC) "lop3.b32 par" S ", " EA S ", " EB S ", " EC S ", 0x96;\n\t"
@@ -928,7 +920,7 @@ __device__ __forceinline__ void decode_tile_plain(const JobParams &J, uint32_t t
     ".reg .b16 h0" S ", h1" S ", h2" S ", h3" S ";\n\t"                                                              \
     ".reg .f32 wl" S ", wh" S ", sg" S ";\n\t"                                                                       \
     ".reg .b32 lim" S ", wthr" S ", hotc" S ";\n\t"                                                                  \
-    ".reg .b64 pr" S ", ss" S ", ad" S ", xw" S ", lc" S ";\n\t"
+    ".reg .b64 pr" S ", ss" S ", ad" S ", lc" S ";\n\t"
 // before the first pass: the cursor leaves its first chunk at ring + chunk size - 2; lim = 0 sends the chain through EP_ROWS
 #define EP_INIT(S, X, AW, BAL, DOFF, CB)                                 \
     "ld.shared.u32 r0, [" EP_CTX "+" CB "+16];\n\t"                      \
@@ -1049,7 +1041,7 @@ __device__ __forceinline__ void decode_tile_plain(const JobParams &J, uint32_t t
         "{\n\t"                                                                                                       \
         EP_ALL(EP_REGS)                                                                                               \
         ".reg .pred pq, pv, pr;\n\t"                                                                                  \
-        ".reg .b32 r0, r1, r2, r3, r4, r5, r6, r7, r8, r9, r10, r11, r12, c0r, c1r, d0r, d1r, f0c, m21, m11, hotb, hotb1;\n\t" \
+        ".reg .b32 r0, r1, r2, r3, r4, r5, r6, r7, r8, r9, r10, r11, r12, c0r, c1r, d0r, d1r, f0c, hotb, hotb1;\n\t" \
         ".reg .b64 ra, rb, l2b1;\n\t"                                                                                 \
         ".reg .f32 k0f, k1f;\n\t"                                                                                     \
         "mov.b64 {k0f, k1f}, " EP_KK ";\n\t"                                                                          \
@@ -1061,7 +1053,6 @@ __device__ __forceinline__ void decode_tile_plain(const JobParams &J, uint32_t t
         "add.u32 hotb, " EP_LUT0 ", " EP_HOTOFF ";\n\t"   /* 2^12-slot streams: hot entries of coset 0, */              \
         "add.u32 hotb1, hotb, 16896;\n\t"                 /* of coset 1; complete array of coset 1 */                   \
         "add.s64 l2b1, " EP_L2B ", 131072;\n\t"                                                                       \
-        "ld.shared.v2.u32 {m21, m11}, [" EP_CTX "+16];\n\t" /* 2^21, 2^11 */                                          \
         EP_ALL(EP_INIT)                                                                                               \
         "bra.uni EP_RARE;\n\t"                                                                                        \
         "EP_LOOP:\n\t"                                                                                                \
@@ -1185,11 +1176,11 @@ __device__ __forceinline__ void decode_tile_plain(const JobParams &J, uint32_t t
 // `first + c`.  A chain whose slot lies past the job's last tile gets that last tile's record, only so that its
 // addresses stay inside the stream, and no block at all.  The number of groups is data here, not control flow the
 // compiler reasons about: every branch on it is a bra.uni on a warp vote.
-// `tables_pending`: the job's lookup tables are still being written (by this CTA's own stores or copies): the
+// `tables`: the job's lookup tables may still be being written (by this CTA's own stores or copies): the
 // tiles' records and first payload chunks are requested first, the CTA barrier comes after.
 template <int DT, int B>
 __device__ __forceinline__ void decode_tiles_fast(const JobParams &J, uint32_t first, uint32_t tiles_per_round, uint32_t lut_addr,
-                                                  CosetFreq cf, uint32_t ring, uint32_t ctx, uint32_t lane, bool tables_pending) {
+                                                  CosetFreq cf, uint32_t ring, uint32_t ctx, uint32_t lane, const TablesWait &tables) {
     constexpr uint32_t BB = Out<DT>::kBlockBytes;
     const uint32_t lt = (1u << lane) - 1u, lane16 = 16u * lane;
     uint32_t x[kChains], a[kChains], bal[kChains], doff[kChains], off[kChains], end[kChains], lead[kChains];
@@ -1216,9 +1207,9 @@ __device__ __forceinline__ void decode_tiles_fast(const JobParams &J, uint32_t f
         x[c] = T.x; a[c] = rg + T.lead; bal[c] = 0; doff[c] = (T.v0 + lane) * BB;
         off[c] = T.off; end[c] = T.end; lead[c] = T.lead;
     }
-    cp_async_wait<1>();           // all but the last chain's third chunk have landed (and the table image, if any)
+    cp_async_wait<1>();           // all but the last chain's third chunk have landed
     __syncwarp();
-    if (tables_pending) __syncthreads();
+    wait_for_tables(tables);
     const uint32_t k0 = __float_as_uint(float((B == 11 ? 4096 : 4194304) - J.zlo));
     const uint64_t kk = pack64(k0, k0);
     const uint64_t out_base = reinterpret_cast<uint64_t>(J.out);
@@ -1261,7 +1252,7 @@ __device__ __forceinline__ void decode_tiles_fast(const JobParams &J, uint32_t f
 // depends on parameters or is a bra.uni on a vote: a guard around each vote would cost 25 cycles.)
 template <int DT>
 __device__ __forceinline__ void decode_tile_few(const JobParams &J, uint32_t first, uint32_t tiles_per_round, uint32_t lut_addr,
-                                                CosetFreq cf, uint32_t ctx, uint32_t lane, bool tables_pending) {
+                                                CosetFreq cf, uint32_t ctx, uint32_t lane, const TablesWait &tables) {
     constexpr uint32_t BB = Out<DT>::kBlockBytes, kHead = 1024;
     const uint32_t warp = threadIdx.x >> 5, space = kStageBytes / tiles_per_round & ~127u;
     const bool valid = first < J.tile_cnt && warp < tiles_per_round;
@@ -1295,9 +1286,9 @@ __device__ __forceinline__ void decode_tile_few(const JobParams &J, uint32_t fir
         sts32(ctx + kCtxChain + kCcWbase, window);
     }
     if (lane == 0) sts32(ctx + kCtxChain + kCcEndo, endo);
-    cp_async_wait<1>();           // the table image, if any, and the first kilobyte
+    cp_async_wait<1>();           // the scales and the first kilobyte
     __syncwarp();
-    if (tables_pending) __syncthreads();
+    wait_for_tables(tables);
     const uint32_t k0 = __float_as_uint(float(4096 - J.zlo)), lt = (1u << lane) - 1u;
     const uint64_t kk = pack64(k0, k0), out_base = reinterpret_cast<uint64_t>(J.out);
     if (J.guess) {
@@ -1342,6 +1333,12 @@ ep_decode_smem_kernel(const __grid_constant__ BatchParams P) {
     const uint32_t ring = lut_addr + kRingBase + warp * (kChains * kRingStride);
     const uint32_t ctx = lut_addr + kCtxBase + warp * kCtxBytes;
     bool tables_in_use = false;
+    TablesWait tables{kTablesThere, lut_addr + kCtxBase + kCtxTablesBar, 1u};
+    if (threadIdx.x == 0) {
+        mbar_init(tables.bar, 1u);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    __syncthreads();
     wait_for_stream();
     for (int j = 0; j < P.n_jobs; ++j) {
         const JobParams &J = P.job[j];
@@ -1355,10 +1352,18 @@ ep_decode_smem_kernel(const __grid_constant__ BatchParams P) {
         if (tables_in_use) __syncthreads();          // every warp is done with the previous job's tables
         // the table image is requested first: the tiles' records and payload (two dependent reads of memory that no
         // cache holds yet) are on their way while it arrives
-        if (J.lut_image) copy_tables_smem(J.lut_image, lut_addr, J.b == 12u);
-        else build_tables_smem(J, lut_addr, warp, lane);
+        if (J.lut_image) {
+            tables.pending = kTablesCopied;
+            tables.parity ^= 1u;
+            if (threadIdx.x == 0) {
+                if (tables_in_use) fence_async_smem();   // the last job's lookups, ordered before this by the barrier above
+                copy_tables_smem(J.lut_image, lut_addr, tables.bar, J.b == 12u);
+            }
+        } else {
+            tables.pending = kTablesBuilt;
+            build_tables_smem(J, lut_addr, warp, lane);
+        }
         const CosetFreq cf = load_coset(J);
-        bool tables_pending = true;
         tables_in_use = true;
         // (a stream with 2^12 slots reaches this kernel only in the configuration of the hot loop: see the launcher)
         const bool fast = DT != EP_FIELDS_I32 && J.per_row >= 32u && (J.b == 11u || J.b == 12u) && J.V < (1u << 20);
@@ -1366,8 +1371,6 @@ ep_decode_smem_kernel(const __grid_constant__ BatchParams P) {
             sts64(ctx + kCtxScales, reinterpret_cast<uint64_t>(J.scales));
             sts32(ctx + kCtxRowBytes, J.row_bytes);
             sts32(ctx + kCtxRowMax, J.row_max);      // the step after a tensor's last block must not read past the scales
-            sts32(ctx + kCtxMul21, 1u << 21);
-            sts32(ctx + kCtxMul11, 1u << 11);
             sts32(ctx + kCtxRowRcp, J.row_rcp);
         }
         __syncwarp();
@@ -1376,21 +1379,18 @@ ep_decode_smem_kernel(const __grid_constant__ BatchParams P) {
             if constexpr (DT != EP_FIELDS_I32) {
                 if (fast) {
                     if (kTwoLevelInLoop && J.b == 12u) {
-                        if constexpr (kTwoLevelInLoop) decode_tiles_fast<DT, 12>(J, base, P.tiles_per_round, lut_addr, cf, ring, ctx, lane, tables_pending);
+                        if constexpr (kTwoLevelInLoop) decode_tiles_fast<DT, 12>(J, base, P.tiles_per_round, lut_addr, cf, ring, ctx, lane, tables);
                     } else if constexpr (FEW) {
-                        decode_tile_few<DT>(J, base, P.tiles_per_round, lut_addr, cf, ctx, lane, tables_pending);
+                        decode_tile_few<DT>(J, base, P.tiles_per_round, lut_addr, cf, ctx, lane, tables);
                     } else {
-                        decode_tiles_fast<DT, 11>(J, base, P.tiles_per_round, lut_addr, cf, ring, ctx, lane, tables_pending);
+                        decode_tiles_fast<DT, 11>(J, base, P.tiles_per_round, lut_addr, cf, ring, ctx, lane, tables);
                     }
-                    tables_pending = false;
+                    tables.pending = kTablesThere;
                     continue;
                 }
             }
-            if (tables_pending) {
-                cp_async_wait<0>();
-                __syncthreads();
-                tables_pending = false;
-            }
+            wait_for_tables(tables);
+            tables.pending = kTablesThere;
             for (uint32_t c = 0; c < kChains; ++c)
                 if (base + c < J.tile_cnt && kChains * warp + c < P.tiles_per_round) decode_tile_plain<DT>(J, J.tile0 + base + c, lut_addr, cf, ring, lane);
         }
@@ -1439,7 +1439,6 @@ struct GemmParams {
 
 constexpr uint32_t kGemmChunk = 256, kGemmSlots = 4;     // payload ring of this kernel
 constexpr uint32_t kGemmRingStride = kGemmChunk * kGemmSlots + kRingMirror;   // 1536
-constexpr uint32_t kSpinLimit = 1u << 18;             // attempts of about a microsecond each at most: a quarter of a second
 // what depends on the number of tokens that are staged.  Up to 16: thirty rows of W per step, x in two units of a whole
 // group.  Up to 32 a group's columns of x fill 16 KB, and with no more than that a unit could be asked for only when the
 // instructions of the group before had read it (10240 x 3840, 32 tokens: 80.9 us): 24 rows per step make room for 32 KB,
@@ -1458,9 +1457,6 @@ struct GemmShape {
     static_assert(kSmem <= 232448, "more shared memory than an sm_100 CTA can have");
 };
 
-__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
-}
 // a test that never waits
 __device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {
     uint32_t ok;
@@ -1487,7 +1483,6 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, uint32_
     sts32(abort_addr, 1u);
     return false;
 }
-__device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 // K-major operand tile with 128-byte swizzle: rows of 128 bytes, groups of eight rows 1024 bytes apart
@@ -1617,6 +1612,7 @@ __global__ void __launch_bounds__(kThreads, 1) ep_decode_gemm_kernel(const __gri
     constexpr uint32_t a_tile_bytes = TPAD * 128u, kUnitTiles = 8192u / a_tile_bytes, kUnitsPerGroup = 4u / kUnitTiles;
     const uint32_t bar_a = lut_addr + G::kBar, bar_afree = bar_a + 64u, bar_mma = bar_a + 128u, bar_b = bar_a + 144u,
                    slot = bar_a + 160u, abort_addr = bar_b + 100u;
+    const TablesWait tables{kTablesCopied, bar_a + 168u, 0u};
     if (tid == 0) {
         for (uint32_t i = 0; i < G::kUnits; ++i) {
             mbar_init(bar_a + 8u * i, 1u);       // the loading lane's arrival; completes when the unit's tiles have landed
@@ -1626,6 +1622,7 @@ __global__ void __launch_bounds__(kThreads, 1) ep_decode_gemm_kernel(const __gri
             mbar_init(bar_mma + 8u * i, 1u);     // the commit after a group's matrix instructions
             mbar_init(bar_b + 8u * i, P.rows_per_step);   // every decoding warp, when its row of the slab is stored
         }
+        mbar_init(tables.bar, 1u);
         sts32(abort_addr, (lut_addr & 1023u) ? 1u : 0u);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -1635,13 +1632,12 @@ __global__ void __launch_bounds__(kThreads, 1) ep_decode_gemm_kernel(const __gri
     }
     // (rows of the slabs that belong to no warp, or whose warp has no row in a CTA's last step, hold what they hold: they make
     // columns of the accumulator that nobody stores)
-    wait_for_stream();
-    copy_tables_smem(J.lut_image, lut_addr, false);
-    const CosetFreq cf = load_coset(J);
-    cp_async_wait<0>();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    wait_for_stream();
+    if (tid == 0) copy_tables_smem(J.lut_image, lut_addr, tables.bar, false);
+    const CosetFreq cf = load_coset(J);
     const uint32_t tmem = lds32(slot);
 
     const uint32_t row_begin = min(blockIdx.x * P.rows_per_cta, P.R), row_end = min(row_begin + P.rows_per_cta, P.R);
@@ -1774,6 +1770,7 @@ __global__ void __launch_bounds__(kThreads, 1) ep_decode_gemm_kernel(const __gri
                 if (at < 2ull * J.total_words) prefetch_l2(J.stream + J.off_payload + at);
             }
             uint32_t x = Tl.x, bal = 0, a = ring + Tl.lead;
+            if (s == 0) wait_for_tables(tables);
             EP_GEMM_ROW_ASM;
             cp_async_wait<0>();              // nothing may still be landing in the ring when the next row starts
             __syncwarp();
