@@ -584,3 +584,65 @@ def test_largest_supported_tensor_byte_offsets_beyond_two_to_the_31():
     with pytest.raises(ep.EntroPackError) as ei:
         ep.decode_tensor(big, d.d_stream, d.d_tile_index, d.d_row_scales, ep.FP32, out.data_ptr())
     assert ei.value.status == -3
+
+
+def _check(blob, dts):
+    d = ep.upload(blob)
+    for dt in dts:
+        got = ep.decode(d, dt)
+        torch.cuda.synchronize()
+        want = oracle.decode(blob.data, ORACLE_DT[dt])[0]
+        assert np.array_equal(_bits(got), want.view(np.uint32) if dt == ep.FP32 else want), f"dtype {dt}"
+    assert ep.last_device_status() == 0
+
+
+@pytest.mark.parametrize("R,C,V,spread", [
+    (512, 512, 32768, 1.0),      # one tile of 80 KB: fits its window
+    (512, 1024, 65536, 3.0),     # one tile of 270 KB: the window moves twice; groups are guessed, and some repeated
+    (512, 1024, 65536, 9.0),     # payload rate above the guess's limit
+    (333, 2056, 28521, 2.0),     # four tiles with ragged ends
+    (64, 256, 33, 3.0),          # rows of 32 blocks: a new row scale in every group; tiles of one group and a lane
+    (301, 264, 50, 2.0),         # rows of 33 blocks, tiles that end inside rows
+    (8, 4096, 1, 3.0),           # tiles of one block
+    (2368, 512, 64, 3.0),        # sixteen tiles per SM
+    (2369, 512, 64, 3.0),        # ... and one tile more: the ordinary loop
+])
+def test_few_tiles_per_sm(R, C, V, spread):
+    rng = np.random.default_rng(9000 + R + C)
+    n = R * C // 8
+    fields = np.zeros((n, 9), np.int32)
+    fields[:, 0] = rng.integers(0, 2, n)
+    fields[:, 1:8] = np.rint(rng.standard_normal((n, 7)) * spread).astype(np.int32)
+    fields[:, 8] = np.rint(rng.standard_normal(n) * spread / 2).astype(np.int32)
+    blob = ep.pack_fields(fields, R, C, 11, V, rng.uniform(0.01, 0.05, R).astype(np.float32))
+    assert ep.decode_scratch_bytes(blob.info) == 0
+    _check(blob, (ep.BF16, ep.INT8, ep.FP32))
+
+
+def test_few_tiles_states_that_need_words_in_successive_steps():
+    # symbols of frequency 1 next to one of frequency close to 2^11: a lane that has just taken a word often needs the next
+    # one at once, which is what the guessing loop takes for granted that it does not
+    rng = np.random.default_rng(91)
+    R, C = 256, 1024
+    n = R * C // 8
+    fields = np.zeros((n, 9), np.int32)
+    for k in range(1, 9):
+        rare = rng.random(n) < 0.05
+        fields[rare, k] = rng.integers(-200, 200, int(rare.sum()))
+    fields[rng.random(n) < 0.01, 0] = 1
+    blob = ep.pack_fields(fields, R, C, 11, 2000, rng.uniform(0.01, 0.05, R).astype(np.float32))
+    assert ep.decode_scratch_bytes(blob.info) == 0 and 16 * blob.info.total_words < 3.6 * 9 * n
+    _check(blob, (ep.FP16, ep.FP8_E4M3))
+
+
+def test_few_tiles_damaged_payload_is_flagged_not_fatal():
+    W = synth.laplace_rows(128, 2048, 92)
+    blob = ep.encode(W, 4.0, tile_vectors=8192)
+    data = blob.data.copy()
+    rng = np.random.default_rng(92)
+    data[blob.info.off_payload:] = rng.integers(0, 256, data.size - blob.info.off_payload, dtype=np.uint8)
+    d = ep.upload(data)
+    ep.decode(d, ep.BF16)
+    torch.cuda.synchronize()
+    assert ep.last_device_status() == -2
+    _check(blob, (ep.BF16,))

@@ -85,6 +85,25 @@ def test_decode_matmul_random_shapes():
         _check(blob, T, 7700 + case)
 
 
+@pytest.mark.parametrize("R,C,T", [
+    (148 * 24, 256, 32),          # one step of 24 rows, one group per row: two half-group units of x per step
+    (148 * 24 + 1, 256, 17),      # two steps
+    (148 * 49, 512, 32),          # three steps, two groups per row: four units in flight
+    (148 * 61, 256, 16),          # three steps for up to 16 tokens, one unit of x per step
+    (148 * 30 + 5, 1024, 1),
+    (3, 4096, 32),                # fewer rows than CTAs
+])
+def test_decode_matmul_at_the_edges_of_its_steps(R, C, T):
+    rng = np.random.default_rng(76)
+    n = R * C // 8
+    fields = np.zeros((n, 9), np.int32)
+    fields[:, 0] = rng.integers(0, 2, n)
+    fields[:, 1:8] = np.rint(rng.standard_normal((n, 7)) * 4).astype(np.int32)
+    fields[:, 8] = np.rint(rng.standard_normal(n) * 2).astype(np.int32)
+    blob = ep.pack_fields(fields, R, C, 11, C // 8, rng.uniform(0.01, 0.05, R).astype(np.float32))
+    _check(blob, T, R + C + T)
+
+
 def test_decode_matmul_more_tokens_than_one_launch_and_repeated_calls():
     W = synth.gaussian_rows(128, 1536, 71)
     blob = ep.encode(W, 4.0, tile_vectors=1536 // 8)
