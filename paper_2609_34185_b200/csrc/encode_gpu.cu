@@ -33,6 +33,12 @@ constexpr uint32_t kMaxTableSymbols = 40960;   // sum of K over the 17 tables th
 constexpr uint32_t kMaxEntries = 2 * kMaxTableSymbols + 2;     // the tile coder's entries (see EncodeTables)
 constexpr double kUnit = 1.1102230246251565e-16;   // 2^-53, the rounding unit of double
 
+// the wait of a kernel that is launched while the one before it ends (launch_chained): before it, only kernel parameters are read
+__device__ __forceinline__ void chained_start() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 // ---- sums over a row ------------------------------------------------------------------------------------
 // The row RMS (Sec. 3.2) and Eq. 13 are defined by sums in double in index order, a chain of dependent additions per
 // row (14 cycles each: 60 us for 8192 of them, whatever the bandwidth).  Here a CTA sums a row in parallel.
@@ -245,11 +251,12 @@ __device__ __forceinline__ bool quantise_fast(const float (&x)[8], float r, uint
 // the rate correction after it are one stream of launches with one wait at the end: the last CTA of a pass evaluates
 // Eq. 10-12 on the counts and leaves the next scale in device memory.
 //
-// A step of the bisection costs about 14 us whatever the sample (launch, clearing and flushing counters, the evaluation's
-// chain of dependent reads), and counting the sample only 4 us more.  So one launch takes three steps: seven scales
-// at once, the bracket's middle and the middles of the brackets that its two, then four, outcomes lead to, each counted
-// and evaluated by CTAs of its own; the last one to finish walks the tree.  (The first launches take one and two steps:
-// the outer candidates of a wide bracket are so fine - s = 0.003 - that all they count goes to global memory, 120 us.)
+// A step of the bisection costs about 12 us whatever the sample (launch, clearing and flushing counters, the evaluation's
+// chain of dependent reads), and counting 2^18 blocks of a sample only 4 us more.  So one launch takes several steps: for
+// three of them seven scales at once, the bracket's middle and the middles of the brackets that its two, then four,
+// outcomes lead to, each counted and evaluated by CTAs of its own; the last one to finish walks the tree.  (The first
+// launches take fewer steps: the outer candidates of a wide bracket are so fine - s = 0.003 - that all they count goes to
+// global memory, 120 us for 2^18 blocks.)  Steps per launch: 1, 2, 3, 3, 3; for samples up to 2^17 blocks 1, 3, 4, 4.
 //
 // Counting: nine increments per block, most of them of a few values around zero.  Each lane has its own column of
 // counters for those (bank = lane: no two lanes of a warp meet), values up to +-256 go to a plain window, the rest to
@@ -265,7 +272,7 @@ constexpr uint32_t kCountSmem = 4 * (kHotWords + kWinWords);
 constexpr uint32_t kEvalSymbols = 24576;
 static_assert(kEvalSymbols <= kHotWords + kWinWords, "evaluation space");
 constexpr uint32_t kFirstCounts = 6144;          // counts that come back with the state; more take a second copy
-constexpr uint32_t kLevels = 3, kCandidates = (1u << kLevels) - 1u;
+constexpr uint32_t kLevels = 4, kCandidates = (1u << kLevels) - 1u;
 
 struct CountDir { int32_t lo[EP_NUM_TABLES]; uint32_t K[EP_NUM_TABLES]; };
 
@@ -297,7 +304,7 @@ struct SearchState {
     uint32_t tiles_done;             //              CTAs of the launch that are done
     Candidate cand[kCandidates];
 };
-constexpr size_t kStateBytes = 6144;
+constexpr size_t kStateBytes = 8192;
 static_assert(sizeof(SearchState) <= kStateBytes, "state area");
 
 // the constants of Eq. 10-12
@@ -838,6 +845,7 @@ __device__ __forceinline__ uint4 encode_entry(uint32_t fF, uint32_t b) {
 
 __global__ void encode_entries_kernel(const uint32_t *__restrict__ fF, uint32_t n, uint32_t b, uint4 *__restrict__ entries) {
     const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+    chained_start();
     if (i < n) entries[i] = encode_entry(fF[i], b);
 }
 
@@ -887,6 +895,7 @@ __global__ void __launch_bounds__(kTileThreadsMax) tile_encode_kernel(const uint
     extern __shared__ __align__(16) uint4 entries_smem[];
     __shared__ uint32_t last_cta, part[kTileThreadsMax];
     const uint32_t tid = threadIdx.x, lane = tid & 31u;
+    chained_start();
     if (IN_SMEM) {
         for (uint32_t i = tid; i < T.total; i += blockDim.x) entries_smem[i] = __ldg(entries_global + i);
         __syncthreads();
@@ -954,16 +963,17 @@ __global__ void __launch_bounds__(kTileThreadsMax) tile_encode_kernel(const uint
     if (tid == blockDim.x - 1u) {
         index[size_t(n_tiles) * 33u] = part[tid];
         state->total_words = part[tid];
+        state->tiles_done = 0;
     }
 }
 
 // Move every tile's words from the end of its area to its place in the payload: one CTA per tile (with a warp per tile the
-// copy of 20 MB took 34 us, all of it waiting for loads), four bytes per lane, the destination aligned.
-constexpr uint32_t kCompactThreads = 128;
-__global__ void __launch_bounds__(kCompactThreads) compact_kernel(const uint16_t *__restrict__ scratch, uint32_t cap,
+// copy of 20 MB took 34 us, all of it waiting for loads; 19 so), four bytes per lane, the destination aligned.
+__global__ void __launch_bounds__(512) compact_kernel(const uint16_t *__restrict__ scratch, uint32_t cap,
                                                                   const uint32_t *__restrict__ counts, const uint32_t *__restrict__ index,
                                                                   uint16_t *__restrict__ payload) {
     const uint32_t tid = threadIdx.x, tile = blockIdx.x;
+    chained_start();
     uint32_t n = counts[tile];
     const uint16_t *src = scratch + size_t(tile) * cap + (cap - n);
     uint16_t *dst = payload + index[size_t(tile) * 33u + 32u];
@@ -977,11 +987,11 @@ __global__ void __launch_bounds__(kCompactThreads) compact_kernel(const uint16_t
         // each pair straddles two aligned words (the one before src starts inside the buffer, as src is not its start)
         const uint32_t *s32 = reinterpret_cast<const uint32_t *>(src - 1);
 #pragma unroll 4
-        for (uint32_t i = tid; i < pairs; i += kCompactThreads) d32[i] = __funnelshift_r(s32[i], s32[i + 1u], 16);
+        for (uint32_t i = tid; i < pairs; i += blockDim.x) d32[i] = __funnelshift_r(s32[i], s32[i + 1u], 16);
     } else {
         const uint32_t *s32 = reinterpret_cast<const uint32_t *>(src);
 #pragma unroll 4
-        for (uint32_t i = tid; i < pairs; i += kCompactThreads) d32[i] = s32[i];
+        for (uint32_t i = tid; i < pairs; i += blockDim.x) d32[i] = s32[i];
     }
     if ((n & 1u) && tid == 0) dst[n - 1u] = src[n - 1u];
 }
@@ -1124,7 +1134,8 @@ public:
         if (o.search_steps == 0) EP_CUDA(cudaMemcpyAsync(&w_.state->s, &s0, 4, cudaMemcpyHostToDevice, st_));
         P.first = 1;
         for (int left = o.search_steps, pass = 0; left > 0; ++pass) {
-            P.levels = uint32_t(std::min<int>(left, std::min<int>(pass + 1, kLevels)));
+            P.levels = uint32_t(std::min(left, n_sample_ * (C_ / 8) <= (1u << 17) ? (pass == 0 ? 1 : std::min<int>(pass + 2, kLevels))
+                                                                                  : std::min<int>(pass + 1, 3)));
             P.last_pass = left == int(P.levels);
             EP_CUDA(launch_count(P, pass > 0));
             left -= int(P.levels);
@@ -1198,20 +1209,19 @@ public:
         T.base[0] = 32u * size;                  // the coset's two entries last
         for (uint32_t j = 0; j < m.t[0].K(); ++j) fF[2u * size + uint32_t(m.t[0].lo) + j] = m.t[0].f[j] | (m.t[0].F[j] << 16);
         EP_CUDA(cudaMemcpyAsync(w_.fF, fF.data(), 4ull * fF.size(), cudaMemcpyHostToDevice, st_));
-        EP_CUDA(cudaMemsetAsync(&w_.state->tiles_done, 0, 4, st_));
-        encode_entries_kernel<<<(T.total + 127u) / 128u, 128, 0, st_>>>(w_.fF, T.total, uint32_t(b), w_.entries);
+        EP_CUDA(launch_chained(encode_entries_kernel, (T.total + 127u) / 128u, 128, 0, w_.fF, T.total, uint32_t(b), w_.entries));
         if (T.total <= kSmemEntries) {
             const size_t smem = 16ull * T.total;
             const uint32_t threads = T.total <= 2048u ? kTileThreads : kTileThreadsMax;
             if (smem > 40u * 1024u)      // (always the same limit: another thread's call must not lower it before the launch)
                 EP_CUDA(cudaFuncSetAttribute(tile_encode_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(16u * kSmemEntries)));
-            tile_encode_kernel<true><<<(n_tiles + threads / 32u - 1u) / (threads / 32u), threads, smem, st_>>>(
-                w_.fields, uint32_t(nvec), V, n_tiles, T, w_.entries, w_.scratch, cap, w_.index, w_.counts, w_.state);
+            EP_CUDA(launch_chained(tile_encode_kernel<true>, (n_tiles + threads / 32u - 1u) / (threads / 32u), threads, smem, w_.fields, uint32_t(nvec), V,
+                                   n_tiles, T, w_.entries, w_.scratch, cap, w_.index, w_.counts, w_.state));
         } else {
-            tile_encode_kernel<false><<<(n_tiles + kTileThreads / 32u - 1u) / (kTileThreads / 32u), kTileThreads, 0, st_>>>(
-                w_.fields, uint32_t(nvec), V, n_tiles, T, w_.entries, w_.scratch, cap, w_.index, w_.counts, w_.state);
+            EP_CUDA(launch_chained(tile_encode_kernel<false>, (n_tiles + kTileThreads / 32u - 1u) / (kTileThreads / 32u), kTileThreads, 0, w_.fields,
+                                   uint32_t(nvec), V, n_tiles, T, w_.entries, w_.scratch, cap, w_.index, w_.counts, w_.state));
         }
-        compact_kernel<<<n_tiles, kCompactThreads, 0, st_>>>(w_.scratch, cap, w_.counts, w_.index, w_.payload);
+        EP_CUDA(launch_chained(compact_kernel, n_tiles, n_tiles < 600u ? 512u : 128u, 0, w_.scratch, cap, w_.counts, w_.index, w_.payload));
         EP_CUDA(cudaMemcpyAsync(&state()->total_words, &w_.state->total_words, 4, cudaMemcpyDeviceToHost, st_));
         if (!sigma_there_ || sigma_of_ != s) refit_kernel<<<R_, kRowThreads, 0, st_>>>(W_, C_, w_.fields, s, nullptr, w_.mu, w_.sigma);
         EP_CUDA(cudaGetLastError());
@@ -1275,6 +1285,21 @@ private:
                 8.0 * double(n), 9.0 * double(n), b};
     }
     // one CTA per SM over all candidates of the pass, each with at least a few hundred blocks
+    // launched while the kernel before it ends; the kernel waits on the device (chained_start)
+    template <class... K, class... A>
+    cudaError_t launch_chained(void (*kernel)(K...), uint32_t grid, uint32_t threads, size_t smem, A... args) {
+        cudaLaunchAttribute attr{};
+        attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr.val.programmaticStreamSerializationAllowed = 1;
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3(grid);
+        cfg.blockDim = dim3(threads);
+        cfg.dynamicSmemBytes = smem;
+        cfg.stream = st_;
+        cfg.attrs = &attr;
+        cfg.numAttrs = 1;
+        return cudaLaunchKernelEx(&cfg, kernel, K(args)...);
+    }
     cudaError_t launch_count(CountParams P, bool follows) {
         const uint32_t cands = (1u << P.levels) - 1u;
         P.ctas = std::max(1u, std::min((P.n_blocks + 255u) / 256u, uint32_t(sms_) / cands));
