@@ -853,10 +853,10 @@ __global__ void encode_entries_kernel(const uint32_t *__restrict__ fF, uint32_t 
 // ascending lane order; the encoder walks groups and fields backwards and fills the tile's word area from its end, writing
 // each step's words as one block in ascending lane order, which is the order the reversed word list of a sequential
 // encoder would have.  A step's chain is compare, shift, multiply-high, shift, multiply-add (about 30 cycles);
-// a group's fields are loaded four groups ahead and its symbols looked up before the steps that need them.
-// IN_SMEM: the symbols' entries in shared memory (up to 12 Ki symbols), else in global memory.  A CTA has four warps -
+// a group's fields are asked for four groups ahead and its symbols looked up before the steps that need them.
+// IN_SMEM: the symbols' entries in shared memory (up to 11 Ki symbols), else in global memory.  A CTA has four warps -
 // tiles spread over the SMs - or sixteen where its table takes so much shared memory that few CTAs fit an SM.
-constexpr uint32_t kTileThreads = 128, kTileThreadsMax = 512, kSmemEntries = 12288;
+constexpr uint32_t kTileThreads = 128, kTileThreadsMax = 512, kSmemEntries = 11264, kAhead = 4;
 
 // A group's nine steps.  A step's words are stored during the next one: ballot, population counts and address (some 60 cycles)
 // stay off the chain of states, and the store is predicated, not a branch.  P / Q: this and the previous step's
@@ -901,7 +901,8 @@ __global__ void __launch_bounds__(kTileThreadsMax) tile_encode_kernel(const uint
         __syncthreads();
     }
     const uint32_t entries = IN_SMEM ? uint32_t(__cvta_generic_to_shared(entries_smem)) : 0u;
-    const uint32_t tile = blockIdx.x * (blockDim.x >> 5) + (tid >> 5);
+    // (the warp's number by a shuffle: known to be warp-uniform, so no guard around the votes)
+    const uint32_t tile = blockIdx.x * (blockDim.x >> 5) + __shfl_sync(0xFFFFFFFFu, tid >> 5, 0);
     if (tile < n_tiles) {
         const uint32_t v0 = tile * V, nv = min(V, n_vec - v0), lt = (1u << lane) - 1u;
         const uint4 *const q = fields + v0;
@@ -909,17 +910,21 @@ __global__ void __launch_bounds__(kTileThreadsMax) tile_encode_kernel(const uint
         uint32_t end = cap;                      // words [end, cap) of the area are written
         uint32_t x = kStateLow;
         const uint32_t groups = (nv + 31u) >> 5;
-        // fields of the next groups: a group takes 0.4 us, a load from DRAM over 1 us
-        constexpr uint32_t kAhead = 4;
-        uint4 next[kAhead];
-#pragma unroll
-        for (uint32_t i = 0; i < kAhead; ++i)
-            next[i] = groups > i ? __ldg(q + min((groups - 1u - i) * 32u + lane, nv - 1u)) : make_uint4(0u, 0u, 0u, 0u);
+        // Fields of the next groups on their way to shared memory, every lane its own 16 bytes: a group takes 0.2 us, a load
+        // from L2 0.4.  (Loads into registers some groups ahead are waited for all together, the newest with the one
+        // that is needed: 0.5 us per group.)
+        const uint32_t staged = uint32_t(__cvta_generic_to_shared(entries_smem)) + (IN_SMEM ? 16u * T.total : 0u) + (tid >> 5) * (kAhead * 512u) + 16u * lane;
+        auto ask = [&](uint32_t g) {             // group g, if there is one
+            if (g < groups)
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(staged + (g % kAhead) * 512u), "l"(q + min(g * 32u + lane, nv - 1u)) : "memory");
+            asm volatile("cp.async.commit_group;" ::: "memory");
+        };
+        for (uint32_t i = 0; i < kAhead; ++i) ask(groups - 1u - i);
         for (uint32_t g = groups; g-- > 0;) {
-            const uint4 cur = next[0];
-#pragma unroll
-            for (uint32_t i = 0; i + 1u < kAhead; ++i) next[i] = next[i + 1u];
-            if (g >= kAhead) next[kAhead - 1u] = __ldg(q + (g - kAhead) * 32u + lane);
+            uint4 cur;
+            asm volatile("cp.async.wait_group %0;" ::"n"(kAhead - 1u) : "memory");
+            asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(cur.x), "=r"(cur.y), "=r"(cur.z), "=r"(cur.w) : "r"(staged + (g % kAhead) * 512u) : "memory");
+            ask(g - kAhead);                     // (past the first group: none, the number wraps)
             const int32_t mc = field16(cur.w, 1);
             const uint32_t w[4] = {cur.x, cur.y, cur.z, cur.w}, coset = (mc & 1) ? entries + T.coset : entries;
             uint32_t at[9];                      // (every offset is in range: these are the fields the tables were counted from)
@@ -936,6 +941,7 @@ __global__ void __launch_bounds__(kTileThreadsMax) tile_encode_kernel(const uint
                               e0 + at[1], e0 + at[0]);
             }
         }
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
         index[size_t(tile) * 33u + lane] = x;
         if (lane == 0) counts[tile] = cap - end;
     }
@@ -1211,14 +1217,15 @@ public:
         EP_CUDA(cudaMemcpyAsync(w_.fF, fF.data(), 4ull * fF.size(), cudaMemcpyHostToDevice, st_));
         EP_CUDA(launch_chained(encode_entries_kernel, (T.total + 127u) / 128u, 128, 0, w_.fF, T.total, uint32_t(b), w_.entries));
         if (T.total <= kSmemEntries) {
-            const size_t smem = 16ull * T.total;
-            const uint32_t threads = T.total <= 2048u ? kTileThreads : kTileThreadsMax;
+                        const uint32_t threads = T.total <= 2048u ? kTileThreads : kTileThreadsMax;
+            const size_t smem = 16ull * T.total + threads / 32u * (kAhead * 512u);
             if (smem > 40u * 1024u)      // (always the same limit: another thread's call must not lower it before the launch)
-                EP_CUDA(cudaFuncSetAttribute(tile_encode_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(16u * kSmemEntries)));
+                EP_CUDA(cudaFuncSetAttribute(tile_encode_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(16u * kSmemEntries + kTileThreadsMax / 32u * (kAhead * 512u))));
             EP_CUDA(launch_chained(tile_encode_kernel<true>, (n_tiles + threads / 32u - 1u) / (threads / 32u), threads, smem, w_.fields, uint32_t(nvec), V,
                                    n_tiles, T, w_.entries, w_.scratch, cap, w_.index, w_.counts, w_.state));
         } else {
-            EP_CUDA(launch_chained(tile_encode_kernel<false>, (n_tiles + kTileThreads / 32u - 1u) / (kTileThreads / 32u), kTileThreads, 0, w_.fields,
+            EP_CUDA(launch_chained(tile_encode_kernel<false>, (n_tiles + kTileThreads / 32u - 1u) / (kTileThreads / 32u), kTileThreads,
+                                   kTileThreads / 32u * (kAhead * 512u), w_.fields,
                                    uint32_t(nvec), V, n_tiles, T, w_.entries, w_.scratch, cap, w_.index, w_.counts, w_.state));
         }
         EP_CUDA(launch_chained(compact_kernel, n_tiles, n_tiles < 600u ? 512u : 128u, 0, w_.scratch, cap, w_.counts, w_.index, w_.payload));
