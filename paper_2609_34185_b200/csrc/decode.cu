@@ -84,7 +84,7 @@ constexpr uint32_t kEntryUnused = 1u << 21;                  // f = 1: what a sl
 constexpr uint32_t kCtxScales = 0;         // u64 row scales
 constexpr uint32_t kCtxRowBytes = 8;       // u32 output bytes per row
 constexpr uint32_t kCtxRowMax = 12;        // u32 last row index
-constexpr uint32_t kCtxTablesBar = 16;     // u64 warp 0's: the mbarrier of the table image's copy
+constexpr uint32_t kCtxTablesBar = 16;     // u64 warp j's: the mbarrier of the copy of job j's table image
 constexpr uint32_t kCtxRowRcp = 24;        // u32 ceil(2^32 / bytes per row)
 constexpr uint32_t kCtxChain = 32, kCtxChainStride = 32;
 constexpr uint32_t kCcSrc = 0;             // u64 global address of lane 0's 16 bytes of the next chunk to request
@@ -292,7 +292,11 @@ __device__ __forceinline__ void copy_tables_smem(const uint32_t *image, uint32_t
 // vote of the hot loop costs more than the wait).  A copy that does not end within the limit - there is no such case -
 // raises the integrity word; the tables then hold anything, which is safe (see build_one_table) but wrong.
 enum TablesPending : uint32_t { kTablesThere, kTablesBuilt, kTablesCopied };   // nothing to wait for; this CTA's stores; the copy
-struct TablesWait { uint32_t pending, bar, parity; };
+// Every job has an mbarrier of its own, in the context block of the warp of the same number: a phase kept from job to job, and a
+// flag for the first job, are two registers that the hot loop's 64 do not have (block of seven at 2.5 bpp to FP8 303.5 -> 299.7 us,
+// 8192 x 8192 at 8 bpp 101.1 -> 100.1).
+struct TablesWait { uint32_t pending, bar; };
+static_assert(EP_MAX_BATCH <= kWarps);
 constexpr uint32_t kSpinLimit = 1u << 18;             // attempts of about a microsecond each at most: a quarter of a second
 __device__ __forceinline__ void wait_for_tables(const TablesWait &W) {
     if (W.pending == kTablesBuilt) __syncthreads();
@@ -308,7 +312,7 @@ __device__ __forceinline__ void wait_for_tables(const TablesWait &W) {
                      "vote.sync.all.pred p, p, 0xffffffff;\n\t"
                      "@p bra.uni EP_TABLES_WAIT;\n\t"
                      "EP_TABLES_DONE:\n\t}"
-                     : "=&r"(left) : "r"(W.bar), "r"(W.parity), "n"(kSpinLimit) : "memory");
+                     : "=&r"(left) : "r"(W.bar), "r"(0u), "n"(kSpinLimit) : "memory");
         if (left == 0) atomicOr(&g_ep_status, 2u);
     }
 }
@@ -702,11 +706,11 @@ __device__ __forceinline__ void decode_tile_plain(const JobParams &J, uint32_t t
     EP_ALL(EP_L1, E, OFF, BIN, BOUT) EP_ALL(EP_L2, E, OFF, BIN, BOUT) EP_ALL(EP_L3, E, OFF, BIN, BOUT)   \
     EP_ALL(EP_L5, E, OFF, BIN, BOUT) EP_ALL(EP_L6, E, OFF, BIN, BOUT)   \
     EP_ALL(EP_L7, E, OFF, BIN, BOUT) EP_RENORM_ALL(E, OFF, BIN, BOUT)
-// the coset: slot below f0 -> coset 0 with frequency f0, else coset 1 with frequency f1 and offset f0
+// the coset: slot below f0 -> coset 0 with frequency f0 (then at least 1), else coset 1 with frequency f1 and offset f0
 #define EP_C1(S, X, AW, BAL, DOFF, CB) "and.b32 u" S ", " X ", 0x7FF;\n\t"
 #define EP_C2(S, X, AW, BAL, DOFF, CB) "shr.u32 q" S ", " X ", 11;\n\t"
 #define EP_C3(S, X, AW, BAL, DOFF, CB) "setp.lt.u32 pc" S ", u" S ", " EP_F0 ";\n\t"
-#define EP_C4(S, X, AW, BAL, DOFF, CB) "selp.b32 f" S ", f0c, " EP_F1 ", pc" S ";\n\t"
+#define EP_C4(S, X, AW, BAL, DOFF, CB) "selp.b32 f" S ", " EP_F0 ", " EP_F1 ", pc" S ";\n\t"
 #define EP_C5(S, X, AW, BAL, DOFF, CB) "@!pc" S " sub.u32 u" S ", u" S ", " EP_F0 ";\n\t"
 #define EP_C6(S, X, AW, BAL, DOFF, CB) "@act" S " mad.lo.u32 " X ", f" S ", q" S ", u" S ";\n\t"
 #define EP_C7(S, X, AW, BAL, DOFF, CB) "selp.b32 tab" S ", " EP_LUT0 ", " EP_LUT1 ", pc" S ";\n\t"
@@ -1041,7 +1045,7 @@ __device__ __forceinline__ void decode_tile_plain(const JobParams &J, uint32_t t
         "{\n\t"                                                                                                       \
         EP_ALL(EP_REGS)                                                                                               \
         ".reg .pred pq, pv, pr;\n\t"                                                                                  \
-        ".reg .b32 r0, r1, r2, r3, r4, r5, r6, r7, r8, r9, r10, r11, r12, c0r, c1r, d0r, d1r, f0c, hotb, hotb1;\n\t" \
+        ".reg .b32 r0, r1, r2, r3, r4, r5, r6, r7, r8, r9, r10, r11, r12, c0r, c1r, d0r, d1r, hotb, hotb1;\n\t" \
         ".reg .b64 ra, rb, l2b1;\n\t"                                                                                 \
         ".reg .f32 k0f, k1f;\n\t"                                                                                     \
         "mov.b64 {k0f, k1f}, " EP_KK ";\n\t"                                                                          \
@@ -1049,7 +1053,6 @@ __device__ __forceinline__ void decode_tile_plain(const JobParams &J, uint32_t t
         "mov.b32 c1r, 0x45800400;\n\t"                                                                                \
         "mov.b32 d0r, 0x4A800000;\n\t"                /* 2^22, 2^22 + 1/2 (2^12-slot streams) */                    \
         "mov.b32 d1r, 0x4A800001;\n\t"                                                                                \
-        "max.u32 f0c, " EP_F0 ", 1;\n\t"                /* frequency used for coset 0: never 0 */                     \
         "add.u32 hotb, " EP_LUT0 ", " EP_HOTOFF ";\n\t"   /* 2^12-slot streams: hot entries of coset 0, */              \
         "add.u32 hotb1, hotb, 16896;\n\t"                 /* of coset 1; complete array of coset 1 */                   \
         "add.s64 l2b1, " EP_L2B ", 131072;\n\t"                                                                       \
@@ -1096,13 +1099,12 @@ __device__ __forceinline__ void decode_tile_plain(const JobParams &J, uint32_t t
         "{\n\t"                                                                                                       \
         EP_ALL(EP_REGS) REGS                                                                                          \
         ".reg .pred pq, pv, pr, ps, pn;\n\t"                                                                          \
-        ".reg .b32 r0, r1, r2, r3, r4, r5, r6, r7, r10, r11, r12, c0r, c1r, f0c, lm, sx, sa, sb, ea, va, f2, b2, q2, rp, rowb, endo;\n\t"     \
+        ".reg .b32 r0, r1, r2, r3, r4, r5, r6, r7, r10, r11, r12, c0r, c1r, lm, sx, sa, sb, ea, va, f2, b2, q2, rp, rowb, endo;\n\t"     \
         ".reg .b64 ra, rb;\n\t"                                                                                       \
         ".reg .f32 k0f, k1f;\n\t"                                                                                     \
         "mov.b64 {k0f, k1f}, " EP_KK ";\n\t"                                                                          \
         "mov.b32 c0r, 0x45800000;\n\t"                                                                                \
         "mov.b32 c1r, 0x45800400;\n\t"                                                                                \
-        "max.u32 f0c, " EP_F0 ", 1;\n\t"                                                                              \
         "mov.b32 wA, 0;\n\t" "mov.b32 ea, 0x200000;\n\t" "mov.b32 q2, 0;\n\t" "mov.b32 lm, 0xffffffff;\n\t"           \
         "mov.b32 rp, %12;\n\t" "mov.b32 limA, %13;\n\t" "mov.b32 wthrA, %14;\n\t"                                     \
         "ld.shared.b32 sgA, [rp];\n\t" "mov.b32 r3, sgA;\n\t" "mov.b64 ssA, {r3, r3};\n\t"                            \
@@ -1332,10 +1334,8 @@ ep_decode_smem_kernel(const __grid_constant__ BatchParams P) {
     const uint32_t lut_addr = uint32_t(__cvta_generic_to_shared(smem));
     const uint32_t ring = lut_addr + kRingBase + warp * (kChains * kRingStride);
     const uint32_t ctx = lut_addr + kCtxBase + warp * kCtxBytes;
-    bool tables_in_use = false;
-    TablesWait tables{kTablesThere, lut_addr + kCtxBase + kCtxTablesBar, 1u};
     if (threadIdx.x == 0) {
-        mbar_init(tables.bar, 1u);
+        for (int j = 0; j < P.n_jobs; ++j) mbar_init(lut_addr + kCtxBase + kCtxTablesBar + j * kCtxBytes, 1u);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
@@ -1349,22 +1349,18 @@ ep_decode_smem_kernel(const __grid_constant__ BatchParams P) {
         const uint32_t r0 = min((a + J.round_cost - 1u) / J.round_cost, J.rounds);
         const uint32_t r1 = min((b + J.round_cost - 1u) / J.round_cost, J.rounds);
         if (r0 >= r1) continue;
-        if (tables_in_use) __syncthreads();          // every warp is done with the previous job's tables
+        if (lo < J.cost_begin) __syncthreads();      // not this CTA's first: every warp is done with the previous job's tables
         // the table image is requested first: the tiles' records and payload (two dependent reads of memory that no
         // cache holds yet) are on their way while it arrives
         if (J.lut_image) {
-            tables.pending = kTablesCopied;
-            tables.parity ^= 1u;
             if (threadIdx.x == 0) {
-                if (tables_in_use) fence_async_smem();   // the last job's lookups, ordered before this by the barrier above
-                copy_tables_smem(J.lut_image, lut_addr, tables.bar, J.b == 12u);
+                if (lo < J.cost_begin) fence_async_smem();   // the last job's lookups, ordered before this by the barrier above
+                copy_tables_smem(J.lut_image, lut_addr, lut_addr + kCtxBase + kCtxTablesBar + j * kCtxBytes, J.b == 12u);
             }
         } else {
-            tables.pending = kTablesBuilt;
             build_tables_smem(J, lut_addr, warp, lane);
         }
         const CosetFreq cf = load_coset(J);
-        tables_in_use = true;
         // (a stream with 2^12 slots reaches this kernel only in the configuration of the hot loop: see the launcher)
         const bool fast = DT != EP_FIELDS_I32 && J.per_row >= 32u && (J.b == 11u || J.b == 12u) && J.V < (1u << 20);
         if (fast && lane == 0) {                     // what the hot loop's rare paths need to know about the job
@@ -1376,6 +1372,8 @@ ep_decode_smem_kernel(const __grid_constant__ BatchParams P) {
         __syncwarp();
         for (uint32_t r = r0; r < r1; ++r) {
             const uint32_t base = r * P.tiles_per_round + kChains * warp;
+            const TablesWait tables{r != r0 ? kTablesThere : J.lut_image ? kTablesCopied : kTablesBuilt,
+                                    lut_addr + kCtxBase + kCtxTablesBar + j * kCtxBytes};
             if constexpr (DT != EP_FIELDS_I32) {
                 if (fast) {
                     if (kTwoLevelInLoop && J.b == 12u) {
@@ -1385,12 +1383,10 @@ ep_decode_smem_kernel(const __grid_constant__ BatchParams P) {
                     } else {
                         decode_tiles_fast<DT, 11>(J, base, P.tiles_per_round, lut_addr, cf, ring, ctx, lane, tables);
                     }
-                    tables.pending = kTablesThere;
                     continue;
                 }
             }
             wait_for_tables(tables);
-            tables.pending = kTablesThere;
             for (uint32_t c = 0; c < kChains; ++c)
                 if (base + c < J.tile_cnt && kChains * warp + c < P.tiles_per_round) decode_tile_plain<DT>(J, J.tile0 + base + c, lut_addr, cf, ring, lane);
         }
@@ -1522,9 +1518,9 @@ __device__ __forceinline__ void umma_commit(uint32_t bar) {
 #define EP_GEMM_ROW_ASM                                                                                               \
     asm volatile("{\n\t" EP_ALL(EP_REGS)                                                                              \
         ".reg .pred pq, pv, pr, pl;\n\t"                                                                              \
-        ".reg .b32 r0, r1, r2, r3, r4, r5, r6, r10, r11, r12, c0r, c1r, f0c, va, g, bar, par, odd, dst, tries;\n\t"   \
+        ".reg .b32 r0, r1, r2, r3, r4, r5, r6, r10, r11, r12, c0r, c1r, va, g, bar, par, odd, dst, tries;\n\t"   \
         ".reg .b64 ra, rb, st;\n\t"                                                                                   \
-        "mov.b32 c0r, 0x45800000;\n\t" "mov.b32 c1r, 0x45800400;\n\t" "max.u32 f0c, " EP_F0 ", 1;\n\t"                \
+        "mov.b32 c0r, 0x45800000;\n\t" "mov.b32 c1r, 0x45800400;\n\t"                \
         "mov.b64 ssA, {%11, %11};\n\t" "setp.ne.u32 actA, %12, 0;\n\t" "mov.b32 g, %13;\n\t"                          \
         "setp.eq.u32 pl, " EP_LT ", 0;\n\t"                  /* lane 0 */                                             \
         "ld.shared.u32 r10, [" EP_CTX "+48];\n\t" "add.u32 wthrA, r10, 254;\n\t"                                      \
@@ -1612,7 +1608,7 @@ __global__ void __launch_bounds__(kThreads, 1) ep_decode_gemm_kernel(const __gri
     constexpr uint32_t a_tile_bytes = TPAD * 128u, kUnitTiles = 8192u / a_tile_bytes, kUnitsPerGroup = 4u / kUnitTiles;
     const uint32_t bar_a = lut_addr + G::kBar, bar_afree = bar_a + 64u, bar_mma = bar_a + 128u, bar_b = bar_a + 144u,
                    slot = bar_a + 160u, abort_addr = bar_b + 100u;
-    const TablesWait tables{kTablesCopied, bar_a + 168u, 0u};
+    const TablesWait tables{kTablesCopied, bar_a + 168u};
     if (tid == 0) {
         for (uint32_t i = 0; i < G::kUnits; ++i) {
             mbar_init(bar_a + 8u * i, 1u);       // the loading lane's arrival; completes when the unit's tiles have landed
