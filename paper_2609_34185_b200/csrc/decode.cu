@@ -84,7 +84,7 @@ constexpr uint32_t kEntryUnused = 1u << 21;                  // f = 1: what a sl
 constexpr uint32_t kCtxScales = 0;         // u64 row scales
 constexpr uint32_t kCtxRowBytes = 8;       // u32 output bytes per row
 constexpr uint32_t kCtxRowMax = 12;        // u32 last row index
-constexpr uint32_t kCtxTablesBar = 16;     // u64 warp j's: the mbarrier of the copy of job j's table image
+constexpr uint32_t kCtxTablesBar = 16;     // u64 mbarrier of the table image's copy (warp j's: of job j's, see ep_decode_smem_kernel)
 constexpr uint32_t kCtxRowRcp = 24;        // u32 ceil(2^32 / bytes per row)
 constexpr uint32_t kCtxChain = 32, kCtxChainStride = 32;
 constexpr uint32_t kCcSrc = 0;             // u64 global address of lane 0's 16 bytes of the next chunk to request
@@ -292,10 +292,7 @@ __device__ __forceinline__ void copy_tables_smem(const uint32_t *image, uint32_t
 // vote of the hot loop costs more than the wait).  A copy that does not end within the limit - there is no such case -
 // raises the integrity word; the tables then hold anything, which is safe (see build_one_table) but wrong.
 enum TablesPending : uint32_t { kTablesThere, kTablesBuilt, kTablesCopied };   // nothing to wait for; this CTA's stores; the copy
-// Every job has an mbarrier of its own, in the context block of the warp of the same number: a phase kept from job to job, and a
-// flag for the first job, are two registers that the hot loop's 64 do not have (block of seven at 2.5 bpp to FP8 303.5 -> 299.7 us,
-// 8192 x 8192 at 8 bpp 101.1 -> 100.1).
-struct TablesWait { uint32_t pending, bar; };
+struct TablesWait { uint32_t pending, bar, parity; };
 static_assert(EP_MAX_BATCH <= kWarps);
 constexpr uint32_t kSpinLimit = 1u << 18;             // attempts of about a microsecond each at most: a quarter of a second
 __device__ __forceinline__ void wait_for_tables(const TablesWait &W) {
@@ -312,7 +309,7 @@ __device__ __forceinline__ void wait_for_tables(const TablesWait &W) {
                      "vote.sync.all.pred p, p, 0xffffffff;\n\t"
                      "@p bra.uni EP_TABLES_WAIT;\n\t"
                      "EP_TABLES_DONE:\n\t}"
-                     : "=&r"(left) : "r"(W.bar), "r"(0u), "n"(kSpinLimit) : "memory");
+                     : "=&r"(left) : "r"(W.bar), "r"(W.parity), "n"(kSpinLimit) : "memory");
         if (left == 0) atomicOr(&g_ep_status, 2u);
     }
 }
@@ -1334,8 +1331,13 @@ ep_decode_smem_kernel(const __grid_constant__ BatchParams P) {
     const uint32_t lut_addr = uint32_t(__cvta_generic_to_shared(smem));
     const uint32_t ring = lut_addr + kRingBase + warp * (kChains * kRingStride);
     const uint32_t ctx = lut_addr + kCtxBase + warp * kCtxBytes;
+    // The hot loop's 64 registers have no room for a phase and a flag kept from job to job, so there every job has an mbarrier of its
+    // own (block of seven at 2.5 bpp to FP8 303.5 -> 299.7 us, 8192 x 8192 at 8 bpp 101.1 -> 100.1).  With few tiles per CTA one
+    // mbarrier and its phase are the faster way (4096 x 4096 at 3 bpp 38.4 us, 39.1 with one per job).
+    bool tables_in_use = false;
+    TablesWait tables{kTablesThere, lut_addr + kCtxBase + kCtxTablesBar, FEW ? 1u : 0u};
     if (threadIdx.x == 0) {
-        for (int j = 0; j < P.n_jobs; ++j) mbar_init(lut_addr + kCtxBase + kCtxTablesBar + j * kCtxBytes, 1u);
+        for (int j = 0; j < (FEW ? 1 : P.n_jobs); ++j) mbar_init(lut_addr + kCtxBase + kCtxTablesBar + j * kCtxBytes, 1u);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
@@ -1349,18 +1351,24 @@ ep_decode_smem_kernel(const __grid_constant__ BatchParams P) {
         const uint32_t r0 = min((a + J.round_cost - 1u) / J.round_cost, J.rounds);
         const uint32_t r1 = min((b + J.round_cost - 1u) / J.round_cost, J.rounds);
         if (r0 >= r1) continue;
-        if (lo < J.cost_begin) __syncthreads();      // not this CTA's first: every warp is done with the previous job's tables
+        const bool again = FEW ? tables_in_use : lo < J.cost_begin;     // (may also be set for a CTA's first job there)
+        if (again) __syncthreads();                  // every warp is done with the previous job's tables
         // the table image is requested first: the tiles' records and payload (two dependent reads of memory that no
         // cache holds yet) are on their way while it arrives
         if (J.lut_image) {
+            tables.pending = kTablesCopied;
+            if constexpr (FEW) tables.parity ^= 1u;
+            else tables.bar = lut_addr + kCtxBase + kCtxTablesBar + j * kCtxBytes;
             if (threadIdx.x == 0) {
-                if (lo < J.cost_begin) fence_async_smem();   // the last job's lookups, ordered before this by the barrier above
-                copy_tables_smem(J.lut_image, lut_addr, lut_addr + kCtxBase + kCtxTablesBar + j * kCtxBytes, J.b == 12u);
+                if (again) fence_async_smem();           // the last job's lookups, ordered before this by the barrier above
+                copy_tables_smem(J.lut_image, lut_addr, tables.bar, J.b == 12u);
             }
         } else {
+            tables.pending = kTablesBuilt;
             build_tables_smem(J, lut_addr, warp, lane);
         }
         const CosetFreq cf = load_coset(J);
+        tables_in_use = true;
         // (a stream with 2^12 slots reaches this kernel only in the configuration of the hot loop: see the launcher)
         const bool fast = DT != EP_FIELDS_I32 && J.per_row >= 32u && (J.b == 11u || J.b == 12u) && J.V < (1u << 20);
         if (fast && lane == 0) {                     // what the hot loop's rare paths need to know about the job
@@ -1372,8 +1380,6 @@ ep_decode_smem_kernel(const __grid_constant__ BatchParams P) {
         __syncwarp();
         for (uint32_t r = r0; r < r1; ++r) {
             const uint32_t base = r * P.tiles_per_round + kChains * warp;
-            const TablesWait tables{r != r0 ? kTablesThere : J.lut_image ? kTablesCopied : kTablesBuilt,
-                                    lut_addr + kCtxBase + kCtxTablesBar + j * kCtxBytes};
             if constexpr (DT != EP_FIELDS_I32) {
                 if (fast) {
                     if (kTwoLevelInLoop && J.b == 12u) {
@@ -1383,10 +1389,12 @@ ep_decode_smem_kernel(const __grid_constant__ BatchParams P) {
                     } else {
                         decode_tiles_fast<DT, 11>(J, base, P.tiles_per_round, lut_addr, cf, ring, ctx, lane, tables);
                     }
+                    tables.pending = kTablesThere;
                     continue;
                 }
             }
             wait_for_tables(tables);
+            tables.pending = kTablesThere;
             for (uint32_t c = 0; c < kChains; ++c)
                 if (base + c < J.tile_cnt && kChains * warp + c < P.tiles_per_round) decode_tile_plain<DT>(J, J.tile0 + base + c, lut_addr, cf, ring, lane);
         }
@@ -1608,7 +1616,7 @@ __global__ void __launch_bounds__(kThreads, 1) ep_decode_gemm_kernel(const __gri
     constexpr uint32_t a_tile_bytes = TPAD * 128u, kUnitTiles = 8192u / a_tile_bytes, kUnitsPerGroup = 4u / kUnitTiles;
     const uint32_t bar_a = lut_addr + G::kBar, bar_afree = bar_a + 64u, bar_mma = bar_a + 128u, bar_b = bar_a + 144u,
                    slot = bar_a + 160u, abort_addr = bar_b + 100u;
-    const TablesWait tables{kTablesCopied, bar_a + 168u};
+    const TablesWait tables{kTablesCopied, bar_a + 168u, 0u};
     if (tid == 0) {
         for (uint32_t i = 0; i < G::kUnits; ++i) {
             mbar_init(bar_a + 8u * i, 1u);       // the loading lane's arrival; completes when the unit's tiles have landed
