@@ -264,13 +264,13 @@ __device__ __forceinline__ bool quantise_fast(const float (&x)[8], float r, uint
 constexpr uint32_t kCountThreads = 1024;
 constexpr int kHotBins = 32, kHotOrigin = -16;   // values with a counter column per lane, per coordinate table
 constexpr uint32_t kHotStride = (kHotBins + 1) * 32;   // words per table: one more row takes what lies outside
-constexpr int kWinBins = 512, kWinOrigin = -256; // values with one counter per CTA, per table
+constexpr int kWinBins = 512, kWinOrigin = -256; // values with one counter per CTA, per table (2048 of them gain nothing at 8 bpp either)
 constexpr uint32_t kHotWords = 16 * kHotStride, kWinWords = EP_NUM_TABLES * kWinBins;
-constexpr uint32_t kCountSmem = 4 * (kHotWords + kWinWords);
-// symbols over all tables that an evaluation holds in shared memory (it reuses the counters' space); with more of
-// them the host takes over
-constexpr uint32_t kEvalSymbols = 24576;
-static_assert(kEvalSymbols <= kHotWords + kWinWords, "evaluation space");
+// symbols over all tables that an evaluation holds in shared memory (it reuses the counters' space): more than a finished stream
+// may have.  A finer scale of the search with more of them is judged by the counts' entropy (see judge_candidate).
+constexpr uint32_t kEvalSymbols = 49152;
+static_assert(kEvalSymbols >= kHotWords + kWinWords && kEvalSymbols >= kMaxTableSymbols, "evaluation space");
+constexpr uint32_t kCountSmem = 4 * kEvalSymbols;
 constexpr uint32_t kFirstCounts = 6144;          // counts that come back with the state; more take a second copy
 constexpr uint32_t kLevels = 4, kCandidates = (1u << kLevels) - 1u;
 
@@ -285,8 +285,8 @@ struct Candidate {
     uint32_t overflow;               // a coordinate left the histogram range
     uint32_t verdict;                // kValid ...
 };
-// a b-bit table exists; the rate lies above the target; too close to say
-constexpr uint32_t kValid = 1, kAbove = 2, kUndecided = 4, kOverflow = 8;
+// a b-bit table exists; the rate lies above the target; too close to say; ...; a table exists, but the counts were not kept
+constexpr uint32_t kValid = 1, kAbove = 2, kUndecided = 4, kOverflow = 8, kNoCounts = 16;
 // what the passes leave for one another and for the host (device memory, zeroed before a search)
 struct SearchState {
     double lo, hi;                   // the bracket
@@ -403,6 +403,13 @@ __device__ __forceinline__ Evaluation gather_counts(const CountParams &P, uint32
         uint32_t *h = P.hist + (k * EP_NUM_TABLES + t) * kHistBins + (lo_of[t] - kHistOrigin);
         unsigned long long sum = 0;
         uint32_t seen = 0;
+        double nlogn = 0.0;
+        if (E.too_many && evaluate)
+#pragma unroll 4
+            for (uint32_t j = lane; j < K; j += 32) {
+                const double n = double(__ldcg(h + j));
+                if (n > 1.0) nlogn += n * log2(n);
+            }
         for (uint32_t j0 = lane; j0 < K; j0 += 8u * 32u) {     // eight loads under way at a time
             uint32_t n[8];
 #pragma unroll
@@ -418,9 +425,14 @@ __device__ __forceinline__ Evaluation gather_counts(const CountParams &P, uint32
                 seen += n[u] != 0;
             }
         }
-        if (!evaluate || E.too_many) continue;
+        if (!evaluate) continue;
         const double total = double(warp_sum(sum));
         seen = warp_sum(seen);
+        if (E.too_many) {                                    // the counts' entropy: no frequencies code them in fewer bits
+            nlogn = warp_sum(nlogn);
+            if (lane == 0) { bits_of[t] = total > 0.0 ? total * log2(total) - nlogn : 0.0; seen_of[t] = seen; }
+            continue;
+        }
         // frequencies: max(1, floor(n 2^b / total)), then the deficit to the largest or the excess from the largest
         const uint32_t M = 1u << P.rate.b;
         uint32_t fsum = 0, best = 0;
@@ -445,14 +457,41 @@ __device__ __forceinline__ Evaluation gather_counts(const CountParams &P, uint32
         if (K && fsum < M) {
             if (lane == 0) f_of[at + 0xFFFFu - (best & 0xFFFFu)] += M - fsum;
         }
-        while (K && fsum > M) {                              // (every turn lowers fsum or leaves)
-            const uint32_t f = best >> 16, take = min(fsum - M, f - 1u);
+        // A turn takes as much as it can from the first of the largest.  An alphabet of thousands with a count of one each, all
+        // raised to a frequency of one, needs hundreds of turns: after two the rest is taken in the same order at once.
+        for (uint32_t turn = 0; K && fsum > M; ++turn) {
+            const uint32_t f = best >> 16, excess = fsum - M, take = min(excess, f - 1u);
             if (f <= 1u) break;                              // more symbols than slots: judged by `worst`
+            if (turn == 2u) {
+                // the smallest `top` for which the frequencies above it, all lowered to one, give no more than the excess
+                uint32_t low = 1u, top = f, taken = 0;
+                while (low < top) {
+                    const uint32_t mid = (low + top) >> 1;
+                    uint32_t more = 0;
+#pragma unroll 8
+                    for (uint32_t j = lane; j < K; j += 32) more += f_of[at + j] > mid ? f_of[at + j] - 1u : 0u;
+                    more = warp_sum(more);
+                    if (more <= excess) { top = mid; taken = more; } else low = mid + 1u;
+                }
+                // of those that equal it the first ones give the rest
+                uint32_t before = 0;
+                for (uint32_t j0 = 0; j0 < K; j0 += 32) {
+                    const uint32_t j = j0 + lane, g = j < K ? f_of[at + j] : 0u;
+                    const bool equal = g == top && top > 1u;
+                    const uint32_t same = __ballot_sync(0xFFFFFFFFu, equal);
+                    const uint32_t gone = taken + (before + __popc(same & ((1u << lane) - 1u))) * (top - 1u);
+                    if (g > top) f_of[at + j] = 1u;
+                    else if (equal && gone < excess) f_of[at + j] = top - min(excess - gone, top - 1u);
+                    before += __popc(same);
+                }
+                break;
+            }
             if (lane == 0) f_of[at + 0xFFFFu - (best & 0xFFFFu)] = f - take;
             fsum -= take;
             __syncwarp();
             if (fsum <= M) break;
             best = 0;
+#pragma unroll 4
             for (uint32_t j = lane; j < K; j += 32) best = max(best, key(f_of[at + j], j));
             best = __reduce_max_sync(0xFFFFFFFFu, best);
         }
@@ -469,7 +508,7 @@ __device__ __forceinline__ Evaluation gather_counts(const CountParams &P, uint32
     __syncthreads();
     E.cce = 0.0;
     E.worst = 0;
-    if (evaluate && !E.too_many && warp == 0) {
+    if (evaluate && warp == 0) {
         E.cce = warp_sum(lane < EP_NUM_TABLES ? bits_of[lane] : 0.0);
         E.worst = __reduce_max_sync(0xFFFFFFFFu, lane < EP_NUM_TABLES ? seen_of[lane] : 0u);
     }
@@ -488,8 +527,8 @@ __device__ __forceinline__ void judge_candidate(const CountParams &P, uint32_t k
     const uint32_t b = __ballot_sync(0xFFFFFFFFu, above) & 7u;
     if (lane != 0) return;
     uint32_t v = kValid | ((b & 2u) ? kAbove : 0u) | ((b == 0u || b == 7u) ? 0u : kUndecided);
+    if (E.too_many) v = (b & 1u) ? kAbove | kNoCounts : kUndecided;  // E.cce is a lower bound
     if (E.worst > (1u << P.rate.b)) v = kAbove;                  // no b-bit table exists for this scale: too fine
-    if (E.too_many) v = kUndecided;
     P.state->cand[k].verdict = v;
     __threadfence();
 }
@@ -513,6 +552,7 @@ __device__ void walk_tree(const CountParams &P) {
             if (v & kOverflow) S.overflow = 1;
             if (v & kUndecided) S.undecided = 1;
             if (v & kValid) last = int32_t(k);
+            if (v & kNoCounts) last = -2;
             const double mid = __dsqrt_rn(__dmul_rn(lo, hi));
             if (v & kAbove) { lo = mid; k = 2u * k + 1u; } else { hi = mid; k = 2u * k + 2u; }
         }
@@ -520,8 +560,8 @@ __device__ void walk_tree(const CountParams &P) {
         S.hi = hi;
         S.s = __double2float_rn(__dsqrt_rn(__dmul_rn(lo, hi)));
         S.closed = 0;
-        if (last >= 0) S.has_last = 1;
-        else if (P.last_pass && S.has_last) S.undecided = 1;     // (its counts are gone)
+        if (last != -1) S.has_last = 1;
+        if (P.last_pass && S.has_last && last < 0) S.undecided = 1;  // (its counts are gone)
         chosen = P.last_pass ? last : -1;
     }
     __syncthreads();
@@ -541,12 +581,12 @@ __device__ void walk_tree(const CountParams &P) {
 __device__ void polish(const CountParams &P, float s, const Evaluation &E) {
     SearchState &S = *P.state;
     S.s_counted = s;
-    if (E.too_many) { S.undecided = 1; S.stop = 1; return; }
     if (E.worst > (1u << P.rate.b)) {                            // before the first move: the host raises b or s
         if (P.step > 0) S.undecided = 1;
         S.stop = 1;
         return;
     }
+    if (E.too_many) { S.undecided = 1; S.stop = 1; return; }
     S.polished = 1;
     if (P.step >= P.last_step) { S.stop = 1; return; }
     const double off = cce_bound(P.rate, E.cce), bits = bits_at(P.rate, E.tables, E.cce);
