@@ -266,10 +266,11 @@ constexpr int kHotBins = 32, kHotOrigin = -16;   // values with a counter column
 constexpr uint32_t kHotStride = (kHotBins + 1) * 32;   // words per table: one more row takes what lies outside
 constexpr int kWinBins = 512, kWinOrigin = -256; // values with one counter per CTA, per table (2048 of them gain nothing at 8 bpp either)
 constexpr uint32_t kHotWords = 16 * kHotStride, kWinWords = EP_NUM_TABLES * kWinBins;
-// symbols over all tables that an evaluation holds in shared memory (it reuses the counters' space): more than a finished stream
-// may have.  A finer scale of the search with more of them is judged by the counts' entropy (see judge_candidate).
-constexpr uint32_t kEvalSymbols = 49152;
-static_assert(kEvalSymbols >= kHotWords + kWinWords && kEvalSymbols >= kMaxTableSymbols, "evaluation space");
+// Symbols over all tables that an evaluation holds in shared memory (it reuses the counters' space; 196 KB for 49152 of them
+// cost the passes 4 % of their time).  A scale of the search with more - heavy tails meet some at 6 bpp - is judged by the
+// entropy of its counts if that is enough, as it is for scales that are far too fine; if not the host takes over.
+constexpr uint32_t kEvalSymbols = kHotWords + kWinWords;
+constexpr uint32_t kManySymbols = 8192;          // with more the counts' entropy is looked at first (see gather_counts)
 constexpr uint32_t kCountSmem = 4 * kEvalSymbols;
 constexpr uint32_t kFirstCounts = 6144;          // counts that come back with the state; more take a second copy
 constexpr uint32_t kLevels = 4, kCandidates = (1u << kLevels) - 1u;
@@ -360,7 +361,11 @@ __device__ __forceinline__ double bits_at(const RateParams &P, double tables, do
     return __dadd_rn(__dadd_rn(__dmul_rn(16.0, ceil(__dmul_rn(left, 0.0625))), P.fixed_bits), tables);
 }
 
-struct Evaluation { double cce, tables; uint32_t worst; bool too_many; };
+// C_CE below is a sum in another order, with this device's log2 (within one unit in the last place; terms of at most 15 bits
+// per field, a few thousand additions).  How far the host's can be:
+__device__ __forceinline__ double cce_bound(const RateParams &P, double cce) { return 1e-11 * (cce + 16.0 * P.fields); }
+
+struct Evaluation { double cce, tables; uint32_t worst; bool too_many, above; };   // above: by the counts' entropy alone
 
 // All threads of a candidate's last CTA: ranges and offsets of its tables, counts to `out`, histogram back to zero; unless
 // only counts are wanted, the frequencies of Sec. 3.3 (integers: the host's exactly), C_CE of Eq. 8 and the largest alphabet.
@@ -395,6 +400,12 @@ __device__ __forceinline__ Evaluation gather_counts(const CountParams &P, uint32
     __syncthreads();
     const bool evaluate = P.mode != kPassCount;
     Evaluation E;
+    // a scale of the search with this many symbols is usually far too fine: the entropy of its counts says so for less
+    const bool many = P.mode == kPassSearch && at_of[EP_NUM_TABLES] > kManySymbols;
+    double total = 0.0;
+    E.cce = 0.0;
+    E.worst = 0;
+    E.above = false;
     E.too_many = at_of[EP_NUM_TABLES] > kEvalSymbols;       // (only full_counts has room for more)
     E.tables = 8.0 * double((8u * EP_NUM_TABLES + 2u * at_of[EP_NUM_TABLES] + 3u) & ~3u);
     const bool keep = !E.too_many || P.mode != kPassSearch;
@@ -404,12 +415,13 @@ __device__ __forceinline__ Evaluation gather_counts(const CountParams &P, uint32
         unsigned long long sum = 0;
         uint32_t seen = 0;
         double nlogn = 0.0;
-        if (E.too_many && evaluate)
-#pragma unroll 4
+        if (many) {
+#pragma unroll 8
             for (uint32_t j = lane; j < K; j += 32) {
-                const double n = double(__ldcg(h + j));
-                if (n > 1.0) nlogn += n * log2(n);
+                const float n = float(__ldcg(h + j));
+                if (n > 1.0f) nlogn += double(n) * double(log2f(n));
             }
+        }
         for (uint32_t j0 = lane; j0 < K; j0 += 8u * 32u) {     // eight loads under way at a time
             uint32_t n[8];
 #pragma unroll
@@ -426,13 +438,21 @@ __device__ __forceinline__ Evaluation gather_counts(const CountParams &P, uint32
             }
         }
         if (!evaluate) continue;
-        const double total = double(warp_sum(sum));
+        total = double(warp_sum(sum));
         seen = warp_sum(seen);
-        if (E.too_many) {                                    // the counts' entropy: no frequencies code them in fewer bits
-            nlogn = warp_sum(nlogn);
-            if (lane == 0) { bits_of[t] = total > 0.0 ? total * log2(total) - nlogn : 0.0; seen_of[t] = seen; }
-            continue;
-        }
+        if (many) nlogn = warp_sum(nlogn);
+        if (lane == 0) { bits_of[t] = many && total > 0.0 ? total * log2(total) - nlogn : 0.0; seen_of[t] = seen; }
+    }
+    if (many) {
+        __syncthreads();
+        double least = -1e-5 * P.rate.fields;                // log2f: an error of 2e-6 per count
+        for (uint32_t t = 0; t < EP_NUM_TABLES; ++t) { least += bits_of[t]; E.worst = max(E.worst, seen_of[t]); }
+        E.above = __ddiv_rn(bits_at(P.rate, E.tables, least - cce_bound(P.rate, least)), P.rate.weights) > P.rate.target;
+        if (E.above || E.too_many) return E;
+        __syncthreads();
+    }
+    if (evaluate && !E.too_many && warp < EP_NUM_TABLES) {
+        const uint32_t t = warp, K = K_of[t], at = at_of[t];
         // frequencies: max(1, floor(n 2^b / total)), then the deficit to the largest or the excess from the largest
         const uint32_t M = 1u << P.rate.b;
         uint32_t fsum = 0, best = 0;
@@ -503,21 +523,15 @@ __device__ __forceinline__ Evaluation gather_counts(const CountParams &P, uint32
             if (f) bits += double(out[at + j]) * (double(P.rate.b) - log2(double(f)));
         }
         bits = warp_sum(bits);
-        if (lane == 0) { bits_of[t] = bits; seen_of[t] = seen; }
+        if (lane == 0) bits_of[t] = bits;
     }
     __syncthreads();
-    E.cce = 0.0;
-    E.worst = 0;
     if (evaluate && warp == 0) {
         E.cce = warp_sum(lane < EP_NUM_TABLES ? bits_of[lane] : 0.0);
         E.worst = __reduce_max_sync(0xFFFFFFFFu, lane < EP_NUM_TABLES ? seen_of[lane] : 0u);
     }
     return E;                                                // (cce and worst in warp 0)
 }
-// C_CE above is a sum in another order, with this device's log2 (within one unit in the last place; terms of at most 15 bits
-// per field, a few thousand additions).  How far the host's can be:
-__device__ __forceinline__ double cce_bound(const RateParams &P, double cce) { return 1e-11 * (cce + 16.0 * P.fields); }
-
 // warp 0 after a candidate of the search is gathered: is its rate above the target?
 __device__ __forceinline__ void judge_candidate(const CountParams &P, uint32_t k, const Evaluation &E) {
     // lane 1 at the estimate, lanes 0 and 2 at the ends of its interval
@@ -527,7 +541,8 @@ __device__ __forceinline__ void judge_candidate(const CountParams &P, uint32_t k
     const uint32_t b = __ballot_sync(0xFFFFFFFFu, above) & 7u;
     if (lane != 0) return;
     uint32_t v = kValid | ((b & 2u) ? kAbove : 0u) | ((b == 0u || b == 7u) ? 0u : kUndecided);
-    if (E.too_many) v = (b & 1u) ? kAbove | kNoCounts : kUndecided;  // E.cce is a lower bound
+    if (E.above) v = kAbove | (E.too_many ? kNoCounts : kValid);
+    else if (E.too_many) v = kUndecided;
     if (E.worst > (1u << P.rate.b)) v = kAbove;                  // no b-bit table exists for this scale: too fine
     P.state->cand[k].verdict = v;
     __threadfence();

@@ -121,3 +121,17 @@ def test_device_encoder_bytes_at_the_edges_of_its_paths(W, bpp, kw):
     host = ep.encode(W, bpp, **kw)
     dev = ep.encode_device(torch.from_numpy(np.ascontiguousarray(W, np.float32)).cuda(), bpp, **kw)
     assert np.array_equal(dev.data, host.data) and dev.report == host.report
+
+
+@pytest.mark.parametrize("maker,shape,bpp,kw", [
+    (synth.laplace_rows, (480, 1024), 6.0, {}),                    # steps of the search judged by the entropy of their counts
+    (synth.laplace_rows, (480, 1024), 8.0, {}),                    # and alphabets whose excess of slots takes hundreds of turns
+    (synth.laplace_rows, (480, 1024), 8.0, dict(b_start=11, b_max=11)),
+    (synth.outlier_rows, (64, 4096), 8.0, {}),
+    (synth.outlier_rows, (512, 1024), 7.0, dict(polish_steps=0)),
+])
+def test_device_encoder_bytes_with_wide_alphabets(maker, shape, bpp, kw):
+    W = maker(*shape, 12)
+    host = ep.encode(W, bpp, **kw)
+    dev = ep.encode_device(torch.from_numpy(W).cuda(), bpp, **kw)
+    assert np.array_equal(dev.data, host.data) and dev.report == host.report
