@@ -165,7 +165,7 @@ int ep_pack_fields(const int32_t *fields, uint32_t R, uint32_t C, int32_t b, uin
  * Eq. 13, tile coding); the final tables are made on the host.  The result is byte for byte the blob ep_encode
  * produces for the same W and options.  d_W is a device copy of W (16-byte
  * aligned), d_workspace a 256-byte aligned device buffer of ep_encode_device_workspace_bytes() bytes
- * (about 52 bytes per 8-weight block and 12 MB).  The call enqueues on `stream` and synchronises it several times;
+ * (about 52 bytes per 8-weight block and 13 MB).  The call enqueues on `stream` and synchronises it several times;
  * it returns the finished host blob.  EP_ERR_UNSUPPORTED (use ep_encode instead) if a lattice coordinate
  * exceeds +-4095 or the tables hold more than 40960 symbols in total.
  * The blob of this call lives in page-locked host memory (the device copies the payload straight into it,

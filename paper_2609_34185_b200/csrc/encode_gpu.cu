@@ -27,10 +27,8 @@ namespace {
 
 using namespace ep;
 
-constexpr int kHistBins = 8192;          // per table, values -4096 .. 4095
-constexpr int kHistOrigin = -4096;
+constexpr int kHistOrigin = -4096;       // kHistBins values per table: -4096 .. 4095
 constexpr uint32_t kMaxTableSymbols = 40960;   // sum of K over the 17 tables that a stream of this back end may have
-constexpr uint32_t kMaxEntries = 2 * kMaxTableSymbols + 2;     // the tile coder's entries (see EncodeTables)
 constexpr double kUnit = 1.1102230246251565e-16;   // 2^-53, the rounding unit of double
 
 // the wait of a kernel that is launched while the one before it ends (launch_chained): before it, only kernel parameters are read
@@ -1090,8 +1088,8 @@ Workspace carve(uint8_t *base, uint32_t R, uint32_t C, uint32_t V) {
     w.hist = reinterpret_cast<uint32_t *>(take(kCandidates * kHistBytes));
     w.cand_counts = reinterpret_cast<uint32_t *>(take(4ull * kCandidates * kEvalSymbols));
     w.full_counts = reinterpret_cast<uint32_t *>(take(kHistBytes));
-    w.fF = reinterpret_cast<uint32_t *>(take(4ull * kMaxEntries));
-    w.entries = reinterpret_cast<uint4 *>(take(16ull * kMaxEntries));
+    w.fF = reinterpret_cast<uint32_t *>(take(4ull * kCoderEntries));
+    w.entries = reinterpret_cast<uint4 *>(take(16ull * kCoderEntries));
     w.counts = reinterpret_cast<uint32_t *>(take(4ull * n_tiles));
     w.fields = reinterpret_cast<uint4 *>(take(16ull * nvec));
     w.scratch = reinterpret_cast<uint16_t *>(take(2ull * cap * n_tiles + 4));
@@ -1238,32 +1236,19 @@ public:
         uint64_t symbols = 0;
         for (int t = 0; t < EP_NUM_TABLES; ++t) symbols += m.t[t].K();
         if (symbols > kMaxTableSymbols) return EP_ERR_UNSUPPORTED;
-        // per field the range of both cosets' tables
-        int32_t lo[9], hi[9];
-        uint32_t first[9], size = 0;
-        for (int k = 0; k < 9; ++k) {
-            lo[k] = hi[k] = 0;                   // (k = 0: the coset itself, 0 or 1)
-            bool any = false;
-            for (int c = 0; c < 2 && k > 0; ++c) {
-                const Table &tb = m.t[table_id(c, k)];
-                if (!tb.K()) continue;
-                lo[k] = any ? std::min(lo[k], tb.lo) : tb.lo;
-                hi[k] = any ? std::max(hi[k], tb.lo + int32_t(tb.K())) : tb.lo + int32_t(tb.K());
-                any = true;
-            }
-            if (k == 0) continue;
-            first[k] = size;
-            size += uint32_t(hi[k] - lo[k]);
-        }
+        const CoderLayout L = coder_layout(m);
+        if (L.entries() > kCoderEntries) return EP_ERR_UNSUPPORTED;      // (no count lies outside the histogram: cannot happen)
+        const uint32_t size = L.size;
         EncodeTables T{};
         T.coset = 16u * size;
-        T.total = 2u * size + 2u;
+        T.total = L.entries();
         std::vector<uint32_t> fF(T.total, 0);
         for (int k = 1; k < 9; ++k) {
-            T.base[k] = 16u * (first[k] - uint32_t(lo[k]));
+            T.base[k] = 16u * (L.first[k] - uint32_t(L.lo[k]));
             for (int c = 0; c < 2; ++c) {
                 const Table &tb = m.t[table_id(c, k)];
-                uint32_t *to = fF.data() + uint32_t(c) * size + first[k] + uint32_t(tb.lo - lo[k]);
+                if (!tb.K()) continue;
+                uint32_t *to = fF.data() + uint32_t(c) * size + L.first[k] + uint32_t(tb.lo - L.lo[k]);
                 for (uint32_t j = 0; j < tb.K(); ++j) to[j] = tb.f[j] | (tb.F[j] << 16);
             }
         }

@@ -88,6 +88,38 @@ struct Model {
 // Eq. 10-11: estimated stored bits of nvec vectors in `rows` rows under model m
 double estimate_bits(const Model &m, int b, uint64_t nvec, uint64_t rows, uint32_t V, double retained, double *cce_out);
 
+// The CUDA back end's tile coder looks a symbol up by (coset, field, value): per field the tables of both cosets cover the same
+// values, from the lower to the higher end of the two, so that coset 1's entries follow coset 0's at one distance; the
+// coset's own two entries come last.  The ranges of the two cosets need not meet - a few large blocks in a tensor of
+// zeros: one coset at -3873, the other at 3872 - so what bounds the entries is not the number of symbols but the
+// values a field can have.
+constexpr int kHistBins = 8192;          // values per table that the CUDA back end counts
+constexpr uint32_t kCoderEntries = 2u * 8u * kHistBins + 2u;
+struct CoderLayout {
+    int32_t lo[9] = {};                  // field k's lowest value (k = 1 .. 8) and
+    uint32_t first[9] = {};              // where its entry is
+    uint32_t size = 0;                   // entries per coset
+    uint32_t entries() const { return 2u * size + 2u; }
+};
+inline CoderLayout coder_layout(const Model &m) {
+    CoderLayout L;
+    for (int k = 1; k < 9; ++k) {
+        int32_t hi = 0;
+        bool any = false;
+        for (int c = 0; c < 2; ++c) {
+            const Table &tb = m.t[table_id(c, k)];
+            if (!tb.K()) continue;
+            const int32_t end = tb.lo + int32_t(tb.K());
+            L.lo[k] = any && L.lo[k] < tb.lo ? L.lo[k] : tb.lo;
+            hi = any && hi > end ? hi : end;
+            any = true;
+        }
+        L.first[k] = L.size;
+        L.size += uint32_t(hi - L.lo[k]);
+    }
+    return L;
+}
+
 // App. "Scale-search settings": complete rows, shape-dependent seed, sorted
 std::vector<uint32_t> sample_rows(uint32_t R, uint32_t C, uint32_t budget_vectors);
 

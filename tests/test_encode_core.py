@@ -1,0 +1,55 @@
+"""Host-side parts of the CUDA encoder back end that need no GPU: small programs over csrc/encoder_core.hpp."""
+import os
+import subprocess
+
+import numpy as np
+import pytest
+
+import paper_2609_34185_b200 as ep
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+
+def _program(tmp_path, body):
+    """Compiles `body` as the main function of a program and returns a function that runs it on numbers."""
+    src, exe = tmp_path / "p.cpp", tmp_path / "p"
+    src.write_text('#include "encoder_core.hpp"\n#include <cstdio>\n#include <cstdlib>\nusing namespace ep;\n'
+                   "int main(int argc, char **argv) {\n" + body + "\nreturn 0;\n}\n")
+    subprocess.run(["g++", "-std=c++17", "-O1", "-I", os.path.join(ROOT, "include"),
+                    "-I", os.path.join(ROOT, "paper_2609_34185_b200", "csrc"), str(src), "-o", str(exe)], check=True)
+    return lambda *a: subprocess.run([str(exe)] + [repr(v) for v in a], check=True, capture_output=True, text=True).stdout.split()
+
+
+def disjoint_cosets():
+    """All zero but two blocks, one on integer and one on half-integer coordinates, far apart: at the fine end of the
+    search the two cosets' tables do not meet (-3873 .. and 3872)."""
+    W = np.zeros((600, 120), np.float32)
+    W[0, 8:16] = -1.0
+    W[1, 8:16] = 1.0
+    W[1, 0] = 0.04
+    return W
+
+
+def test_coder_entries_hold_cosets_that_do_not_meet(tmp_path):
+    run = _program(tmp_path, """
+        Model m;
+        for (int t = 0; t < EP_NUM_TABLES; ++t) { m.t[t].lo = atoi(argv[1 + t]); m.t[t].n.resize(atoi(argv[18 + t])); }
+        const CoderLayout L = coder_layout(m);
+        bool inside = true;
+        for (int k = 1; k < 9; ++k)
+            for (int c = 0; c < 2; ++c) {
+                const Table &tb = m.t[table_id(c, k)];
+                const int64_t at = int64_t(L.first[k]) + tb.lo - L.lo[k], next = k < 8 ? L.first[k + 1] : L.size;
+                if (tb.K()) inside = inside && at >= L.first[k] && at + tb.K() <= next;
+            }
+        printf("%u %u %d\\n", L.entries(), kCoderEntries, int(inside));""")
+    info = ep.encode(disjoint_cosets(), 8.0).info
+    assert sum(info.table_K) <= 40960                        # a stream that the device encoder takes
+    entries, room, inside = map(int, run(*info.table_min, *info.table_K))
+    assert 2 * 40960 + 2 < entries <= room and inside        # more than two entries per symbol of any such stream
+    # the widest there can be: a value at either end of what the passes count, in every field
+    entries, room, inside = map(int, run(0, *[-4096] * 8, *[4095] * 8, 2, *[1] * 16))
+    assert entries == room and inside
+    # a tensor with one coset only, and tables that share a range
+    assert run(0, *[-3] * 8, *[0] * 8, 1, *[7] * 8, *[0] * 8)[0] == str(2 * 8 * 7 + 2)
+    assert run(0, *[-3] * 8, *[-2] * 8, 2, *[7] * 16)[0] == str(2 * 8 * 8 + 2)

@@ -7,6 +7,7 @@ import torch
 import oracle
 import paper_2609_34185_b200 as ep
 from paper_2609_34185_b200 import synth
+from test_encode_core import disjoint_cosets
 
 pytestmark = pytest.mark.gpu
 
@@ -138,4 +139,12 @@ def test_device_encoder_bytes_with_wide_alphabets(maker, shape, bpp, kw):
     W = maker(*shape, 12)
     host = ep.encode(W, bpp, **kw)
     dev = ep.encode_device(torch.from_numpy(W).cuda(), bpp, **kw)
+    assert np.array_equal(dev.data, host.data) and dev.report == host.report
+
+
+@pytest.mark.parametrize("bpp", [8.0, 2.0])
+def test_device_encoder_bytes_with_cosets_that_do_not_meet(bpp):
+    W = disjoint_cosets()
+    host = ep.encode(W, bpp)
+    dev = ep.encode_device(torch.from_numpy(W).cuda(), bpp)
     assert np.array_equal(dev.data, host.data) and dev.report == host.report
