@@ -1160,12 +1160,15 @@ public:
         if (!mail_) throw std::bad_alloc();
     }
     ~DeviceBackend() override {
+        // a call that ends early must not leave a copy into the page-locked buffers behind, which the next call may have then
+        if (under_way_) cudaStreamSynchronize(st_);
         if (event_) cudaEventDestroy(event_);
         if (mail_) g_mail_slot.release(mail_, mail_cap_);
     }
 
     int prepare(const std::vector<uint32_t> &sample) override {
         n_sample_ = uint32_t(sample.size());
+        under_way_ = true;
         EP_CUDA(cudaEventCreateWithFlags(&event_, cudaEventDisableTiming));
         int dev = 0;
         EP_CUDA(cudaGetDevice(&dev));
@@ -1293,6 +1296,7 @@ public:
             const uint64_t total = state()->total_words;
             if (total >= (1ull << 31)) return EP_ERR_UNSUPPORTED;
             if (total <= room) {
+                under_way_ = false;
                 end_blob(L, total, out);
                 return EP_OK;
             }
@@ -1409,6 +1413,7 @@ private:
     size_t mail_cap_ = 0;
     uint32_t n_sample_ = 0;
     cudaEvent_t event_ = nullptr;
+    bool under_way_ = false;         // the stream may still work for this call
     bool sigma_there_ = false;       // w_.sigma holds the row scales of the kept quantisation, which is at scale sigma_of_
     float sigma_of_ = 0.0f;
 };

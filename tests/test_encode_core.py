@@ -53,3 +53,16 @@ def test_coder_entries_hold_cosets_that_do_not_meet(tmp_path):
     # a tensor with one coset only, and tables that share a range
     assert run(0, *[-3] * 8, *[0] * 8, 1, *[7] * 8, *[0] * 8)[0] == str(2 * 8 * 7 + 2)
     assert run(0, *[-3] * 8, *[-2] * 8, 2, *[7] * 16)[0] == str(2 * 8 * 8 + 2)
+
+
+def test_encode_that_fails_leaves_no_copy_under_way(tmp_path):
+    # the page-locked buffer of the counts goes back to the process when the call ends: nothing may be on its way into it
+    exe, csrc = str(tmp_path / "fake_device"), os.path.join(ROOT, "paper_2609_34185_b200", "csrc")
+    nvcc = os.environ.get("NVCC") or "/usr/local/cuda/bin/nvcc"
+    subprocess.run([nvcc, "-gencode", "arch=compute_100a,code=sm_100a", "-O0", "-std=c++17", "-cudart", "none", "-Xcompiler", "-pthread",
+                    "-I", os.path.join(ROOT, "include"), "-I", csrc, "-o", exe, os.path.join(ROOT, "tests", "fake_device.cpp")]
+                   + [os.path.join(csrc, f) for f in ("encode_gpu.cu", "encoder.cpp", "stream.cpp")], check=True)
+    run = lambda buffers: subprocess.run([exe, str(buffers)], check=True, capture_output=True, text=True).stdout.split()
+    assert run(2) == ["0", "0"]
+    assert run(0) == ["-6", "0"]          # no memory for the counts
+    assert run(1) == ["-6", "0"]          # none for the blob: the tile coder and its copies are queued by then
