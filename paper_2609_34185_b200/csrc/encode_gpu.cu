@@ -614,10 +614,10 @@ __device__ void polish(const CountParams &P, float s, const Evaluation &E) {
         if (!(per_doubling >= 0.5)) per_doubling = 0.5;
         if (per_doubling > 4.0) per_doubling = 4.0;
     }
+    // log2 and exp2 may differ from the host's in the last place; 1e-10 is far above what that makes of an ordinary move
+    const double near = fmax(1e-10, next_scale_error(log_s, S.last_log_s, P.step > 0, __dsub_rn(est, P.rate.target), per_doubling));
     S.last_log_s = log_s;
     S.last_rate = est;
-    // log2 and exp2 may differ from the host's in the last place (of numbers up to ten, divided by a slope of at least 1/2, and
-    // by a move of at least 2^-20 in the secant): far less than 1e-8
     const double moved = exp2(__dadd_rn(log_s, __ddiv_rn(__dsub_rn(est, P.rate.target), per_doubling)));
     auto next = [&](double m) {
         if (!(m >= P.lo0)) m = P.lo0;
@@ -625,7 +625,7 @@ __device__ void polish(const CountParams &P, float s, const Evaluation &E) {
         return __double2float_rn(m);
     };
     const float to = next(moved);
-    if (next(moved * (1.0 - 1e-10)) != to || next(moved * (1.0 + 1e-10)) != to) { S.undecided = 1; S.stop = 1; return; }
+    if (next(moved * (1.0 - near)) != to || next(moved * (1.0 + near)) != to) { S.undecided = 1; S.stop = 1; return; }
     if (to == s) { S.stop = 1; return; }
     S.s = to;
 }

@@ -120,6 +120,29 @@ inline CoderLayout coder_layout(const Model &m) {
     return L;
 }
 
+// Rate correction in a back end of its own arithmetic: how far, relatively, the next scale 2^(log_s + off_target / per_doubling)
+// can be from run_encode's if log2 and exp2 are within one unit in the last place there and here (two between them;
+// u = 2^-52), and everything else is rounded as there.  The secant divides by log_s - last_log_s, which scales next
+// to each other make as small as 2^-23.5: then two such units of log_s are 1e-8 of the slope.
+#ifdef __CUDACC__
+__host__ __device__
+#endif
+inline double next_scale_error(double log_s, double last_log_s, bool secant, double off_target, double per_doubling) {
+    const double u = 2.220446049250313e-16;
+    const double size = log_s < 0 ? -log_s : log_s, last = last_log_s < 0 ? -last_log_s : last_log_s;
+    double slope = 2.0 * u;                          // relative, clamping to [1/2, 4] does not add to it
+    if (secant) {
+        const double moved = log_s < last_log_s ? last_log_s - log_s : log_s - last_log_s;
+        const double off = 2.0 * u * (size + last) + u * moved;
+        if (!(off < 0.25 * moved)) return 1.0;       // says nothing
+        slope += 1.34 * off / moved;                 // 1 / (1 - 1/4)
+    }
+    double step = off_target / per_doubling;
+    if (step < 0) step = -step;
+    const double exponent = 2.0 * u * size + step * (slope + 2.0 * u) + u * (size + step);
+    return 0.7 * exponent + 8.0 * u;                 // ln 2, exp2 on either side and the roundings of a comparison
+}
+
 // App. "Scale-search settings": complete rows, shape-dependent seed, sorted
 std::vector<uint32_t> sample_rows(uint32_t R, uint32_t C, uint32_t budget_vectors);
 

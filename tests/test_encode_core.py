@@ -13,7 +13,7 @@ ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 def _program(tmp_path, body):
     """Compiles `body` as the main function of a program and returns a function that runs it on numbers."""
     src, exe = tmp_path / "p.cpp", tmp_path / "p"
-    src.write_text('#include "encoder_core.hpp"\n#include <cstdio>\n#include <cstdlib>\nusing namespace ep;\n'
+    src.write_text('#include "encoder_core.hpp"\n#include <algorithm>\n#include <cmath>\n#include <cstdio>\n#include <cstdlib>\nusing namespace ep;\n'
                    "int main(int argc, char **argv) {\n" + body + "\nreturn 0;\n}\n")
     subprocess.run(["g++", "-std=c++17", "-O1", "-I", os.path.join(ROOT, "include"),
                     "-I", os.path.join(ROOT, "paper_2609_34185_b200", "csrc"), str(src), "-o", str(exe)], check=True)
@@ -66,3 +66,37 @@ def test_encode_that_fails_leaves_no_copy_under_way(tmp_path):
     assert run(2) == ["0", "0"]
     assert run(0) == ["-6", "0"]          # no memory for the counts
     assert run(1) == ["-6", "0"]          # none for the blob: the tile coder and its copies are queued by then
+
+
+def test_next_scale_error_covers_another_log2_and_exp2(tmp_path):
+    # run_encode's secant step with log2 and exp2 two units in the last place off, in every combination, over moves from
+    # neighbouring scales to whole doublings
+    run = _program(tmp_path, """
+        auto ulps = [](double v, int n) { for (; n > 0; --n) v = std::nextafter(v, 1e9); for (; n < 0; ++n) v = std::nextafter(v, -1e9); return v; };
+        uint64_t st = 7;
+        auto rnd = [&] { st = st * 6364136223846793005ull + 1442695040888963407ull; return double(st >> 11) / 9007199254740992.0; };
+        double worst = 0.0, neighbours = 0.0, ordinary = 0.0;
+        for (int i = 0; i < 20000; ++i) {
+            const float s = float(std::exp2(-9.0 + 12.0 * rnd()));
+            const bool next_to = i % 2 == 0;
+            const float before = next_to ? std::nextafter(s, rnd() < 0.5 ? 0.0f : 9.0f) : float(double(s) * std::exp2((rnd() < 0.5 ? -1 : 1) * std::exp2(-12.0 * rnd())));
+            const double a = std::log2(double(s)), p = std::log2(double(before)), target = 0.08 * (rnd() - 0.5), slope = 0.4 + 4.0 * rnd();
+            const double gained = -slope * (a - p);                            // the rates differ by this: a slope inside and outside the clamps
+            auto move = [&](int da, int dp, int de, double *per_out) {
+                double per = -gained / (ulps(a, da) - ulps(p, dp));
+                if (!(per >= 0.5)) per = 0.5;
+                if (per > 4.0) per = 4.0;
+                if (per_out) *per_out = per;
+                return ulps(std::exp2(ulps(a, da) + target / per), de);
+            };
+            double per;
+            const double here = move(0, 0, 0, &per), bound = next_scale_error(a, p, true, target, per);
+            (next_to ? neighbours : ordinary) = std::max(next_to ? neighbours : ordinary, bound);
+            for (int da = -2; da <= 2; ++da)
+                for (int dp = -2; dp <= 2; ++dp)
+                    for (int de = -2; de <= 2; ++de) worst = std::max(worst, std::fabs(move(da, dp, de, nullptr) / here - 1.0) / bound);
+        }
+        printf("%g %g %g\\n", worst, neighbours, ordinary);""")
+    worst, neighbours, ordinary = map(float, run())
+    assert 0.1 < worst <= 1.0                  # covered, and not by orders of magnitude too much
+    assert neighbours > 1e-10 > ordinary       # no fixed 1e-10 covers neighbouring scales
