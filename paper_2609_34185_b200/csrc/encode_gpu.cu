@@ -299,7 +299,7 @@ struct SearchState {
     uint32_t stop;                   // the full passes are over
     uint32_t polished;               // ... because the rate correction ended (0: the tensor overflows the tables, the host decides)
     CountDir last, full;
-    uint32_t total_words;            // tile coding: words of the payload
+    uint64_t total_words;            // tile coding: words of the payload (more than a blob can hold are still told apart)
     uint32_t tiles_done;             //              CTAs of the launch that are done
     Candidate cand[kCandidates];
 };
@@ -946,7 +946,8 @@ __global__ void __launch_bounds__(kTileThreadsMax) tile_encode_kernel(const uint
                                                                       uint16_t *__restrict__ scratch, uint32_t cap,
                                                                       uint32_t *__restrict__ index, uint32_t *__restrict__ counts, SearchState *state) {
     extern __shared__ __align__(16) uint4 entries_smem[];
-    __shared__ uint32_t last_cta, part[kTileThreadsMax];
+    __shared__ uint32_t last_cta;
+    __shared__ uint64_t part[kTileThreadsMax];
     const uint32_t tid = threadIdx.x, lane = tid & 31u;
     chained_start();
     if (IN_SMEM) {
@@ -1007,20 +1008,20 @@ __global__ void __launch_bounds__(kTileThreadsMax) tile_encode_kernel(const uint
     __threadfence();
     const uint32_t per = (n_tiles + blockDim.x - 1u) / blockDim.x;
     const uint32_t t0 = min(tid * per, n_tiles), t1 = min(t0 + per, n_tiles);
-    uint32_t sum = 0;
+    uint64_t sum = 0;
     for (uint32_t t = t0; t < t1; ++t) sum += __ldcg(counts + t);
     part[tid] = sum;
     __syncthreads();
     for (uint32_t d = 1; d < blockDim.x; d <<= 1) {
-        const uint32_t add = tid >= d ? part[tid - d] : 0u;
+        const uint64_t add = tid >= d ? part[tid - d] : 0u;
         __syncthreads();
         part[tid] += add;
         __syncthreads();
     }
-    uint32_t at = part[tid] - sum;
+    uint32_t at = uint32_t(part[tid] - sum);
     for (uint32_t t = t0; t < t1; ++t) { index[size_t(t) * 33u + 32u] = at; at += __ldcg(counts + t); }
     if (tid == blockDim.x - 1u) {
-        index[size_t(n_tiles) * 33u] = part[tid];
+        index[size_t(n_tiles) * 33u] = uint32_t(part[tid]);
         state->total_words = part[tid];
         state->tiles_done = 0;
     }
@@ -1272,18 +1273,18 @@ public:
                                    uint32_t(nvec), V, n_tiles, T, w_.entries, w_.scratch, cap, w_.index, w_.counts, w_.state));
         }
         EP_CUDA(launch_chained(compact_kernel, n_tiles, n_tiles < 600u ? 512u : 128u, 0, w_.scratch, cap, w_.counts, w_.index, w_.payload));
-        EP_CUDA(cudaMemcpyAsync(&state()->total_words, &w_.state->total_words, 4, cudaMemcpyDeviceToHost, st_));
+        EP_CUDA(cudaMemcpyAsync(&state()->total_words, &w_.state->total_words, sizeof(state()->total_words), cudaMemcpyDeviceToHost, st_));
         if (!sigma_there_ || sigma_of_ != s) refit_kernel<<<R_, kRowThreads, 0, st_>>>(W_, C_, w_.fields, s, nullptr, w_.mu, w_.sigma);
         EP_CUDA(cudaGetLastError());
         return EP_OK;
     }
     int end_finish(float s, int b, uint32_t V, const Model &m, double cce, ep_blob *out) override {
         const uint64_t nvec = uint64_t(R_) * (C_ / 8), n_tiles = (nvec + V - 1) / V;
-        // How many words the tiles have is known when the device is done; the copy is issued now, for a few more than the
-        // entropy says (coding loses about 1e-5 of it, and a tile's states keep some bits), never for more than the words' area
-        // holds.  Were they more even so, the blob is laid out again.
-        const uint64_t guess = uint64_t(cce / 16.0 * 1.001) + 8u * n_tiles + 256u;
-        uint64_t room = std::min(guess, std::min<uint64_t>(9ull * V * n_tiles, (1ull << 31) - 1u));
+        // how many words the tiles have is known when the device is done; the copy is issued now, for a few more than that.  Were they
+        // more even so, the blob is laid out again
+        const uint64_t before = kHeaderBytes + m.section_bytes() + 4ull * R_ + uint64_t(kTileRecordBytes) * n_tiles + 4u;
+        uint64_t room = payload_room(cce, n_tiles, 9ull * V * n_tiles, before);
+        if (!room) return EP_ERR_UNSUPPORTED;
         out->acquire = pinned_acquire;
         out->release = pinned_release;
         for (;;) {

@@ -155,6 +155,17 @@ int begin_blob(const Model &m, uint32_t R, uint32_t C, int b, uint32_t V, float 
                BlobLayout *at);
 void end_blob(const BlobLayout &at, uint64_t total_words, ep_blob *out);
 
+// How many payload words to lay a blob out for before the tile coder is done, given C_CE of the final tables, the words' area
+// and the bytes before the payload: a few more than the entropy says (coding loses about 1e-5 of it, and a tile's states
+// keep some bits), never more than the area holds or a blob can have (its section offsets and its size are 32-bit).
+// 0: the tiles have more than a blob can hold whatever their states keep (at most 16 bits each).
+inline uint64_t payload_room(double cce_bits, uint64_t n_tiles, uint64_t area_words, uint64_t bytes_before) {
+    const uint64_t bytes = (1ull << 32) - 1u, most = bytes_before < bytes ? (bytes - bytes_before) / 2u : 0u;
+    if (0.98 * cce_bits / 16.0 - double(kStates * n_tiles) > double(most)) return 0;
+    const uint64_t guess = uint64_t(cce_bits / 16.0 * 1.001) + 8u * n_tiles + 256u, room = guess < area_words ? guess : area_words;
+    return room < most ? room : most;
+}
+
 // header + tables + scales + tile index + payload; `states` holds 32 words per tile, tile t's payload is
 // tile_words[t] .. + tile_len[t].
 int assemble_blob(const Model &m, uint32_t R, uint32_t C, int b, uint32_t V, const float *sigma, float s_info,

@@ -100,3 +100,20 @@ def test_next_scale_error_covers_another_log2_and_exp2(tmp_path):
     worst, neighbours, ordinary = map(float, run())
     assert 0.1 < worst <= 1.0                  # covered, and not by orders of magnitude too much
     assert neighbours > 1e-10 > ordinary       # no fixed 1e-10 covers neighbouring scales
+
+
+def test_payload_room_fits_the_blob(tmp_path):
+    # the blob is laid out before its words are counted: the room must not refuse a blob that is within 32-bit offsets, and a
+    # blob of the returned size always is
+    run = _program(tmp_path, """printf("%llu", (unsigned long long)payload_room(atof(argv[1]), atoll(argv[2]), atoll(argv[3]), atoll(argv[4])));""")
+    room = lambda words, tiles, area, before: int(run(16.0 * words, tiles, area, before)[0])
+    tiles, before = 1 << 20, (1 << 20) * 132 + 500_000
+    for size in (1 << 20, 1 << 28, (1 << 32) - 4_000_000, (1 << 32) - 3):
+        words = (size - before) // 2
+        if words < 0:
+            continue
+        got = room(words, tiles, 1 << 36, before)
+        assert words <= got and before + 2 * got < 1 << 32
+    assert room(1 << 40, 10, 1 << 41, 1000) == 0                      # hopeless
+    assert room(1500, 3, 2000, 1000) == 1501 + 24 + 256           # an ordinary tensor: 0.1 % and a little per tile
+    assert room(1000, 3, 1010, 1000) == 1010                          # never more than the area holds
