@@ -896,7 +896,9 @@ __device__ __forceinline__ uint4 encode_entry(uint32_t fF, uint32_t b) {
     return make_uint4(rcp, f << (31u - b), M - f, sh | (F << 16));
 }
 
-__global__ void encode_entries_kernel(const uint32_t *__restrict__ fF, uint32_t n, uint32_t b, uint4 *__restrict__ entries) {
+// (A kernel that comes up while the one before it runs takes that one's results by ordinary loads: __restrict__ and the
+// read-only path promise that nobody writes the data while the kernel exists, and let a load move above the wait.)
+__global__ void encode_entries_kernel(const uint32_t *fF, uint32_t n, uint32_t b, uint4 *entries) {
     const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
     chained_start();
     if (i < n) entries[i] = encode_entry(fF[i], b);
@@ -940,18 +942,17 @@ constexpr uint32_t kTileThreads = 128, kTileThreadsMax = 512, kSmemEntries = 112
         : "+r"(x), "+r"(end) : "l"(area), "r"(lt), "r"(act), RT(A8), RT(A7), RT(A6), RT(A5), RT(A4), RT(A3), RT(A2), RT(A1), RT(A0) : "memory")
 
 template <bool IN_SMEM>
-__global__ void __launch_bounds__(kTileThreadsMax) tile_encode_kernel(const uint4 *__restrict__ fields, uint32_t n_vec, uint32_t V,
+__global__ void __launch_bounds__(kTileThreadsMax) tile_encode_kernel(const uint4 *fields, uint32_t n_vec, uint32_t V,
                                                                       uint32_t n_tiles, const __grid_constant__ EncodeTables T,
-                                                                      const uint4 *__restrict__ entries_global,
-                                                                      uint16_t *__restrict__ scratch, uint32_t cap,
-                                                                      uint32_t *__restrict__ index, uint32_t *__restrict__ counts, SearchState *state) {
+                                                                      const uint4 *entries_global, uint16_t *scratch, uint32_t cap,
+                                                                      uint32_t *index, uint32_t *counts, SearchState *state) {
     extern __shared__ __align__(16) uint4 entries_smem[];
     __shared__ uint32_t last_cta;
     __shared__ uint64_t part[kTileThreadsMax];
     const uint32_t tid = threadIdx.x, lane = tid & 31u;
     chained_start();
     if (IN_SMEM) {
-        for (uint32_t i = tid; i < T.total; i += blockDim.x) entries_smem[i] = __ldg(entries_global + i);
+        for (uint32_t i = tid; i < T.total; i += blockDim.x) entries_smem[i] = entries_global[i];
         __syncthreads();
     }
     const uint32_t entries = IN_SMEM ? uint32_t(__cvta_generic_to_shared(entries_smem)) : 0u;
@@ -991,7 +992,7 @@ __global__ void __launch_bounds__(kTileThreadsMax) tile_encode_kernel(const uint
                 EP_CODE_GROUP("ld.shared.v4.u32", "r", at[8], at[7], at[6], at[5], at[4], at[3], at[2], at[1], at[0]);
             } else {
                 const uint64_t e0 = reinterpret_cast<uint64_t>(entries_global);
-                EP_CODE_GROUP("ld.global.nc.v4.u32", "l", e0 + at[8], e0 + at[7], e0 + at[6], e0 + at[5], e0 + at[4], e0 + at[3], e0 + at[2],
+                EP_CODE_GROUP("ld.global.v4.u32", "l", e0 + at[8], e0 + at[7], e0 + at[6], e0 + at[5], e0 + at[4], e0 + at[3], e0 + at[2],
                               e0 + at[1], e0 + at[0]);
             }
         }
@@ -1029,9 +1030,8 @@ __global__ void __launch_bounds__(kTileThreadsMax) tile_encode_kernel(const uint
 
 // Move every tile's words from the end of its area to its place in the payload: one CTA per tile (with a warp per tile the
 // copy of 20 MB took 34 us, all of it waiting for loads; 19 so), four bytes per lane, the destination aligned.
-__global__ void __launch_bounds__(512) compact_kernel(const uint16_t *__restrict__ scratch, uint32_t cap,
-                                                                  const uint32_t *__restrict__ counts, const uint32_t *__restrict__ index,
-                                                                  uint16_t *__restrict__ payload) {
+__global__ void __launch_bounds__(512) compact_kernel(const uint16_t *scratch, uint32_t cap, const uint32_t *counts, const uint32_t *index,
+                                                      uint16_t *payload) {
     const uint32_t tid = threadIdx.x, tile = blockIdx.x;
     chained_start();
     uint32_t n = counts[tile];

@@ -1,9 +1,9 @@
 """Host-side parts of the CUDA encoder back end that need no GPU: small programs over csrc/encoder_core.hpp."""
 import os
+import re
 import subprocess
 
 import numpy as np
-import pytest
 
 import paper_2609_34185_b200 as ep
 
@@ -117,3 +117,15 @@ def test_payload_room_fits_the_blob(tmp_path):
     assert room(1 << 40, 10, 1 << 41, 1000) == 0                      # hopeless
     assert room(1500, 3, 2000, 1000) == 1501 + 24 + 256           # an ordinary tensor: 0.1 % and a little per tile
     assert room(1000, 3, 1010, 1000) == 1010                          # never more than the area holds
+
+
+def test_kernels_that_come_up_early_read_by_ordinary_loads():
+    # what the predecessor of such a kernel writes must not be declared read-only in it: the load may then move above the wait
+    text = open(os.path.join(ROOT, "paper_2609_34185_b200", "csrc", "encode_gpu.cu")).read()
+    kernels = {re.search(r"(\w+)\(", k.split(")", 1)[1] if k.startswith(" __launch_bounds__") else k).group(1): k
+               for k in re.split(r"__global__ void", text)[1:]}
+    chained = {name: k.split("\n}\n")[0] for name, k in kernels.items() if "chained_start();" in k.split("\n}\n")[0]}
+    assert {"encode_entries_kernel", "tile_encode_kernel", "compact_kernel"} <= set(chained)
+    assert set(re.findall(r"launch_chained\((\w+_kernel)", text)) <= set(chained)
+    for name, k in chained.items():
+        assert not re.search(r"__restrict__|__ldg\(|\.nc\.", k), name
