@@ -1443,15 +1443,14 @@ struct GemmParams {
 
 constexpr uint32_t kGemmChunk = 256, kGemmSlots = 4;     // payload ring of this kernel
 constexpr uint32_t kGemmRingStride = kGemmChunk * kGemmSlots + kRingMirror;   // 1536
-// what depends on the number of tokens that are staged.  Up to 16: thirty rows of W per step, x in two units of a whole
-// group.  Up to 32 a group's columns of x fill 16 KB, and with no more than that a unit could be asked for only when the
-// instructions of the group before had read it (10240 x 3840, 32 tokens: 80.9 us): 24 rows per step make room for 32 KB,
-// four units of half a group each.
-template <uint32_t TPAD>
+// what depends on the rows per step.  Thirty leave 16 KB for x: two units of a whole group for up to 16 tokens, of half a group
+// for up to 32, and then a unit can be asked for only when the instructions half a group before have read it.  24 make room for
+// 32 KB, four units of half a group each, for up to 32 tokens; where that takes more steps it is the slower one (see the launcher).
+template <uint32_t ROWS>
 struct GemmShape {
-    static constexpr uint32_t kRows = TPAD == 16 ? 30 : 24;              // most rows of W per step: one per decoding warp
-    static constexpr uint32_t kN = TPAD == 16 ? 32 : 24;                 // rows of the B operand
-    static constexpr uint32_t kUnits = TPAD == 16 ? 2 : 4;               // units of x, 8 KB each
+    static constexpr uint32_t kRows = ROWS;                              // most rows of W per step: one per decoding warp
+    static constexpr uint32_t kN = (ROWS + 7u) & ~7u;                    // rows of the B operand
+    static constexpr uint32_t kUnits = ROWS > 24 ? 2 : 4;                // units of x, 8 KB each
     static constexpr uint32_t kBTile = kN * 128, kSlab = 4 * kBTile;     // B: per slab four 64-column tiles of kN rows
     static constexpr uint32_t kA = (kRingBase + kRows * kGemmRingStride + 1023u) & ~1023u;   // A operand (swizzled tiles start on 1024-byte boundaries)
     static constexpr uint32_t kB = kA + kUnits * 8192;
@@ -1600,7 +1599,7 @@ __device__ __forceinline__ void umma_commit(uint32_t bar) {
           "r"(P.groups), "r"(b_dst), "r"(bar_mma), "r"(bar_b), "n"(G::kSlab), "n"(kSpinLimit)                         \
         : "memory")
 
-template <uint32_t TPAD>
+template <uint32_t TPAD, uint32_t ROWS>
 __global__ void __launch_bounds__(kThreads, 1) ep_decode_gemm_kernel(const __grid_constant__ GemmParams P,
                                                                      const __grid_constant__ CUtensorMap x_map) {
     extern __shared__ __align__(16) uint8_t smem[];      // (the operand tiles need 1024: checked at run time, see abort word)
@@ -1609,7 +1608,7 @@ __global__ void __launch_bounds__(kThreads, 1) ep_decode_gemm_kernel(const __gri
     // of the decoding loop, which cost 500 of 1700 cycles per group)
     const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = __shfl_sync(0xFFFFFFFFu, tid >> 5, 0);
     const uint32_t lut_addr = uint32_t(__cvta_generic_to_shared(smem));
-    using G = GemmShape<TPAD>;
+    using G = GemmShape<ROWS>;
     const uint32_t a_base = lut_addr + G::kA, b_base = lut_addr + G::kB;
     // A holds two or four units of x: four tiles of 64 columns x 16 rows each (one group's columns), or two tiles x 32 rows
     // (half a group's).  Per unit one mbarrier "landed" and one "read"; per slab of B one "rows stored" and one "read".
@@ -2609,17 +2608,24 @@ extern "C" int ep_decode_gemm(const ep_info *info, const void *d_stream, const v
     // rows spread evenly over the SMs, and a CTA's rows over the fewest steps (thirty warps share an SM's issue slots: three
     // steps of 24 rows take less time than 30 + 30 + 10)
     P.rows_per_cta = (I.R + uint32_t(sms) - 1u) / uint32_t(sms);
-    const uint32_t most = P.Tpad == 16u ? GemmShape<16>::kRows : GemmShape<32>::kRows;
-    P.steps = (P.rows_per_cta + most - 1u) / most;
+    auto steps_of = [&](uint32_t rows) { return (P.rows_per_cta + rows - 1u) / rows; };
+    // 17 to 32 tokens: the shape that takes fewer steps, else that with four units of x.  4096 columns at 4 bpp, 32 tokens, us,
+    // steps of 24 / 30 rows at most: 10 rows per SM 19.9 / 20.3, 23: 23.5 / 24.0, 28: 37.0 / 26.2, 56: 57.5 / 48.5, 70: 65.6 / 63.9,
+    // 91: 79.5 / 81.0, 120: 108.2 / 91.9.
+    const uint32_t most = P.Tpad == 16u || steps_of(30u) < steps_of(24u) ? 30u : 24u;
+    P.steps = steps_of(most);
     P.rows_per_step = (P.rows_per_cta + P.steps - 1u) / P.steps;
     P.groups = I.C / 256u;
     if (I.n_tiles != I.R) return EP_ERR_BAD_ARG;
+    const auto kernel = P.Tpad == 16u ? ep_decode_gemm_kernel<16, 30> : most == 30u ? ep_decode_gemm_kernel<32, 30> : ep_decode_gemm_kernel<32, 24>;
+    const uint32_t smem = most == 30u ? GemmShape<30>::kSmem : GemmShape<24>::kSmem;
     static bool configured[64] = {};
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return EP_ERR_CUDA;
     if (dev < 0 || dev >= 64 || !configured[dev]) {
-        if (cudaFuncSetAttribute(ep_decode_gemm_kernel<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(GemmShape<16>::kSmem)) != cudaSuccess ||
-            cudaFuncSetAttribute(ep_decode_gemm_kernel<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(GemmShape<32>::kSmem)) != cudaSuccess)
+        if (cudaFuncSetAttribute(ep_decode_gemm_kernel<16, 30>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(GemmShape<30>::kSmem)) != cudaSuccess ||
+            cudaFuncSetAttribute(ep_decode_gemm_kernel<32, 30>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(GemmShape<30>::kSmem)) != cudaSuccess ||
+            cudaFuncSetAttribute(ep_decode_gemm_kernel<32, 24>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(GemmShape<24>::kSmem)) != cudaSuccess)
             return EP_ERR_CUDA;
         if (dev >= 0 && dev < 64) configured[dev] = true;
     }
@@ -2642,9 +2648,7 @@ extern "C" int ep_decode_gemm(const ep_info *info, const void *d_stream, const v
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
         return EP_ERR_CUDA;
     const uint32_t threads = 32u * (2u + P.rows_per_step < kMinWarps ? kMinWarps : 2u + P.rows_per_step);
-    const cudaError_t e = P.Tpad == 16u ? launch_next(ep_decode_gemm_kernel<16>, grid, threads, GemmShape<16>::kSmem, st, P, x_map)
-                                        : launch_next(ep_decode_gemm_kernel<32>, grid, threads, GemmShape<32>::kSmem, st, P, x_map);
-    return e == cudaSuccess ? EP_OK : EP_ERR_CUDA;
+    return launch_next(kernel, grid, threads, smem, st, P, x_map) == cudaSuccess ? EP_OK : EP_ERR_CUDA;
 }
 
 extern "C" int ep_last_device_status(void *stream) {

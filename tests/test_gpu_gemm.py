@@ -104,6 +104,24 @@ def test_decode_matmul_at_the_edges_of_its_steps(R, C, T):
     _check(blob, T, R + C + T)
 
 
+@pytest.mark.parametrize("R,C,T", [
+    (148 * 25, 256, 32),          # one step of 25 rows, a single group per row: both units of x in one group
+    (148 * 30, 512, 17),          # one full step
+    (148 * 28 - 3, 1024, 32),     # a last CTA with fewer rows
+    (148 * 60, 256, 20),          # two full steps
+    (148 * 73, 512, 32),          # three steps of 25 rows instead of four of 19
+])
+def test_decode_matmul_of_17_to_32_tokens_in_thirty_rows(R, C, T):
+    rng = np.random.default_rng(77)
+    n = R * C // 8
+    fields = np.zeros((n, 9), np.int32)
+    fields[:, 0] = rng.integers(0, 2, n)
+    fields[:, 1:8] = np.rint(rng.standard_normal((n, 7)) * 4).astype(np.int32)
+    fields[:, 8] = np.rint(rng.standard_normal(n) * 2).astype(np.int32)
+    blob = ep.pack_fields(fields, R, C, 11, C // 8, rng.uniform(0.01, 0.05, R).astype(np.float32))
+    _check(blob, T, R + C + T)
+
+
 def test_decode_matmul_more_tokens_than_one_launch_and_repeated_calls():
     W = synth.gaussian_rows(128, 1536, 71)
     blob = ep.encode(W, 4.0, tile_vectors=1536 // 8)
