@@ -48,7 +48,10 @@ constexpr uint32_t kTilesPerRound = kWarps * kChains;        // tiles per CTA at
 // Most tiles per CTA for decode_tile_few: its 512 threads may use 128 registers.  1792-block tiles at 4 bpp to BF16, us, this
 // loop / the ordinary one: 4 tiles 37.1 / 40.0, 8: 38.7 / 41.3, 12: 41.8 / 43.8, 16: 45.4 / 46.6.
 constexpr uint32_t kFewTiles = 16;
-constexpr uint32_t kMinWarps = 8;                            // threads that copy the tables, however few tiles a CTA has
+constexpr uint32_t kMinWarps = 8;                            // warps of a CTA, however few tiles it has
+// ... that builds its tables itself: a warp per table (1024 x 1024 at 6 bpp in tiles of 64 blocks, no prepared image, us: 8 warps
+// 13.3, 16 warps 9.8).
+constexpr uint32_t kBuildWarps = EP_NUM_TABLES - 1;
 static_assert(kTilesPerRound == ep::kDecodeTilesPerCta, "tile-size suggestions assume this many tiles per CTA");
 constexpr uint32_t kLutEntries = 2048;                       // 2^11 slots per table
 constexpr uint32_t kLutStride = kLutEntries * 4;             // bytes per table in shared memory
@@ -2208,7 +2211,10 @@ cudaError_t launch_smem_as(const BatchParams &P, uint32_t grid, uint32_t warps, 
         if (e != cudaSuccess) return e;
         if (dev >= 0 && dev < 64) configured[dev] = true;
     }
-    return launch_next(ep_decode_smem_kernel<DT, FEW>, grid, 32u * (warps < kMinWarps ? kMinWarps : warps), kSmemBytes, st, P);
+    uint32_t least = kMinWarps;
+    for (int i = 0; i < P.n_jobs; ++i)
+        if (!P.job[i].lut_image) least = kBuildWarps;
+    return launch_next(ep_decode_smem_kernel<DT, FEW>, grid, 32u * (warps < least ? least : warps), kSmemBytes, st, P);
 }
 template <int DT>
 cudaError_t launch_smem(const BatchParams &P, uint32_t grid, cudaStream_t st) {

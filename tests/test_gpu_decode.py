@@ -646,3 +646,27 @@ def test_few_tiles_damaged_payload_is_flagged_not_fatal():
     torch.cuda.synchronize()
     assert ep.last_device_status() == -2
     _check(blob, (ep.BF16,))
+
+
+@pytest.mark.parametrize("R,C,V,b", [
+    (512, 512, 32768, 11),       # one tile, sixteen warps that build a table each
+    (1024, 1024, 64, 11),        # 14 tiles per CTA
+    (1184, 512, 64, 11),         # eight
+    (2369, 512, 64, 11),         # 17: the ordinary loop
+    (400, 264, 100, 9),          # the plain loop
+])
+def test_tables_built_by_the_cta_with_any_number_of_tiles(R, C, V, b):
+    rng = np.random.default_rng(9300 + R)
+    n = R * C // 8
+    fields = np.zeros((n, 9), np.int32)
+    fields[:, 0] = rng.integers(0, 2, n)
+    fields[:, 1:8] = np.rint(rng.standard_normal((n, 7)) * 6).astype(np.int32)
+    fields[:, 8] = np.rint(rng.standard_normal(n) * 3).astype(np.int32)
+    blob = ep.pack_fields(fields, R, C, b, V, rng.uniform(0.01, 0.05, R).astype(np.float32))
+    built, prepared = ep.upload(blob, prepare=False), ep.upload(blob)
+    want = oracle.decode(blob.data, oracle.BF16)[0]
+    assert np.array_equal(_bits(ep.decode(built, ep.BF16)), want)
+    outs = [torch.empty(R, C, dtype=torch.bfloat16, device="cuda") for _ in range(3)]
+    ep.decode_many([prepared, built, built], ep.BF16, outs)         # both kinds of job in one launch
+    torch.cuda.synchronize()
+    assert all(np.array_equal(_bits(o), want) for o in outs) and ep.last_device_status() == 0
