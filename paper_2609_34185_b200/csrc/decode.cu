@@ -293,7 +293,9 @@ __device__ __forceinline__ void copy_tables_smem(const uint32_t *image, uint32_t
 
 // How the job's lookup tables come about, and the wait for them.  All branches are on votes or parameters (a guard around each
 // vote of the hot loop costs more than the wait).  A copy that does not end within the limit - there is no such case -
-// raises the integrity word; the tables then hold anything, which is safe (see build_one_table) but wrong.
+// raises the integrity word and ends the warp, whose tiles are not written: what an SM's shared memory held before has neither
+// frequencies of at least 1 nor codes inside the second level, which the loops' addresses rely on.  (A barrier that waits for
+// all threads of a CTA does not wait for those that have ended, and only a warp that saw a phase end arms the next one.)
 enum TablesPending : uint32_t { kTablesThere, kTablesBuilt, kTablesCopied };   // nothing to wait for; this CTA's stores; the copy
 struct TablesWait { uint32_t pending, bar, parity; };
 static_assert(EP_MAX_BATCH <= kWarps);
@@ -301,19 +303,19 @@ constexpr uint32_t kSpinLimit = 1u << 18;             // attempts of about a mic
 __device__ __forceinline__ void wait_for_tables(const TablesWait &W) {
     if (W.pending == kTablesBuilt) __syncthreads();
     if (W.pending == kTablesCopied) {
-        uint32_t left;
-        asm volatile("{\n\t.reg .pred p;\n\tmov.b32 %0, %3;\n\t"
+        asm volatile("{\n\t.reg .pred p;\n\t.reg .b32 left;\n\tmov.b32 left, %2;\n\t"
                      "EP_TABLES_WAIT:\n\t"
-                     "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, 1000;\n\t"
+                     "mbarrier.try_wait.parity.shared::cta.b64 p, [%0], %1, 1000;\n\t"
                      "vote.sync.all.pred p, p, 0xffffffff;\n\t"
                      "@p bra.uni EP_TABLES_DONE;\n\t"
-                     "sub.u32 %0, %0, 1;\n\t"
-                     "setp.ne.u32 p, %0, 0;\n\t"
+                     "sub.u32 left, left, 1;\n\t"
+                     "setp.ne.u32 p, left, 0;\n\t"
                      "vote.sync.all.pred p, p, 0xffffffff;\n\t"
                      "@p bra.uni EP_TABLES_WAIT;\n\t"
+                     "red.global.or.b32 [%3], 2;\n\t"
+                     "exit;\n\t"
                      "EP_TABLES_DONE:\n\t}"
-                     : "=&r"(left) : "r"(W.bar), "r"(W.parity), "n"(kSpinLimit) : "memory");
-        if (left == 0) atomicOr(&g_ep_status, 2u);
+                     ::"r"(W.bar), "r"(W.parity), "n"(kSpinLimit), "l"(&g_ep_status) : "memory");
     }
 }
 

@@ -1,6 +1,9 @@
 """GPU parity: the fused CUDA decoder against the oracle, element by element, through the C ABI.
 Both directions (library stream -> oracle decoder is covered on CPU; here library stream and oracle
 stream -> GPU decoder), all output types, ragged shapes, and the full-size benchmark configurations."""
+import os
+import subprocess
+
 import numpy as np
 import pytest
 import torch
@@ -670,3 +673,14 @@ def test_tables_built_by_the_cta_with_any_number_of_tiles(R, C, V, b):
     ep.decode_many([prepared, built, built], ep.BF16, outs)         # both kinds of job in one launch
     torch.cuda.synchronize()
     assert all(np.array_equal(_bits(o), want) for o in outs) and ep.last_device_status() == 0
+
+
+def test_wait_for_a_table_image_that_never_comes_ends_the_warps(tmp_path):
+    # the limit of the wait: status set, no warp goes on with the tables, the CTA's barriers still open
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    csrc, exe = os.path.join(root, "paper_2609_34185_b200", "csrc"), str(tmp_path / "tables_wait")
+    subprocess.run([os.environ.get("NVCC") or "/usr/local/cuda/bin/nvcc", "-gencode", "arch=compute_100a,code=sm_100a", "-std=c++17",
+                    "-Xcompiler", "-pthread", "-I", os.path.join(root, "include"), "-I", csrc, "-o", exe,
+                    os.path.join(root, "tests", "tables_wait.cu"), os.path.join(csrc, "stream.cpp")], check=True)
+    out = subprocess.run([exe], check=True, capture_output=True, text=True, timeout=60).stdout.split()
+    assert out == ["-2", "0", "32"]
