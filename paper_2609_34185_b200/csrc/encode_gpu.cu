@@ -1210,7 +1210,15 @@ public:
         F.lo0 = o.bracket_lo;
         F.hi0 = o.bracket_hi;
         F.last_step = o.polish_steps;
-        for (F.step = 0; F.step <= o.polish_steps; ++F.step) EP_CUDA(launch_count(F, F.step > 0 || o.search_steps > 0));
+        for (F.step = 0;; ++F.step) {
+            EP_CUDA(launch_count(F, F.step > 0 || o.search_steps > 0));
+            if (F.step == o.polish_steps) break;
+            if (F.step % 8 == 7) {               // a caller may allow any number of corrections: is there still something to correct?
+                EP_CUDA(cudaMemcpyAsync(&state()->stop, &w_.state->stop, sizeof(state()->stop), cudaMemcpyDeviceToHost, st_));
+                EP_CUDA(cudaStreamSynchronize(st_));
+                if (state()->stop) break;
+            }
+        }
         // the row scales of the quantisation that is there now: while the host looks at the counts the GPU has nothing else to
         // do (and if the host goes on to another scale, finish makes them again)
         const int rc = fetch(true, [&] {

@@ -148,3 +148,17 @@ def test_device_encoder_bytes_with_cosets_that_do_not_meet(bpp):
     host = ep.encode(W, bpp)
     dev = ep.encode_device(torch.from_numpy(W).cuda(), bpp)
     assert np.array_equal(dev.data, host.data) and dev.report == host.report
+
+
+@pytest.mark.timeout(60)
+@pytest.mark.parametrize("maker,bpp,steps", [
+    (synth.gaussian_rows, 4.0, 2**31 - 1),        # as many corrections as it takes, which are few
+    (synth.laplace_rows, 6.0, 1000),
+    (synth.laplace_rows, 6.0, 7),                 # the last pass before the device is asked whether it has stopped
+    (synth.laplace_rows, 6.0, 8),
+])
+def test_device_encoder_with_any_number_of_rate_corrections(maker, bpp, steps):
+    W = maker(64, 1024, 21)
+    host = ep.encode(W, bpp, polish_steps=steps)
+    dev = ep.encode_device(torch.from_numpy(W).cuda(), bpp, polish_steps=steps)
+    assert np.array_equal(dev.data, host.data) and dev.report == host.report
