@@ -30,21 +30,13 @@
 
 namespace {
 
-// Tiles a warp decodes side by side (1 to 4) and warps per CTA.  The loop below is written for any number of
-// chains per warp, their instructions interleaved line by line; measured on B200 (8192 x 8192 at 4 bpp to FP16 /
-// the 372 M-parameter layer at 3.5 bpp to BF16, Gparams/s): 32 warps x 1 chain 985 / 1171, 24 x 2 940 / 1104,
-// 16 x 3 781 / 889, 12 x 4 677 / 744.  The loop is bound by the issue slots, the ALU pipe and the shared-memory
-// pipe together (each about 70 % busy), not by the latency of one chain: what counts is the number of warps.
-#ifndef EP_CHAINS
-#define EP_CHAINS 1
-#endif
-#ifndef EP_WARPS
-#define EP_WARPS (EP_CHAINS == 1 ? 32 : 48 / EP_CHAINS)
-#endif
-constexpr uint32_t kChains = EP_CHAINS;
-constexpr int kWarps = EP_WARPS;                             // warps per CTA (one CTA per SM)
+// A warp decodes one tile at a time.  Two, three or four with their instructions interleaved and 24, 16 or 12 warps were slower
+// (8192 x 8192 at 4 bpp to FP16 / the 372 M-parameter layer at 3.5 bpp to BF16, Gparams/s: 32 warps with one 985 / 1171, 24 with two
+// 940 / 1104, 16 with three 781 / 889, 12 with four 677 / 744): the loop is bound by the issue slots, the ALU pipe and the
+// shared-memory pipe together (each about 70 % busy), not by the latency of one tile's chain of steps.
+constexpr int kWarps = 32;                                   // warps per CTA (one CTA per SM)
 constexpr int kThreads = kWarps * 32;
-constexpr uint32_t kTilesPerRound = kWarps * kChains;        // tiles per CTA at a time, at most (see split_rounds)
+constexpr uint32_t kTilesPerRound = kWarps;                  // tiles per CTA at a time, at most (see split_rounds)
 // Most tiles per CTA for decode_tile_few: its 512 threads may use 128 registers.  1792-block tiles at 4 bpp to BF16, us, this
 // loop / the ordinary one: 4 tiles 37.1 / 40.0, 8: 38.7 / 41.3, 12: 41.8 / 43.8, 16: 45.4 / 46.6.
 constexpr uint32_t kFewTiles = 16;
@@ -57,25 +49,24 @@ constexpr uint32_t kLutEntries = 2048;                       // 2^11 slots per t
 constexpr uint32_t kLutStride = kLutEntries * 4;             // bytes per table in shared memory
 constexpr uint32_t kCosetStride = 8 * kLutStride;            // the eight tables of coset 1 follow those of coset 0
 constexpr uint32_t kLutBytes = 16 * kLutStride;              // 131072
-// Payload ring of a chain: three chunks of 512 bytes (one cp.async round of a warp, 16 bytes per lane) plus a mirror
+// Payload ring of a tile: three chunks of 512 bytes (one cp.async round of a warp, 16 bytes per lane) plus a mirror
 // of its first 512 bytes.  (Measured and dropped: 64 rings of four 256-byte chunks for two tiles per warp at 32 warps.)
 constexpr uint32_t kChunk = 512, kRingSlots = 3;
 constexpr uint32_t kRingBytes = kRingSlots * kChunk;         // 1536
 constexpr uint32_t kRingMirror = 512;                        // >= 7 words * 32 lanes * 2 bytes + one lane span (62)
-constexpr uint32_t kRingStride = kRingBytes + kRingMirror;   // 2048 per chain
-constexpr uint32_t kCtxBytes = 32 + 32 * kChains;            // per warp: what the rare paths of the hot loop need
+constexpr uint32_t kRingStride = kRingBytes + kRingMirror;   // 2048 per warp
+constexpr uint32_t kCtxBytes = 64;                           // per warp: what the rare paths of the hot loop need
 constexpr uint32_t kCtxBase = kLutBytes;
 constexpr uint32_t kRingBase = kCtxBase + kWarps * kCtxBytes;
 // 2^12-slot streams: per table, the entries of the kHotSpan coordinate values around zero are kept in shared memory
-// (the rest is read from global memory); this fills what the tables, rings and context blocks of the 32-warp build
+// (the rest is read from global memory); this fills what the tables, rings and context blocks
 // leave of the 227 KB
 constexpr uint32_t kHotSpan = 528;                           // coordinate codes per table in the hot window
 constexpr uint32_t kHotBytes = 16 * kHotSpan * 4;            // 33792
 constexpr uint32_t kColdCodes = 4096;                        // codes per table in the complete entry array (global memory)
 constexpr uint32_t kColdBytes = 16 * kColdCodes * 4;         // 262144
-constexpr uint32_t kHotBase = kRingBase + kWarps * kChains * kRingStride;
-constexpr bool kTwoLevelInLoop = EP_CHAINS == 1 && kHotBase + kHotBytes <= 232448;
-constexpr uint32_t kSmemBytes = kHotBase + (kTwoLevelInLoop ? kHotBytes : 0);   // 232448 in the default build
+constexpr uint32_t kHotBase = kRingBase + kWarps * kRingStride;
+constexpr uint32_t kSmemBytes = kHotBase + kHotBytes;          // 232448
 static_assert(kSmemBytes <= 232448, "more shared memory than an sm_100 CTA can have");
 constexpr uint32_t kStageBytes = kSmemBytes - kRingBase;     // with few tiles per CTA: room for their whole payloads (see decode_tile_few)
 constexpr uint32_t kCodeMask = 0x001FF800u;                  // 10-bit code field
@@ -83,13 +74,13 @@ constexpr uint32_t kExp4096 = 0x45800000u;                   // fp32 bit pattern
 constexpr uint32_t kOwnSlots = 16;                           // table build: slots of a symbol that its own lane writes
 constexpr uint32_t kEntryUnused = 1u << 21;                  // f = 1: what a slot no symbol owns holds (damaged tables)
 
-// per-warp context block (byte offsets); chain c has its part at kCtxChain + c * kCtxChainStride
+// per-warp context block (byte offsets): the job's part, and the tile's from kCtxChain on
 constexpr uint32_t kCtxScales = 0;         // u64 row scales
 constexpr uint32_t kCtxRowBytes = 8;       // u32 output bytes per row
 constexpr uint32_t kCtxRowMax = 12;        // u32 last row index
 constexpr uint32_t kCtxTablesBar = 16;     // u64 mbarrier of the table image's copy (warp j's: of job j's, see ep_decode_smem_kernel)
 constexpr uint32_t kCtxRowRcp = 24;        // u32 ceil(2^32 / bytes per row)
-constexpr uint32_t kCtxChain = 32, kCtxChainStride = 32;
+constexpr uint32_t kCtxChain = 32;
 constexpr uint32_t kCcSrc = 0;             // u64 global address of lane 0's 16 bytes of the next chunk to request
 constexpr uint32_t kCcRem = 8;             // s32 payload bytes from there to the end of the payload (may be <= 0)
 constexpr uint32_t kCcDst = 12;            // u32 ring address of lane 0's 16 bytes of that chunk's slot
@@ -132,7 +123,7 @@ struct JobParams {
 struct BatchParams {
     JobParams job[EP_MAX_BATCH];
     uint32_t cost_per_cta;        // ceil(sum of rounds * round_cost over all jobs / CTAs of the launch)
-    uint32_t tiles_per_round;     // tiles a CTA works on at a time: one per warp and chain, at most kTilesPerRound
+    uint32_t tiles_per_round;     // tiles a CTA works on at a time: one per warp, at most kTilesPerRound
     int32_t n_jobs;
 };
 
@@ -282,13 +273,13 @@ __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
 __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 __device__ __forceinline__ void copy_tables_smem(const uint32_t *image, uint32_t lut_addr, uint32_t bar, bool two_level) {
     constexpr uint32_t kPiece = 32768;
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(kLutBytes + (kTwoLevelInLoop && two_level ? kHotBytes : 0u)) : "memory");
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(kLutBytes + (two_level ? kHotBytes : 0u)) : "memory");
     auto piece = [&](uint32_t dst, uint32_t src, uint32_t bytes) {
         asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                      ::"r"(dst), "l"(reinterpret_cast<uint64_t>(image) + src), "r"(bytes), "r"(bar) : "memory");
     };
     for (uint32_t o = 0; o < kLutBytes; o += kPiece) piece(lut_addr + o, o, kPiece);
-    if (kTwoLevelInLoop && two_level) piece(lut_addr + kHotBase, kLutBytes, kHotBytes);      // the hot part of the second level follows the image
+    if (two_level) piece(lut_addr + kHotBase, kLutBytes, kHotBytes);      // the hot part of the second level follows the image
 }
 
 // How the job's lookup tables come about, and the wait for them.  All branches are on votes or parameters (a guard around each
@@ -524,7 +515,7 @@ __device__ __forceinline__ void ring_service(uint32_t ring, uint64_t a0, uint32_
     threshold = CHUNK * (cur + 1u);
 }
 
-// what a chain needs to know about its tile
+// what a warp needs to know about its tile
 struct TileSetup {
     uint32_t x;            // this lane's state, forced into [2^15, 2^31) (a no-op for a valid stream)
     uint32_t off, end;     // first payload word of the tile and of the next one
@@ -584,155 +575,84 @@ __device__ __forceinline__ void decode_tile_plain(const JobParams &J, uint32_t t
     if (__any_sync(0xFFFFFFFFu, bad) && lane == 0) atomicOr(&g_ep_status, 1u);
 }
 
-// ---- the hot loop in PTX: several tiles per warp ----------------------------------------------------------
-// All groups of EP_CHAINS tiles ("chains" A, B, ...), written as one asm statement so that every branch can be
-// marked warp-uniform (bra.uni), the chains' instructions can be interleaved, and the rare work - refilling a
-// payload ring, moving to the next row, a tile's end - sits out of line behind ONE warp vote per loop pass.
+// ---- the hot loop in PTX -------------------------------------------------------------------------------------
+// All groups of a tile, written as one asm statement so that every branch can be marked warp-uniform (bra.uni) and the rare
+// work - refilling the payload ring, moving to the next row, the tile's end - sits out of line behind ONE warp vote per loop
+// pass.
 //
-// Word addresses.  Lane l of a chain keeps its own address a_l of the word it would take in the current step.
+// Word addresses.  Lane l keeps its own address a_l of the word it would take in the current step.
 // With bal_k the ballot of the lanes that need a word after step k,
 //     a_l(k) = a_l(k-1) + 2 popc((bal_k & below_l) | (bal_{k-1} & ~below_l)):
 // the words taken in step k-1 by lanes l and above, plus those taken in step k by the lanes below.  The two
 // masks are disjoint, so one bit-select and ONE population count per step replace the prefix count and the
 // cursor advance (lane 0's address is the tile's word cursor before the step).
 //
-// Loop-carried per chain: x state, a word address, bal last ballot, doff byte offset of this lane's block in the
+// Loop-carried: x state, a word address, bal last ballot, doff byte offset of this lane's block in the
 // output; inside the asm: lim = first doff at which this lane leaves its row or the tile, wthr = ring address at
 // which the cursor leaves its 512-byte chunk (minus 2), ss = the row scale twice, act = lane has a block.
-// A chain whose tile has ended (or that never had one) runs along with all lanes inactive: states and
-// addresses stand still, nothing is stored.
+// A warp without a tile runs with all lanes inactive: states and addresses stand still, nothing is stored.
 //
-// asm operands: chain c has x, a, bal, doff at %(4c) .. %(4c+3); then come the shared inputs, named here:
-#if EP_CHAINS == 1
-#define EP_LT "%4"
-#define EP_LUT0 "%5"
-#define EP_LUT1 "%6"
-#define EP_CTX "%7"
-#define EP_KK "%8"
-#define EP_OUT "%9"
-#define EP_F0 "%10"
-#define EP_F1 "%11"
-#define EP_L16 "%12"
-#define EP_L2B "%13"
-#define EP_HS2 "%14"
-#define EP_HOTOFF "%15"
-#elif EP_CHAINS == 2
-#define EP_LT "%8"     /* lanes below this one (mask) */
-#define EP_LUT0 "%9"   /* tables of coset 0 */
-#define EP_LUT1 "%10"  /* tables of coset 1 */
-#define EP_CTX "%11"   /* this warp's context block */
-#define EP_KK "%12"    /* {4096 - zlo, 4096 - zlo} as fp32 pair */
-#define EP_OUT "%13"   /* output base address */
-#define EP_F0 "%14"    /* frequency of coset 0 */
-#define EP_F1 "%15"    /* frequency of coset 1, at least 1 */
-#define EP_L16 "%16"   /* 16 * lane */
-#define EP_L2B "%17"   /* 2^12-slot streams: the complete second-level array (global memory), */
-#define EP_HS2 "%18"   /* twice the first code of the hot window, */
-#define EP_HOTOFF "%19"  /* offset of the hot part in shared memory */
-#elif EP_CHAINS == 3
-#define EP_LT "%12"
-#define EP_LUT0 "%13"
-#define EP_LUT1 "%14"
-#define EP_CTX "%15"
-#define EP_KK "%16"
-#define EP_OUT "%17"
-#define EP_F0 "%18"
-#define EP_F1 "%19"
-#define EP_L16 "%20"
-#define EP_L2B "%21"
-#define EP_HS2 "%22"
-#define EP_HOTOFF "%23"
-#else
-#define EP_LT "%16"
-#define EP_LUT0 "%17"
-#define EP_LUT1 "%18"
-#define EP_CTX "%19"
-#define EP_KK "%20"
-#define EP_OUT "%21"
-#define EP_F0 "%22"
-#define EP_F1 "%23"
-#define EP_L16 "%24"
-#define EP_L2B "%25"
-#define EP_HS2 "%26"
-#define EP_HOTOFF "%27"
-#endif
-// one macro call per chain: M(S = suffix, X, AW, BAL, DOFF, CB = byte offset of the chain's context, more...)
-#define EP_CH_A(M, ...) M("A", "%0", "%1", "%2", "%3", "32", ##__VA_ARGS__)
-#define EP_CH_B(M, ...) M("B", "%4", "%5", "%6", "%7", "64", ##__VA_ARGS__)
-#define EP_CH_C(M, ...) M("C", "%8", "%9", "%10", "%11", "96", ##__VA_ARGS__)
-#define EP_CH_D(M, ...) M("D", "%12", "%13", "%14", "%15", "128", ##__VA_ARGS__)
-#if EP_CHAINS == 1
-#define EP_ALL(M, ...) EP_CH_A(M, ##__VA_ARGS__)
-#elif EP_CHAINS == 2
-#define EP_ALL(M, ...) EP_CH_A(M, ##__VA_ARGS__) EP_CH_B(M, ##__VA_ARGS__)
-#elif EP_CHAINS == 3
-#define EP_ALL(M, ...) EP_CH_A(M, ##__VA_ARGS__) EP_CH_B(M, ##__VA_ARGS__) EP_CH_C(M, ##__VA_ARGS__)
-#else
-#define EP_ALL(M, ...) EP_CH_A(M, ##__VA_ARGS__) EP_CH_B(M, ##__VA_ARGS__) EP_CH_C(M, ##__VA_ARGS__) EP_CH_D(M, ##__VA_ARGS__)
-#endif
+// asm operands: x, a, bal, doff are %0 .. %3; then come the inputs, named here:
+#define EP_LT "%4"      /* lanes below this one (mask) */
+#define EP_LUT0 "%5"    /* tables of coset 0 */
+#define EP_LUT1 "%6"    /* tables of coset 1 */
+#define EP_CTX "%7"     /* this warp's context block */
+#define EP_KK "%8"      /* {4096 - zlo, 4096 - zlo} as fp32 pair */
+#define EP_OUT "%9"     /* output base address */
+#define EP_F0 "%10"     /* frequency of coset 0 */
+#define EP_F1 "%11"     /* frequency of coset 1, at least 1 */
+#define EP_L16 "%12"    /* 16 * lane */
+#define EP_L2B "%13"    /* 2^12-slot streams: the complete second-level array (global memory), */
+#define EP_HS2 "%14"    /* twice the first code of the hot window, */
+#define EP_HOTOFF "%15" /* offset of the hot part in shared memory */
 
 #define EP_CM "0x1FF800"
-// The loop body is written line by line: every macro below emits ONE instruction for ONE chain, and EP_ALL
-// repeats it for all chains before the next line follows.  The assembler keeps this order, so a chain's next
-// dependent instruction comes only after the other chains' same instruction: that distance, not the
-// scheduler, is what hides the latencies inside a warp.
-// Common parameters of a line: S, X, AW, BAL, DOFF, CB (see EP_CH_A); then E = name of the entry register
-// (a suffix is added), OFF = byte offset of the field's table, BIN / BOUT = which register holds the previous /
-// receives the new ballot: NA, NB (temporaries) or BL (the chain's loop-carried operand).
-#define EP_B_NA(S, BAL) "na" S
-#define EP_B_NB(S, BAL) "nb" S
-#define EP_B_BL(S, BAL) BAL
+// One macro per line of the loop body.  E = name of the entry register (a suffix is added), OFF = byte offset of the field's table,
+// BIN / BOUT = the register that holds the previous / receives the new ballot.
 // a coordinate field: table OFF / 8192 of the lane's coset (Eq. 18)
 // slot address 4 (x & 0x7FF) + tab as 4 x - 8192 (x >> 11) + tab: two multiply-adds instead of a mask and one (the
 // multiply-add pipe has room, the ALU pipe has not; measured + 0.3 % / + 0.8 % on the 8192^2 tensor / the layer)
-#define EP_L1(S, X, AW, BAL, DOFF, CB, E, OFF, BIN, BOUT) "shr.u32 q" S ", " X ", 11;\n\t" "mad.lo.u32 u" S ", q" S ", 0xFFFFE000, tab" S ";\n\t"
-#define EP_L2(S, X, AW, BAL, DOFF, CB, E, OFF, BIN, BOUT) "mad.lo.u32 u" S ", " X ", 4, u" S ";\n\t"
-#define EP_L3(S, X, AW, BAL, DOFF, CB, E, OFF, BIN, BOUT) "ld.shared.u32 " E S ", [u" S "+" OFF "];\n\t"
-#define EP_L5(S, X, AW, BAL, DOFF, CB, E, OFF, BIN, BOUT) "shr.u32 f" S ", " E S ", 21;\n\t"
-#define EP_L6(S, X, AW, BAL, DOFF, CB, E, OFF, BIN, BOUT) "and.b32 bi" S ", " E S ", 0x7FF;\n\t"
-#define EP_L7(S, X, AW, BAL, DOFF, CB, E, OFF, BIN, BOUT) "@act" S " mad.lo.u32 " X ", f" S ", q" S ", bi" S ";\n\t"
+#define EP_L1 "shr.u32 qA, %0, 11;\n\t" "mad.lo.u32 uA, qA, 0xFFFFE000, tabA;\n\t"
+#define EP_L2 "mad.lo.u32 uA, %0, 4, uA;\n\t"
+#define EP_L3(E, OFF) "ld.shared.u32 " E "A, [uA+" OFF "];\n\t"
+#define EP_L5(E) "shr.u32 fA, " E "A, 21;\n\t"
+#define EP_L6(E) "and.b32 biA, " E "A, 0x7FF;\n\t"
+#define EP_L7 "@actA mad.lo.u32 %0, fA, qA, biA;\n\t"
 // renormalisation: lanes whose state fell below 2^15 take a word each, in lane order
-#define EP_L8(S, X, AW, BAL, DOFF, CB, E, OFF, BIN, BOUT) "setp.lt.and.u32 p" S ", " X ", 32768, act" S ";\n\t"
-#define EP_L9(S, X, AW, BAL, DOFF, CB, E, OFF, BIN, BOUT) "vote.sync.ballot.b32 " EP_B_##BOUT(S, BAL) ", p" S ", 0xffffffff;\n\t"
-#define EP_L10(S, X, AW, BAL, DOFF, CB, E, OFF, BIN, BOUT) \
-    "lop3.b32 t" S ", " EP_LT ", " EP_B_##BOUT(S, BAL) ", " EP_B_##BIN(S, BAL) ", 0xCA;\n\t"
-#define EP_L11(S, X, AW, BAL, DOFF, CB, E, OFF, BIN, BOUT) "popc.b32 t" S ", t" S ";\n\t"
-#define EP_L12(S, X, AW, BAL, DOFF, CB, E, OFF, BIN, BOUT) "mad.lo.u32 " AW ", t" S ", 2, " AW ";\n\t"
-#define EP_L13(S, X, AW, BAL, DOFF, CB, E, OFF, BIN, BOUT) "ld.shared.u16 w" S ", [" AW "];\n\t"
-#define EP_L14(S, X, AW, BAL, DOFF, CB, E, OFF, BIN, BOUT) "@p" S " mad.lo.u32 " X ", " X ", 65536, w" S ";\n\t"
-#define EP_RENORM_ALL(E, OFF, BIN, BOUT)                                                             \
-    EP_ALL(EP_L8, E, OFF, BIN, BOUT) EP_ALL(EP_L9, E, OFF, BIN, BOUT) EP_ALL(EP_L10, E, OFF, BIN, BOUT)  \
-    EP_ALL(EP_L11, E, OFF, BIN, BOUT) EP_ALL(EP_L12, E, OFF, BIN, BOUT) EP_ALL(EP_L13, E, OFF, BIN, BOUT) \
-    EP_ALL(EP_L14, E, OFF, BIN, BOUT)
-#define EP_STEP_ALL(E, OFF, BIN, BOUT)                                                               \
-    EP_ALL(EP_L1, E, OFF, BIN, BOUT) EP_ALL(EP_L2, E, OFF, BIN, BOUT) EP_ALL(EP_L3, E, OFF, BIN, BOUT)   \
-    EP_ALL(EP_L5, E, OFF, BIN, BOUT) EP_ALL(EP_L6, E, OFF, BIN, BOUT)   \
-    EP_ALL(EP_L7, E, OFF, BIN, BOUT) EP_RENORM_ALL(E, OFF, BIN, BOUT)
+#define EP_L8 "setp.lt.and.u32 pA, %0, 32768, actA;\n\t"
+#define EP_L9(BOUT) "vote.sync.ballot.b32 " BOUT ", pA, 0xffffffff;\n\t"
+#define EP_L10(BIN, BOUT) "lop3.b32 tA, " EP_LT ", " BOUT ", " BIN ", 0xCA;\n\t"
+#define EP_L11 "popc.b32 tA, tA;\n\t"
+#define EP_L12 "mad.lo.u32 %1, tA, 2, %1;\n\t"
+#define EP_L13 "ld.shared.u16 wA, [%1];\n\t"
+#define EP_L14 "@pA mad.lo.u32 %0, %0, 65536, wA;\n\t"
+#define EP_RENORM_ALL(BIN, BOUT) EP_L8 EP_L9(BOUT) EP_L10(BIN, BOUT) EP_L11 EP_L12 EP_L13 EP_L14
+#define EP_STEP_ALL(E, OFF, BIN, BOUT) EP_L1 EP_L2 EP_L3(E, OFF) EP_L5(E) EP_L6(E) EP_L7 EP_RENORM_ALL(BIN, BOUT)
 // the coset: slot below f0 -> coset 0 with frequency f0 (then at least 1), else coset 1 with frequency f1 and offset f0
-#define EP_C1(S, X, AW, BAL, DOFF, CB) "and.b32 u" S ", " X ", 0x7FF;\n\t"
-#define EP_C2(S, X, AW, BAL, DOFF, CB) "shr.u32 q" S ", " X ", 11;\n\t"
-#define EP_C3(S, X, AW, BAL, DOFF, CB) "setp.lt.u32 pc" S ", u" S ", " EP_F0 ";\n\t"
-#define EP_C4(S, X, AW, BAL, DOFF, CB) "selp.b32 f" S ", " EP_F0 ", " EP_F1 ", pc" S ";\n\t"
-#define EP_C5(S, X, AW, BAL, DOFF, CB) "@!pc" S " sub.u32 u" S ", u" S ", " EP_F0 ";\n\t"
-#define EP_C6(S, X, AW, BAL, DOFF, CB) "@act" S " mad.lo.u32 " X ", f" S ", q" S ", u" S ";\n\t"
-#define EP_C7(S, X, AW, BAL, DOFF, CB) "selp.b32 tab" S ", " EP_LUT0 ", " EP_LUT1 ", pc" S ";\n\t"
-#define EP_C8(S, X, AW, BAL, DOFF, CB) "selp.b32 cc" S ", c0r, c1r, pc" S ";\n\t"
+#define EP_C1 "and.b32 uA, %0, 0x7FF;\n\t"
+#define EP_C2 "shr.u32 qA, %0, 11;\n\t"
+#define EP_C3 "setp.lt.u32 pcA, uA, " EP_F0 ";\n\t"
+#define EP_C4 "selp.b32 fA, " EP_F0 ", " EP_F1 ", pcA;\n\t"
+#define EP_C5 "@!pcA sub.u32 uA, uA, " EP_F0 ";\n\t"
+#define EP_C6 "@actA mad.lo.u32 %0, fA, qA, uA;\n\t"
+#define EP_C7 "selp.b32 tabA, " EP_LUT0 ", " EP_LUT1 ", pcA;\n\t"
+#define EP_C8 "selp.b32 ccA, c0r, c1r, pcA;\n\t"
 #define EP_COSET_ALL                                                                                 \
-    EP_ALL(EP_C1) EP_ALL(EP_C2) EP_ALL(EP_C3) EP_ALL(EP_C4) EP_ALL(EP_C5) EP_ALL(EP_C6) EP_ALL(EP_C7) EP_ALL(EP_C8) \
-    EP_RENORM_ALL("", "", BL, NA)
+    EP_C1 EP_C2 EP_C3 EP_C4 EP_C5 EP_C6 EP_C7 EP_C8                                                                   \
+    EP_RENORM_ALL("%2", "naA")
 // Eq. 5 and the product of Eq. 19 for two neighbouring weights: 4096 + code (+ 1/2) as fp32, minus 4096 - zlo, times sigma
-#define EP_XA(S, X, AW, BAL, DOFF, CB, E) "lop3.b32 xa" S ", " E S ", " EP_CM ", cc" S ", 0xEA;\n\t"
-#define EP_XB(S, X, AW, BAL, DOFF, CB, E) "lop3.b32 xb" S ", " E S ", " EP_CM ", cc" S ", 0xEA;\n\t"
-#define EP_P1(S, X, AW, BAL, DOFF, CB) "mov.b64 pr" S ", {xa" S ", xb" S "};\n\t"
-#define EP_P2(S, X, AW, BAL, DOFF, CB) "sub.rn.f32x2 pr" S ", pr" S ", " EP_KK ";\n\t"
-#define EP_P3(S, X, AW, BAL, DOFF, CB) "mul.rn.f32x2 pr" S ", pr" S ", ss" S ";\n\t"
-#define EP_P4(S, X, AW, BAL, DOFF, CB) "mov.b64 {wl" S ", wh" S "}, pr" S ";\n\t"
-#define EP_PAIR_ALL EP_ALL(EP_P1) EP_ALL(EP_P2) EP_ALL(EP_P3) EP_ALL(EP_P4)
+#define EP_XA(E) "lop3.b32 xaA, " E "A, " EP_CM ", ccA, 0xEA;\n\t"
+#define EP_XB(E) "lop3.b32 xbA, " E "A, " EP_CM ", ccA, 0xEA;\n\t"
+#define EP_P1 "mov.b64 prA, {xaA, xbA};\n\t"
+#define EP_P2 "sub.rn.f32x2 prA, prA, " EP_KK ";\n\t"
+#define EP_P3 "mul.rn.f32x2 prA, prA, ssA;\n\t"
+#define EP_P4 "mov.b64 {wlA, whA}, prA;\n\t"
+#define EP_PAIR_ALL EP_P1 EP_P2 EP_P3 EP_P4
 // parity of z1 + ... + z7 = xor of the codes' lowest bits (bit 11 of the entries; zlo is even): the lowest bit of z8
-#define EP_PAR3(S, X, AW, BAL, DOFF, CB, EA, EB, EC) "lop3.b32 par" S ", " EA S ", " EB S ", " EC S ", 0x96;\n\t"
-#define EP_PARX(S, X, AW, BAL, DOFF, CB) "lop3.b32 par" S ", par" S ", 0x800, cc" S ", 0xEA;\n\t"
-#define EP_X8(S, X, AW, BAL, DOFF, CB) "lop3.b32 xb" S ", e8" S ", " EP_CM ", par" S ", 0xEA;\n\t"
-#define EP_ADDR(S, X, AW, BAL, DOFF, CB) "mad.wide.u32 ad" S ", " DOFF ", 1, " EP_OUT ";\n\t"
+#define EP_PAR3(EA, EB, EC) "lop3.b32 parA, " EA "A, " EB "A, " EC "A, 0x96;\n\t"
+#define EP_PARX "lop3.b32 parA, parA, 0x800, ccA, 0xEA;\n\t"
+#define EP_X8 "lop3.b32 xbA, e8A, " EP_CM ", parA, 0xEA;\n\t"
+#define EP_ADDR "mad.wide.u32 adA, %3, 1, " EP_OUT ";\n\t"
 
 // ---- streams with 2^12 slots per table (b = 12: the paper's setting for 8 bpp targets) ------------------------
 // Sixteen tables of 4096 four-byte entries would not fit shared memory, so the lookup has two levels.  Shared memory
@@ -741,65 +661,59 @@ __device__ __forceinline__ void decode_tile_plain(const JobParams &J, uint32_t t
 // mantissa of 2^22 (bit 0 = the coset's half, bit 1 = one) - and it addresses the second level, one word per (table,
 // code): f << 16 | F.  Entries of the kHotSpan codes around zero sit in shared memory, all of them in global memory.
 // HOFF / COFF = byte offset of the field's table in the hot part / in the complete array.
-#define EP_N1(S, X, AW, BAL, DOFF, CB, E, OFF, BIN, BOUT, HOFF, COFF) "and.b32 u" S ", " X ", 0xFFF;\n\t"
-#define EP_N2(S, X, AW, BAL, DOFF, CB, E, OFF, BIN, BOUT, HOFF, COFF) "mad.lo.u32 t" S ", u" S ", 2, tab" S ";\n\t"
-#define EP_N3(S, X, AW, BAL, DOFF, CB, E, OFF, BIN, BOUT, HOFF, COFF) "ld.shared.u16 " E S ", [t" S "+" OFF "];\n\t"
+#define EP_N1 "and.b32 uA, %0, 0xFFF;\n\t"
+#define EP_N2 "mad.lo.u32 tA, uA, 2, tabA;\n\t"
+#define EP_N3(E, OFF) "ld.shared.u16 " E "A, [tA+" OFF "];\n\t"
 /* codes inside the hot window: entry in shared memory; the others: global memory */
-#define EP_N4(S, X, AW, BAL, DOFF, CB, E, OFF, BIN, BOUT, HOFF, COFF) "sub.u32 w" S ", " E S ", " EP_HS2 ";\n\t"
-#define EP_N5(S, X, AW, BAL, DOFF, CB, E, OFF, BIN, BOUT, HOFF, COFF) "setp.lt.u32 pc" S ", w" S ", 1056;\n\t"
-#define EP_N6(S, X, AW, BAL, DOFF, CB, E, OFF, BIN, BOUT, HOFF, COFF) "mad.lo.u32 t" S ", w" S ", 2, hotc" S ";\n\t"
-#define EP_N7(S, X, AW, BAL, DOFF, CB, E, OFF, BIN, BOUT, HOFF, COFF) "mad.wide.u32 ad" S ", " E S ", 2, lc" S ";\n\t"
-#define EP_N8(S, X, AW, BAL, DOFF, CB, E, OFF, BIN, BOUT, HOFF, COFF) \
-    "@pc" S " ld.shared.u32 w" S ", [t" S "+" HOFF "];\n\t" "@!pc" S " ld.global.nc.u32 w" S ", [ad" S "+" COFF "];\n\t"
-#define EP_N9(S, X, AW, BAL, DOFF, CB, E, OFF, BIN, BOUT, HOFF, COFF) "shr.u32 q" S ", " X ", 12;\n\t"
-#define EP_N10(S, X, AW, BAL, DOFF, CB, E, OFF, BIN, BOUT, HOFF, COFF) "shr.u32 f" S ", w" S ", 16;\n\t"
-#define EP_N11(S, X, AW, BAL, DOFF, CB, E, OFF, BIN, BOUT, HOFF, COFF) "and.b32 bi" S ", w" S ", 0xFFFF;\n\t"
-#define EP_N12(S, X, AW, BAL, DOFF, CB, E, OFF, BIN, BOUT, HOFF, COFF) "sub.u32 bi" S ", u" S ", bi" S ";\n\t"
-#define EP_N13(S, X, AW, BAL, DOFF, CB, E, OFF, BIN, BOUT, HOFF, COFF) "@act" S " mad.lo.u32 " X ", f" S ", q" S ", bi" S ";\n\t"
-#define EP_STEP12_ALL(E, OFF, BIN, BOUT, HOFF, COFF)                                                             \
-    EP_ALL(EP_N1, E, OFF, BIN, BOUT, HOFF, COFF) EP_ALL(EP_N2, E, OFF, BIN, BOUT, HOFF, COFF)                    \
-    EP_ALL(EP_N3, E, OFF, BIN, BOUT, HOFF, COFF) EP_ALL(EP_N4, E, OFF, BIN, BOUT, HOFF, COFF)                    \
-    EP_ALL(EP_N5, E, OFF, BIN, BOUT, HOFF, COFF) EP_ALL(EP_N6, E, OFF, BIN, BOUT, HOFF, COFF)                    \
-    EP_ALL(EP_N7, E, OFF, BIN, BOUT, HOFF, COFF) EP_ALL(EP_N8, E, OFF, BIN, BOUT, HOFF, COFF)                    \
-    EP_ALL(EP_N9, E, OFF, BIN, BOUT, HOFF, COFF) EP_ALL(EP_N10, E, OFF, BIN, BOUT, HOFF, COFF)                   \
-    EP_ALL(EP_N11, E, OFF, BIN, BOUT, HOFF, COFF) EP_ALL(EP_N12, E, OFF, BIN, BOUT, HOFF, COFF)                  \
-    EP_ALL(EP_N13, E, OFF, BIN, BOUT, HOFF, COFF) EP_RENORM_ALL(E, OFF, BIN, BOUT)
-#define EP_C1_12(S, X, AW, BAL, DOFF, CB) "and.b32 u" S ", " X ", 0xFFF;\n\t"
-#define EP_C2_12(S, X, AW, BAL, DOFF, CB) "shr.u32 q" S ", " X ", 12;\n\t"
+#define EP_N4(E) "sub.u32 wA, " E "A, " EP_HS2 ";\n\t"
+#define EP_N5 "setp.lt.u32 pcA, wA, 1056;\n\t"
+#define EP_N6 "mad.lo.u32 tA, wA, 2, hotcA;\n\t"
+#define EP_N7(E) "mad.wide.u32 adA, " E "A, 2, lcA;\n\t"
+#define EP_N8(HOFF, COFF)                                                                                             \
+    "@pcA ld.shared.u32 wA, [tA+" HOFF "];\n\t" "@!pcA ld.global.nc.u32 wA, [adA+" COFF "];\n\t"
+#define EP_N9 "shr.u32 qA, %0, 12;\n\t"
+#define EP_N10 "shr.u32 fA, wA, 16;\n\t"
+#define EP_N11 "and.b32 biA, wA, 0xFFFF;\n\t"
+#define EP_N12 "sub.u32 biA, uA, biA;\n\t"
+#define EP_N13 "@actA mad.lo.u32 %0, fA, qA, biA;\n\t"
+#define EP_STEP12_ALL(E, OFF, BIN, BOUT, HOFF, COFF)                                                                  \
+    EP_N1 EP_N2 EP_N3(E, OFF) EP_N4(E) EP_N5 EP_N6 EP_N7(E) EP_N8(HOFF, COFF) EP_N9 EP_N10 EP_N11 EP_N12 EP_N13 EP_RENORM_ALL(BIN, BOUT)
+#define EP_C1_12 "and.b32 uA, %0, 0xFFF;\n\t"
+#define EP_C2_12 "shr.u32 qA, %0, 12;\n\t"
 /* per coset: 2^22 (+ 1/2) as fp32, the hot part and the complete array of its eight tables */
-#define EP_C8_12(S, X, AW, BAL, DOFF, CB) "selp.b32 cc" S ", d0r, d1r, pc" S ";\n\t"
-#define EP_C9_12(S, X, AW, BAL, DOFF, CB) "selp.b32 hotc" S ", hotb, hotb1, pc" S ";\n\t"
-#define EP_C10_12(S, X, AW, BAL, DOFF, CB) "selp.b64 lc" S ", " EP_L2B ", l2b1, pc" S ";\n\t"
+#define EP_C8_12 "selp.b32 ccA, d0r, d1r, pcA;\n\t"
+#define EP_C9_12 "selp.b32 hotcA, hotb, hotb1, pcA;\n\t"
+#define EP_C10_12 "selp.b64 lcA, " EP_L2B ", l2b1, pcA;\n\t"
 #define EP_COSET12_ALL                                                                               \
-    EP_ALL(EP_C1_12) EP_ALL(EP_C2_12) EP_ALL(EP_C3) EP_ALL(EP_C4) EP_ALL(EP_C5) EP_ALL(EP_C6) EP_ALL(EP_C7)  \
-    EP_ALL(EP_C8_12) EP_ALL(EP_C9_12) EP_ALL(EP_C10_12) EP_RENORM_ALL("", "", BL, NA)
+    EP_C1_12 EP_C2_12 EP_C3 EP_C4 EP_C5 EP_C6 EP_C7                                                                   \
+    EP_C8_12 EP_C9_12 EP_C10_12 EP_RENORM_ALL("%2", "naA")
 // Eq. 5: 2^22 + code (+ 1/2) as fp32; z8 = 2m + parity of (z1 + ... + z7), the parity from bit 1 of the xor of the
 // looked-up values (zlo is even)
-#define EP_XA12(S, X, AW, BAL, DOFF, CB, E) "or.b32 xa" S ", " E S ", cc" S ";\n\t"
-#define EP_XB12(S, X, AW, BAL, DOFF, CB, E) "or.b32 xb" S ", " E S ", cc" S ";\n\t"
-#define EP_PARX12(S, X, AW, BAL, DOFF, CB) "lop3.b32 par" S ", par" S ", 0x2, cc" S ", 0xEA;\n\t"
-#define EP_X8_12(S, X, AW, BAL, DOFF, CB) "or.b32 xb" S ", e8" S ", par" S ";\n\t"
+#define EP_XA12(E) "or.b32 xaA, " E "A, ccA;\n\t"
+#define EP_XB12(E) "or.b32 xbA, " E "A, ccA;\n\t"
+#define EP_PARX12 "lop3.b32 parA, parA, 0x2, ccA, 0xEA;\n\t"
+#define EP_X8_12 "or.b32 xbA, e8A, parA;\n\t"
 // the nine steps and the arithmetic of one group, 2^11-slot and 2^12-slot streams
 #define EP_BODY11(CVT)                                                                                                \
         EP_COSET_ALL                                                                                                  \
-        EP_STEP_ALL("e1", "0", NA, NB)     EP_ALL(EP_XA, "e1")                                                        \
-        EP_STEP_ALL("e2", "8192", NB, NA)  EP_ALL(EP_XB, "e2") EP_PAIR_ALL EP_ALL(CVT, "0")                           \
-        EP_STEP_ALL("e3", "16384", NA, NB) EP_ALL(EP_PAR3, "e1", "e2", "e3") EP_ALL(EP_XA, "e3")                      \
-        EP_STEP_ALL("e4", "24576", NB, NA) EP_ALL(EP_XB, "e4") EP_PAIR_ALL EP_ALL(CVT, "1")                           \
-        EP_STEP_ALL("e5", "32768", NA, NB) EP_ALL(EP_PAR3, "par", "e4", "e5") EP_ALL(EP_XA, "e5")                     \
-        EP_STEP_ALL("e6", "40960", NB, NA) EP_ALL(EP_XB, "e6") EP_PAIR_ALL EP_ALL(CVT, "2")                           \
-        EP_STEP_ALL("e7", "49152", NA, NB) EP_ALL(EP_PAR3, "par", "e6", "e7") EP_ALL(EP_XA, "e7")                     \
-        EP_STEP_ALL("e8", "57344", NB, BL) EP_ALL(EP_PARX) EP_ALL(EP_X8) EP_PAIR_ALL EP_ALL(CVT, "3")
+        EP_STEP_ALL("e1", "0", "naA", "nbA")     EP_XA("e1")                                                          \
+        EP_STEP_ALL("e2", "8192", "nbA", "naA")  EP_XB("e2") EP_PAIR_ALL CVT("0")                                     \
+        EP_STEP_ALL("e3", "16384", "naA", "nbA") EP_PAR3("e1", "e2", "e3") EP_XA("e3")                                \
+        EP_STEP_ALL("e4", "24576", "nbA", "naA") EP_XB("e4") EP_PAIR_ALL CVT("1")                                     \
+        EP_STEP_ALL("e5", "32768", "naA", "nbA") EP_PAR3("par", "e4", "e5") EP_XA("e5")                               \
+        EP_STEP_ALL("e6", "40960", "nbA", "naA") EP_XB("e6") EP_PAIR_ALL CVT("2")                                     \
+        EP_STEP_ALL("e7", "49152", "naA", "nbA") EP_PAR3("par", "e6", "e7") EP_XA("e7")                               \
+        EP_STEP_ALL("e8", "57344", "nbA", "%2") EP_PARX EP_X8 EP_PAIR_ALL CVT("3")
 #define EP_BODY12(CVT)                                                                                                \
         EP_COSET12_ALL                                                                                                \
-        EP_STEP12_ALL("e1", "0", NA, NB, "0", "0")             EP_ALL(EP_XA12, "e1")                                  \
-        EP_STEP12_ALL("e2", "8192", NB, NA, "2112", "16384")   EP_ALL(EP_XB12, "e2") EP_PAIR_ALL EP_ALL(CVT, "0")     \
-        EP_STEP12_ALL("e3", "16384", NA, NB, "4224", "32768")  EP_ALL(EP_PAR3, "e1", "e2", "e3") EP_ALL(EP_XA12, "e3") \
-        EP_STEP12_ALL("e4", "24576", NB, NA, "6336", "49152")  EP_ALL(EP_XB12, "e4") EP_PAIR_ALL EP_ALL(CVT, "1")     \
-        EP_STEP12_ALL("e5", "32768", NA, NB, "8448", "65536")  EP_ALL(EP_PAR3, "par", "e4", "e5") EP_ALL(EP_XA12, "e5") \
-        EP_STEP12_ALL("e6", "40960", NB, NA, "10560", "81920") EP_ALL(EP_XB12, "e6") EP_PAIR_ALL EP_ALL(CVT, "2")     \
-        EP_STEP12_ALL("e7", "49152", NA, NB, "12672", "98304") EP_ALL(EP_PAR3, "par", "e6", "e7") EP_ALL(EP_XA12, "e7") \
-        EP_STEP12_ALL("e8", "57344", NB, BL, "14784", "114688") EP_ALL(EP_PARX12) EP_ALL(EP_X8_12) EP_PAIR_ALL EP_ALL(CVT, "3")
+        EP_STEP12_ALL("e1", "0", "naA", "nbA", "0", "0")             EP_XA12("e1")                                    \
+        EP_STEP12_ALL("e2", "8192", "nbA", "naA", "2112", "16384")   EP_XB12("e2") EP_PAIR_ALL CVT("0")               \
+        EP_STEP12_ALL("e3", "16384", "naA", "nbA", "4224", "32768")  EP_PAR3("e1", "e2", "e3") EP_XA12("e3")          \
+        EP_STEP12_ALL("e4", "24576", "nbA", "naA", "6336", "49152")  EP_XB12("e4") EP_PAIR_ALL CVT("1")               \
+        EP_STEP12_ALL("e5", "32768", "naA", "nbA", "8448", "65536")  EP_PAR3("par", "e4", "e5") EP_XA12("e5")         \
+        EP_STEP12_ALL("e6", "40960", "nbA", "naA", "10560", "81920") EP_XB12("e6") EP_PAIR_ALL CVT("2")               \
+        EP_STEP12_ALL("e7", "49152", "naA", "nbA", "12672", "98304") EP_PAR3("par", "e6", "e7") EP_XA12("e7")         \
+        EP_STEP12_ALL("e8", "57344", "nbA", "%2", "14784", "114688") EP_PARX12 EP_X8_12 EP_PAIR_ALL CVT("3")
 
 // ---- the same group with a shorter chain, for few tiles per SM (2^11-slot streams) ---------------------------------
 // With a couple of warps per scheduler the time of a group is the latency of its nine steps, and in EP_BODY11 a step is one
@@ -816,20 +730,20 @@ __device__ __forceinline__ void decode_tile_plain(const JobParams &J, uint32_t t
         "shr.u32 qA, %0, 11;\n\t" "shr.u32 fA, " E "A, 21;\n\t" "and.b32 biA, " E "A, 0x7FF;\n\t"                     \
         "@actA mad.lo.u32 %0, fA, qA, biA;\n\t" EP_T_RENORM(BIN, BOUT) EP_T_TAKE
 #define EP_T_COSET                                                                                                    \
-        EP_ALL(EP_C1) EP_ALL(EP_C2) EP_ALL(EP_C3) EP_ALL(EP_C4) EP_ALL(EP_C5) EP_ALL(EP_C6) EP_ALL(EP_C7) EP_ALL(EP_C8)
+        EP_C1 EP_C2 EP_C3 EP_C4 EP_C5 EP_C6 EP_C7 EP_C8
 #define EP_BODY11_SHORT(CVT)                                                                                          \
         EP_T_COSET EP_T_RENORM("%2", "naA") EP_T_TAKE                                                                 \
-        EP_T_STEP("e1", "0", "naA", "nbA")     EP_ALL(EP_XA, "e1")                                                    \
-        EP_T_STEP("e2", "8192", "nbA", "naA")  EP_ALL(EP_XB, "e2") EP_PAIR_ALL EP_ALL(CVT, "0")                       \
-        EP_T_STEP("e3", "16384", "naA", "nbA") EP_ALL(EP_PAR3, "e1", "e2", "e3") EP_ALL(EP_XA, "e3")                  \
-        EP_T_STEP("e4", "24576", "nbA", "naA") EP_ALL(EP_XB, "e4") EP_PAIR_ALL EP_ALL(CVT, "1")                       \
-        EP_T_STEP("e5", "32768", "naA", "nbA") EP_ALL(EP_PAR3, "par", "e4", "e5") EP_ALL(EP_XA, "e5")                 \
-        EP_T_STEP("e6", "40960", "nbA", "naA") EP_ALL(EP_XB, "e6") EP_PAIR_ALL EP_ALL(CVT, "2")                       \
-        EP_T_STEP("e7", "49152", "naA", "nbA") EP_ALL(EP_PAR3, "par", "e6", "e7") EP_ALL(EP_XA, "e7")                 \
+        EP_T_STEP("e1", "0", "naA", "nbA")     EP_XA("e1")                                                            \
+        EP_T_STEP("e2", "8192", "nbA", "naA")  EP_XB("e2") EP_PAIR_ALL CVT("0")                                       \
+        EP_T_STEP("e3", "16384", "naA", "nbA") EP_PAR3("e1", "e2", "e3") EP_XA("e3")                                  \
+        EP_T_STEP("e4", "24576", "nbA", "naA") EP_XB("e4") EP_PAIR_ALL CVT("1")                                       \
+        EP_T_STEP("e5", "32768", "naA", "nbA") EP_PAR3("par", "e4", "e5") EP_XA("e5")                                 \
+        EP_T_STEP("e6", "40960", "nbA", "naA") EP_XB("e6") EP_PAIR_ALL CVT("2")                                       \
+        EP_T_STEP("e7", "49152", "naA", "nbA") EP_PAR3("par", "e6", "e7") EP_XA("e7")                                 \
         "and.b32 uA, va, 0x7FF;\n\t" "mad.lo.u32 uA, uA, 4, tabA;\n\t" "ld.shared.u32 e8A, [uA+57344];\n\t"           \
         "shr.u32 qA, %0, 11;\n\t" "shr.u32 fA, e8A, 21;\n\t" "and.b32 biA, e8A, 0x7FF;\n\t"                           \
         "@actA mad.lo.u32 %0, fA, qA, biA;\n\t" EP_T_RENORM("nbA", "%2")                                              \
-        EP_ALL(EP_PARX) EP_ALL(EP_X8) EP_PAIR_ALL EP_ALL(CVT, "3")
+        EP_PARX EP_X8 EP_PAIR_ALL CVT("3")
 #define EP_SHORT_FIN EP_T_TAKE      /* the last words go into the states after the loop's test: its vote fills the wait */
 
 // EP_BODY11_GUESS: a lane that takes a word in step k hardly ever takes another in step k + 1 (its state is then at least
@@ -866,135 +780,119 @@ __device__ __forceinline__ void decode_tile_plain(const JobParams &J, uint32_t t
         "setp.lt.and.u32 pA, %0, 32768, actA;\n\t" "vote.sync.ballot.b32 naA, pA, 0xffffffff;\n\t"                    \
         EP_G_STEP("e1", "0", "naA", "%2", "pA", "nbA", "ps", "", "", "")                                              \
         EP_G_STEP("e2", "8192", "nbA", "naA", "ps", "%2", "pA", EP_G_TAIL("e1", "pA"), EP_G_TAIL_REST("e1", "pA"),    \
-                  EP_ALL(EP_XA, "e1"))                                                                                \
+                  EP_XA("e1"))                                                                                        \
         EP_G_STEP("e3", "16384", "%2", "nbA", "pA", "naA", "ps", EP_G_TAIL("e2", "ps"), EP_G_TAIL_REST("e2", "ps"),   \
-                  EP_ALL(EP_XB, "e2") EP_PAIR_ALL EP_ALL(CVT, "0"))                                                   \
+                  EP_XB("e2") EP_PAIR_ALL CVT("0"))                                                                   \
         EP_G_STEP("e4", "24576", "naA", "%2", "ps", "nbA", "pA", EP_G_TAIL("e3", "pA"), EP_G_TAIL_REST("e3", "pA"),   \
-                  EP_ALL(EP_PAR3, "e1", "e2", "e3") EP_ALL(EP_XA, "e3"))                                              \
+                  EP_PAR3("e1", "e2", "e3") EP_XA("e3"))                                                              \
         EP_G_STEP("e5", "32768", "nbA", "naA", "pA", "%2", "ps", EP_G_TAIL("e4", "ps"), EP_G_TAIL_REST("e4", "ps"),   \
-                  EP_ALL(EP_XB, "e4") EP_PAIR_ALL EP_ALL(CVT, "1"))                                                   \
+                  EP_XB("e4") EP_PAIR_ALL CVT("1"))                                                                   \
         EP_G_STEP("e6", "40960", "%2", "nbA", "ps", "naA", "pA", EP_G_TAIL("e5", "pA"), EP_G_TAIL_REST("e5", "pA"),   \
-                  EP_ALL(EP_PAR3, "par", "e4", "e5") EP_ALL(EP_XA, "e5"))                                             \
+                  EP_PAR3("par", "e4", "e5") EP_XA("e5"))                                                             \
         EP_G_STEP("e7", "49152", "naA", "%2", "pA", "nbA", "ps", EP_G_TAIL("e6", "ps"), EP_G_TAIL_REST("e6", "ps"),   \
-                  EP_ALL(EP_XB, "e6") EP_PAIR_ALL EP_ALL(CVT, "2"))                                                   \
+                  EP_XB("e6") EP_PAIR_ALL CVT("2"))                                                                   \
         EP_G_STEP("e8", "57344", "nbA", "naA", "ps", "%2", "pA", EP_G_TAIL("e7", "pA"), EP_G_TAIL_REST("e7", "pA"),   \
-                  EP_ALL(EP_PAR3, "par", "e6", "e7") EP_ALL(EP_XA, "e7"))                                             \
+                  EP_PAR3("par", "e6", "e7") EP_XA("e7"))                                                             \
         EP_G_RANK("%2", "nbA") EP_G_TAIL("e8", "ps")                                                                  \
         "mad.lo.u32 %1, tA, 2, %1;\n\t" "@pA ld.shared.u16 wA, [%1];\n\t" EP_G_TAIL_REST("e8", "ps")                  \
-        EP_ALL(EP_PARX) EP_ALL(EP_X8) EP_PAIR_ALL EP_ALL(CVT, "3")
+        EP_PARX EP_X8 EP_PAIR_ALL CVT("3")
 #define EP_G_REGS ".reg .b32 ke1, ke2, ke3, ke4, ke5, ke6, ke7, ke8, le1, le2, le3, le4, le5, le6, le7, le8;\n\t"
 #define EP_G_KEEP2(A) "st.volatile.shared.u32 [" EP_CTX "+60], k" A ";\n\t" "st.volatile.shared.u32 [" EP_CTX "+60], l" A ";\n\t"
 #define EP_G_KEEP EP_G_KEEP2("e1") EP_G_KEEP2("e2") EP_G_KEEP2("e3") EP_G_KEEP2("e4") EP_G_KEEP2("e5") EP_G_KEEP2("e6") EP_G_KEEP2("e7") EP_G_KEEP2("e8")
 #define EP_GUESS_FIN "@pA mad.lo.u32 %0, %0, 65536, wA;\n\t"
 
-// per output type: CVT(S, j, lo, hi) turns weights 2j, 2j+1 into their stored form, STORE(S) writes the block
-#define EP_CVT_BF16(S, X, AW, BAL, DOFF, CB, J) "cvt.rn.bf16x2.f32 o" J S ", wh" S ", wl" S ";\n\t"
-#define EP_CVT_FP16(S, X, AW, BAL, DOFF, CB, J) "cvt.rn.satfinite.f16x2.f32 o" J S ", wh" S ", wl" S ";\n\t"
-#define EP_ST_16(S, X, AW, BAL, DOFF, CB) "@act" S " st.global.v4.b32 [ad" S "], {o0" S ", o1" S ", o2" S ", o3" S "};\n\t"
-#define EP_CVT_E4M3(S, X, AW, BAL, DOFF, CB, J) "cvt.rn.satfinite.e4m3x2.f32 h" J S ", wh" S ", wl" S ";\n\t"
-#define EP_CVT_E5M2(S, X, AW, BAL, DOFF, CB, J) "cvt.rn.satfinite.e5m2x2.f32 h" J S ", wh" S ", wl" S ";\n\t"
-#define EP_ST_F8(S, X, AW, BAL, DOFF, CB)                                                    \
-    "mov.b32 o0" S ", {h0" S ", h1" S "};\n\t"                           \
-    "mov.b32 o1" S ", {h2" S ", h3" S "};\n\t"                           \
-    "@act" S " st.global.v2.b32 [ad" S "], {o0" S ", o1" S "};\n\t"
-#define EP_CVT_FP32(S, X, AW, BAL, DOFF, CB, J) "mov.b32 ia" J S ", wl" S ";\n\t" "mov.b32 ib" J S ", wh" S ";\n\t"
-#define EP_ST_FP32(S, X, AW, BAL, DOFF, CB)                                                  \
-    "@act" S " st.global.v4.b32 [ad" S "], {ia0" S ", ib0" S ", ia1" S ", ib1" S "};\n\t" \
-    "@act" S " st.global.v4.b32 [ad" S "+16], {ia2" S ", ib2" S ", ia3" S ", ib3" S "};\n\t"
+// per output type: CVT(j) turns weights 2j, 2j+1 into their stored form, STORE writes the block
+#define EP_CVT_BF16(J) "cvt.rn.bf16x2.f32 o" J "A, whA, wlA;\n\t"
+#define EP_CVT_FP16(J) "cvt.rn.satfinite.f16x2.f32 o" J "A, whA, wlA;\n\t"
+#define EP_ST_16 "@actA st.global.v4.b32 [adA], {o0A, o1A, o2A, o3A};\n\t"
+#define EP_CVT_E4M3(J) "cvt.rn.satfinite.e4m3x2.f32 h" J "A, whA, wlA;\n\t"
+#define EP_CVT_E5M2(J) "cvt.rn.satfinite.e5m2x2.f32 h" J "A, whA, wlA;\n\t"
+#define EP_ST_F8                                                                                                      \
+    "mov.b32 o0A, {h0A, h1A};\n\t"                                                                                    \
+    "mov.b32 o1A, {h2A, h3A};\n\t"                                                                                    \
+    "@actA st.global.v2.b32 [adA], {o0A, o1A};\n\t"
+#define EP_CVT_FP32(J) "mov.b32 ia" J "A, wlA;\n\t" "mov.b32 ib" J "A, whA;\n\t"
+#define EP_ST_FP32                                                                                                    \
+    "@actA st.global.v4.b32 [adA], {ia0A, ib0A, ia1A, ib1A};\n\t"                                                     \
+    "@actA st.global.v4.b32 [adA+16], {ia2A, ib2A, ia3A, ib3A};\n\t"
 /* one-byte integers: round to nearest even into s32 (out-of-range values end at INT_MIN / INT_MAX, NaN at 0), then
    saturate and pack four at a time: cvt.pack d, a, b, c gives (c << 16) | sat(a) << 8 | sat(b) */
-#define EP_CVT_I8(S, X, AW, BAL, DOFF, CB, J) "cvt.rni.s32.f32 ia" J S ", wl" S ";\n\t" "cvt.rni.s32.f32 ib" J S ", wh" S ";\n\t"
-#define EP_ST_INT8(S, X, AW, BAL, DOFF, CB)                                                  \
-    "cvt.pack.sat.s8.s32.b32 o2" S ", ib1" S ", ia1" S ", 0;\n\t"        \
-    "cvt.pack.sat.s8.s32.b32 o0" S ", ib0" S ", ia0" S ", o2" S ";\n\t"  \
-    "cvt.pack.sat.s8.s32.b32 o3" S ", ib3" S ", ia3" S ", 0;\n\t"        \
-    "cvt.pack.sat.s8.s32.b32 o1" S ", ib2" S ", ia2" S ", o3" S ";\n\t"  \
-    "@act" S " st.global.v2.b32 [ad" S "], {o0" S ", o1" S "};\n\t"
-#define EP_ST_UINT8(S, X, AW, BAL, DOFF, CB)                                                 \
-    "cvt.pack.sat.u8.s32.b32 o2" S ", ib1" S ", ia1" S ", 0;\n\t"        \
-    "cvt.pack.sat.u8.s32.b32 o0" S ", ib0" S ", ia0" S ", o2" S ";\n\t"  \
-    "cvt.pack.sat.u8.s32.b32 o3" S ", ib3" S ", ia3" S ", 0;\n\t"        \
-    "cvt.pack.sat.u8.s32.b32 o1" S ", ib2" S ", ia2" S ", o3" S ";\n\t"  \
-    "@act" S " st.global.v2.b32 [ad" S "], {o0" S ", o1" S "};\n\t"
+#define EP_CVT_I8(J) "cvt.rni.s32.f32 ia" J "A, wlA;\n\t" "cvt.rni.s32.f32 ib" J "A, whA;\n\t"
+#define EP_ST_INT8                                                                                                    \
+    "cvt.pack.sat.s8.s32.b32 o2A, ib1A, ia1A, 0;\n\t"                                                                 \
+    "cvt.pack.sat.s8.s32.b32 o0A, ib0A, ia0A, o2A;\n\t"                                                               \
+    "cvt.pack.sat.s8.s32.b32 o3A, ib3A, ia3A, 0;\n\t"                                                                 \
+    "cvt.pack.sat.s8.s32.b32 o1A, ib2A, ia2A, o3A;\n\t"                                                               \
+    "@actA st.global.v2.b32 [adA], {o0A, o1A};\n\t"
+#define EP_ST_UINT8                                                                                                   \
+    "cvt.pack.sat.u8.s32.b32 o2A, ib1A, ia1A, 0;\n\t"                                                                 \
+    "cvt.pack.sat.u8.s32.b32 o0A, ib0A, ia0A, o2A;\n\t"                                                               \
+    "cvt.pack.sat.u8.s32.b32 o3A, ib3A, ia3A, 0;\n\t"                                                                 \
+    "cvt.pack.sat.u8.s32.b32 o1A, ib2A, ia2A, o3A;\n\t"                                                               \
+    "@actA st.global.v2.b32 [adA], {o0A, o1A};\n\t"
 
-// registers of one chain
-#define EP_REGS(S, X, AW, BAL, DOFF, CB)                                                                             \
-    ".reg .pred p" S ", pc" S ", act" S ";\n\t"                                                                      \
-    ".reg .b32 u" S ", q" S ", f" S ", bi" S ", t" S ", w" S ", tab" S ", cc" S ", par" S ", na" S ", nb" S ";\n\t"  \
-    ".reg .b32 e1" S ", e2" S ", e3" S ", e4" S ", e5" S ", e6" S ", e7" S ", e8" S ", xa" S ", xb" S ";\n\t"        \
-    ".reg .b32 o0" S ", o1" S ", o2" S ", o3" S ", ia0" S ", ib0" S ", ia1" S ", ib1" S ", ia2" S ", ib2" S ", ia3" S ", ib3" S ";\n\t" \
-    ".reg .b16 h0" S ", h1" S ", h2" S ", h3" S ";\n\t"                                                              \
-    ".reg .f32 wl" S ", wh" S ", sg" S ";\n\t"                                                                       \
-    ".reg .b32 lim" S ", wthr" S ", hotc" S ";\n\t"                                                                  \
-    ".reg .b64 pr" S ", ss" S ", ad" S ", lc" S ";\n\t"
-// before the first pass: the cursor leaves its first chunk at ring + chunk size - 2; lim = 0 sends the chain through EP_ROWS
-#define EP_INIT(S, X, AW, BAL, DOFF, CB)                                 \
-    "ld.shared.u32 r0, [" EP_CTX "+" CB "+16];\n\t"                      \
-    "add.u32 wthr" S ", r0, 510;\n\t"                                    \
-    "mov.u32 lim" S ", 0;\n\t"
+#define EP_REGS                                                                                                       \
+    ".reg .pred pA, pcA, actA;\n\t"                                                                                   \
+    ".reg .b32 uA, qA, fA, biA, tA, wA, tabA, ccA, parA, naA, nbA;\n\t"                                               \
+    ".reg .b32 e1A, e2A, e3A, e4A, e5A, e6A, e7A, e8A, xaA, xbA;\n\t"                                                 \
+    ".reg .b32 o0A, o1A, o2A, o3A, ia0A, ib0A, ia1A, ib1A, ia2A, ib2A, ia3A, ib3A;\n\t"                               \
+    ".reg .b16 h0A, h1A, h2A, h3A;\n\t"                                                                               \
+    ".reg .f32 wlA, whA, sgA;\n\t"                                                                                    \
+    ".reg .b32 limA, wthrA, hotcA;\n\t"                                                                               \
+    ".reg .b64 prA, ssA, adA, lcA;\n\t"
+// before the first pass: the cursor leaves its first chunk at ring + chunk size - 2; lim = 0 sends the tile through EP_ROWS
+#define EP_INIT                                                                                                       \
+    "ld.shared.u32 r0, [" EP_CTX "+32+16];\n\t"                                                                       \
+    "add.u32 wthrA, r0, 510;\n\t"                                                                                     \
+    "mov.u32 limA, 0;\n\t"
 
-#define EP_ADVANCE(S, X, AW, BAL, DOFF, CB, GROUP_BYTES) "add.u32 " DOFF ", " DOFF ", " GROUP_BYTES ";\n\t"
-// go on only if no lane of the chain left its chunk or reached its lim
-#define EP_CALM(S, X, AW, BAL, DOFF, CB)                                 \
-    "setp.lt.and.u32 pq, " AW ", wthr" S ", pq;\n\t"                     \
-    "setp.lt.and.u32 pq, " DOFF ", lim" S ", pq;\n\t"
-#define EP_CALM0(S, X, AW, BAL, DOFF, CB)                                \
-    "setp.lt.u32 pq, " AW ", wthr" S ";\n\t"                             \
-    "setp.lt.and.u32 pq, " DOFF ", lim" S ", pq;\n\t"
-#if EP_CHAINS == 1
-#define EP_CALM_ALL EP_CH_A(EP_CALM0)
-#elif EP_CHAINS == 2
-#define EP_CALM_ALL EP_CH_A(EP_CALM0) EP_CH_B(EP_CALM)
-#elif EP_CHAINS == 3
-#define EP_CALM_ALL EP_CH_A(EP_CALM0) EP_CH_B(EP_CALM) EP_CH_C(EP_CALM)
-#else
-#define EP_CALM_ALL EP_CH_A(EP_CALM0) EP_CH_B(EP_CALM) EP_CH_C(EP_CALM) EP_CH_D(EP_CALM)
-#endif
+#define EP_ADVANCE(GROUP_BYTES) "add.u32 %3, %3, " GROUP_BYTES ";\n\t"
+// go on only if no lane left its chunk or reached its lim
+#define EP_CALM_ALL "setp.lt.u32 pq, %1, wthrA;\n\t" "setp.lt.and.u32 pq, %3, limA, pq;\n\t"
 
-// some lane of the chain reached its lim (also run once on entry): where is each lane now?
-// CB = byte offset of the chain's part of the context block.  row = doff / bytes per row by a multiply-high
-// with ceil(2^32 / bytes per row), which is at most one too large.
-#define EP_ROWS(S, X, AW, BAL, DOFF, CB)                                 \
-    "setp.ge.u32 pr, " DOFF ", lim" S ";\n\t"                                                                  \
+// some lane reached its lim (also run once on entry): where is each lane now?
+// row = doff / bytes per row by a multiply-high with ceil(2^32 / bytes per row), which is at most one too large.
+#define EP_ROWS                                                                                                       \
+    "setp.ge.u32 pr, %3, limA;\n\t"                                                                                   \
     "vote.sync.any.pred pr, pr, 0xffffffff;\n\t"                                                               \
-    "@!pr bra.uni EP_ROWS_END_" S ";\n\t"                                                                      \
+    "@!pr bra.uni EP_ROWS_END_A;\n\t"                                                                                 \
     "ld.shared.v2.u32 {r0, r1}, [" EP_CTX "+8];\n\t"    /* bytes per row, last row */                          \
-    "ld.shared.u32 r2, [" EP_CTX "+" CB "+24];\n\t"     /* offset after the tile's last block */               \
+    "ld.shared.u32 r2, [" EP_CTX "+32+24];\n\t"     /* offset after the tile's last block */                          \
     "ld.shared.u32 r5, [" EP_CTX "+24];\n\t"                                                                   \
-    "mul.hi.u32 r3, " DOFF ", r5;\n\t"                                                                         \
+    "mul.hi.u32 r3, %3, r5;\n\t"                                                                                      \
     "mul.lo.u32 r4, r3, r0;\n\t"                                                                               \
-    "setp.gt.u32 pv, r4, " DOFF ";\n\t"                                                                        \
+    "setp.gt.u32 pv, r4, %3;\n\t"                                                                                     \
     "@pv sub.u32 r3, r3, 1;\n\t"                                                                               \
     "mad.lo.u32 r4, r3, r0, r0;\n\t"                    /* offset at which this lane enters the next row */    \
-    "min.u32 lim" S ", r4, r2;\n\t"                                                                            \
-    "setp.lt.u32 act" S ", " DOFF ", r2;\n\t"                                                                  \
-    "@!act" S " mov.u32 lim" S ", 0xffffffff;\n\t"      /* a lane without a block never asks again */          \
+    "min.u32 limA, r4, r2;\n\t"                                                                                       \
+    "setp.lt.u32 actA, %3, r2;\n\t"                                                                                   \
+    "@!actA mov.u32 limA, 0xffffffff;\n\t"      /* a lane without a block never asks again */                         \
     "min.u32 r3, r3, r1;\n\t"                                                                                  \
     "ld.shared.u64 ra, [" EP_CTX "];\n\t"                                                                      \
     "mul.wide.u32 rb, r3, 4;\n\t"                                                                              \
     "add.s64 ra, ra, rb;\n\t"                                                                                  \
     "ld.global.nc.b32 r4, [ra];\n\t"                                                                           \
-    "mov.b64 ss" S ", {r4, r4};\n\t"                                                                           \
-    "mov.b32 sg" S ", r4;\n\t"                                                                                 \
-    "EP_ROWS_END_" S ":\n\t"
-#define EP_ANY_ACT(S, X, AW, BAL, DOFF, CB) "or.pred pr, pr, act" S ";\n\t"
+    "mov.b64 ssA, {r4, r4};\n\t"                                                                                      \
+    "mov.b32 sgA, r4;\n\t"                                                                                            \
+    "EP_ROWS_END_A:\n\t"
+#define EP_ANY_ACT "or.pred pr, pr, actA;\n\t"
 
-// The chain's cursor left its 512-byte chunk (a group takes at most 448 + 62 bytes, so it is in the next one):
+// The cursor left its 512-byte chunk (a group takes at most 448 + 62 bytes, so it is in the next one):
 // request the chunk two ahead of the cursor's new one into the slot that became free, wait for all requests but
 // this newest one, and move every address back by the ring's length when the cursor's chunk is the one in slot 0
 // again.  The context keeps the request state ready to use: source address, bytes left, destination.
-#define EP_SERVICE(S, X, AW, BAL, DOFF, CB)                              \
-    "setp.ge.u32 pr, " AW ", wthr" S ";\n\t"                                                                   \
+#define EP_SERVICE                                                                                                    \
+    "setp.ge.u32 pr, %1, wthrA;\n\t"                                                                                  \
     "vote.sync.any.pred pr, pr, 0xffffffff;\n\t"                                                               \
-    "@!pr bra.uni EP_SVC_END_" S ";\n\t"                                                                       \
-    "shfl.sync.idx.b32 r6, " AW ", 0, 31, 0xffffffff;\n\t"                                                     \
-    "popc.b32 r0, " BAL ";\n\t"                                                                                \
+    "@!pr bra.uni EP_SVC_END_A;\n\t"                                                                                  \
+    "shfl.sync.idx.b32 r6, %1, 0, 31, 0xffffffff;\n\t"                                                                \
+    "popc.b32 r0, %2;\n\t"                                                                                            \
     "mad.lo.u32 r6, r0, 2, r6;\n\t"                     /* the cursor's address */                             \
-    "add.u32 r0, wthr" S ", 2;\n\t"                     /* end of the chunk it was in */                       \
+    "add.u32 r0, wthrA, 2;\n\t"                     /* end of the chunk it was in */                                  \
     "setp.lt.u32 pq, r6, r0;\n\t"                                                                              \
-    "@pq bra.uni EP_SVC_END_" S ";\n\t"                 /* (a lane address ran ahead of the cursor: not yet) */ \
-    "ld.shared.v4.u32 {r11, r12, r1, r2}, [" EP_CTX "+" CB "];\n\t"  /* source, bytes left, destination */     \
-    "ld.shared.u32 r10, [" EP_CTX "+" CB "+16];\n\t"    /* ring base */                                        \
+    "@pq bra.uni EP_SVC_END_A;\n\t"                 /* (a lane address ran ahead of the cursor: not yet) */           \
+    "ld.shared.v4.u32 {r11, r12, r1, r2}, [" EP_CTX "+32];\n\t"  /* source, bytes left, destination */                \
+    "ld.shared.u32 r10, [" EP_CTX "+32+16];\n\t"    /* ring base */                                                   \
     "mov.b64 ra, {r11, r12};\n\t"                                                                              \
     "sub.s32 r3, r1, " EP_L16 ";\n\t"                                                                          \
     "min.s32 r3, r3, 16;\n\t"                           /* bytes of this lane's 16 inside the payload */       \
@@ -1012,40 +910,24 @@ __device__ __forceinline__ void decode_tile_plain(const JobParams &J, uint32_t t
     "sub.u32 r4, r2, r10;\n\t"                                                                                 \
     "setp.ge.u32 pv, r4, 1536;\n\t"                                                                            \
     "selp.b32 r2, r10, r2, pv;\n\t"                                                                            \
-    "st.shared.v4.u32 [" EP_CTX "+" CB "], {r11, r12, r1, r2};\n\t"                                            \
+    "st.shared.v4.u32 [" EP_CTX "+32], {r11, r12, r1, r2};\n\t"                                                       \
     "cp.async.wait_group 1;\n\t"                                                                               \
     "bar.warp.sync 0xffffffff;\n\t"                                                                            \
-    "add.u32 wthr" S ", wthr" S ", 512;\n\t"            /* the cursor's chunk is the next slot's */            \
-    "sub.u32 r4, wthr" S ", r10;\n\t"                                                                          \
+    "add.u32 wthrA, wthrA, 512;\n\t"            /* the cursor's chunk is the next slot's */                           \
+    "sub.u32 r4, wthrA, r10;\n\t"                                                                                     \
     "setp.lt.u32 pq, r4, 2046;\n\t"                                                                            \
-    "@pq bra.uni EP_SVC_END_" S ";\n\t"                                                                        \
-    "sub.u32 wthr" S ", wthr" S ", 1536;\n\t"           /* past the third slot: everything back by the ring */ \
-    "sub.u32 " AW ", " AW ", 1536;\n\t"                                                                        \
-    "ld.shared.u32 r5, [" EP_CTX "+" CB "+20];\n\t"                                                            \
+    "@pq bra.uni EP_SVC_END_A;\n\t"                                                                                   \
+    "sub.u32 wthrA, wthrA, 1536;\n\t"           /* past the third slot: everything back by the ring */                \
+    "sub.u32 %1, %1, 1536;\n\t"                                                                                       \
+    "ld.shared.u32 r5, [" EP_CTX "+32+20];\n\t"                                                                       \
     "sub.u32 r5, r5, 1536;\n\t"                                                                                \
-    "st.shared.u32 [" EP_CTX "+" CB "+20], r5;\n\t"                                                            \
-    "EP_SVC_END_" S ":\n\t"
-
-#if EP_CHAINS == 1
-#define EP_LOOP_OPERANDS                                                                                              \
-        : "+&r"(x[0]), "+&r"(a[0]), "+&r"(bal[0]), "+&r"(doff[0])
-#elif EP_CHAINS == 2
-#define EP_LOOP_OPERANDS                                                                                              \
-        : "+&r"(x[0]), "+&r"(a[0]), "+&r"(bal[0]), "+&r"(doff[0]), "+&r"(x[1]), "+&r"(a[1]), "+&r"(bal[1]), "+&r"(doff[1])
-#elif EP_CHAINS == 3
-#define EP_LOOP_OPERANDS                                                                                              \
-        : "+&r"(x[0]), "+&r"(a[0]), "+&r"(bal[0]), "+&r"(doff[0]), "+&r"(x[1]), "+&r"(a[1]), "+&r"(bal[1]), "+&r"(doff[1]), \
-          "+&r"(x[2]), "+&r"(a[2]), "+&r"(bal[2]), "+&r"(doff[2])
-#else
-#define EP_LOOP_OPERANDS                                                                                              \
-        : "+&r"(x[0]), "+&r"(a[0]), "+&r"(bal[0]), "+&r"(doff[0]), "+&r"(x[1]), "+&r"(a[1]), "+&r"(bal[1]), "+&r"(doff[1]), \
-          "+&r"(x[2]), "+&r"(a[2]), "+&r"(bal[2]), "+&r"(doff[2]), "+&r"(x[3]), "+&r"(a[3]), "+&r"(bal[3]), "+&r"(doff[3])
-#endif
+    "st.shared.u32 [" EP_CTX "+32+20], r5;\n\t"                                                                       \
+    "EP_SVC_END_A:\n\t"
 
 #define EP_TILES_LOOP_ASM(BODY, CVT, STORE, GROUP_BYTES)                                                                    \
     asm volatile(                                                                                                     \
         "{\n\t"                                                                                                       \
-        EP_ALL(EP_REGS)                                                                                               \
+        EP_REGS                                                                                                       \
         ".reg .pred pq, pv, pr;\n\t"                                                                                  \
         ".reg .b32 r0, r1, r2, r3, r4, r5, r6, r7, r8, r9, r10, r11, r12, c0r, c1r, d0r, d1r, hotb, hotb1;\n\t" \
         ".reg .b64 ra, rb, l2b1;\n\t"                                                                                 \
@@ -1058,28 +940,28 @@ __device__ __forceinline__ void decode_tile_plain(const JobParams &J, uint32_t t
         "add.u32 hotb, " EP_LUT0 ", " EP_HOTOFF ";\n\t"   /* 2^12-slot streams: hot entries of coset 0, */              \
         "add.u32 hotb1, hotb, 16896;\n\t"                 /* of coset 1; complete array of coset 1 */                   \
         "add.s64 l2b1, " EP_L2B ", 131072;\n\t"                                                                       \
-        EP_ALL(EP_INIT)                                                                                               \
+        EP_INIT                                                                                                       \
         "bra.uni EP_RARE;\n\t"                                                                                        \
         "EP_LOOP:\n\t"                                                                                                \
         BODY(CVT)                                                                                                     \
-        EP_ALL(EP_ADDR) EP_ALL(STORE)                                                                                \
-        EP_ALL(EP_ADVANCE, #GROUP_BYTES)                                                                              \
+        EP_ADDR STORE                                                                                                 \
+        EP_ADVANCE(#GROUP_BYTES)                                                                                      \
         /* one vote for everything rare */                                                                            \
         EP_CALM_ALL                                                                                                   \
         "vote.sync.all.pred pq, pq, 0xffffffff;\n\t"                                                                  \
         "@pq bra.uni EP_LOOP;\n\t"                                                                                    \
         "EP_RARE:\n\t"                                                                                                \
-        EP_ALL(EP_ROWS)                                                                                               \
+        EP_ROWS                                                                                                       \
         "setp.lt.u32 pr, " EP_LT ", 0;\n\t"          /* false */                                                                                   \
-        EP_ALL(EP_ANY_ACT)                                                                                            \
+        EP_ANY_ACT                                                                                                    \
         "vote.sync.any.pred pr, pr, 0xffffffff;\n\t"                                                                  \
         "@!pr bra.uni EP_DONE;\n\t"                                                                                   \
-        EP_ALL(EP_SERVICE)                                                                                            \
+        EP_SERVICE                                                                                                    \
         "bra.uni EP_LOOP;\n\t"                                                                                        \
         "EP_DONE:\n\t"                                                                                                \
         "}"                                                                                                           \
         /* every read-write operand is early-clobber: the loop reads the inputs after it has updated them */         \
-        EP_LOOP_OPERANDS                                                                                              \
+        : "+&r"(x), "+&r"(a), "+&r"(bal), "+&r"(doff)                                                                 \
         : "r"(lt), "r"(lut_addr), "r"(lut_addr + kCosetStride), "r"(ctx), "l"(kk), "l"(out_base), "r"(cf.f0),         \
           "r"(cf.f1), "r"(lane16), "l"(l2base), "r"(hs2), "n"(kHotBase)                                             \
         : "memory")
@@ -1094,12 +976,12 @@ __device__ __forceinline__ void decode_tile_plain(const JobParams &J, uint32_t t
         "@!pr bra.uni EP_RARE;\n\t"                                                                                   \
         "mov.b32 %0, sx;\n\t" "mov.b32 %1, sa;\n\t" "mov.b32 %2, sb;\n\t" "sub.u32 %3, %3, " #GROUP_BYTES ";\n\t"     \
         EP_BODY11_SHORT(CVT) EP_SHORT_FIN                                                                             \
-        EP_ALL(EP_ADDR) EP_ALL(STORE) EP_ALL(EP_ADVANCE, #GROUP_BYTES)
+        EP_ADDR STORE EP_ADVANCE(#GROUP_BYTES)
 #define EP_GUESS_NONE(CVT, STORE, GROUP_BYTES)
 #define EP_FEW_LOOP_ASM(BODY, FIN, GUESS, REGS, KEEP, CVT, STORE, GROUP_BYTES)                                        \
     asm volatile(                                                                                                     \
         "{\n\t"                                                                                                       \
-        EP_ALL(EP_REGS) REGS                                                                                          \
+        EP_REGS REGS                                                                                                  \
         ".reg .pred pq, pv, pr, ps, pn;\n\t"                                                                          \
         ".reg .b32 r0, r1, r2, r3, r4, r5, r6, r7, r10, r11, r12, c0r, c1r, lm, sx, sa, sb, ea, va, f2, b2, q2, rp, rowb, endo;\n\t"     \
         ".reg .b64 ra, rb;\n\t"                                                                                       \
@@ -1117,7 +999,7 @@ __device__ __forceinline__ void decode_tile_plain(const JobParams &J, uint32_t t
         "@!pr bra.uni EP_DONE;\n\t"                                                                                   \
         "EP_LOOP:\n\t"                                                                                                \
         BODY(CVT)                                                                                                     \
-        EP_ALL(EP_ADDR) EP_ALL(STORE) EP_ALL(EP_ADVANCE, #GROUP_BYTES)                                                \
+        EP_ADDR STORE EP_ADVANCE(#GROUP_BYTES)                                                                        \
         EP_CALM_ALL                                                                                                   \
         "setp.ge.and.u32 pq, lm, 32768, pq;\n\t"                                                                      \
         "vote.sync.all.pred pq, pq, 0xffffffff;\n\t"                                                                  \
@@ -1175,43 +1057,35 @@ __device__ __forceinline__ void decode_tile_plain(const JobParams &J, uint32_t t
           "r"(rp), "r"(lim), "r"(wthr)                                                                                \
         : "memory")
 
-// kChains tiles of a tensor whose rows hold at least 32 blocks and whose tables have 2^B slots (B = 11: one-level
-// tables; B = 12: two levels, see EP_M1); chain c takes tile
-// `first + c`.  A chain whose slot lies past the job's last tile gets that last tile's record, only so that its
-// addresses stay inside the stream, and no block at all.  The number of groups is data here, not control flow the
-// compiler reasons about: every branch on it is a bra.uni on a warp vote.
+// One tile of a tensor whose rows hold at least 32 blocks and whose tables have 2^B slots (B = 11: one-level tables; B = 12: two
+// levels, see EP_N1).  A warp whose slot lies past the job's last tile gets that last tile's record, only so that its addresses
+// stay inside the stream, and no block at all.  The number of groups is data here, not control flow the compiler
+// reasons about: every branch on it is a bra.uni on a warp vote.
 // `tables`: the job's lookup tables may still be being written (by this CTA's own stores or copies): the
-// tiles' records and first payload chunks are requested first, the CTA barrier comes after.
+// tile's record and first payload chunks are requested first, the wait comes after.
 template <int DT, int B>
-__device__ __forceinline__ void decode_tiles_fast(const JobParams &J, uint32_t first, uint32_t tiles_per_round, uint32_t lut_addr,
+__device__ __forceinline__ void decode_tile_fast(const JobParams &J, uint32_t first, uint32_t tiles_per_round, uint32_t lut_addr,
                                                   CosetFreq cf, uint32_t ring, uint32_t ctx, uint32_t lane, const TablesWait &tables) {
     constexpr uint32_t BB = Out<DT>::kBlockBytes;
     const uint32_t lt = (1u << lane) - 1u, lane16 = 16u * lane;
-    uint32_t x[kChains], a[kChains], bal[kChains], doff[kChains], off[kChains], end[kChains], lead[kChains];
-    bool valid[kChains];
-#pragma unroll
-    for (uint32_t c = 0; c < kChains; ++c) {
-        // (a warp without a tile in this round - the job's last round, or a CTA with more warps than tiles - has no block)
-        valid[c] = first + c < J.tile_cnt && kChains * (threadIdx.x >> 5) + c < tiles_per_round;
-        const uint32_t tile = J.tile0 + min(first + c, J.tile_cnt - 1u);
-        const uint32_t rg = ring + c * kRingStride, cctx = ctx + kCtxChain + c * kCtxChainStride;
-        const TileSetup T = tile_setup(J, tile, valid[c], lane);
-        for (uint32_t k = 0; k < kRingSlots; ++k) ring_issue(rg, T.a0, T.room, k, lane);
-        // the record of the tile this chain takes in the CTA's next round (132 bytes: two lines), into L2
-        if (lane < 2u && tile + tiles_per_round < J.n_tiles) prefetch_l2(J.tile_index + size_t(tile + tiles_per_round) * 33u + 32u * lane);
-        if (lane == 0) {                 // the next request is chunk 3, into slot 0
-            prefetch_l2(J.scales + min(T.v0 / J.per_row, J.row_max));      // the first row scale the loop will ask for
-            sts64(cctx + kCcSrc, T.a0 + kRingBytes);
-            sts32(cctx + kCcRem, T.room - kRingBytes);
-            sts32(cctx + kCcDst, rg);
-            sts32(cctx + kCcRing, rg);
-            sts32(cctx + kCcWbase, rg);
-            sts32(cctx + kCcEndo, (T.v0 + T.nv) * BB);
-        }
-        x[c] = T.x; a[c] = rg + T.lead; bal[c] = 0; doff[c] = (T.v0 + lane) * BB;
-        off[c] = T.off; end[c] = T.end; lead[c] = T.lead;
+    // (a warp without a tile in this round - the job's last round, or a CTA with more warps than tiles - has no block)
+    const bool valid = first < J.tile_cnt && (threadIdx.x >> 5) < tiles_per_round;
+    const uint32_t tile = J.tile0 + min(first, J.tile_cnt - 1u), cctx = ctx + kCtxChain;
+    const TileSetup T = tile_setup(J, tile, valid, lane);
+    for (uint32_t k = 0; k < kRingSlots; ++k) ring_issue(ring, T.a0, T.room, k, lane);
+    // the record of the tile this warp takes in the CTA's next round (132 bytes: two lines), into L2
+    if (lane < 2u && tile + tiles_per_round < J.n_tiles) prefetch_l2(J.tile_index + size_t(tile + tiles_per_round) * 33u + 32u * lane);
+    if (lane == 0) {                 // the next request is chunk 3, into slot 0
+        prefetch_l2(J.scales + min(T.v0 / J.per_row, J.row_max));      // the first row scale the loop will ask for
+        sts64(cctx + kCcSrc, T.a0 + kRingBytes);
+        sts32(cctx + kCcRem, T.room - kRingBytes);
+        sts32(cctx + kCcDst, ring);
+        sts32(cctx + kCcRing, ring);
+        sts32(cctx + kCcWbase, ring);
+        sts32(cctx + kCcEndo, (T.v0 + T.nv) * BB);
     }
-    cp_async_wait<1>();           // all but the last chain's third chunk have landed
+    uint32_t x = T.x, a = ring + T.lead, bal = 0, doff = (T.v0 + lane) * BB;
+    cp_async_wait<1>();           // all but the third chunk have landed
     __syncwarp();
     wait_for_tables(tables);
     const uint32_t k0 = __float_as_uint(float((B == 11 ? 4096 : 4194304) - J.zlo));
@@ -1236,23 +1110,18 @@ __device__ __forceinline__ void decode_tiles_fast(const JobParams &J, uint32_t f
         else if constexpr (DT == EP_UINT8) EP_TILES_LOOP_ASM(EP_BODY12, EP_CVT_I8, EP_ST_UINT8, 256);
         else EP_TILES_LOOP_ASM(EP_BODY12, EP_CVT_I8, EP_ST_INT8, 256);
     }
-    cp_async_wait<0>();           // nothing may still be landing in the rings when the next tiles start
+    cp_async_wait<0>();           // nothing may still be landing in the ring when the next tile starts
     __syncwarp();
     // integrity: the encoder started every state at 2^15 and a tile's words end where the next tile's begin
-    bool bad = false;
-#pragma unroll
-    for (uint32_t c = 0; c < kChains; ++c) {
-        const uint32_t cur = __shfl_sync(0xFFFFFFFFu, a[c], 0) + 2u * __popc(bal[c]) -
-                             lds32(ctx + kCtxChain + c * kCtxChainStride + kCcWbase);
-        bad |= valid[c] && ((x[c] != ep::kStateLow) || (off[c] + ((cur - lead[c]) >> 1) != end[c]));
-    }
+    const uint32_t cur = __shfl_sync(0xFFFFFFFFu, a, 0) + 2u * __popc(bal) - lds32(cctx + kCcWbase);
+    const bool bad = valid && ((x != ep::kStateLow) || (T.off + ((cur - T.lead) >> 1) != T.end));
     if (__any_sync(0xFFFFFFFFu, bad) && lane == 0) atomicOr(&g_ep_status, 1u);
-    __syncwarp();                 // the context block is rewritten by the next tiles
+    __syncwarp();                 // the context block is rewritten by the next tile
 }
 
 // One tile of a CTA that has few of them (2^11-slot streams, rows of 32 blocks or more), decoded by the loop that is short in
 // latency, not in instructions.  The tiles of a round share the space of the 32 rings and of the hot window: 8 KB for each
-// of twelve, which holds a tile's row scales and, usually, all of its payload.  (As in decode_tiles_fast every branch
+// of twelve, which holds a tile's row scales and, usually, all of its payload.  (As in decode_tile_fast every branch
 // depends on parameters or is a bra.uni on a vote: a guard around each vote would cost 25 cycles.)
 template <int DT>
 __device__ __forceinline__ void decode_tile_few(const JobParams &J, uint32_t first, uint32_t tiles_per_round, uint32_t lut_addr,
@@ -1325,7 +1194,7 @@ __device__ __forceinline__ void decode_tile_few(const JobParams &J, uint32_t fir
 // usually inside one job - and sets the lookup tables up again when the stretch crosses into the next job.  Everything
 // that steers this (loop bounds, job changes) depends on blockIdx and kernel parameters only, so the compiler
 // sees warp-uniform control flow and puts no divergence guards around the warp votes of the hot loop; in the last
-// round of a job a chain past the job's last tile goes through the same code with no block to decode.
+// round of a job a warp past the job's last tile goes through the same code with no block to decode.
 // FEW: launches of few tiles per CTA (see decode_tile_few); a kernel of its own because it may use 128 registers where 32 warps
 // leave 64.
 template <int DT, bool FEW>
@@ -1334,7 +1203,7 @@ ep_decode_smem_kernel(const __grid_constant__ BatchParams P) {
     extern __shared__ __align__(16) uint8_t smem[];
     const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
     const uint32_t lut_addr = uint32_t(__cvta_generic_to_shared(smem));
-    const uint32_t ring = lut_addr + kRingBase + warp * (kChains * kRingStride);
+    const uint32_t ring = lut_addr + kRingBase + warp * kRingStride;
     const uint32_t ctx = lut_addr + kCtxBase + warp * kCtxBytes;
     // The hot loop's 64 registers have no room for a phase and a flag kept from job to job, so there every job has an mbarrier of its
     // own (block of seven at 2.5 bpp to FP8 303.5 -> 299.7 us, 8192 x 8192 at 8 bpp 101.1 -> 100.1).  With few tiles per CTA one
@@ -1384,15 +1253,15 @@ ep_decode_smem_kernel(const __grid_constant__ BatchParams P) {
         }
         __syncwarp();
         for (uint32_t r = r0; r < r1; ++r) {
-            const uint32_t base = r * P.tiles_per_round + kChains * warp;
+            const uint32_t base = r * P.tiles_per_round + warp;
             if constexpr (DT != EP_FIELDS_I32) {
                 if (fast) {
-                    if (kTwoLevelInLoop && J.b == 12u) {
-                        if constexpr (kTwoLevelInLoop) decode_tiles_fast<DT, 12>(J, base, P.tiles_per_round, lut_addr, cf, ring, ctx, lane, tables);
+                    if (J.b == 12u) {
+                        decode_tile_fast<DT, 12>(J, base, P.tiles_per_round, lut_addr, cf, ring, ctx, lane, tables);
                     } else if constexpr (FEW) {
                         decode_tile_few<DT>(J, base, P.tiles_per_round, lut_addr, cf, ctx, lane, tables);
                     } else {
-                        decode_tiles_fast<DT, 11>(J, base, P.tiles_per_round, lut_addr, cf, ring, ctx, lane, tables);
+                        decode_tile_fast<DT, 11>(J, base, P.tiles_per_round, lut_addr, cf, ring, ctx, lane, tables);
                     }
                     tables.pending = kTablesThere;
                     continue;
@@ -1400,8 +1269,7 @@ ep_decode_smem_kernel(const __grid_constant__ BatchParams P) {
             }
             wait_for_tables(tables);
             tables.pending = kTablesThere;
-            for (uint32_t c = 0; c < kChains; ++c)
-                if (base + c < J.tile_cnt && kChains * warp + c < P.tiles_per_round) decode_tile_plain<DT>(J, J.tile0 + base + c, lut_addr, cf, ring, lane);
+            if (base < J.tile_cnt && warp < P.tiles_per_round) decode_tile_plain<DT>(J, J.tile0 + base, lut_addr, cf, ring, lane);
         }
     }
 }
@@ -1528,7 +1396,7 @@ __device__ __forceinline__ void umma_commit(uint32_t bar) {
 #define EP_F0 "%9"
 #define EP_F1 "%10"
 #define EP_GEMM_ROW_ASM                                                                                               \
-    asm volatile("{\n\t" EP_ALL(EP_REGS)                                                                              \
+    asm volatile("{\n\t" EP_REGS                                                                                      \
         ".reg .pred pq, pv, pr, pl;\n\t"                                                                              \
         ".reg .b32 r0, r1, r2, r3, r4, r5, r6, r10, r11, r12, c0r, c1r, va, g, bar, par, odd, dst, tries;\n\t"   \
         ".reg .b64 ra, rb, st;\n\t"                                                                                   \
@@ -2220,8 +2088,8 @@ cudaError_t launch_smem_as(const BatchParams &P, uint32_t grid, uint32_t warps, 
 }
 template <int DT>
 cudaError_t launch_smem(const BatchParams &P, uint32_t grid, cudaStream_t st) {
-    const uint32_t warps = (P.tiles_per_round + kChains - 1u) / kChains;
-    bool few = kChains == 1 && warps <= kFewTiles;
+    const uint32_t warps = P.tiles_per_round;
+    bool few = warps <= kFewTiles;
     for (int i = 0; i < P.n_jobs && few; ++i)        // room for a tile's row scales and a window of 4 KB
         few = 4u * (uint64_t(P.job[i].V) / P.job[i].per_row + 3u) + 128u + 4096u <= kStageBytes / warps;
     return few ? launch_smem_as<DT, true>(P, grid, warps, st) : launch_smem_as<DT, false>(P, grid, warps, st);
@@ -2231,7 +2099,7 @@ size_t large_table_bytes(const ep_info &I) { return size_t(EP_NUM_TABLES) * (siz
 
 // 2^12-slot streams whose coordinates span at most kColdCodes values decode from two-level tables in the hot loop
 bool fits_two_level(const ep_info &I) {
-    if (!kTwoLevelInLoop || I.b != 12) return false;
+    if (I.b != 12) return false;
     const Range r = coord_range(I);
     const int64_t zlo = even_base(r);
     return r.any && r.hi - zlo < int64_t(kColdCodes) && zlo >= -(int64_t(1) << 20);   // 2^22 - zlo and 2^22 + code: one exponent
@@ -2585,7 +2453,7 @@ extern "C" int ep_decode_gemm(const ep_info *info, const void *d_stream, const v
     if (reinterpret_cast<uintptr_t>(d_tables) & 255) return EP_ERR_SCRATCH;
     if (I.table_K[0] == 0 || I.table_min[0] < 0 || int64_t(I.table_min[0]) + I.table_K[0] > 2) return EP_ERR_BAD_STREAM;
     // one tile per row, whole groups per row, 32 rows per CTA, tables in shared memory, 32 warps of one tile each
-    if (kChains != 1 || kWarps != 32 || I.b != 11 || !fits_smem_tables(I) || I.V != I.C / 8 || I.C % 256 || T > 32 ||
+    if (I.b != 11 || !fits_smem_tables(I) || I.V != I.C / 8 || I.C % 256 || T > 32 ||
         I.total_words >= (1ull << 30) || uint64_t(I.R) * I.C >= (1ull << 32))
         return EP_ERR_UNSUPPORTED;
     const int sms = num_sms();
