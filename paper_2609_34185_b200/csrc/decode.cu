@@ -719,7 +719,8 @@ __device__ __forceinline__ void decode_tile_plain(const JobParams &J, uint32_t t
 // With a couple of warps per scheduler the time of a group is the latency of its nine steps, and in EP_BODY11 a step is one
 // chain: slot address and lookup (41 cycles), new state (8), ballot (18), rank (20), word (29), back into the state (4).
 // EP_BODY11_SHORT: the next slot is taken from the word itself, not from the state that the word goes into (va = the word
-// where one was taken, else the state: their low eleven bits are the same).  1138 -> 1066 cycles per group.
+// where one was taken, else the state: their low eleven bits are the same).  1362 -> 1276 cycles per group (one tile per SM, 2.5 bpp to
+// BF16, launches of 1792- and 3640-block tiles compared, 1965 MHz).
 #define EP_T_RENORM(BIN, BOUT)                                                                                        \
         "setp.lt.and.u32 pA, %0, 32768, actA;\n\t" "vote.sync.ballot.b32 " BOUT ", pA, 0xffffffff;\n\t"               \
         "mov.b32 va, %0;\n\t" "lop3.b32 tA, " EP_LT ", " BOUT ", " BIN ", 0xCA;\n\t" "popc.b32 tA, tA;\n\t"           \
@@ -751,14 +752,16 @@ __device__ __forceinline__ void decode_tile_plain(const JobParams &J, uint32_t t
 // So the ballot of step k + 1 is taken of the lanes that did not take a word in step k, whose lookup has not waited for
 // step k's words.  The lanes that did follow with a lookup of their own and are back for the lookup of step k + 2.  If one
 // of them falls below 2^15 all the same (`lm`, the smallest such state), the ballots were wrong, and the group is decoded
-// again from its saved start by EP_BODY11_SHORT: no result depends on the guess.  Two steps take 160 cycles this way.
+// again from its saved start by EP_BODY11_SHORT: no result depends on the guess.
 // The order below follows the times at which operands arrive (a warp issues in order): rank of the words, the late lanes'
 // end of the previous step (TAIL, predicate NP from two steps ago), lookup, word, work for the output (FILL), the late
 // lanes' lookup, new state and ballot.
-// The assembler has an order of its own, 11 % slower (it takes the lookup of the late lanes and the work for the output
+// The assembler has an order of its own, 10 % slower (it takes the lookup of the late lanes and the work for the output
 // to where the ballot waits for them), but it moves nothing across a read of the clock: one after each ballot and one
-// after each word's load keep the order: 1070 -> 965 cycles per group.  (Their values have to be used: EP_G_KEEP, once
-// per tile.)
+// after each word's load keep the order: 1215 -> 1101 cycles per group at 2.5 bpp, 1229 -> 1117 at 4.  (Their values have to be
+// used: EP_G_KEEP, once per tile.)  That is a property of this assembler (CUDA 12.9), not of the language; whether
+// another one still keeps to it shows in tiles of 1792 blocks, four per SM at 2.5 bpp to BF16: 32.2 us, 35.6 without the
+// reads, 37.4 with EP_BODY11_SHORT, 39.3 with the ring.
 // PB / PPB: ballots of the previous step and the one before; PP: the lanes that took a word; NB / NP: this step's.
 #define EP_G_TAIL(E, P)                                                                                               \
         "shr.u32 f2, ea, 21;\n\t" "and.b32 b2, ea, 0x7FF;\n\t" "@" P " mad.lo.u32 %0, f2, q2, b2;\n\t"
@@ -1120,8 +1123,8 @@ __device__ __forceinline__ void decode_tile_fast(const JobParams &J, uint32_t fi
 }
 
 // One tile of a CTA that has few of them (2^11-slot streams, rows of 32 blocks or more), decoded by the loop that is short in
-// latency, not in instructions.  The tiles of a round share the space of the 32 rings and of the hot window: 8 KB for each
-// of twelve, which holds a tile's row scales and, usually, all of its payload.  (As in decode_tile_fast every branch
+// latency, not in instructions.  The tiles of a round share the space of the 32 rings and of the hot window: 6 KB for each
+// of sixteen, 12 KB for each of eight, which holds a tile's row scales and, usually, all of its payload.  (As in decode_tile_fast every branch
 // depends on parameters or is a bra.uni on a vote: a guard around each vote would cost 25 cycles.)
 template <int DT>
 __device__ __forceinline__ void decode_tile_few(const JobParams &J, uint32_t first, uint32_t tiles_per_round, uint32_t lut_addr,
@@ -1305,10 +1308,9 @@ ep_decode_smem_kernel(const __grid_constant__ BatchParams P) {
 // end (wrong output, status flag set) instead of hanging.
 struct GemmParams {
     JobParams J;
-    const uint16_t *x;            // [T, C] bf16, row-major
     float *y;                     // [T, R] fp32, row-major
     uint32_t T, Tpad;             // tokens; rows of x that are staged (16 or 32)
-    uint32_t R, C;
+    uint32_t R;
     uint32_t rows_per_cta;        // CTA k takes rows [k, k + 1) * rows_per_cta,
     uint32_t rows_per_step, steps;   // rows_per_step at a time
     uint32_t groups;              // C / 256
@@ -2061,10 +2063,13 @@ uint32_t split_rounds(BatchParams &P, uint32_t sms) {
         // The guess costs ten instructions per step and, at 4 bpp (3.5 bits per symbol), the repetition of one group in 70 (at
         // 5 bpp one in 25, at 6 one in 6).  1792-block tiles, us, with / without: 2.5 bpp 4 tiles 32.7 / 36.8, 8: 37.0 / 38.4,
         // 10: 43.1 / 41.1; 4 bpp 4 tiles 34.4 / 37.1, 8: 38.4 / 38.7; 4.5 bpp 4 tiles 34.9 / 37.1, 8: 39.7 / 38.7.
+        // 3640: 2.5 bpp 4 tiles 64.9 / 74.8, 8: 73.0 / 78.8, 12: 88.0 / 85.9; 4 bpp 4 tiles 67.0 / 75.1, 8: 77.5 / 80.9.  896: 2.5 bpp 8
+        // tiles 20.2 / 21.4; 4 bpp 4 tiles 18.9 / 20.5, 8: 21.5 / 21.4; 5 bpp 4 tiles 20.7 / 20.5.  Tiles of 224 blocks, seven
+        // groups, are over before it pays: 4 bpp 4 tiles 7.7 / 7.7, 8: 8.6 / 8.0.
         J.guess = (lo <= 4u && J.payload_bits <= 4.2f) || (lo <= 8u && J.payload_bits <= 3.6f);
     }
     const uint32_t grid = uint32_t(rounds_total < sms ? rounds_total : sms);
-    // (a tensor has under 2^27 blocks, so sixteen of them cost under 2^26 groups: 32-bit arithmetic in the kernel)
+    // (a tensor has under 2^27 blocks, so sixteen of them cost under 2^28 groups and rounds: 32-bit arithmetic in the kernel)
     if (cost + grid >= (1ull << 31)) return 0;
     P.cost_per_cta = uint32_t((cost + grid - 1u) / grid);
     return grid;
@@ -2452,7 +2457,7 @@ extern "C" int ep_decode_gemm(const ep_info *info, const void *d_stream, const v
         return EP_ERR_BAD_ARG;
     if (reinterpret_cast<uintptr_t>(d_tables) & 255) return EP_ERR_SCRATCH;
     if (I.table_K[0] == 0 || I.table_min[0] < 0 || int64_t(I.table_min[0]) + I.table_K[0] > 2) return EP_ERR_BAD_STREAM;
-    // one tile per row, whole groups per row, 32 rows per CTA, tables in shared memory, 32 warps of one tile each
+    // one tile per row (a warp decodes a row), whole groups per row, tables in shared memory
     if (I.b != 11 || !fits_smem_tables(I) || I.V != I.C / 8 || I.C % 256 || T > 32 ||
         I.total_words >= (1ull << 30) || uint64_t(I.R) * I.C >= (1ull << 32))
         return EP_ERR_UNSUPPORTED;
@@ -2475,14 +2480,13 @@ extern "C" int ep_decode_gemm(const ep_info *info, const void *d_stream, const v
     J.tile_cnt = I.n_tiles;
     J.row_max = I.R - 1u;
     fill_table_params(J, I);
-    P.x = static_cast<const uint16_t *>(d_x);
     P.y = d_y;
     P.T = T;
     P.Tpad = T <= 16 ? 16u : 32u;
     P.R = I.R;
-    P.C = I.C;
-    // rows spread evenly over the SMs, and a CTA's rows over the fewest steps (thirty warps share an SM's issue slots: three
-    // steps of 24 rows take less time than 30 + 30 + 10)
+    // rows spread evenly over the SMs, and a CTA's rows evenly over the fewest steps (a step lasts as long as its warps share an
+    // SM's issue slots; 16 tokens, us, even steps / steps of 30 and a rest: 70 rows per SM of 10240 x 3840 53.5 / 58.4, 31 rows of 2048
+    // columns 19.7 / 24.0, 50 23.0 / 24.5, 62 29.8 / 34.1)
     P.rows_per_cta = (I.R + uint32_t(sms) - 1u) / uint32_t(sms);
     auto steps_of = [&](uint32_t rows) { return (P.rows_per_cta + rows - 1u) / rows; };
     // 17 to 32 tokens: the shape that takes fewer steps, else that with four units of x.  4096 columns at 4 bpp, 32 tokens, us,

@@ -202,7 +202,7 @@ struct EncodeBackend {
     virtual int begin_finish(float s, int b, uint32_t V, const Model &m) = 0;
     virtual int end_finish(float s, int b, uint32_t V, const Model &m, double cce_bits, ep_blob *out) = 0;
     // per-row rate-distortion refinement of the kept quantisation (Sec. 3.5, Alg. 2); on success `m` holds the
-    // counts of the refined fields and finish() uses the refined row scales.  Optional.
+    // counts of the refined fields and end_finish() uses the refined row scales.  Optional.
     virtual int refine(float /*s*/, int /*b*/, uint32_t /*V*/, const ep_encode_opts & /*o*/, Model & /*m*/) { return EP_ERR_UNSUPPORTED; }
 };
 
