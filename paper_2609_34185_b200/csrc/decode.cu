@@ -483,7 +483,7 @@ __device__ __forceinline__ void decode_group_plain(uint32_t &x, uint32_t &wa, ui
 // 16 bytes; it lives in ring slot c mod SLOTS, and a chunk in one of the slots that make up the ring's first 512
 // bytes is written a second time behind the ring's end.  `room` = bytes from a0 to the end of the payload: nothing
 // beyond it is read (cp.async zero-fills the rest).  The decode kernel's rings are 3 x 512 bytes; the kernel that
-// feeds the tensor cores needs the shared memory for its operands and takes 4 x 256.
+// feeds the tensor cores needs the shared memory for its operands and takes 4 x 256 where these leave no more (see GemmShape).
 template <uint32_t CHUNK = kChunk, uint32_t SLOTS = kRingSlots>
 __device__ __forceinline__ void ring_issue(uint32_t ring, uint64_t a0, uint32_t room, uint32_t c, uint32_t lane) {
     if (lane < CHUNK / 16u) {
@@ -1300,7 +1300,7 @@ ep_decode_smem_kernel(const __grid_constant__ BatchParams P) {
 // 10240 x 3840, 16 tokens: steps of 30 + 30 + 10 rows, each ended by a CTA barrier around the read-out, the group in C++:
 // 74.3 us.
 //
-// Shared memory: the lookup tables (128 KB), a payload ring of 4 x 256 + 512 bytes for each decoding warp, then A (units
+// Shared memory: the lookup tables (128 KB), a payload ring of 4 x 256 + 512 or 3 x 512 + 512 bytes for each decoding warp, then A (units
 // of x, refilled by the loading warp as soon as the instructions that read them are done), B (two slabs: the warps decode
 // the next group while the tensor core reads the last one) and the mbarriers; see GemmShape.  What bounds the token count:
 // a group's columns of x must be in flight while the group is decoded (about 1 us), and every CTA re-reads x from L2.
@@ -1316,18 +1316,22 @@ struct GemmParams {
     uint32_t groups;              // C / 256
 };
 
-constexpr uint32_t kGemmChunk = 256, kGemmSlots = 4;     // payload ring of this kernel
-constexpr uint32_t kGemmRingStride = kGemmChunk * kGemmSlots + kRingMirror;   // 1536
-// what depends on the rows per step.  Thirty leave 16 KB for x: two units of a whole group for up to 16 tokens, of half a group
-// for up to 32, and then a unit can be asked for only when the instructions half a group before have read it.  24 make room for
-// 32 KB, four units of half a group each, for up to 32 tokens; where that takes more steps it is the slower one (see the launcher).
-template <uint32_t ROWS>
+// What depends on the rows per step.  Thirty leave 16 KB for x: two units of a whole group for up to 16 tokens, of half a group
+// for up to 32, and then a unit can be asked for only when the instructions half a group before have read it, and payload rings
+// of 4 x 256 bytes.  24 rows make room for 16 KB more: for up to 32 tokens four units of half a group each, for up to 16 (whose
+// two units are enough) rings of 3 x 512 bytes, which are served half as often: 27 of 250 instructions per group were the ring's.
+// 4 bpp, 16 tokens, us, 4 x 256 / 3 x 512: 70 rows per SM of 3840 columns 53.4 / 51.9, 31 of 2048 19.6 / 19.0, 23 at 5 bpp
+// 13.4 / 13.1.  Where 24 rows take more steps than thirty they are the slower ones (see the launcher).
+template <uint32_t TPAD, uint32_t ROWS>
 struct GemmShape {
+    static constexpr bool kWide = TPAD == 16 && ROWS <= 24;
+    static constexpr uint32_t kChunk = kWide ? 512 : 256, kSlots = kWide ? 3 : 4, kRing = kChunk * kSlots;   // payload ring of a decoding warp
+    static constexpr uint32_t kRingStride = kRing + kRingMirror;
     static constexpr uint32_t kRows = ROWS;                              // most rows of W per step: one per decoding warp
     static constexpr uint32_t kN = (ROWS + 7u) & ~7u;                    // rows of the B operand
-    static constexpr uint32_t kUnits = ROWS > 24 ? 2 : 4;                // units of x, 8 KB each
+    static constexpr uint32_t kUnits = TPAD == 16 || ROWS > 24 ? 2 : 4;                // units of x, 8 KB each
     static constexpr uint32_t kBTile = kN * 128, kSlab = 4 * kBTile;     // B: per slab four 64-column tiles of kN rows
-    static constexpr uint32_t kA = (kRingBase + kRows * kGemmRingStride + 1023u) & ~1023u;   // A operand (swizzled tiles start on 1024-byte boundaries)
+    static constexpr uint32_t kA = (kRingBase + kRows * kRingStride + 1023u) & ~1023u;   // A operand (swizzled tiles start on 1024-byte boundaries)
     static constexpr uint32_t kB = kA + kUnits * 8192;
     static constexpr uint32_t kBar = kB + 2 * kSlab;                     // mbarriers, tensor-memory address, abort word
     static constexpr uint32_t kSmem = kBar + 256;
@@ -1377,12 +1381,12 @@ __device__ __forceinline__ void umma_commit(uint32_t bar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
 
-// A row's groups (EP_BODY11_SHORT) with operands of its own: %0 .. %3 = x, a, bal and the group counter q, which goes on from
+// A row's groups (BODY) with operands of its own: %0 .. %3 = x, a, bal and the group counter q, which goes on from
 // row to row.  In C++ around a group's asm this took 324 instructions per group, 80 of them guards around the votes and 40
 // for the ring; thirty warps are bound by just that number.
 // Per group: is the slab free, i.e. is the tensor core done with the group two before (tested ahead of the decode; a fresh
 // barrier passes for parity 1)?  Decode, wait if need be (kSpinLimit tries, or until the abort word is set), store the
-// block, arrive; then the ring (EP_SERVICE's steps for 4 chunks of 256 bytes; a group may leave two of them).
+// block, arrive; then the ring (EP_SERVICE's steps, for either ring; a group may leave two chunks of 256 bytes).
 #undef EP_LT
 #undef EP_LUT0
 #undef EP_LUT1
@@ -1397,7 +1401,7 @@ __device__ __forceinline__ void umma_commit(uint32_t bar) {
 #define EP_KK "%8"
 #define EP_F0 "%9"
 #define EP_F1 "%10"
-#define EP_GEMM_ROW_ASM                                                                                               \
+#define EP_GEMM_ROW_ASM(BODY, FIN)                                                                                            \
     asm volatile("{\n\t" EP_REGS                                                                                      \
         ".reg .pred pq, pv, pr, pl;\n\t"                                                                              \
         ".reg .b32 r0, r1, r2, r3, r4, r5, r6, r10, r11, r12, c0r, c1r, va, g, bar, par, odd, dst, tries;\n\t"   \
@@ -1405,12 +1409,12 @@ __device__ __forceinline__ void umma_commit(uint32_t bar) {
         "mov.b32 c0r, 0x45800000;\n\t" "mov.b32 c1r, 0x45800400;\n\t"                \
         "mov.b64 ssA, {%11, %11};\n\t" "setp.ne.u32 actA, %12, 0;\n\t" "mov.b32 g, %13;\n\t"                          \
         "setp.eq.u32 pl, " EP_LT ", 0;\n\t"                  /* lane 0 */                                             \
-        "ld.shared.u32 r10, [" EP_CTX "+48];\n\t" "add.u32 wthrA, r10, 254;\n\t"                                      \
+        "ld.shared.u32 r10, [" EP_CTX "+48];\n\t" "add.u32 wthrA, r10, %19 - 2;\n\t"                                      \
         "EP_LOOP:\n\t"                                                                                                \
         "and.b32 odd, %3, 1;\n\t" "mad.lo.u32 bar, odd, 8, %15;\n\t" "mad.lo.u32 dst, odd, %17, %14;\n\t"             \
         "shr.u32 par, %3, 1;\n\t" "and.b32 par, par, 1;\n\t" "xor.b32 par, par, 1;\n\t"                               \
         "mbarrier.test_wait.parity.shared::cta.b64 pv, [bar], par;\n\t"                                               \
-        EP_BODY11_SHORT(EP_CVT_BF16)                                                                                  \
+        BODY(EP_CVT_BF16)                                                                                             \
         "vote.sync.all.pred pv, pv, 0xffffffff;\n\t"                                                                  \
         "@pv bra.uni EP_FREE;\n\t"                                                                                    \
         "mov.b32 tries, %18;\n\t"                                                                                     \
@@ -1433,7 +1437,7 @@ __device__ __forceinline__ void umma_commit(uint32_t bar) {
         "add.u32 %3, %3, 1;\n\t" "sub.u32 g, g, 1;\n\t"                                                               \
         "setp.lt.u32 pq, %1, wthrA;\n\t" "setp.ne.and.u32 pq, g, 0, pq;\n\t"                                          \
         "vote.sync.all.pred pq, pq, 0xffffffff;\n\t"                                                                  \
-        EP_SHORT_FIN                                                                                                  \
+        FIN                                                                                                           \
         "@pq bra.uni EP_LOOP;\n\t"                                                                                    \
         "setp.eq.u32 pr, g, 0;\n\t"                                                                                   \
         "vote.sync.any.pred pr, pr, 0xffffffff;\n\t"                                                                  \
@@ -1447,23 +1451,23 @@ __device__ __forceinline__ void umma_commit(uint32_t bar) {
         "mov.b64 ra, {r11, r12};\n\t"                                                                                 \
         "popc.b32 r4, " EP_LT ";\n\t" "shl.b32 r4, r4, 4;\n\t"        /* 16 * lane */                                 \
         "sub.s32 r3, r1, r4;\n\t" "min.s32 r3, r3, 16;\n\t"                                                           \
-        "setp.gt.s32 pv, r3, 0;\n\t" "setp.lt.and.u32 pv, r4, 256, pv;\n\t"                                           \
+        "setp.gt.s32 pv, r3, 0;\n\t" "setp.lt.and.u32 pv, r4, %19, pv;\n\t"                                           \
         "mad.wide.u32 rb, r4, 1, ra;\n\t" "add.u32 r5, r2, r4;\n\t"                                                   \
         "@pv cp.async.cg.shared.global [r5], [rb], 16, r3;\n\t"                                                       \
         "sub.u32 r4, r2, r10;\n\t" "setp.lt.and.u32 pq, r4, 512, pv;\n\t"   /* slots 0 and 1 are written to the mirror as well */ \
-        "@pq cp.async.cg.shared.global [r5+1024], [rb], 16, r3;\n\t"                                                  \
+        "@pq cp.async.cg.shared.global [r5+%20], [rb], 16, r3;\n\t"                                                  \
         "cp.async.commit_group;\n\t"                                                                                  \
-        "add.cc.u32 r11, r11, 256;\n\t" "addc.u32 r12, r12, 0;\n\t" "sub.s32 r1, r1, 256;\n\t"                        \
-        "add.u32 r2, r2, 256;\n\t" "setp.ge.u32 pv, r4, 768;\n\t" "selp.b32 r2, r10, r2, pv;\n\t"                     \
+        "add.cc.u32 r11, r11, %19;\n\t" "addc.u32 r12, r12, 0;\n\t" "sub.s32 r1, r1, %19;\n\t"                        \
+        "add.u32 r2, r2, %19;\n\t" "setp.ge.u32 pv, r4, %20 - %19;\n\t" "selp.b32 r2, r10, r2, pv;\n\t"                     \
         "bar.warp.sync 0xffffffff;\n\t"                                                                               \
         "st.shared.v4.u32 [" EP_CTX "+32], {r11, r12, r1, r2};\n\t"                                                   \
         "cp.async.wait_group 1;\n\t"                                                                                  \
         "bar.warp.sync 0xffffffff;\n\t"                                                                               \
-        "add.u32 wthrA, wthrA, 256;\n\t" "sub.u32 r4, wthrA, r10;\n\t" "setp.lt.u32 pq, r4, 1278;\n\t"                \
+        "add.u32 wthrA, wthrA, %19;\n\t" "sub.u32 r4, wthrA, r10;\n\t" "setp.lt.u32 pq, r4, %20 + %19 - 2;\n\t"                \
         "vote.sync.all.pred pq, pq, 0xffffffff;\n\t"                                                                  \
         "@pq bra.uni EP_RING;\n\t"                                                                                    \
-        "sub.u32 wthrA, wthrA, 1024;\n\t" "sub.u32 %1, %1, 1024;\n\t"   /* past the fourth slot: everything back by the ring */ \
-        "ld.shared.u32 r5, [" EP_CTX "+52];\n\t" "sub.u32 r5, r5, 1024;\n\t"                                          \
+        "sub.u32 wthrA, wthrA, %20;\n\t" "sub.u32 %1, %1, %20;\n\t"   /* past the fourth slot: everything back by the ring */ \
+        "ld.shared.u32 r5, [" EP_CTX "+52];\n\t" "sub.u32 r5, r5, %20;\n\t"                                           \
         "bar.warp.sync 0xffffffff;\n\t"                                                                               \
         "st.shared.u32 [" EP_CTX "+52], r5;\n\t"                                                                      \
         "bra.uni EP_RING;\n\t"                                                                                        \
@@ -1471,7 +1475,7 @@ __device__ __forceinline__ void umma_commit(uint32_t bar) {
         "}"                                                                                                           \
         : "+&r"(x), "+&r"(a), "+&r"(bal), "+&r"(q)                                                                    \
         : "r"(lt), "r"(lut_addr), "r"(lut_addr + kCosetStride), "r"(ctx), "l"(kk), "r"(cf.f0), "r"(cf.f1), "r"(sigma), "r"(act), \
-          "r"(P.groups), "r"(b_dst), "r"(bar_mma), "r"(bar_b), "n"(G::kSlab), "n"(kSpinLimit)                         \
+          "r"(P.groups), "r"(b_dst), "r"(bar_mma), "r"(bar_b), "n"(G::kSlab), "n"(kSpinLimit), "n"(G::kChunk), "n"(G::kRing)                         \
         : "memory")
 
 template <uint32_t TPAD, uint32_t ROWS>
@@ -1483,7 +1487,7 @@ __global__ void __launch_bounds__(kThreads, 1) ep_decode_gemm_kernel(const __gri
     // of the decoding loop, which cost 500 of 1700 cycles per group)
     const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = __shfl_sync(0xFFFFFFFFu, tid >> 5, 0);
     const uint32_t lut_addr = uint32_t(__cvta_generic_to_shared(smem));
-    using G = GemmShape<ROWS>;
+    using G = GemmShape<TPAD, ROWS>;
     const uint32_t a_base = lut_addr + G::kA, b_base = lut_addr + G::kB;
     // A holds two or four units of x: four tiles of 64 columns x 16 rows each (one group's columns), or two tiles x 32 rows
     // (half a group's).  Per unit one mbarrier "landed" and one "read"; per slab of B one "rows stored" and one "read".
@@ -1616,7 +1620,7 @@ __global__ void __launch_bounds__(kThreads, 1) ep_decode_gemm_kernel(const __gri
         }
     } else if (warp < 2u + P.rows_per_step) {
         // ---- the decoding warps: one row of W each, group by group into the slabs of B ----
-        const uint32_t w = warp - 2u, lt = (1u << lane) - 1u, ring = lut_addr + kRingBase + w * kGemmRingStride, ctx = lut_addr + kCtxBase + w * kCtxBytes;
+        const uint32_t w = warp - 2u, lt = (1u << lane) - 1u, ring = lut_addr + kRingBase + w * G::kRingStride, ctx = lut_addr + kCtxBase + w * kCtxBytes;
         const uint32_t k0 = __float_as_uint(float(4096 - J.zlo));
         const uint64_t kk = pack64(k0, k0);
         // where this lane's block of a group goes in a slab: 64-column tile lane / 8, row = w, piece lane % 8 of the row
@@ -1626,7 +1630,7 @@ __global__ void __launch_bounds__(kThreads, 1) ep_decode_gemm_kernel(const __gri
             const uint32_t r = row_begin + s * P.rows_per_step + w, act = r < row_end ? 1u : 0u;   // a CTA's last step may be short
             const uint32_t tile = min(r, P.R - 1u);                     // = the row of W
             const TileSetup Tl = tile_setup(J, tile, true, lane);
-            for (uint32_t c = 0; c < kGemmSlots; ++c) ring_issue<kGemmChunk, kGemmSlots>(ring, Tl.a0, Tl.room, c, lane);
+            for (uint32_t c = 0; c < G::kSlots; ++c) ring_issue<G::kChunk, G::kSlots>(ring, Tl.a0, Tl.room, c, lane);
             const uint32_t sigma = __float_as_uint(__ldg(J.scales + tile));
             // the row this warp takes in the next step: its record is asked for now and, when that is here, the start of
             // its payload is brought into L2, so that the next step does not begin with two reads from DRAM in a row
@@ -1635,8 +1639,8 @@ __global__ void __launch_bounds__(kThreads, 1) ep_decode_gemm_kernel(const __gri
             const uint32_t off_next = __ldg(rec_next + 32);
             if (has_next && lane == 0) prefetch_l2(rec_next);
             if (lane == 0) {                 // the next request is chunk 4, into slot 0
-                sts64(ctx + kCtxChain + kCcSrc, Tl.a0 + kGemmChunk * kGemmSlots);
-                sts32(ctx + kCtxChain + kCcRem, Tl.room - kGemmChunk * kGemmSlots);
+                sts64(ctx + kCtxChain + kCcSrc, Tl.a0 + G::kRing);
+                sts32(ctx + kCtxChain + kCcRem, Tl.room - G::kRing);
                 sts32(ctx + kCtxChain + kCcDst, ring);
                 sts32(ctx + kCtxChain + kCcRing, ring);
                 sts32(ctx + kCtxChain + kCcWbase, ring);
@@ -1649,7 +1653,11 @@ __global__ void __launch_bounds__(kThreads, 1) ep_decode_gemm_kernel(const __gri
             }
             uint32_t x = Tl.x, bal = 0, a = ring + Tl.lead;
             if (s == 0) wait_for_tables(tables);
-            EP_GEMM_ROW_ASM;
+            // The short chain loses to the plain one's smaller number of instructions only where x takes twice the room.  4 bpp, us,
+            // short / plain: 16 tokens 8192 x 8192 79.1 / 80.3, 10240 x 3840 51.9 / 51.5; 32 tokens 4096 x 4096 26.3 / 25.6, 10240 x 3840
+            // 63.2 / 61.1.
+            if constexpr (TPAD == 16u) EP_GEMM_ROW_ASM(EP_BODY11_SHORT, EP_SHORT_FIN);
+            else EP_GEMM_ROW_ASM(EP_BODY11, "");
             cp_async_wait<0>();              // nothing may still be landing in the ring when the next row starts
             __syncwarp();
             const uint32_t pos = __shfl_sync(0xFFFFFFFFu, a, 0) + 2u * __popc(bal) - lds32(ctx + kCtxChain + kCcWbase);
@@ -2489,23 +2497,26 @@ extern "C" int ep_decode_gemm(const ep_info *info, const void *d_stream, const v
     // columns 19.7 / 24.0, 50 23.0 / 24.5, 62 29.8 / 34.1)
     P.rows_per_cta = (I.R + uint32_t(sms) - 1u) / uint32_t(sms);
     auto steps_of = [&](uint32_t rows) { return (P.rows_per_cta + rows - 1u) / rows; };
-    // 17 to 32 tokens: the shape that takes fewer steps, else that with four units of x.  4096 columns at 4 bpp, 32 tokens, us,
+    // The shape that takes fewer steps, else that with the larger rings or four units of x.  4096 columns at 4 bpp, 32 tokens, us,
     // steps of 24 / 30 rows at most: 10 rows per SM 19.9 / 20.3, 23: 23.5 / 24.0, 28: 37.0 / 26.2, 56: 57.5 / 48.5, 70: 65.6 / 63.9,
     // 91: 79.5 / 81.0, 120: 108.2 / 91.9.
-    const uint32_t most = P.Tpad == 16u || steps_of(30u) < steps_of(24u) ? 30u : 24u;
+    const uint32_t most = steps_of(30u) < steps_of(24u) ? 30u : 24u;
     P.steps = steps_of(most);
     P.rows_per_step = (P.rows_per_cta + P.steps - 1u) / P.steps;
     P.groups = I.C / 256u;
     if (I.n_tiles != I.R) return EP_ERR_BAD_ARG;
-    const auto kernel = P.Tpad == 16u ? ep_decode_gemm_kernel<16, 30> : most == 30u ? ep_decode_gemm_kernel<32, 30> : ep_decode_gemm_kernel<32, 24>;
-    const uint32_t smem = most == 30u ? GemmShape<30>::kSmem : GemmShape<24>::kSmem;
+    const auto kernel = P.Tpad == 16u ? (most == 30u ? ep_decode_gemm_kernel<16, 30> : ep_decode_gemm_kernel<16, 24>)
+                                      : (most == 30u ? ep_decode_gemm_kernel<32, 30> : ep_decode_gemm_kernel<32, 24>);
+    const uint32_t smem = P.Tpad == 16u ? (most == 30u ? GemmShape<16, 30>::kSmem : GemmShape<16, 24>::kSmem)
+                                        : (most == 30u ? GemmShape<32, 30>::kSmem : GemmShape<32, 24>::kSmem);
     static bool configured[64] = {};
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return EP_ERR_CUDA;
     if (dev < 0 || dev >= 64 || !configured[dev]) {
-        if (cudaFuncSetAttribute(ep_decode_gemm_kernel<16, 30>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(GemmShape<30>::kSmem)) != cudaSuccess ||
-            cudaFuncSetAttribute(ep_decode_gemm_kernel<32, 30>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(GemmShape<30>::kSmem)) != cudaSuccess ||
-            cudaFuncSetAttribute(ep_decode_gemm_kernel<32, 24>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(GemmShape<24>::kSmem)) != cudaSuccess)
+        if (cudaFuncSetAttribute(ep_decode_gemm_kernel<16, 30>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(GemmShape<16, 30>::kSmem)) != cudaSuccess ||
+            cudaFuncSetAttribute(ep_decode_gemm_kernel<16, 24>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(GemmShape<16, 24>::kSmem)) != cudaSuccess ||
+            cudaFuncSetAttribute(ep_decode_gemm_kernel<32, 30>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(GemmShape<32, 30>::kSmem)) != cudaSuccess ||
+            cudaFuncSetAttribute(ep_decode_gemm_kernel<32, 24>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(GemmShape<32, 24>::kSmem)) != cudaSuccess)
             return EP_ERR_CUDA;
         if (dev >= 0 && dev < 64) configured[dev] = true;
     }

@@ -122,6 +122,24 @@ def test_decode_matmul_of_17_to_32_tokens_in_thirty_rows(R, C, T):
     _check(blob, T, R + C + T)
 
 
+@pytest.mark.parametrize("R,C,T,spread", [
+    (40, 8192, 16, 60),           # a group takes half a chunk of the wide ring: it goes round several times
+    (148 * 24, 1024, 16, 4),      # one full step of 24 rows
+    (148 * 24 + 1, 512, 1, 60),   # two steps, the last CTA with fewer rows
+    (148 * 48 - 5, 256, 9, 1),    # two full steps of one group per row
+    (148 * 70, 768, 13, 20),      # three steps
+])
+def test_decode_matmul_of_up_to_16_tokens_in_24_rows(R, C, T, spread):
+    rng = np.random.default_rng(78)
+    n = R * C // 8
+    fields = np.zeros((n, 9), np.int32)
+    fields[:, 0] = rng.integers(0, 2, n)
+    fields[:, 1:8] = np.rint(rng.standard_normal((n, 7)) * spread).astype(np.int32)
+    fields[:, 8] = np.rint(rng.standard_normal(n) * spread / 2).astype(np.int32)
+    blob = ep.pack_fields(fields, R, C, 11, C // 8, rng.uniform(0.01, 0.05, R).astype(np.float32))
+    _check(blob, T, R + C + T)
+
+
 def test_decode_matmul_more_tokens_than_one_launch_and_repeated_calls():
     W = synth.gaussian_rows(128, 1536, 71)
     blob = ep.encode(W, 4.0, tile_vectors=1536 // 8)
