@@ -37,6 +37,20 @@ __device__ __forceinline__ void chained_start() {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
+// All threads of a CTA: is it the last of `n` CTAs to get here?  What the others did before they got here is there for the last one.
+// One thread's fences next to the atomic order the whole CTA's accesses (a barrier orders them within the CTA, and fences are
+// cumulative).  With a fence in each of 1024 threads the six passes of 512 x 1024 at 4 bpp, first to last, took 98.6 us, 96.4 so.
+__device__ __forceinline__ bool arrive_last(uint32_t *counter, uint32_t n, uint32_t &shared_flag) {
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        shared_flag = atomicAdd(counter, 1u) == n - 1u;
+        __threadfence();
+    }
+    __syncthreads();
+    return shared_flag != 0;
+}
+
 // ---- sums over a row ------------------------------------------------------------------------------------
 // The row RMS (Sec. 3.2) and Eq. 13 are defined by sums in double in index order, a chain of dependent additions per
 // row (14 cycles each: 60 us for 8192 of them, whatever the bandwidth).  Here a CTA sums a row in parallel.
@@ -543,7 +557,6 @@ __device__ __forceinline__ void judge_candidate(const CountParams &P, uint32_t k
     else if (E.too_many) v = kUndecided;
     if (E.worst > (1u << P.rate.b)) v = kAbove;                  // no b-bit table exists for this scale: too fine
     P.state->cand[k].verdict = v;
-    __threadfence();
 }
 
 // all threads of the pass's last CTA: the steps' outcomes in order
@@ -764,19 +777,11 @@ __global__ void __launch_bounds__(kCountThreads, 1) quantise_count_kernel(const 
         atomicMax(&S.from[tid], range_from[tid]);
         atomicMax(&S.to[tid], range_to[tid]);
     }
-    __threadfence();
-    __syncthreads();
-    if (tid == 0) last_cta = atomicAdd(&S.finished, 1u) == P.ctas - 1u;
-    __syncthreads();
-    if (!last_cta) return;
-    __threadfence();
+    if (!arrive_last(&S.finished, P.ctas, last_cta)) return;
     const Evaluation E = gather_counts(P, k, P.mode == kPassSearch ? P.cand_counts + size_t(k) * kEvalSymbols : P.full_counts, sm);
     if (P.mode == kPassSearch) {
         if (tid < 32u) judge_candidate(P, k, E);
-        if (tid == 0) last_cta = atomicAdd(&P.state->closed, 1u) == (1u << P.levels) - 2u;
-        __syncthreads();
-        if (!last_cta) return;
-        __threadfence();
+        if (!arrive_last(&P.state->closed, (1u << P.levels) - 1u, last_cta)) return;
         walk_tree(P);
         return;
     }
@@ -1001,12 +1006,7 @@ __global__ void __launch_bounds__(kTileThreadsMax) tile_encode_kernel(const uint
         if (lane == 0) counts[tile] = cap - end;
     }
     // the last CTA turns the counts into offsets (the tile records' last words and the final one)
-    __threadfence();
-    __syncthreads();
-    if (tid == 0) last_cta = atomicAdd(&state->tiles_done, 1u) == gridDim.x - 1u;
-    __syncthreads();
-    if (!last_cta) return;
-    __threadfence();
+    if (!arrive_last(&state->tiles_done, gridDim.x, last_cta)) return;
     const uint32_t per = (n_tiles + blockDim.x - 1u) / blockDim.x;
     const uint32_t t0 = min(tid * per, n_tiles), t1 = min(t0 + per, n_tiles);
     uint64_t sum = 0;
