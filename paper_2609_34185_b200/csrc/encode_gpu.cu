@@ -469,13 +469,17 @@ __device__ __forceinline__ Evaluation gather_counts(const CountParams &P, uint32
         const uint32_t M = 1u << P.rate.b;
         uint32_t fsum = 0, best = 0;
         auto key = [](uint32_t f, uint32_t j) { return (f << 16) | (0xFFFFu - j); };      // f <= 2^15, j < 2^13: first of the largest
+        // (one division per table instead of one per symbol, and four symbols' chains side by side: the passes of 10240 x 3840
+        // at 4 bpp, first to last, 258.1 -> 254.8 us, of 480 x 7512 at 8 bpp 333.2 -> 327.4)
+        const double per_total = __ddiv_rn(1.0, total);      // (not used for an empty table)
+#pragma unroll 4
         for (uint32_t j = lane; j < K; j += 32) {
             const uint32_t n = f_of[at + j];
             uint32_t f = 0;
             if (n) {
                 const double nM = double(n) * double(M);                                  // below 2^47: exact
-                uint32_t q = uint32_t(nM / total);
-                const double r = __fma_rn(-double(q), total, nM);                         // exact: the quotient is off by one at most
+                uint32_t q = uint32_t(nM * per_total);                                    // off by one at most: 2^15 times 2^-52
+                const double r = __fma_rn(-double(q), total, nM);                         // exact
                 if (r < 0.0) --q; else if (r >= total) ++q;
                 f = max(q, 1u);
             }
