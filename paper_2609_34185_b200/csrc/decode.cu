@@ -38,7 +38,7 @@ constexpr int kWarps = 32;                                   // warps per CTA (o
 constexpr int kThreads = kWarps * 32;
 constexpr uint32_t kTilesPerRound = kWarps;                  // tiles per CTA at a time, at most (see split_rounds)
 // Most tiles per CTA for decode_tile_few: its 512 threads may use 128 registers.  1792-block tiles at 4 bpp to BF16, us, this
-// loop / the ordinary one: 4 tiles 37.1 / 40.0, 8: 38.7 / 41.3, 12: 41.8 / 43.8, 16: 45.4 / 46.6.
+// loop / the ordinary one: 4 tiles 33.3 / 40.0, 8: 36.7 / 41.3, 12: 41.4 / 43.8, 16: 45.2 / 46.6.
 constexpr uint32_t kFewTiles = 16;
 constexpr uint32_t kMinWarps = 8;                            // warps of a CTA, however few tiles it has
 // ... that builds its tables itself: a warp per table (1024 x 1024 at 6 bpp in tiles of 64 blocks, no prepared image, us: 8 warps
@@ -753,56 +753,77 @@ __device__ __forceinline__ void decode_tile_plain(const JobParams &J, uint32_t t
 // step k's words.  The lanes that did follow with a lookup of their own and are back for the lookup of step k + 2.  If one
 // of them falls below 2^15 all the same (`lm`, the smallest such state), the ballots were wrong, and the group is decoded
 // again from its saved start by EP_BODY11_SHORT: no result depends on the guess.
+// The body is for groups in which every lane has a block (a tile's last one, if it is not full, takes EP_BODY11_SHORT): without
+// the lane's flag in every update it has 25 instructions per step instead of 30.
 // The order below follows the times at which operands arrive (a warp issues in order): rank of the words, the late lanes'
-// end of the previous step (TAIL, predicate NP from two steps ago), lookup, word, work for the output (FILL), the late
-// lanes' lookup, new state and ballot.
-// The assembler has an order of its own, 10 % slower (it takes the lookup of the late lanes and the work for the output
-// to where the ballot waits for them), but it moves nothing across a read of the clock: one after each ballot and one
-// after each word's load keep the order: 1215 -> 1101 cycles per group at 2.5 bpp, 1229 -> 1117 at 4.  (Their values have to be
-// used: EP_G_KEEP, once per tile.)  That is a property of this assembler (CUDA 12.9), not of the language; whether
-// another one still keeps to it shows in tiles of 1792 blocks, four per SM at 2.5 bpp to BF16: 32.2 us, 35.6 without the
-// reads, 37.4 with EP_BODY11_SHORT, 39.3 with the ring.
+// end of the previous step (TAIL, predicate NP from two steps ago), lookup, word, work for the output (FILL), new state, the late
+// lanes' lookup, ballot.  Kept, it is 750 cycles per group by the latencies of the instructions (logic and multiply-add 4, population
+// count 17, comparison and ballot 17, shared memory 25).  The assembler has an order of its own, and moves nothing across a
+// signal to dependent launches, which has no effect after the kernel's first one and takes 4 cycles, nor across a read of
+// the clock, which takes 10 (and whose value has to be used: KEEP, once per tile): one after the word's load and one after the
+// ballot or at the step's end keep the order.  (That is a property of this assembler, CUDA 12.9, not of the language.)  Which is best
+// depends on what the output takes.  1792-block tiles at 3.5 bpp, us, three / eight tiles per SM, signals at the end, signals after
+// the ballot, clock reads after the ballot: BF16 32.7 / 36.0, 33.1 / 36.5, 33.2 / 36.7 (without fences, never-taken branches or warp
+// barriers 36 and more); FP32 33.5 / 37.0, 33.0 / 36.8, 33.4 / 37.5; E4M3 33.5 / 36.9, 33.6 / 36.7, 32.8 / 36.0; INT8 33.7 / 37.0,
+// 33.2 / 36.3, 32.9 / 36.6.  With the lane's flag and clock reads they took 33.4 / 37.3 (BF16), 34.3 / 38.5, 33.2 / 37.1, 33.4 / 37.6;
+// EP_BODY11_SHORT takes 37.0 / 38.8.
 // PB / PPB: ballots of the previous step and the one before; PP: the lanes that took a word; NB / NP: this step's.
-#define EP_G_TAIL(E, P)                                                                                               \
-        "shr.u32 f2, ea, 21;\n\t" "and.b32 b2, ea, 0x7FF;\n\t" "@" P " mad.lo.u32 %0, f2, q2, b2;\n\t"
-#define EP_G_TAIL_REST(E, P) "@" P " min.u32 lm, lm, %0;\n\t" "@" P " mov.b32 " E "A, ea;\n\t"
+// K: EP_K16, EP_K32 or EP_K8, by the bits of the output type
+#define EP_G_SIGNAL "griddepcontrol.launch_dependents;\n\t"
+#define EP_K16_WORD(E) EP_G_SIGNAL
+#define EP_K16_BALLOT(E)
+#define EP_K16_END EP_G_SIGNAL
+#define EP_K32_WORD(E) EP_G_SIGNAL
+#define EP_K32_BALLOT(E) EP_G_SIGNAL
+#define EP_K32_END
+#define EP_K8_WORD(E) "mov.u32 k" E ", %%clock;\n\t"
+#define EP_K8_BALLOT(E) "mov.u32 l" E ", %%clock;\n\t"
+#define EP_K8_END
+#define EP_K8_REG(R) ".reg .b32 " R ";\n\t" "mov.b32 " R ", 0;\n\t"
+#define EP_K8_ST(R) "st.volatile.shared.u32 [" EP_CTX "+60], " R ";\n\t"
+#define EP_K8_ALL(DO) DO("ke1") DO("ke2") DO("ke3") DO("ke4") DO("ke5") DO("ke6") DO("ke7") DO("ke8") DO("le1") DO("le2") DO("le3") DO("le4") DO("le5") \
+        DO("le6") DO("le7") DO("le8")
+#define EP_K8_REGS EP_K8_ALL(EP_K8_REG)      /* (without the first values E4M3 takes 33.6 and 36.9 us instead of 32.8 and 36.0) */
+#define EP_K8_KEEP EP_K8_ALL(EP_K8_ST)
+#define EP_G_TAIL(P) "shr.u32 f2, ea, 21;\n\t" "and.b32 b2, ea, 0x7FF;\n\t" "@" P " mad.lo.u32 %0, f2, q2, b2;\n\t"
+#define EP_G_REST(E, P) "@" P " min.u32 lm, lm, %0;\n\t" "@" P " mov.b32 " E "A, ea;\n\t"
 #define EP_G_RANK(PB, PPB) "lop3.b32 tA, " EP_LT ", " PB ", " PPB ", 0xCA;\n\t" "popc.b32 tA, tA;\n\t"
-#define EP_G_STEP(E, OFF, PB, PPB, PP, NB, NP, TAIL, TAILREST, FILL)                                                  \
+#define EP_G_STEP(K, E, OFF, PB, PPB, PP, NB, NP, TAIL, REST, FILL)                                                   \
         EP_G_RANK(PB, PPB) TAIL                                                                                       \
         "and.b32 uA, %0, 0x7FF;\n\t" "mad.lo.u32 uA, uA, 4, tabA;\n\t" "ld.shared.u32 " E "A, [uA+" OFF "];\n\t"      \
-        "mad.lo.u32 %1, tA, 2, %1;\n\t" "@" PP " ld.shared.u16 wA, [%1];\n\t" "mov.u32 k" E ", %%clock;\n\t"          \
-        "shr.u32 qA, %0, 11;\n\t" "not.pred pn, " PP ";\n\t" "and.pred pn, pn, actA;\n\t" TAILREST FILL               \
-        "and.b32 va, wA, 0x7FF;\n\t" "mad.lo.u32 va, va, 4, tabA;\n\t" "@" PP " ld.shared.u32 ea, [va+" OFF "];\n\t"  \
-        "shr.u32 fA, " E "A, 21;\n\t" "and.b32 biA, " E "A, 0x7FF;\n\t" "@pn mad.lo.u32 %0, fA, qA, biA;\n\t"         \
-        "setp.lt.and.u32 " NP ", %0, 32768, pn;\n\t" "vote.sync.ballot.b32 " NB ", " NP ", 0xffffffff;\n\t"           \
-        "mov.u32 l" E ", %%clock;\n\t"                                                                                \
-        "@" PP " mad.lo.u32 %0, %0, 65536, wA;\n\t" "shr.u32 q2, %0, 11;\n\t"
-#define EP_BODY11_GUESS(CVT)                                                                                          \
+        "mad.lo.u32 %1, tA, 2, %1;\n\t" "@" PP " ld.shared.u16 wA, [%1];\n\t" K##_WORD(E)                             \
+        "shr.u32 qA, %0, 11;\n\t" REST FILL                                                                           \
+        "shr.u32 fA, " E "A, 21;\n\t" "and.b32 biA, " E "A, 0x7FF;\n\t" "and.b32 va, wA, 0x7FF;\n\t"                  \
+        "@!" PP " mad.lo.u32 %0, fA, qA, biA;\n\t" "mad.lo.u32 va, va, 4, tabA;\n\t"                                  \
+        "setp.lt.and.u32 " NP ", %0, 32768, !" PP ";\n\t" "@" PP " ld.shared.u32 ea, [va+" OFF "];\n\t"               \
+        "vote.sync.ballot.b32 " NB ", " NP ", 0xffffffff;\n\t" K##_BALLOT(E)                                         \
+        "@" PP " mad.lo.u32 %0, %0, 65536, wA;\n\t" "shr.u32 q2, %0, 11;\n\t" K##_END
+#define EP_BODY11_GUESS(K, CVT)                                                                                       \
         "mov.b32 lm, 0xffffffff;\n\t" "mov.b32 sx, %0;\n\t" "mov.b32 sa, %1;\n\t" "mov.b32 sb, %2;\n\t"               \
-        EP_T_COSET                                                                                                    \
-        "setp.lt.and.u32 pA, %0, 32768, actA;\n\t" "vote.sync.ballot.b32 naA, pA, 0xffffffff;\n\t"                    \
-        EP_G_STEP("e1", "0", "naA", "%2", "pA", "nbA", "ps", "", "", "")                                              \
-        EP_G_STEP("e2", "8192", "nbA", "naA", "ps", "%2", "pA", EP_G_TAIL("e1", "pA"), EP_G_TAIL_REST("e1", "pA"),    \
-                  EP_XA("e1"))                                                                                        \
-        EP_G_STEP("e3", "16384", "%2", "nbA", "pA", "naA", "ps", EP_G_TAIL("e2", "ps"), EP_G_TAIL_REST("e2", "ps"),   \
+        EP_C1 EP_C2 EP_C3 EP_C4 EP_C5 "mad.lo.u32 %0, fA, qA, uA;\n\t" EP_C7 EP_C8                                    \
+        "setp.lt.u32 pA, %0, 32768;\n\t" "vote.sync.ballot.b32 naA, pA, 0xffffffff;\n\t"                              \
+        EP_G_STEP(K, "e1", "0", "naA", "%2", "pA", "nbA", "ps", "", "", "")                                              \
+        EP_G_STEP(K, "e2", "8192", "nbA", "naA", "ps", "%2", "pA", EP_G_TAIL("pA"), EP_G_REST("e1", "pA"), EP_XA("e1"))  \
+        EP_G_STEP(K, "e3", "16384", "%2", "nbA", "pA", "naA", "ps", EP_G_TAIL("ps"), EP_G_REST("e2", "ps"),              \
                   EP_XB("e2") EP_PAIR_ALL CVT("0"))                                                                   \
-        EP_G_STEP("e4", "24576", "naA", "%2", "ps", "nbA", "pA", EP_G_TAIL("e3", "pA"), EP_G_TAIL_REST("e3", "pA"),   \
+        EP_G_STEP(K, "e4", "24576", "naA", "%2", "ps", "nbA", "pA", EP_G_TAIL("pA"), EP_G_REST("e3", "pA"),              \
                   EP_PAR3("e1", "e2", "e3") EP_XA("e3"))                                                              \
-        EP_G_STEP("e5", "32768", "nbA", "naA", "pA", "%2", "ps", EP_G_TAIL("e4", "ps"), EP_G_TAIL_REST("e4", "ps"),   \
+        EP_G_STEP(K, "e5", "32768", "nbA", "naA", "pA", "%2", "ps", EP_G_TAIL("ps"), EP_G_REST("e4", "ps"),              \
                   EP_XB("e4") EP_PAIR_ALL CVT("1"))                                                                   \
-        EP_G_STEP("e6", "40960", "%2", "nbA", "ps", "naA", "pA", EP_G_TAIL("e5", "pA"), EP_G_TAIL_REST("e5", "pA"),   \
+        EP_G_STEP(K, "e6", "40960", "%2", "nbA", "ps", "naA", "pA", EP_G_TAIL("pA"), EP_G_REST("e5", "pA"),              \
                   EP_PAR3("par", "e4", "e5") EP_XA("e5"))                                                             \
-        EP_G_STEP("e7", "49152", "naA", "%2", "pA", "nbA", "ps", EP_G_TAIL("e6", "ps"), EP_G_TAIL_REST("e6", "ps"),   \
+        EP_G_STEP(K, "e7", "49152", "naA", "%2", "pA", "nbA", "ps", EP_G_TAIL("ps"), EP_G_REST("e6", "ps"),              \
                   EP_XB("e6") EP_PAIR_ALL CVT("2"))                                                                   \
-        EP_G_STEP("e8", "57344", "nbA", "naA", "ps", "%2", "pA", EP_G_TAIL("e7", "pA"), EP_G_TAIL_REST("e7", "pA"),   \
+        EP_G_STEP(K, "e8", "57344", "nbA", "naA", "ps", "%2", "pA", EP_G_TAIL("pA"), EP_G_REST("e7", "pA"),              \
                   EP_PAR3("par", "e6", "e7") EP_XA("e7"))                                                             \
-        EP_G_RANK("%2", "nbA") EP_G_TAIL("e8", "ps")                                                                  \
-        "mad.lo.u32 %1, tA, 2, %1;\n\t" "@pA ld.shared.u16 wA, [%1];\n\t" EP_G_TAIL_REST("e8", "ps")                  \
+        EP_G_RANK("%2", "nbA") EP_G_TAIL("ps")                                                                        \
+        "mad.lo.u32 %1, tA, 2, %1;\n\t" "@pA ld.shared.u16 wA, [%1];\n\t" EP_G_REST("e8", "ps")                       \
         EP_PARX EP_X8 EP_PAIR_ALL CVT("3")
-#define EP_G_REGS ".reg .b32 ke1, ke2, ke3, ke4, ke5, ke6, ke7, ke8, le1, le2, le3, le4, le5, le6, le7, le8;\n\t"
-#define EP_G_KEEP2(A) "st.volatile.shared.u32 [" EP_CTX "+60], k" A ";\n\t" "st.volatile.shared.u32 [" EP_CTX "+60], l" A ";\n\t"
-#define EP_G_KEEP EP_G_KEEP2("e1") EP_G_KEEP2("e2") EP_G_KEEP2("e3") EP_G_KEEP2("e4") EP_G_KEEP2("e5") EP_G_KEEP2("e6") EP_G_KEEP2("e7") EP_G_KEEP2("e8")
+#define EP_BODY11_GUESS16(CVT) EP_BODY11_GUESS(EP_K16, CVT)
+#define EP_BODY11_GUESS32(CVT) EP_BODY11_GUESS(EP_K32, CVT)
+#define EP_BODY11_GUESS8(CVT) EP_BODY11_GUESS(EP_K8, CVT)
 #define EP_GUESS_FIN "@pA mad.lo.u32 %0, %0, 65536, wA;\n\t"
+#define EP_GUESS_INIT "mov.b32 wA, 0;\n\t" "mov.b32 ea, 0x200000;\n\t" "mov.b32 q2, 0;\n\t"
 
 // per output type: CVT(j) turns weights 2j, 2j+1 into their stored form, STORE writes the block
 #define EP_CVT_BF16(J) "cvt.rn.bf16x2.f32 o" J "A, whA, wlA;\n\t"
@@ -972,27 +993,32 @@ __device__ __forceinline__ void decode_tile_plain(const JobParams &J, uint32_t t
 // ---- the loop for few tiles per SM: one tile per warp, its whole payload in shared memory ---------------------------
 // Nothing else covers a warp's stalls here, so the rare work is kept short as well: no ring to refill, and the tile's row
 // scales are in shared memory too (a load from global memory at a row's start: 700 cycles every C / 256 groups).
-// GUESS: EP_GUESS_CHECK with EP_BODY11_GUESS - a group whose guess failed is decoded again and stored over -, else empty.
-#define EP_GUESS_CHECK(CVT, STORE, GROUP_BYTES)                                                                       \
+// FULL and REDO are for EP_BODY11_GUESS: a tile's last group, if not every lane has a block in it, and a group whose guess
+// failed (stored over) are decoded by EP_BODY11_SHORT.
+#define EP_GUESS_TEST "setp.ge.and.u32 pq, lm, 32768, pq;\n\t"
+// all lanes have a block, or the other body
+#define EP_GUESS_FULL "vote.sync.all.pred pr, actA, 0xffffffff;\n\t" "@!pr bra.uni EP_OTHER;\n\t"
+#define EP_GUESS_REDO(CVT, STORE, GROUP_BYTES)                                                                        \
         "setp.lt.u32 pr, lm, 32768;\n\t"                                                                              \
         "vote.sync.any.pred pr, pr, 0xffffffff;\n\t"                                                                  \
         "@!pr bra.uni EP_RARE;\n\t"                                                                                   \
         "mov.b32 %0, sx;\n\t" "mov.b32 %1, sa;\n\t" "mov.b32 %2, sb;\n\t" "sub.u32 %3, %3, " #GROUP_BYTES ";\n\t"     \
+        "EP_OTHER:\n\t"                                                                                               \
         EP_BODY11_SHORT(CVT) EP_SHORT_FIN                                                                             \
         EP_ADDR STORE EP_ADVANCE(#GROUP_BYTES)
-#define EP_GUESS_NONE(CVT, STORE, GROUP_BYTES)
-#define EP_FEW_LOOP_ASM(BODY, FIN, GUESS, REGS, KEEP, CVT, STORE, GROUP_BYTES)                                        \
+#define EP_REDO_NONE(CVT, STORE, GROUP_BYTES)
+#define EP_FEW_LOOP_ASM(BODY, FIN, INIT, FULL, TEST, REDO, KEEP, CVT, STORE, GROUP_BYTES)                             \
     asm volatile(                                                                                                     \
         "{\n\t"                                                                                                       \
-        EP_REGS REGS                                                                                                  \
-        ".reg .pred pq, pv, pr, ps, pn;\n\t"                                                                          \
+        EP_REGS                                                                                                       \
+        ".reg .pred pq, pv, pr, ps;\n\t"                                                                              \
         ".reg .b32 r0, r1, r2, r3, r4, r5, r6, r7, r10, r11, r12, c0r, c1r, lm, sx, sa, sb, ea, va, f2, b2, q2, rp, rowb, endo;\n\t"     \
         ".reg .b64 ra, rb;\n\t"                                                                                       \
         ".reg .f32 k0f, k1f;\n\t"                                                                                     \
         "mov.b64 {k0f, k1f}, " EP_KK ";\n\t"                                                                          \
         "mov.b32 c0r, 0x45800000;\n\t"                                                                                \
         "mov.b32 c1r, 0x45800400;\n\t"                                                                                \
-        "mov.b32 wA, 0;\n\t" "mov.b32 ea, 0x200000;\n\t" "mov.b32 q2, 0;\n\t" "mov.b32 lm, 0xffffffff;\n\t"           \
+        INIT                                                                                                          \
         "mov.b32 rp, %12;\n\t" "mov.b32 limA, %13;\n\t" "mov.b32 wthrA, %14;\n\t"                                     \
         "ld.shared.b32 sgA, [rp];\n\t" "mov.b32 r3, sgA;\n\t" "mov.b64 ssA, {r3, r3};\n\t"                            \
         "ld.shared.u32 rowb, [" EP_CTX "+8];\n\t"                                                                     \
@@ -1000,15 +1026,16 @@ __device__ __forceinline__ void decode_tile_plain(const JobParams &J, uint32_t t
         "setp.lt.u32 actA, %3, endo;\n\t" "@!actA mov.u32 limA, 0xffffffff;\n\t"                                      \
         "vote.sync.any.pred pr, actA, 0xffffffff;\n\t"                                                                \
         "@!pr bra.uni EP_DONE;\n\t"                                                                                   \
+        FULL                                                                                                          \
         "EP_LOOP:\n\t"                                                                                                \
         BODY(CVT)                                                                                                     \
         EP_ADDR STORE EP_ADVANCE(#GROUP_BYTES)                                                                        \
         EP_CALM_ALL                                                                                                   \
-        "setp.ge.and.u32 pq, lm, 32768, pq;\n\t"                                                                      \
+        TEST                                                                                                          \
         "vote.sync.all.pred pq, pq, 0xffffffff;\n\t"                                                                  \
         FIN                                                                                                           \
         "@pq bra.uni EP_LOOP;\n\t"                                                                                    \
-        GUESS(CVT, STORE, GROUP_BYTES)                                                                                \
+        REDO(CVT, STORE, GROUP_BYTES)                                                                                 \
         "EP_RARE:\n\t"                                                                                                \
         /* lanes that reached their lim: into the next row (rows hold 32 blocks or more), or past the tile's last block */ \
         "setp.ge.u32 pv, %3, limA;\n\t"                                                                               \
@@ -1023,7 +1050,7 @@ __device__ __forceinline__ void decode_tile_plain(const JobParams &J, uint32_t t
         "EP_ROWS_END:\n\t"                                                                                            \
         "setp.ge.u32 pr, %1, wthrA;\n\t"                                                                              \
         "vote.sync.any.pred pr, pr, 0xffffffff;\n\t"                                                                  \
-        "@!pr bra.uni EP_LOOP;\n\t"                                                                                   \
+        "@!pr bra.uni EP_WINDOW_END;\n\t"                                                                             \
         /* the cursor reached what was still on its way when the loop began */                                        \
         "cp.async.wait_group 0;\n\t"                                                                                  \
         "bar.warp.sync 0xffffffff;\n\t"                                                                               \
@@ -1031,7 +1058,7 @@ __device__ __forceinline__ void decode_tile_plain(const JobParams &J, uint32_t t
         "ld.shared.v2.u32 {r10, r5}, [" EP_CTX "+48];\n\t"            /* window, address of position 0 */             \
         "setp.lt.u32 pq, wthrA, r2;\n\t"                                                                              \
         "mov.b32 wthrA, r2;\n\t"                                                                                      \
-        "@pq bra.uni EP_LOOP;\n\t"                                                                                    \
+        "@pq bra.uni EP_WINDOW_END;\n\t"                                                                              \
         /* or the window's end: the window moves on to the cursor (lane 0's address is the lowest), and all of it is copied */ \
         "shfl.sync.idx.b32 r3, %1, 0, 31, 0xffffffff;\n\t"                                                            \
         "sub.u32 r3, r3, r10;\n\t" "and.b32 r3, r3, 0xfffffff0;\n\t"                                                  \
@@ -1052,6 +1079,8 @@ __device__ __forceinline__ void decode_tile_plain(const JobParams &J, uint32_t t
         "@pv bra.uni EP_FILL;\n\t"                                                                                    \
         "cp.async.wait_all;\n\t"                                                                                      \
         "bar.warp.sync 0xffffffff;\n\t"                                                                               \
+        "EP_WINDOW_END:\n\t"                                                                                          \
+        FULL                                                                                                          \
         "bra.uni EP_LOOP;\n\t"                                                                                        \
         "EP_DONE:\n\t" KEEP                                                                                           \
         "}"                                                                                                           \
@@ -1059,6 +1088,9 @@ __device__ __forceinline__ void decode_tile_plain(const JobParams &J, uint32_t t
         : "r"(lt), "r"(lut_addr), "r"(lut_addr + kCosetStride), "r"(ctx), "l"(kk), "l"(out_base), "r"(cf.f0), "r"(cf.f1), \
           "r"(rp), "r"(lim), "r"(wthr)                                                                                \
         : "memory")
+
+#define EP_FEW_GUESS_ASM(BODY, REGS, KEEP, CVT, STORE, GROUP_BYTES)                                                   \
+    EP_FEW_LOOP_ASM(BODY, EP_GUESS_FIN, REGS EP_GUESS_INIT, EP_GUESS_FULL, EP_GUESS_TEST, EP_GUESS_REDO, KEEP, CVT, STORE, GROUP_BYTES)
 
 // One tile of a tensor whose rows hold at least 32 blocks and whose tables have 2^B slots (B = 11: one-level tables; B = 12: two
 // levels, see EP_N1).  A warp whose slot lies past the job's last tile gets that last tile's record, only so that its addresses
@@ -1168,21 +1200,21 @@ __device__ __forceinline__ void decode_tile_few(const JobParams &J, uint32_t fir
     const uint32_t k0 = __float_as_uint(float(4096 - J.zlo)), lt = (1u << lane) - 1u;
     const uint64_t kk = pack64(k0, k0), out_base = reinterpret_cast<uint64_t>(J.out);
     if (J.guess) {
-        if constexpr (DT == EP_BF16) EP_FEW_LOOP_ASM(EP_BODY11_GUESS, EP_GUESS_FIN, EP_GUESS_CHECK, EP_G_REGS, EP_G_KEEP, EP_CVT_BF16, EP_ST_16, 512);
-        else if constexpr (DT == EP_FP16) EP_FEW_LOOP_ASM(EP_BODY11_GUESS, EP_GUESS_FIN, EP_GUESS_CHECK, EP_G_REGS, EP_G_KEEP, EP_CVT_FP16, EP_ST_16, 512);
-        else if constexpr (DT == EP_FP8_E4M3) EP_FEW_LOOP_ASM(EP_BODY11_GUESS, EP_GUESS_FIN, EP_GUESS_CHECK, EP_G_REGS, EP_G_KEEP, EP_CVT_E4M3, EP_ST_F8, 256);
-        else if constexpr (DT == EP_FP8_E5M2) EP_FEW_LOOP_ASM(EP_BODY11_GUESS, EP_GUESS_FIN, EP_GUESS_CHECK, EP_G_REGS, EP_G_KEEP, EP_CVT_E5M2, EP_ST_F8, 256);
-        else if constexpr (DT == EP_FP32) EP_FEW_LOOP_ASM(EP_BODY11_GUESS, EP_GUESS_FIN, EP_GUESS_CHECK, EP_G_REGS, EP_G_KEEP, EP_CVT_FP32, EP_ST_FP32, 1024);
-        else if constexpr (DT == EP_UINT8) EP_FEW_LOOP_ASM(EP_BODY11_GUESS, EP_GUESS_FIN, EP_GUESS_CHECK, EP_G_REGS, EP_G_KEEP, EP_CVT_I8, EP_ST_UINT8, 256);
-        else EP_FEW_LOOP_ASM(EP_BODY11_GUESS, EP_GUESS_FIN, EP_GUESS_CHECK, EP_G_REGS, EP_G_KEEP, EP_CVT_I8, EP_ST_INT8, 256);
+        if constexpr (DT == EP_BF16) EP_FEW_GUESS_ASM(EP_BODY11_GUESS16, "", "", EP_CVT_BF16, EP_ST_16, 512);
+        else if constexpr (DT == EP_FP16) EP_FEW_GUESS_ASM(EP_BODY11_GUESS16, "", "", EP_CVT_FP16, EP_ST_16, 512);
+        else if constexpr (DT == EP_FP8_E4M3) EP_FEW_GUESS_ASM(EP_BODY11_GUESS8, EP_K8_REGS, EP_K8_KEEP, EP_CVT_E4M3, EP_ST_F8, 256);
+        else if constexpr (DT == EP_FP8_E5M2) EP_FEW_GUESS_ASM(EP_BODY11_GUESS8, EP_K8_REGS, EP_K8_KEEP, EP_CVT_E5M2, EP_ST_F8, 256);
+        else if constexpr (DT == EP_FP32) EP_FEW_GUESS_ASM(EP_BODY11_GUESS32, "", "", EP_CVT_FP32, EP_ST_FP32, 1024);
+        else if constexpr (DT == EP_UINT8) EP_FEW_GUESS_ASM(EP_BODY11_GUESS8, EP_K8_REGS, EP_K8_KEEP, EP_CVT_I8, EP_ST_UINT8, 256);
+        else EP_FEW_GUESS_ASM(EP_BODY11_GUESS8, EP_K8_REGS, EP_K8_KEEP, EP_CVT_I8, EP_ST_INT8, 256);
     } else {
-        if constexpr (DT == EP_BF16) EP_FEW_LOOP_ASM(EP_BODY11_SHORT, EP_SHORT_FIN, EP_GUESS_NONE, "", "", EP_CVT_BF16, EP_ST_16, 512);
-        else if constexpr (DT == EP_FP16) EP_FEW_LOOP_ASM(EP_BODY11_SHORT, EP_SHORT_FIN, EP_GUESS_NONE, "", "", EP_CVT_FP16, EP_ST_16, 512);
-        else if constexpr (DT == EP_FP8_E4M3) EP_FEW_LOOP_ASM(EP_BODY11_SHORT, EP_SHORT_FIN, EP_GUESS_NONE, "", "", EP_CVT_E4M3, EP_ST_F8, 256);
-        else if constexpr (DT == EP_FP8_E5M2) EP_FEW_LOOP_ASM(EP_BODY11_SHORT, EP_SHORT_FIN, EP_GUESS_NONE, "", "", EP_CVT_E5M2, EP_ST_F8, 256);
-        else if constexpr (DT == EP_FP32) EP_FEW_LOOP_ASM(EP_BODY11_SHORT, EP_SHORT_FIN, EP_GUESS_NONE, "", "", EP_CVT_FP32, EP_ST_FP32, 1024);
-        else if constexpr (DT == EP_UINT8) EP_FEW_LOOP_ASM(EP_BODY11_SHORT, EP_SHORT_FIN, EP_GUESS_NONE, "", "", EP_CVT_I8, EP_ST_UINT8, 256);
-        else EP_FEW_LOOP_ASM(EP_BODY11_SHORT, EP_SHORT_FIN, EP_GUESS_NONE, "", "", EP_CVT_I8, EP_ST_INT8, 256);
+        if constexpr (DT == EP_BF16) EP_FEW_LOOP_ASM(EP_BODY11_SHORT, EP_SHORT_FIN, "", "", "", EP_REDO_NONE, "", EP_CVT_BF16, EP_ST_16, 512);
+        else if constexpr (DT == EP_FP16) EP_FEW_LOOP_ASM(EP_BODY11_SHORT, EP_SHORT_FIN, "", "", "", EP_REDO_NONE, "", EP_CVT_FP16, EP_ST_16, 512);
+        else if constexpr (DT == EP_FP8_E4M3) EP_FEW_LOOP_ASM(EP_BODY11_SHORT, EP_SHORT_FIN, "", "", "", EP_REDO_NONE, "", EP_CVT_E4M3, EP_ST_F8, 256);
+        else if constexpr (DT == EP_FP8_E5M2) EP_FEW_LOOP_ASM(EP_BODY11_SHORT, EP_SHORT_FIN, "", "", "", EP_REDO_NONE, "", EP_CVT_E5M2, EP_ST_F8, 256);
+        else if constexpr (DT == EP_FP32) EP_FEW_LOOP_ASM(EP_BODY11_SHORT, EP_SHORT_FIN, "", "", "", EP_REDO_NONE, "", EP_CVT_FP32, EP_ST_FP32, 1024);
+        else if constexpr (DT == EP_UINT8) EP_FEW_LOOP_ASM(EP_BODY11_SHORT, EP_SHORT_FIN, "", "", "", EP_REDO_NONE, "", EP_CVT_I8, EP_ST_UINT8, 256);
+        else EP_FEW_LOOP_ASM(EP_BODY11_SHORT, EP_SHORT_FIN, "", "", "", EP_REDO_NONE, "", EP_CVT_I8, EP_ST_INT8, 256);
     }
     cp_async_wait<0>();           // nothing may still be landing in the stage when the next tile starts
     __syncwarp();
@@ -2068,13 +2100,14 @@ uint32_t split_rounds(BatchParams &P, uint32_t sms) {
         J.round_cost = rounds_total <= sms ? 1u : (J.V + 31u) / 32u;
         J.cost_begin = uint32_t(cost);
         cost += uint64_t(J.rounds) * J.round_cost;
-        // The guess costs ten instructions per step and, at 4 bpp (3.5 bits per symbol), the repetition of one group in 70 (at
-        // 5 bpp one in 25, at 6 one in 6).  1792-block tiles, us, with / without: 2.5 bpp 4 tiles 32.7 / 36.8, 8: 37.0 / 38.4,
-        // 10: 43.1 / 41.1; 4 bpp 4 tiles 34.4 / 37.1, 8: 38.4 / 38.7; 4.5 bpp 4 tiles 34.9 / 37.1, 8: 39.7 / 38.7.
-        // 3640: 2.5 bpp 4 tiles 64.9 / 74.8, 8: 73.0 / 78.8, 12: 88.0 / 85.9; 4 bpp 4 tiles 67.0 / 75.1, 8: 77.5 / 80.9.  896: 2.5 bpp 8
-        // tiles 20.2 / 21.4; 4 bpp 4 tiles 18.9 / 20.5, 8: 21.5 / 21.4; 5 bpp 4 tiles 20.7 / 20.5.  Tiles of 224 blocks, seven
+        // The guess costs nine instructions per step and, at 4 bpp (3.5 bits per symbol), the repetition of one group in 70 (at
+        // 5 bpp one in 25, at 6 one in 6).  1792-block tiles, us, with / without: 2.5 bpp 4 tiles 31.9 / 37.1, 8: 35.3 / 38.5,
+        // 10: 40.4 / 40.6, 12: 41.0 / 40.9; 4 bpp 4 tiles 33.3 / 37.1, 8: 36.7 / 38.9, 10: 41.6 / 41.0; 4.5 bpp 4 tiles 34.3 / 37.1, 8:
+        // 37.8 / 39.0; 5 bpp 4 tiles 36.3 / 37.2, 8: 40.0 / 39.1; 5.5 bpp 4 tiles 41.5 / 37.2.
+        // 3640: 2.5 bpp 4 tiles 63.5 / 74.4, 8: 70.7 / 78.3, 12: 83.5 / 86.0; 4 bpp 4 tiles 66.0 / 74.9, 8: 75.4 / 80.1.  896: 2.5 bpp 8
+        // tiles 19.8 / 21.0; 4 bpp 4 tiles 18.8 / 20.3, 8: 21.1 / 21.3; 5 bpp 4 tiles 20.6 / 20.4.  Tiles of 224 blocks, seven
         // groups, are over before it pays: 4 bpp 4 tiles 7.7 / 7.7, 8: 8.6 / 8.0.
-        J.guess = (lo <= 4u && J.payload_bits <= 4.2f) || (lo <= 8u && J.payload_bits <= 3.6f);
+        J.guess = (lo <= 4u && J.payload_bits <= (J.V > 1024u ? 4.5f : 4.2f)) || (lo <= 8u && J.V >= 512u && J.payload_bits <= 4.1f);
     }
     const uint32_t grid = uint32_t(rounds_total < sms ? rounds_total : sms);
     // (a tensor has under 2^27 blocks, so sixteen of them cost under 2^28 groups and rounds: 32-bit arithmetic in the kernel)

@@ -622,6 +622,26 @@ def test_few_tiles_per_sm(R, C, V, spread):
     _check(blob, (ep.BF16, ep.INT8, ep.FP32))
 
 
+@pytest.mark.parametrize("R,C,V", [
+    (40, 256, 31),        # no full group at all
+    (40, 256, 32),        # one full group
+    (60, 320, 33),        # a full group and a group of one lane; rows of 40 blocks: most groups cross a row
+    (70, 1024, 63),
+    (64, 256, 2047),      # a tile whose last group misses one lane, and a tile of one block
+    (300, 264, 130),      # rows of 33 blocks; the last tile ends inside a group
+])
+def test_few_tiles_whose_last_group_is_not_full(R, C, V):
+    rng = np.random.default_rng(9300 + R + V)
+    n = R * C // 8
+    fields = np.zeros((n, 9), np.int32)
+    fields[:, 0] = rng.integers(0, 2, n)
+    fields[:, 1:8] = np.rint(rng.standard_normal((n, 7)) * 1.2).astype(np.int32)
+    fields[:, 8] = np.rint(rng.standard_normal(n) * 0.8).astype(np.int32)
+    blob = ep.pack_fields(fields, R, C, 11, V, rng.uniform(0.01, 0.05, R).astype(np.float32))
+    assert 16 * blob.info.total_words < 3.6 * 9 * n
+    _check(blob, (ep.BF16, ep.FP8_E4M3, ep.UINT8, ep.FP32))
+
+
 def test_few_tiles_states_that_need_words_in_successive_steps():
     # symbols of frequency 1 next to one of frequency close to 2^11: a lane that has just taken a word often needs the next
     # one at once, which is what the guessing loop takes for granted that it does not
