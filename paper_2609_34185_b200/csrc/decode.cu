@@ -2100,14 +2100,9 @@ uint32_t split_rounds(BatchParams &P, uint32_t sms) {
         J.round_cost = rounds_total <= sms ? 1u : (J.V + 31u) / 32u;
         J.cost_begin = uint32_t(cost);
         cost += uint64_t(J.rounds) * J.round_cost;
-        // The guess costs nine instructions per step and, at 4 bpp (3.5 bits per symbol), the repetition of one group in 70 (at
-        // 5 bpp one in 25, at 6 one in 6).  1792-block tiles, us, with / without: 2.5 bpp 4 tiles 31.9 / 37.1, 8: 35.3 / 38.5,
-        // 10: 40.4 / 40.6, 12: 41.0 / 40.9; 4 bpp 4 tiles 33.3 / 37.1, 8: 36.7 / 38.9, 10: 41.6 / 41.0; 4.5 bpp 4 tiles 34.3 / 37.1, 8:
-        // 37.8 / 39.0; 5 bpp 4 tiles 36.3 / 37.2, 8: 40.0 / 39.1; 5.5 bpp 4 tiles 41.5 / 37.2.
-        // 3640: 2.5 bpp 4 tiles 63.5 / 74.4, 8: 70.7 / 78.3, 12: 83.5 / 86.0; 4 bpp 4 tiles 66.0 / 74.9, 8: 75.4 / 80.1.  896: 2.5 bpp 8
-        // tiles 19.8 / 21.0; 4 bpp 4 tiles 18.8 / 20.3, 8: 21.1 / 21.3; 5 bpp 4 tiles 20.6 / 20.4.  Tiles of 224 blocks, seven
-        // groups, are over before it pays: 4 bpp 4 tiles 7.7 / 7.7, 8: 8.6 / 8.0.
-        J.guess = (lo <= 4u && J.payload_bits <= (J.V > 1024u ? 4.5f : 4.2f)) || (lo <= 8u && J.V >= 512u && J.payload_bits <= 4.1f);
+        uint32_t tables = 0, symbols = 0;                    // of the coordinates
+        for (int t = 1; t < EP_NUM_TABLES; ++t) { tables += J.tK[t] != 0; symbols += J.tK[t]; }
+        J.guess = tables && ep::guess_pays(lo, J.V < J.n_vec ? J.V : J.n_vec, J.payload_bits, double(symbols) / tables);
     }
     const uint32_t grid = uint32_t(rounds_total < sms ? rounds_total : sms);
     // (a tensor has under 2^27 blocks, so sixteen of them cost under 2^28 groups and rounds: 32-bit arithmetic in the kernel)

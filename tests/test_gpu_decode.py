@@ -642,6 +642,27 @@ def test_few_tiles_whose_last_group_is_not_full(R, C, V):
     _check(blob, (ep.BF16, ep.FP8_E4M3, ep.UINT8, ep.FP32))
 
 
+@pytest.mark.parametrize("R,C,V,spread", [
+    (300, 256, 40, 0.4),          # a full group and a group of eight lanes
+    (40, 320, 63, 0.7),           # rows of 40 blocks
+    (64, 256, 64, 0.7),
+    (75, 1024, 65, 0.7),          # two full groups and one lane
+    (111, 264, 95, 0.9),          # rows of 33 blocks, tiles that end inside rows
+    (1184, 2048, 257, 1.0),       # eight tiles per SM
+])
+def test_few_tiles_short_tiles_at_rates_that_are_guessed(R, C, V, spread):
+    rng = np.random.default_rng(9400 + R + V)
+    n = R * C // 8
+    fields = np.zeros((n, 9), np.int32)
+    fields[:, 0] = rng.integers(0, 2, n)
+    fields[:, 1:8] = np.rint(rng.standard_normal((n, 7)) * spread).astype(np.int32)
+    fields[:, 8] = np.rint(rng.standard_normal(n) * spread).astype(np.int32)
+    blob = ep.pack_fields(fields, R, C, 11, V, rng.uniform(0.01, 0.05, R).astype(np.float32))
+    assert ep.decode_scratch_bytes(blob.info) == 0
+    assert 16 * blob.info.total_words < (4.9 - 42 / V ** 0.5 if R > 1000 else 5.1 - 29 / V ** 0.5) * 9 * n
+    _check(blob, (ep.BF16, ep.FP8_E4M3, ep.UINT8, ep.FP32))
+
+
 def test_few_tiles_states_that_need_words_in_successive_steps():
     # symbols of frequency 1 next to one of frequency close to 2^11: a lane that has just taken a word often needs the next
     # one at once, which is what the guessing loop takes for granted that it does not

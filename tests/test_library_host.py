@@ -3,6 +3,7 @@ streams on the same inputs), library stream -> oracle decoder, structural valida
 import ctypes
 import os
 import re
+import subprocess
 
 import numpy as np
 import pytest
@@ -184,3 +185,27 @@ def test_bench_tile_size_rules_mirror_the_library():
         for shapes in (synth.BLOCK_SHAPES, [(8192, 8192)], [(4096, 4096), (4096, 11008), (11008, 4096)]):
             for ctas in (148, 132, 0):
                 assert bench.suggest_v_batch_py(shapes, vmax, ctas) == ep.suggest_tile_vectors_batch(shapes, bpp, ctas)
+
+
+@pytest.mark.parametrize("rows,bits,taken,left", [
+    # tiles per SM and blocks per tile at which the guessing loop was measured ahead, and behind
+    (synth.gaussian_rows, 2.4, ((4, 256), (8, 384)), ((4, 64), (9, 3640))),
+    (synth.laplace_rows, 2.8, ((4, 512), (8, 1792)), ((4, 128), (8, 256))),
+    (synth.gaussian_rows, 3.6, ((1, 704), (4, 896), (5, 1792), (8, 1280)), ((4, 256), (8, 512))),
+    (synth.laplace_rows, 3.7, ((4, 3640),), ((4, 256), (8, 704), (8, 1024), (5, 1792), (8, 3640))),
+    (synth.gaussian_rows, 3.9, ((4, 1024), (8, 3640), (6, 2560)), ((4, 384), (8, 512))),
+    (synth.student_t_rows, 3.9, (), ((8, 704), (8, 1792), (8, 3640))),
+    (synth.gaussian_rows, 4.3, ((4, 2560), (2, 3640)), ((4, 704), (8, 1280), (12, 3640))),
+    (synth.laplace_rows, 4.3, (), ((4, 1792), (1, 3640), (8, 3640))),
+])
+def test_guess_of_the_few_tile_loop_is_taken_where_it_was_measured_ahead(tmp_path, rows, bits, taken, left):
+    I = ep.encode(rows(512, 1024, 31), bits * 9 / 8 + 0.3, tile_vectors=512, b_start=11, b_max=11).info
+    symbols, bits = sum(I.table_K[1:]) / 16, 16 * I.total_words / (9 * I.R * I.C / 8)
+    src, exe = tmp_path / "p.cpp", tmp_path / "p"
+    src.write_text('#include "stream.hpp"\n#include <cstdio>\nint main() {\n'
+                   + "".join(f'    std::printf("%d ", int(ep::guess_pays({n}u, {v}u, {bits!r}, {symbols!r})));\n' for n, v in taken + left)
+                   + "}\n")
+    subprocess.run(["g++", "-std=c++17", "-I", os.path.join(ROOT, "include"), "-I", os.path.join(ROOT, "paper_2609_34185_b200", "csrc"),
+                    str(src), "-o", str(exe)], check=True)
+    got = subprocess.run([str(exe)], check=True, capture_output=True, text=True).stdout.split()
+    assert got == ["1"] * len(taken) + ["0"] * len(left)
