@@ -2524,12 +2524,8 @@ extern "C" int ep_decode_gemm(const ep_info *info, const void *d_stream, const v
     // SM's issue slots; 16 tokens, us, even steps / steps of 30 and a rest: 70 rows per SM of 10240 x 3840 53.5 / 58.4, 31 rows of 2048
     // columns 19.7 / 24.0, 50 23.0 / 24.5, 62 29.8 / 34.1)
     P.rows_per_cta = (I.R + uint32_t(sms) - 1u) / uint32_t(sms);
-    auto steps_of = [&](uint32_t rows) { return (P.rows_per_cta + rows - 1u) / rows; };
-    // The shape that takes fewer steps, else that with the larger rings or four units of x.  4096 columns at 4 bpp, 32 tokens, us,
-    // steps of 24 / 30 rows at most: 10 rows per SM 19.9 / 20.3, 23: 23.5 / 24.0, 28: 37.0 / 26.2, 56: 57.5 / 48.5, 70: 65.6 / 63.9,
-    // 91: 79.5 / 81.0, 120: 108.2 / 91.9.
-    const uint32_t most = steps_of(30u) < steps_of(24u) ? 30u : 24u;
-    P.steps = steps_of(most);
+    const uint32_t most = ep::gemm_rows_per_step(T, P.rows_per_cta, I.C);
+    P.steps = (P.rows_per_cta + most - 1u) / most;
     P.rows_per_step = (P.rows_per_cta + P.steps - 1u) / P.steps;
     P.groups = I.C / 256u;
     if (I.n_tiles != I.R) return EP_ERR_BAD_ARG;

@@ -65,6 +65,17 @@ inline bool guess_pays(uint32_t tiles, uint32_t blocks, double bits, double symb
     return bits <= 4.9 - (wide ? 48.0 : 34.0) / root && !(wide && bits > 3.6);
 }
 
+// ep_decode_gemm: most rows of W per step, 30 or 24 (what each leaves room for: GemmShape), for CTAs of `rows` rows.
+// The one that takes fewer steps.  4096 columns at 4 bpp, 32 tokens, us, 24 / 30: 10 rows per SM 19.9 / 20.3, 23: 23.5 / 24.0, 28:
+// 37.0 / 26.2, 56: 57.5 / 48.5, 70: 65.6 / 63.9, 91: 79.5 / 81.0, 120: 108.2 / 91.9.
+// With equal steps 24 for 17 to 32 tokens (four units of x), and up to 16 tokens for the larger payload rings, but for short rows, for which
+// they ask for more than a row has.  16 tokens, 4 bpp, graph of launches, us, 24 / 30: 256 columns 16 rows 4.9 / 4.7, 512 columns
+// 20 rows 5.9 / 5.7 (one token 6.0 / 5.8), 768 columns 70 rows 14.7 / 15.4 (one token 20 rows 7.0 / 6.8), 1024 columns 70 rows 17.4 / 17.9.
+inline uint32_t gemm_rows_per_step(uint32_t tokens, uint32_t rows, uint32_t columns) {
+    const auto steps = [rows](uint32_t most) { return (rows + most - 1u) / most; };
+    return steps(30u) < steps(24u) || (tokens <= 16u && columns <= 512u) ? 30u : 24u;
+}
+
 int parse_info(const void *blob, size_t n, ep_info *out);
 
 }  // namespace ep

@@ -122,14 +122,12 @@ def test_decode_matmul_of_17_to_32_tokens_in_thirty_rows(R, C, T):
     _check(blob, T, R + C + T)
 
 
-@pytest.mark.parametrize("R,C,T,spread", [
-    (40, 8192, 16, 60),           # a group takes half a chunk of the wide ring: it goes round several times
-    (148 * 24, 1024, 16, 4),      # one full step of 24 rows
-    (148 * 24 + 1, 512, 1, 60),   # two steps, the last CTA with fewer rows
-    (148 * 48 - 5, 256, 9, 1),    # two full steps of one group per row
-    (148 * 70, 768, 13, 20),      # three steps
-])
-def test_decode_matmul_of_up_to_16_tokens_in_24_rows(R, C, T, spread):
+def _rows_per_step(T, per_sm, C):
+    """Most rows per step of the shape that the launcher takes."""
+    return 30 if -(-per_sm // 30) < -(-per_sm // 24) or (T <= 16 and C <= 512) else 24
+
+
+def _check_spread(R, C, T, spread):
     rng = np.random.default_rng(78)
     n = R * C // 8
     fields = np.zeros((n, 9), np.int32)
@@ -138,6 +136,32 @@ def test_decode_matmul_of_up_to_16_tokens_in_24_rows(R, C, T, spread):
     fields[:, 8] = np.rint(rng.standard_normal(n) * spread / 2).astype(np.int32)
     blob = ep.pack_fields(fields, R, C, 11, C // 8, rng.uniform(0.01, 0.05, R).astype(np.float32))
     _check(blob, T, R + C + T)
+
+
+@pytest.mark.parametrize("per_sm,short,C,T,spread", [
+    (1, 108, 8192, 16, 60),       # a group takes half a chunk of the wide ring: it goes round several times
+    (24, 0, 1024, 16, 4),         # one full step of 24 rows
+    (31, 40, 768, 1, 60),         # two steps, fewer rows in the second and in the last CTA
+    (48, 5, 768, 9, 1),           # two full steps
+    (70, 0, 768, 13, 20),         # three steps
+])
+def test_decode_matmul_of_up_to_16_tokens_in_24_rows(per_sm, short, C, T, spread):
+    assert _rows_per_step(T, per_sm, C) == 24
+    _check_spread(torch.cuda.get_device_properties(0).multi_processor_count * per_sm - short, C, T, spread)
+
+
+@pytest.mark.parametrize("per_sm,short,C,T,spread", [
+    (28, 3, 4096, 16, 4),         # several times round the ring of 4 x 256 bytes; the last CTA with fewer rows
+    (30, 0, 512, 9, 20),          # one full step
+    (60, 0, 768, 16, 20),         # two full steps
+    (73, 0, 256, 13, 60),         # three steps of 25 rows, one group per row
+    (25, 147, 512, 1, 60),        # one step of 25 rows
+    (48, 5, 256, 9, 1),           # two steps of 24 rows: short rows stay with the small ring
+    (1, 108, 512, 16, 4),
+])
+def test_decode_matmul_of_up_to_16_tokens_in_30_rows(per_sm, short, C, T, spread):
+    assert _rows_per_step(T, per_sm, C) == 30
+    _check_spread(torch.cuda.get_device_properties(0).multi_processor_count * per_sm - short, C, T, spread)
 
 
 def test_decode_matmul_more_tokens_than_one_launch_and_repeated_calls():

@@ -209,3 +209,17 @@ def test_guess_of_the_few_tile_loop_is_taken_where_it_was_measured_ahead(tmp_pat
                     str(src), "-o", str(exe)], check=True)
     got = subprocess.run([str(exe)], check=True, capture_output=True, text=True).stdout.split()
     assert got == ["1"] * len(taken) + ["0"] * len(left)
+
+
+def test_rows_per_step_of_the_fused_product(tmp_path):
+    # tokens, rows per SM, columns -> the shape that was measured ahead
+    cases = [(16, 70, 3840, 24), (16, 28, 4096, 30), (16, 56, 8192, 30), (16, 20, 512, 30), (1, 24, 256, 30), (16, 70, 512, 30),
+             (16, 70, 768, 24), (16, 16, 1024, 24), (32, 20, 256, 24), (17, 70, 512, 24), (32, 28, 1024, 30), (32, 91, 4096, 24),
+             (16, 25, 4096, 30), (16, 31, 4096, 24), (16, 73, 4096, 30), (16, 1, 1024, 24)]
+    src, exe = tmp_path / "p.cpp", tmp_path / "p"
+    src.write_text('#include "stream.hpp"\n#include <cstdio>\nint main() {\n'
+                   + "".join(f'    std::printf("%u ", ep::gemm_rows_per_step({t}u, {r}u, {c}u));\n' for t, r, c, _ in cases) + "}\n")
+    subprocess.run(["g++", "-std=c++17", "-I", os.path.join(ROOT, "include"), "-I", os.path.join(ROOT, "paper_2609_34185_b200", "csrc"),
+                    str(src), "-o", str(exe)], check=True)
+    got = subprocess.run([str(exe)], check=True, capture_output=True, text=True).stdout.split()
+    assert got == [str(c[3]) for c in cases]
