@@ -753,15 +753,16 @@ __device__ __forceinline__ void decode_tile_plain(const JobParams &J, uint32_t t
 // step k's words.  The lanes that did follow with a lookup of their own and are back for the lookup of step k + 2.  If one
 // of them falls below 2^15 all the same (`lm`, the smallest such state), the ballots were wrong, and the group is decoded
 // again from its saved start by EP_BODY11_SHORT: no result depends on the guess.
-// The body is for groups in which every lane has a block (a tile's last one, if it is not full, takes EP_BODY11_SHORT): without
-// the lane's flag in every update it has 25 instructions per step instead of 30.
+// The body is for groups in which every lane has a block (a tile's last one, if it is not full, takes EP_BODY11_SHORT), so its updates
+// carry no lane's flag: 25 instructions per step with the two fences, 27 with flags (EP_T_STEP has 15).
 // The order below follows the times at which operands arrive (a warp issues in order): rank of the words, the late lanes'
 // end of the previous step (TAIL, predicate NP from two steps ago), lookup, word, work for the output (FILL), new state, the late
 // lanes' lookup, ballot.  Kept, it is 750 cycles per group by the latencies of the instructions (logic and multiply-add 4, population
 // count 17, comparison and ballot 17, shared memory 25).  The assembler has an order of its own, and moves nothing across a
 // signal to dependent launches, which has no effect after the kernel's first one and takes 4 cycles, nor across a read of
 // the clock, which takes 10 (and whose value has to be used: KEEP, once per tile): one after the word's load and one after the
-// ballot or at the step's end keep the order.  (That is a property of this assembler, CUDA 12.9, not of the language.)  Which is best
+// ballot or at the step's end keep the order.  (That is a property of this assembler, CUDA 12.9, not of the language: another one is
+// warned of below.)  Which is best
 // depends on what the output takes.  1792-block tiles at 3.5 bpp, us, three / eight tiles per SM, signals at the end, signals after
 // the ballot, clock reads after the ballot: BF16 32.7 / 36.0, 33.1 / 36.5, 33.2 / 36.7 (without fences, never-taken branches or warp
 // barriers 36 and more); FP32 33.5 / 37.0, 33.0 / 36.8, 33.4 / 37.5; E4M3 33.5 / 36.9, 33.6 / 36.7, 32.8 / 36.0; INT8 33.7 / 37.0,
@@ -769,6 +770,9 @@ __device__ __forceinline__ void decode_tile_plain(const JobParams &J, uint32_t t
 // EP_BODY11_SHORT takes 37.0 / 38.8.
 // PB / PPB: ballots of the previous step and the one before; PP: the lanes that took a word; NB / NP: this step's.
 // K: EP_K16, EP_K32 or EP_K8, by the bits of the output type
+#if __CUDACC_VER_MAJOR__ != 12 || __CUDACC_VER_MINOR__ != 9
+#warning "the order of EP_BODY11_GUESS was measured with CUDA 12.9: time it again, against EP_BODY11_SHORT and with other fences"
+#endif
 #define EP_G_SIGNAL "griddepcontrol.launch_dependents;\n\t"
 #define EP_K16_WORD(E) EP_G_SIGNAL
 #define EP_K16_BALLOT(E)
@@ -1369,6 +1373,9 @@ struct GemmShape {
     static constexpr uint32_t kSmem = kBar + 256;
     static constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((kN >> 3) << 17) | ((64u >> 4) << 24);   // f32 += bf16 x bf16, K-major both, N = kN, M = 64
     static_assert(kSmem <= 232448, "more shared memory than an sm_100 CTA can have");
+    // a group begins before its chunk's last two bytes and reads 510 bytes at most: all chunks but the newest hold them, behind the
+    // ring's end the mirror does
+    static_assert((kSlots - 1u) * kChunk >= kChunk - 2u + 510u && kRingMirror >= 510u && kRingMirror % kChunk == 0);
 };
 
 // a test that never waits
@@ -1486,7 +1493,7 @@ __device__ __forceinline__ void umma_commit(uint32_t bar) {
         "setp.gt.s32 pv, r3, 0;\n\t" "setp.lt.and.u32 pv, r4, %19, pv;\n\t"                                           \
         "mad.wide.u32 rb, r4, 1, ra;\n\t" "add.u32 r5, r2, r4;\n\t"                                                   \
         "@pv cp.async.cg.shared.global [r5], [rb], 16, r3;\n\t"                                                       \
-        "sub.u32 r4, r2, r10;\n\t" "setp.lt.and.u32 pq, r4, 512, pv;\n\t"   /* slots 0 and 1 are written to the mirror as well */ \
+        "sub.u32 r4, r2, r10;\n\t" "setp.lt.and.u32 pq, r4, 512, pv;\n\t"   /* the ring's first 512 bytes are written to the mirror as well */ \
         "@pq cp.async.cg.shared.global [r5+%20], [rb], 16, r3;\n\t"                                                  \
         "cp.async.commit_group;\n\t"                                                                                  \
         "add.cc.u32 r11, r11, %19;\n\t" "addc.u32 r12, r12, 0;\n\t" "sub.s32 r1, r1, %19;\n\t"                        \
@@ -1498,7 +1505,7 @@ __device__ __forceinline__ void umma_commit(uint32_t bar) {
         "add.u32 wthrA, wthrA, %19;\n\t" "sub.u32 r4, wthrA, r10;\n\t" "setp.lt.u32 pq, r4, %20 + %19 - 2;\n\t"                \
         "vote.sync.all.pred pq, pq, 0xffffffff;\n\t"                                                                  \
         "@pq bra.uni EP_RING;\n\t"                                                                                    \
-        "sub.u32 wthrA, wthrA, %20;\n\t" "sub.u32 %1, %1, %20;\n\t"   /* past the fourth slot: everything back by the ring */ \
+        "sub.u32 wthrA, wthrA, %20;\n\t" "sub.u32 %1, %1, %20;\n\t"   /* past the last slot: everything back by the ring */ \
         "ld.shared.u32 r5, [" EP_CTX "+52];\n\t" "sub.u32 r5, r5, %20;\n\t"                                           \
         "bar.warp.sync 0xffffffff;\n\t"                                                                               \
         "st.shared.u32 [" EP_CTX "+52], r5;\n\t"                                                                      \
@@ -1670,7 +1677,7 @@ __global__ void __launch_bounds__(kThreads, 1) ep_decode_gemm_kernel(const __gri
             const uint32_t *rec_next = J.tile_index + size_t(min(r + P.rows_per_step, P.R - 1u)) * 33u;
             const uint32_t off_next = __ldg(rec_next + 32);
             if (has_next && lane == 0) prefetch_l2(rec_next);
-            if (lane == 0) {                 // the next request is chunk 4, into slot 0
+            if (lane == 0) {                 // the next request is chunk kSlots, into slot 0
                 sts64(ctx + kCtxChain + kCcSrc, Tl.a0 + G::kRing);
                 sts32(ctx + kCtxChain + kCcRem, Tl.room - G::kRing);
                 sts32(ctx + kCtxChain + kCcDst, ring);
@@ -1685,9 +1692,13 @@ __global__ void __launch_bounds__(kThreads, 1) ep_decode_gemm_kernel(const __gri
             }
             uint32_t x = Tl.x, bal = 0, a = ring + Tl.lead;
             if (s == 0) wait_for_tables(tables);
-            // The short chain loses to the plain one's smaller number of instructions only where x takes twice the room.  4 bpp, us,
-            // short / plain: 16 tokens 8192 x 8192 79.1 / 80.3, 10240 x 3840 51.9 / 51.5; 32 tokens 4096 x 4096 26.3 / 25.6, 10240 x 3840
-            // 63.2 / 61.1.
+            // The short chain saves latency, the plain one instructions.  4096 columns at 4 bpp, us, short / plain:
+            //   16 tokens, 24 rows per step at most: 4 rows per SM 15.40 / 15.61, 12: 17.18 / 17.20, 24: 21.00 / 20.83, 70: 54.04 / 53.59;
+            //   up to 30: 28 rows 23.16 / 23.50, 60: 43.13 / 43.82 (10240 x 3840 51.9 / 51.5, 8192 x 8192 79.1 / 80.3);
+            //   32 tokens: 1 row 17.93 / 17.96, 4: 18.60 / 18.48, 16: 21.59 / 21.32, 24: 24.96 / 24.30, 28: 25.99 / 25.29, 70: 65.29 / 63.08
+            //   (256 columns 1 - 8 rows: 4.56 / 4.61).
+            // Up to 16 tokens either is ahead by 1 % or so, by shape and rows; beyond, waiting for x hides the chain.  Both in one kernel,
+            // chosen by the number of groups, took every product of 17 to 32 tokens 0.5 - 1 % longer.
             if constexpr (TPAD == 16u) EP_GEMM_ROW_ASM(EP_BODY11_SHORT, EP_SHORT_FIN);
             else EP_GEMM_ROW_ASM(EP_BODY11, "");
             cp_async_wait<0>();              // nothing may still be landing in the ring when the next row starts
