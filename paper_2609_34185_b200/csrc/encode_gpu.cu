@@ -1,7 +1,8 @@
 // CUDA back end of the EntroPack encoder (paper Sec. 3.2-3.6): row RMS, E8 quantisation with field
 // histograms, the bisection of Algorithm 1, the rate correction, row-scale refit and tiled 32-state rANS encoding run on the
-// GPU; the final tables are made on the host from the counts (a few kilobytes), by the code of the host back end, which also
-// takes over a search whose decisions the device leaves open.  Both back ends produce the same bytes for the same input.
+// GPU, one stream of launches without a wait in between.  The final tables are made there, for coding, and on the host, for the
+// blob, from the same counts (a few kilobytes) by the code of the host back end, which compares the two; that also takes over a search
+// whose decisions the device leaves open.  Both back ends produce the same bytes for the same input.
 //
 // Every result that enters the stream is the host code's bit for bit.  Where the host's operation order is
 // expensive here (two divisions per weight, sums in index order), the kernel computes the value another way together
@@ -12,7 +13,10 @@
 #include <mutex>
 
 #include <algorithm>
+#include <atomic>
+#include <chrono>
 #include <cmath>
+#include <cstddef>
 #include <cstring>
 #include <new>
 #include <vector>
@@ -29,6 +33,7 @@ using namespace ep;
 
 constexpr int kHistOrigin = -4096;       // kHistBins values per table: -4096 .. 4095
 constexpr uint32_t kMaxTableSymbols = 40960;   // sum of K over the 17 tables that a stream of this back end may have
+constexpr uint32_t kFewEntries = 2048, kSmemEntries = 11264;   // tile coder: entries in shared memory with several CTAs per SM, with one
 constexpr double kUnit = 1.1102230246251565e-16;   // 2^-53, the rounding unit of double
 
 // the wait of a kernel that is launched while the one before it ends (launch_chained): before it, only kernel parameters are read
@@ -80,11 +85,19 @@ __device__ __forceinline__ float rms_result(double acc, uint32_t C) {
     return __double2float_rn(m);
 }
 
-__global__ void __launch_bounds__(kRowThreads) row_rms_kernel(const float *__restrict__ W, uint32_t C, float *__restrict__ mu) {
+// The first kClearCtas CTAs clear the state and the histograms of the search (as memsets before this kernel they and their gaps took 10 us).
+constexpr uint32_t kClearCtas = 148;
+__global__ void __launch_bounds__(kRowThreads) row_rms_kernel(const float *__restrict__ W, uint32_t C, float *__restrict__ mu, uint4 *__restrict__ clear, uint32_t n_clear) {
     __shared__ double part[kRowThreads / 32];
     __shared__ __align__(16) float4 stage[kRowThreads];
     const uint32_t tid = threadIdx.x, n4 = C / 4;
-    const float4 *x = reinterpret_cast<const float4 *>(W + size_t(blockIdx.x) * C);   // 16-byte aligned: C % 8 == 0
+    if (blockIdx.x < kClearCtas) {
+#pragma unroll 4
+        for (uint32_t i = blockIdx.x * kRowThreads + tid; i < n_clear; i += kClearCtas * kRowThreads) clear[i] = make_uint4(0u, 0u, 0u, 0u);
+        return;
+    }
+    const uint32_t row = blockIdx.x - kClearCtas;
+    const float4 *x = reinterpret_cast<const float4 *>(W + size_t(row) * C);   // 16-byte aligned: C % 8 == 0
     double acc = 0.0;
     auto add = [&](const float4 v) {
         const double a = double(v.x), b = double(v.y), c = double(v.z), d = double(v.w);
@@ -102,7 +115,7 @@ __global__ void __launch_bounds__(kRowThreads) row_rms_kernel(const float *__res
     const double sum = cta_sum(acc, part), off = order_bound(C, sum);
     const float lo = rms_result(__dsub_rn(sum, off), C), hi = rms_result(__dadd_rn(sum, off), C);
     if (lo == hi) {
-        if (tid == 0) mu[blockIdx.x] = lo;
+        if (tid == 0) mu[row] = lo;
         return;
     }
     acc = 0.0;                                   // index order
@@ -119,7 +132,7 @@ __global__ void __launch_bounds__(kRowThreads) row_rms_kernel(const float *__res
                 acc = __dadd_rn(acc, __dmul_rn(double(v.w), double(v.w)));
             }
     }
-    if (tid == 0) mu[blockIdx.x] = rms_result(acc, C);
+    if (tid == 0) mu[row] = rms_result(acc, C);
 }
 
 // ---- E8 quantisation (Eq. 2-4) ---------------------------------------------------------------------------
@@ -287,6 +300,28 @@ constexpr uint32_t kCountSmem = 4 * kEvalSymbols;
 constexpr uint32_t kFirstCounts = 6144;          // counts that come back with the state; more take a second copy
 constexpr uint32_t kLevels = 4, kCandidates = (1u << kLevels) - 1u;
 
+// Symbols' entries by (coset, field, value): the two cosets' tables of a field have the same range here (the wider of
+// both ends), so that the second coset's entries follow at one distance.
+struct EncodeTables {
+    uint32_t base[9];                // byte offset of value 0's entry of field k (0: the coset) under coset 0, modulo 2^32
+    uint32_t coset;                  // bytes from coset 0's entries to coset 1's
+    uint32_t total;                  // entries
+};
+
+// What Eq. 17 needs of a symbol, without a division: x / f for x < 2^31 is umulhi(x, rcp) >> sh with
+// sh = ceil(log2 f) - 1 and rcp = ceil(2^(32 + sh) / f) (Granlund and Montgomery, "Division by invariant integers using
+// multiplication", 1994; exact for 31-bit x).  f = 1 takes rcp = 2^32 - 1, which gives x - 1, and an offset that
+// makes up for it.  With q = x / f the new state is q 2^b + x mod f + F = x + (2^b - f) q + F.
+// {rcp, first state that gives off a word: f 2^(31-b), 2^b - f, sh | offset << 16}
+__device__ __forceinline__ uint4 encode_entry(uint32_t fF, uint32_t b) {
+    const uint32_t M = 1u << b, f = max(fF & 0xFFFFu, 1u), F = fF >> 16;
+    if (f == 1u) return make_uint4(0xFFFFFFFFu, 1u << (31u - b), M - 1u, (F + M - 1u) << 16);
+    const uint32_t sh = 31u - __clz(int(f - 1u));
+    // (the quotient has at most 32 integer bits and a fraction of at least 1 / f: its ceiling is right in double)
+    const uint32_t rcp = uint32_t(ceil(__ddiv_rn(double(1ull << (32u + sh)), double(f))));
+    return make_uint4(rcp, f << (31u - b), M - f, sh | (F << 16));
+}
+
 struct CountDir { int32_t lo[EP_NUM_TABLES]; uint32_t K[EP_NUM_TABLES]; };
 
 // one scale of a pass (device memory)
@@ -313,8 +348,10 @@ struct SearchState {
     uint32_t stop;                   // the full passes are over
     uint32_t polished;               // ... because the rate correction ended (0: the tensor overflows the tables, the host decides)
     CountDir last, full;
-    uint64_t total_words;            // tile coding: words of the payload (more than a blob can hold are still told apart)
+    EncodeTables coder;              // tile coding: where the symbols' entries are,
+    uint32_t code;                   //              whether they are there and the tiles are to be coded,
     uint32_t tiles_done;             //              CTAs of the launch that are done
+    uint32_t reported;               // CTAs that have brought their share of this and of the counts to the host
     Candidate cand[kCandidates];
 };
 constexpr size_t kStateBytes = 8192;
@@ -336,6 +373,8 @@ struct CountParams {
     SearchState *state;
     uint32_t *cand_counts;           // per candidate kEvalSymbols
     uint32_t *last_counts, *full_counts;
+    uint4 *entries;                  // rate correction: the tile coder's entries, made by the pass that ends it, and
+    uint32_t *full_freq;             // the frequencies they are of (null: not wanted)
     uint32_t n_blocks, C, per_row;
     uint32_t mode, levels, ctas;     // ctas: per candidate
     uint32_t first;                  // first pass of the search: the bracket is {lo0, hi0}; of the rate correction: step 0
@@ -381,9 +420,11 @@ struct Evaluation { double cce, tables; uint32_t worst; bool too_many, above; };
 
 // All threads of a candidate's last CTA: ranges and offsets of its tables, counts to `out`, histogram back to zero; unless
 // only counts are wanted, the frequencies of Sec. 3.3 (integers: the host's exactly), C_CE of Eq. 8 and the largest alphabet.
-__device__ __forceinline__ Evaluation gather_counts(const CountParams &P, uint32_t k, uint32_t *out, uint32_t *f_of) {
-    __shared__ int32_t lo_of[EP_NUM_TABLES];
-    __shared__ uint32_t K_of[EP_NUM_TABLES], at_of[EP_NUM_TABLES + 1], seen_of[EP_NUM_TABLES];
+struct Ranges { int32_t lo[EP_NUM_TABLES]; uint32_t K[EP_NUM_TABLES], at[EP_NUM_TABLES + 1]; };    // a candidate's tables and where they start
+__device__ __forceinline__ Evaluation gather_counts(const CountParams &P, uint32_t k, uint32_t *out, uint32_t *f_of, Ranges &D) {
+    int32_t *const lo_of = D.lo;
+    uint32_t *const K_of = D.K, *const at_of = D.at;
+    __shared__ uint32_t seen_of[EP_NUM_TABLES];
     __shared__ double bits_of[EP_NUM_TABLES];
     Candidate &S = P.state->cand[k];
     const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
@@ -647,11 +688,68 @@ __device__ void polish(const CountParams &P, float s, const Evaluation &E) {
     S.s = to;
 }
 
+// All threads of the CTA that ended the rate correction: the tile coder's entries of the frequencies that gather_counts left in
+// shared memory, laid out as coder_layout does, so that coding starts without the host's tables (which are the same numbers: the
+// host compares them).  Alphabets beyond the coder's shared memory are left to the host.
+__device__ __noinline__ void make_coder(const CountParams &P, const uint32_t *f_of, const Ranges &D) {
+    const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+    int32_t lo = 0, hi = 0;                      // lane k: field k
+    if (lane >= 1u && lane < 9u) {
+        bool any = false;
+#pragma unroll
+        for (uint32_t c = 0; c < 2u; ++c) {
+            const uint32_t t = 8u * c + lane;
+            if (!D.K[t]) continue;
+            const int32_t end = D.lo[t] + int32_t(D.K[t]);
+            lo = any ? min(lo, D.lo[t]) : D.lo[t];
+            hi = any ? max(hi, end) : end;
+            any = true;
+        }
+    }
+    uint32_t upto = uint32_t(hi - lo);
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const uint32_t n = __shfl_up_sync(0xFFFFFFFFu, upto, d);
+        if (lane >= uint32_t(d)) upto += n;
+    }
+    const uint32_t first = upto - uint32_t(hi - lo), size = __shfl_sync(0xFFFFFFFFu, upto, 31);
+    if (D.at[EP_NUM_TABLES] > kMaxTableSymbols || 2u * size + 2u > kSmemEntries) return;
+    if (warp < EP_NUM_TABLES) {
+        const uint32_t t = warp, k = t ? ((t - 1u) & 7u) + 1u : 0u, K = D.K[t], at = D.at[t];
+        const uint32_t begin = t ? (t > 8u ? size : 0u) + __shfl_sync(0xFFFFFFFFu, first, int(k)) + uint32_t(D.lo[t] - __shfl_sync(0xFFFFFFFFu, lo, int(k)))
+                                 : 2u * size + uint32_t(D.lo[0]);
+        uint32_t F = 0;
+        for (uint32_t j0 = 0; j0 < K; j0 += 32u) {
+            const uint32_t j = j0 + lane, f = j < K ? f_of[at + j] : 0u;
+            uint32_t incl = f;
+#pragma unroll
+            for (int d = 1; d < 32; d <<= 1) {
+                const uint32_t n = __shfl_up_sync(0xFFFFFFFFu, incl, d);
+                if (lane >= uint32_t(d)) incl += n;
+            }
+            if (j < K) {
+                P.entries[begin + j] = encode_entry(f | (F + incl - f) << 16, uint32_t(P.rate.b));
+                P.full_freq[at + j] = f;
+            }
+            F += __shfl_sync(0xFFFFFFFFu, incl, 31);
+        }
+    } else if (warp == EP_NUM_TABLES && lane < 9u) {
+        EncodeTables &T = P.state->coder;
+        T.base[lane] = lane ? 16u * (first - uint32_t(lo)) : 32u * size;
+        if (lane == 0) {
+            T.coset = 16u * size;
+            T.total = 2u * size + 2u;
+            P.state->code = 1;
+        }
+    }
+}
+
 __global__ void __launch_bounds__(kCountThreads, 1) quantise_count_kernel(const __grid_constant__ CountParams P) {
     extern __shared__ __align__(16) uint32_t sm[];
     uint32_t *const hot = sm, *const win = sm + kHotWords;
-    __shared__ uint32_t range_from[EP_NUM_TABLES], range_to[EP_NUM_TABLES], last_cta;
+    __shared__ uint32_t range_from[EP_NUM_TABLES], range_to[EP_NUM_TABLES], last_cta, ended;
     __shared__ float s_shared;
+    __shared__ Ranges ranges;
     const uint32_t tid = threadIdx.x, lane = tid & 31u;
     const uint32_t k = blockIdx.x / P.ctas, part = blockIdx.x - k * P.ctas;      // candidate, and this CTA's share of the blocks
     Candidate &S = P.state->cand[k];
@@ -767,13 +865,15 @@ __global__ void __launch_bounds__(kCountThreads, 1) quantise_count_kernel(const 
         if (n) atomicAdd(&win[(1u + t) * kWinBins + uint32_t(int32_t(u) + kHotOrigin - kWinOrigin)], n);
     }
     __syncthreads();
+    static_assert(kWinBins % 32 == 0, "a warp's 32 counters are of one table");
     for (uint32_t j = tid; j < kWinWords; j += kCountThreads) {
-        const uint32_t n = win[j];
-        if (n) {
-            const uint32_t t = j / kWinBins, g = j % kWinBins + uint32_t(kWinOrigin - kHistOrigin);
-            atomicAdd(P.hist + (k * EP_NUM_TABLES + t) * kHistBins + g, n);
-            atomicMax(&range_from[t], kHistBins - g);
-            atomicMax(&range_to[t], g + 1u);
+        const uint32_t n = win[j], some = __ballot_sync(0xFFFFFFFFu, n != 0u);
+        if (!some) continue;
+        const uint32_t t = j / kWinBins, g = j % kWinBins + uint32_t(kWinOrigin - kHistOrigin), g0 = g - lane;
+        if (n) atomicAdd(P.hist + (k * EP_NUM_TABLES + t) * kHistBins + g, n);
+        if (lane == 0) {                         // the range of the 32: its first and last counter that is not zero
+            atomicMax(&range_from[t], kHistBins - (g0 + uint32_t(__ffs(int(some)) - 1)));
+            atomicMax(&range_to[t], g0 + 32u - uint32_t(__clz(int(some))));
         }
     }
     __syncthreads();
@@ -782,7 +882,7 @@ __global__ void __launch_bounds__(kCountThreads, 1) quantise_count_kernel(const 
         atomicMax(&S.to[tid], range_to[tid]);
     }
     if (!arrive_last(&S.finished, P.ctas, last_cta)) return;
-    const Evaluation E = gather_counts(P, k, P.mode == kPassSearch ? P.cand_counts + size_t(k) * kEvalSymbols : P.full_counts, sm);
+    const Evaluation E = gather_counts(P, k, P.mode == kPassSearch ? P.cand_counts + size_t(k) * kEvalSymbols : P.full_counts, sm, ranges);
     if (P.mode == kPassSearch) {
         if (tid < 32u) judge_candidate(P, k, E);
         if (!arrive_last(&P.state->closed, (1u << P.levels) - 1u, last_cta)) return;
@@ -796,7 +896,11 @@ __global__ void __launch_bounds__(kCountThreads, 1) quantise_count_kernel(const 
     if (tid == 0) {
         if (__ldcg(&S.overflow)) P.state->overflow = 1;
         if (P.mode == kPassPolish) polish(P, s, E);
+        const SearchState &G = *P.state;
+        ended = P.entries && __ldcg(&G.polished) && __ldcg(&G.stop) && !__ldcg(&G.undecided) && !__ldcg(&G.overflow);
     }
+    __syncthreads();
+    if (ended) make_coder(P, sm, ranges);
 }
 
 // ---- Eq. 13: row scales ----------------------------------------------------------------------------------
@@ -856,6 +960,8 @@ __global__ void __launch_bounds__(kRowThreads) refit_kernel(const float *__restr
     if (state) s = state->s_counted;             // launched behind the search, before the host knows the scale
     const float m = __ldg(mu + blockIdx.x);
     const float lo = refit_result(__dsub_rn(xp, off), pp, s, m), hi = refit_result(__dadd_rn(xp, off), pp, s, m);
+    // (launched while the tile coder runs, whose results it does not use; what is launched behind it, however, does)
+    if (blockIdx.x == gridDim.x - 1u) asm volatile("griddepcontrol.wait;" ::: "memory");
     if (lo == hi) {
         if (tid == 0) sigma[blockIdx.x] = lo;
         return;
@@ -883,28 +989,6 @@ __global__ void __launch_bounds__(kRowThreads) refit_kernel(const float *__restr
 }
 
 // ---- tile coding (Sec. 3.6 / App. "Tiled rANS implementation", Eq. 17) ---------------------------------------
-// Symbols' entries by (coset, field, value): the two cosets' tables of a field have the same range here (the wider of
-// both ends), so that the second coset's entries follow at one distance.
-struct EncodeTables {
-    uint32_t base[9];                // byte offset of value 0's entry of field k (0: the coset) under coset 0, modulo 2^32
-    uint32_t coset;                  // bytes from coset 0's entries to coset 1's
-    uint32_t total;                  // entries
-};
-
-// What Eq. 17 needs of a symbol, without a division: x / f for x < 2^31 is umulhi(x, rcp) >> sh with
-// sh = ceil(log2 f) - 1 and rcp = ceil(2^(32 + sh) / f) (Granlund and Montgomery, "Division by invariant integers using
-// multiplication", 1994; exact for 31-bit x).  f = 1 takes rcp = 2^32 - 1, which gives x - 1, and an offset that
-// makes up for it.  With q = x / f the new state is q 2^b + x mod f + F = x + (2^b - f) q + F.
-// {rcp, first state that gives off a word: f 2^(31-b), 2^b - f, sh | offset << 16}
-__device__ __forceinline__ uint4 encode_entry(uint32_t fF, uint32_t b) {
-    const uint32_t M = 1u << b, f = max(fF & 0xFFFFu, 1u), F = fF >> 16;
-    if (f == 1u) return make_uint4(0xFFFFFFFFu, 1u << (31u - b), M - 1u, (F + M - 1u) << 16);
-    const uint32_t sh = 31u - __clz(int(f - 1u));
-    // (the quotient has at most 32 integer bits and a fraction of at least 1 / f: its ceiling is right in double)
-    const uint32_t rcp = uint32_t(ceil(__ddiv_rn(double(1ull << (32u + sh)), double(f))));
-    return make_uint4(rcp, f << (31u - b), M - f, sh | (F << 16));
-}
-
 // (A kernel that comes up while the one before it runs takes that one's results by ordinary loads: __restrict__ and the
 // read-only path promise that nobody writes the data while the kernel exists, and let a load move above the wait.)
 __global__ void encode_entries_kernel(const uint32_t *fF, uint32_t n, uint32_t b, uint4 *entries) {
@@ -920,7 +1004,7 @@ __global__ void encode_entries_kernel(const uint32_t *fF, uint32_t n, uint32_t b
 // a group's fields are asked for four groups ahead and its symbols looked up before the steps that need them.
 // IN_SMEM: the symbols' entries in shared memory (up to 11 Ki symbols), else in global memory.  A CTA has four warps -
 // tiles spread over the SMs - or sixteen where its table takes so much shared memory that few CTAs fit an SM.
-constexpr uint32_t kTileThreads = 128, kTileThreadsMax = 512, kSmemEntries = 11264, kAhead = 4;
+constexpr uint32_t kTileThreads = 128, kTileThreadsMax = 512, kAhead = 4, kReportCtas = 8;
 
 // A group's nine steps.  A step's words are stored during the next one: ballot, population counts and address (some 60 cycles)
 // stay off the chain of states, and the store is predicated, not a branch.  P / Q: this and the previous step's
@@ -950,16 +1034,74 @@ constexpr uint32_t kTileThreads = 128, kTileThreadsMax = 512, kSmemEntries = 112
         EP_CODE_COUNT("ba") EP_CODE_STORE("pa", "ba", "ha") "}"                                                                                          \
         : "+r"(x), "+r"(end) : "l"(area), "r"(lt), "r"(act), RT(A8), RT(A7), RT(A6), RT(A5), RT(A4), RT(A3), RT(A2), RT(A1), RT(A0) : "memory")
 
+// The tables' place is in device memory: made by the pass that ended the search, or brought by the host.  A launch is for tables of more
+// than `above` and at most `most` entries (which the host does not know yet when it launches) and does nothing else.
+struct Report {                      // what `ctas` CTAs of the launch, behind those that code, bring to the host meanwhile
+    uint32_t ctas;
+    const uint32_t *last_counts, *full_counts, *full_freq;
+    uint32_t *mail;                  // page-locked: as DeviceBackend's mail
+};
+struct TileParams {
+    const uint4 *fields;
+    uint32_t n_vec, V, n_tiles, cap, above, most;
+    const uint4 *entries;
+    uint16_t *scratch;
+    uint32_t *index, *counts;
+    SearchState *state;
+    volatile uint64_t *total_words;  // page-locked: words of the payload (more than a blob can hold are still told apart)
+    Report report;
+};
+constexpr size_t kMailLast = kStateBytes, kMailFull = kMailLast + 4ull * kEvalSymbols, kMailFreq = kMailFull + 4ull * EP_NUM_TABLES * kHistBins,
+                 kMailDone = kMailFreq + 4ull * kMaxTableSymbols, kMailBytes = kMailDone + 64;      // done: u32 there, u32, u64 words
+
+__device__ __noinline__ void report_search(const TileParams &P, uint32_t cta) {
+    SearchState &S = *P.state;
+    const uint32_t at = cta * blockDim.x + threadIdx.x, step = P.report.ctas * blockDim.x, lane = threadIdx.x & 31u;
+    auto bring = [&](size_t to, const uint32_t *from, uint32_t n) {
+#pragma unroll 8
+        for (uint32_t i = at; i < n; i += step) P.report.mail[to / 4u + i] = __ldcg(from + i);
+    };
+    const uint32_t n_last = warp_sum(lane < EP_NUM_TABLES ? __ldcg(&S.last.K[lane]) : 0u), n_full = warp_sum(lane < EP_NUM_TABLES ? __ldcg(&S.full.K[lane]) : 0u);
+    bring(0, reinterpret_cast<const uint32_t *>(&S), uint32_t(offsetof(SearchState, cand) / 4u));
+    if (__ldcg(&S.has_last)) bring(kMailLast, P.report.last_counts, min(n_last, kEvalSymbols));
+    bring(kMailFull, P.report.full_counts, n_full);
+    if (__ldcg(&S.code)) bring(kMailFreq, P.report.full_freq, n_full);
+    __syncthreads();
+    if (threadIdx.x) return;
+    __threadfence_system();          // (cumulative: the whole CTA's stores)
+    if (atomicAdd(&S.reported, 1u) == P.report.ctas - 1u) {
+        __threadfence_system();
+        *const_cast<volatile uint32_t *>(P.report.mail + kMailDone / 4u) = 1u;
+    }
+}
+
 template <bool IN_SMEM>
-__global__ void __launch_bounds__(kTileThreadsMax) tile_encode_kernel(const uint4 *fields, uint32_t n_vec, uint32_t V,
-                                                                      uint32_t n_tiles, const __grid_constant__ EncodeTables T,
-                                                                      const uint4 *entries_global, uint16_t *scratch, uint32_t cap,
-                                                                      uint32_t *index, uint32_t *counts, SearchState *state) {
+__global__ void __launch_bounds__(kTileThreadsMax) tile_encode_kernel(const __grid_constant__ TileParams P) {
     extern __shared__ __align__(16) uint4 entries_smem[];
     __shared__ uint32_t last_cta;
-    __shared__ uint64_t part[kTileThreadsMax];
-    const uint32_t tid = threadIdx.x, lane = tid & 31u;
+    __shared__ uint64_t part[kTileThreadsMax / 32];
+    __shared__ EncodeTables tables;
+    __shared__ uint32_t code;
+    const uint32_t tid = threadIdx.x, lane = tid & 31u, coders = gridDim.x - P.report.ctas;
+    const uint32_t n_vec = P.n_vec, V = P.V, n_tiles = P.n_tiles, cap = P.cap;
+    const uint4 *const fields = P.fields, *const entries_global = P.entries;
+    uint16_t *const scratch = P.scratch;
+    uint32_t *const index = P.index, *const counts = P.counts;
+    SearchState *const state = P.state;
     chained_start();
+    if (blockIdx.x >= coders) {
+        report_search(P, blockIdx.x - coders);
+        return;
+    }
+    if (tid < sizeof(EncodeTables) / 4u) reinterpret_cast<uint32_t *>(&tables)[tid] = __ldcg(reinterpret_cast<const uint32_t *>(&state->coder) + tid);
+    if (tid == sizeof(EncodeTables) / 4u) code = __ldcg(&state->code);
+    __syncthreads();
+    EncodeTables T;                  // (by shuffles: known to be warp-uniform, see the warp's number below)
+#pragma unroll
+    for (int k = 0; k < 9; ++k) T.base[k] = __shfl_sync(0xFFFFFFFFu, tables.base[k], 0);
+    T.coset = __shfl_sync(0xFFFFFFFFu, tables.coset, 0);
+    T.total = __shfl_sync(0xFFFFFFFFu, tables.total, 0);
+    if (!__shfl_sync(0xFFFFFFFFu, code, 0) || T.total <= P.above || T.total > P.most) return;
     if (IN_SMEM) {
         for (uint32_t i = tid; i < T.total; i += blockDim.x) entries_smem[i] = entries_global[i];
         __syncthreads();
@@ -1010,24 +1152,41 @@ __global__ void __launch_bounds__(kTileThreadsMax) tile_encode_kernel(const uint
         if (lane == 0) counts[tile] = cap - end;
     }
     // the last CTA turns the counts into offsets (the tile records' last words and the final one)
-    if (!arrive_last(&state->tiles_done, gridDim.x, last_cta)) return;
-    const uint32_t per = (n_tiles + blockDim.x - 1u) / blockDim.x;
-    const uint32_t t0 = min(tid * per, n_tiles), t1 = min(t0 + per, n_tiles);
-    uint64_t sum = 0;
-    for (uint32_t t = t0; t < t1; ++t) sum += __ldcg(counts + t);
-    part[tid] = sum;
-    __syncthreads();
-    for (uint32_t d = 1; d < blockDim.x; d <<= 1) {
-        const uint64_t add = tid >= d ? part[tid - d] : 0u;
+    if (!arrive_last(&state->tiles_done, coders, last_cta)) return;
+    // (eight tiles per thread and turn, their loads under way together: one after another they took 0.7 us each, 16 us for 2743 tiles)
+    const uint32_t warps = blockDim.x >> 5;
+    uint64_t all = 0;
+    for (uint32_t t0 = 0; t0 < n_tiles; t0 += 8u * blockDim.x) {
+        const uint32_t t = t0 + 8u * tid;
+        uint32_t n[8];
+#pragma unroll
+        for (uint32_t u = 0; u < 8u; ++u) n[u] = t + u < n_tiles ? __ldcg(counts + t + u) : 0u;
+        uint64_t sum = 0;
+#pragma unroll
+        for (uint32_t u = 0; u < 8u; ++u) sum += n[u];
+        uint64_t upto = sum;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const uint64_t before = __shfl_up_sync(0xFFFFFFFFu, upto, d);
+            if (lane >= uint32_t(d)) upto += before;
+        }
+        if (lane == 31u) part[tid >> 5] = upto;
         __syncthreads();
-        part[tid] += add;
+        uint64_t at = all + upto - sum;
+        for (uint32_t w = 0; w < warps; ++w) {
+            if (w < tid >> 5) at += part[w];
+            all += part[w];
+        }
+#pragma unroll
+        for (uint32_t u = 0; u < 8u; ++u) {
+            if (t + u < n_tiles) index[size_t(t + u) * 33u + 32u] = uint32_t(at);
+            at += n[u];
+        }
         __syncthreads();
     }
-    uint32_t at = uint32_t(part[tid] - sum);
-    for (uint32_t t = t0; t < t1; ++t) { index[size_t(t) * 33u + 32u] = at; at += __ldcg(counts + t); }
-    if (tid == blockDim.x - 1u) {
-        index[size_t(n_tiles) * 33u] = uint32_t(part[tid]);
-        state->total_words = part[tid];
+    if (tid == 0) {
+        index[size_t(n_tiles) * 33u] = uint32_t(all);
+        *P.total_words = all;
         state->tiles_done = 0;
     }
 }
@@ -1035,9 +1194,10 @@ __global__ void __launch_bounds__(kTileThreadsMax) tile_encode_kernel(const uint
 // Move every tile's words from the end of its area to its place in the payload: one CTA per tile (with a warp per tile the
 // copy of 20 MB took 34 us, all of it waiting for loads; 19 so), four bytes per lane, the destination aligned.
 __global__ void __launch_bounds__(512) compact_kernel(const uint16_t *scratch, uint32_t cap, const uint32_t *counts, const uint32_t *index,
-                                                      uint16_t *payload) {
+                                                      const SearchState *state, uint16_t *payload) {
     const uint32_t tid = threadIdx.x, tile = blockIdx.x;
     chained_start();
+    if (!__ldcg(&state->code)) return;           // nothing was coded
     uint32_t n = counts[tile];
     const uint16_t *src = scratch + size_t(tile) * cap + (cap - n);
     uint16_t *dst = payload + index[size_t(tile) * 33u + 32u];
@@ -1167,23 +1327,22 @@ public:
     ~DeviceBackend() override {
         // a call that ends early must not leave a copy into the page-locked buffers behind, which the next call may have then
         if (under_way_) cudaStreamSynchronize(st_);
-        if (event_) cudaEventDestroy(event_);
         if (mail_) g_mail_slot.release(mail_, mail_cap_);
     }
 
     int prepare(const std::vector<uint32_t> &sample) override {
         n_sample_ = uint32_t(sample.size());
         under_way_ = true;
-        EP_CUDA(cudaEventCreateWithFlags(&event_, cudaEventDisableTiming));
         int dev = 0;
         EP_CUDA(cudaGetDevice(&dev));
         EP_CUDA(cudaDeviceGetAttribute(&sms_, cudaDevAttrMultiProcessorCount, dev));
         EP_CUDA(cudaFuncSetAttribute(quantise_count_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kCountSmem)));
         EP_CUDA(cudaMemcpyAsync(w_.rows, sample.data(), 4ull * n_sample_, cudaMemcpyHostToDevice, st_));
-        EP_CUDA(cudaMemsetAsync(w_.state, 0, kStateBytes, st_));
-        EP_CUDA(cudaMemsetAsync(w_.hist, 0, kCandidates * kHistBytes, st_));       // every pass leaves it zero again
-        row_rms_kernel<<<R_, kRowThreads, 0, st_>>>(W_, C_, w_.mu);
+        // the state, and the histograms behind it (every pass leaves them zero again)
+        const size_t clear = size_t(reinterpret_cast<uint8_t *>(w_.hist) - reinterpret_cast<uint8_t *>(w_.state)) + kCandidates * kHistBytes;
+        row_rms_kernel<<<R_ + kClearCtas, kRowThreads, 0, st_>>>(W_, C_, w_.mu, reinterpret_cast<uint4 *>(w_.state), uint32_t(clear / 16u));
         EP_CUDA(cudaGetLastError());
+        state_clear_ = true;
         return EP_OK;
     }
     int count_sample(float s, Model &m) override { return count(w_.rows, n_sample_, s, nullptr, m); }
@@ -1191,7 +1350,10 @@ public:
 
     int search(const SearchJob &job, const ep_encode_opts &o, SearchResult &r, bool *done) override {
         *done = false;
-        EP_CUDA(cudaMemsetAsync(w_.state, 0, kStateBytes, st_));
+        if (!state_clear_) EP_CUDA(cudaMemsetAsync(w_.state, 0, kStateBytes, st_));
+        state_clear_ = false;
+        // with the refinement of rows (which this back end leaves to the host) the last pass's tables are not the final ones
+        const bool ahead = o.rdo_candidates <= 1;
         CountParams P = params(w_.rows, n_sample_, 0.0f, nullptr);
         P.mode = kPassSearch;
         P.rate = rate_params(job.target_bpp, o.retained_bits, job.sample_vectors, job.sample_rows, job.V, job.b);
@@ -1214,6 +1376,8 @@ public:
         F.lo0 = o.bracket_lo;
         F.hi0 = o.bracket_hi;
         F.last_step = o.polish_steps;
+        F.entries = ahead ? w_.entries : nullptr;
+        F.full_freq = w_.fF;
         for (F.step = 0;; ++F.step) {
             EP_CUDA(launch_count(F, F.step > 0 || o.search_steps > 0));
             if (F.step == o.polish_steps) break;
@@ -1223,18 +1387,33 @@ public:
                 if (state()->stop) break;
             }
         }
-        // the row scales of the quantisation that is there now: while the host looks at the counts the GPU has nothing else to
-        // do (and if the host goes on to another scale, finish makes them again)
-        const int rc = fetch(true, [&] {
-            refit_kernel<<<R_, kRowThreads, 0, st_>>>(W_, C_, w_.fields, 0.0f, w_.state, w_.mu, w_.sigma);
-            return cudaGetLastError();
-        });
+        int rc = EP_OK;
+        if (ahead) {
+            // The tiles are coded and the row scales made without waiting for the host, which meanwhile makes its own tables of the same
+            // counts.  If the search goes on on the host, what was coded is not used.  Whole encode, copied back, with the clearing in
+            // row_rms_kernel and the faster prefix sum of the tiles: 10240 x 3840 at 4 bpp 1249 -> 1209 us, 512 x 1024 240 -> 222.
+            // The refit runs beside the tile coder: one after the other they took 109 us for 10240 x 3840, together 90.
+            std::memset(mail_ + kMailDone, 0, kMailBytes - kMailDone);
+            const uint32_t n_tiles = uint32_t((uint64_t(R_) * (C_ / 8) + V_ - 1) / V_);
+            EP_CUDA(launch_coder(n_tiles, 0u, kFewEntries, true));
+            EP_CUDA(launch_beside(refit_kernel, R_, kRowThreads, 0, W_, C_, static_cast<const uint4 *>(w_.fields), 0.0f, static_cast<const SearchState *>(w_.state),
+                                   static_cast<const float *>(w_.mu), w_.sigma));
+            EP_CUDA(launch_coder(n_tiles, kFewEntries, kSmemEntries, false));
+            EP_CUDA(launch_compact(n_tiles));
+            rc = await_report();
+        } else {
+            rc = fetch(true);
+            if (!rc) refit_kernel<<<R_, kRowThreads, 0, st_>>>(W_, C_, w_.fields, 0.0f, w_.state, w_.mu, w_.sigma);
+            EP_CUDA(cudaGetLastError());
+        }
         if (rc) return rc;
         const SearchState &S = *state();
         if (S.undecided) {
             EP_CUDA(cudaMemsetAsync(w_.state, 0, kStateBytes, st_));
             return EP_OK;
         }
+        coded_ = ahead && S.code;
+        coded_b_ = job.b;
         r.s = sigma_of_ = S.s_counted;
         sigma_there_ = true;
         r.polished = S.polished != 0;
@@ -1248,10 +1427,10 @@ public:
     int begin_finish(float s, int b, uint32_t V, const Model &m) override {
         const uint64_t nvec = uint64_t(R_) * (C_ / 8);
         const uint32_t n_tiles = uint32_t((nvec + V - 1) / V);
-        const uint32_t cap = 9u * V;
         uint64_t symbols = 0;
         for (int t = 0; t < EP_NUM_TABLES; ++t) symbols += m.t[t].K();
         if (symbols > kMaxTableSymbols) return EP_ERR_UNSUPPORTED;
+        if (coded_ && sigma_there_ && sigma_of_ == s && coded_b_ == b && V == V_ && coded_with(m)) return EP_OK;
         const CoderLayout L = coder_layout(m);
         if (L.entries() > kCoderEntries) return EP_ERR_UNSUPPORTED;      // (no count lies outside the histogram: cannot happen)
         const uint32_t size = L.size;
@@ -1271,23 +1450,16 @@ public:
         T.base[0] = 32u * size;                  // the coset's two entries last
         for (uint32_t j = 0; j < m.t[0].K(); ++j) fF[2u * size + uint32_t(m.t[0].lo) + j] = m.t[0].f[j] | (m.t[0].F[j] << 16);
         EP_CUDA(cudaMemcpyAsync(w_.fF, fF.data(), 4ull * fF.size(), cudaMemcpyHostToDevice, st_));
+        struct { EncodeTables T; uint32_t code, tiles_done; } coder = {T, 1u, 0u};
+        static_assert(offsetof(SearchState, code) == offsetof(SearchState, coder) + sizeof(EncodeTables) &&
+                      offsetof(SearchState, tiles_done) == offsetof(SearchState, code) + 4, "one copy");
+        EP_CUDA(cudaMemcpyAsync(&w_.state->coder, &coder, sizeof(coder), cudaMemcpyHostToDevice, st_));
+        std::memset(mail_ + kMailDone, 0, kMailBytes - kMailDone);
         EP_CUDA(launch_chained(encode_entries_kernel, (T.total + 127u) / 128u, 128, 0, w_.fF, T.total, uint32_t(b), w_.entries));
-        if (T.total <= kSmemEntries) {
-            const uint32_t threads = T.total <= 2048u ? kTileThreads : kTileThreadsMax;
-            const size_t smem = 16ull * T.total + threads / 32u * (kAhead * 512u);
-            if (smem > 40u * 1024u)      // (always the same limit: another thread's call must not lower it before the launch)
-                EP_CUDA(cudaFuncSetAttribute(tile_encode_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(16u * kSmemEntries + kTileThreadsMax / 32u * (kAhead * 512u))));
-            EP_CUDA(launch_chained(tile_encode_kernel<true>, (n_tiles + threads / 32u - 1u) / (threads / 32u), threads, smem, w_.fields, uint32_t(nvec), V,
-                                   n_tiles, T, w_.entries, w_.scratch, cap, w_.index, w_.counts, w_.state));
-        } else {
-            EP_CUDA(launch_chained(tile_encode_kernel<false>, (n_tiles + kTileThreads / 32u - 1u) / (kTileThreads / 32u), kTileThreads,
-                                   kTileThreads / 32u * (kAhead * 512u), w_.fields,
-                                   uint32_t(nvec), V, n_tiles, T, w_.entries, w_.scratch, cap, w_.index, w_.counts, w_.state));
-        }
-        // (few CTAs: more threads per tile.  Whole encode, us, 512 / 128 threads: 37 tiles 247.4 / 251.0, 289 346.1 / 348.3, 577 397.8 / 397.9,
-        // 1153 528.5 / 528.1, 2305 at 8 bpp 836.9 / 829.1, 4610 1320.7 / 1310.6)
-        EP_CUDA(launch_chained(compact_kernel, n_tiles, n_tiles < 600u ? 512u : 128u, 0, w_.scratch, cap, w_.counts, w_.index, w_.payload));
-        EP_CUDA(cudaMemcpyAsync(&state()->total_words, &w_.state->total_words, sizeof(state()->total_words), cudaMemcpyDeviceToHost, st_));
+        if (T.total <= kFewEntries) EP_CUDA(launch_coder(n_tiles, 0u, kFewEntries, false));
+        else if (T.total <= kSmemEntries) EP_CUDA(launch_coder(n_tiles, kFewEntries, kSmemEntries, false));
+        else EP_CUDA(launch_coder(n_tiles, kSmemEntries, ~0u, false));
+        EP_CUDA(launch_compact(n_tiles));
         if (!sigma_there_ || sigma_of_ != s) refit_kernel<<<R_, kRowThreads, 0, st_>>>(W_, C_, w_.fields, s, nullptr, w_.mu, w_.sigma);
         EP_CUDA(cudaGetLastError());
         return EP_OK;
@@ -1308,7 +1480,7 @@ public:
             if (rc) return rc;
             EP_CUDA(cudaMemcpyAsync(out->data() + L.off_scales, w_.sigma, L.total - L.off_scales, cudaMemcpyDeviceToHost, st_));
             EP_CUDA(cudaStreamSynchronize(st_));
-            const uint64_t total = state()->total_words;
+            const uint64_t total = *total_words();
             if (total >= (1ull << 31)) return EP_ERR_UNSUPPORTED;
             if (total <= room) {
                 under_way_ = false;
@@ -1320,11 +1492,80 @@ public:
     }
 
 private:
-    // mail: state, counts of the last step, counts of the full pass
-    static constexpr size_t kMailBytes = kStateBytes + 4ull * kEvalSymbols + kHistBytes;
+    // mail: state, counts of the last step, counts and frequencies of the full pass, what kernels write there themselves
     SearchState *state() { return reinterpret_cast<SearchState *>(mail_); }
-    uint32_t *last_counts() { return reinterpret_cast<uint32_t *>(mail_ + kStateBytes); }
-    uint32_t *full_counts() { return last_counts() + kEvalSymbols; }
+    uint32_t *last_counts() { return reinterpret_cast<uint32_t *>(mail_ + kMailLast); }
+    uint32_t *full_counts() { return reinterpret_cast<uint32_t *>(mail_ + kMailFull); }
+    volatile uint32_t *reported() { return reinterpret_cast<volatile uint32_t *>(mail_ + kMailDone); }
+    volatile uint64_t *total_words() { return reinterpret_cast<volatile uint64_t *>(mail_ + kMailDone + 8); }
+    // the device's frequencies are the model's
+    bool coded_with(const Model &m) const {
+        const uint32_t *f = reinterpret_cast<const uint32_t *>(mail_ + kMailFreq);
+        for (const Table &t : m.t) {
+            if (t.f.size() != t.K() || std::memcmp(f, t.f.data(), 4ull * t.K())) return false;
+            f += t.K();
+        }
+        return true;
+    }
+    // Tile coder for tables of more than `above` and at most `most` entries.  Few entries: four warps per CTA while the tiles then fit the
+    // SMs at once (five such CTAs per SM), else eight, four times, or sixteen, three times
+    cudaError_t launch_coder(uint32_t n_tiles, uint32_t above, uint32_t most, bool report) {
+        const bool in_smem = most <= kSmemEntries;
+        uint32_t threads = kTileThreads;
+        if (in_smem) threads = most > kFewEntries || n_tiles > 32u * uint32_t(sms_) ? kTileThreadsMax : n_tiles > 20u * uint32_t(sms_) ? 2u * kTileThreads : kTileThreads;
+        const size_t stage = kAhead * 512u, smem = threads / 32u * stage + (in_smem ? 16ull * most : 0u);
+        TileParams P{};
+        P.fields = w_.fields;
+        P.n_vec = uint32_t(uint64_t(R_) * (C_ / 8));
+        P.V = V_;
+        P.n_tiles = n_tiles;
+        P.cap = 9u * V_;
+        P.above = above;
+        P.most = most;
+        P.entries = w_.entries;
+        P.scratch = w_.scratch;
+        P.index = w_.index;
+        P.counts = w_.counts;
+        P.state = w_.state;
+        P.total_words = total_words();
+        if (report) P.report = {kReportCtas, w_.last_counts, w_.full_counts, w_.fF, reinterpret_cast<uint32_t *>(mail_)};
+        if (smem > 40u * 1024u) {    // (always the same limit: another thread's call must not lower it before the launch)
+            const cudaError_t e = cudaFuncSetAttribute(tile_encode_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                       int(16u * kSmemEntries + kTileThreadsMax / 32u * (kAhead * 512u)));
+            if (e != cudaSuccess) return e;
+        }
+        const uint32_t ctas = (n_tiles + threads / 32u - 1u) / (threads / 32u) + P.report.ctas;
+        // Behind a counting pass not while that still runs: its CTAs leave an SM no registers for others, so the first SMs it leaves would get
+        // all coding CTAs of a small tensor (512 x 1024: 30 - 50 us instead of 20)
+        if (report) {
+            tile_encode_kernel<true><<<ctas, threads, smem, st_>>>(P);
+            return cudaGetLastError();
+        }
+        return in_smem ? launch_chained(tile_encode_kernel<true>, ctas, threads, smem, P) : launch_chained(tile_encode_kernel<false>, ctas, threads, smem, P);
+    }
+    // (few CTAs: more threads per tile.  Whole encode, us, 512 / 128 threads: 37 tiles 247.4 / 251.0, 289 346.1 / 348.3, 577 397.8 / 397.9,
+    // 1153 528.5 / 528.1, 2305 at 8 bpp 836.9 / 829.1, 4610 1320.7 / 1310.6)
+    cudaError_t launch_compact(uint32_t n_tiles) {
+        return launch_chained(compact_kernel, n_tiles, n_tiles < 600u ? 512u : 128u, 0, static_cast<const uint16_t *>(w_.scratch), 9u * V_,
+                              static_cast<const uint32_t *>(w_.counts), static_cast<const uint32_t *>(w_.index), static_cast<const SearchState *>(w_.state), w_.payload);
+    }
+    // Until the search's report is here (report_search).  The stream's own end is waited for if it takes very long: an error shows there, and a
+    // report that still is not here is fetched.
+    int await_report() {
+        const auto since = std::chrono::steady_clock::now();
+        for (uint32_t i = 1; !*reported(); ++i) {
+            if (i % 1024u == 0 && std::chrono::steady_clock::now() - since > std::chrono::milliseconds(50)) {
+                EP_CUDA(cudaStreamSynchronize(st_));
+                if (!*reported()) return fetch(true);
+                break;
+            }
+#if defined(__x86_64__)
+            __builtin_ia32_pause();
+#endif
+        }
+        std::atomic_thread_fence(std::memory_order_acquire);
+        return state()->overflow && !state()->undecided ? EP_ERR_UNSUPPORTED : EP_OK;     // a coordinate beyond +-4095: use the host encoder
+    }
 
     CountParams params(const uint32_t *rows, uint32_t n_rows, float s, uint4 *fields) {
         CountParams P{};
@@ -1365,6 +1606,11 @@ private:
         cfg.numAttrs = 1;
         return cudaLaunchKernelEx(&cfg, kernel, K(args)...);
     }
+    // launched while the kernel before it runs, whose results it does not use: the kernel does not wait until its end
+    template <class... K, class... A>
+    cudaError_t launch_beside(void (*kernel)(K...), uint32_t grid, uint32_t threads, size_t smem, A... args) {
+        return launch_chained(kernel, grid, threads, smem, args...);
+    }
     // one CTA per SM over all candidates of the pass, each with at least a few hundred blocks
     cudaError_t launch_count(CountParams P, bool follows) {
         const uint32_t cands = (1u << P.levels) - 1u;
@@ -1389,13 +1635,10 @@ private:
         return n;
     }
     // state and counts to the host: most alphabets fit the first copy
-    template <class Meanwhile>
-    int fetch(bool last, Meanwhile launch) {
+    int fetch(bool last) {
         EP_CUDA(cudaMemcpyAsync(mail_, w_.state, kStateBytes + (last ? 4ull * kFirstCounts : 0), cudaMemcpyDeviceToHost, st_));
         EP_CUDA(cudaMemcpyAsync(full_counts(), w_.full_counts, 4ull * kFirstCounts, cudaMemcpyDeviceToHost, st_));
-        EP_CUDA(cudaEventRecord(event_, st_));
-        EP_CUDA(launch());
-        EP_CUDA(cudaEventSynchronize(event_));
+        EP_CUDA(cudaStreamSynchronize(st_));
         const SearchState &S = *state();
         // (after a step it could not decide a search may have gone where the host's does not)
         if (S.overflow && !(last && S.undecided)) return EP_ERR_UNSUPPORTED;     // a coordinate beyond +-4095: use the host encoder
@@ -1413,7 +1656,7 @@ private:
     int count(const uint32_t *rows, uint32_t n_rows, float s, uint4 *fields, Model &m) {
         EP_CUDA(launch_count(params(rows, n_rows, s, fields), false));
         sigma_there_ = false;
-        const int rc = fetch(false, [] { return cudaSuccess; });
+        const int rc = fetch(false);
         if (rc) return rc;
         m.from_counts(state()->full.lo, state()->full.K, full_counts());
         return EP_OK;
@@ -1427,10 +1670,12 @@ private:
     uint8_t *mail_ = nullptr;        // page-locked: the copies back are plain DMA
     size_t mail_cap_ = 0;
     uint32_t n_sample_ = 0;
-    cudaEvent_t event_ = nullptr;
     bool under_way_ = false;         // the stream may still work for this call
     bool sigma_there_ = false;       // w_.sigma holds the row scales of the kept quantisation, which is at scale sigma_of_
     float sigma_of_ = 0.0f;
+    bool state_clear_ = false;       // the search's state is zero
+    bool coded_ = false;             // the tiles are coded (or being coded) from the counts of the last search, at precision
+    int coded_b_ = 0;
 };
 
 uint32_t tile_vectors_of(const ep_encode_opts &o, double target_bpp) {

@@ -162,3 +162,35 @@ def test_device_encoder_with_any_number_of_rate_corrections(maker, bpp, steps):
     host = ep.encode(W, bpp, polish_steps=steps)
     dev = ep.encode_device(torch.from_numpy(W).cuda(), bpp, polish_steps=steps)
     assert np.array_equal(dev.data, host.data) and dev.report == host.report
+
+
+@pytest.mark.parametrize("shape,V", [
+    ((128, 1024), 16),            # 1024 tiles: one turn of the last CTA's prefix sum
+    ((129, 1024), 16),            # and eight more
+    ((370, 1024), 16),            # 2960 tiles, the last number of four-warp CTAs
+    ((371, 1024), 16),            # eight warps per CTA
+    ((592, 1024), 16),            # 4736 tiles, their last number
+    ((593, 1024), 16),            # sixteen
+    ((64, 8), 1),                 # tiles of one block
+])
+def test_device_encoder_bytes_by_number_of_tiles(shape, V):
+    W = synth.gaussian_rows(*shape, 31)
+    host = ep.encode(W, 4.0, tile_vectors=V)
+    dev = ep.encode_device(torch.from_numpy(W).cuda(), 4.0, tile_vectors=V)
+    assert np.array_equal(dev.data, host.data) and dev.report == host.report
+
+
+def test_device_encoder_codes_again_where_the_host_moves_on():
+    # sampled rows with few distinct coordinates, the others Laplacian: the scale found on the sample gives the full tensor alphabets that
+    # do not fit, so the host goes to the next precision or, at the highest, to coarser scales of its own
+    R, C, budget = 128, 4096, 1 << 13
+    rows = oracle.sample_rows(R, C, budget)
+    W = synth.laplace_rows(R, C, 44)
+    W[rows] = np.random.Generator(np.random.PCG64(45)).uniform(-0.02, 0.02, (len(rows), C)).astype(np.float32)
+    Wd, moved = torch.from_numpy(W).cuda(), set()
+    for kw in (dict(b_max=9), dict(b_max=9, polish_steps=0), dict(b_max=12)):
+        host = ep.encode(W, 9.0, sample_vectors=budget, b_start=9, **kw)
+        dev = ep.encode_device(Wd, 9.0, sample_vectors=budget, b_start=9, **kw)
+        assert np.array_equal(dev.data, host.data) and dev.report == host.report
+        moved.add(host.report["b"])
+    assert len(moved) == 2
