@@ -331,20 +331,22 @@ struct Candidate {
     uint32_t from[EP_NUM_TABLES], to[EP_NUM_TABLES];
     uint32_t finished;               // its CTAs that are done
     uint32_t overflow;               // a coordinate left the histogram range
-    uint32_t verdict;                // kValid ...
 };
-// a b-bit table exists; the rate lies above the target; too close to say; ...; a table exists, but the counts were not kept
-constexpr uint32_t kValid = 1, kAbove = 2, kUndecided = 4, kOverflow = 8, kNoCounts = 16;
+// A candidate's verdict, four bits: a b-bit table exists; the rate lies above the target; too close to say (with kAbove, without kValid: a table
+// exists, but the counts were not kept); a coordinate left the histogram range.  A pass's verdicts come together in one 64-bit word: the
+// candidates' last CTAs add theirs and a one to its highest four bits, so that the one whose addition was the last has them all in hand.
+constexpr uint32_t kValid = 1, kAbove = 2, kUndecided = 4, kOverflow = 8, kNoCounts = kAbove | kUndecided;
+static_assert(kCandidates <= 15, "fifteen verdicts and their count in 64 bits");
 // what the passes leave for one another and for the host (device memory, zeroed before a search)
 struct SearchState {
     double lo, hi;                   // the bracket
     double last_log_s, last_rate;    // rate correction: the last point
+    unsigned long long verdicts;     // of the running pass's candidates
     float s;                         // the next pass's scale
     float s_counted;                 // the scale of the full counts
     uint32_t has_last;               // `last` holds the counts of the last step whose rate was evaluated
     uint32_t undecided;              // a decision within the rounding error, or too many symbols: the host repeats the search
     uint32_t overflow;               // a coordinate left the histogram range
-    uint32_t closed;                 // candidates of the running pass that are evaluated
     uint32_t stop;                   // the full passes are over
     uint32_t polished;               // ... because the rate correction ended (0: the tensor overflows the tables, the host decides)
     CountDir last, full;
@@ -589,59 +591,50 @@ __device__ __forceinline__ Evaluation gather_counts(const CountParams &P, uint32
     }
     return E;                                                // (cce and worst in warp 0)
 }
-// warp 0 after a candidate of the search is gathered: is its rate above the target?
-__device__ __forceinline__ void judge_candidate(const CountParams &P, uint32_t k, const Evaluation &E) {
+// warp 0 after a candidate of the search is gathered: is its rate above the target?  The verdict in lane 0
+__device__ __forceinline__ uint32_t judge_candidate(const CountParams &P, uint32_t k, const Evaluation &E) {
     // lane 1 at the estimate, lanes 0 and 2 at the ends of its interval
-    const uint32_t lane = threadIdx.x & 31u;
+    const uint32_t lane = threadIdx.x & 31u, overflow = __ldcg(&P.state->cand[k].overflow);
     const double cce = E.cce + (double(lane) - 1.0) * cce_bound(P.rate, E.cce);
     const bool above = __ddiv_rn(bits_at(P.rate, E.tables, cce), P.rate.weights) > P.rate.target;
     const uint32_t b = __ballot_sync(0xFFFFFFFFu, above) & 7u;
-    if (lane != 0) return;
     uint32_t v = kValid | ((b & 2u) ? kAbove : 0u) | ((b == 0u || b == 7u) ? 0u : kUndecided);
-    if (E.above) v = kAbove | (E.too_many ? kNoCounts : kValid);
+    if (E.above) v = E.too_many ? kNoCounts : kAbove | kValid;
     else if (E.too_many) v = kUndecided;
     if (E.worst > (1u << P.rate.b)) v = kAbove;                  // no b-bit table exists for this scale: too fine
-    P.state->cand[k].verdict = v;
+    return v | (overflow ? kOverflow : 0u);
 }
 
-// all threads of the pass's last CTA: the steps' outcomes in order
-__device__ void walk_tree(const CountParams &P) {
-    __shared__ int32_t chosen;
+// Thread 0 of the pass's last CTA: the steps' outcomes in order.  Returns the candidate whose counts the host gets, or -1
+__device__ __forceinline__ int32_t walk_tree(const CountParams &P, unsigned long long verdicts) {
     SearchState &S = *P.state;
-    if (threadIdx.x == 0) {
-        double lo = P.first ? P.lo0 : S.lo, hi = P.first ? P.hi0 : S.hi;
-        int32_t last = -1;
-        uint32_t k = 0, verdict[kCandidates];
-#pragma unroll
-        for (uint32_t i = 0; i < kCandidates; ++i) verdict[i] = __ldcg(&S.cand[i].verdict) | (__ldcg(&S.cand[i].overflow) ? kOverflow : 0u);
-#pragma unroll
-        for (uint32_t i = 0; i < kCandidates; ++i) S.cand[i].overflow = 0;
-        for (uint32_t l = 0; l < P.levels; ++l) {
-            uint32_t v = verdict[0];
-#pragma unroll
-            for (uint32_t i = 1; i < kCandidates; ++i) if (i == k) v = verdict[i];
-            if (v & kOverflow) S.overflow = 1;
-            if (v & kUndecided) S.undecided = 1;
-            if (v & kValid) last = int32_t(k);
-            if (v & kNoCounts) last = -2;
-            const double mid = __dsqrt_rn(__dmul_rn(lo, hi));
-            if (v & kAbove) { lo = mid; k = 2u * k + 1u; } else { hi = mid; k = 2u * k + 2u; }
-        }
-        S.lo = lo;
-        S.hi = hi;
-        S.s = __double2float_rn(__dsqrt_rn(__dmul_rn(lo, hi)));
-        S.closed = 0;
-        if (last != -1) S.has_last = 1;
-        if (P.last_pass && S.has_last && last < 0) S.undecided = 1;  // (its counts are gone)
-        chosen = P.last_pass ? last : -1;
+    double lo = P.first ? P.lo0 : __ldcg(&S.lo), hi = P.first ? P.hi0 : __ldcg(&S.hi);
+    int32_t last = -1;
+    uint32_t k = 0;
+    for (uint32_t l = 0; l < P.levels; ++l) {
+        const uint32_t v = uint32_t(verdicts >> (4u * k)) & 15u, kind = v & (kValid | kAbove | kUndecided);
+        if (v & kOverflow) S.overflow = 1;
+        if ((v & kUndecided) && kind != kNoCounts) S.undecided = 1;
+        if (v & kValid) last = int32_t(k);
+        if (kind == kNoCounts) last = -2;
+        const double mid = __dsqrt_rn(__dmul_rn(lo, hi));
+        if (v & kAbove) { lo = mid; k = 2u * k + 1u; } else { hi = mid; k = 2u * k + 2u; }
     }
-    __syncthreads();
-    if (chosen < 0) return;
-    // the host reports the rate of the last evaluated step: its counts
-    const Candidate &c = S.cand[chosen];
+    S.lo = lo;
+    S.hi = hi;
+    S.s = __double2float_rn(__dsqrt_rn(__dmul_rn(lo, hi)));
+    S.verdicts = 0;
+    if (last != -1) S.has_last = 1;
+    if (P.last_pass && __ldcg(&S.has_last) && last < 0) S.undecided = 1;  // (its counts are gone)
+    return P.last_pass ? last : -1;
+}
+// All threads: the host reports the rate of the last evaluated step - its counts
+__device__ __forceinline__ void keep_last(const CountParams &P, uint32_t k) {
+    SearchState &S = *P.state;
+    const Candidate &c = S.cand[k];
     uint32_t n = 0;
     for (int t = 0; t < EP_NUM_TABLES; ++t) n += __ldcg(&c.dir.K[t]);
-    for (uint32_t i = threadIdx.x; i < n; i += kCountThreads) P.last_counts[i] = __ldcg(P.cand_counts + size_t(chosen) * kEvalSymbols + i);
+    for (uint32_t i = threadIdx.x; i < n; i += kCountThreads) P.last_counts[i] = __ldcg(P.cand_counts + size_t(k) * kEvalSymbols + i);
     if (threadIdx.x < EP_NUM_TABLES) {
         S.last.lo[threadIdx.x] = __ldcg(&c.dir.lo[threadIdx.x]);
         S.last.K[threadIdx.x] = __ldcg(&c.dir.K[threadIdx.x]);
@@ -884,9 +877,22 @@ __global__ void __launch_bounds__(kCountThreads, 1) quantise_count_kernel(const 
     if (!arrive_last(&S.finished, P.ctas, last_cta)) return;
     const Evaluation E = gather_counts(P, k, P.mode == kPassSearch ? P.cand_counts + size_t(k) * kEvalSymbols : P.full_counts, sm, ranges);
     if (P.mode == kPassSearch) {
-        if (tid < 32u) judge_candidate(P, k, E);
-        if (!arrive_last(&P.state->closed, (1u << P.levels) - 1u, last_cta)) return;
-        walk_tree(P);
+        __shared__ int32_t chosen;
+        if (tid < 32u) {
+            const uint32_t v = judge_candidate(P, k, E);
+            if (lane == 0) {
+                S.overflow = 0;                                // (for the next pass)
+                if (P.last_pass) __threadfence();              // the counts, which another CTA may copy (stored before gather_counts' last barrier)
+                const unsigned long long mine = (static_cast<unsigned long long>(v) << (4u * k)) + (1ull << 60);
+                const unsigned long long before = atomicAdd(&P.state->verdicts, mine);
+                chosen = -1;
+                if ((before >> 60) == (1u << P.levels) - 2u) chosen = walk_tree(P, before + mine);
+                if (P.last_pass) __threadfence();
+            }
+        }
+        if (!P.last_pass) return;
+        __syncthreads();
+        if (chosen >= 0) keep_last(P, uint32_t(chosen));
         return;
     }
     if (tid < EP_NUM_TABLES) {
