@@ -276,12 +276,17 @@ __device__ __forceinline__ bool quantise_fast(const float (&x)[8], float r, uint
 // the rate correction after it are one stream of launches with one wait at the end: the last CTA of a pass evaluates
 // Eq. 10-12 on the counts and leaves the next scale in device memory.
 //
-// A step of the bisection costs about 12 us whatever the sample (launch, clearing and flushing counters, the evaluation's
-// chain of dependent reads), and counting 2^18 blocks of a sample only 4 us more.  So one launch takes several steps: for
-// three of them seven scales at once, the bracket's middle and the middles of the brackets that its two, then four,
-// outcomes lead to, each counted and evaluated by CTAs of its own; the last one to finish walks the tree.  (The first
-// launches take fewer steps: the outer candidates of a wide bracket are so fine - s = 0.003 - that all they count goes to
-// global memory, 120 us for 2^18 blocks.)  Steps per launch: 1, 2, 3, 3, 3; for samples up to 2^17 blocks 1, 3, 4, 4.
+// A pass costs about 12 us whatever the sample (launch, clearing and flushing counters, the evaluation's chain of dependent reads), and
+// counting 2^18 blocks of a sample only 4 us more.  So a pass counts and evaluates several scales at once, each by CTAs of its own, and the
+// last CTA to finish takes as many steps of the bisection as it has scales for.  Which scales a step looks at depends on the
+// steps before it, but where they lead can be foretold: after the first step by the one-bit-per-doubling law of Eq. 9, later by
+// interpolation between the ends of the bracket.  The scales of a pass are those that the bisection meets if the target is at the foretold
+// scale, or a little to either side of it; a step whose scale is not among them is left to the next pass.  No decision depends on
+// the forecast.  Where the passes that are left could not end the bisection one step at a time, a pass takes the whole tree of its next
+// four steps, fifteen scales; that many passes are launched that this always ends it, and those that find it ended cost 2 us each.
+// Twelve steps usually take three passes.  (Fixed trees: 1, 2, 3, 3, 3 steps per launch, for samples up to 2^17 blocks 1, 3, 4, 4.  The
+// first launches took fewer steps because the outer scales of a wide bracket are so fine - s = 0.003 - that all they count goes to
+// global memory, 120 us for 2^18 blocks; the forecast does not look at them.)
 //
 // Counting: nine increments per block, most of them of a few values around zero.  Each lane has its own column of
 // counters for those (bank = lane: no two lanes of a warp meet), values up to +-256 go to a plain window, the rest to
@@ -298,7 +303,7 @@ constexpr uint32_t kEvalSymbols = kHotWords + kWinWords;
 constexpr uint32_t kManySymbols = 8192;          // with more the counts' entropy is looked at first (see gather_counts)
 constexpr uint32_t kCountSmem = 4 * kEvalSymbols;
 constexpr uint32_t kFirstCounts = 6144;          // counts that come back with the state; more take a second copy
-constexpr uint32_t kLevels = 4, kCandidates = (1u << kLevels) - 1u;
+constexpr uint32_t kLevels = 4, kCandidates = (1u << kLevels) - 1u;   // a whole tree of steps
 
 // Symbols' entries by (coset, field, value): the two cosets' tables of a field have the same range here (the wider of
 // both ends), so that the second coset's entries follow at one distance.
@@ -339,7 +344,10 @@ constexpr uint32_t kValid = 1, kAbove = 2, kUndecided = 4, kOverflow = 8, kNoCou
 static_assert(kCandidates <= 15, "fifteen verdicts and their count in 64 bits");
 // what the passes leave for one another and for the host (device memory, zeroed before a search)
 struct SearchState {
-    double lo, hi;                   // the bracket
+    double lo, hi;                   // the bracket,
+    double rate_lo, rate_hi;         // the rates at its ends (NaN: not known)
+    double mid[kCandidates], rate[kCandidates];   // scales of the next or running pass, and their rates
+    uint32_t scales, left;           // how many scales (0: the bisection has ended), steps still to take
     double last_log_s, last_rate;    // rate correction: the last point
     unsigned long long verdicts;     // of the running pass's candidates
     float s;                         // the next pass's scale
@@ -378,9 +386,11 @@ struct CountParams {
     uint4 *entries;                  // rate correction: the tile coder's entries, made by the pass that ends it, and
     uint32_t *full_freq;             // the frequencies they are of (null: not wanted)
     uint32_t n_blocks, C, per_row;
-    uint32_t mode, levels, ctas;     // ctas: per candidate
-    uint32_t first;                  // first pass of the search: the bracket is {lo0, hi0}; of the rate correction: step 0
-    uint32_t last_pass;              // last pass of the search
+    uint32_t mode;
+    uint32_t first;                  // first pass of the search: one scale, the middle of the bracket {lo0, hi0}
+    uint32_t steps;                  // first pass of the search: steps to take
+    uint32_t most;                   // scales of the next pass, at most, and
+    uint32_t after;                  // passes of the search behind the next one
     float s;                         // mode kPassCount
     RateParams rate;
     double lo0, hi0;                 // the search bracket
@@ -591,42 +601,100 @@ __device__ __forceinline__ Evaluation gather_counts(const CountParams &P, uint32
     }
     return E;                                                // (cce and worst in warp 0)
 }
-// warp 0 after a candidate of the search is gathered: is its rate above the target?  The verdict in lane 0
-__device__ __forceinline__ uint32_t judge_candidate(const CountParams &P, uint32_t k, const Evaluation &E) {
+// warp 0 after a candidate of the search is gathered: is its rate above the target?  The verdict in lane 0, the rate in lane 1
+__device__ __forceinline__ uint32_t judge_candidate(const CountParams &P, uint32_t k, const Evaluation &E, double &rate) {
     // lane 1 at the estimate, lanes 0 and 2 at the ends of its interval
     const uint32_t lane = threadIdx.x & 31u, overflow = __ldcg(&P.state->cand[k].overflow);
     const double cce = E.cce + (double(lane) - 1.0) * cce_bound(P.rate, E.cce);
-    const bool above = __ddiv_rn(bits_at(P.rate, E.tables, cce), P.rate.weights) > P.rate.target;
-    const uint32_t b = __ballot_sync(0xFFFFFFFFu, above) & 7u;
+    rate = __ddiv_rn(bits_at(P.rate, E.tables, cce), P.rate.weights);
+    const uint32_t b = __ballot_sync(0xFFFFFFFFu, rate > P.rate.target) & 7u;
     uint32_t v = kValid | ((b & 2u) ? kAbove : 0u) | ((b == 0u || b == 7u) ? 0u : kUndecided);
     if (E.above) v = E.too_many ? kNoCounts : kAbove | kValid;
     else if (E.too_many) v = kUndecided;
     if (E.worst > (1u << P.rate.b)) v = kAbove;                  // no b-bit table exists for this scale: too fine
+    if (E.above || E.too_many || v == kAbove) rate = nan("");    // not known
     return v | (overflow ? kOverflow : 0u);
 }
 
-// Thread 0 of the pass's last CTA: the steps' outcomes in order.  Returns the candidate whose counts the host gets, or -1
-__device__ __forceinline__ int32_t walk_tree(const CountParams &P, unsigned long long verdicts) {
+// Warp 0 of a pass's last CTA: as many steps as there are scales for, in order, and the scales of the next pass.  Returns (in every lane) the
+// candidate whose counts the host gets, or -1.
+__device__ __noinline__ int32_t take_steps(const CountParams &P, unsigned long long verdicts) {
     SearchState &S = *P.state;
+    const uint32_t lane = threadIdx.x & 31u, n = P.first ? 1u : __ldcg(&S.scales);
+    const double nothing = nan("");
     double lo = P.first ? P.lo0 : __ldcg(&S.lo), hi = P.first ? P.hi0 : __ldcg(&S.hi);
+    double rate_lo = P.first ? nothing : __ldcg(&S.rate_lo), rate_hi = P.first ? nothing : __ldcg(&S.rate_hi);
+    uint32_t left = P.first ? P.steps : __ldcg(&S.left), undecided = 0, overflow = 0;
+    // lane k: scale, verdict and rate of candidate k
+    const double scale = lane >= n ? -1.0 : P.first ? __dsqrt_rn(__dmul_rn(lo, hi)) : __ldcg(&S.mid[min(lane, kCandidates - 1u)]);
+    const double rate = __ldcg(&S.rate[min(lane, kCandidates - 1u)]);
+    const uint32_t verdict = uint32_t(verdicts >> (4u * min(lane, kCandidates - 1u))) & 15u;
     int32_t last = -1;
-    uint32_t k = 0;
-    for (uint32_t l = 0; l < P.levels; ++l) {
-        const uint32_t v = uint32_t(verdicts >> (4u * k)) & 15u, kind = v & (kValid | kAbove | kUndecided);
-        if (v & kOverflow) S.overflow = 1;
-        if ((v & kUndecided) && kind != kNoCounts) S.undecided = 1;
+    while (left) {
+        const double mid = __dsqrt_rn(__dmul_rn(lo, hi));
+        const uint32_t at = __ballot_sync(0xFFFFFFFFu, scale == mid);
+        if (!at) break;
+        const uint32_t k = uint32_t(__ffs(int(at)) - 1), v = __shfl_sync(0xFFFFFFFFu, verdict, int(k)), kind = v & (kValid | kAbove | kUndecided);
+        const double r = __shfl_sync(0xFFFFFFFFu, rate, int(k));
+        overflow |= v & kOverflow;
+        undecided |= kind != kNoCounts && (v & kUndecided);
         if (v & kValid) last = int32_t(k);
         if (kind == kNoCounts) last = -2;
-        const double mid = __dsqrt_rn(__dmul_rn(lo, hi));
-        if (v & kAbove) { lo = mid; k = 2u * k + 1u; } else { hi = mid; k = 2u * k + 2u; }
+        if (v & kAbove) { lo = mid; rate_lo = r; } else { hi = mid; rate_hi = r; }
+        --left;
     }
-    S.lo = lo;
-    S.hi = hi;
-    S.s = __double2float_rn(__dsqrt_rn(__dmul_rn(lo, hi)));
-    S.verdicts = 0;
-    if (last != -1) S.has_last = 1;
-    if (P.last_pass && __ldcg(&S.has_last) && last < 0) S.undecided = 1;  // (its counts are gone)
-    return P.last_pass ? last : -1;
+    if (lane == 0) {
+        S.lo = lo;
+        S.hi = hi;
+        S.rate_lo = rate_lo;
+        S.rate_hi = rate_hi;
+        S.left = left;
+        S.s = __double2float_rn(__dsqrt_rn(__dmul_rn(lo, hi)));
+        S.verdicts = 0;
+        if (overflow) S.overflow = 1;
+        if (undecided) S.undecided = 1;
+        if (last != -1) S.has_last = 1;
+        if (!left && last < 0 && __ldcg(&S.has_last)) S.undecided = 1;       // (the last step's counts are gone)
+    }
+    if (!left) {
+        if (lane == 0) S.scales = 0;
+        return last;
+    }
+    // the next pass's scales.  The forecast is in fp32 (in double it took 7 us); the scales themselves are the bisection's, to the bit
+    uint32_t next = 0;
+    const float x_lo = log2f(float(lo)), x_hi = log2f(float(hi)), width = x_hi - x_lo, target = float(P.rate.target), r_lo = float(rate_lo), r_hi = float(rate_hi);
+    const bool both = r_lo > r_hi;
+    // (the rate bends by a few hundredths of a bit per doubling of the scale and doubling)
+    const float off = both ? fmaxf(0.004f, 0.04f * width * width) : 0.12f;
+    const float x = both ? x_lo + width * __fdividef(r_lo - target, r_lo - r_hi) : r_lo == r_lo ? x_lo + (r_lo - target) : x_hi - (target - r_hi);
+    if (x == x && left - 1u <= kLevels * P.after) {
+        // lanes 0, 1, 2 follow the bisection to the foretold scale and to either side of it
+        __shared__ double path[30];
+        const float to = exp2f(x + (lane == 1u ? off : lane == 2u ? -off : 0.0f));
+        double a = lo, b = hi;
+        float w = width;
+        uint32_t levels = 0;
+        for (; levels < min(left, 10u) && w > 0.5f * off; ++levels, w *= 0.5f) {
+            const double mid = __dsqrt_rn(__dmul_rn(a, b));
+            if (lane < 3u) path[3u * levels + lane] = mid;
+            if (float(mid) < to) a = mid; else b = mid;
+        }
+        __syncwarp();
+        // step by step, the two others where they differ from the first
+        const double mine = lane < 3u * levels ? path[lane] : 0.0, first = lane < 3u * levels ? path[lane - lane % 3u] : 0.0;
+        const bool want = lane < 3u * levels && (lane % 3u == 0u || mine != first);
+        const uint32_t wanted = __ballot_sync(0xFFFFFFFFu, want), at = __popc(wanted & ((1u << lane) - 1u));
+        if (want && at < P.most) S.mid[at] = mine;
+        next = min(uint32_t(__popc(wanted)), P.most);
+    }
+    if (!next) {
+        next = (1u << min(left, kLevels)) - 1u;
+        double a = lo, b = hi;
+        bracket_of(min(lane, kCandidates - 1u), a, b);
+        if (lane < next) S.mid[lane] = __dsqrt_rn(__dmul_rn(a, b));
+    }
+    if (lane == 0) S.scales = next;
+    return -1;
 }
 // All threads: the host reports the rate of the last evaluated step - its counts
 __device__ __forceinline__ void keep_last(const CountParams &P, uint32_t k) {
@@ -744,13 +812,11 @@ __global__ void __launch_bounds__(kCountThreads, 1) quantise_count_kernel(const 
     __shared__ float s_shared;
     __shared__ Ranges ranges;
     const uint32_t tid = threadIdx.x, lane = tid & 31u;
-    const uint32_t k = blockIdx.x / P.ctas, part = blockIdx.x - k * P.ctas;      // candidate, and this CTA's share of the blocks
-    Candidate &S = P.state->cand[k];
     // Launched before the previous pass has ended (see launch_count): only W, mu and rows, which are older than that, are
-    // read before the wait, and only then may the next launch come up.
-    const uint32_t v0 = uint32_t(uint64_t(P.n_blocks) * part / P.ctas), v1 = uint32_t(uint64_t(P.n_blocks) * (part + 1u) / P.ctas);
-    uint32_t v = v0 + tid;                                                       // (n_blocks < 2^31: see the launcher)
-    uint32_t i = v / P.per_row, col = v - i * P.per_row;                         // rows of later blocks follow without divisions
+    // read before the wait, and only then may the next launch come up.  A pass with several scales learns behind the wait how many they are.
+    const bool listed = P.mode == kPassSearch && !P.first;
+    uint32_t k = 0, ctas = gridDim.x, part = blockIdx.x;                         // candidate, its CTAs and this one's share of the blocks
+    uint32_t v = 0, v1 = 0, i = 0, col = 0;
     const uint32_t row_step = kCountThreads / P.per_row, col_step = kCountThreads % P.per_row;
     float4 lo4 = make_float4(0.f, 0.f, 0.f, 0.f), hi4 = lo4;
     float mu = 1.0f;
@@ -761,20 +827,33 @@ __global__ void __launch_bounds__(kCountThreads, 1) quantise_count_kernel(const 
         hi4 = __ldg(src + 1);
         mu = __ldg(P.mu + r);
     };
-    if (v < v1) load();
+    auto begin = [&]() {
+        v = uint32_t(uint64_t(P.n_blocks) * part / ctas) + tid;                  // (n_blocks < 2^31: see the launcher)
+        v1 = uint32_t(uint64_t(P.n_blocks) * (part + 1u) / ctas);
+        i = v / P.per_row;
+        col = v - i * P.per_row;                                                 // rows of later blocks follow without divisions
+        if (v < v1) load();
+    };
+    if (!listed) begin();
     for (uint32_t j = tid; j < (kHotWords + kWinWords) / 4u; j += kCountThreads) reinterpret_cast<uint4 *>(sm)[j] = make_uint4(0u, 0u, 0u, 0u);
     if (tid < EP_NUM_TABLES) { range_from[tid] = 0; range_to[tid] = 0; }
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (P.mode == kPassPolish && __ldcg(&P.state->stop)) return;                 // (the same for all CTAs: set by an earlier launch)
+    const uint32_t scales = listed ? __ldcg(&P.state->scales) : 1u;
+    if (!scales) return;
+    if (listed) {
+        ctas = min(gridDim.x / scales, max((P.n_blocks + 255u) / 256u, 1u));
+        k = blockIdx.x / ctas;
+        part = blockIdx.x - k * ctas;
+        if (k >= scales) return;
+        begin();
+    }
+    Candidate &S = P.state->cand[k];
     if (tid == 0) {
-        if (P.mode == kPassSearch) {
-            double lo = P.first ? P.lo0 : __ldcg(&P.state->lo), hi = P.first ? P.hi0 : __ldcg(&P.state->hi);
-            bracket_of(k, lo, hi);
-            s_shared = __double2float_rn(__dsqrt_rn(__dmul_rn(lo, hi)));
-        } else {
-            s_shared = P.mode == kPassPolish ? __ldcg(&P.state->s) : P.s;
-        }
+        if (listed) s_shared = __double2float_rn(__ldcg(&P.state->mid[k]));
+        else if (P.mode == kPassSearch) s_shared = __double2float_rn(__dsqrt_rn(__dmul_rn(P.lo0, P.hi0)));
+        else s_shared = P.mode == kPassPolish ? __ldcg(&P.state->s) : P.s;
     }
     __syncthreads();
     const float s = s_shared;
@@ -874,23 +953,27 @@ __global__ void __launch_bounds__(kCountThreads, 1) quantise_count_kernel(const 
         atomicMax(&S.from[tid], range_from[tid]);
         atomicMax(&S.to[tid], range_to[tid]);
     }
-    if (!arrive_last(&S.finished, P.ctas, last_cta)) return;
+    if (!arrive_last(&S.finished, ctas, last_cta)) return;
     const Evaluation E = gather_counts(P, k, P.mode == kPassSearch ? P.cand_counts + size_t(k) * kEvalSymbols : P.full_counts, sm, ranges);
     if (P.mode == kPassSearch) {
         __shared__ int32_t chosen;
         if (tid < 32u) {
-            const uint32_t v = judge_candidate(P, k, E);
+            double rate;
+            const uint32_t verdict = judge_candidate(P, k, E, rate);
+            unsigned long long mine = 0, before = 0;
+            if (lane == 1u) P.state->rate[k] = rate;
+            __syncwarp();
             if (lane == 0) {
                 S.overflow = 0;                                // (for the next pass)
-                if (P.last_pass) __threadfence();              // the counts, which another CTA may copy (stored before gather_counts' last barrier)
-                const unsigned long long mine = (static_cast<unsigned long long>(v) << (4u * k)) + (1ull << 60);
-                const unsigned long long before = atomicAdd(&P.state->verdicts, mine);
-                chosen = -1;
-                if ((before >> 60) == (1u << P.levels) - 2u) chosen = walk_tree(P, before + mine);
-                if (P.last_pass) __threadfence();
+                __threadfence();                               // the rate, and the counts, stored before gather_counts' last barrier
+                mine = (static_cast<unsigned long long>(verdict) << (4u * k)) + (1ull << 60);
+                before = atomicAdd(&P.state->verdicts, mine);
+                __threadfence();
             }
+            before = __shfl_sync(0xFFFFFFFFu, before + mine, 0);
+            const int32_t last = (before >> 60) == scales ? take_steps(P, before) : -1;
+            if (lane == 0) chosen = last;
         }
-        if (!P.last_pass) return;
         __syncthreads();
         if (chosen >= 0) keep_last(P, uint32_t(chosen));
         return;
@@ -1367,14 +1450,15 @@ public:
         P.hi0 = o.bracket_hi;
         const float s0 = float(std::sqrt(o.bracket_lo * o.bracket_hi));
         if (o.search_steps == 0) EP_CUDA(cudaMemcpyAsync(&w_.state->s, &s0, 4, cudaMemcpyHostToDevice, st_));
-        P.first = 1;
-        for (int left = o.search_steps, pass = 0; left > 0; ++pass) {
-            P.levels = uint32_t(std::min(left, n_sample_ * (C_ / 8) <= (1u << 17) ? (pass == 0 ? 1 : std::min<int>(pass + 2, kLevels))
-                                                                                  : std::min<int>(pass + 1, 3)));
-            P.last_pass = left == int(P.levels);
+        // the first step, then passes of several scales: as many as the steps take four at a time, and one that the forecast may lose.
+        // Up to 2^17 blocks fifteen scales cost little more than nine, beyond it they do
+        P.steps = uint32_t(o.search_steps);
+        P.most = P.n_blocks <= (1u << 17) ? kCandidates : 9u;
+        const uint32_t passes = o.search_steps < 2 ? uint32_t(o.search_steps) : 2u + (P.steps - 1u + kLevels - 1u) / kLevels;
+        for (uint32_t pass = 0; pass < passes; ++pass) {
+            P.first = pass == 0;
+            P.after = passes - std::min(passes, pass + 2u);
             EP_CUDA(launch_count(P, pass > 0));
-            left -= int(P.levels);
-            P.first = 0;
         }
         CountParams F = params(nullptr, R_, 0.0f, w_.fields);
         F.mode = kPassPolish;
@@ -1588,7 +1672,6 @@ private:
         P.n_blocks = n_rows * P.per_row;
         P.C = C_;
         P.mode = kPassCount;
-        P.levels = 1;
         P.s = s;
         return P;
     }
@@ -1617,17 +1700,17 @@ private:
     cudaError_t launch_beside(void (*kernel)(K...), uint32_t grid, uint32_t threads, size_t smem, A... args) {
         return launch_chained(kernel, grid, threads, smem, args...);
     }
-    // one CTA per SM over all candidates of the pass, each with at least a few hundred blocks
+    // one CTA per SM, each with at least a few hundred blocks
     cudaError_t launch_count(CountParams P, bool follows) {
-        const uint32_t cands = (1u << P.levels) - 1u;
-        P.ctas = std::max(1u, std::min((P.n_blocks + 255u) / 256u, uint32_t(sms_) / cands));
+        const bool listed = P.mode == kPassSearch && !P.first;
+        const uint32_t ctas = listed ? uint32_t(sms_) : std::max(1u, std::min((P.n_blocks + 255u) / 256u, uint32_t(sms_)));
         // A pass's last CTA works on alone for 8 us; with programmatic launch the next pass's CTAs come up meanwhile, load
         // their first blocks and clear their counters.  Not the first pass: it reads what the kernel before it writes.
         cudaLaunchAttribute attr{};
         attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
         attr.val.programmaticStreamSerializationAllowed = 1;
         cudaLaunchConfig_t cfg{};
-        cfg.gridDim = dim3(cands * P.ctas);
+        cfg.gridDim = dim3(ctas);
         cfg.blockDim = dim3(kCountThreads);
         cfg.dynamicSmemBytes = kCountSmem;
         cfg.stream = st_;
