@@ -523,19 +523,25 @@ struct TileSetup {
     uint64_t a0;           // global address of chunk 0
     uint32_t lead, room;   // cursor position inside chunk 0; payload bytes from a0 on
 };
-__device__ __forceinline__ TileSetup tile_setup(const JobParams &J, uint32_t tile, bool valid, uint32_t lane) {
+// from a record's words: this lane's state, the tile's and the next one's first payload word (the blocks are left to the caller)
+__device__ __forceinline__ TileSetup tile_setup(const JobParams &J, uint32_t state, uint32_t off, uint32_t end) {
     TileSetup T;
-    const uint32_t *rec = J.tile_index + size_t(tile) * 33u;
-    T.x = max(rec[lane] & 0x7FFFFFFFu, ep::kStateLow);
-    T.off = min(rec[32], J.total_words);    // a damaged index must not move reads outside the payload
-    T.end = (tile + 1 < J.n_tiles) ? rec[33 + 32] : rec[33];
-    T.v0 = tile * J.V;
-    T.nv = valid ? min(J.V, J.n_vec - T.v0) : 0u;
+    T.x = max(state & 0x7FFFFFFFu, ep::kStateLow);
+    T.off = min(off, J.total_words);        // a damaged index must not move reads outside the payload
+    T.end = end;
+    T.v0 = T.nv = 0;
     const uint64_t pay = reinterpret_cast<uint64_t>(J.stream + J.off_payload);
     const uint64_t first = pay + 2ull * T.off;
     T.a0 = first & ~15ull;
     T.lead = uint32_t(first - T.a0);
     T.room = uint32_t(pay + 2ull * J.total_words - T.a0);     // the payload is shorter than 2 GB
+    return T;
+}
+__device__ __forceinline__ TileSetup tile_setup(const JobParams &J, uint32_t tile, bool valid, uint32_t lane) {
+    const uint32_t *rec = J.tile_index + size_t(tile) * 33u;
+    TileSetup T = tile_setup(J, rec[lane], rec[32], (tile + 1 < J.n_tiles) ? rec[33 + 32] : rec[33]);
+    T.v0 = tile * J.V;
+    T.nv = valid ? min(J.V, J.n_vec - T.v0) : 0u;
     return T;
 }
 
@@ -1443,10 +1449,10 @@ __device__ __forceinline__ void umma_commit(uint32_t bar) {
 #define EP_KK "%8"
 #define EP_F0 "%9"
 #define EP_F1 "%10"
-#define EP_GEMM_ROW_ASM(BODY, FIN)                                                                                            \
+#define EP_GEMM_ROW_ASM(BODY)                                                                                                 \
     asm volatile("{\n\t" EP_REGS                                                                                      \
         ".reg .pred pq, pv, pr, pl;\n\t"                                                                              \
-        ".reg .b32 r0, r1, r2, r3, r4, r5, r6, r10, r11, r12, c0r, c1r, va, g, bar, par, odd, dst, tries;\n\t"   \
+        ".reg .b32 r0, r1, r2, r3, r4, r5, r6, r10, r11, r12, c0r, c1r, g, bar, par, odd, dst, tries;\n\t"   \
         ".reg .b64 ra, rb, st;\n\t"                                                                                   \
         "mov.b32 c0r, 0x45800000;\n\t" "mov.b32 c1r, 0x45800400;\n\t"                \
         "mov.b64 ssA, {%11, %11};\n\t" "setp.ne.u32 actA, %12, 0;\n\t" "mov.b32 g, %13;\n\t"                          \
@@ -1479,7 +1485,6 @@ __device__ __forceinline__ void umma_commit(uint32_t bar) {
         "add.u32 %3, %3, 1;\n\t" "sub.u32 g, g, 1;\n\t"                                                               \
         "setp.lt.u32 pq, %1, wthrA;\n\t" "setp.ne.and.u32 pq, g, 0, pq;\n\t"                                          \
         "vote.sync.all.pred pq, pq, 0xffffffff;\n\t"                                                                  \
-        FIN                                                                                                           \
         "@pq bra.uni EP_LOOP;\n\t"                                                                                    \
         "setp.eq.u32 pr, g, 0;\n\t"                                                                                   \
         "vote.sync.any.pred pr, pr, 0xffffffff;\n\t"                                                                  \
@@ -1667,19 +1672,24 @@ __global__ void __launch_bounds__(kThreads, 1) ep_decode_gemm_kernel(const __gri
         const uint64_t kk = pack64(k0, k0);
         // where this lane's block of a group goes in a slab: 64-column tile lane / 8, row = w, piece lane % 8 of the row
         const uint32_t b_dst = b_base + (lane >> 3) * G::kBTile + w * 128u + (((lane & 7u) ^ (w & 7u)) << 4);
+        // A row's record and scale are read a step ahead, so that a step begins with one read - its payload's - and not with two in a row
+        // (10240 x 3840 at 4 bpp, 16 tokens, three steps of 15 groups: 51.1 -> 50.3 us; 24 rows of
+        // 2048 columns at 3 bpp 12.3 -> 11.95).
+        struct { uint32_t x, off, end, sigma; } next;
+        auto ask = [&](uint32_t r) {
+            const uint32_t tile = min(r, P.R - 1u);                     // = the row of W
+            const uint32_t *rec = J.tile_index + size_t(tile) * 33u;
+            next = {__ldg(rec + lane), __ldg(rec + 32), __ldg(rec + (tile + 1u < J.n_tiles ? 65u : 33u)), __float_as_uint(__ldg(J.scales + tile))};
+        };
+        ask(row_begin + w);
         uint32_t q = 0;
         for (uint32_t s = 0; s < P.steps; ++s) {
             const uint32_t r = row_begin + s * P.rows_per_step + w, act = r < row_end ? 1u : 0u;   // a CTA's last step may be short
-            const uint32_t tile = min(r, P.R - 1u);                     // = the row of W
-            const TileSetup Tl = tile_setup(J, tile, true, lane);
+            const TileSetup Tl = tile_setup(J, next.x, next.off, next.end);
+            const uint32_t sigma = next.sigma;
             for (uint32_t c = 0; c < G::kSlots; ++c) ring_issue<G::kChunk, G::kSlots>(ring, Tl.a0, Tl.room, c, lane);
-            const uint32_t sigma = __float_as_uint(__ldg(J.scales + tile));
-            // the row this warp takes in the next step: its record is asked for now and, when that is here, the start of
-            // its payload is brought into L2, so that the next step does not begin with two reads from DRAM in a row
             const bool has_next = r + P.rows_per_step < row_end;
-            const uint32_t *rec_next = J.tile_index + size_t(min(r + P.rows_per_step, P.R - 1u)) * 33u;
-            const uint32_t off_next = __ldg(rec_next + 32);
-            if (has_next && lane == 0) prefetch_l2(rec_next);
+            ask(r + P.rows_per_step);
             if (lane == 0) {                 // the next request is chunk kSlots, into slot 0
                 sts64(ctx + kCtxChain + kCcSrc, Tl.a0 + G::kRing);
                 sts32(ctx + kCtxChain + kCcRem, Tl.room - G::kRing);
@@ -1689,21 +1699,17 @@ __global__ void __launch_bounds__(kThreads, 1) ep_decode_gemm_kernel(const __gri
             }
             cp_async_wait<1>();
             __syncwarp();
-            if (has_next) {                  // 4 KB: the ring's first fill and more
-                const uint64_t at = 2ull * min(off_next, J.total_words) + 128u * lane;
+            if (has_next) {                  // the start of the next row's payload, into L2: 4 KB, the ring's first fill and more
+                const uint64_t at = 2ull * min(next.off, J.total_words) + 128u * lane;
                 if (at < 2ull * J.total_words) prefetch_l2(J.stream + J.off_payload + at);
             }
             uint32_t x = Tl.x, bal = 0, a = ring + Tl.lead;
             if (s == 0) wait_for_tables(tables);
-            // The short chain saves latency, the plain one instructions.  4096 columns at 4 bpp, us, short / plain:
-            //   16 tokens, 24 rows per step at most: 4 rows per SM 15.40 / 15.61, 12: 17.18 / 17.20, 24: 21.00 / 20.83, 70: 54.04 / 53.59;
-            //   up to 30: 28 rows 23.16 / 23.50, 60: 43.13 / 43.82 (10240 x 3840 51.9 / 51.5, 8192 x 8192 79.1 / 80.3);
-            //   32 tokens: 1 row 17.93 / 17.96, 4: 18.60 / 18.48, 16: 21.59 / 21.32, 24: 24.96 / 24.30, 28: 25.99 / 25.29, 70: 65.29 / 63.08
-            //   (256 columns 1 - 8 rows: 4.56 / 4.61).
-            // Up to 16 tokens either is ahead by 1 % or so, by shape and rows; beyond, waiting for x hides the chain.  Both in one kernel,
-            // chosen by the number of groups, took every product of 17 to 32 tokens 0.5 - 1 % longer.
-            if constexpr (TPAD == 16u) EP_GEMM_ROW_ASM(EP_BODY11_SHORT, EP_SHORT_FIN);
-            else EP_GEMM_ROW_ASM(EP_BODY11, "");
+            // The loop with fewer instructions (EP_BODY11); with the shorter chain of EP_BODY11_SHORT, one instruction more per step, us:
+            //   16 tokens: 10240 x 3840 50.34 (this one 50.25), 4096 x 4096 22.80 (22.48), 8192 x 8192 79.7 (78.4), 60 rows per SM of 2560 columns
+            //   29.14 (28.75), 4 rows of 4096 14.91 (15.02), 31 rows at 5 bpp 31.62 (31.81);
+            //   32 tokens: 24 rows per SM of 4096 columns 24.96 (24.30), 70 rows 65.29 (63.08).
+            EP_GEMM_ROW_ASM(EP_BODY11);
             cp_async_wait<0>();              // nothing may still be landing in the ring when the next row starts
             __syncwarp();
             const uint32_t pos = __shfl_sync(0xFFFFFFFFu, a, 0) + 2u * __popc(bal) - lds32(ctx + kCtxChain + kCcWbase);
