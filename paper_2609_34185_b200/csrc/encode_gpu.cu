@@ -1426,7 +1426,9 @@ public:
         EP_CUDA(cudaGetDevice(&dev));
         EP_CUDA(cudaDeviceGetAttribute(&sms_, cudaDevAttrMultiProcessorCount, dev));
         EP_CUDA(cudaFuncSetAttribute(quantise_count_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kCountSmem)));
-        EP_CUDA(cudaMemcpyAsync(w_.rows, sample.data(), 4ull * n_sample_, cudaMemcpyHostToDevice, st_));
+        // (a sample of all rows, as smaller tensors have it, needs no list)
+        sample_rows_ = n_sample_ < R_ ? w_.rows : nullptr;
+        if (sample_rows_) EP_CUDA(cudaMemcpyAsync(w_.rows, sample.data(), 4ull * n_sample_, cudaMemcpyHostToDevice, st_));
         // the state, and the histograms behind it (every pass leaves them zero again)
         const size_t clear = size_t(reinterpret_cast<uint8_t *>(w_.hist) - reinterpret_cast<uint8_t *>(w_.state)) + kCandidates * kHistBytes;
         row_rms_kernel<<<R_ + kClearCtas, kRowThreads, 0, st_>>>(W_, C_, w_.mu, reinterpret_cast<uint4 *>(w_.state), uint32_t(clear / 16u));
@@ -1434,7 +1436,7 @@ public:
         state_clear_ = true;
         return EP_OK;
     }
-    int count_sample(float s, Model &m) override { return count(w_.rows, n_sample_, s, nullptr, m); }
+    int count_sample(float s, Model &m) override { return count(sample_rows_, n_sample_, s, nullptr, m); }
     int count_full(float s, Model &m) override { return count(nullptr, R_, s, w_.fields, m); }
 
     int search(const SearchJob &job, const ep_encode_opts &o, SearchResult &r, bool *done) override {
@@ -1443,7 +1445,7 @@ public:
         state_clear_ = false;
         // with the refinement of rows (which this back end leaves to the host) the last pass's tables are not the final ones
         const bool ahead = o.rdo_candidates <= 1;
-        CountParams P = params(w_.rows, n_sample_, 0.0f, nullptr);
+        CountParams P = params(sample_rows_, n_sample_, 0.0f, nullptr);
         P.mode = kPassSearch;
         P.rate = rate_params(job.target_bpp, o.retained_bits, job.sample_vectors, job.sample_rows, job.V, job.b);
         P.lo0 = o.bracket_lo;
@@ -1759,6 +1761,7 @@ private:
     uint8_t *mail_ = nullptr;        // page-locked: the copies back are plain DMA
     size_t mail_cap_ = 0;
     uint32_t n_sample_ = 0;
+    const uint32_t *sample_rows_ = nullptr;      // null: all rows
     bool under_way_ = false;         // the stream may still work for this call
     bool sigma_there_ = false;       // w_.sigma holds the row scales of the kept quantisation, which is at scale sigma_of_
     float sigma_of_ = 0.0f;

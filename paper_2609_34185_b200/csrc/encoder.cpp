@@ -192,6 +192,7 @@ std::vector<uint32_t> sample_rows(uint32_t R, uint32_t C, uint32_t budget_vector
     n = std::min(n, R);
     std::vector<uint32_t> idx(R);
     for (uint32_t i = 0; i < R; ++i) idx[i] = i;
+    if (n == R) return idx;                      // all rows, in whatever order they are drawn
     uint64_t st = (uint64_t(R) << 32) + uint64_t(C);
     for (uint32_t i = 0; i < n; ++i) {
         const uint32_t j = i + uint32_t(splitmix64(st) % uint64_t(R - i));
