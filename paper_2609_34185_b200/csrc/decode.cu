@@ -267,18 +267,20 @@ __device__ __forceinline__ void build_tables_smem(const JobParams &J, uint32_t l
 // the prepared image of the same sixteen tables, 128 KB: one thread asks for it, the copy engine brings it in.  (256 threads
 // with 16 bytes per cp.async kept the load pipe busy for a microsecond, and the first tile's payload queued behind
 // it: 3.6 us from a launch's turn to its first group.)  Whoever reads the tables waits for the mbarrier first.
+// One copy: asking for four of 32 KB took the asking warp 0.8 us, by which its own tile then began later (8192 x 8192 at 4 bpp 59.25 -> 59.0 us,
+// block of seven at 2.5 bpp to FP8 302.9 -> 300.4, at 3.5 to BF16 310.5 -> 309.5).  Asked for by another warp - one more than tiles, or the
+// last - the same, and 1 % slower where few tiles decode without the guess.
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
 }
 __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 __device__ __forceinline__ void copy_tables_smem(const uint32_t *image, uint32_t lut_addr, uint32_t bar, bool two_level) {
-    constexpr uint32_t kPiece = 32768;
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(kLutBytes + (two_level ? kHotBytes : 0u)) : "memory");
     auto piece = [&](uint32_t dst, uint32_t src, uint32_t bytes) {
         asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                      ::"r"(dst), "l"(reinterpret_cast<uint64_t>(image) + src), "r"(bytes), "r"(bar) : "memory");
     };
-    for (uint32_t o = 0; o < kLutBytes; o += kPiece) piece(lut_addr + o, o, kPiece);
+    piece(lut_addr, 0u, kLutBytes);
     if (two_level) piece(lut_addr + kHotBase, kLutBytes, kHotBytes);      // the hot part of the second level follows the image
 }
 
