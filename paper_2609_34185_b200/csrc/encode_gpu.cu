@@ -341,13 +341,13 @@ struct Candidate {
 // exists, but the counts were not kept); a coordinate left the histogram range.  A pass's verdicts come together in one 64-bit word: the
 // candidates' last CTAs add theirs and a one to its highest four bits, so that the one whose addition was the last has them all in hand.
 constexpr uint32_t kValid = 1, kAbove = 2, kUndecided = 4, kOverflow = 8, kNoCounts = kAbove | kUndecided;
-static_assert(kCandidates <= 15, "fifteen verdicts and their count in 64 bits");
+static_assert(kCandidates == kMostScales, "fifteen verdicts and their count in 64 bits");
 // what the passes leave for one another and for the host (device memory, zeroed before a search)
 struct SearchState {
     double lo, hi;                   // the bracket,
     double rate_lo, rate_hi;         // the rates at its ends (NaN: not known)
     double mid[kCandidates], rate[kCandidates];   // scales of the next or running pass, and their rates
-    uint32_t scales, left;           // how many scales (0: the bisection has ended), steps still to take
+    uint32_t scales, left;           // how many scales, with the pass that counts them (scales_word; 0: the bisection has ended), steps still to take
     double last_log_s, last_rate;    // rate correction: the last point
     unsigned long long verdicts;     // of the running pass's candidates
     float s;                         // the next pass's scale
@@ -387,7 +387,7 @@ struct CountParams {
     uint32_t *full_freq;             // the frequencies they are of (null: not wanted)
     uint32_t n_blocks, C, per_row;
     uint32_t mode;
-    uint32_t first;                  // first pass of the search: one scale, the middle of the bracket {lo0, hi0}
+    uint32_t pass;                   // of the search; the first, 0, counts one scale, the middle of the bracket {lo0, hi0}
     uint32_t steps;                  // first pass of the search: steps to take
     uint32_t most;                   // scales of the next pass, at most, and
     uint32_t after;                  // passes of the search behind the next one
@@ -616,17 +616,18 @@ __device__ __forceinline__ uint32_t judge_candidate(const CountParams &P, uint32
     return v | (overflow ? kOverflow : 0u);
 }
 
-// Warp 0 of a pass's last CTA: as many steps as there are scales for, in order, and the scales of the next pass.  Returns (in every lane) the
+// Warp 0 of a pass's last CTA: as many steps as the pass's n scales are for, in order, and the scales of the next pass.  Returns (in every lane) the
 // candidate whose counts the host gets, or -1.
-__device__ __noinline__ int32_t take_steps(const CountParams &P, unsigned long long verdicts) {
+__device__ __noinline__ int32_t take_steps(const CountParams &P, uint32_t n, unsigned long long verdicts) {
     SearchState &S = *P.state;
-    const uint32_t lane = threadIdx.x & 31u, n = P.first ? 1u : __ldcg(&S.scales);
+    const bool first_pass = P.pass == 0u;
+    const uint32_t lane = threadIdx.x & 31u;
     const double nothing = nan("");
-    double lo = P.first ? P.lo0 : __ldcg(&S.lo), hi = P.first ? P.hi0 : __ldcg(&S.hi);
-    double rate_lo = P.first ? nothing : __ldcg(&S.rate_lo), rate_hi = P.first ? nothing : __ldcg(&S.rate_hi);
-    uint32_t left = P.first ? P.steps : __ldcg(&S.left), undecided = 0, overflow = 0;
+    double lo = first_pass ? P.lo0 : __ldcg(&S.lo), hi = first_pass ? P.hi0 : __ldcg(&S.hi);
+    double rate_lo = first_pass ? nothing : __ldcg(&S.rate_lo), rate_hi = first_pass ? nothing : __ldcg(&S.rate_hi);
+    uint32_t left = first_pass ? P.steps : __ldcg(&S.left), undecided = 0, overflow = 0;
     // lane k: scale, verdict and rate of candidate k
-    const double scale = lane >= n ? -1.0 : P.first ? __dsqrt_rn(__dmul_rn(lo, hi)) : __ldcg(&S.mid[min(lane, kCandidates - 1u)]);
+    const double scale = lane >= n ? -1.0 : first_pass ? __dsqrt_rn(__dmul_rn(lo, hi)) : __ldcg(&S.mid[min(lane, kCandidates - 1u)]);
     const double rate = __ldcg(&S.rate[min(lane, kCandidates - 1u)]);
     const uint32_t verdict = uint32_t(verdicts >> (4u * min(lane, kCandidates - 1u))) & 15u;
     int32_t last = -1;
@@ -657,7 +658,7 @@ __device__ __noinline__ int32_t take_steps(const CountParams &P, unsigned long l
         if (!left && last < 0 && __ldcg(&S.has_last)) S.undecided = 1;       // (the last step's counts are gone)
     }
     if (!left) {
-        if (lane == 0) S.scales = 0;
+        if (lane == 0) S.scales = scales_word(P.pass + 1u, 0u);
         return last;
     }
     // the next pass's scales.  The forecast is in fp32 (in double it took 7 us); the scales themselves are the bisection's, to the bit
@@ -693,7 +694,7 @@ __device__ __noinline__ int32_t take_steps(const CountParams &P, unsigned long l
         bracket_of(min(lane, kCandidates - 1u), a, b);
         if (lane < next) S.mid[lane] = __dsqrt_rn(__dmul_rn(a, b));
     }
-    if (lane == 0) S.scales = next;
+    if (lane == 0) S.scales = scales_word(P.pass + 1u, next);
     return -1;
 }
 // All threads: the host reports the rate of the last evaluated step - its counts
@@ -814,7 +815,7 @@ __global__ void __launch_bounds__(kCountThreads, 1) quantise_count_kernel(const 
     const uint32_t tid = threadIdx.x, lane = tid & 31u;
     // Launched before the previous pass has ended (see launch_count): only W, mu and rows, which are older than that, are
     // read before the wait, and only then may the next launch come up.  A pass with several scales learns behind the wait how many they are.
-    const bool listed = P.mode == kPassSearch && !P.first;
+    const bool listed = P.mode == kPassSearch && P.pass > 0u;
     uint32_t k = 0, ctas = gridDim.x, part = blockIdx.x;                         // candidate, its CTAs and this one's share of the blocks
     uint32_t v = 0, v1 = 0, i = 0, col = 0;
     const uint32_t row_step = kCountThreads / P.per_row, col_step = kCountThreads % P.per_row;
@@ -840,12 +841,13 @@ __global__ void __launch_bounds__(kCountThreads, 1) quantise_count_kernel(const 
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (P.mode == kPassPolish && __ldcg(&P.state->stop)) return;                 // (the same for all CTAs: set by an earlier launch)
-    const uint32_t scales = listed ? __ldcg(&P.state->scales) : 1u;
+    const uint32_t scales = listed ? scales_of(__ldcg(&P.state->scales), P.pass) : 1u;
     if (!scales) return;
     if (listed) {
-        ctas = min(gridDim.x / scales, max((P.n_blocks + 255u) / 256u, 1u));
-        k = blockIdx.x / ctas;
-        part = blockIdx.x - k * ctas;
+        const PassShare share = pass_share(gridDim.x, blockIdx.x, scales, P.n_blocks);
+        k = share.scale;
+        part = share.part;
+        ctas = share.ctas;
         if (k >= scales) return;
         begin();
     }
@@ -971,7 +973,7 @@ __global__ void __launch_bounds__(kCountThreads, 1) quantise_count_kernel(const 
                 __threadfence();
             }
             before = __shfl_sync(0xFFFFFFFFu, before + mine, 0);
-            const int32_t last = (before >> 60) == scales ? take_steps(P, before) : -1;
+            const int32_t last = (before >> 60) == scales ? take_steps(P, scales, before) : -1;
             if (lane == 0) chosen = last;
         }
         __syncthreads();
@@ -1458,7 +1460,7 @@ public:
         P.most = P.n_blocks <= (1u << 17) ? kCandidates : 9u;
         const uint32_t passes = o.search_steps < 2 ? uint32_t(o.search_steps) : 2u + (P.steps - 1u + kLevels - 1u) / kLevels;
         for (uint32_t pass = 0; pass < passes; ++pass) {
-            P.first = pass == 0;
+            P.pass = pass;
             P.after = passes - std::min(passes, pass + 2u);
             EP_CUDA(launch_count(P, pass > 0));
         }
@@ -1704,7 +1706,7 @@ private:
     }
     // one CTA per SM, each with at least a few hundred blocks
     cudaError_t launch_count(CountParams P, bool follows) {
-        const bool listed = P.mode == kPassSearch && !P.first;
+        const bool listed = P.mode == kPassSearch && P.pass > 0u;
         const uint32_t ctas = listed ? uint32_t(sms_) : std::max(1u, std::min((P.n_blocks + 255u) / 256u, uint32_t(sms_)));
         // A pass's last CTA works on alone for 8 us; with programmatic launch the next pass's CTAs come up meanwhile, load
         // their first blocks and clear their counters.  Not the first pass: it reads what the kernel before it writes.

@@ -56,6 +56,12 @@ struct ep_blob {
     size_t size() const { return ext ? ext_size : heap.size(); }
 };
 
+#ifdef __CUDACC__
+#define EP_HOST_DEVICE __host__ __device__
+#else
+#define EP_HOST_DEVICE
+#endif
+
 namespace ep {
 
 constexpr double kEta = 1e-12;
@@ -124,10 +130,7 @@ inline CoderLayout coder_layout(const Model &m) {
 // can be from run_encode's if log2 and exp2 are within one unit in the last place there and here (two between them;
 // u = 2^-52), and everything else is rounded as there.  The secant divides by log_s - last_log_s, which scales next
 // to each other make as small as 2^-23.5: then two such units of log_s are 1e-8 of the slope.
-#ifdef __CUDACC__
-__host__ __device__
-#endif
-inline double next_scale_error(double log_s, double last_log_s, bool secant, double off_target, double per_doubling) {
+EP_HOST_DEVICE inline double next_scale_error(double log_s, double last_log_s, bool secant, double off_target, double per_doubling) {
     const double u = 2.220446049250313e-16;
     const double size = log_s < 0 ? -log_s : log_s, last = last_log_s < 0 ? -last_log_s : last_log_s;
     double slope = 2.0 * u;                          // relative, clamping to [1/2, 4] does not add to it
@@ -141,6 +144,22 @@ inline double next_scale_error(double log_s, double last_log_s, bool secant, dou
     if (step < 0) step = -step;
     const double exponent = 2.0 * u * size + step * (slope + 2.0 * u) + u * (size + step);
     return 0.7 * exponent + 8.0 * u;                 // ln 2, exp2 on either side and the roundings of a comparison
+}
+
+// A pass of the CUDA back end's search counts `scales` scales, each with the same number of the grid's CTAs.  The CTAs that are left over do
+// nothing, and nobody waits for them: one that starts late - another stream's kernel, or another encode, held its SM - may read the
+// number of scales after the pass's last CTA has stored the next pass's.  So the number is stored together with its pass, and a CTA takes a
+// number of any other pass for none.  (The others' numbers and scales stand until they have all arrived.)
+struct PassShare { uint32_t scale, part, ctas; };        // this CTA's scale (>= scales: left over), its share of the blocks, of how many
+EP_HOST_DEVICE inline PassShare pass_share(uint32_t grid, uint32_t cta, uint32_t scales, uint32_t n_blocks) {
+    const uint32_t fit = grid / scales, useful = (n_blocks + 255u) / 256u, ctas = fit < useful ? fit : useful;
+    return {cta / ctas, cta % ctas, ctas};
+}
+constexpr uint32_t kMostScales = 15;
+EP_HOST_DEVICE inline uint32_t scales_word(uint32_t pass, uint32_t scales) { return pass * 16u + scales; }
+EP_HOST_DEVICE inline uint32_t scales_of(uint32_t word, uint32_t pass) {
+    const uint32_t scales = word - pass * 16u;
+    return scales <= kMostScales ? scales : 0u;
 }
 
 // App. "Scale-search settings": complete rows, shape-dependent seed, sorted

@@ -129,3 +129,29 @@ def test_kernels_that_come_up_early_read_by_ordinary_loads():
     assert set(re.findall(r"launch_chained\((\w+_kernel)", text)) <= set(chained)
     for name, k in chained.items():
         assert not re.search(r"__restrict__|__ldg\(|\.nc\.", k), name
+
+
+def test_a_late_cta_takes_no_part_in_the_next_pass(tmp_path):
+    # a CTA of a search pass that has no share of it may read the number of scales after the pass's last CTA has stored the next pass's
+    run = _program(tmp_path, """
+        int wrong = 0, spare = 0;
+        for (uint32_t grid : {15u, 16u, 132u, 148u, 160u})
+            for (uint32_t n_blocks : {1u, 256u, 3000u, 65536u, 1u << 20})
+                for (uint32_t pass = 1; pass < 6; ++pass)
+                    for (uint32_t n = 1; n <= 15; ++n) {
+                        const uint32_t word = scales_word(pass, n);
+                        if (scales_of(word, pass) != n) ++wrong;               // what the others read
+                        for (uint32_t later = pass + 1; later < 8; ++later)
+                            for (uint32_t m = 0; m <= 15; ++m) {
+                                // (0: the search has ended; and no later pass counts the scales of an earlier one)
+                                if (scales_of(word, later)) ++wrong;
+                                const uint32_t seen = scales_of(scales_word(later, m), pass);
+                                for (uint32_t cta = 0; cta < grid; ++cta) {
+                                    if (pass_share(grid, cta, n, n_blocks).scale < n) continue;
+                                    ++spare;
+                                    if (seen && pass_share(grid, cta, seen, n_blocks).scale < seen) ++wrong;
+                                }
+                            }
+                    }
+        printf("%d %d\\n", wrong, spare > 0);""")
+    assert run() == ["0", "1"]

@@ -1,5 +1,7 @@
 """The CUDA encoder back end against the host encoder: the same bytes for the same input, and therefore
 (tests/test_library_host.py) the oracle's bytes as well."""
+import threading
+
 import numpy as np
 import pytest
 import torch
@@ -194,3 +196,32 @@ def test_device_encoder_codes_again_where_the_host_moves_on():
         assert np.array_equal(dev.data, host.data) and dev.report == host.report
         moved.add(host.report["b"])
     assert len(moved) == 2
+
+
+def test_device_encoder_bytes_with_several_encodes_at_once():
+    # CTAs of one call's passes start late where another call holds the SMs: two threads, each with a stream and a workspace of its own
+    jobs = [[(synth.gaussian_rows(256, 2048, 91), 4.0, {}), (synth.laplace_rows(64, 4096, 92), 6.0, dict(search_steps=9))],
+            [(synth.student_t_rows(700, 1032, 93), 3.0, dict(sample_vectors=3000)), (synth.gaussian_rows(1024, 4096, 94), 5.0, {})]]
+    refs = [[ep.encode(W, bpp, **kw).data for W, bpp, kw in mine] for mine in jobs]
+    devs = [[torch.from_numpy(W).cuda() for W, _, _ in mine] for mine in jobs]
+    workspaces = [torch.empty(max(W.size for W, _, _ in mine) * 8 + (16 << 20), dtype=torch.uint8, device="cuda") for mine in jobs]
+    streams, wrong, failed = [torch.cuda.Stream() for _ in jobs], [], []
+    torch.cuda.synchronize()
+
+    def work(t):
+        torch.cuda.set_device(devs[t][0].device)
+        try:
+            for turn in range(40):
+                for i, (_, bpp, kw) in enumerate(jobs[t]):
+                    got = ep.encode_device(devs[t][i], bpp, workspace=workspaces[t], stream=streams[t], **kw)
+                    if not np.array_equal(got.data, refs[t][i]):
+                        wrong.append((t, i, turn))
+        except ep.EntroPackError as e:
+            failed.append((t, e))
+
+    threads = [threading.Thread(target=work, args=(t,)) for t in range(len(jobs))]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not wrong and not failed
