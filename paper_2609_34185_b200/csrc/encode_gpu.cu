@@ -1502,7 +1502,7 @@ public:
         }
         if (rc) return rc;
         const SearchState &S = *state();
-        if (S.undecided) {
+        if (S.undecided || S.left) {             // (steps left: cannot happen, and the scale would not be the bisection's)
             EP_CUDA(cudaMemsetAsync(w_.state, 0, kStateBytes, st_));
             return EP_OK;
         }
@@ -1707,7 +1707,7 @@ private:
     // one CTA per SM, each with at least a few hundred blocks
     cudaError_t launch_count(CountParams P, bool follows) {
         const bool listed = P.mode == kPassSearch && P.pass > 0u;
-        const uint32_t ctas = listed ? uint32_t(sms_) : std::max(1u, std::min((P.n_blocks + 255u) / 256u, uint32_t(sms_)));
+        const uint32_t ctas = listed ? pass_grid(uint32_t(sms_)) : std::max(1u, std::min((P.n_blocks + 255u) / 256u, uint32_t(sms_)));
         // A pass's last CTA works on alone for 8 us; with programmatic launch the next pass's CTAs come up meanwhile, load
         // their first blocks and clear their counters.  Not the first pass: it reads what the kernel before it writes.
         cudaLaunchAttribute attr{};

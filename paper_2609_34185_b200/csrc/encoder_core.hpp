@@ -149,13 +149,15 @@ EP_HOST_DEVICE inline double next_scale_error(double log_s, double last_log_s, b
 // A pass of the CUDA back end's search counts `scales` scales, each with the same number of the grid's CTAs.  The CTAs that are left over do
 // nothing, and nobody waits for them: one that starts late - another stream's kernel, or another encode, held its SM - may read the
 // number of scales after the pass's last CTA has stored the next pass's.  So the number is stored together with its pass, and a CTA takes a
-// number of any other pass for none.  (The others' numbers and scales stand until they have all arrived.)
+// number of any other pass for none.  (The others' numbers and scales stand until they have all arrived.)  One CTA per SM, but never fewer than
+// a pass may have scales: a process limited to a share of the GPU may see fewer SMs than that.
+constexpr uint32_t kMostScales = 15;
+inline uint32_t pass_grid(uint32_t sms) { return sms > kMostScales ? sms : kMostScales; }
 struct PassShare { uint32_t scale, part, ctas; };        // this CTA's scale (>= scales: left over), its share of the blocks, of how many
 EP_HOST_DEVICE inline PassShare pass_share(uint32_t grid, uint32_t cta, uint32_t scales, uint32_t n_blocks) {
     const uint32_t fit = grid / scales, useful = (n_blocks + 255u) / 256u, ctas = fit < useful ? fit : useful;
     return {cta / ctas, cta % ctas, ctas};
 }
-constexpr uint32_t kMostScales = 15;
 EP_HOST_DEVICE inline uint32_t scales_word(uint32_t pass, uint32_t scales) { return pass * 16u + scales; }
 EP_HOST_DEVICE inline uint32_t scales_of(uint32_t word, uint32_t pass) {
     const uint32_t scales = word - pass * 16u;

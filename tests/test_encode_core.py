@@ -155,3 +155,41 @@ def test_a_late_cta_takes_no_part_in_the_next_pass(tmp_path):
                     }
         printf("%d %d\\n", wrong, spare > 0);""")
     assert run() == ["0", "1"]
+
+
+def test_every_scale_of_a_pass_is_counted_whole_on_any_number_of_sms(tmp_path):
+    run = _program(tmp_path, """
+        int wrong = 0;
+        for (uint32_t sms = 1; sms <= 160; ++sms)
+            for (uint32_t n_blocks : {1u, 255u, 257u, 4000u, 1u << 18, (1u << 31) - 1u})
+                for (uint32_t n = 1; n <= kMostScales; ++n) {
+                    std::vector<std::vector<int>> seen(n);
+                    for (uint32_t cta = 0; cta < pass_grid(sms); ++cta) {
+                        const PassShare s = pass_share(pass_grid(sms), cta, n, n_blocks);
+                        if (s.scale >= n) continue;
+                        seen[s.scale].resize(s.ctas);
+                        if (s.part < s.ctas) ++seen[s.scale][s.part]; else ++wrong;
+                    }
+                    for (const auto &parts : seen) {
+                        if (parts.empty()) ++wrong;
+                        for (int times : parts) wrong += times != 1;
+                    }
+                }
+        printf("%d\\n", wrong);""")
+    assert run() == ["0"]
+
+
+def _search_program(tmp_path):
+    exe, csrc, obj = str(tmp_path / "search_state"), os.path.join(ROOT, "paper_2609_34185_b200", "csrc"), str(tmp_path / "fake_device.o")
+    nvcc = os.environ.get("NVCC") or "/usr/local/cuda/bin/nvcc"
+    flags = ["-gencode", "arch=compute_100a,code=sm_100a", "-O0", "-std=c++17", "-Xcompiler", "-pthread", "-I", os.path.join(ROOT, "include"), "-I", csrc]
+    subprocess.run([nvcc, "-c", "-Dmain=fake_main", "-DcudaLaunchKernelExC=fake_launch", *flags, "-o", obj, os.path.join(ROOT, "tests", "fake_device.cpp")], check=True)
+    subprocess.run([nvcc, "-cudart", "none", *flags, "-o", exe, os.path.join(ROOT, "tests", "search_state.cu"), obj]
+                   + [os.path.join(csrc, f) for f in ("encoder.cpp", "stream.cpp")], check=True)
+    return lambda *a: subprocess.run([exe] + [str(v) for v in a], check=True, capture_output=True, text=True).stdout.split()
+
+
+def test_a_search_that_has_not_ended_is_left_to_the_host(tmp_path):
+    run = _search_program(tmp_path)
+    assert run(0) == ["0", "1"]
+    assert run(1) == ["0", "0"]           # steps not taken: the scale is not the bisection's
