@@ -352,7 +352,7 @@ struct SearchState {
     unsigned long long verdicts;     // of the running pass's candidates
     float s;                         // the next pass's scale
     float s_counted;                 // the scale of the full counts
-    uint32_t has_last;               // `last` holds the counts of the last step whose rate was evaluated
+    uint32_t has_last, lost;         // a step's rate was evaluated; `last` does not hold the counts of the last such step
     uint32_t undecided;              // a decision within the rounding error, or too many symbols: the host repeats the search
     uint32_t overflow;               // a coordinate left the histogram range
     uint32_t stop;                   // the full passes are over
@@ -617,7 +617,9 @@ __device__ __forceinline__ uint32_t judge_candidate(const CountParams &P, uint32
 }
 
 // Warp 0 of a pass's last CTA: as many steps as the pass's n scales are for, in order, and the scales of the next pass.  Returns (in every lane) the
-// candidate whose counts the host gets, or -1.
+// candidate whose counts are to be kept, or -1: the host gets those of the last step whose scale had a table.  That step is usually one of the
+// last pass, but while the bracket's finer end has no table, all steps of the next pass may be without one.  (Kept by the last pass only, 4 of 24 searches
+// at 9 bits - 96 x 1024, Laplace, for a rate above that of the finest scale with a table - were left to the host, 9 of 24 with Student-t rows.)
 __device__ __noinline__ int32_t take_steps(const CountParams &P, uint32_t n, unsigned long long verdicts) {
     SearchState &S = *P.state;
     const bool first_pass = P.pass == 0u;
@@ -644,6 +646,8 @@ __device__ __noinline__ int32_t take_steps(const CountParams &P, uint32_t n, uns
         if (v & kAbove) { lo = mid; rate_lo = r; } else { hi = mid; rate_hi = r; }
         --left;
     }
+    const bool keep = last >= 0 && (!left || rate_lo != rate_lo);
+    const uint32_t lost = last == -1 ? (first_pass ? 0u : __ldcg(&S.lost)) : !keep;
     if (lane == 0) {
         S.lo = lo;
         S.hi = hi;
@@ -655,11 +659,12 @@ __device__ __noinline__ int32_t take_steps(const CountParams &P, uint32_t n, uns
         if (overflow) S.overflow = 1;
         if (undecided) S.undecided = 1;
         if (last != -1) S.has_last = 1;
-        if (!left && last < 0 && __ldcg(&S.has_last)) S.undecided = 1;       // (the last step's counts are gone)
+        S.lost = lost;
+        if (!left && lost) S.undecided = 1;
     }
     if (!left) {
         if (lane == 0) S.scales = scales_word(P.pass + 1u, 0u);
-        return last;
+        return keep ? last : -1;
     }
     // the next pass's scales.  The forecast is in fp32 (in double it took 7 us); the scales themselves are the bisection's, to the bit
     uint32_t next = 0;
@@ -695,9 +700,9 @@ __device__ __noinline__ int32_t take_steps(const CountParams &P, uint32_t n, uns
         if (lane < next) S.mid[lane] = __dsqrt_rn(__dmul_rn(a, b));
     }
     if (lane == 0) S.scales = scales_word(P.pass + 1u, next);
-    return -1;
+    return keep ? last : -1;
 }
-// All threads: the host reports the rate of the last evaluated step - its counts
+// All threads: the host reports the rate of the last evaluated step - its counts, until a later one's replace them
 __device__ __forceinline__ void keep_last(const CountParams &P, uint32_t k) {
     SearchState &S = *P.state;
     const Candidate &c = S.cand[k];

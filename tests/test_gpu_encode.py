@@ -1,5 +1,7 @@
 """The CUDA encoder back end against the host encoder: the same bytes for the same input, and therefore
 (tests/test_library_host.py) the oracle's bytes as well."""
+import os
+import subprocess
 import threading
 
 import numpy as np
@@ -9,7 +11,7 @@ import torch
 import oracle
 import paper_2609_34185_b200 as ep
 from paper_2609_34185_b200 import synth
-from test_encode_core import disjoint_cosets
+from test_encode_core import ROOT, disjoint_cosets
 
 pytestmark = pytest.mark.gpu
 
@@ -225,3 +227,21 @@ def test_device_encoder_bytes_with_several_encodes_at_once():
     for t in threads:
         t.join()
     assert not wrong and not failed
+
+
+def test_device_encoder_ends_searches_that_meet_scales_without_tables(tmp_path):
+    # the target is above what the finest scale with a table gives, so the last steps of a search often find no table: the
+    # counts of the last step that had one are of an earlier pass
+    exe, csrc = str(tmp_path / "search_done"), os.path.join(ROOT, "paper_2609_34185_b200", "csrc")
+    nvcc = os.environ.get("NVCC") or "/usr/local/cuda/bin/nvcc"
+    subprocess.run([nvcc, "-gencode", "arch=compute_100a,code=sm_100a", "-O1", "-std=c++17", "-Xcompiler", "-ffp-contract=off,-pthread",
+                    "-I", os.path.join(ROOT, "include"), "-I", csrc, "-o", exe, os.path.join(ROOT, "tests", "search_done.cu")]
+                   + [os.path.join(csrc, f) for f in ("encoder.cpp", "stream.cpp")], check=True)
+    Ws = [synth.laplace_rows(96, 1024, 700 + i) for i in range(24)]
+    np.stack(Ws).tofile(tmp_path / "w.bin")
+    run = subprocess.run([exe, str(tmp_path / "w.bin"), "24", "96", "1024", "12.0", "9"], check=True, capture_output=True, text=True, timeout=60)
+    assert run.stdout.split() == ["1"] * 24
+    for W in Ws[:6]:
+        host = ep.encode(W, 12.0, b_start=9, b_max=9, polish_steps=0)
+        dev = ep.encode_device(torch.from_numpy(W).cuda(), 12.0, b_start=9, b_max=9, polish_steps=0)
+        assert np.array_equal(dev.data, host.data) and dev.report == host.report
