@@ -1511,7 +1511,7 @@ public:
             EP_CUDA(cudaMemsetAsync(w_.state, 0, kStateBytes, st_));
             return EP_OK;
         }
-        coded_ = ahead && S.code;
+        coded_ = ahead && S.code && *reported();      // (without the report the frequencies to compare are not here)
         coded_b_ = job.b;
         r.s = sigma_of_ = S.s_counted;
         sigma_there_ = true;

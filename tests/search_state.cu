@@ -19,7 +19,7 @@
 #undef private
 
 namespace {
-uint32_t steps_left = 0;
+uint32_t steps_left = 0, coded = 0, entries_made = 0;
 }
 
 extern "C" cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t *, const void *kernel, void **args) {
@@ -27,14 +27,17 @@ extern "C" cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t *, const voi
         const CountParams &P = *static_cast<const CountParams *>(args[0]);
         SearchState &S = *P.state;
         if (P.mode == kPassSearch) S.left = steps_left;
-        if (P.mode == kPassPolish) { S.polished = S.stop = 1; S.s_counted = 0.5f; }
+        if (P.mode == kPassPolish) { S.polished = S.stop = 1; S.s_counted = 0.5f; S.code = coded; }
     }
+    if (kernel == reinterpret_cast<const void *>(encode_entries_kernel)) ++entries_made;
     return cudaSuccess;
 }
 
-// argument: the steps of the bisection that the passes leave undone.  Prints the call's status and whether the host takes its result
+// arguments: the steps of the bisection that the passes leave undone; have they made the tile coder's entries?  Prints the call's status,
+// whether the host takes its result, and how often it has entries made for the tile coder then
 int main(int, char **argv) {
     steps_left = uint32_t(std::atoi(argv[1]));
+    coded = uint32_t(std::atoi(argv[2]));
     const uint32_t R = 16, C = 64, V = 32;
     const size_t need = carve(nullptr, R, C, V).bytes;
     void *ws = nullptr, *W = nullptr;
@@ -48,6 +51,7 @@ int main(int, char **argv) {
     ep::SearchResult found;
     bool done = false;
     if (!rc) rc = be.search({4.0, 11, V, R * C / 8, R}, o, found, &done);
-    std::printf("%d %d\n", rc, int(done));
+    if (!rc && done) rc = be.begin_finish(found.s, 11, V, found.full);
+    std::printf("%d %d %u\n", rc, int(done), entries_made);
     return 0;
 }
