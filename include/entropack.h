@@ -162,17 +162,18 @@ int ep_pack_fields(const int32_t *fields, uint32_t R, uint32_t C, int32_t b, uin
                    const float *row_scales, float s_info, int32_t threads, ep_blob **out);
 
 /* The same encoder with the heavy steps on the GPU (row RMS, E8 quantisation and field histograms, the search,
- * Eq. 13, tile coding); the final tables are made on the host.  The result is byte for byte the blob ep_encode
- * produces for the same W and options.  d_W is a device copy of W (16-byte
+ * Eq. 13, tile coding).  The final tables are made there for coding and on the host for the blob, and compared.
+ * The result is byte for byte the blob ep_encode produces for the same W and options.  d_W is a device copy of W (16-byte
  * aligned), d_workspace a 256-byte aligned device buffer of ep_encode_device_workspace_bytes() bytes
- * (about 52 bytes per 8-weight block and 13 MB).  The call enqueues on `stream` and synchronises it several times;
- * it returns the finished host blob.  EP_ERR_UNSUPPORTED (use ep_encode instead) if a lattice coordinate
+ * (about 52 bytes per 8-weight block and 13 MB).  The call enqueues on `stream`, busy-waits for the search's results - 5 ms
+ * at most, one core per calling thread; earlier work on the stream counts - and synchronises the stream once, more often
+ * where those take longer or the host has to take over part of the search; it returns the finished host blob.  EP_ERR_UNSUPPORTED (use ep_encode instead) if a lattice coordinate
  * exceeds +-4095 or the tables hold more than 40960 symbols in total.
  * The blob of this call lives in page-locked host memory (the device copies the payload straight into it,
  * and a later upload of the blob runs at full bus speed).  Page-locking costs milliseconds, so ep_blob_free
  * keeps the buffer of the most recently freed such blob (one per process at most, the larger one when two
  * compete) for the next call whose blob fits; a model converted tensor by tensor allocates once or twice.
- * A second page-locked buffer of 0.7 MB (the counts of the passes) is kept the same way. */
+ * A second page-locked buffer of 0.8 MB (counts and frequencies of the passes) is kept the same way. */
 size_t ep_encode_device_workspace_bytes(uint32_t R, uint32_t C, double target_bpp, const ep_encode_opts *opts);
 int ep_encode_device(const float *d_W, uint32_t R, uint32_t C, double target_bpp, const ep_encode_opts *opts,
                      void *d_workspace, size_t workspace_bytes, void *stream, ep_blob **out);

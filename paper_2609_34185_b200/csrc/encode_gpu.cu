@@ -1648,12 +1648,13 @@ private:
         return launch_chained(compact_kernel, n_tiles, n_tiles < 600u ? 512u : 128u, 0, static_cast<const uint16_t *>(w_.scratch), 9u * V_,
                               static_cast<const uint32_t *>(w_.counts), static_cast<const uint32_t *>(w_.index), static_cast<const SearchState *>(w_.state), w_.payload);
     }
-    // Until the search's report is here (report_search).  The stream's own end is waited for if it takes very long: an error shows there, and a
-    // report that still is not here is fetched.
+    // Until the search's report is here (report_search).  If that takes longer than 5 ms - a very large tensor, earlier work on the stream - the
+    // stream's own end is waited for, in the way that the process has its threads wait: an error shows there, and a report that still
+    // is not here is fetched.  (The host's tables then come behind the coder: some 40 us of a long call.)
     int await_report() {
         const auto since = std::chrono::steady_clock::now();
         for (uint32_t i = 1; !*reported(); ++i) {
-            if (i % 1024u == 0 && std::chrono::steady_clock::now() - since > std::chrono::milliseconds(50)) {
+            if (i % 1024u == 0 && std::chrono::steady_clock::now() - since > std::chrono::milliseconds(5)) {
                 EP_CUDA(cudaStreamSynchronize(st_));
                 if (!*reported()) return fetch(true);
                 break;

@@ -34,7 +34,7 @@ extern "C" cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t *, const voi
 }
 
 // arguments: the steps of the bisection that the passes leave undone; have they made the tile coder's entries?  Prints the call's status,
-// whether the host takes its result, and how often it has entries made for the tile coder then
+// whether the host takes its result, how often it has entries made for the tile coder then, and the milliseconds that the search kept its core
 int main(int, char **argv) {
     steps_left = uint32_t(std::atoi(argv[1]));
     coded = uint32_t(std::atoi(argv[2]));
@@ -50,8 +50,10 @@ int main(int, char **argv) {
     int rc = be.prepare(ep::sample_rows(R, C, o.sample_vectors));
     ep::SearchResult found;
     bool done = false;
+    const std::clock_t since = std::clock();
     if (!rc) rc = be.search({4.0, 11, V, R * C / 8, R}, o, found, &done);
+    const int busy = int(1000 * (std::clock() - since) / CLOCKS_PER_SEC);
     if (!rc && done) rc = be.begin_finish(found.s, 11, V, found.full);
-    std::printf("%d %d %u\n", rc, int(done), entries_made);
+    std::printf("%d %d %u %d\n", rc, int(done), entries_made, busy);
     return 0;
 }
