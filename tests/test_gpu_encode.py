@@ -245,3 +245,27 @@ def test_device_encoder_ends_searches_that_meet_scales_without_tables(tmp_path):
         host = ep.encode(W, 12.0, b_start=9, b_max=9, polish_steps=0)
         dev = ep.encode_device(torch.from_numpy(W).cuda(), 12.0, b_start=9, b_max=9, polish_steps=0)
         assert np.array_equal(dev.data, host.data) and dev.report == host.report
+
+
+@pytest.mark.parametrize("shape", [(64, 1024), (1100, 1024)])        # up to fifteen scales per pass; more than 2^17 blocks: nine
+@pytest.mark.parametrize("bpp,kw", [
+    (4.0, dict(search_steps=1)),
+    (4.0, dict(search_steps=2)),
+    (4.0, dict(search_steps=3)),
+    (4.0, dict(search_steps=4)),
+    (4.0, dict(search_steps=7)),
+    (4.0, dict(search_steps=14)),
+    (4.0, dict(search_steps=60)),                                     # the bracket's ends meet
+    (4.0, dict(bracket_lo=0.2, bracket_hi=0.3)),
+    (4.0, dict(bracket_lo=0.25, bracket_hi=0.25000001)),              # the same scale all the way
+    (3.0, dict(bracket_lo=0.05, bracket_hi=0.1)),                     # the target is on one side of the bracket: one-sided forecasts to the end,
+    (6.0, dict(bracket_lo=0.5, bracket_hi=2.0)),
+    (6.0, dict(bracket_lo=0.5, bracket_hi=2.0, polish_steps=0)),
+    (12.0, dict(b_start=9, b_max=9, polish_steps=0)),                 # beyond every scale with a table: trees of four steps
+    (12.0, dict(b_start=9, b_max=9, polish_steps=0, search_steps=6)),
+])
+def test_device_encoder_searches_like_the_hosts(shape, bpp, kw):
+    W = synth.laplace_rows(*shape, 77)
+    host = ep.encode(W, bpp, **kw)
+    dev = ep.encode_device(torch.from_numpy(W).cuda(), bpp, **kw)
+    assert np.array_equal(dev.data, host.data) and dev.report == host.report
