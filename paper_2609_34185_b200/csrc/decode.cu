@@ -622,7 +622,7 @@ __device__ __forceinline__ void decode_tile_plain(const JobParams &J, uint32_t t
 // multiply-add pipe has room, the ALU pipe has not; measured + 0.3 % / + 0.8 % on the 8192^2 tensor / the layer).  4 x + tab
 // comes first: it is there when the shift is, so the lookup waits for one multiply-add behind the shift, not for two.  The warps
 // of a full SM spend 62 % of their cycles waiting for operands, so four cycles per step are felt: 8192 x 8192 at 4 bpp to FP16 59.76 ->
-// 59.2 us, block of seven at 3.5 bpp to BF16 313.7 -> 310.6, at 2.5 bpp to FP8 303.6 -> 302.9 (2^12 slots: not this code).
+// 59.2 us, block of seven at 3.5 bpp to BF16 313.7 -> 310.6, at 2.5 bpp to FP8 303.6 -> 302.9 (streams of 2^12 slots have lookups of their own).
 #define EP_L1 "mad.lo.u32 uA, %0, 4, tabA;\n\t" "shr.u32 qA, %0, 11;\n\t"
 #define EP_L2 "mad.lo.u32 uA, qA, 0xFFFFE000, uA;\n\t"
 #define EP_L3(E, OFF) "ld.shared.u32 " E "A, [uA+" OFF "];\n\t"

@@ -430,9 +430,10 @@ __device__ __forceinline__ double cce_bound(const RateParams &P, double cce) { r
 
 struct Evaluation { double cce, tables; uint32_t worst; bool too_many, above; };   // above: by the counts' entropy alone
 
+struct Ranges { int32_t lo[EP_NUM_TABLES]; uint32_t K[EP_NUM_TABLES], at[EP_NUM_TABLES + 1]; };    // a candidate's tables and where they start
+
 // All threads of a candidate's last CTA: ranges and offsets of its tables, counts to `out`, histogram back to zero; unless
 // only counts are wanted, the frequencies of Sec. 3.3 (integers: the host's exactly), C_CE of Eq. 8 and the largest alphabet.
-struct Ranges { int32_t lo[EP_NUM_TABLES]; uint32_t K[EP_NUM_TABLES], at[EP_NUM_TABLES + 1]; };    // a candidate's tables and where they start
 __device__ __forceinline__ Evaluation gather_counts(const CountParams &P, uint32_t k, uint32_t *out, uint32_t *f_of, Ranges &D) {
     int32_t *const lo_of = D.lo;
     uint32_t *const K_of = D.K, *const at_of = D.at;
@@ -1705,7 +1706,8 @@ private:
         cfg.numAttrs = 1;
         return cudaLaunchKernelEx(&cfg, kernel, K(args)...);
     }
-    // launched while the kernel before it runs, whose results it does not use: the kernel does not wait until its end
+    // Launched while the kernel before it runs, whose results it does not use, so the kernel does its work without waiting.  But what is launched behind
+    // it, and only waits for it, may use them: one of its CTAs has to wait all the same before it ends (refit_kernel: the last)
     template <class... K, class... A>
     cudaError_t launch_beside(void (*kernel)(K...), uint32_t grid, uint32_t threads, size_t smem, A... args) {
         return launch_chained(kernel, grid, threads, smem, args...);

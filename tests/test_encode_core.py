@@ -4,6 +4,7 @@ import re
 import subprocess
 
 import numpy as np
+import pytest
 
 import paper_2609_34185_b200 as ep
 
@@ -179,8 +180,10 @@ def test_every_scale_of_a_pass_is_counted_whole_on_any_number_of_sms(tmp_path):
     assert run() == ["0"]
 
 
-def _search_program(tmp_path):
-    exe, csrc, obj = str(tmp_path / "search_state"), os.path.join(ROOT, "paper_2609_34185_b200", "csrc"), str(tmp_path / "fake_device.o")
+@pytest.fixture(scope="module")
+def search_program(tmp_path_factory):
+    tmp = tmp_path_factory.mktemp("search_state")
+    exe, csrc, obj = str(tmp / "search_state"), os.path.join(ROOT, "paper_2609_34185_b200", "csrc"), str(tmp / "fake_device.o")
     nvcc = os.environ.get("NVCC") or "/usr/local/cuda/bin/nvcc"
     flags = ["-gencode", "arch=compute_100a,code=sm_100a", "-O0", "-std=c++17", "-Xcompiler", "-pthread", "-I", os.path.join(ROOT, "include"), "-I", csrc]
     subprocess.run([nvcc, "-c", "-Dmain=fake_main", "-DcudaLaunchKernelExC=fake_launch", *flags, "-o", obj, os.path.join(ROOT, "tests", "fake_device.cpp")], check=True)
@@ -189,17 +192,17 @@ def _search_program(tmp_path):
     return lambda *a: subprocess.run([exe] + [str(v) for v in a], check=True, capture_output=True, text=True).stdout.split()
 
 
-def test_a_search_that_has_not_ended_is_left_to_the_host(tmp_path):
-    run = _search_program(tmp_path)
+def test_a_search_that_has_not_ended_is_left_to_the_host(search_program):
+    run = search_program
     assert run(0, 0)[:3] == ["0", "1", "1"]
     assert run(1, 0)[:3] == ["0", "0", "0"]   # steps not taken: the scale is not the bisection's
 
 
-def test_frequencies_that_did_not_come_are_not_compared(tmp_path):
+def test_frequencies_that_did_not_come_are_not_compared(search_program):
     # the launches end without the report: state and counts are fetched, the frequencies in the page-locked buffer are those of an earlier call
-    assert _search_program(tmp_path)(0, 1)[:3] == ["0", "1", "1"]
+    assert search_program(0, 1)[:3] == ["0", "1", "1"]
 
 
-def test_a_report_that_takes_long_does_not_keep_the_core(tmp_path):
+def test_a_report_that_takes_long_does_not_keep_the_core(search_program):
     # earlier work on the stream, for instance: after a few milliseconds the thread waits as the process has its threads wait
-    assert int(_search_program(tmp_path)(0, 0)[3]) < 25
+    assert int(search_program(0, 0)[3]) < 25
